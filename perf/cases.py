@@ -348,3 +348,140 @@ def tolerance(case):
     else:
         k = case["hidden"] if kind == "outliers" else case["k"]
     return {"rel": min(7e-4, max(4e-5, 1.2e-7 * k))}
+
+
+# ------------------------------------------------------------------------------- in 64 bits, plain torch
+_QMAX = {"int8": 127.0, "e4m3": 448.0, "e5m2": 57344.0}
+
+
+def _oriented(t, contract_dim):
+    """The operand as [batch, non-contracting, contracting]."""
+    t = t.cuda()
+    t = t if t.dim() == 3 else t.unsqueeze(0)
+    return t if contract_dim == -1 else t.transpose(1, 2)
+
+
+def _uniform(shape, seed, stream):
+    """Draw of every element in C order: word i mod 4 of Philox4x32-10 on block i div 4, its upper 24 bits."""
+    n, mask = math.prod(shape), 0xFFFFFFFF
+    i = torch.arange((n + 3) // 4, device="cuda", dtype=torch.int64)
+    c = [i & mask, i >> 32, torch.full_like(i, stream), torch.zeros_like(i)]
+    k0, k1 = seed & mask, (seed >> 32) & mask
+
+    def product(m, x):                               # high and low word of the 64-bit product, in halves
+        a, b = (m >> 16) * x, (m & 0xFFFF) * x
+        s = ((a & 0xFFFF) << 16) + (b & mask)
+        return ((a >> 16) + (b >> 32) + (s >> 32)) & mask, s & mask
+    for _ in range(10):
+        (h0, l0), (h1, l1) = product(0xD2511F53, c[0]), product(0xCD9E8D57, c[2])
+        c = [h1 ^ c[1] ^ k0, l1, h0 ^ c[3] ^ k1, l0]
+        k0, k1 = (k0 + 0x9E3779B9) & mask, (k1 + 0xBB67AE85) & mask
+    return ((torch.stack(c, 1).reshape(-1)[:n] >> 8).double() / 2.0 ** 24).reshape(shape)
+
+
+def _quantized(x, fmt, gran, draw=None):
+    """(values of the codes as float64, scales, the fp32 quotients) of an oriented operand."""
+    x = x.float()
+    top = x.abs().amax(-1, keepdim=True) if gran == "channel" else x.abs().amax().reshape(1, 1, 1)
+    delta = torch.where(top > 0, top / torch.tensor(_QMAX[fmt], device="cuda"), torch.ones_like(top))
+    t = x / delta
+    a = t.clamp(-_QMAX[fmt], _QMAX[fmt])
+    if draw is not None:
+        m, emin = {"int8": (0, 0), "e4m3": (3, -6), "e5m2": (2, -14)}[fmt]
+        d = a.abs().double()
+        e = torch.frexp(d).exponent.double() - 1
+        step = torch.ones_like(d) if fmt == "int8" else torch.exp2(e.clamp(min=emin) - m)
+        lo = torch.floor(d / step) * step
+        v = torch.copysign(lo + step * (draw * step < d - lo), a.double())
+    elif fmt == "int8":
+        v = a.round().double()
+    else:
+        v = a.to(torch.float8_e4m3fn if fmt == "e4m3" else torch.float8_e5m2).double()
+    return v, delta.double(), t
+
+
+def _reduce(c, q, d):
+    diff = (c - q).abs()
+    be = torch.where(d > 0, diff / d, torch.zeros_like(d))
+    return [be.sum(), be.max(), (diff * diff).sum(), (c * c).sum(), (d * d).sum()]
+
+
+def _exact_record(l, r, ql, qr):
+    """Eq. 3 sums of oriented operands and their quantized values, blocks of output rows at a time."""
+    (vl, dl, _), (vr, dr, _) = ql, qr
+    vl, vr = vl * dl, vr * dr
+    l, r = l.double(), r.double()
+    total = None
+    rows = max(1, (1 << 27) // r.shape[1])
+    for b in range(0, l.shape[0], max(1, rows // l.shape[1])):
+        bs = slice(b, b + max(1, rows // l.shape[1]))
+        for i in range(0, l.shape[1], rows):
+            x = l[bs, i:i + rows]
+            rt = r[bs].transpose(1, 2)
+            part = _reduce(x @ rt, vl[bs, i:i + rows] @ vr[bs].transpose(1, 2), x.abs() @ rt.abs())
+            total = part if total is None else [max(p, t) if k == 1 else p + t for k, (p, t) in enumerate(zip(part, total))]
+    return [float(t) for t in total]
+
+
+def _record_dict(rows, counts):
+    names = ("sum_be", "max_be", "sum_diff2", "sum_ref2", "sum_den2")
+    d = {k: torch.tensor([row[i] for row in rows], dtype=torch.float64) for i, k in enumerate(names)}
+    d["count"] = torch.tensor(counts, dtype=torch.int64)
+    d["device_error"] = torch.zeros(len(rows), dtype=torch.int32)
+    return d
+
+
+def exact(case, seed):
+    """What run() returns for these inputs, in 64 bits.  None for the quantize cases: their outputs are bytes
+    and fp32 scales that are compared bit for bit."""
+    kind = case["kind"]
+    if kind == "quantize":
+        return None
+    with torch.no_grad():
+        s = prepare({**case, "planned": False} if kind == "probe" else case, seed)
+        if kind == "probe":
+            l, r = _oriented(s["L"], s["cl"]), _oriented(s["R"], s["cr"])
+            ql = _quantized(l, case["left"], case["gran"], _uniform(l.shape, 7, 0) if case["rounding"] == "stochastic_l" else None)
+            qr = _quantized(r, case["right"], case["gran"], _uniform(r.shape, 7, 1) if case["rounding"] == "stochastic_r" else None)
+            d = _record_dict([_exact_record(l, r, ql, qr)], [l.shape[0] * l.shape[1] * r.shape[1]])
+            return d if case["planned"] else {k: float(v[0]) for k, v in d.items()}
+        if kind in ("pass", "outliers"):
+            if kind == "pass":
+                products = _pass_probes(case, lambda t, cd: (t, cd))
+                tensors = s["tensors"]
+            else:
+                tensors = s
+                products = [("X", -1, "W", -2, f, f, g, g) for f in ("e4m3", "e5m2", "int8") for g in ("tensor", "channel")]
+            rows, counts = [], []
+            for l, cl, r, cr, fl, fr, gl, gr, *_ in products:
+                x, y = _oriented(tensors[l], cl), _oriented(tensors[r], cr)
+                rows.append(_exact_record(x, y, _quantized(x, fl, gl), _quantized(y, fr, gr)))
+                counts.append(x.shape[0] * x.shape[1] * y.shape[1])
+            return _record_dict(rows, counts)
+        if kind == "analyse":
+            x = _oriented(s["x"], -1)
+            v, delta, t = _quantized(x, case["fmt"], case["gran"])
+            x = x.double()
+            n, mean = x.numel(), x.mean()
+            m2, m3, m4 = (((x - mean) ** k).mean() for k in (2, 3, 4))
+            err, nz = (x - v * delta).abs(), x != 0
+            over = nz & (t.abs().double() > _QMAX[case["fmt"]])
+            under = nz & ~over & (v == 0)
+            mid = nz & ~over & ~under
+            re = torch.where(nz, err / x.abs(), torch.zeros_like(x))
+            e2 = err * err
+            sums = {"sum%d" % k: float((x ** k).sum()) for k in (1, 2, 3, 4)}
+            f = {"sum_re": re.sum(), "sum_re_round": re[mid].sum(), "max_re_round": re[mid].max(), "err2_round": e2[mid].sum(),
+                 "err2_overflow": e2[over].sum(), "err2_underflow": e2[under].sum(), "sum_x2": (x * x).sum()}
+            counts = {"count": n, "n_nonzero": int(nz.sum()), "n_overflow": int(over.sum()), "n_underflow": int(under.sum())}
+            return {**sums, "max_abs": float(x.abs().max()), "mean": float(mean), "variance": float(m2),
+                    "skew": float(m3 / m2 ** 1.5), "kurtosis": float(m4 / m2 ** 2),
+                    "error": {**{k: float(w) for k, w in f.items()}, **counts}, "device_error": 0}
+        l, r = s["l"], s["r"]
+        (vl, dl, _), (vr, dr, _) = _quantized(l, case["fmt"], case["gran"]), _quantized(r, case["fmt"], case["gran"])
+        l, r = l.double(), r.double()
+        c, d = l @ r.transpose(1, 2), l.abs() @ r.abs().transpose(1, 2)
+        q = (vl * dl) @ (vr * dr).transpose(1, 2)
+        names = ("sum_be", "max_be", "sum_diff2", "sum_ref2", "sum_den2")
+        return {"q": q, "c": c, "d": d, **{k: float(w) for k, w in zip(names, _reduce(c, q, d))}, "count": c.numel(),
+                "device_error": 0}
