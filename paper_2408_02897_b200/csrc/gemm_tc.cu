@@ -10,11 +10,11 @@
 //                        two-formats-in-one-pass probe (four accumulators fill tensor memory);
 //   tc_gemm_wide_kernel  256 x 256 tiles, two accumulator buffers: stand-alone products on outputs at
 //                        least 256 wide;
-//   tc_group_kernel      the fused probe (Eq. 3 record of one probe, or of up to 16 probes, per
-//                        persistent launch): reference L.R, denominator |L|.|R| and 8-bit product side
-//                        by side in tensor memory, |L| fed to the MMAs from tensor memory by converter
-//                        warps, the Eq. 3 statistics reduced in the epilogue; no M x N matrix ever
-//                        goes to HBM.  Its own comment describes roles and barriers.
+//   tc_group_kernel      the fused probe (Eq. 3 records of one probe or of many per persistent launch):
+//                        reference L.R and denominator |L|.|R| once per pair of operands, then the
+//                        8-bit products of all probes of that pair, |L| fed to the MMAs from tensor
+//                        memory by converter warps, the Eq. 3 statistics reduced in the epilogue; no
+//                        M x N matrix ever goes to HBM.  Its own comment describes roles and barriers.
 // Common to all: the MMA warp runs its loop converged and one elected lane issues; the epilogue
 // warps read the accumulators with tcgen05.ld (a warp may touch the lane quarter warp_id % 4; the
 // two warps of a quarter split the columns); a CTA keeps Eq. 3 statistics in registers across tiles
@@ -26,9 +26,12 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstdlib>
 #include <mutex>
+#include <type_traits>
+#include <vector>
 
 #include "qm_internal.h"
 
@@ -92,8 +95,6 @@ struct KernelArgs {
   // is result[1] and its per-CTA records follow the first format's gridDim.x records
   const float* dl2; const float* dr2;
   uint32_t idesc_lp2;
-  double* row_stats;                     // Probe (one format): optional [batch * M][5] per-row sums
-  const uint32_t* err_also[2];           // Probe (one format): further error words to report in the record, or null
 };
 
 // ------------------------------------------------------------------ PTX wrappers
@@ -390,66 +391,6 @@ __device__ __forceinline__ void stats16(const uint32_t* rc, const uint32_t* rd, 
     s.r2 = fma2(cv2, cv2, s.r2);
     s.n2 = fma2(dd2, dd2, s.n2);
   }
-}
-
-// The same statistics for the grouped kernel, which first brings a chunk into one form (the
-// 8-bit accumulator as fp32, dead columns zeroed) so that one instantiation per scale layout
-// serves every format and the ragged edge.  PER_COL: the right operand has a scale per column
-// (dr_s), otherwise kd2 holds (-delta_l delta_r) twice.
-struct StatsG {
-  float be0, be1;
-  uint64_t d2, r2, n2;
-  float mx;
-};
-template <bool PER_COL>
-__device__ __forceinline__ void stats16g(const uint32_t* rc, const uint32_t* rd, const uint32_t* rq, uint64_t kd2,
-                                         const float* dr_s, StatsG& s) {
-#pragma unroll
-  for (int j = 0; j < 16; j += 2) {
-    const uint64_t a2 = pack2(__uint_as_float(rq[j]), __uint_as_float(rq[j + 1]));
-    const uint64_t cv2 = pack2(__uint_as_float(rc[j]), __uint_as_float(rc[j + 1]));
-    const float d0 = __uint_as_float(rd[j]), d1 = __uint_as_float(rd[j + 1]);
-    const uint64_t dd2 = pack2(d0, d1);
-    uint64_t diff2;                                              // C - A dl dr
-    if (PER_COL) diff2 = fma2(mul2(a2, kd2), *reinterpret_cast<const uint64_t*>(dr_s + j), cv2);
-    else diff2 = fma2(a2, kd2, cv2);
-    // D == 0 implies C == Q == 0, so clamping the divisor keeps BE = 0 there without a branch
-    const uint64_t be2 = mul2(diff2, pack2(rcp_approx(fmaxf(d0, 1e-37f)), rcp_approx(fmaxf(d1, 1e-37f))));
-    float b0, b1;
-    unpack2(be2, b0, b1);
-    s.be0 += fabsf(b0);
-    s.be1 += fabsf(b1);
-    s.mx = fmaxf(s.mx, fmaxf(fabsf(b0), fabsf(b1)));
-    s.d2 = fma2(diff2, diff2, s.d2);
-    s.r2 = fma2(cv2, cv2, s.r2);
-    s.n2 = fma2(dd2, dd2, s.n2);
-  }
-}
-// Chunk CH (16 columns) of a warp's share of a tile: rq holds its 8-bit accumulators as read from
-// tensor memory; n_live < 16 only at the ragged edge of the matrix, whose dead columns count as zeros.
-template <int CH>
-__device__ __forceinline__ void stats_chunk(uint32_t (&rc)[64], uint32_t (&rd)[64], uint32_t (&rq)[16], int n_live,
-                                            bool is_i8, bool per_col, uint64_t kd2, const float* dr_s, StatsG& st) {
-  if (is_i8) {
-#pragma unroll
-    for (int k = 0; k < 16; ++k) rq[k] = __float_as_uint((float)(int)rq[k]);
-  }
-  if (n_live < 16) {
-#pragma unroll
-    for (int k = 0; k < 16; ++k)
-      if (k >= n_live) { rc[CH * 16 + k] = 0u; rd[CH * 16 + k] = 0u; rq[k] = 0u; }
-  }
-  if (per_col) stats16g<true>(&rc[CH * 16], &rd[CH * 16], rq, kd2, dr_s + CH * 16, st);
-  else stats16g<false>(&rc[CH * 16], &rd[CH * 16], rq, kd2, nullptr, st);
-}
-// Adds one tile's share of a row's Eq. 3 sums to the optional per-row check output.
-__device__ __forceinline__ void row_stats_add(double* rs, const StatsG& st) {
-  float x0, x1;
-  atomicAdd(rs + 0, (double)st.be0 + (double)st.be1);
-  atomicMax(reinterpret_cast<unsigned long long*>(rs + 1), (unsigned long long)__double_as_longlong((double)st.mx));
-  unpack2(st.d2, x0, x1); atomicAdd(rs + 2, (double)x0 + (double)x1);
-  unpack2(st.r2, x0, x1); atomicAdd(rs + 3, (double)x0 + (double)x1);
-  unpack2(st.n2, x0, x1); atomicAdd(rs + 4, (double)x0 + (double)x1);
 }
 
 template <int MODE, int LPKIND, int LPKIND2>
@@ -1043,45 +984,61 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 }
 
 // ------------------------------------------------------------------ the fused probe kernel
-// One persistent launch computes the Eq. 3 records of up to kMaxGroup probes (one probe is a
-// group of one).  A launch per probe pays, each time, the kernel's set-up and drain, the launch
-// gap, and the last wave of a tile count that is not a multiple of the 74 CTA pairs; here the
-// tiles of all probes form one sequence.  The host orders the probes by descending contraction
-// length (tile cost) and the sequence is dealt to the pairs back and forth (round r gives pair p
-// position r P + p when r is even and r P + P-1-p when it is odd), which for descending costs
-// balances the pairs to within one tile of the cheapest kind.  The operand maps, scales, shapes
-// and the 8-bit MMA kind are read per tile from a table in the kernel's parameter space.  A
-// pair's positions increase, so it meets each probe in one run: when the probe changes, the
-// epilogue warps reduce their statistics and write the CTA's record of the probe they leave.
+// One persistent launch computes the Eq. 3 records of many probes.  Probes of the same two operands
+// (a sweep of formats or granularities over one product) share the reference L.R and the
+// denominator |L|.|R|, which do not depend on the format, so they form one UNIT: per output tile the
+// reference and denominator products run once, then the 8-bit products of the unit's probes
+// (VARIANTS, up to kMaxVar) one after the other, each over the whole contraction.
 //
-// What bounds this kernel is shared-memory bandwidth: per 64-deep k-block the tensor cores need
-// 640 cycles, and with all six operand tiles (L, |L|, codes, R, |R|, codes) staged in shared
-// memory an SM writes 60 KB and reads 60 KB per k-block, which takes it 940.  So the left operand
-// of the denominator product |L|.|R| is not staged in shared memory: converter warps read this
-// CTA's 128 rows of the L tile, clear the sign bits and store the result into TENSOR memory, from
-// where the denominator MMAs take their A operand; the same warps write the |R| half-tile into
-// the stage.  No |x| copy exists in HBM, TMA brings 36 KB per k-block, the MMAs read 44 KB and the
-// converters move 32 KB.
+// The tiles of all units form one sequence.  The host orders the units by descending tile cost and
+// the sequence is dealt to the CTA pairs back and forth (round r gives pair p position r P + p when r
+// is even and r P + P-1-p when it is odd), which for descending costs balances the pairs to within
+// one tile of the cheapest kind.  The operand maps, scales, shapes and the 8-bit MMA kinds come
+// from a table in the kernel's parameter space.  A pair's positions increase, so it meets each unit in
+// one run: when the unit changes, the epilogue warps reduce their statistics and write the CTA's
+// records of the probes they leave.
+//
+// What bounds this kernel is shared-memory bandwidth, about 128 B per clock and SM for TMA writes, MMA
+// operand reads and ordinary accesses together, and under sustained load the power limit.  Per 64
+// contraction entries of a 256 x 128 tile the reference and denominator products move 72 KB (24 KB
+// by TMA, 16 KB of MMA operands, 32 KB by the converters; 512 tensor cycles) and an 8-bit product 24 KB
+// (12 + 12; 128 tensor cycles).  A product in F formats so costs 72 + 24 F KB per k-block against F
+// times 112 for separate probes with all three products side by side.  Measured (16384 x 4096 x 1024,
+// fused kernel only, same GPU): one format 284 us (separate 282), three 420 (793), six 660 (1624).
+// Running the products one after the other, instead of side by side on narrower tiles, is what keeps
+// the tiles 128 wide: five accumulators side by side would leave room for 64 columns each, at 256 KB
+// per 128 columns against the 144 KB here.
+//
+// The left operand of the reference and denominator products is not read from shared memory by the tensor
+// cores: converter warps read this CTA's 128 rows of the L tile once and store them, and the same with
+// the sign bits cleared, into TENSOR memory, from where both products take their A operand; they also
+// write the |R| half-tile into the stage.  No |x| copy exists in HBM.  Taking only |L| from tensor
+// memory (four stages of it instead of two of both) measured 3 to 8 % slower (the MMAs then read L from
+// shared memory); half-block stages, an |R| copy by two other warps and prefetching the next
+// block's values ahead of the fences each measured 5 to 20 % slower.
 //
 // Roles in each CTA (512 threads = 4 warpgroups; registers are re-divided with setmaxnreg):
-//   warp 0        TMA producer: per k-block the bf16 tiles of L and R and both code tiles into a
-//                 ring of kStages stages; a CTA's loads complete on its own `full` barrier.
+//   warp 0        TMA producer: blocks of the ring of kStages stages in the order of consumption: per tile
+//                 the k-blocks of L and R (64 entries deep), then per variant those of its codes
+//                 (128 deep); both kinds bring 128 bytes per row.  A CTA's loads complete on its own `full`.
 //   warp 1        allocates tensor memory; in the leader CTA it runs the MMA loop converged and
-//                 one elected lane issues the pair's MMAs; tcgen05.commit frees a stage (shared
-//                 and tensor memory) in both CTAs (`empty`).
+//                 one elected lane issues the pair's MMAs; tcgen05.commit frees a stage in both CTAs (`empty`).
 //   warps 2, 3    idle (they fill the first warpgroup).
 //   warps 4..7    converters, one per tensor-memory lane quarter: thread = one of the CTA's 128
-//                 left-operand rows.
+//                 left-operand rows.  Blocks of codes need no conversion: they only pass on that they landed.
 //   warps 8..15   epilogue.
-// Tensor memory: columns 0..127 reference L.R, 128..255 denominator |L|.|R|, 256..383 the 8-bit
-// product, 384..511 four stages of |L| (32 columns of two bf16 each per stage; the shared-memory
-// ring has five stages, so TMA runs a k-block further ahead than the converters can).  The epilogue
-// copies its reference and denominator columns into registers and hands those two blocks back
-// at once (`tmem_empty`), after which the MMA warp issues the next tile's reference and
-// denominator MMAs for as many k-blocks as there are stages; the 8-bit MMAs of those k-blocks
-// follow when the epilogue has finished the 8-bit block (`lp_done`).  No M x N matrix ever goes
-// to HBM.
-constexpr int kMaxGroup = 16;
+// Tensor memory: columns 0..127 reference, 128..255 denominator, 256..383 and 384..511 two 8-bit
+// accumulators.  The second one doubles as two stages of L and |L| (32 columns of two bf16 each): it
+// is only written between a tile's denominator product and the next tile's, because variant f of F uses
+// accumulator (F-1-f) & 1, so that the last variant of a tile never needs it and the next tile's
+// converters start under the last variant's MMAs.
+//   The epilogue copies its reference and denominator columns into registers when they are complete
+// (`rd_full`) and hands both blocks back at once (`rd_empty`); while the first 8-bit product runs it
+// forms the sums of C^2 and D^2 and replaces D by its reciprocal, so that evaluating a variant costs
+// 3 to 4 instructions per output.  The 8-bit accumulators come and go through `lp_full` / `lp_done`, one
+// pair of barriers each; `abs_free` tells this CTA's converters that the second one has been read.  No
+// M x N matrix ever goes to HBM.
+constexpr int kMaxVar = 6;                     // probes of one unit (three formats at two granularities)
 constexpr int kProbeThreads = 512;
 constexpr int kFirstEpiWarp = 8;               // warps 8..15: lane quarter = warp % 4 holds for both groups
 // registers per thread after the split (launch: 128 each): 56 + 104 + 176 + 176 = 4 x 128
@@ -1089,79 +1046,108 @@ constexpr int kRegsCtl = 56, kRegsConv = 104, kRegsEpi = 176;
 static_assert(kRegsCtl + kRegsConv + 2 * kRegsEpi <= 4 * 128, "the split must fit what the block was launched with");
 
 struct CfgP {
-  static constexpr int kStages = 5;          // stages of shared memory (TMA ring)
-  static constexpr int kAbsStages = 4;       // stages of |L| in tensor memory (128 columns / 32)
-  // stage: L, R, |R| (written by the converters), codes of L, codes of R
-  static constexpr uint32_t kOffL = 0, kOffR = kABf16, kOffRa = kOffR + kBBf16, kOffCl = kOffRa + kBBf16;
-  static constexpr uint32_t kOffCr = kOffCl + kALp;
-  static constexpr uint32_t kStageBytes = kOffCr + kBLp;             // 44 KB
-  static constexpr uint32_t kTileBytes = kStages * kStageBytes;      // 220 KB
-  static constexpr uint32_t kColRef = 0, kColDen = 128, kColLp = 256, kColAbsL = 384;   // tensor-memory columns
+  static constexpr int kStages = 6;          // stages of shared memory (TMA ring)
+  static constexpr int kTmemStages = 2;       // stages of L and |L| in tensor memory (128 columns / 64)
+  static constexpr int kLpDepth = 128;       // contraction entries of a block of codes
+  // stage: L, R, |R| (written by the converters); or codes of L, codes of R.  All rows are 128 bytes.
+  static constexpr uint32_t kOffL = 0, kOffR = kABf16, kOffRa = kOffR + kBBf16;
+  static constexpr uint32_t kStageBytes = kOffRa + kBBf16;           // 32 KB
+  static constexpr uint32_t kTileBytes = kStages * kStageBytes;      // 192 KB
+  static constexpr uint32_t kColRef = 0, kColDen = 128, kColLp = 256, kColL = 384;   // tensor-memory columns
 };
 
-// What the roles need of a probe for every tile, copied to shared memory once per CTA: the
+// What the roles need of a unit for every tile, copied to shared memory once per CTA: the
 // launch's table sits in the kernel's parameter space, and reads of it with an index known only
-// at run time go through the small constant cache, which eleven kilobytes of table thrash.
-struct WalkInfo {
+// at run time go through the small constant cache, which a table of this size thrashes.
+struct alignas(16) WalkInfo {
   int32_t tile_begin, per_b, inner, num_kb;         // per_b = tiles_m * tiles_n (tiles per batch element);
                                                     // inner = tiles_n: column tiles run fastest, -tiles_m: row tiles do
-  int32_t half_n, kind;
-  uint32_t idesc_ref, idesc_lp;
+  int32_t half_n, n_var, var_begin, K;
 };
+struct VarInfo { uint32_t idesc, flags; };
+enum : uint32_t { kVarI8 = 1, kVarScalePerRow = 2, kVarScalePerCol = 4, kVarRowStats = 8 };
 
+template <int UNITS, int VARS>
 struct SharedP {
-  uint64_t full[CfgP::kStages];     // per CTA: this CTA's loads of a stage have landed
-  uint64_t ready[CfgP::kAbsStages]; // leader: both CTAs' converters have seen their loads land and have written
-                                    //         |L| (tensor memory) and |R| (stage)
-  uint64_t empty[CfgP::kStages];    // per CTA: the pair's MMAs have finished with the k-block of the stage
-  uint64_t tmem_full;               // per CTA: the tile's accumulators are complete
-  uint64_t tmem_empty;              // leader: both CTAs' epilogues have copied out reference and denominator
-  uint64_t lp_done;                 // leader: both CTAs' epilogues have finished a tile
+  uint64_t full[CfgP::kStages];     // per CTA: this CTA's loads of a block have landed
+  uint64_t ready[CfgP::kStages];    // leader: both CTAs' converters have seen their loads land and, for L and R,
+                                    //         have written L and |L| (tensor memory) and |R| (stage)
+  uint64_t empty[CfgP::kStages];    // per CTA: the pair's MMAs have finished with the block of the stage
+  uint64_t rd_full;                 // per CTA: the tile's reference and denominator are complete
+  uint64_t rd_empty;                // leader: both CTAs' epilogues have copied them out
+  uint64_t lp_full[2];              // per CTA: an 8-bit accumulator is complete
+  uint64_t lp_done[2];              // leader: both CTAs' epilogues have read it
+  uint64_t abs_free;                // per CTA: this CTA's epilogue has read the tile's last use of the second 8-bit accumulator
   uint64_t drain;                   // leader, give-up path only: every MMA issued so far has completed
   uint32_t tmem_base;
   uint32_t abort_flag;
   uint32_t is_last;
-  uint32_t issued;                  // k-blocks whose loads the producer has issued (read on the give-up path)
-  float delta_r[2][kBlockN];
-  double red[5][kEpiWarps];
-  WalkInfo walk[kMaxGroup];
+  uint32_t issued;                  // blocks whose loads the producer has issued (read on the give-up path)
+  float delta_r[2][kMaxVar][kBlockN];
+  // per warp and pair of rows (lanes l and l + 16): sum BE, sum diff^2, max BE of each variant of the unit
+  double2 sums[kMaxVar][kEpiWarps][16];
+  float maxima[kMaxVar][kEpiWarps][16];
+  double red[3 * kMaxVar + 2][kEpiWarps];
+  float dl_tensor[kMaxVar], dr_tensor[kMaxVar];     // per-tensor scales of the unit in hand (1 where per channel)
+  WalkInfo walk[UNITS];
+  VarInfo var[VARS];
 };
 
-struct GroupProblem {
-  CUtensorMap maps[4];        // L, R, codes L, codes R
-  KernelArgs a;               // num_tiles, tiles_m, tiles_n: of this probe
+struct GroupUnit {
+  CUtensorMap maps[2];        // L, R
+  int32_t M, N, K;
+  int32_t tiles_m, tiles_n;
   int32_t tile_begin;         // position of its first tile in the sequence
-  int32_t kind;               // kKindF8 or kKindI8
   int32_t half_n;             // right-operand rows each CTA stages: 64, or 32 for outputs at most 64 wide
   int32_t m_fastest;          // the tiles of a batch element are walked down the rows first (below)
-  uint32_t idesc_ref;         // instruction descriptor of the bf16 MMAs (N = 2 * half_n)
+  int32_t var_begin, n_var;
 };
+struct GroupVar {
+  CUtensorMap maps[2];        // codes of L, codes of R
+  const float* dl; const float* dr;
+  double* partials;           // gridDim.x records
+  qm_metric_result* result;
+  double* row_stats;          // optional [batch * M][5] per-row sums
+  uint32_t* err_word;
+  const uint32_t* err_also[2];           // further error words to report in the record, or null
+  uint64_t count;             // batch * M * N
+  uint32_t flags;             // kVar...; per-channel scales are indexed by batch * M + row, batch * N + column
+  uint32_t idesc_lp;          // instruction descriptor of the 8-bit MMA
+};
+template <int UNITS, int VARS>
 struct GroupTable {
-  int32_t n, total_tiles;
-  uint32_t stop_after_kb;     // test hook: the producer issues no k-block beyond this many (0xffffffff: off)
-  uint32_t pad0;
+  static constexpr int kUnits = UNITS, kVars = VARS;
+  int32_t n, n_var, total_tiles;
+  uint32_t stop_after_kb;     // test hook: the producer issues no block beyond this many (0xffffffff: off)
   uint64_t wait_limit_ns;     // bound of every barrier wait
-  int32_t pad[10];
-  GroupProblem p[kMaxGroup];
+  uint32_t* done_counter;     // zero on entry; counts finished CTAs
+  uint32_t* err0;             // a wait that runs out is reported here and in every record
+  GroupUnit u[UNITS];
+  GroupVar v[VARS];
 };
+// A launch's table has to fit into 32 764 bytes of kernel parameters.  24 units hold the 18 products
+// of an encoder layer in one launch; a single probe passes a table of its own size (1 KB).
+using TableBig = GroupTable<24, 56>;
+using TableOne = GroupTable<1, 1>;
+static_assert(sizeof(TableBig) <= 32764, "kernel parameters");
 
 // position of pair `pair` in round r of the back-and-forth deal
 __device__ __forceinline__ int group_position(int r, int pair, int num_pairs) {
   return r * num_pairs + ((r & 1) ? num_pairs - 1 - pair : pair);
 }
 
-// The tiles of one CTA pair in order, k-block by k-block: every role walks the same sequence.
-// A pair's positions ascend, so the search for a position's probe continues from the probe in hand.
+// The tiles of one CTA pair in order: every role walks the same sequence.
+// A pair's positions ascend, so the search for a position's unit continues from the unit in hand.
 struct TileWalk {
   const WalkInfo* wk;
   int n, total_tiles;
   int r, pair, num_pairs;
-  int pi, num_kb, kb, half_n;
+  int pi, num_kb, half_n, n_var, var_begin, K;
   TileCoord tc;
   bool valid;
   __device__ __forceinline__ void start(const WalkInfo* wk_, int n_, int total_tiles_, int pair_, int num_pairs_) {
     wk = wk_; n = n_; total_tiles = total_tiles_;
-    r = -1; pair = pair_; num_pairs = num_pairs_; kb = 0; num_kb = 0; pi = 0; half_n = 0; valid = true;
+    r = -1; pair = pair_; num_pairs = num_pairs_; num_kb = 0; pi = 0; half_n = 0; valid = true;
     next_tile();
   }
   // moves to the pair's next tile; valid = false when there is none
@@ -1174,7 +1160,8 @@ struct TileWalk {
         continue;
       }
       while (pi + 1 < n && pos >= wk[pi + 1].tile_begin) ++pi;
-      const int4 w4 = *reinterpret_cast<const int4*>(&wk[pi]);          // tile_begin, per_b, inner, num_kb
+      const int4 w4 = reinterpret_cast<const int4*>(&wk[pi])[0];        // tile_begin, per_b, inner, num_kb
+      const int4 x4 = reinterpret_cast<const int4*>(&wk[pi])[1];        // half_n, n_var, var_begin, K
       const int t = pos - w4.x;
       tc.b = t / w4.y;
       const int rem = t - tc.b * w4.y;
@@ -1183,14 +1170,26 @@ struct TileWalk {
       tc.m_tile = w4.z < 0 ? inner_i : outer_i;
       tc.n_tile = w4.z < 0 ? outer_i : inner_i;
       num_kb = w4.w;
-      half_n = wk[pi].half_n;
-      kb = 0;
+      half_n = x4.x; n_var = x4.y; var_begin = x4.z; K = x4.w;
       return;
     }
   }
-  // moves to the next k-block of the sequence
-  __device__ __forceinline__ void next_kb() {
-    if (++kb >= num_kb) next_tile();
+  // what the MMA warp needs, known to be the same in all lanes
+  __device__ __forceinline__ void make_uniform() {
+    num_kb = __shfl_sync(0xffffffffu, num_kb, 0);
+    half_n = __shfl_sync(0xffffffffu, half_n, 0);
+    n_var = __shfl_sync(0xffffffffu, n_var, 0);
+    var_begin = __shfl_sync(0xffffffffu, var_begin, 0);
+    K = __shfl_sync(0xffffffffu, K, 0);
+  }
+  __device__ __forceinline__ int lp_blocks() const { return (K + CfgP::kLpDepth - 1) / CfgP::kLpDepth; }
+};
+
+// Position in the ring of stages.
+struct Ring {
+  uint32_t s = 0, parity = 0;       // stage, and the parity of its use
+  __device__ __forceinline__ void next() {
+    if (++s == (uint32_t)CfgP::kStages) { s = 0; parity ^= 1u; }
   }
 };
 
@@ -1244,6 +1243,14 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
         "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
       : "memory");
 }
+// 32 lanes x 8 consecutive 32-bit columns.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+      : "r"(taddr)
+      : "memory");
+}
 // D[256 x N] (+)= A[256 x 16] . B[N x 16]^T across the CTA pair, A (bf16) taken from tensor memory:
 // each CTA's 128 rows at the same column address, two values per 32-bit column.
 __device__ __forceinline__ void mma_pair_a_tmem(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc,
@@ -1261,40 +1268,104 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
   return v;
 }
 
+// Eq. 3 statistics of one row of one variant's tile.
+struct StatsV {
+  float be0, be1, mx;
+  uint64_t d2;
+};
+// Eight consecutive columns of a row: reference rc, reciprocal denominator ri, raw 8-bit accumulator rq.
+// PER_COL: the right operand has a scale per column (dr_s) and kd2 holds -delta_l twice, otherwise
+// kd2 holds (-delta_l delta_r) twice.
+template <bool PER_COL>
+__device__ __forceinline__ void eval8(const uint32_t* rc, const uint32_t* ri, uint32_t (&rq)[8], bool is_i8, uint64_t kd2,
+                                      const float* dr_s, StatsV& s) {
+  if (is_i8) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) rq[j] = __float_as_uint((float)(int)rq[j]);
+  }
+#pragma unroll
+  for (int j = 0; j < 8; j += 2) {
+    const uint64_t a2 = pack2(__uint_as_float(rq[j]), __uint_as_float(rq[j + 1]));
+    const uint64_t cv2 = pack2(__uint_as_float(rc[j]), __uint_as_float(rc[j + 1]));
+    uint64_t diff2;                                              // C - A dl dr
+    if (PER_COL) diff2 = fma2(mul2(a2, kd2), *reinterpret_cast<const uint64_t*>(dr_s + j), cv2);
+    else diff2 = fma2(a2, kd2, cv2);
+    const uint64_t be2 = mul2(diff2, pack2(__uint_as_float(ri[j]), __uint_as_float(ri[j + 1])));
+    float b0, b1;
+    unpack2(be2, b0, b1);
+    s.be0 += fabsf(b0);
+    s.be1 += fabsf(b1);
+    s.mx = fmaxf(s.mx, fmaxf(fabsf(b0), fabsf(b1)));
+    s.d2 = fma2(diff2, diff2, s.d2);
+  }
+}
+// One variant of a tile for this warp's lane quarter and columns: the accumulator comes eight columns at
+// a time, the next eight on their way while eight are evaluated; `release` runs (converged) as soon as
+// the last ones are in registers.  live = columns of this warp that exist in the matrix (may be <= 0).
+template <bool PER_COL, typename Release>
+__device__ __forceinline__ void eval_variant(uint32_t taddr, const uint32_t (&rc)[64], const uint32_t (&ri)[64], int live,
+                                             bool is_i8, uint64_t kd2, const float* dr_s, StatsV& st, Release release) {
+  uint32_t q0[8], q1[8];
+  if (live <= 0) { release(); return; }
+  tmem_ld8(taddr, q0);
+  tmem_ld_wait();
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {                    // 16 columns per step
+    if (p * 16 >= live) break;
+    const bool more = p < 3 && (p + 1) * 16 < live;
+    tmem_ld8(taddr + p * 16 + 8, q1);
+    eval8<PER_COL>(&rc[p * 16], &ri[p * 16], q0, is_i8, kd2, dr_s + p * 16, st);
+    tmem_ld_wait();
+    if (more) tmem_ld8(taddr + p * 16 + 16, q0);
+    else release();
+    eval8<PER_COL>(&rc[p * 16 + 8], &ri[p * 16 + 8], q1, is_i8, kd2, dr_s + p * 16 + 8, st);
+    if (more) tmem_ld_wait();
+  }
+}
+
+template <typename Table>
 __global__ void __launch_bounds__(kProbeThreads, 1)
-tc_group_kernel(const __grid_constant__ GroupTable tab) {
+tc_group_kernel(const __grid_constant__ Table tab) {
   using C = CfgP;
-  constexpr int kStages = C::kStages, kAbs = C::kAbsStages;
+  using Sh = SharedP<Table::kUnits, Table::kVars>;
+  constexpr int kStages = C::kStages, kTmemStages = C::kTmemStages;
   extern __shared__ uint8_t smem_raw[];
   // tiles start on a 1024-byte boundary (the 128-byte swizzle atom); the offset is the same in
   // both CTAs of the pair because their dynamic shared memory starts at the same address
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  SharedP* sh = reinterpret_cast<SharedP*>(tiles + C::kTileBytes);
+  Sh* sh = reinterpret_cast<Sh*>(tiles + C::kTileBytes);
   const uint32_t tile_base = smem_u32(tiles);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // the shuffle tells the compiler that the warp index, and with it every role's control flow, is the same in
+  // all lanes: the operands of tcgen05 instructions then stay in uniform registers
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
-  const Waiter w{&sh->abort_flag, tab.p[0].a.err_word, tab.wait_limit_ns};   // a timed-out wait is reported in probe 0's word
+  const Waiter w{&sh->abort_flag, tab.err0, tab.wait_limit_ns};
 
   if (warp == 0) {
-    // fetch the tensor maps of this pair's first tile into the descriptor cache
+    // fetch the operand maps of this pair's first tile into the descriptor cache
     const int pos = group_position(0, pair, num_pairs);
     if (pos < tab.total_tiles && lane < 4) {
       int pi = 0;
-      while (pi + 1 < tab.n && pos >= tab.p[pi + 1].tile_begin) ++pi;
-      asm volatile("prefetch.tensormap [%0];" ::"l"(&tab.p[pi].maps[lane]) : "memory");
+      while (pi + 1 < tab.n && pos >= tab.u[pi + 1].tile_begin) ++pi;
+      const CUtensorMap* m = lane < 2 ? &tab.u[pi].maps[lane] : &tab.v[tab.u[pi].var_begin].maps[lane - 2];
+      asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
     }
   }
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&sh->full[s]), 1);
+      mbar_init(smem_u32(&sh->ready[s]), 2 * 4);          // four converter warps in each CTA
       mbar_init(smem_u32(&sh->empty[s]), 1);
     }
-    for (int s = 0; s < kAbs; ++s) mbar_init(smem_u32(&sh->ready[s]), 2 * 4);   // four converter warps in each CTA
-    mbar_init(smem_u32(&sh->tmem_full), 1);
-    mbar_init(smem_u32(&sh->tmem_empty), 2 * kEpiWarps);
-    mbar_init(smem_u32(&sh->lp_done), 2 * kEpiWarps);
+    mbar_init(smem_u32(&sh->rd_full), 1);
+    mbar_init(smem_u32(&sh->rd_empty), 2 * kEpiWarps);
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(smem_u32(&sh->lp_full[b]), 1);
+      mbar_init(smem_u32(&sh->lp_done[b]), 2 * kEpiWarps);
+    }
+    mbar_init(smem_u32(&sh->abs_free), kEpiWarps);
     mbar_init(smem_u32(&sh->drain), 1);
     sh->abort_flag = 0;
     sh->is_last = 0;
@@ -1306,14 +1377,17 @@ tc_group_kernel(const __grid_constant__ GroupTable tab) {
                      smem_u32(&sh->tmem_base)), "r"(512u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
-  if (warp == 2 && lane < tab.n) {
-    const GroupProblem& pr = tab.p[lane];
-    WalkInfo wi;
-    wi.tile_begin = pr.tile_begin; wi.per_b = pr.a.tiles_m * pr.a.tiles_n;
-    wi.inner = pr.m_fastest ? -pr.a.tiles_m : pr.a.tiles_n;
-    wi.num_kb = (int)((pr.a.K + kBlockK - 1) / kBlockK);
-    wi.half_n = pr.half_n; wi.kind = pr.kind; wi.idesc_ref = pr.idesc_ref; wi.idesc_lp = pr.a.idesc_lp;
-    sh->walk[lane] = wi;
+  if (warp == 2) {
+    for (int i = lane; i < tab.n; i += 32) {
+      const GroupUnit& u = tab.u[i];
+      WalkInfo wi;
+      wi.tile_begin = u.tile_begin; wi.per_b = u.tiles_m * u.tiles_n;
+      wi.inner = u.m_fastest ? -u.tiles_m : u.tiles_n;
+      wi.num_kb = (u.K + kBlockK - 1) / kBlockK;
+      wi.half_n = u.half_n; wi.n_var = u.n_var; wi.var_begin = u.var_begin; wi.K = u.K;
+      sh->walk[i] = wi;
+    }
+    for (int i = lane; i < tab.n_var; i += 32) sh->var[i] = VarInfo{tab.v[i].idesc_lp, tab.v[i].flags};
   }
   tc_fence_before();
   __syncthreads();
@@ -1329,90 +1403,107 @@ tc_group_kernel(const __grid_constant__ GroupTable tab) {
       // ---------------------------------------------------------- TMA producer (both CTAs)
       if (lane == 0) {
         TileWalk tw;
-        tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
-        for (uint32_t g = 0; tw.valid; ++g, tw.next_kb()) {
-          const int s = g % kStages;
-          const uint32_t use = g / kStages;
-          if (g >= tab.stop_after_kb) break;                  // test hook: the consumers' waits run out
-          if (use > 0 && !w.wait(smem_u32(&sh->empty[s]), (use - 1) & 1)) break;
-          const GroupProblem& pr = tab.p[tw.pi];
+        Ring ring;
+        uint32_t g = 0;
+        bool ok = true;
+        auto load = [&](const CUtensorMap* maps, uint32_t bytes, int k0, int r0, int c0, int b) {
+          // test hook: the consumers' waits run out
+          if (g >= tab.stop_after_kb || (g >= (uint32_t)kStages && !w.wait(smem_u32(&sh->empty[ring.s]), ring.parity ^ 1u))) {
+            ok = false;
+            return;
+          }
+          const uint32_t bar = smem_u32(&sh->full[ring.s]), base = tile_base + ring.s * C::kStageBytes;
+          mbar_expect_tx(bar, bytes);
+          tma_load_3d_local(base + C::kOffR, &maps[1], bar, k0, c0, b);     // the converters read this one
+          tma_load_3d_local(base + C::kOffL, &maps[0], bar, k0, r0, b);
+          sh->issued = ++g;
+          ring.next();
+        };
+        for (tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs); tw.valid && ok; tw.next_tile()) {
           const int r0 = tw.tc.m_tile * kPairM + (int)rank * kBlockM;     // this CTA's left-operand rows
           const int c0 = tw.tc.n_tile * kBlockN + (int)rank * tw.half_n;  // this CTA's half of the right operand
-          const uint32_t bar = smem_u32(&sh->full[s]);
-          mbar_expect_tx(bar, kABf16 + kALp + (uint32_t)tw.half_n * (kBlockK * 2 + kBlockK));
-          const uint32_t base = tile_base + s * C::kStageBytes;
-          const int k0 = tw.kb * kBlockK;
-          tma_load_3d_local(base + C::kOffR, &pr.maps[1], bar, k0, c0, tw.tc.b);     // the converters read this one
-          tma_load_3d_local(base + C::kOffL, &pr.maps[0], bar, k0, r0, tw.tc.b);
-          tma_load_3d_local(base + C::kOffCl, &pr.maps[2], bar, k0, r0, tw.tc.b);
-          tma_load_3d_local(base + C::kOffCr, &pr.maps[3], bar, k0, c0, tw.tc.b);
-          sh->issued = g + 1;
+          const uint32_t bytes = kABf16 + (uint32_t)tw.half_n * 128u;
+          for (int kb = 0; kb < tw.num_kb && ok; ++kb) load(tab.u[tw.pi].maps, bytes, kb * kBlockK, r0, c0, tw.tc.b);
+          const int nb = tw.lp_blocks();
+          for (int f = 0; f < tw.n_var && ok; ++f)
+            for (int kb = 0; kb < nb && ok; ++kb) load(tab.v[tw.var_begin + f].maps, bytes, kb * C::kLpDepth, r0, c0, tw.tc.b);
         }
       }
     } else if (warp == 1 && rank == 0) {
       // ---------------------------------------------------------- MMA issuer (leader CTA, converged warp)
       const bool lead = elect_one();
-      uint32_t idesc_bf16 = 0;                 // of the tile in hand
-      auto issue_ref_den = [&](uint32_t gg, int kb) {
-        const uint32_t s = gg % kStages, base = tile_base + s * C::kStageBytes;
-        const uint64_t dl = smem_desc(base + C::kOffL, 128), dr = smem_desc(base + C::kOffR, 128);
-#pragma unroll
-        for (int k = 0; k < kBlockK / 16; ++k)   // 16 bf16 = 32 bytes = 2 descriptor units per step
-          mma_pair<kKindF16>(tmem_base + C::kColRef, dl + 2 * k, dr + 2 * k, idesc_bf16, (kb | k) != 0, lead);
-        const uint64_t da = smem_desc(base + C::kOffRa, 128);
-        const uint32_t ta = tmem_base + C::kColAbsL + 32u * (gg % kAbs);
-#pragma unroll
-        for (int k = 0; k < kBlockK / 16; ++k)   // 16 bf16 = 8 columns of tensor memory per step
-          mma_pair_a_tmem(tmem_base + C::kColDen, ta + 8u * k, da + 2 * k, idesc_bf16, (kb | k) != 0, lead);
-      };
-      auto issue_lp = [&](uint32_t gg, int kb, int kind, uint32_t idesc_lp) {
-        const uint32_t base = tile_base + (gg % kStages) * C::kStageBytes;
-        const uint64_t cl = smem_desc(base + C::kOffCl, 64), cr = smem_desc(base + C::kOffCr, 64);
-#pragma unroll
-        for (int k = 0; k < kBlockK / 32; ++k) {  // 32 codes = 32 bytes per step
-          if (kind == kKindI8) mma_pair<kKindI8>(tmem_base + C::kColLp, cl + 2 * k, cr + 2 * k, idesc_lp, (kb | k) != 0, lead);
-          else mma_pair<kKindF8>(tmem_base + C::kColLp, cl + 2 * k, cr + 2 * k, idesc_lp, (kb | k) != 0, lead);
-        }
-      };
-      auto wait_stage = [&](uint32_t gg) {
-        if (!w.wait_warp(smem_u32(&sh->ready[gg % kAbs]), (gg / kAbs) & 1)) return false;
+      TileWalk tw;
+      Ring ring;
+      auto wait_block = [&]() {
+        if (!w.wait_warp(smem_u32(&sh->ready[ring.s]), ring.parity)) return false;
         tc_fence_after();
         return true;
       };
-      TileWalk tw;
-      tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
-      uint32_t g = 0;
+      // One elected lane issues a block's MMAs and the commit that frees the block in both CTAs.
+      auto issue_rd = [&](uint32_t base, int kb, uint32_t idesc, uint32_t empty_bar) {
+        const uint64_t dr = smem_desc(base + C::kOffR, 128), da = smem_desc(base + C::kOffRa, 128);
+        const uint32_t ta = tmem_base + C::kColL + 64u * (kb & (kTmemStages - 1));
+        if (lead) {
+#pragma unroll
+          for (int k = 0; k < kBlockK / 16; ++k)   // 16 bf16 = 32 bytes = 2 descriptor units = 8 columns of tensor memory per step
+            mma_pair_a_tmem(tmem_base + C::kColRef, ta + 8u * k, dr + 2 * k, idesc, k ? 1u : (uint32_t)kb, true);
+#pragma unroll
+          for (int k = 0; k < kBlockK / 16; ++k)
+            mma_pair_a_tmem(tmem_base + C::kColDen, ta + 32u + 8u * k, da + 2 * k, idesc, k ? 1u : (uint32_t)kb, true);
+          tc_commit_pair(empty_bar, true);
+        }
+      };
+      auto issue_lp = [&](auto kind, uint32_t base, uint32_t td, int kb, int steps, uint32_t idesc, uint32_t empty_bar) {
+        const uint64_t cl = smem_desc(base + C::kOffL, 128), cr = smem_desc(base + C::kOffR, 128);
+        if (lead) {
+#pragma unroll
+          for (int k = 0; k < C::kLpDepth / 32; ++k)
+            if (k < steps) mma_pair<decltype(kind)::value>(td, cl + 2 * k, cr + 2 * k, idesc, k ? 1u : (uint32_t)kb, true);
+          tc_commit_pair(empty_bar, true);
+        }
+      };
+      uint32_t lp_uses0 = 0, lp_uses1 = 0;           // variants put into each 8-bit accumulator so far
       bool ok = true;
-      for (uint32_t it = 0; tw.valid && ok; ++it, tw.next_tile()) {
-        const WalkInfo& wi = sh->walk[tw.pi];
-        const int num_kb = tw.num_kb, kind = wi.kind;
-        const uint32_t idesc_lp = wi.idesc_lp;
-        idesc_bf16 = wi.idesc_ref;
+      uint32_t it = 0;
+      for (tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs); tw.valid && ok; ++it, tw.next_tile()) {
         // the reference and denominator blocks come back when both epilogues have copied the
-        // previous tile's values out; the 8-bit block when they have finished that tile
-        if (it > 0 && !w.wait_warp(smem_u32(&sh->tmem_empty), (it - 1) & 1)) break;
+        // previous tile's values out
+        if (it > 0 && !w.wait_warp(smem_u32(&sh->rd_empty), (it - 1) & 1)) break;
         tc_fence_after();
-        const int n_ahead = num_kb < kAbs ? num_kb : kAbs;
-        for (int j = 0; j < n_ahead && ok; ++j) {
-          ok = wait_stage(g + j);
-          if (ok) issue_ref_den(g + j, j);
+        tw.make_uniform();
+        const uint32_t idesc_ref = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n);
+        for (int kb = 0; kb < tw.num_kb; ++kb) {
+          ok = wait_block();
+          if (!ok) break;
+          issue_rd(tile_base + ring.s * C::kStageBytes, kb, idesc_ref, smem_u32(&sh->empty[ring.s]));
+          ring.next();
         }
         if (!ok) break;
-        if (it > 0 && !w.wait_warp(smem_u32(&sh->lp_done), (it - 1) & 1)) break;
-        tc_fence_after();
-        int kb = 0;
-        for (; kb < n_ahead; ++kb, ++g) {
-          issue_lp(g, kb, kind, idesc_lp);
-          tc_commit_pair(smem_u32(&sh->empty[g % kStages]), lead);
+        tc_commit_pair(smem_u32(&sh->rd_full), lead);
+        const int nb = tw.lp_blocks();
+        for (int f = 0; f < tw.n_var && ok; ++f) {
+          const int b = (tw.n_var - 1 - f) & 1;
+          const uint32_t idesc = __shfl_sync(0xffffffffu, sh->var[tw.var_begin + f].idesc, 0);
+          const bool is_i8 = __shfl_sync(0xffffffffu, sh->var[tw.var_begin + f].flags, 0) & kVarI8;
+          // both epilogues have read what this accumulator held; the second one's columns have also
+          // been this tile's L, which the denominator MMAs must have finished with
+          const uint32_t uses = b ? lp_uses1 : lp_uses0;
+          ok = uses == 0 || w.wait_warp(smem_u32(&sh->lp_done[b]), (uses - 1) & 1);
+          if (ok && b == 1) ok = w.wait_warp(smem_u32(&sh->rd_full), it & 1);
+          tc_fence_after();
+          const uint32_t td = tmem_base + C::kColLp + 128u * b;
+          for (int kb = 0; kb < nb && ok; ++kb) {
+            ok = wait_block();
+            if (!ok) break;
+            const int steps = (tw.K - kb * C::kLpDepth + 31) / 32;          // of 32 codes; the rest of the block is fill
+            const uint32_t base = tile_base + ring.s * C::kStageBytes, bar = smem_u32(&sh->empty[ring.s]);
+            if (is_i8) issue_lp(std::integral_constant<int, kKindI8>{}, base, td, kb, steps, idesc, bar);
+            else issue_lp(std::integral_constant<int, kKindF8>{}, base, td, kb, steps, idesc, bar);
+            ring.next();
+          }
+          if (ok) tc_commit_pair(smem_u32(&sh->lp_full[b]), lead);
+          if (b) ++lp_uses1; else ++lp_uses0;
         }
-        for (; kb < num_kb && ok; ++kb, ++g) {
-          ok = wait_stage(g);
-          if (!ok) break;
-          issue_ref_den(g, kb);
-          issue_lp(g, kb, kind, idesc_lp);
-          tc_commit_pair(smem_u32(&sh->empty[g % kStages]), lead);        // frees the k-block in both CTAs
-        }
-        if (ok) tc_commit_pair(smem_u32(&sh->tmem_full), lead);           // this tile's accumulators are complete
       }
     }
   } else if (warp < kFirstEpiWarp) {
@@ -1421,199 +1512,276 @@ tc_group_kernel(const __grid_constant__ GroupTable tab) {
     // Thread t of the four warps owns row t of this CTA's 128 left-operand rows (its warp's
     // tensor-memory lane quarter holds that row): once the stage has landed it reads its row of the
     // L tile from shared memory (128-byte swizzle: 16-byte chunk c of row r sits at c ^ (r & 7),
-    // which makes these row-per-thread reads conflict-free), clears the sign bits and stores the
-    // 32 words into the stage's tensor-memory columns.  (Loading the rows with plain global loads
+    // which makes these row-per-thread reads conflict-free) and stores the 32 words, and the same with
+    // the sign bits cleared, into the stage's tensor-memory columns.  (Loading the rows with plain global loads
     // instead, to spare shared memory the 16 KB, was tried: a warp then touches 32 lines per
     // instruction and the converters became the bottleneck, 1.6 x slower overall.)  The |R|
     // half-tile is a flat sign-cleared copy of the R half-tile (8 KB: four vectors per thread).
     const int q = warp & 3;
     const int t = q * 32 + lane;                   // 0..127
     const uint32_t ready_leader = map_to_cta(smem_u32(&sh->ready[0]), 0);
-    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + C::kColAbsL;
-    const uint32_t row_off = (uint32_t)t * 128u, sw = (uint32_t)t & 7u;
+    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + C::kColL;
+    const uint32_t row_off = (uint32_t)t * 128u, sw = (uint32_t)t & 7u, m = 0x7fff7fffu;
     TileWalk tw;
-    tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
+    Ring ring;
+    uint32_t it = 0, abs_uses = 0;                 // completions of abs_free awaited so far
+    bool lent = false;                             // the previous tile's variants have used the L columns
     bool ok = true;
-    for (uint32_t g = 0; ok && tw.valid; ++g, tw.next_kb()) {
-      const uint32_t s = g % kStages, sa = g % kAbs, m = 0x7fff7fffu;
-      // the tensor-memory columns were last read by the MMAs of k-block g - kAbs (its commit also
-      // covers every earlier k-block, so the |R| slot of the stage is free as well)
-      if (g >= (uint32_t)kAbs) {
-        const uint32_t gp = g - kAbs;
-        if (!w.wait_warp(smem_u32(&sh->empty[gp % kStages]), (gp / kStages) & 1)) { ok = false; break; }
-      }
-      if (!w.wait_warp(smem_u32(&sh->full[s]), (g / kStages) & 1)) { ok = false; break; }
-      tc_fence_after();
-      const uint32_t base = tile_base + s * C::kStageBytes;
-      uint4 v[8], u[4];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = lds128(base + C::kOffL + row_off + (((uint32_t)j ^ sw) << 4));
-      const uint32_t rsrc = base + C::kOffR + (uint32_t)t * 16u;
+    for (tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs); tw.valid && ok; ++it, tw.next_tile()) {
+      // the L columns are free once the previous tile's denominator is complete and whatever
+      // variants it put there have been read
+      if (it > 0) ok = w.wait_warp(smem_u32(&sh->rd_full), (it - 1) & 1);
+      if (ok && lent) ok = w.wait_warp(smem_u32(&sh->abs_free), abs_uses++ & 1);
+      lent = tw.n_var > 1;
       const int r_vec = tw.half_n * 8;                           // 16-byte vectors of the R half-tile that are in use
+      for (int kb = 0; kb < tw.num_kb && ok; ++kb) {
+        const uint32_t s = ring.s;
+        ok = w.wait_warp(smem_u32(&sh->full[s]), ring.parity);
+        if (!ok) break;
+        const uint32_t base = tile_base + s * C::kStageBytes;
+        uint4 v[8], u[4];
+        const uint32_t rsrc = base + C::kOffR + (uint32_t)t * 16u;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) u[j] = t + 128 * j < r_vec ? lds128(rsrc + (uint32_t)j * 2048u) : make_uint4(0u, 0u, 0u, 0u);
-      uint32_t a[32];
+        for (int j = 0; j < 4; ++j) u[j] = t + 128 * j < r_vec ? lds128(rsrc + (uint32_t)j * 2048u) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        a[4 * j] = v[j].x & m; a[4 * j + 1] = v[j].y & m; a[4 * j + 2] = v[j].z & m; a[4 * j + 3] = v[j].w & m;
+        for (int j = 0; j < 8; ++j) v[j] = lds128(base + C::kOffL + row_off + (((uint32_t)j ^ sw) << 4));
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (t + 128 * j < r_vec)
+            sts128(rsrc + (C::kOffRa - C::kOffR) + (uint32_t)j * 2048u, make_uint4(u[j].x & m, u[j].y & m, u[j].z & m, u[j].w & m));
+        uint32_t a[32];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) { a[4 * j] = v[j].x; a[4 * j + 1] = v[j].y; a[4 * j + 2] = v[j].z; a[4 * j + 3] = v[j].w; }
+        if (kb >= kTmemStages) {
+          // the tensor-memory columns were last read by the MMAs of the block kTmemStages before this one
+          const uint32_t sp = s >= (uint32_t)kTmemStages ? s - kTmemStages : s + kStages - kTmemStages;
+          const uint32_t pp = s >= (uint32_t)kTmemStages ? ring.parity : ring.parity ^ 1u;
+          ok = w.wait_warp(smem_u32(&sh->empty[sp]), pp);
+          if (!ok) break;
+        }
+        tc_fence_after();
+        const uint32_t tcol = taddr + 64u * (uint32_t)(kb & (kTmemStages - 1));
+        tmem_st32(tcol, a);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) a[j] &= m;
+        tmem_st32(tcol + 32u, a);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // generic-proxy writes -> the tensor core's reads
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(ready_leader + s * 8u);
+        ring.next();
       }
-      tmem_st32(taddr + 32u * sa, a);
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (t + 128 * j < r_vec)
-          sts128(rsrc + (C::kOffRa - C::kOffR) + (uint32_t)j * 2048u, make_uint4(u[j].x & m, u[j].y & m, u[j].z & m, u[j].w & m));
-      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // generic-proxy writes -> the tensor core's reads
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(ready_leader + sa * 8u);
+      // blocks of codes: only passed on
+      const int n_code_blocks = tw.n_var * tw.lp_blocks();
+      for (int kb = 0; kb < n_code_blocks && ok; ++kb) {
+        ok = w.wait_warp(smem_u32(&sh->full[ring.s]), ring.parity);
+        if (!ok) break;
+        if (lane == 0) mbar_arrive_cluster(ready_leader + ring.s * 8u);
+        ring.next();
+      }
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
     // ------------------------------------------------------------ epilogue (warps 8..15, both CTAs)
     // A warp may touch the tensor-memory lane quarter warp % 4; the two warps of a quarter split
-    // the columns.  Copy this warp's 64 columns of the reference and denominator blocks into
-    // registers, hand those two blocks back to the MMA lane, then walk the 8-bit block in chunks
-    // of 16 columns; the statistics arithmetic runs under the next tile's main loop.
+    // the columns.
     const int q = warp & 3;
     const int ew = warp - kFirstEpiWarp;           // 0..7
     const int h = ew >> 2;                         // which half of the tile's columns
     const int et = ew * 32 + lane;                 // 0..255
-    const uint32_t tmem_empty_leader = map_to_cta(smem_u32(&sh->tmem_empty), 0);
-    double acc[5] = {0, 0, 0, 0, 0};               // of the probe in hand: sum BE, max BE, sum diff^2, C^2, D^2
-    int cur = -1;                                  // the probe in hand
-    // reduce the statistics of probe `pi` over the CTA and write its record (all 256 threads call)
+    const uint32_t rd_empty_leader = map_to_cta(smem_u32(&sh->rd_empty), 0);
+    const uint32_t lp_done_leader = map_to_cta(smem_u32(&sh->lp_done[0]), 0);
+    double acc_r2 = 0.0, acc_n2 = 0.0;             // of the unit in hand: sum C^2, D^2 of this thread's rows
+    int cur = -1;                                  // the unit in hand
+    // reduce the statistics of unit `pi` over the CTA and write its records (all 256 threads call)
     auto flush = [&](int pi) {
-#pragma unroll
-      for (int i = 0; i < 5; ++i) {
-        double x = acc[i];
+      const int nv = sh->walk[pi].n_var, v0 = sh->walk[pi].var_begin;
+      for (int i = 0; i < 3 * nv + 2; ++i) {
+        // values 3v, 3v + 1, 3v + 2: sum BE, max BE, sum diff^2 of variant v; the last two: sum C^2, D^2
+        const int v = i / 3, k = i - 3 * v;
+        double x = 0.0;
+        if (i >= 3 * nv) x = i == 3 * nv ? acc_r2 : acc_n2;
+        else if (lane < 16) x = k == 1 ? (double)sh->maxima[v][ew][lane] : (k == 0 ? sh->sums[v][ew][lane].x : sh->sums[v][ew][lane].y);
+        const bool is_max = i < 3 * nv && k == 1;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
           const double y = __shfl_xor_sync(0xffffffffu, x, o);
-          x = i == 1 ? fmax(x, y) : x + y;
+          x = is_max ? fmax(x, y) : x + y;
         }
         if (lane == 0) sh->red[i][ew] = x;
-        acc[i] = 0.0;
       }
+      acc_r2 = acc_n2 = 0.0;
       asm volatile("bar.sync 1, 256;" ::: "memory");
-      if (et < 5) {
+      if (et < 5 * nv) {
+        const int v = et / 5, k = et - 5 * v;
+        const int i = k < 3 ? 3 * v + k : 3 * nv + (k - 3);
         double x = 0.0;
-        for (int k = 0; k < kEpiWarps; ++k) x = et == 1 ? fmax(x, sh->red[et][k]) : x + sh->red[et][k];
-        __stcg(tab.p[pi].a.partials + (int64_t)blockIdx.x * kPartialDoubles + et, x);
+        for (int j = 0; j < kEpiWarps; ++j) x = k == 1 ? fmax(x, sh->red[i][j]) : x + sh->red[i][j];
+        __stcg(tab.v[v0 + v].partials + (int64_t)blockIdx.x * kPartialDoubles + k, x);
         __threadfence();
       }
       asm volatile("bar.sync 1, 256;" ::: "memory");       // red[] may be reused
     };
-    uint32_t met = 0;                              // bit pi: this CTA has had tiles of probe pi
-    // of the probe in hand (reloaded when the probe changes, not per tile)
-    bool per_col = false, pc_l = false, is_i8 = false, narrow = false;
-    float dr_tensor = 1.f, dl_tensor = 0.f;
-    int pM = 0, pN = 0;                            // a probe's M and N are below 2^31 (its tensor maps require it)
+    uint32_t met = 0;                              // bit pi: this CTA has had tiles of unit pi
+    int pM = 0, pN = 0;                            // of the unit in hand; below 2^31 (its tensor maps require it)
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+    uint32_t lp_parity = 0;                        // bit b: parity of the next use of 8-bit accumulator b
+    bool dead = false;                             // a wait for an 8-bit accumulator ran out
     TileWalk tw;
     tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
     for (uint32_t it = 0; tw.valid; ++it) {
-      const int pi = tw.pi;
+      const int pi = tw.pi, n_var = tw.n_var, v0 = tw.var_begin;
       if (pi != cur) {
         if (cur >= 0) flush(cur);
         cur = pi;
         met |= 1u << pi;
-        const GroupProblem& pr = tab.p[pi];
-        per_col = pr.a.pc_r != 0; pc_l = pr.a.pc_l != 0; is_i8 = pr.kind == kKindI8; narrow = pr.half_n < 64;
-        pM = (int)pr.a.M; pN = (int)pr.a.N;
-        dr_tensor = per_col ? 1.f : __ldg(pr.a.dr);
-        dl_tensor = pc_l ? 0.f : __ldg(pr.a.dl);
+        pM = tab.u[pi].M; pN = tab.u[pi].N;
+        for (int v = 0; v < n_var; ++v)
+          if (lane < 16) { sh->sums[v][ew][lane] = make_double2(0.0, 0.0); sh->maxima[v][ew][lane] = 0.f; }
+        if (et < n_var) {                           // read after the barrier below
+          const GroupVar& gv = tab.v[v0 + et];
+          sh->dl_tensor[et] = gv.flags & kVarScalePerRow ? 1.f : __ldg(gv.dl);
+          sh->dr_tensor[et] = gv.flags & kVarScalePerCol ? 1.f : __ldg(gv.dr);
+        }
       }
       const TileCoord tc = tw.tc;
-      float* dr_s = sh->delta_r[it & 1];
-      if (per_col && et < kBlockN) {
-        const int col = tc.n_tile * kBlockN + et;
-        dr_s[et] = col < pN ? __ldg(tab.p[pi].a.dr + (int64_t)tc.b * pN + col) : 0.f;
+      for (int v = 0; v < n_var; ++v) {
+        if ((sh->var[v0 + v].flags & kVarScalePerCol) && et < kBlockN) {
+          const int col = tc.n_tile * kBlockN + et;
+          sh->delta_r[it & 1][v][et] = col < pN ? __ldg(tab.v[v0 + v].dr + (int64_t)tc.b * pN + col) : 0.f;
+        }
       }
       const int row = tc.m_tile * kPairM + (int)rank * kBlockM + q * 32 + lane;
       const bool row_ok = row < pM;
-      float dlv = dl_tensor;
-      if (pc_l) dlv = row_ok ? __ldg(tab.p[pi].a.dl + (int64_t)tc.b * pM + row) : 0.f;
       // the two warps of a lane quarter split the tile's columns: 64 each, or 32 each where the
       // tile is 64 wide (outputs at most 64 wide)
+      const bool narrow = tw.half_n < 64;
       const int cw = narrow ? 32 : 64, cbase = h * cw;
       const int colw = tc.n_tile * kBlockN + cbase;                  // first column of this warp
+      const int live = pN - colw < cw ? pN - colw : cw;              // its columns that exist; <= 0: none
 
-      const bool ok = w.wait(smem_u32(&sh->tmem_full), it & 1);
-      // one barrier publishes delta_r and makes the give-up decision uniform over the epilogue
+      const bool ok = !dead && w.wait(smem_u32(&sh->rd_full), it & 1);
+      // one barrier publishes the scales and makes the give-up decision uniform over the epilogue
       if (epi_barrier_any(!ok)) break;
       tc_fence_after();
-      // live = columns of this warp that exist in the matrix
-      const int live = pN - colw < cw ? pN - colw : cw;          // <= 0: none
-      const uint32_t lp_addr = lane_addr + C::kColLp + cbase;
-      const uint32_t lp_done_leader = map_to_cta(smem_u32(&sh->lp_done), 0);
-      const float* const drc = dr_s + cbase;
-      uint32_t rc[64], rd[64], rq0[16];
+      uint32_t rc[64], rd[64];
       tmem_ld32(lane_addr + C::kColRef + cbase, *reinterpret_cast<uint32_t(*)[32]>(&rc[0]));
       tmem_ld32(lane_addr + C::kColDen + cbase, *reinterpret_cast<uint32_t(*)[32]>(&rd[0]));
       if (!narrow) {
         tmem_ld32(lane_addr + C::kColRef + cbase + 32, *reinterpret_cast<uint32_t(*)[32]>(&rc[32]));
         tmem_ld32(lane_addr + C::kColDen + cbase + 32, *reinterpret_cast<uint32_t(*)[32]>(&rd[32]));
       }
-      if (live > 0) tmem_ld16(lp_addr, rq0);
       tmem_ld_wait();
-      // The reference and denominator blocks are in registers: the MMA lane may start the next
-      // tile's bf16 MMAs.  The 8-bit block follows in two steps, its first 16 columns with the
-      // loads above and the rest once the first chunk has been evaluated (which frees the
-      // registers the rest is read into); then the MMA lane may start the next tile's 8-bit MMAs as well, while the
-      // remaining chunks are still being evaluated.  Every warp arrives on each barrier exactly
-      // once per tile.
+      // in registers: the MMA warp may start the next tile's reference and denominator as soon as
+      // it is through with this tile's variants
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) {
-        mbar_arrive_cluster(tmem_empty_leader);
-        if (live <= 16) mbar_arrive_cluster(lp_done_leader);      // nothing further to read
-      }
-      StatsG st{0.f, 0.f, 0ull, 0ull, 0ull, 0.f};
-      const float kd = -dlv * dr_tensor;
-      const uint64_t kd2 = per_col ? pack2(-dlv, -dlv) : pack2(kd, kd);
-      if (live > 0) stats_chunk<0>(rc, rd, rq0, live, is_i8, per_col, kd2, drc, st);
-      if (live > 16) {
-        // chunk 1 into the first chunk's registers, chunks 2 and 3 into those of the first
-        // chunk's reference and denominator values
-        uint32_t(&rq2)[16] = *reinterpret_cast<uint32_t(*)[16]>(&rc[0]);
-        uint32_t(&rq3)[16] = *reinterpret_cast<uint32_t(*)[16]>(&rd[0]);
-        tmem_ld16(lp_addr + 16, rq0);
-        if (live > 32) tmem_ld16(lp_addr + 32, rq2);
-        if (live > 48) tmem_ld16(lp_addr + 48, rq3);
-        tmem_ld_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(lp_done_leader);
-        stats_chunk<1>(rc, rd, rq0, live - 16, is_i8, per_col, kd2, drc, st);
-        if (live > 32) stats_chunk<2>(rc, rd, rq2, live - 32, is_i8, per_col, kd2, drc, st);
-        if (live > 48) stats_chunk<3>(rc, rd, rq3, live - 48, is_i8, per_col, kd2, drc, st);
-      }
-      if (row_ok) {
+      if (lane == 0) mbar_arrive_cluster(rd_empty_leader);
+      // sums of C^2 and D^2, and D replaced by its reciprocal (all under the first 8-bit product).
+      // D == 0 implies C == Q == 0, so clamping the divisor keeps BE = 0 there without a branch.
+      {
+        uint64_t r22 = 0ull, n22 = 0ull;
+        auto prepare = [&](int j0) {
+#pragma unroll
+          for (int j = 0; j < 32; j += 2) {
+            const uint64_t cv2 = pack2(__uint_as_float(rc[j0 + j]), __uint_as_float(rc[j0 + j + 1]));
+            const float d0 = __uint_as_float(rd[j0 + j]), d1 = __uint_as_float(rd[j0 + j + 1]);
+            const uint64_t dd2 = pack2(d0, d1);
+            r22 = fma2(cv2, cv2, r22);
+            n22 = fma2(dd2, dd2, n22);
+            rd[j0 + j] = __float_as_uint(rcp_approx(fmaxf(d0, 1e-37f)));
+            rd[j0 + j + 1] = __float_as_uint(rcp_approx(fmaxf(d1, 1e-37f)));
+          }
+        };
+        if (live < cw) {                                 // ragged edge: columns beyond the matrix count as zeros
+#pragma unroll
+          for (int k = 0; k < 64; ++k)
+            if (k >= live) { rc[k] = 0u; rd[k] = 0u; }
+        }
+        prepare(0);
+        if (!narrow) prepare(32);
         float x0, x1;
-        acc[0] += (double)st.be0 + (double)st.be1;
-        unpack2(st.d2, x0, x1); acc[2] += (double)x0 + (double)x1;
-        unpack2(st.r2, x0, x1); acc[3] += (double)x0 + (double)x1;
-        unpack2(st.n2, x0, x1); acc[4] += (double)x0 + (double)x1;
-        acc[1] = fmax(acc[1], (double)st.mx);
-        double* const rows = tab.p[pi].a.row_stats;
-        if (rows) row_stats_add(rows + ((int64_t)tc.b * pM + row) * 5, st);
+        unpack2(r22, x0, x1);
+        const double r2d = (double)x0 + (double)x1;
+        unpack2(n22, x0, x1);
+        const double n2d = (double)x0 + (double)x1;
+        if (row_ok) {
+          acc_r2 += r2d;
+          acc_n2 += n2d;
+          for (int v = 0; v < n_var; ++v) {
+            if (!(sh->var[v0 + v].flags & kVarRowStats)) continue;       // the optional per-row check output
+            double* const rs = tab.v[v0 + v].row_stats + ((int64_t)tc.b * pM + row) * 5;
+            atomicAdd(rs + 3, r2d);
+            atomicAdd(rs + 4, n2d);
+          }
+        }
+      }
+      for (int f = 0; f < n_var; ++f) {
+        const int b = (n_var - 1 - f) & 1;
+        const uint32_t flags = sh->var[v0 + f].flags;
+        const bool per_col = (flags & kVarScalePerCol) != 0, is_i8 = (flags & kVarI8) != 0;
+        float dlv = sh->dl_tensor[f];
+        if (flags & kVarScalePerRow) dlv = row_ok ? __ldg(tab.v[v0 + f].dl + (int64_t)tc.b * pM + row) : 0.f;
+        const float kd = per_col ? -dlv : -dlv * sh->dr_tensor[f];
+        if (!w.wait_warp(smem_u32(&sh->lp_full[b]), (lp_parity >> b) & 1u)) { dead = true; break; }
+        lp_parity ^= 1u << b;
+        tc_fence_after();
+        const uint32_t taddr = lane_addr + C::kColLp + 128u * b + cbase;
+        StatsV st{0.f, 0.f, 0.f, 0ull};
+        auto release = [&]() {
+          // read to the end: the MMA warp may overwrite it and, after the tile's last use of the second
+          // accumulator (once per tile, or the converters' wait could miss a phase of the barrier), this
+          // CTA's converters may.  Every warp arrives exactly once per use.
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) {
+            mbar_arrive_cluster(lp_done_leader + 8u * b);
+            if (f == n_var - 2) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&sh->abs_free)) : "memory");
+          }
+        };
+        if (per_col) eval_variant<true>(taddr, rc, rd, live, is_i8, pack2(kd, kd), sh->delta_r[it & 1][f] + cbase, st, release);
+        else eval_variant<false>(taddr, rc, rd, live, is_i8, pack2(kd, kd), sh->delta_r[0][0], st, release);
+        double be = 0.0, d2 = 0.0;
+        float mx = 0.f;
+        if (row_ok) {
+          float x0, x1;
+          unpack2(st.d2, x0, x1);
+          be = (double)st.be0 + (double)st.be1;
+          d2 = (double)x0 + (double)x1;
+          mx = st.mx;
+          if (flags & kVarRowStats) {
+            double* const rs = tab.v[v0 + f].row_stats + ((int64_t)tc.b * pM + row) * 5;
+            atomicAdd(rs + 0, be);
+            atomicMax(reinterpret_cast<unsigned long long*>(rs + 1), (unsigned long long)__double_as_longlong((double)mx));
+            atomicAdd(rs + 2, d2);
+          }
+        }
+        be += __shfl_xor_sync(0xffffffffu, be, 16);
+        d2 += __shfl_xor_sync(0xffffffffu, d2, 16);
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+        if (lane < 16) {
+          double2& a = sh->sums[f][ew][lane];
+          a.x += be;
+          a.y += d2;
+          sh->maxima[f][ew][lane] = fmaxf(sh->maxima[f][ew][lane], mx);
+        }
       }
       tw.next_tile();
     }
     if (cur >= 0) flush(cur);
     // the records of the probes this CTA never met are zero
-    if (et == 0) {
-      for (int pi = 0; pi < tab.n; ++pi) {
-        if (met & (1u << pi)) continue;
-        double* rec = tab.p[pi].a.partials + (int64_t)blockIdx.x * kPartialDoubles;
-        for (int i = 0; i < 5; ++i) __stcg(rec + i, 0.0);
-      }
+    for (int pi = 0; pi < tab.n; ++pi) {
+      if (met & (1u << pi)) continue;
+      const int v0 = sh->walk[pi].var_begin;
+      if (et < 5 * sh->walk[pi].n_var)
+        __stcg(tab.v[v0 + et / 5].partials + (int64_t)blockIdx.x * kPartialDoubles + et % 5, 0.0);
     }
+    __threadfence();
     asm volatile("bar.sync 1, 256;" ::: "memory");
     if (et == 0) {
       __threadfence();
-      const uint32_t prev = atomicAdd(tab.p[0].a.done_counter, 1u);
+      const uint32_t prev = atomicAdd(tab.done_counter, 1u);
       sh->is_last = prev == gridDim.x - 1 ? 1u : 0u;
     }
     asm volatile("bar.sync 1, 256;" ::: "memory");
@@ -1621,10 +1789,9 @@ tc_group_kernel(const __grid_constant__ GroupTable tab) {
       // last CTA: every record of every probe is visible; each epilogue warp takes probes
       // ew, ew + 8, ...; fixed-order sum (lane l takes records l, l+32, ...)
       __threadfence();
-      uint32_t* const err0 = tab.p[0].a.err_word;
-      const uint32_t timed_out = err0 ? (*reinterpret_cast<volatile uint32_t*>(err0) & QM_DEVERR_TIMEOUT) : 0u;
-      for (int pi = ew; pi < tab.n; pi += kEpiWarps) {
-        const KernelArgs& a = tab.p[pi].a;
+      const uint32_t timed_out = tab.err0 ? (*reinterpret_cast<volatile uint32_t*>(tab.err0) & QM_DEVERR_TIMEOUT) : 0u;
+      for (int vi = ew; vi < tab.n_var; vi += kEpiWarps) {
+        const GroupVar& a = tab.v[vi];
         double s5[5] = {0, 0, 0, 0, 0};
         for (int i = lane; i < (int)gridDim.x; i += 32) {
           const double* rec = a.partials + (int64_t)i * kPartialDoubles;
@@ -1847,39 +2014,48 @@ qm_status launch_wide(const CUtensorMap& ma, const CUtensorMap& mb, KernelArgs k
 
 }  // namespace
 
-int tc_group_max() { return kMaxGroup; }
-
 namespace {
-constexpr size_t kProbeSmem = (size_t)CfgP::kTileBytes + sizeof(SharedP) + 1024;
+template <typename Table>
+constexpr size_t probe_smem() { return (size_t)CfgP::kTileBytes + sizeof(SharedP<Table::kUnits, Table::kVars>) + 1024; }
 
 // Bound of the fused kernels' barrier waits and the producer's test hook (see qm_debug_* in qm.h).
 std::atomic<uint64_t> g_wait_limit_ns{1000000000ull};
 std::atomic<uint32_t> g_stop_after_kb{0xffffffffu};
+
+template <typename Table>
+qm_status probe_kernel_ready() {
+  static bool attr_done[kMaxDevices] = {};
+  const int dev = current_device();
+  if (dev < 0) return QM_ERR_UNSUPPORTED;
+  if (!attr_done[dev]) {
+    // the kernel re-divides the registers its block was launched with (setmaxnreg): refuse to
+    // launch if the compiler gave it fewer than the split adds up to, because an increase that
+    // cannot be served waits forever
+    cudaFuncAttributes fa{};
+    QM_CUDA_OK(cudaFuncGetAttributes(&fa, tc_group_kernel<Table>));
+    if (fa.numRegs * 4 < kRegsCtl + kRegsConv + 2 * kRegsEpi) return QM_ERR_UNSUPPORTED;
+  }
+  return allow_smem(tc_group_kernel<Table>, probe_smem<Table>(), attr_done);
+}
 
 // CTA pairs of the fused probe kernel that can be resident at once (its footprint is the largest
 // of all modes, so its residency bounds every grid); queried once per device.
 qm_status probe_residency() {
   const int dev = current_device();
   if (dev < 0) return QM_ERR_UNSUPPORTED;
-  static bool attr_done[kMaxDevices] = {};
-  const qm_status as = allow_smem(tc_group_kernel, kProbeSmem, attr_done);
+  qm_status as = probe_kernel_ready<TableBig>();
+  if (as == QM_OK) as = probe_kernel_ready<TableOne>();
   if (as != QM_OK) return as;
   if (g_max_pairs[dev] == 0) {
-    // the kernel re-divides the registers its block was launched with (setmaxnreg): refuse to
-    // launch if the compiler gave it fewer than the split adds up to, because an increase that
-    // cannot be served waits forever
-    cudaFuncAttributes fa{};
-    QM_CUDA_OK(cudaFuncGetAttributes(&fa, tc_group_kernel));
-    if (fa.numRegs * 4 < kRegsCtl + kRegsConv + 2 * kRegsEpi) return QM_ERR_UNSUPPORTED;
     cudaLaunchConfig_t q{};
     q.gridDim = dim3((unsigned)(2 * (sm_count() / 2))); q.blockDim = dim3(kProbeThreads);
-    q.dynamicSmemBytes = kProbeSmem;
+    q.dynamicSmemBytes = probe_smem<TableBig>();
     cudaLaunchAttribute qa[1];
     qa[0].id = cudaLaunchAttributeClusterDimension;
     qa[0].val.clusterDim.x = 2; qa[0].val.clusterDim.y = 1; qa[0].val.clusterDim.z = 1;
     q.attrs = qa; q.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tc_group_kernel, &q) == cudaSuccess && n > 0)
+    if (cudaOccupancyMaxActiveClusters(&n, tc_group_kernel<TableBig>, &q) == cudaSuccess && n > 0)
       g_max_pairs[dev] = n < sm_count() / 2 ? n : sm_count() / 2;
     else
       g_max_pairs[dev] = sm_count() / 2;
@@ -1887,69 +2063,77 @@ qm_status probe_residency() {
   }
   return QM_OK;
 }
-}  // namespace
 
-void set_wait_limit_ns(uint64_t ns) { g_wait_limit_ns.store(ns ? ns : 1000000000ull); }
-void set_stop_after_kb(uint32_t kb) { g_stop_after_kb.store(kb); }
+// The probes of one unit, by their index in the caller's list.
+struct UnitPlan {
+  GemmShape g;
+  int n_var;
+  int probe[kMaxVar];
+};
 
-qm_status launch_tc_probe_group(const TcProbeArgs* ps, int n, cudaStream_t s) {
-  if (n < 1 || n > kMaxGroup) return QM_ERR_INVALID_ARG;
-  // descending contraction length = descending tile cost
-  int order[kMaxGroup];
-  for (int i = 0; i < n; ++i) order[i] = i;
-  for (int i = 1; i < n; ++i)
-    for (int j = i; j > 0 && ps[order[j]].g.K > ps[order[j - 1]].g.K; --j) {
-      const int t = order[j]; order[j] = order[j - 1]; order[j - 1] = t;
-    }
-  static GroupTable tab;               // 11 KB: kept off the stack; guarded by the mutex below
+bool same_products(const TcProbeArgs& a, const TcProbeArgs& b) {
+  return a.l == b.l && a.l_ld == b.l_ld && a.l_sb == b.l_sb && a.r == b.r && a.r_ld == b.r_ld && a.r_sb == b.r_sb &&
+         a.g.M == b.g.M && a.g.N == b.g.N && a.g.K == b.g.K && a.g.batch == b.g.batch;
+}
+
+template <typename Table>
+qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, cudaStream_t s) {
+  static Table tab;                    // up to 29 KB: kept off the stack; guarded by the mutex below
   static std::mutex mu;
   std::lock_guard<std::mutex> lock(mu);
+  const TcProbeArgs& first = ps[units[0].probe[0]];
   tab.n = n;
+  tab.n_var = 0;
   tab.wait_limit_ns = g_wait_limit_ns.load();
   tab.stop_after_kb = g_stop_after_kb.load();
+  tab.done_counter = first.done_counter;
+  tab.err0 = first.err_word;
   int64_t total = 0;
   for (int k = 0; k < n; ++k) {
-    const TcProbeArgs& p = ps[order[k]];
-    if (!shape_ok(p.g) || p.cl2) return QM_ERR_UNSUPPORTED;
-    const GemmShape g = p.g;
+    const UnitPlan& up = units[k];
+    const GemmShape g = up.g;
+    const TcProbeArgs& p0 = ps[up.probe[0]];
     const int64_t ldc = qm_code_ld(g.K);
-    GroupProblem& gp = tab.p[k];
+    GroupUnit& gu = tab.u[k];
     // outputs at most 64 wide (the context and score-gradient products of attention): MMAs of N = 64,
     // half as many right-operand rows staged
     const int half_n = g.N <= 64 ? 32 : kHalfN;
-    const bool ok = make_map(&gp.maps[0], p.l, true, kBlockM, g.K, g.M, g.batch, p.l_ld, p.l_sb) &&
-                    make_map(&gp.maps[1], p.r, true, half_n, g.K, g.N, g.batch, p.r_ld, p.r_sb) &&
-                    make_map(&gp.maps[2], p.cl, false, kBlockM, g.K, g.M, g.batch, ldc, g.M * ldc) &&
-                    make_map(&gp.maps[3], p.cr, false, half_n, g.K, g.N, g.batch, ldc, g.N * ldc);
-    if (!ok) return QM_ERR_CUDA;
+    if (!make_map(&gu.maps[0], p0.l, true, kBlockM, g.K, g.M, g.batch, p0.l_ld, p0.l_sb) ||
+        !make_map(&gu.maps[1], p0.r, true, half_n, g.K, g.N, g.batch, p0.r_ld, p0.r_sb))
+      return QM_ERR_CUDA;
     KernelArgs ka{};
     fill_tiles(&ka, g);
-    ka.dl = p.dl; ka.pc_l = p.gran_l == QM_GRAN_CHANNEL; ka.dr = p.dr; ka.pc_r = p.gran_r == QM_GRAN_CHANNEL;
-    ka.partials = p.partials; ka.done_counter = p.done_counter; ka.result = p.result;
-    ka.count = (uint64_t)(g.M * g.N * g.batch);
-    ka.err_word = p.err_word; ka.idesc_lp = lp_idesc(p.fmt_l, p.fmt_r, 2 * half_n);
-    ka.row_stats = p.row_stats;
-    ka.err_also[0] = p.err_also[0]; ka.err_also[1] = p.err_also[1];
-    gp.a = ka;
-    gp.half_n = half_n;
+    gu.M = (int32_t)g.M; gu.N = (int32_t)g.N; gu.K = (int32_t)g.K;
+    gu.tiles_m = ka.tiles_m; gu.tiles_n = ka.tiles_n;
+    gu.tile_begin = (int32_t)total;
+    gu.half_n = half_n;
     // Tiles that run at the same time should share the LARGER operand's blocks, so that it is
     // streamed from HBM once and the smaller one is what gets fetched again (from L2, if it fits):
     // the tiles of a batch element are walked along the shorter side first.
-    gp.m_fastest = g.M < g.N ? 1 : 0;
-    gp.idesc_ref = make_idesc(1, 1, 1, kPairM, 2 * half_n);
-    gp.kind = p.fmt_l == QM_FMT_INT8 ? kKindI8 : kKindF8;
-    gp.tile_begin = (int32_t)total;
+    gu.m_fastest = g.M < g.N ? 1 : 0;
+    gu.var_begin = tab.n_var; gu.n_var = up.n_var;
     total += ka.num_tiles;
-    if (total >= (1ll << 31)) return QM_ERR_UNSUPPORTED;
+    for (int j = 0; j < up.n_var; ++j) {
+      const TcProbeArgs& p = ps[up.probe[j]];
+      GroupVar& v = tab.v[tab.n_var++];
+      if (!make_map(&v.maps[0], p.cl, false, kBlockM, g.K, g.M, g.batch, ldc, g.M * ldc, true) ||
+          !make_map(&v.maps[1], p.cr, false, half_n, g.K, g.N, g.batch, ldc, g.N * ldc, true))
+        return QM_ERR_CUDA;
+      v.dl = p.dl; v.dr = p.dr;
+      v.partials = p.partials; v.result = p.result; v.row_stats = p.row_stats;
+      v.err_word = p.err_word; v.err_also[0] = p.err_also[0]; v.err_also[1] = p.err_also[1];
+      v.count = (uint64_t)(g.M * g.N * g.batch);
+      v.flags = (p.fmt_l == QM_FMT_INT8 ? kVarI8 : 0u) | (p.gran_l == QM_GRAN_CHANNEL ? kVarScalePerRow : 0u) |
+                (p.gran_r == QM_GRAN_CHANNEL ? kVarScalePerCol : 0u) | (p.row_stats ? kVarRowStats : 0u);
+      v.idesc_lp = lp_idesc(p.fmt_l, p.fmt_r, 2 * half_n);
+    }
   }
   tab.total_tiles = (int32_t)total;
-  const qm_status rs = probe_residency();
-  if (rs != QM_OK) return rs;
   const int pairs = max_pairs();
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(2 * (total < pairs ? total : pairs)));
   cfg.blockDim = dim3(kProbeThreads);
-  cfg.dynamicSmemBytes = kProbeSmem;
+  cfg.dynamicSmemBytes = probe_smem<Table>();
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1961,10 +2145,54 @@ qm_status launch_tc_probe_group(const TcProbeArgs* ps, int n, cudaStream_t s) {
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   profile_events(&ev0, &ev1);
   if (ev0) QM_CUDA_OK(cudaEventRecord(ev0, s));
-  QM_CUDA_OK(cudaLaunchKernelEx(&cfg, tc_group_kernel, tab));
+  QM_CUDA_OK(cudaLaunchKernelEx(&cfg, tc_group_kernel<Table>, tab));
   if (ev1) QM_CUDA_OK(cudaEventRecord(ev1, s));
   count_launch();
   return QM_OK;
+}
+}  // namespace
+
+void set_wait_limit_ns(uint64_t ns) { g_wait_limit_ns.store(ns ? ns : 1000000000ull); }
+void set_stop_after_kb(uint32_t kb) { g_stop_after_kb.store(kb); }
+
+qm_status launch_tc_probes(const TcProbeArgs* ps, int n, cudaStream_t s) {
+  if (n < 1) return QM_ERR_INVALID_ARG;
+  qm_status st = probe_residency();
+  if (st != QM_OK) return st;
+  // units: probes of the same operands, up to the first probe whose extents are refused
+  std::vector<UnitPlan> units;
+  units.reserve((size_t)n);
+  qm_status refused = QM_OK;
+  for (int i = 0; i < n; ++i) {
+    if (!shape_ok(ps[i].g) || ps[i].cl2) { refused = QM_ERR_UNSUPPORTED; break; }
+    UnitPlan* u = nullptr;
+    for (UnitPlan& c : units)
+      if (c.n_var < kMaxVar && same_products(ps[c.probe[0]], ps[i])) { u = &c; break; }
+    if (!u) {
+      units.push_back(UnitPlan{ps[i].g, 0, {}});
+      u = &units.back();
+    }
+    u->probe[u->n_var++] = i;
+  }
+  // descending tile cost: kilobytes through shared memory per 64 contraction entries
+  std::stable_sort(units.begin(), units.end(), [](const UnitPlan& a, const UnitPlan& b) {
+    return a.g.K * (88 + 24 * a.n_var) > b.g.K * (88 + 24 * b.n_var);
+  });
+  for (size_t u0 = 0; u0 < units.size() && st == QM_OK;) {
+    size_t u1 = u0;
+    int64_t tiles = 0;
+    int vars = 0;
+    while (u1 < units.size() && (int)(u1 - u0) < TableBig::kUnits && vars + units[u1].n_var <= TableBig::kVars &&
+           tiles + tile_count(units[u1].g) < (1ll << 31)) {
+      vars += units[u1].n_var;
+      tiles += tile_count(units[u1].g);
+      ++u1;
+    }
+    st = u1 - u0 == 1 && vars == 1 ? launch_units<TableOne>(ps, &units[u0], 1, s)
+                                   : launch_units<TableBig>(ps, &units[u0], (int)(u1 - u0), s);
+    u0 = u1;
+  }
+  return st != QM_OK ? st : refused;
 }
 
 // per format; a launch writes one record per CTA of its grid
@@ -1974,7 +2202,7 @@ int tc_probe_records(GemmShape) {
 }
 
 qm_status launch_tc_probe(const TcProbeArgs& p, cudaStream_t s) {
-  if (!p.cl2) return launch_tc_probe_group(&p, 1, s);       // one format: a group of one
+  if (!p.cl2) return launch_tc_probes(&p, 1, s);            // one format: a unit of one
   if (!shape_ok(p.g)) return QM_ERR_UNSUPPORTED;
   const qm_status rs = probe_residency();
   if (rs != QM_OK) return rs;

@@ -610,6 +610,7 @@ qm_status qm_probe_layer_host(const qm_operand* L_host, const qm_operand* R_host
 namespace {
 constexpr int kBatchStreams = 8;      // streams of the pool
 constexpr int kCopyEvents = 64;       // chunks of a host batch that can wait for their own copies
+constexpr int kHostChunk = 16;        // probes of a chunk of a host batch
 struct BatchStreams {
   std::mutex issue;            // one batch at a time is put into the streams (host side only)
   bool ready = false;
@@ -843,16 +844,11 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
     QM_CUDA_OK(cudaEventRecord(b->join[j], b->s[j]));
     QM_CUDA_OK(cudaStreamWaitEvent(user, b->join[j], 0));
   }
-  // Pass 3: the caller's stream has waited for every chain; the fused kernels go to it as
-  // persistent launches of up to tc_group_max() probes.  (Running a second chunk's chains under
-  // the first chunk's launch measured slower: the chains wait for the SMs the launch holds.)
+  // Pass 3: the caller's stream has waited for every chain; the fused kernels go to it in as few
+  // persistent launches as hold them, probes of the same operands sharing their reference and
+  // denominator products.  (Running a second launch's chains under the first launch measured
+  // slower: the chains wait for the SMs the launch holds.)
   std::vector<TcProbeArgs> args;
-  auto flush_group = [&]() -> qm_status {
-    if (args.empty()) return QM_OK;
-    const qm_status e = launch_tc_probe_group(args.data(), (int)args.size(), user);
-    args.clear();
-    return e;
-  };
   for (int32_t i = 0; i < good && st == QM_OK; ++i) {
     if (!plans[i].tc) continue;
     const Planned& pl = plans[i];
@@ -879,13 +875,8 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
     p.result = out + i;
     p.row_stats = cfg[i].row_stats;
     args.push_back(p);
-    if ((int)args.size() == tc_group_max()) {
-      const qm_status g = flush_group();
-      if (g != QM_OK && st == QM_OK) st = g;
-    }
   }
-  const qm_status g = flush_group();
-  if (g != QM_OK && st == QM_OK) st = g;
+  if (!args.empty()) st = launch_tc_probes(args.data(), (int)args.size(), user);
   return st != QM_OK ? st : refused;
 }
 
@@ -932,14 +923,14 @@ qm_status qm_probe_batch_host(int32_t n, const qm_operand* L_host, const qm_oper
   qm_status st = batch_streams(&bs);
   if (st != QM_OK) return st;
   // Every distinct host operand is copied once, on a stream of the library's own and in the order
-  // in which the probes first name them.  The probes go to the device in chunks of one fused
-  // launch's worth, each chunk as a device batch (which prepares every distinct operand of the
+  // in which the probes first name them.  The probes go to the device in chunks of
+  // kHostChunk, each chunk as a device batch (which prepares every distinct operand of the
   // chunk once) that waits only for the copies it needs: the copies of later chunks run under the
   // kernels of earlier ones.  Order the probes so that those of one product are neighbours and the
   // first chunks need only the first tensors.
   std::vector<qm_operand> Ld((size_t)n), Rd((size_t)n);
   std::vector<HostCopy> seen;
-  const int32_t chunk = tc_group_max();
+  const int32_t chunk = kHostChunk;
   const bool pipelined = (n + chunk - 1) / chunk <= kCopyEvents;
   std::lock_guard<std::mutex> lock(bs->host_issue);
   QM_CUDA_OK(cudaEventRecord(bs->copy_fork, user));               // the copies follow the work already in the stream

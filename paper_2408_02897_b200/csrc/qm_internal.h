@@ -158,10 +158,11 @@ struct TcProbeArgs {
 };
 int tc_probe_records(GemmShape g);
 qm_status launch_tc_probe(const TcProbeArgs& a, cudaStream_t s);
-// Up to tc_group_max() one-format probes as one persistent launch (every probe's operands must be
-// prepared already; each writes its own record; the first probe's done_counter counts the CTAs).
-int tc_group_max();
-qm_status launch_tc_probe_group(const TcProbeArgs* ps, int n, cudaStream_t s);
+// One-format probes in as few persistent launches as their number allows, those of the same two operands
+// sharing the reference and denominator products (every probe's operands must be prepared
+// already; each writes its own record; the done_counter of one probe per launch counts the CTAs).
+// Probes from the first one with refused extents on are not run; the ones before it are.
+qm_status launch_tc_probes(const TcProbeArgs* ps, int n, cudaStream_t s);
 // Bound of every barrier wait of the fused probe kernel (0 restores the default of one second), and
 // a hook for testing the give-up path: the producer issues no more than this many k-blocks
 // per CTA (0xffffffff: off), so that the consumers' waits run out.

@@ -1,0 +1,57 @@
+"""Probes of the same operands in one batch share their reference and denominator products: every record
+must be the one the probe gives on its own, for every number of formats and granularities per product."""
+import pytest
+import torch
+
+import oracle
+import paper_2408_02897_b200 as qm
+from paper_2408_02897_b200 import binding, workloads
+
+pytestmark = pytest.mark.gpu
+
+FIELDS = ("sum_be", "max_be", "sum_diff2", "sum_ref2", "sum_den2")
+VARIANTS = [("e4m3", "tensor", "rtne"), ("int8", "channel", "rtne"), ("e5m2", "tensor", "stochastic_r"), ("int8", "tensor", "rtne"),
+            ("e4m3", "channel", "rtne"), ("e5m2", "channel", "rtne"), ("e5m2", "channel", "stochastic_both")]
+
+
+def operands(M, N, K, batch, seed):
+    rng = workloads._rng(seed)
+    shape = (lambda r: (r, K)) if batch == 1 else (lambda r: (batch, r, K))
+    return workloads.normal(rng, shape(M)), workloads.normal(rng, shape(N), 0.02)
+
+
+def as_batch(Lo, Ro, variants):
+    b = qm.ProbeBatch([(Lo, Ro, f, f, g, g) for f, g, _ in variants])
+    for c, (_, _, r) in zip(b.cfg, variants):
+        c.round, c.seed = binding.ROUND[r], 5
+    b.launch()
+    torch.cuda.synchronize()
+    return b.results()
+
+
+# 1 .. 7 variants (six fill a unit, the seventh starts another); contraction below, at and past a block of 64 and
+# of 128, more blocks than the ring has stages, outputs at most 64 wide, ragged edges, several tiles per CTA pair
+@pytest.mark.parametrize("n_var", [1, 2, 3, 4, 5, 6, 7])
+@pytest.mark.parametrize("M,N,K,batch", [(256, 128, 64, 1), (130, 40, 80, 1), (300, 200, 128, 1), (257, 129, 1040, 1),
+                                         (96, 64, 48, 200), (512, 96, 192, 60)])
+def test_records_do_not_depend_on_what_shares_the_products(n_var, M, N, K, batch):
+    L, R = operands(M, N, K, batch, 100 + n_var)
+    Ld, Rd = L.cuda(), R.cuda()
+    Lo, Ro = qm.operand_of(Ld, -1), qm.operand_of(Rd, -1)
+    got = as_batch(Lo, Ro, VARIANTS[:n_var])
+    for (f, g, r), rec in zip(VARIANTS, got):
+        alone = qm.qm_probe_layer(Lo, Ro, f, f, g, g, "bf16", rounding=r, seed=5).record()
+        assert rec.device_error == 0 and rec.record()["count"] == alone["count"] == M * N * batch
+        for k in FIELDS:     # the same fp32 terms; only the order of the fp64 additions over tiles may differ
+            assert abs(rec.record()[k] - alone[k]) <= 1e-12 * abs(alone[k]), (f, g, r, k)
+
+
+def test_shared_products_against_the_oracle():
+    L, R = operands(300, 200, 272, 1, 7)
+    Ld, Rd = L.cuda(), R.cuda()
+    variants = [v for v in VARIANTS if v[2] == "rtne"]
+    got = as_batch(qm.operand_of(Ld, -1), qm.operand_of(Rd, -1), variants)
+    for (f, g, _), rec in zip(variants, got):
+        want = oracle.probe(L.float().numpy(), R.float().numpy().T, f, f, g, g)
+        for k in FIELDS:     # the tolerances of the one-probe tests: fp32 accumulation with truncation
+            assert abs(rec.record()[k] - want[k]) <= (1e-3 if k == "max_be" else 1e-4) * abs(want[k]), (f, g, k)
