@@ -402,9 +402,7 @@ static qm_status probe_phases(const qm_operand* Lo, const qm_operand* Ro, const 
     p.row_stats = cfg->row_stats;
     return launch_tc_probe(p, s);           // the last CTA writes the record
   }
-  st = launch_simt_probe(L, R, cl, cfg->fmt_l, dl, cfg->gran_l, cr, cfg->fmt_r, dr, cfg->gran_r, part, s);
-  if (st != QM_OK) return st;
-  return launch_metric_finalize(part, w.n_part, (uint64_t)(g.M * g.N * g.batch), err, out, s);
+  return launch_simt_probe(L, R, cl, cfg->fmt_l, dl, cfg->gran_l, cr, cfg->fmt_r, dr, cfg->gran_r, part, err + 1, err, out, s);
 }
 
 qm_status qm_probe_layer(const qm_operand* Lo, const qm_operand* Ro, const qm_probe_cfg* cfg,

@@ -127,10 +127,12 @@ qm_status launch_simt_gemm_lp(const uint8_t* cl, int fmt_l, const float* dl, int
                               const uint8_t* cr, int fmt_r, const float* dr, int gran_r,
                               GemmShape g, float* out_descaled, void* out_raw, cudaStream_t s);
 int simt_probe_blocks(GemmShape g);
-// Fused CUDA-core probe: three accumulators per output, Eq. 3 partials per CTA.
+// Fused CUDA-core probe: three accumulators per output, Eq. 3 partials per CTA, the record written by
+// the last CTA to finish (done_counter: zero on entry).
 qm_status launch_simt_probe(const View& L, const View& R, const uint8_t* cl, int fmt_l,
                             const float* dl, int gran_l, const uint8_t* cr, int fmt_r,
-                            const float* dr, int gran_r, double* partials, cudaStream_t s);
+                            const float* dr, int gran_r, double* partials, uint32_t* done_counter,
+                            uint32_t* err_word, qm_metric_result* out, cudaStream_t s);
 
 // ---- tensor-core GEMMs (gemm_tc.cu) ---------------------------------------
 struct TcProbeArgs {
