@@ -268,7 +268,7 @@ __host__ __device__ constexpr uint32_t make_idesc(uint32_t c_fmt, uint32_t a_fmt
   return (c_fmt << 4) | (a_fmt << 7) | (b_fmt << 10) | ((n >> 3) << 17) | ((m >> 4) << 24);
 }
 
-struct Shared {
+struct alignas(16) Shared {
   uint64_t full[kMaxStages];     // used in the leader CTA: both CTAs' loads of a stage have landed
   uint64_t empty[kMaxStages];    // per CTA: the pair's MMAs have finished reading the stage
   uint64_t tmem_full;            // per CTA: the tile's accumulators are complete
@@ -393,6 +393,30 @@ __device__ __forceinline__ void stats16(const uint32_t* rc, const uint32_t* rd, 
   }
 }
 
+// 32 rows x 32 columns of output from a warp that holds a row per lane: through 4 KB of shared memory (16-byte
+// units permuted with the row: conflict-free both ways), so that every store instruction writes whole
+// 128-byte lines.  A row per thread puts the 32 lanes of a store on 32 lines, sixteen bytes each; with
+// short contractions those stores, not the MMAs, were what a tile took: 4096 x 3072 x 768 42 us, staged 20.
+// Outputs whose rows do not all start on 16 bytes are written a column per lane.
+__device__ __forceinline__ void store_chunk(uint4* stage, int lane, const uint32_t (&r)[32], uint32_t* out, int64_t ld, int rows,
+                                            int cols, bool vec_ok) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j) stage[lane * 8 + (j ^ (lane & 7))] = make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+  __syncwarp();
+  if (cols == 32 && vec_ok) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int row = 4 * i + (lane >> 3), u = lane & 7;
+      if (row < rows) *reinterpret_cast<uint4*>(out + row * ld + 4 * u) = stage[row * 8 + (u ^ (row & 7))];
+    }
+  } else {
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(stage);
+    for (int row = 0; row < rows; ++row)
+      if (lane < cols) out[row * ld + lane] = w[row * 32 + (((lane >> 2) ^ (row & 7)) << 2) + (lane & 3)];
+  }
+  __syncwarp();
+}
+
 template <int MODE, int LPKIND, int LPKIND2>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_constant__ CUtensorMap map_r,
@@ -410,7 +434,8 @@ tc_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_constant__ CUt
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   Shared* sh = reinterpret_cast<Shared*>(tiles + (size_t)kStages * C::kStageBytes);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // known to the compiler to be the same in all lanes (see tc_group_kernel)
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();                   // 0 = leader
   const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
   const int num_kb = (int)((a.K + kBlockK - 1) / kBlockK);
@@ -660,6 +685,11 @@ tc_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_constant__ CUt
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&sh->lp_done), 0));
       } else {
+        uint4* const stage = reinterpret_cast<uint4*>(sh + 1) + (warp - 2) * 256;      // 4 KB per epilogue warp
+        const int64_t row0 = row - lane;
+        const int rows_live = (int)(a.M - row0 < 32 ? a.M - row0 : 32);      // <= 0: none
+        const bool vec_ok = (a.N & 3) == 0 && (reinterpret_cast<uintptr_t>(a.out_descaled) & 15) == 0 &&
+                            (reinterpret_cast<uintptr_t>(a.out_raw) & 15) == 0;
 #pragma unroll 1
         for (int c = 0; c < 2; ++c) {
           const int cc0 = h * 64 + c * 32;          // first column of this chunk inside the tile
@@ -669,20 +699,18 @@ tc_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_constant__ CUt
           uint32_t r[32];
           tmem_ld32(lane_addr + cc0, r);
           tmem_ld_wait();
-          if (row_ok) {
-            const int64_t o = ((int64_t)tc.b * a.M + row) * a.N + col0;
+          const int64_t o0 = ((int64_t)tc.b * a.M + row0) * a.N + col0;
+          if (MODE == kRefOnly) {
+            store_chunk(stage, lane, r, reinterpret_cast<uint32_t*>(a.out_descaled) + o0, a.N, rows_live, n_live, vec_ok);
+          } else {
+            if (a.out_raw) store_chunk(stage, lane, r, reinterpret_cast<uint32_t*>(a.out_raw) + o0, a.N, rows_live, n_live, vec_ok);
+            if (a.out_descaled) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              if (j < n_live) {
-                if (MODE == kRefOnly) {
-                  a.out_descaled[o + j] = __uint_as_float(r[j]);
-                } else {
-                  const float acc = LPKIND == kKindI8 ? (float)(int)r[j] : __uint_as_float(r[j]);
-                  const float drj = per_col ? dr_s[cc0 + j] : dr_tensor;
-                  if (a.out_descaled) a.out_descaled[o + j] = acc * (dlv * drj);
-                  if (a.out_raw) reinterpret_cast<uint32_t*>(a.out_raw)[o + j] = r[j];
-                }
+              for (int j = 0; j < 32; ++j) {
+                const float acc = LPKIND == kKindI8 ? (float)(int)r[j] : __uint_as_float(r[j]);
+                r[j] = __float_as_uint(acc * (dlv * (per_col ? dr_s[cc0 + j] : dr_tensor)));
               }
+              store_chunk(stage, lane, r, reinterpret_cast<uint32_t*>(a.out_descaled) + o0, a.N, rows_live, n_live, vec_ok);
             }
           }
         }
@@ -776,11 +804,11 @@ tc_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_constant__ CUt
 // accumulator buffers (2 x 256 tensor-memory columns), so the epilogue of one tile runs under the
 // main loop of the next.  A k-block is 128 BYTES of contraction per row for every operand type
 // (64 bf16 or 128 codes), so all tiles are 128-byte-swizzled 16 KB blocks: a stage is this CTA's
-// 128 left rows and its 128-row half of the right tile, 32 KB, six stages.  Roles, barriers,
+// 128 left rows and its 128-row half of the right tile, 32 KB, five stages.  Roles, barriers,
 // bounded waits and the exit protocol are those of tc_kernel.
 constexpr int kWideN = 256;
 constexpr int kWideHalfN = 128;
-constexpr int kWideStages = 6;
+constexpr int kWideStages = 5;
 constexpr uint32_t kWideTile = 128 * 128;                 // 16 KB
 constexpr uint32_t kWideStageBytes = 2 * kWideTile;
 
@@ -792,6 +820,7 @@ struct SharedWide {
   uint32_t tmem_base;
   uint32_t abort_flag;
   float delta_r[2][kWideN];
+  uint4 stage[kEpiWarps][32 * 8];  // output chunks on their way out, 4 KB per epilogue warp
 };
 
 // KIND: kKindF16 (bf16 x bf16 -> fp32 output), kKindF8 / kKindI8 (descaled and/or raw output)
@@ -802,7 +831,8 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   extern __shared__ uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   SharedWide* sh = reinterpret_cast<SharedWide*>(tiles + (size_t)kWideStages * kWideStageBytes);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // known to the compiler to be the same in all lanes (see tc_group_kernel)
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
   constexpr int kElemsPerBlock = KIND == kKindF16 ? 64 : 128;          // contraction elements per k-block
@@ -884,10 +914,12 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           tc_fence_after();
           const uint32_t base = smem_u32(tiles + (size_t)s * kWideStageBytes);
           const uint64_t da = smem_desc(base, 128), db = smem_desc(base + kWideTile, 128);
+          if (lead) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k)             // 32 bytes of contraction per instruction
-            mma_pair<KIND>(tmem_base + buf * kWideN, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0, lead);
-          tc_commit_pair(smem_u32(&sh->empty[s]), lead);
+            for (int k = 0; k < 4; ++k)           // 32 bytes of contraction per instruction
+              mma_pair<KIND>(tmem_base + buf * kWideN, da + 2 * k, db + 2 * k, idesc, k ? 1u : (uint32_t)kb, true);
+            tc_commit_pair(smem_u32(&sh->empty[s]), true);
+          }
         }
         if (ok) tc_commit_pair(smem_u32(&sh->tmem_full[buf]), lead);
       }
@@ -903,6 +935,7 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     // 16-byte stores need 16-byte aligned rows: output bases aligned and N a multiple of 4
     const bool vec_ok = (a.N & 3) == 0 && (reinterpret_cast<uintptr_t>(a.out_descaled) & 15) == 0 &&
                         (reinterpret_cast<uintptr_t>(a.out_raw) & 15) == 0;
+    uint4* const stage = sh->stage[warp - 2];
     uint32_t it = 0;
     for (int t = pair; t < a.num_tiles; t += num_pairs, ++it) {
       const TileCoord tc = tile_coord(t, a);
@@ -912,8 +945,9 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         const int64_t col = (int64_t)tc.n_tile * kWideN + et;
         dr_s[et] = col < a.N ? __ldg(a.dr + (int64_t)tc.b * a.N + col) : 0.f;
       }
-      const int64_t row = (int64_t)tc.m_tile * kPairM + rank * kBlockM + q * 32 + lane;
+      const int64_t row0 = (int64_t)tc.m_tile * kPairM + rank * kBlockM + q * 32, row = row0 + lane;
       const bool row_ok = row < a.M;
+      const int rows_live = (int)(a.M - row0 < 32 ? a.M - row0 : 32);      // <= 0: none
       float dlv = dl_tensor;
       if (KIND != kKindF16 && a.pc_l) dlv = row_ok ? __ldg(a.dl + (int64_t)tc.b * a.M + row) : 0.f;
       const bool ok = mbar_wait(smem_u32(&sh->tmem_full[buf]), (it >> 1) & 1, abort_flag, a.err_word);
@@ -929,40 +963,18 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         uint32_t r[32];
         tmem_ld32(lane_addr + cc0, r);
         tmem_ld_wait();
-        if (row_ok) {
-          const int64_t o = ((int64_t)tc.b * a.M + row) * a.N + col0;
-          if (n_live == 32 && vec_ok) {
-            // 128 bytes per thread and chunk: whole lines
+        const int64_t o0 = ((int64_t)tc.b * a.M + row0) * a.N + col0;     // first row of the warp, first column of the chunk
+        if (KIND == kKindF16) {
+          store_chunk(stage, lane, r, reinterpret_cast<uint32_t*>(a.out_descaled) + o0, a.N, rows_live, n_live, vec_ok);
+        } else {
+          if (a.out_raw) store_chunk(stage, lane, r, reinterpret_cast<uint32_t*>(a.out_raw) + o0, a.N, rows_live, n_live, vec_ok);
+          if (a.out_descaled) {
 #pragma unroll
-            for (int j = 0; j < 32; j += 4) {
-              if (KIND == kKindF16) {
-                *reinterpret_cast<uint4*>(a.out_descaled + o + j) = make_uint4(r[j], r[j + 1], r[j + 2], r[j + 3]);
-              } else {
-                if (a.out_raw)
-                  *reinterpret_cast<uint4*>(reinterpret_cast<uint32_t*>(a.out_raw) + o + j) =
-                      make_uint4(r[j], r[j + 1], r[j + 2], r[j + 3]);
-                if (a.out_descaled) {
-                  float4 v;
-                  float* pv = &v.x;
-#pragma unroll
-                  for (int e = 0; e < 4; ++e) {
-                    const float acc = KIND == kKindI8 ? (float)(int)r[j + e] : __uint_as_float(r[j + e]);
-                    pv[e] = acc * (dlv * (per_col ? dr_s[cc0 + j + e] : dr_tensor));
-                  }
-                  *reinterpret_cast<float4*>(a.out_descaled + o + j) = v;
-                }
-              }
+            for (int j = 0; j < 32; ++j) {
+              const float acc = KIND == kKindI8 ? (float)(int)r[j] : __uint_as_float(r[j]);
+              r[j] = __float_as_uint(acc * (dlv * (per_col ? dr_s[cc0 + j] : dr_tensor)));
             }
-          } else {
-            for (int j = 0; j < n_live; ++j) {
-              if (KIND == kKindF16) {
-                a.out_descaled[o + j] = __uint_as_float(r[j]);
-              } else {
-                const float acc = KIND == kKindI8 ? (float)(int)r[j] : __uint_as_float(r[j]);
-                if (a.out_descaled) a.out_descaled[o + j] = acc * (dlv * (per_col ? dr_s[cc0 + j] : dr_tensor));
-                if (a.out_raw) reinterpret_cast<uint32_t*>(a.out_raw)[o + j] = r[j];
-              }
-            }
+            store_chunk(stage, lane, r, reinterpret_cast<uint32_t*>(a.out_descaled) + o0, a.N, rows_live, n_live, vec_ok);
           }
         }
       }
@@ -1902,7 +1914,8 @@ uint32_t lp_idesc(int fmt_l, int fmt_r, int n = kBlockN) {
 
 template <int MODE>
 size_t smem_bytes() {
-  return (size_t)Cfg<MODE>::kStages * Cfg<MODE>::kStageBytes + sizeof(Shared) + 1024;
+  // the plain products' output goes out through 4 KB per epilogue warp, behind the control block
+  return (size_t)Cfg<MODE>::kStages * Cfg<MODE>::kStageBytes + sizeof(Shared) + 1024 + (MODE == kProbe2 ? 0 : kEpiWarps * 4096);
 }
 
 int64_t tile_count(GemmShape g) {
