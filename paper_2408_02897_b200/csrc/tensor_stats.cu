@@ -128,6 +128,91 @@ struct Batch {
       f[6] = fmaxf(f[6], rr);
     }
   }
+  // The same sums for eight elements under one scale, for the common case that the scale is in the range of
+  // the two-wide quotient and no element is anywhere near overflow (else false, and nothing is done).  Then
+  //   an element underflows exactly when its code is zero and it is not, and its error is the element itself:
+  //     RE = 1, so it counts instead of being computed, and err - (err where the code is not zero) is its error;
+  //   an element below 1e-36 has code zero, so clamping the divisor changes nothing;
+  //   INT8 rounds by adding and subtracting 1.5 2^23 (round to nearest even for |t| < 2^22).
+  // Where no lane of the warp can have a zero code (FP8 codes reach far down, so that is the rule for them) the
+  // second class is left out.  15 to 20 instructions per element, most of them two-wide, against 50 one at a time.
+  uint64_t e2r = 0ull, e2u = 0ull, xx = 0ull;       // two-wide sums of squares: rounding class, underflowed, all
+  float rr = 0.f;                                   // sum RE of the rounding class
+  uint32_t n_unit = 0;                              // underflowed elements: RE 1 each
+  template <bool ZERO_CODES>
+  __device__ __forceinline__ void error8(const Vec8& v, const QuotientPair& quot, uint64_t ndelta2) {
+    uint64_t minus1;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(minus1) : "f"(-1.f));
+    uint32_t zero_codes = 0, zeros = 0;
+#pragma unroll
+    for (int e = 0; e < 8; e += 2) {
+      uint64_t x2, g2, err2, rcp2, rr2;
+      asm("mov.b64 %0, {%1, %2};" : "=l"(x2) : "f"(v.v[e]), "f"(v.v[e + 1]));
+      const uint64_t t2 = quot(x2);
+      float g0, g1, c0, c1;
+      if (FMT == QM_FMT_INT8) {
+        uint64_t magic, nmagic;
+        asm("mov.b64 %0, {%1, %1};" : "=l"(magic) : "f"(12582912.f));
+        asm("mov.b64 %0, {%1, %1};" : "=l"(nmagic) : "f"(-12582912.f));
+        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(g2) : "l"(t2), "l"(magic));
+        asm("add.rn.f32x2 %0, %0, %1;" : "+l"(g2) : "l"(nmagic));
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(g0), "=f"(g1) : "l"(g2));
+      } else {
+        float t0, t1;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(t0), "=f"(t1) : "l"(t2));
+        decode2<FMT>(quant2<FMT>(t0, t1), g0, g1);
+        asm("mov.b64 %0, {%1, %2};" : "=l"(g2) : "f"(g0), "f"(g1));
+      }
+      asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(err2) : "l"(g2), "l"(ndelta2), "l"(x2));      // x - value(code) delta
+      c0 = fabsf(v.v[e]);
+      c1 = fabsf(v.v[e + 1]);
+      if (ZERO_CODES) {
+        float e0, e1;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(e0), "=f"(e1) : "l"(err2));
+        zero_codes += g0 == 0.f;
+        zero_codes += g1 == 0.f;
+        zeros += c0 == 0.f;
+        zeros += c1 == 0.f;
+        e0 = g0 == 0.f ? 0.f : e0;                                 // the rounding class
+        e1 = g1 == 0.f ? 0.f : e1;
+        uint64_t er2, eu2;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(er2) : "f"(e0), "f"(e1));
+        asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(eu2) : "l"(er2), "l"(minus1), "l"(err2));   // the underflowed class
+        asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(e2u) : "l"(eu2));
+        err2 = er2;
+        c0 = fmaxf(c0, 1e-37f);
+        c1 = fmaxf(c1, 1e-37f);
+      }
+      asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(c0));
+      asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(c1));
+      asm("mov.b64 %0, {%1, %2};" : "=l"(rcp2) : "f"(c0), "f"(c1));
+      asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(rr2) : "l"(err2), "l"(rcp2));
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(c0), "=f"(c1) : "l"(rr2));
+      rr += fabsf(c0);
+      rr += fabsf(c1);
+      asm("max.f32 %0, %0, %1, %2;" : "+f"(f[6]) : "f"(fabsf(c0)), "f"(fabsf(c1)));
+      asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(e2r) : "l"(err2));
+      asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(xx) : "l"(x2));
+    }
+    n[0] += 8u - zeros;
+    n_unit += zero_codes - zeros;
+  }
+  __device__ __forceinline__ bool error8_fast(const Vec8& v, const QuotientPair& quot, float delta) {
+    // half the smallest positive value of the format: what lies above it has a code
+    constexpr float kHalfMin = FMT == QM_FMT_INT8 ? 0.5f : (FMT == QM_FMT_E4M3 ? 0x1p-10f : 0x1p-17f);
+    float mx_x = 0.f, mn_x = 3.4e38f;
+#pragma unroll
+    for (int e = 0; e < 8; e += 2) {
+      asm("max.f32 %0, %0, %1, %2;" : "+f"(mx_x) : "f"(fabsf(v.v[e])), "f"(fabsf(v.v[e + 1])));
+      asm("min.f32 %0, %0, %1, %2;" : "+f"(mn_x) : "f"(fabsf(v.v[e])), "f"(fabsf(v.v[e + 1])));
+    }
+    if (!(QuotientPair::serves(delta) && mx_x <= delta * (0.9999f * fmt_qmax(FMT)))) return false;
+    uint64_t ndelta2;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(ndelta2) : "f"(-delta));
+    if (__any_sync(__activemask(), !(mn_x > delta * (1.0001f * kHalfMin)))) error8<true>(v, quot, ndelta2);
+    else error8<false>(v, quot, ndelta2);
+    return true;
+  }
   __device__ __forceinline__ void flush(Acc& acc) {
     if (KIND == kStats) {
       fold_stats();
@@ -135,9 +220,22 @@ struct Batch {
       acc.d[4] = fmax(acc.d[4], (double)f[4]);
     } else {
 #pragma unroll
-      for (int i = 0; i < 6; ++i) acc.d[i] += (double)f[i];
-      acc.d[6] += (double)n[0]; acc.d[7] += (double)n[1]; acc.d[8] += (double)n[2];
-      acc.d[9] = fmax(acc.d[9], (double)f[6]);
+      for (int i = 0; i < 5; ++i) { acc.d[i] += (double)f[i]; f[i] = 0.f; }
+      float a, b;
+      acc.d[0] += (double)rr; acc.d[1] += (double)rr;
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(e2r)); acc.d[2] += (double)(a + b);
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(e2u)); acc.d[4] += (double)(a + b);
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(xx)); acc.d[5] += (double)(a + b) + (double)f[5];
+      f[5] = 0.f; rr = 0.f;
+      e2r = e2u = xx = 0ull;
+    }
+  }
+  // what is carried in whole numbers, or as a maximum, to the end of the pass
+  __device__ __forceinline__ void finish(Acc& acc) {
+    if (KIND == kError) {
+      acc.d[0] += (double)n_unit;
+      acc.d[6] = (double)n[0]; acc.d[7] = (double)n[1]; acc.d[8] = (double)(n[2] + n_unit);
+      acc.d[9] = (double)f[6];
     }
   }
 };
@@ -290,10 +388,13 @@ tensor_pass_kernel(const Lines p, double* __restrict__ partials, uint32_t* __res
     o = line - b * p.outer;
     return (int64_t)b * p.batch_stride + (int64_t)o * p.line_stride + (int64_t)j * 8;
   };
+  const float delta0 = KIND == kError && p.delta_mode == 0 ? __ldg(p.delta) : 1.f;
+  const QuotientPair quot0(delta0);
   auto process = [&](Batch<KIND, FMT>& bt, const Vec8& v, uint32_t b, uint32_t o, uint32_t j, int live) {
     if (KIND == kStats) { bt.stats(v); return; }
     if (p.delta_mode != 2) {
-      const float d = p.delta_mode == 0 ? __ldg(p.delta) : __ldg(p.delta + (int64_t)b * p.delta_batch + o);
+      const float d = p.delta_mode == 0 ? delta0 : __ldg(p.delta + (int64_t)b * p.delta_batch + o);
+      if (bt.error8_fast(v, p.delta_mode == 0 ? quot0 : QuotientPair(d), d)) return;
       const Quotient q(d);
 #pragma unroll
       for (int e = 0; e < 8; e += 2) bt.error2(v.v[e], v.v[e + 1], q(v.v[e]), q(v.v[e + 1]), d, d);
@@ -311,8 +412,9 @@ tensor_pass_kernel(const Lines p, double* __restrict__ partials, uint32_t* __res
   // loads in flight per thread: four for the bandwidth-bound statistics, two for the
   // arithmetic-bound error split (fewer registers, more resident warps)
   constexpr int U = KIND == kError ? 2 : 4;
+  Batch<KIND, FMT> bt;
   for (uint32_t g0 = blockIdx.x * kThreads + threadIdx.x; g0 < p.total_groups; g0 += U * stride) {
-    Batch<KIND, FMT> bt;
+    if (KIND == kStats) bt = Batch<KIND, FMT>();
     const bool full = whole_groups && (uint64_t)g0 + (uint64_t)(U - 1) * stride < p.total_groups;
     if (full) {
       // all loads of the batch are issued before any arithmetic
@@ -346,6 +448,7 @@ tensor_pass_kernel(const Lines p, double* __restrict__ partials, uint32_t* __res
     }
     bt.flush(acc);
   }
+  bt.finish(acc);
 
   finish_pass<KIND>(acc, partials, counter, result, count);
 }
@@ -421,7 +524,8 @@ qm_status launch_tensor_stats(const View& x, qm_tensor_stats_result* out, void* 
     QM_CUDA_OK(cudaMemsetAsync(counter, 0, sizeof(uint32_t), s));
     const uint64_t n_vec = bytes / 32;
     int64_t blocks = (int64_t)((n_vec + kThreads - 1) / kThreads);
-    const int64_t cap = (int64_t)sm_count() * 8 < kMaxBlocks ? (int64_t)sm_count() * 8 : kMaxBlocks;
+    // one wave: four blocks of this kernel's registers fit an SM
+    const int64_t cap = (int64_t)sm_count() * 4 < kMaxBlocks ? (int64_t)sm_count() * 4 : kMaxBlocks;
     if (blocks > cap) blocks = cap;
     const uint8_t* src = static_cast<const uint8_t*>(x.data);
     const bool stream = bytes > (64u << 20);
