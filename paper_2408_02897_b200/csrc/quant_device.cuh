@@ -155,6 +155,8 @@ struct QuotientPair {
 // GUARD: the scale may come from elsewhere, so x r can overflow and the corrections then evaluate
 // inf - inf; fminf returns its non-NaN operand, which turns that case into the largest float and
 // lets the conversion saturate, as the division would.
+// INT8 under the operand's own scale: |t| <= 127 (1 + 2^-23), so t + 1.5 2^23 is t rounded to nearest even
+// with its two's complement in the low mantissa bits, two elements per instruction and no conversion.
 template <int FMT, bool GUARD = false>
 __device__ __forceinline__ uint32_t quant_bf16_pair(uint32_t w, const QuotientPair& quot) {
   uint64_t x2;
@@ -168,7 +170,11 @@ __device__ __forceinline__ uint32_t quant_bf16_pair(uint32_t w, const QuotientPa
     return quant2<FMT>(__uint_as_float(q0), __uint_as_float(q1));
   }
   if (FMT == QM_FMT_INT8) {
-    return quant2<FMT>(__uint_as_float(q0), __uint_as_float(q1));
+    uint64_t magic, r2;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(magic) : "f"(12582912.f));
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r2) : "l"(q2), "l"(magic));
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(q0), "=r"(q1) : "l"(r2));
+    return __byte_perm(q0, q1, 0x0040);                     // (the upper half is not looked at)
   } else {
     // a negative input that rounds to zero is -0 in the FP8 formats: give the quotient its sign back
     q0 |= (w << 16) & 0x80000000u;
@@ -177,24 +183,22 @@ __device__ __forceinline__ uint32_t quant_bf16_pair(uint32_t w, const QuotientPa
   }
 }
 
+// Four codes of the four bf16 values in two words.
+template <int FMT, bool GUARD = false>
+__device__ __forceinline__ uint32_t quant_bf16_quad(uint32_t w0, uint32_t w1, const QuotientPair& quot) {
+  return __byte_perm(quant_bf16_pair<FMT, GUARD>(w0, quot), quant_bf16_pair<FMT, GUARD>(w1, quot), 0x5410);
+}
 // Sixteen codes of sixteen consecutive bf16 values (two 128-bit words).
 template <int FMT, bool GUARD = false>
 __device__ __forceinline__ uint4 quant_bf16x16(const uint4& a, const uint4& b, const QuotientPair& quot) {
-  uint4 r;
-  r.x = quant_bf16_pair<FMT, GUARD>(a.x, quot) | (quant_bf16_pair<FMT, GUARD>(a.y, quot) << 16);
-  r.y = quant_bf16_pair<FMT, GUARD>(a.z, quot) | (quant_bf16_pair<FMT, GUARD>(a.w, quot) << 16);
-  r.z = quant_bf16_pair<FMT, GUARD>(b.x, quot) | (quant_bf16_pair<FMT, GUARD>(b.y, quot) << 16);
-  r.w = quant_bf16_pair<FMT, GUARD>(b.z, quot) | (quant_bf16_pair<FMT, GUARD>(b.w, quot) << 16);
-  return r;
+  return make_uint4(quant_bf16_quad<FMT, GUARD>(a.x, a.y, quot), quant_bf16_quad<FMT, GUARD>(a.z, a.w, quot),
+                    quant_bf16_quad<FMT, GUARD>(b.x, b.y, quot), quant_bf16_quad<FMT, GUARD>(b.z, b.w, quot));
 }
 
 // Eight codes of eight consecutive bf16 values (one 128-bit word).
 template <int FMT, bool GUARD = false>
 __device__ __forceinline__ uint2 quant_bf16x8(const uint4& a, const QuotientPair& quot) {
-  uint2 r;
-  r.x = quant_bf16_pair<FMT, GUARD>(a.x, quot) | (quant_bf16_pair<FMT, GUARD>(a.y, quot) << 16);
-  r.y = quant_bf16_pair<FMT, GUARD>(a.z, quot) | (quant_bf16_pair<FMT, GUARD>(a.w, quot) << 16);
-  return r;
+  return make_uint2(quant_bf16_quad<FMT, GUARD>(a.x, a.y, quot), quant_bf16_quad<FMT, GUARD>(a.z, a.w, quot));
 }
 
 template <int FMT>
@@ -236,8 +240,19 @@ struct Rounding {
 // otherwise.  Both sides of the comparison are exact in fp32 (hi - lo is a power of two and
 // |t| - lo a difference inside one binade), so the decision equals the one taken in exact
 // arithmetic.  The sign of t is kept.
+//   In a format's normal range that comparison is one of whole numbers: with the grid m mantissa bits
+// wide and frac the 23 - m bits of |t| below it, u (hi - lo) < |t| - lo is (word >> 8) < frac << (m + 1),
+// which is (word >> (9 + m)) < frac; adding the complement of that draw to the magnitude's bits carries into the
+// grid's last bit exactly then.  What lies above the largest magnitude saturates in the conversion either way.
 template <int FMT>
 __device__ __forceinline__ float sr_value(float t, uint32_t word) {
+  if (FMT != QM_FMT_INT8) {
+    constexpr int m = FMT == QM_FMT_E4M3 ? 3 : 2;                        // mantissa bits
+    constexpr int emin = FMT == QM_FMT_E4M3 ? -6 : -14;                  // smallest normal exponent
+    constexpr uint32_t below = (1u << (23 - m)) - 1u;
+    if (fabsf(t) >= __uint_as_float((uint32_t)(127 + emin) << 23))
+      return __uint_as_float((__float_as_uint(t) + (~word >> (9 + m))) & ~below);
+  }
   const float a = fminf(fabsf(t), fmt_qmax(FMT));
   const float u = (float)(word >> 8) * 5.9604644775390625e-8f;          // 2^-24, exact
   float lo, spacing;
@@ -247,18 +262,42 @@ __device__ __forceinline__ float sr_value(float t, uint32_t word) {
   } else {
     constexpr int m = FMT == QM_FMT_E4M3 ? 3 : 2;                        // mantissa bits
     constexpr int emin = FMT == QM_FMT_E4M3 ? -6 : -14;                  // smallest normal exponent
-    const float min_normal = __uint_as_float((uint32_t)(127 + emin) << 23);
-    if (a >= min_normal) {
-      const uint32_t bits = __float_as_uint(a) & ~((1u << (23 - m)) - 1u);   // mantissa cut to m bits
-      lo = __uint_as_float(bits);
-      spacing = __uint_as_float(((bits >> 23) - m) << 23);
-    } else {
-      spacing = __uint_as_float((uint32_t)(127 + emin - m) << 23);       // the subnormal step
-      lo = floorf(a * __uint_as_float((uint32_t)(127 - emin + m) << 23)) * spacing;
-    }
+    spacing = __uint_as_float((uint32_t)(127 + emin - m) << 23);         // the subnormal step
+    lo = floorf(a * __uint_as_float((uint32_t)(127 - emin + m) << 23)) * spacing;
   }
   const float r = (u * spacing < a - lo) ? lo + spacing : lo;
   return copysignf(r, t);
+}
+
+// Four codes from four quotients and the four words of their counter block: sr_value and the conversion for four
+// elements together (its branch once per four, INT8 without conversion instructions but for the draw's).
+template <int FMT>
+__device__ __forceinline__ uint32_t sr_quad(const float (&t)[4], const uint32_t (&draw)[4]) {
+  float v[4];
+  if (FMT == QM_FMT_INT8) {
+    uint32_t c[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float a = fminf(fabsf(t[i]), 127.f);
+      const float lo = __fadd_rz(a, 8388608.f) - 8388608.f;                 // floor(a)
+      const float up = (float)(draw[i] >> 8) < (a - lo) * 16777216.f ? 1.f : 0.f;
+      // the code's two's complement in the low mantissa bits
+      c[i] = __float_as_uint(copysignf(lo + up, t[i]) + 12582912.f);
+    }
+    return __byte_perm(__byte_perm(c[0], c[1], 0x0040), __byte_perm(c[2], c[3], 0x0040), 0x5410);
+  } else {
+    constexpr int m = FMT == QM_FMT_E4M3 ? 3 : 2;                            // mantissa bits
+    constexpr int emin = FMT == QM_FMT_E4M3 ? -6 : -14;                      // smallest normal exponent
+    constexpr uint32_t below = (1u << (23 - m)) - 1u;
+    if (fminf(fminf(fabsf(t[0]), fabsf(t[1])), fminf(fabsf(t[2]), fabsf(t[3]))) >= __uint_as_float((uint32_t)(127 + emin) << 23)) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = __uint_as_float((__float_as_uint(t[i]) + below - (draw[i] >> (9 + m))) & ~below);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = sr_value<FMT>(t[i], draw[i]);
+    }
+    return __byte_perm(quant2<FMT>(v[0], v[1]), quant2<FMT>(v[2], v[3]), 0x5410);
+  }
 }
 
 // Eight consecutive elements whose first has number idx0 in the operand.  ALIGNED: idx0 is a
@@ -276,21 +315,55 @@ __device__ __forceinline__ uint2 quant8_sr(const Vec8& x, const Quotient& quot, 
     philox4x32_10((uint32_t)c, (uint32_t)(c >> 32), rnd.stream, 0u, rnd.k0, rnd.k1,
                   *reinterpret_cast<uint32_t(*)[4]>(&w[4 * b]));
   }
-  float t[8];
+  uint32_t r[2];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    uint32_t word = w[i];
-    if (!ALIGNED) {
-      // word first + i without dynamic indexing of the register array
+  for (int h = 0; h < 2; ++h) {
+    float t[4];
+    uint32_t word[4];
 #pragma unroll
-      for (int f = 1; f < 4; ++f)
-        if (first == f) word = w[f + i];
+    for (int i = 0; i < 4; ++i) {
+      word[i] = w[4 * h + i];
+      if (!ALIGNED) {
+        // word first + i without dynamic indexing of the register array
+#pragma unroll
+        for (int f = 1; f < 4; ++f)
+          if (first == f) word[i] = w[f + 4 * h + i];
+      }
+      t[i] = quot(x.v[4 * h + i]);
     }
-    t[i] = sr_value<FMT>(quot(x.v[i]), word);
+    r[h] = sr_quad<FMT>(t, word);
   }
-  uint2 r;
-  r.x = quant2<FMT>(t[0], t[1]) | (quant2<FMT>(t[2], t[3]) << 16);
-  r.y = quant2<FMT>(t[4], t[5]) | (quant2<FMT>(t[6], t[7]) << 16);
+  return make_uint2(r[0], r[1]);
+}
+// Sixteen consecutive bf16 values whose first has a number divisible by four, under a scale the two-wide
+// quotient serves.
+template <int FMT, bool GUARD>
+__device__ __forceinline__ uint4 quant_bf16x16_sr(const uint4& a, const uint4& b, const QuotientPair& quot, const Rounding& rnd,
+                                                  uint64_t idx0) {
+  uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+  uint4 r = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    uint32_t draw[4];
+    const uint64_t blk = (idx0 >> 2) + k;
+    philox4x32_10((uint32_t)blk, (uint32_t)(blk >> 32), rnd.stream, 0u, rnd.k0, rnd.k1, draw);
+    float t[4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint32_t x = w[h];
+      uint64_t x2;
+      asm("mov.b64 %0, {%1, %2};" : "=l"(x2) : "r"(x << 16), "r"(x & 0xffff0000u));
+      const uint64_t q2 = quot(x2);
+      float q0, q1;
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(q0), "=f"(q1) : "l"(q2));
+      if (GUARD) { q0 = fminf(fabsf(q0), 3.402823466e38f); q1 = fminf(fabsf(q1), 3.402823466e38f); }
+      t[2 * h] = copysignf(q0, __uint_as_float(x << 16));            // keeps the sign of a zero input
+      t[2 * h + 1] = copysignf(q1, __uint_as_float(x));
+    }
+    r = make_uint4(r.y, r.z, r.w, sr_quad<FMT>(t, draw));
+#pragma unroll
+    for (int h = 0; h < 6; ++h) w[h] = w[h + 2];
+  }
   return r;
 }
 // The same, choosing the variant from idx0 (uniform over a launch whenever rows are a multiple of 4 long).

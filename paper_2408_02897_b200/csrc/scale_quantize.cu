@@ -13,10 +13,12 @@ namespace {
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
 absmax_tensor_kernel(const T* __restrict__ x, int64_t rows, int64_t c, int64_t row_stride,
-                     uint32_t* __restrict__ amax) {
+                     const FastDiv by_vec, uint32_t* __restrict__ amax) {
   pdl_prologue();
   const int64_t vec_per_row = c >> 3;
   const int64_t total_vec = rows * vec_per_row;
+  const bool narrow = total_vec < (1ll << 32);       // by_vec divides 32-bit indices by vec_per_row
+  auto row_of = [&](int64_t j) { return narrow ? (int64_t)by_vec.div((uint32_t)j) : j / vec_per_row; };
   uint32_t acc = 0;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -49,14 +51,14 @@ absmax_tensor_kernel(const T* __restrict__ x, int64_t rows, int64_t c, int64_t r
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         int64_t j = i + u * stride;
-        int64_t r = j / vec_per_row, k = j - r * vec_per_row;
+        const int64_t r = row_of(j), k = j - r * vec_per_row;
         v[u] = Loader<T>::load8(x + r * row_stride + k * 8);
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) acc = absmax8(v[u], acc);
     }
     for (; i < total_vec; i += stride) {
-      int64_t r = i / vec_per_row, k = i - r * vec_per_row;
+      const int64_t r = row_of(i), k = i - r * vec_per_row;
       acc = absmax8(Loader<T>::load8(x + r * row_stride + k * 8), acc);
     }
   }
@@ -346,6 +348,35 @@ quantize_dense_kernel(const uint4* __restrict__ x, uint32_t total_chunks, const 
   }
 }
 
+// The same tensors with stochastic rounding: a thread takes one chunk of sixteen elements, four counter blocks.
+// Bound by the draws (ten rounds of two wide multiplications per four elements) beside HBM: 16384 x 4096
+// with its max|x| pass 138 us one element at a time, 103 us so.
+template <int FMT>
+__global__ void __launch_bounds__(kThreads, 4)
+quantize_dense_sr_kernel(const uint4* __restrict__ x, uint32_t total_chunks, const DeltaSrc ds, const FastDiv by_chunks,
+                         uint32_t chunks_per_row, uint4* __restrict__ codes, const Rounding rnd) {
+  pdl_prologue();
+  const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
+  if (i >= total_chunks) return;
+  const uint4 a = __ldg(x + 2 * (size_t)i), b = __ldg(x + 2 * (size_t)i + 1);
+  uint32_t row = 0;
+  if (ds.per_channel) row = by_chunks.div(i);
+  const float d = ds.per_channel ? ds.get(row, i == row * chunks_per_row) : ds.get(0, i == 0);
+  const uint64_t number = (uint64_t)i * 16u;              // of the chunk's first element: rows are dense
+  if (QuotientPair::serves(d)) {
+    const QuotientPair qp(d);
+    codes[i] = ds.from_amax ? quant_bf16x16_sr<FMT, false>(a, b, qp, rnd, number) : quant_bf16x16_sr<FMT, true>(a, b, qp, rnd, number);
+    return;
+  }
+  const Quotient quot(d);
+  const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+  Vec8 f[2];
+#pragma unroll
+  for (int h = 0; h < 8; ++h) { f[h >> 2].v[2 * (h & 3)] = bf16_lo(w[h]); f[h >> 2].v[2 * (h & 3) + 1] = bf16_hi(w[h]); }
+  const uint2 q0 = quant8_sr<FMT, true>(f[0], quot, rnd, number), q1 = quant8_sr<FMT, true>(f[1], quot, rnd, number + 8);
+  codes[i] = make_uint4(q0.x, q0.y, q1.x, q1.y);
+}
+
 // ---------------------------------------------------------------- several formats in one pass
 // A sweep of formats quantizes the same tensor two or three times (Table 1).  These kernels read
 // it once and write the codes of every format in MASK (bit f = qm_format f), with per-tensor
@@ -432,7 +463,8 @@ quantize_dense_multi_kernel(const uint4* __restrict__ x, uint32_t total_chunks, 
 }
 
 // ---------------------------------------------------------------- quantize + transpose through shared memory
-// Storage [c][nc] (nc contiguous, bf16), c a multiple of 128 and nc a multiple of 64.  A block
+// Storage [c][nc] (nc contiguous, bf16), c a multiple of 16 (EDGE: c not a multiple of 128 or nc not one of 64;
+// rows and columns beyond the matrix are loaded as zeros and not written).  A block
 // takes a tile of 128 contraction rows x 64 columns: it loads the tile with whole-line reads (8
 // threads per 128-byte row), reads it back column-wise (a thread takes 16 contraction entries of two
 // adjacent columns; consecutive lanes read consecutive words: conflict-free), quantizes, and hands
@@ -440,21 +472,51 @@ quantize_dense_multi_kernel(const uint4* __restrict__ x, uint32_t total_chunks, 
 // output row) to global memory through a second shared-memory tile so that every store instruction
 // writes whole lines: 16-byte chunk ch of output row n sits at ch ^ ((n >> 1) & 7), which keeps
 // both the column-wise writes and the row-wise reads of that tile conflict-free.
+template <int MASK> struct TileSmem {
+  static constexpr int kFormats = (MASK & 1) + (MASK >> 1 & 1) + (MASK >> 2 & 1);
+  static constexpr int kVec = kFormats * 64 * 8 + 64 * 16;        // 16-byte units: 24, 32 or 40 KB for one, two or three formats
+  static __device__ __forceinline__ int slot(int f) { return (f > 0 ? MASK & 1 : 0) + (f > 1 ? MASK >> 1 & 1 : 0); }
+};
 // d_lo / d_hi: the scales of the thread's two columns, per format in MASK (bit f = qm_format f).
-template <int MASK, bool GUARD>
+// SR: stochastic rounding (rnd); c is a multiple of 4, so sixteen entries are four counter blocks.
+template <int MASK, bool GUARD, bool EDGE, bool SR = false>
 __device__ __forceinline__ void transpose_tile(const __nv_bfloat16* __restrict__ x, int64_t nc, int64_t c, int64_t s_c,
                                                int64_t s_b, const float (&d_lo)[3], const float (&d_hi)[3],
                                                uint8_t* const (&codes)[3], int64_t ldc,
-                                               __nv_bfloat16* __restrict__ kmaj_copy, uint4* smem) {
+                                               __nv_bfloat16* __restrict__ kmaj_copy, uint4* smem,
+                                               const Rounding& rnd = Rounding{}) {
   const int t = threadIdx.x;
   const int64_t b = blockIdx.z, n0 = (int64_t)blockIdx.x * 64, k0 = (int64_t)blockIdx.y * 128;
-  // phase 1: 128 rows x 128 bytes, four 16-byte loads per thread in flight
-  {
+  const int64_t pitch = s_c >> 3;                                     // row stride in 16-byte units
+  // 128 rows x 128 bytes, four 16-byte loads per thread in flight
+  auto fetch = [&](uint4 (&v)[4]) {
     const uint4* src = reinterpret_cast<const uint4*>(x + b * s_b + k0 * s_c + n0);
-    const int64_t pitch = s_c >> 3;                                   // row stride in 16-byte units
-    uint4 v[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) v[i] = __ldg(src + (int64_t)((t >> 3) + 32 * i) * pitch + (t & 7));
+    for (int i = 0; i < 4; ++i) {
+      const int64_t at = (int64_t)((t >> 3) + 32 * i) * pitch + (t & 7);
+      if (!EDGE) {
+        v[i] = __ldg(src + at);
+      } else {
+        const int64_t left = nc - (n0 + 8 * (t & 7));                // columns of this vector that exist
+        v[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (k0 + (t >> 3) + 32 * i < c && left > 0) {
+          if (left >= 8) {
+            v[i] = __ldg(src + at);
+          } else {
+            const unsigned short* e = reinterpret_cast<const unsigned short*>(src + at);
+            uint32_t h[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) h[j] = j < left ? (uint32_t)__ldg(e + j) : 0u;
+            v[i] = make_uint4(h[0] | h[1] << 16, h[2] | h[3] << 16, h[4] | h[5] << 16, h[6] | h[7] << 16);
+          }
+        }
+      }
+    }
+  };
+  // phase 1: the tile into shared memory
+  {
+    uint4 v[4];
+    fetch(v);
 #pragma unroll
     for (int i = 0; i < 4; ++i) smem[((t >> 3) + 32 * i) * 8 + (t & 7)] = v[i];
   }
@@ -465,16 +527,16 @@ __device__ __forceinline__ void transpose_tile(const __nv_bfloat16* __restrict__
 #pragma unroll
   for (int j = 0; j < 16; ++j) w[j] = reinterpret_cast<const uint32_t*>(smem)[(16 * g + j) * 32 + pcol];
   __syncthreads();                                                     // the output tiles reuse the input tile's memory
-  uint4* const s_codes = smem;                                         // [3][64 rows][8 chunks]
-  uint4* const s_kmaj = smem + 3 * 64 * 8;                             // [64 rows][16 chunks]
+  uint4* const s_codes = smem;                                         // [formats][64 rows][8 chunks]
+  uint4* const s_kmaj = s_codes + TileSmem<MASK>::kFormats * 64 * 8;   // [64 rows][16 chunks]
   const uint32_t sw = (uint32_t)pcol & 7u;
-#pragma unroll
+#pragma unroll SR ? 1 : 2
   for (int col = 0; col < 2; ++col) {
     const int n = 2 * pcol + col;
     uint32_t pw[8];                                                    // this column's 16 values, two bf16 per word
 #pragma unroll
     for (int j = 0; j < 8; ++j)
-      pw[j] = col == 0 ? __byte_perm(w[2 * j], w[2 * j + 1], 0x5410) : __byte_perm(w[2 * j], w[2 * j + 1], 0x7632);
+      pw[j] = __byte_perm(w[2 * j], w[2 * j + 1], col == 0 ? 0x5410 : 0x7632);
     const uint4 a = make_uint4(pw[0], pw[1], pw[2], pw[3]), bb = make_uint4(pw[4], pw[5], pw[6], pw[7]);
     if (kmaj_copy) {
       s_kmaj[n * 16 + ((2 * g) ^ sw)] = a;
@@ -485,9 +547,11 @@ __device__ __forceinline__ void transpose_tile(const __nv_bfloat16* __restrict__
       if (!(MASK & (1 << f))) continue;
       const float d = col == 0 ? d_lo[f] : d_hi[f];
       uint4 cw;
+      const uint64_t number = (uint64_t)(b * nc + n0 + n) * (uint64_t)c + (uint64_t)(k0 + 16 * g);    // of the first entry
       if (QuotientPair::serves(d)) {
         const QuotientPair qp(d);
-        cw = f == 0 ? quant_bf16x16<0, GUARD>(a, bb, qp) : f == 1 ? quant_bf16x16<1, GUARD>(a, bb, qp) : quant_bf16x16<2, GUARD>(a, bb, qp);
+        if (SR) cw = f == 0 ? quant_bf16x16_sr<0, GUARD>(a, bb, qp, rnd, number) : f == 1 ? quant_bf16x16_sr<1, GUARD>(a, bb, qp, rnd, number) : quant_bf16x16_sr<2, GUARD>(a, bb, qp, rnd, number);
+        else cw = f == 0 ? quant_bf16x16<0, GUARD>(a, bb, qp) : f == 1 ? quant_bf16x16<1, GUARD>(a, bb, qp) : quant_bf16x16<2, GUARD>(a, bb, qp);
       } else {
         const Quotient quot(d);
         Vec8 lo, hi;
@@ -496,11 +560,17 @@ __device__ __forceinline__ void transpose_tile(const __nv_bfloat16* __restrict__
           lo.v[2 * j] = bf16_lo(pw[j]); lo.v[2 * j + 1] = bf16_hi(pw[j]);
           hi.v[2 * j] = bf16_lo(pw[4 + j]); hi.v[2 * j + 1] = bf16_hi(pw[4 + j]);
         }
-        const uint2 q0 = f == 0 ? quant8<0>(lo, quot) : f == 1 ? quant8<1>(lo, quot) : quant8<2>(lo, quot);
-        const uint2 q1 = f == 0 ? quant8<0>(hi, quot) : f == 1 ? quant8<1>(hi, quot) : quant8<2>(hi, quot);
+        uint2 q0, q1;
+        if (SR) {
+          q0 = f == 0 ? quant8_sr<0, true>(lo, quot, rnd, number) : f == 1 ? quant8_sr<1, true>(lo, quot, rnd, number) : quant8_sr<2, true>(lo, quot, rnd, number);
+          q1 = f == 0 ? quant8_sr<0, true>(hi, quot, rnd, number + 8) : f == 1 ? quant8_sr<1, true>(hi, quot, rnd, number + 8) : quant8_sr<2, true>(hi, quot, rnd, number + 8);
+        } else {
+          q0 = f == 0 ? quant8<0>(lo, quot) : f == 1 ? quant8<1>(lo, quot) : quant8<2>(lo, quot);
+          q1 = f == 0 ? quant8<0>(hi, quot) : f == 1 ? quant8<1>(hi, quot) : quant8<2>(hi, quot);
+        }
         cw = make_uint4(q0.x, q0.y, q1.x, q1.y);
       }
-      s_codes[(f * 64 + n) * 8 + ((uint32_t)g ^ sw)] = cw;
+      s_codes[(TileSmem<MASK>::slot(f) * 64 + n) * 8 + ((uint32_t)g ^ sw)] = cw;
     }
   }
   __syncthreads();
@@ -511,7 +581,8 @@ __device__ __forceinline__ void transpose_tile(const __nv_bfloat16* __restrict__
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const int row = (t >> 3) + 32 * i, ch = t & 7;
-      const uint4 v = s_codes[(f * 64 + row) * 8 + (ch ^ ((row >> 1) & 7))];
+      if (EDGE && (n0 + row >= nc || k0 + ch * 16 >= ldc)) continue;
+      const uint4 v = s_codes[(TileSmem<MASK>::slot(f) * 64 + row) * 8 + (ch ^ ((row >> 1) & 7))];
       *reinterpret_cast<uint4*>(codes[f] + (b * nc + n0 + row) * ldc + k0 + ch * 16) = v;
     }
   }
@@ -519,48 +590,47 @@ __device__ __forceinline__ void transpose_tile(const __nv_bfloat16* __restrict__
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int row = (t >> 4) + 16 * i, ch = t & 15;
+      if (EDGE && (n0 + row >= nc || k0 + ch * 8 >= c)) continue;
       const uint4 v = s_kmaj[row * 16 + (ch ^ ((row >> 1) & 7))];
       *reinterpret_cast<uint4*>(kmaj_copy + (b * nc + n0 + row) * c + k0 + ch * 8) = v;
     }
   }
 }
 
-constexpr int kTileSmemVec = 3 * 64 * 8 + 64 * 16;                    // 40 KB in 16-byte units
-
 // One format, scales from a DeltaSrc (per tensor or per output row, finished or from max|x|).
-template <int FMT>
-__global__ void __launch_bounds__(kThreads)
+template <int FMT, bool EDGE, bool SR>
+__global__ void __launch_bounds__(kThreads, SR ? 3 : 1)
 quantize_transpose_tile_kernel(const __nv_bfloat16* __restrict__ x, int64_t nc, int64_t c, int64_t s_c, int64_t s_b,
                                const DeltaSrc ds, uint8_t* __restrict__ codes, int64_t ldc,
-                               __nv_bfloat16* __restrict__ kmaj_copy) {
+                               __nv_bfloat16* __restrict__ kmaj_copy, const Rounding rnd) {
   pdl_prologue();
-  __shared__ uint4 smem[kTileSmemVec];
+  __shared__ uint4 smem[TileSmem<1 << FMT>::kVec];
   const int pcol = threadIdx.x & 31, g = threadIdx.x >> 5;
-  const int64_t orow = (int64_t)blockIdx.z * nc + (int64_t)blockIdx.x * 64 + 2 * pcol;
+  const int64_t col = (int64_t)blockIdx.x * 64 + 2 * pcol, orow = (int64_t)blockIdx.z * nc + col;
   float d_lo[3] = {1.f, 1.f, 1.f}, d_hi[3] = {1.f, 1.f, 1.f};
   if (ds.per_channel) {
-    d_lo[FMT] = ds.get(orow, blockIdx.y == 0 && g == 0);
-    d_hi[FMT] = ds.get(orow + 1, blockIdx.y == 0 && g == 0);
+    if (!EDGE || col < nc) d_lo[FMT] = ds.get(orow, blockIdx.y == 0 && g == 0);
+    if (!EDGE || col + 1 < nc) d_hi[FMT] = ds.get(orow + 1, blockIdx.y == 0 && g == 0);
   } else {
     d_lo[FMT] = d_hi[FMT] = ds.get(0, blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0);
   }
   uint8_t* const cd[3] = {codes, codes, codes};
-  if (ds.from_amax) transpose_tile<1 << FMT, false>(x, nc, c, s_c, s_b, d_lo, d_hi, cd, ldc, kmaj_copy, smem);
-  else transpose_tile<1 << FMT, true>(x, nc, c, s_c, s_b, d_lo, d_hi, cd, ldc, kmaj_copy, smem);
+  if (ds.from_amax) transpose_tile<1 << FMT, false, EDGE, SR>(x, nc, c, s_c, s_b, d_lo, d_hi, cd, ldc, kmaj_copy, smem, rnd);
+  else transpose_tile<1 << FMT, true, EDGE, SR>(x, nc, c, s_c, s_b, d_lo, d_hi, cd, ldc, kmaj_copy, smem, rnd);
 }
 
 // Every format in MASK from one read, per-tensor scales from the tensor's max|x|.
-template <int MASK>
+template <int MASK, bool EDGE>
 __global__ void __launch_bounds__(kThreads)
 quantize_transpose_tile_multi_kernel(const __nv_bfloat16* __restrict__ x, int64_t nc, int64_t c, int64_t s_c,
                                      int64_t s_b, const uint32_t* __restrict__ amax, const MultiOut o, int64_t ldc,
                                      __nv_bfloat16* __restrict__ kmaj_copy) {
   pdl_prologue();
-  __shared__ uint4 smem[kTileSmemVec];
+  __shared__ uint4 smem[TileSmem<MASK>::kVec];
   float d[3];
   multi_scales<MASK>(amax, o, blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0, d);
   uint8_t* const cd[3] = {o.codes[0], o.codes[1], o.codes[2]};
-  transpose_tile<MASK, false>(x, nc, c, s_c, s_b, d, d, cd, ldc, kmaj_copy, smem);
+  transpose_tile<MASK, false, EDGE>(x, nc, c, s_c, s_b, d, d, cd, ldc, kmaj_copy, smem);
 }
 
 // ---------------------------------------------------------------- fused per-row scale + quantize
@@ -834,7 +904,7 @@ void absmax_dense(const T* p, int64_t n, uint32_t* amax, cudaStream_t s) {
   const uintptr_t a0 = reinterpret_cast<uintptr_t>(p), a1 = a0 + (uintptr_t)n * sizeof(T);
   const uintptr_t m0 = (a0 + 31) & ~(uintptr_t)31, m1 = a1 & ~(uintptr_t)31;
   if (m1 <= m0) {
-    launch_pdl(absmax_tensor_kernel<T>, dim3(1), dim3(kThreads), 0, s, p, 1, n, n, amax);
+    launch_pdl(absmax_tensor_kernel<T>, dim3(1), dim3(kThreads), 0, s, p, 1, n, n, FastDiv(), amax);
     return;
   }
   const uint64_t n_vec = (m1 - m0) / 32;
@@ -845,9 +915,12 @@ void absmax_dense(const T* p, int64_t n, uint32_t* amax, cudaStream_t s) {
   else
     launch_pdl(absmax_dense_kernel<T, 4, false>, grid, dim3(kThreads), 0, s, mid, n_vec, amax);
   const int64_t head = (int64_t)((m0 - a0) / sizeof(T)), tail = (int64_t)((a1 - m1) / sizeof(T));
-  if (head > 0) launch_pdl(absmax_tensor_kernel<T>, dim3(1), dim3(32), 0, s, p, 1, head, head, amax);
-  if (tail > 0) launch_pdl(absmax_tensor_kernel<T>, dim3(1), dim3(32), 0, s, p + (n - tail), 1, tail, tail, amax);
+  if (head > 0) launch_pdl(absmax_tensor_kernel<T>, dim3(1), dim3(32), 0, s, p, 1, head, head, FastDiv(), amax);
+  if (tail > 0) launch_pdl(absmax_tensor_kernel<T>, dim3(1), dim3(32), 0, s, p + (n - tail), 1, tail, tail, FastDiv(), amax);
 }
+
+// divisor of absmax_tensor_kernel for rows of n elements (of no use, and not used, below 8 or from 2^35 on)
+FastDiv vec_div(int64_t n) { return n / 8 > 0 && n / 8 < (1ll << 32) ? FastDiv((uint32_t)(n / 8)) : FastDiv(); }
 
 template <typename T>
 qm_status absmax_t(const View& x, int gran, uint32_t* amax, cudaStream_t s) {
@@ -861,11 +934,11 @@ qm_status absmax_t(const View& x, int gran, uint32_t* amax, cudaStream_t s) {
         absmax_dense<T>(p, n, amax, s);
       } else if (even) {
         launch_pdl(absmax_tensor_kernel<T>, dim3(grid_for(x.nc * x.batch * x.c / 8 + 1, 8)), dim3(kThreads), 0, s, 
-            p, x.nc * x.batch, x.c, x.s_nc, amax);
+            p, x.nc * x.batch, x.c, x.s_nc, vec_div(x.c), amax);
       } else {
         for (int64_t b = 0; b < x.batch; ++b)
           launch_pdl(absmax_tensor_kernel<T>, dim3(grid_for(x.nc * x.c / 8 + 1, 8)), dim3(kThreads), 0, s, 
-              p + b * x.s_b, x.nc, x.c, x.s_nc, amax);
+              p + b * x.s_b, x.nc, x.c, x.s_nc, vec_div(x.c), amax);
       }
     } else {
       const int64_t rows = x.nc * x.batch;
@@ -890,11 +963,11 @@ qm_status absmax_t(const View& x, int gran, uint32_t* amax, cudaStream_t s) {
           absmax_dense<T>(p, n, amax, s);
         else
           launch_pdl(absmax_tensor_kernel<T>, dim3(grid_for(n / 8 + 1, 8)), dim3(kThreads), 0, s,
-              p, x.c * x.batch, x.nc, x.s_c, amax);
+              p, x.c * x.batch, x.nc, x.s_c, vec_div(x.nc), amax);
       } else {
         for (int64_t b = 0; b < x.batch; ++b)
           launch_pdl(absmax_tensor_kernel<T>, dim3(grid_for(x.nc * x.c / 8 + 1, 8)), dim3(kThreads), 0, s,
-              p + b * x.s_b, x.c, x.nc, x.s_c, amax);
+              p + b * x.s_b, x.c, x.nc, x.s_c, vec_div(x.nc), amax);
       }
     } else {
       const int64_t col_blocks = (x.nc + 255) / 256;
@@ -912,12 +985,13 @@ qm_status absmax_t(const View& x, int gran, uint32_t* amax, cudaStream_t s) {
   return QM_OK;
 }
 
-// The shared-memory transposing kernels serve bf16 views whose contraction is strided, in whole
-// tiles of 128 contraction entries x 64 columns.
+// The shared-memory transposing kernels serve bf16 views whose contraction is strided and a multiple of 16
+// long (codes and copy then go out in whole 16-byte vectors), in tiles of 128 contraction entries x 64 columns.
 bool tile_transposable(const View& x) {
-  return x.dtype == QM_DT_BF16 && !x.c_contig() && (x.c & 127) == 0 && (x.nc & 63) == 0 && x.c / 128 <= 65535 &&
-         x.batch <= 65535;
+  return x.dtype == QM_DT_BF16 && !x.c_contig() && (x.c & 15) == 0 && (x.c + 127) / 128 <= 65535 && x.batch <= 65535;
 }
+bool tile_edges(const View& x) { return (x.c & 127) || (x.nc & 63); }
+dim3 tile_grid(const View& x) { return dim3((unsigned)((x.nc + 63) / 64), (unsigned)((x.c + 127) / 128), (unsigned)x.batch); }
 
 template <typename T, int FMT>
 qm_status quantize_t(const View& x, int gran, const float* delta, bool from_amax, float* delta_out,
@@ -931,10 +1005,12 @@ qm_status quantize_t(const View& x, int gran, const float* delta, bool from_amax
   if (x.c_contig()) {
     const int64_t total = x.nc * x.batch * (ldc >> 4);
     if (total >= (1ll << 32) || x.nc >= (1ll << 32)) return QM_ERR_UNSUPPORTED;   // 32-bit chunk index
-    // (stochastic rounding takes the general kernels: the draws cost more than the fast paths save)
-    const bool dense = !rnd.stochastic && x.dtype == QM_DT_BF16 && x.s_nc == x.c && (x.c & 15) == 0 &&
-                       (x.batch == 1 || x.s_b == x.nc * x.c);
-    if (dense) {
+    const bool dense = x.dtype == QM_DT_BF16 && x.s_nc == x.c && (x.c & 15) == 0 && (x.batch == 1 || x.s_b == x.nc * x.c);
+    if (dense && rnd.stochastic && !abs_copy) {
+      launch_pdl(quantize_dense_sr_kernel<FMT>, dim3((unsigned)((total + kThreads - 1) / kThreads)), dim3(kThreads), 0, s,
+                 reinterpret_cast<const uint4*>(x.data), (uint32_t)total, ds, FastDiv((uint32_t)(ldc >> 4)), (uint32_t)(ldc >> 4),
+                 reinterpret_cast<uint4*>(codes), rnd);
+    } else if (dense && !rnd.stochastic) {
       const uint4* src = reinterpret_cast<const uint4*>(x.data);
       const FastDiv by_chunks((uint32_t)(ldc >> 4));
       const bool big = total >= (int64_t)sm_count() * 8 * kThreads * 4;
@@ -960,11 +1036,14 @@ qm_status quantize_t(const View& x, int gran, const float* delta, bool from_amax
                                      x.c * 2, x.nc, cudaMemcpyDeviceToDevice, s));
     }
   } else {
-    if (!rnd.stochastic && !abs_copy && tile_transposable(x)) {
-      dim3 grid((unsigned)(x.nc / 64), (unsigned)(x.c / 128), (unsigned)x.batch);
-      launch_pdl(quantize_transpose_tile_kernel<FMT>, dim3(grid), dim3(kThreads), 0, s,
-                 static_cast<const __nv_bfloat16*>(x.data), x.nc, x.c, x.s_c, x.s_b, ds, codes, ldc,
-                 static_cast<__nv_bfloat16*>(kmaj_copy));
+    if (!abs_copy && tile_transposable(x)) {
+#define QM_TT(E, S)                                                                                            \
+  launch_pdl(quantize_transpose_tile_kernel<FMT, E, S>, tile_grid(x), dim3(kThreads), 0, s,                    \
+             static_cast<const __nv_bfloat16*>(x.data), x.nc, x.c, x.s_c, x.s_b, ds, codes, ldc,               \
+             static_cast<__nv_bfloat16*>(kmaj_copy), rnd)
+      if (tile_edges(x)) { if (rnd.stochastic) QM_TT(true, true); else QM_TT(true, false); }
+      else { if (rnd.stochastic) QM_TT(false, true); else QM_TT(false, false); }
+#undef QM_TT
       count_launch();
       QM_CUDA_OK(cudaGetLastError());
       return QM_OK;
@@ -1119,10 +1198,11 @@ qm_status launch_quantize_multi(const View& x, int gran, const uint32_t* amax, i
     }
 #undef QM_DM
   } else {
-    dim3 grid((unsigned)(x.nc / 64), (unsigned)(x.c / 128), (unsigned)x.batch);
     const __nv_bfloat16* src = static_cast<const __nv_bfloat16*>(x.data);
     __nv_bfloat16* km = static_cast<__nv_bfloat16*>(kmaj_copy);
-#define QM_TM(M) launch_pdl(quantize_transpose_tile_multi_kernel<M>, grid, dim3(kThreads), 0, s, src, x.nc, x.c, x.s_c, x.s_b, amax, o, ldc, km)
+#define QM_TM(M)                                                                                                                                          \
+  launch_pdl(tile_edges(x) ? quantize_transpose_tile_multi_kernel<M, true> : quantize_transpose_tile_multi_kernel<M, false>, tile_grid(x), \
+             dim3(kThreads), 0, s, src, x.nc, x.c, x.s_c, x.s_b, amax, o, ldc, km)
     switch (mask) {
       case 3: QM_TM(3); break;
       case 5: QM_TM(5); break;
