@@ -358,10 +358,11 @@ qm_status qm_quantize_error(const qm_operand* x, int32_t fmt, int32_t gran, cons
  * ws_bytes[i]) computes.  The probes are independent, so the library runs the
  * scale/quantize kernels of all operands beside one another on a few streams of
  * its own (created on the first call on each device, kept until the process
- * exits) and then the fused kernels of all tensor-core probes as one persistent
- * launches of up to 16 probes over the tiles of all of them (the sums of a
- * record are then taken over another tile-to-CTA assignment than in
- * qm_probe_layer and may differ in the last bits).  A measurement pass asks
+ * exits) and then the fused kernel over the tiles of all tensor-core probes, in
+ * as few persistent launches as hold them.  Probes of the same two operands
+ * share their reference and denominator products (the sums of a record are
+ * taken over another tile-to-CTA assignment than in qm_probe_layer and may
+ * differ in the last bits).  A measurement pass asks
  * for the same preparation many times over (a sweep of formats over one layer,
  * an activation that feeds several products, a gradient that appears in dgrad
  * and wgrad): inside a batch, operands that describe the same memory (same
