@@ -607,8 +607,9 @@ qm_status qm_probe_layer_host(const qm_operand* L_host, const qm_operand* R_host
 // ---- batches of probes over the library's own streams ------------------------------------------
 namespace {
 constexpr int kBatchStreams = 8;      // streams of the pool
-constexpr int kCopyEvents = 64;       // chunks of a host batch that can wait for their own copies
-constexpr int kHostChunk = 16;        // probes of a chunk of a host batch
+constexpr int kCopyEvents = 64;       // a host batch's chunks take turns with these events
+constexpr int kHostChunk = 16;        // probes of a chunk of a host batch, at most
+constexpr size_t kHostChunkBytes = 8u << 20;    // and the copies after which a chunk ends with its product
 struct BatchStreams {
   std::mutex issue;            // one batch at a time is put into the streams (host side only)
   bool ready = false;
@@ -921,23 +922,26 @@ qm_status qm_probe_batch_host(int32_t n, const qm_operand* L_host, const qm_oper
   qm_status st = batch_streams(&bs);
   if (st != QM_OK) return st;
   // Every distinct host operand is copied once, on a stream of the library's own and in the order
-  // in which the probes first name them.  The probes go to the device in chunks of
-  // kHostChunk, each chunk as a device batch (which prepares every distinct operand of the
-  // chunk once) that waits only for the copies it needs: the copies of later chunks run under the
-  // kernels of earlier ones.  Order the probes so that those of one product are neighbours and the
-  // first chunks need only the first tensors.
+  // in which the probes first name them.  The probes go to the device in chunks, each chunk as a device
+  // batch (which prepares every distinct operand of the chunk once) that waits only for the copies it
+  // needs: the copies of later chunks run under the kernels of earlier ones.  A chunk ends after
+  // kHostChunk probes, or with the product at which it has brought kHostChunkBytes: 8 MB are about 150 us of
+  // the link, several times what a further chunk costs in launches, and what is left for the end is the
+  // kernels of the last product alone.  Order the probes so that those of one product are neighbours and
+  // the first chunks need only the first tensors.
   std::vector<qm_operand> Ld((size_t)n), Rd((size_t)n);
   std::vector<HostCopy> seen;
-  const int32_t chunk = kHostChunk;
-  const bool pipelined = (n + chunk - 1) / chunk <= kCopyEvents;
   std::lock_guard<std::mutex> lock(bs->host_issue);
   QM_CUDA_OK(cudaEventRecord(bs->copy_fork, user));               // the copies follow the work already in the stream
   QM_CUDA_OK(cudaStreamWaitEvent(bs->copy, bs->copy_fork, 0));
   qm_status refused = QM_OK;
-  int32_t good = 0, issued = 0;
-  for (int32_t c0 = 0; c0 < n && st == QM_OK && refused == QM_OK; c0 += chunk) {
-    const int32_t c1 = c0 + chunk < n ? c0 + chunk : n;
-    for (good = c0; good < c1; ++good) {
+  int32_t good = 0, issued = 0, n_chunks = 0;
+  while (good < n && st == QM_OK && refused == QM_OK) {
+    const int32_t c0 = good, c1 = c0 + kHostChunk < n ? c0 + kHostChunk : n;
+    size_t copied = 0;
+    for (; good < c1; ++good) {
+      if (copied >= kHostChunkBytes && (L_host[good].data != L_host[good - 1].data || R_host[good].data != R_host[good - 1].data))
+        break;
       for (int side = 0; side < 2 && refused == QM_OK; ++side) {
         const qm_operand& x = side ? R_host[good] : L_host[good];
         void* stage = side ? r_stage[good] : l_stage[good];
@@ -947,6 +951,7 @@ qm_status qm_probe_batch_host(int32_t n, const qm_operand* L_host, const qm_oper
         if (!dev) {
           QM_CUDA_OK(cudaMemcpyAsync(stage, x.data, bytes, cudaMemcpyHostToDevice, bs->copy));
           seen.push_back(HostCopy{x.data, bytes, stage});
+          copied += bytes;
           dev = stage;
         }
         qm_operand& d = side ? Rd[good] : Ld[good];
@@ -956,14 +961,14 @@ qm_status qm_probe_batch_host(int32_t n, const qm_operand* L_host, const qm_oper
       if (refused != QM_OK) break;
     }
     // this chunk's copies (and all earlier ones) are in the copy stream: the caller's stream waits for them
-    cudaEvent_t ev = bs->copied[pipelined ? c0 / chunk : 0];
+    // (a wait that is already in a stream keeps to the record it was given, so events may be recorded again)
+    cudaEvent_t ev = bs->copied[n_chunks++ % kCopyEvents];
     QM_CUDA_OK(cudaEventRecord(ev, bs->copy));
     QM_CUDA_OK(cudaStreamWaitEvent(user, ev, 0));
     if (good > c0) {
       st = qm_probe_batch(good - c0, Ld.data() + c0, Rd.data() + c0, cfg + c0, out_dev + c0, ws + c0, ws_bytes + c0, user);
       if (st == QM_OK) issued = good;
     }
-    if (!pipelined) QM_CUDA_OK(cudaStreamSynchronize(user));       // the one event is about to be recorded again
   }
   if (issued > 0)
     QM_CUDA_OK(cudaMemcpyAsync(out_host, out_dev, sizeof(qm_metric_result) * (size_t)issued, cudaMemcpyDeviceToHost, user));
