@@ -106,7 +106,7 @@ int64_t delta_count(const View& v, int gran) { return gran == QM_GRAN_TENSOR ? 1
 size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
 
 struct Workspace {
-  size_t off_err, off_ml, off_mr, off_dl, off_dr, off_cl, off_cr, off_al, off_ar, off_kl, off_kr, off_part, total;
+  size_t off_err, off_ml, off_mr, off_dl, off_dr, off_cl, off_cr, off_al, off_ar, off_kl, off_kr, off_part, off_pl, off_pr, total;
   int n_part;
   bool tc;
 };
@@ -136,6 +136,10 @@ Workspace plan(const View& L, const View& R, const qm_probe_cfg& cfg, bool with_
   GemmShape g{L.nc, R.nc, L.c, L.batch};
   w.n_part = w.tc ? tc_probe_records(g) : simt_probe_blocks(g);
   w.off_part = take(sizeof(double) * kPartialDoubles * (size_t)w.n_part);
+  // partial maxima of the two-launch preparation (their size must not depend on rounding or grouping: a
+  // workspace may be asked for without them)
+  w.off_pl = take(sizeof(uint32_t) * pair_partial_words(L, cfg.gran_l));
+  w.off_pr = take(sizeof(uint32_t) * pair_partial_words(R, cfg.gran_r));
   w.total = o;
   return w;
 }
@@ -360,8 +364,24 @@ static qm_status probe_phases(const qm_operand* Lo, const qm_operand* Ro, const 
   uint8_t* cl = base + w.off_cl;
   uint8_t* cr = base + w.off_cr;
   double* part = reinterpret_cast<double*>(base + w.off_part);
+  const StochasticDraw draw_l{cfg->seed, 0u}, draw_r{cfg->seed, 1u};
+  const StochasticDraw* dl_draw = (cfg->round & QM_ROUND_STOCHASTIC_L) ? &draw_l : nullptr;
+  const StochasticDraw* dr_draw = (cfg->round & QM_ROUND_STOCHASTIC_R) ? &draw_r : nullptr;
+  void* kl = (w.tc && !L.c_contig()) ? base + w.off_kl : nullptr;
+  void* kr = (w.tc && !R.c_contig()) ? base + w.off_kr : nullptr;
+  // operands of modest size: both in two launches, the first of which clears the control words
+  auto grouped = [](const View& v, int gran, int groups) { return gran == QM_GRAN_CHANNEL && groups > 0 && groups < v.batch; };
+  const bool pair = (phases & kPrepare) == kPrepare && !clear_later && !grouped(L, cfg->gran_l, cfg->batch_groups_l) &&
+                    !grouped(R, cfg->gran_r, cfg->batch_groups_r) &&
+                    pair_prepare_serves(L, cfg->gran_l, dl_draw != nullptr, R, cfg->gran_r, dr_draw != nullptr);
   // the error word, the finished-CTA counter and both max|x| buffers are adjacent: one clear
-  if ((phases & kClear) && clear_later && clear_later->n < kClearMax) {
+  if (pair) {
+    const PairSide side[2] = {
+        {L, cfg->fmt_l, cfg->gran_l, dl_draw, reinterpret_cast<uint32_t*>(base + w.off_pl), dl, cl, kl},
+        {R, cfg->fmt_r, cfg->gran_r, dr_draw, reinterpret_cast<uint32_t*>(base + w.off_pr), dr, cr, kr}};
+    st = launch_pair_prepare(side, err, 64, s);
+    if (st != QM_OK) return st;
+  } else if ((phases & kClear) && clear_later && clear_later->n < kClearMax) {
     clear_later->ptr[clear_later->n] = base;                 // cleared with others by one kernel
     clear_later->words[clear_later->n++] = (uint32_t)(w.off_dl / 4);
   } else if (phases & kClear) {
@@ -371,19 +391,14 @@ static qm_status probe_phases(const qm_operand* Lo, const qm_operand* Ro, const 
     QM_CUDA_OK(cudaMemsetAsync(cfg->row_stats, 0, sizeof(double) * QM_ROW_STATS * (size_t)(L.batch * L.nc), s));
   uint32_t* ml = reinterpret_cast<uint32_t*>(base + w.off_ml);
   uint32_t* mr = reinterpret_cast<uint32_t*>(base + w.off_mr);
-  // the fused kernel forms |L| and |R| tiles in shared memory: no |x| copy is written
+  // the fused kernel forms |L| and |R| on chip: no |x| copy is written
   void* al = nullptr;
   void* ar = nullptr;
-  void* kl = (w.tc && !L.c_contig()) ? base + w.off_kl : nullptr;
-  void* kr = (w.tc && !R.c_contig()) ? base + w.off_kr : nullptr;
-  const StochasticDraw draw_l{cfg->seed, 0u}, draw_r{cfg->seed, 1u};
-  const StochasticDraw* dl_draw = (cfg->round & QM_ROUND_STOCHASTIC_L) ? &draw_l : nullptr;
-  const StochasticDraw* dr_draw = (cfg->round & QM_ROUND_STOCHASTIC_R) ? &draw_r : nullptr;
-  if (phases & kPrepareL) {
+  if ((phases & kPrepareL) && !pair) {
     st = prepare_operand(L, cfg->fmt_l, cfg->gran_l, ml, dl, cl, al, kl, err, dl_draw, cfg->batch_groups_l, s);
     if (st != QM_OK) return st;
   }
-  if (phases & kPrepareR) {
+  if ((phases & kPrepareR) && !pair) {
     st = prepare_operand(R, cfg->fmt_r, cfg->gran_r, mr, dr, cr, ar, kr, err, dr_draw, cfg->batch_groups_r, s);
     if (st != QM_OK) return st;
   }

@@ -94,6 +94,21 @@ qm_status launch_quantize(const View& x, int fmt, int gran, const float* delta, 
 qm_status launch_quantize_multi(const View& x, int gran, const uint32_t* amax, int nf, const int* fmts,
                                 float* const* delta_out, uint32_t* const* err_word, uint8_t* const* codes,
                                 void* kmaj_copy, cudaStream_t s);
+// Scale and quantize both operands of a probe in two launches (max|x|, then codes), for operands of modest
+// size.  `partial` needs pair_partial_words 32-bit words, not cleared; the first launch clears
+// `control` (at most 256 words), whose first word then takes QM_DEVERR_NONFINITE.
+struct PairSide {
+  View v;
+  int fmt, gran;
+  const StochasticDraw* draw;             // null: round to nearest even
+  uint32_t* partial;
+  float* delta;
+  uint8_t* codes;
+  void* kmaj;                             // contraction-major bf16 copy of a strided contraction, or null
+};
+size_t pair_partial_words(const View& v, int gran);
+bool pair_prepare_serves(const View& l, int gran_l, bool draw_l, const View& r, int gran_r, bool draw_r);
+qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint32_t control_words, cudaStream_t s);
 // Single pass per row: absmax, delta, codes (contiguous contraction, per-channel).
 qm_status launch_scale_quantize_rows(const View& x, int fmt, float* delta_out, uint8_t* codes,
                                      void* abs_copy, uint32_t* err_word, cudaStream_t s);

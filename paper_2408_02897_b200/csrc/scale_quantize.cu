@@ -478,15 +478,15 @@ template <int MASK> struct TileSmem {
   static __device__ __forceinline__ int slot(int f) { return (f > 0 ? MASK & 1 : 0) + (f > 1 ? MASK >> 1 & 1 : 0); }
 };
 // d_lo / d_hi: the scales of the thread's two columns, per format in MASK (bit f = qm_format f).
-// SR: stochastic rounding (rnd); c is a multiple of 4, so sixteen entries are four counter blocks.
+// tile: column tile, contraction tile, batch element.  SR: stochastic rounding (rnd); c is a multiple of 4, so sixteen entries are four counter blocks.
 template <int MASK, bool GUARD, bool EDGE, bool SR = false>
 __device__ __forceinline__ void transpose_tile(const __nv_bfloat16* __restrict__ x, int64_t nc, int64_t c, int64_t s_c,
                                                int64_t s_b, const float (&d_lo)[3], const float (&d_hi)[3],
                                                uint8_t* const (&codes)[3], int64_t ldc,
-                                               __nv_bfloat16* __restrict__ kmaj_copy, uint4* smem,
+                                               __nv_bfloat16* __restrict__ kmaj_copy, uint4* smem, const uint3 tile,
                                                const Rounding& rnd = Rounding{}) {
   const int t = threadIdx.x;
-  const int64_t b = blockIdx.z, n0 = (int64_t)blockIdx.x * 64, k0 = (int64_t)blockIdx.y * 128;
+  const int64_t b = tile.z, n0 = (int64_t)tile.x * 64, k0 = (int64_t)tile.y * 128;
   const int64_t pitch = s_c >> 3;                                     // row stride in 16-byte units
   // 128 rows x 128 bytes, four 16-byte loads per thread in flight
   auto fetch = [&](uint4 (&v)[4]) {
@@ -615,8 +615,8 @@ quantize_transpose_tile_kernel(const __nv_bfloat16* __restrict__ x, int64_t nc, 
     d_lo[FMT] = d_hi[FMT] = ds.get(0, blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0);
   }
   uint8_t* const cd[3] = {codes, codes, codes};
-  if (ds.from_amax) transpose_tile<1 << FMT, false, EDGE, SR>(x, nc, c, s_c, s_b, d_lo, d_hi, cd, ldc, kmaj_copy, smem, rnd);
-  else transpose_tile<1 << FMT, true, EDGE, SR>(x, nc, c, s_c, s_b, d_lo, d_hi, cd, ldc, kmaj_copy, smem, rnd);
+  if (ds.from_amax) transpose_tile<1 << FMT, false, EDGE, SR>(x, nc, c, s_c, s_b, d_lo, d_hi, cd, ldc, kmaj_copy, smem, blockIdx, rnd);
+  else transpose_tile<1 << FMT, true, EDGE, SR>(x, nc, c, s_c, s_b, d_lo, d_hi, cd, ldc, kmaj_copy, smem, blockIdx, rnd);
 }
 
 // Every format in MASK from one read, per-tensor scales from the tensor's max|x|.
@@ -630,21 +630,20 @@ quantize_transpose_tile_multi_kernel(const __nv_bfloat16* __restrict__ x, int64_
   float d[3];
   multi_scales<MASK>(amax, o, blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0, d);
   uint8_t* const cd[3] = {o.codes[0], o.codes[1], o.codes[2]};
-  transpose_tile<MASK, false, EDGE>(x, nc, c, s_c, s_b, d, d, cd, ldc, kmaj_copy, smem);
+  transpose_tile<MASK, false, EDGE>(x, nc, c, s_c, s_b, d, d, cd, ldc, kmaj_copy, smem, blockIdx);
 }
 
 // ---------------------------------------------------------------- fused per-row scale + quantize
 // G lanes own one row: pass 1 reduces max|x| over the row, pass 2 re-reads it (from L1/L2: the
 // same lanes touched it a moment ago) and writes codes.  HBM sees each element once.
 template <typename T, int FMT, int G>
-__global__ void __launch_bounds__(kThreads)
-scale_quantize_rows_kernel(const T* __restrict__ x, int64_t nc, int64_t c, int64_t s_nc,
-                           int64_t batch, int64_t s_b, float qmax, float* __restrict__ delta_out,
-                           uint8_t* __restrict__ codes, int64_t ldc,
-                           __nv_bfloat16* __restrict__ abs_copy, uint32_t* __restrict__ err_word) {
-  pdl_prologue();
+__device__ __forceinline__ void scale_quantize_rows(const T* __restrict__ x, int64_t nc, int64_t c, int64_t s_nc,
+                                                    int64_t batch, int64_t s_b, float qmax, float* __restrict__ delta_out,
+                                                    uint8_t* __restrict__ codes, int64_t ldc,
+                                                    __nv_bfloat16* __restrict__ abs_copy, uint32_t* __restrict__ err_word,
+                                                    int64_t block) {
   const int64_t rows = nc * batch;
-  const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
+  const int64_t row = (block * blockDim.x + threadIdx.x) / G;
   const int sub = threadIdx.x % G;
   const bool live = row < rows;
   const int64_t b = live ? row / nc : 0, r = live ? row - b * nc : 0;
@@ -689,6 +688,16 @@ scale_quantize_rows_kernel(const T* __restrict__ x, int64_t nc, int64_t c, int64
         for (int j = 0; j < 8 && k0 + j < c; ++j) a[j] = __float2bfloat16_rn(fabsf(v.v[j]));
     }
   }
+}
+
+template <typename T, int FMT, int G>
+__global__ void __launch_bounds__(kThreads)
+scale_quantize_rows_kernel(const T* __restrict__ x, int64_t nc, int64_t c, int64_t s_nc,
+                           int64_t batch, int64_t s_b, float qmax, float* __restrict__ delta_out,
+                           uint8_t* __restrict__ codes, int64_t ldc,
+                           __nv_bfloat16* __restrict__ abs_copy, uint32_t* __restrict__ err_word) {
+  pdl_prologue();
+  scale_quantize_rows<T, FMT, G>(x, nc, c, s_nc, batch, s_b, qmax, delta_out, codes, ldc, abs_copy, err_word, blockIdx.x);
 }
 
 // ---------------------------------------------------------------- fused per-row, row held in registers
@@ -757,17 +766,14 @@ scale_quantize_rows_reg_kernel(const __nv_bfloat16* __restrict__ x, int64_t nc, 
 // ---------------------------------------------------------------- quantize + transpose
 // Storage [c][nc] (nc contiguous) -> codes [nc][ldc] and optional bf16 copies [nc][c].
 // A 64(c) x 64(nc) tile goes through shared memory.
-template <typename T, int FMT>
-__global__ void __launch_bounds__(kThreads)
-quantize_transpose_kernel(const T* __restrict__ x, int64_t nc, int64_t c, int64_t s_c, int64_t s_b,
-                          const DeltaSrc ds,
-                          uint8_t* __restrict__ codes, int64_t ldc,
-                          __nv_bfloat16* __restrict__ abs_copy, __nv_bfloat16* __restrict__ kmaj_copy,
-                          const Rounding rnd) {
-  pdl_prologue();
-  __shared__ float tile[64][65];     // +1 column spreads the transposed accesses over the banks
-  const int64_t b = blockIdx.z;
-  const int64_t c0 = (int64_t)blockIdx.y * 64, n0 = (int64_t)blockIdx.x * 64;
+// scale(output row, whether this thread also stores it): the row's Eq. 1 scale.
+template <typename T, int FMT, typename Scale>
+__device__ __forceinline__ void transpose_general(const T* __restrict__ x, int64_t nc, int64_t c, int64_t s_c, int64_t s_b,
+                                                  Scale scale, uint8_t* __restrict__ codes, int64_t ldc,
+                                                  __nv_bfloat16* __restrict__ abs_copy, __nv_bfloat16* __restrict__ kmaj_copy,
+                                                  const Rounding& rnd, float (&tile)[64][65], const uint3 at) {
+  const int64_t b = at.z;
+  const int64_t c0 = (int64_t)at.y * 64, n0 = (int64_t)at.x * 64;
   const T* base = x + b * s_b;
   const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;    // 8 column-chunks x 32 rows
 #pragma unroll
@@ -786,9 +792,6 @@ quantize_transpose_kernel(const T* __restrict__ x, int64_t nc, int64_t c, int64_
   }
   __syncthreads();
   // output: row n (64 of them), 64 contraction entries = 8 chunks of 8
-  const float d_tensor = ds.per_channel
-                             ? 0.f
-                             : ds.get(0, blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0);
 #pragma unroll
   for (int it = 0; it < 2; ++it) {
     const int nrow = ty + it * 32;
@@ -799,7 +802,7 @@ quantize_transpose_kernel(const T* __restrict__ x, int64_t nc, int64_t c, int64_
     Vec8 v;
 #pragma unroll
     for (int j = 0; j < 8; ++j) v.v[j] = tile[tx * 8 + j][nrow];
-    const Quotient quot(ds.per_channel ? ds.get(b * nc + nn, blockIdx.y == 0 && tx == 0) : d_tensor);
+    const Quotient quot(scale(b * nc + nn, at.y == 0 && tx == 0));
     const int64_t orow = b * nc + nn;
     *reinterpret_cast<uint2*>(codes + orow * ldc + k0) =
         rnd.stochastic ? quant8_sr<FMT>(v, quot, rnd, (uint64_t)orow * (uint64_t)c + (uint64_t)k0)
@@ -816,6 +819,21 @@ quantize_transpose_kernel(const T* __restrict__ x, int64_t nc, int64_t c, int64_
       }
     }
   }
+}
+
+template <typename T, int FMT>
+__global__ void __launch_bounds__(kThreads)
+quantize_transpose_kernel(const T* __restrict__ x, int64_t nc, int64_t c, int64_t s_c, int64_t s_b,
+                          const DeltaSrc ds, uint8_t* __restrict__ codes, int64_t ldc,
+                          __nv_bfloat16* __restrict__ abs_copy, __nv_bfloat16* __restrict__ kmaj_copy,
+                          const Rounding rnd) {
+  pdl_prologue();
+  __shared__ float tile[64][65];     // +1 column spreads the transposed accesses over the banks
+  const float d_tensor = ds.per_channel
+                             ? 0.f
+                             : ds.get(0, blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0);
+  transpose_general<T, FMT>(x, nc, c, s_c, s_b, [&](int64_t row, bool writer) { return ds.per_channel ? ds.get(row, writer) : d_tensor; },
+                            codes, ldc, abs_copy, kmaj_copy, rnd, tile, blockIdx);
 }
 
 // ---------------------------------------------------------------- quantize + transpose, bf16 fast path
@@ -889,6 +907,205 @@ quantize_transpose_bf16_kernel(const __nv_bfloat16* __restrict__ x, int64_t nc, 
       }
     }
   }
+}
+
+// ---------------------------------------------------------------- both operands of a probe in two launches
+// A probe of modest operands is bound by its chain of launches, not by what they do: clear, max|x| and
+// quantize for one operand, the same for the other, products.  Here one kernel takes the maxima of both
+// operands and one quantizes both, so that the operands run side by side and the chain is three launches
+// long.  The maxima are partial ones, stored (not combined by atomics), so nothing has to be cleared first:
+//   one scale per tensor:      a maximum per block of the first kernel (at most kPairBlocks);
+//   one per strided channel:   a maximum per column and slice of the contraction (at most kPairSlices);
+//   one per contiguous row:    none, the second kernel reduces a row itself.
+constexpr int kPairBlocks = 256, kPairSlices = 8;
+enum { kPairChunks = 0, kPairRows = 1, kPairTiles = 2, kPairGeneral = 3 };
+
+struct PairOperand {
+  View v;
+  int32_t per_channel;
+  int32_t blocks_max, n_partial;          // blocks of the first kernel; partial maxima per scale
+  int32_t blocks_quant, path;             // blocks of the second kernel, and how it walks the operand
+  uint32_t gx, gy;                        // tiles: column tiles, contraction tiles
+  uint32_t groups_per_line, total_groups, lines;   // the tensor as lines of contiguous groups of eight; lines per batch element
+  FastDiv by_groups, by_lines, by_chunks, by_nc, by_gx, by_gy;
+  uint32_t* partial;
+  float* delta;
+  uint8_t* codes;
+  __nv_bfloat16* kmaj;
+  Rounding rnd;
+};
+struct PairArgs {
+  PairOperand op[2];
+  uint32_t* control;                      // cleared by the first kernel; its first word takes the error flags
+  uint32_t control_words;
+};
+
+template <typename T>
+__device__ __forceinline__ void pair_max(const PairOperand& o, uint32_t block, uint32_t (&s)[32][64]) {
+  const View& v = o.v;
+  const T* x = static_cast<const T*>(v.data);
+  if (!o.per_channel) {
+    const bool along_c = v.s_c == 1;
+    const int64_t inner = along_c ? v.c : v.nc, line_stride = along_c ? v.s_nc : v.s_c;
+    const uint32_t stride = (uint32_t)o.blocks_max * kThreads;
+    uint32_t acc = 0;
+    for (uint32_t g0 = block * kThreads + threadIdx.x; g0 < o.total_groups; g0 += 4 * stride) {
+      Vec8 w[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t g = g0 + u * stride < o.total_groups ? g0 + u * stride : g0;      // repeats change no maximum
+        const uint32_t line = o.by_groups.div(g), b = o.by_lines.div(line);
+        const int64_t k = (int64_t)(g - line * o.groups_per_line) * 8;
+        const T* p = x + (int64_t)b * v.s_b + (int64_t)(line - b * o.lines) * line_stride + k;
+        if (k + 8 <= inner) {
+          w[u] = Loader<T>::load8(p);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) w[u].v[j] = k + j < inner ? Loader<T>::load1(p, j) : 0.f;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) acc = absmax8(w[u], acc);
+    }
+    acc = block_max(acc);
+    if (threadIdx.x == 0) o.partial[block] = acc;
+    return;
+  }
+  // a column each: 64 columns of one batch element, one slice of the contraction
+  const uint32_t slice = block % (uint32_t)o.n_partial, rest = block / (uint32_t)o.n_partial;
+  const uint32_t b = o.by_gx.div(rest), cb = rest - b * o.gx;
+  const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
+  const int64_t col0 = (int64_t)cb * 64 + tx * 8, per = (v.c + o.n_partial - 1) / o.n_partial;
+  const int64_t r0 = slice * per, r1 = r0 + per < v.c ? r0 + per : v.c;
+  const T* base = x + (int64_t)b * v.s_b + col0;
+  uint32_t acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  if (col0 < v.nc) {
+    const int live = v.nc - col0 < 8 ? (int)(v.nc - col0) : 8;
+#pragma unroll 4
+    for (int64_t r = r0 + ty; r < r1; r += 32) {
+      Vec8 w;
+      if (live == 8) {
+        w = Loader<T>::load8(base + r * v.s_c);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) w.v[j] = j < live ? Loader<T>::load1(base, r * v.s_c + j) : 0.f;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) acc[j] = max(acc[j], absbits_f32(__float_as_uint(w.v[j])));
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) s[ty][tx * 8 + j] = acc[j];
+  __syncthreads();
+  if (threadIdx.x < 64) {
+    uint32_t m = 0;
+    for (int j = 0; j < 32; ++j) m = max(m, s[j][threadIdx.x]);
+    const int64_t col = (int64_t)cb * 64 + threadIdx.x;
+    if (col < v.nc) o.partial[((int64_t)slice * v.batch + b) * v.nc + col] = m;
+  }
+}
+
+__global__ void __launch_bounds__(kThreads) pair_max_kernel(const PairArgs a) {
+  pdl_prologue();
+  __shared__ uint32_t s[32][64];
+  if (blockIdx.x == 0 && threadIdx.x < a.control_words) a.control[threadIdx.x] = 0u;
+  const bool right = blockIdx.x >= (uint32_t)a.op[0].blocks_max;
+  const PairOperand& o = right ? a.op[1] : a.op[0];
+  const uint32_t block = right ? blockIdx.x - a.op[0].blocks_max : blockIdx.x;
+  if (block >= (uint32_t)o.blocks_max) return;          // (where neither operand has maxima one block still clears)
+  if (o.v.dtype == QM_DT_BF16) pair_max<__nv_bfloat16>(o, block, s);
+  else pair_max<float>(o, block, s);
+}
+
+template <typename T, int FMT>
+__device__ __forceinline__ void pair_quantize(const PairOperand& o, uint32_t* err, uint32_t block, uint4* smem) {
+  const View& v = o.v;
+  const T* x = static_cast<const T*>(v.data);
+  const int64_t ldc = (v.c + 15) & ~(int64_t)15;
+  const float qmax = fmt_qmax(FMT);
+  if (o.path == kPairRows) {
+    scale_quantize_rows<T, FMT, 32>(x, v.nc, v.c, v.s_nc, v.batch, v.s_b, qmax, o.delta, o.codes, ldc, nullptr, err, block);
+    return;
+  }
+  // the scale of an output row from its partial maxima; the thread that is told to stores it
+  auto finish = [&](uint32_t bits, int64_t at, bool writer) {
+    const float d = bits == 0 ? 1.0f : __fdiv_rn(__uint_as_float(bits), qmax);
+    if (writer) {
+      o.delta[at] = d;
+      if (bits >= 0x7f800000u) atomicOr(err, QM_DEVERR_NONFINITE);
+    }
+    return d;
+  };
+  float d_tensor = 1.f;
+  if (!o.per_channel) {
+    uint32_t m = 0;
+    for (int i = threadIdx.x & 31; i < o.n_partial; i += 32) m = max(m, __ldg(o.partial + i));
+    d_tensor = finish(warp_max(m), 0, block == 0 && threadIdx.x == 0);
+  }
+  auto scale = [&](int64_t row, bool writer) {
+    if (!o.per_channel) return d_tensor;
+    uint32_t m = 0;
+    for (int i = 0; i < o.n_partial; ++i) m = max(m, __ldg(o.partial + (int64_t)i * v.batch * v.nc + row));
+    return finish(m, row, writer);
+  };
+  if (o.path == kPairChunks) {              // contiguous contraction: sixteen elements per thread
+    const uint32_t chunks = (uint32_t)(ldc >> 4), i = block * kThreads + threadIdx.x;
+    if (i >= (uint32_t)(v.nc * v.batch) * chunks) return;
+    const uint32_t row = o.by_chunks.div(i), b = o.by_nc.div(row);
+    const int64_t k0 = (int64_t)(i - row * chunks) * 16;
+    const T* p = x + (int64_t)b * v.s_b + (int64_t)(row - b * (uint32_t)v.nc) * v.s_nc + k0;
+    uint4* dst = reinterpret_cast<uint4*>(o.codes + (int64_t)row * ldc + k0);
+    const uint64_t number = (uint64_t)row * (uint64_t)v.c + (uint64_t)k0;
+    if (sizeof(T) == 2 && k0 + 16 <= v.c && QuotientPair::serves(d_tensor) && (!o.rnd.stochastic || (number & 3) == 0)) {
+      const uint4 lo = __ldg(reinterpret_cast<const uint4*>(p)), hi = __ldg(reinterpret_cast<const uint4*>(p) + 1);
+      const QuotientPair qp(d_tensor);
+      *dst = o.rnd.stochastic ? quant_bf16x16_sr<FMT, false>(lo, hi, qp, o.rnd, number) : quant_bf16x16<FMT>(lo, hi, qp);
+      return;
+    }
+    const Quotient quot(d_tensor);
+    uint2 q[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      Vec8 w;
+      if (k0 + 8 * h + 8 <= v.c) {
+        w = Loader<T>::load8(p + 8 * h);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) w.v[j] = k0 + 8 * h + j < v.c ? Loader<T>::load1(p, 8 * h + j) : 0.f;
+      }
+      q[h] = o.rnd.stochastic ? quant8_sr<FMT>(w, quot, o.rnd, number + 8 * h) : quant8<FMT>(w, quot);
+    }
+    *dst = make_uint4(q[0].x, q[0].y, q[1].x, q[1].y);
+    return;
+  }
+  // strided contraction: tiles
+  const uint32_t rest = o.by_gx.div(block), bz = o.by_gy.div(rest);
+  const uint3 at = make_uint3(block - rest * o.gx, rest - bz * o.gy, bz);
+  if (o.path == kPairGeneral) {
+    transpose_general<T, FMT>(x, v.nc, v.c, v.s_c, v.s_b, scale, o.codes, ldc, nullptr, o.kmaj, o.rnd,
+                              *reinterpret_cast<float(*)[64][65]>(smem), at);
+    return;
+  }
+  if constexpr (sizeof(T) == 2) {
+    const int64_t col = (int64_t)at.x * 64 + 2 * (threadIdx.x & 31), orow = (int64_t)at.z * v.nc + col;
+    const bool writer = at.y == 0 && threadIdx.x < 32;
+    float d_lo[3] = {1.f, 1.f, 1.f}, d_hi[3] = {1.f, 1.f, 1.f};
+    if (col < v.nc) d_lo[FMT] = scale(orow, writer);
+    if (col + 1 < v.nc) d_hi[FMT] = scale(orow + 1, writer);
+    uint8_t* const cd[3] = {o.codes, o.codes, o.codes};
+    if (o.rnd.stochastic) transpose_tile<1 << FMT, false, true, true>(x, v.nc, v.c, v.s_c, v.s_b, d_lo, d_hi, cd, ldc, o.kmaj, smem, at, o.rnd);
+    else transpose_tile<1 << FMT, false, true, false>(x, v.nc, v.c, v.s_c, v.s_b, d_lo, d_hi, cd, ldc, o.kmaj, smem, at);
+  }
+}
+
+// F0, F1: the operands' formats; T: their element type.
+template <typename T, int F0, int F1>
+__global__ void __launch_bounds__(kThreads) pair_quantize_kernel(const PairArgs a) {
+  pdl_prologue();
+  __shared__ uint4 smem[TileSmem<1>::kVec];             // a bf16 tile with codes and copy, or a 64 x 65 fp32 tile
+  static_assert(sizeof(float) * 64 * 65 <= sizeof(uint4) * TileSmem<1>::kVec, "the general tile has to fit");
+  if (blockIdx.x < (uint32_t)a.op[0].blocks_quant) pair_quantize<T, F0>(a.op[0], a.control, blockIdx.x, smem);
+  else pair_quantize<T, F1>(a.op[1], a.control, blockIdx.x - a.op[0].blocks_quant, smem);
 }
 
 int grid_for(int64_t work_items, int per_sm) {
@@ -1112,6 +1329,86 @@ qm_status scale_quantize_rows_t(const View& x, float* delta_out, uint8_t* codes,
 qm_status launch_absmax(const View& x, int gran, uint32_t* amax_bits, cudaStream_t s) {
   return x.dtype == QM_DT_BF16 ? absmax_t<__nv_bfloat16>(x, gran, amax_bits, s)
                                : absmax_t<float>(x, gran, amax_bits, s);
+}
+
+// Which operands the two-launch form takes: up to 2^22 elements, and no rows with stochastic rounding under a
+// scale each, whose maxima nobody would have taken.  Whole probes, six launches against three: 128 x 128 x 128
+// 21.7 / 18.7 us, fp32 128 x 256 x 256 24.1 / 20.6, 2000 x 1000 x 704 31.6 / 28.0, 4096 x 2048 x 1024 with
+// operands of 4 M and 2 M elements 65.4 / 63.6; with both at 2^23 elements a single operand's own kernels fill
+// the GPU and are the faster ones (4096 x 2048 x 2048, strided: 101 / 113).
+static bool pair_size(const View& v) {
+  return v.nc <= (1 << 22) && v.c <= (1 << 22) && v.batch <= (1 << 15) && v.nc * v.c <= (1ll << 22) && v.nc * v.c * v.batch <= (1ll << 22);
+}
+static bool pair_serves(const View& v, int gran, bool stochastic) {
+  return pair_size(v) && !(gran == QM_GRAN_CHANNEL && v.c_contig() && stochastic);
+}
+
+size_t pair_partial_words(const View& v, int gran) {
+  if (!pair_size(v)) return 0;
+  if (gran == QM_GRAN_TENSOR) return kPairBlocks;
+  return v.c_contig() ? 0 : (size_t)(kPairSlices * v.nc * v.batch);
+}
+
+bool pair_prepare_serves(const View& l, int gran_l, bool draw_l, const View& r, int gran_r, bool draw_r) {
+  return l.dtype == r.dtype && pair_serves(l, gran_l, draw_l) && pair_serves(r, gran_r, draw_r);
+}
+
+qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint32_t control_words, cudaStream_t s) {
+  PairArgs a{};
+  a.control = control; a.control_words = control_words;
+  for (int i = 0; i < 2; ++i) {
+    const PairSide& in = side[i];
+    PairOperand& o = a.op[i];
+    const View& v = in.v;
+    o.v = v; o.per_channel = in.gran == QM_GRAN_CHANNEL;
+    o.partial = in.partial; o.delta = in.delta; o.codes = in.codes; o.kmaj = static_cast<__nv_bfloat16*>(in.kmaj);
+    if (in.draw) { o.rnd.stochastic = 1; o.rnd.k0 = (uint32_t)in.draw->seed; o.rnd.k1 = (uint32_t)(in.draw->seed >> 32); o.rnd.stream = in.draw->stream; }
+    const bool tiles = tile_transposable(v);
+    const int64_t ldc = qm_code_ld(v.c);
+    if (v.c_contig()) {
+      const int64_t chunks = ldc >> 4, threads = v.nc * v.batch * (o.per_channel ? 32 : chunks);
+      o.path = o.per_channel ? kPairRows : kPairChunks;
+      o.blocks_quant = (int32_t)((threads + kThreads - 1) / kThreads);
+      o.by_chunks = FastDiv((uint32_t)chunks); o.by_nc = FastDiv((uint32_t)v.nc);
+    } else {
+      o.path = tiles ? kPairTiles : kPairGeneral;
+      o.gx = (uint32_t)((v.nc + 63) / 64);
+      o.gy = (uint32_t)(tiles ? (v.c + 127) / 128 : (ldc + 63) / 64);
+      o.by_gx = FastDiv(o.gx); o.by_gy = FastDiv(o.gy);
+      o.blocks_quant = (int32_t)((int64_t)o.gx * o.gy * v.batch);
+    }
+    if (!o.per_channel) {
+      const int64_t inner = v.c_contig() ? v.c : v.nc;
+      o.lines = (uint32_t)(v.c_contig() ? v.nc : v.c);
+      o.groups_per_line = (uint32_t)((inner + 7) / 8);
+      o.total_groups = (uint32_t)(o.groups_per_line * (int64_t)o.lines * v.batch);
+      o.by_groups = FastDiv(o.groups_per_line); o.by_lines = FastDiv(o.lines);
+      const int64_t want = ((int64_t)o.total_groups + 4 * kThreads - 1) / (4 * kThreads);
+      o.blocks_max = (int32_t)(want < kPairBlocks ? want : kPairBlocks);
+      o.n_partial = o.blocks_max;
+    } else if (!v.c_contig()) {
+      // slices of at least 128 contraction entries
+      const int64_t want = (v.c + 127) / 128;
+      o.n_partial = (int32_t)(want < kPairSlices ? want : kPairSlices);
+      o.blocks_max = (int32_t)((int64_t)o.gx * v.batch * o.n_partial);
+    }
+  }
+  const unsigned maxima = (unsigned)(a.op[0].blocks_max + a.op[1].blocks_max);
+  QM_CUDA_OK(launch_pdl(pair_max_kernel, dim3(maxima > 0 ? maxima : 1), dim3(kThreads), 0, s, a));
+  const dim3 grid((unsigned)(a.op[0].blocks_quant + a.op[1].blocks_quant));
+  const bool bf16 = side[0].v.dtype == QM_DT_BF16;
+#define QM_PQ(F0, F1)                                                                                            \
+  QM_CUDA_OK(bf16 ? launch_pdl(pair_quantize_kernel<__nv_bfloat16, F0, F1>, grid, dim3(kThreads), 0, s, a)        \
+                  : launch_pdl(pair_quantize_kernel<float, F0, F1>, grid, dim3(kThreads), 0, s, a))
+  const int f0 = side[0].fmt, f1 = side[1].fmt;
+  if (f0 == QM_FMT_INT8) QM_PQ(QM_FMT_INT8, QM_FMT_INT8);          // (INT8 goes with INT8 only)
+  else if (f0 == QM_FMT_E4M3 && f1 == QM_FMT_E4M3) QM_PQ(QM_FMT_E4M3, QM_FMT_E4M3);
+  else if (f0 == QM_FMT_E4M3) QM_PQ(QM_FMT_E4M3, QM_FMT_E5M2);
+  else if (f1 == QM_FMT_E4M3) QM_PQ(QM_FMT_E5M2, QM_FMT_E4M3);
+  else QM_PQ(QM_FMT_E5M2, QM_FMT_E5M2);
+#undef QM_PQ
+  count_launch(2);
+  return QM_OK;
 }
 
 qm_status launch_share_amax(uint32_t* amax_bits, int64_t batch, int64_t groups, int64_t nc, cudaStream_t s) {
