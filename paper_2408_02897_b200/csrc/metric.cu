@@ -18,25 +18,12 @@ __device__ __forceinline__ double warp_maxd(double v) {
   return v;
 }
 
-// |diff| / d, correctly rounded but for rare last-bit cases: the reciprocal, one product and one residual
-// correction where nothing can leave the normal range, the division elsewhere.
-__device__ __forceinline__ float quotient(float diff, float d) {
-  const float n = fabsf(diff);
-  if (d >= 1e-30f && d <= 1e30f && n >= 1e-30f && n <= 1e30f) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
-    const float q = n * r;
-    return fmaf(fmaf(-q, d, n), r, q);
-  }
-  return d != 0.f ? __fdiv_rn(n, d) : 0.f;
-}
-
 // Eq. 3 sums of a short run of elements in fp32, folded into fp64 by the caller.
 struct Run {
   float be = 0, mx = 0, d2 = 0, r2 = 0, n2 = 0;
   __device__ __forceinline__ void add(float c, float q, float d) {
     const float diff = c - q;
-    const float b = quotient(diff, d);
+    const float b = d != 0.f ? __fdiv_rn(fabsf(diff), d) : 0.f;
     be += b; mx = fmaxf(mx, b);
     d2 = fmaf(diff, diff, d2); r2 = fmaf(c, c, r2); n2 = fmaf(d, d, n2);
   }

@@ -117,6 +117,26 @@ def test_metric_reduction(n):
     assert abs(got["max_be"] - want["max_be"]) <= 1e-6 * want["max_be"]
 
 
+@pytest.mark.parametrize("base", [0, 1])          # the wide loads, and arrays off a 16-byte boundary
+def test_metric_divides_as_ieee(base):
+    # one element that is not zero per call: the record then holds its quotient.  Exponents over the whole range of
+    # fp32, quotients that overflow, that are subnormal, that vanish
+    rng = np.random.default_rng(26)
+    n = np.concatenate([np.float32([1e20, 1e15, 3e38, 1e-30, 1e-40, 1e30, 1e-30, 0.0, 5.0]),
+                        (rng.uniform(1, 2, 60) * np.exp2(rng.integers(-126, 128, 60))).astype(np.float32)])
+    d = np.concatenate([np.float32([1e-20, 1e-25, 1e-38, 1e30, 2e-40, 1e-30, 1e10, 3.0, 0.0]),
+                        (rng.uniform(1, 2, 60) * np.exp2(rng.integers(-126, 128, 60))).astype(np.float32)])
+    with np.errstate(over="ignore", under="ignore"):
+        want = np.divide(n, d, out=np.zeros_like(n), where=d != 0)
+    c, q, den = (torch.zeros(2049, device="cuda")[base:base + 2048] for _ in range(3))
+    for i, w in enumerate(want):
+        at = int(rng.integers(2048))
+        c[at], den[at] = float(n[i]), float(d[i])
+        got = qm.qm_metric(c, q, den)
+        assert got.sum_be == got.max_be == float(w), (n[i], d[i], got.sum_be, w)
+        c[at] = den[at] = 0.0
+
+
 # ------------------------------------------------------------------ 256-column tiles (outputs at least 256 wide)
 @pytest.mark.parametrize("shape", [(1, 300, 600, 144), (2, 130, 258, 272), (1, 4096, 3072, 256), (3, 256, 512, 1040)])
 @pytest.mark.parametrize("gran", [("tensor", "tensor"), ("channel", "channel")])
