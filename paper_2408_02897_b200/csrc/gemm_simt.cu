@@ -93,7 +93,7 @@ struct Fetch {
     for (int i = 0; i < NV; ++i) {
       const int t = threadIdx.x + i * kThreads;
       const int64_t row = row0 + t / (KC / 4), k = k0 + 4 * (t % (KC / 4));
-      // rows of codes are a multiple of 16 long, zero beyond K
+      // rows of codes are a multiple of 16 long, zero beyond K where the probe made them
       c[i] = row < o.rows && k < ldc ? __ldg(reinterpret_cast<const uint32_t*>(o.codes + (b * o.rows + row) * ldc + k)) : 0u;
       if (!VALUES) continue;
       if (along_k) {
@@ -101,6 +101,14 @@ struct Fetch {
       } else {
         const int64_t r4 = row0 + 4 * (t % (ROWS / 4)), kk = k0 + t / (ROWS / 4);
         v[i] = get4(o, b * o.s_b + kk * o.s_c + r4, kk < K ? o.rows - r4 : 0);
+      }
+    }
+    // a caller's codes (plain product) count as zero beyond K, whatever their padding holds
+    if (!VALUES && k0 + KC > K) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const int64_t left = K - (k0 + 4 * ((threadIdx.x + i * kThreads) % (KC / 4)));
+        if (left < 4) c[i] &= left > 0 ? (1u << (8 * (int)left)) - 1u : 0u;
       }
     }
   }

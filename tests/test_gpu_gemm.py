@@ -62,6 +62,22 @@ def test_fp8_gemm_exact_on_small_values(simt, fmts):
     assert np.array_equal(raw.astype(np.float64), acc)
 
 
+@pytest.mark.parametrize("fmt", ["int8", "e4m3", "e5m2"])
+@pytest.mark.parametrize("K", [1, 30, 99, 148, 160])
+@pytest.mark.parametrize("M,N", [(40, 33), (900, 1010)])          # tiles with and without a split contraction
+def test_cuda_core_product_ignores_the_padding_of_codes(fmt, K, M, N):
+    rng = np.random.default_rng(30)
+    cl, cr = rand_codes(rng, fmt, (1, M, K)), rand_codes(rng, fmt, (1, N, K))
+    one = torch.ones(1, device="cuda")
+    outs = []
+    for fill in (0, 0x7f):                                           # zero, and NaN in the FP8 formats
+        pl, pr = pad_codes(cl), pad_codes(cr)
+        pl[..., K:] = pr[..., K:] = fill
+        outs.append(qm.qm_gemm(torch.from_numpy(pl).cuda(), fmt, one, "tensor", torch.from_numpy(pr).cuda(), fmt, one, "tensor",
+                               K, use_simt=True)[0])
+    assert torch.equal(*outs)
+
+
 @pytest.mark.parametrize("simt", [False, True])
 @pytest.mark.parametrize("fmts", [("e4m3", "e4m3"), ("e5m2", "e4m3"), ("e4m3", "e5m2")])
 @pytest.mark.parametrize("shape", [(1, 256, 384, 512), (2, 100, 260, 1040)])
