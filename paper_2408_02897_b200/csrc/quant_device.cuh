@@ -289,7 +289,10 @@ __device__ __forceinline__ uint32_t sr_quad(const float (&t)[4], const uint32_t 
     constexpr int m = FMT == QM_FMT_E4M3 ? 3 : 2;                            // mantissa bits
     constexpr int emin = FMT == QM_FMT_E4M3 ? -6 : -14;                      // smallest normal exponent
     constexpr uint32_t below = (1u << (23 - m)) - 1u;
-    if (fminf(fminf(fabsf(t[0]), fabsf(t[1])), fminf(fabsf(t[2]), fabsf(t[3]))) >= __uint_as_float((uint32_t)(127 + emin) << 23)) {
+    float least = fabsf(t[0]);          // NaN if one of the four is (sr_value gives it the largest magnitude)
+#pragma unroll
+    for (int i = 1; i < 4; ++i) asm("min.NaN.f32 %0, %0, %1;" : "+f"(least) : "f"(fabsf(t[i])));
+    if (least >= __uint_as_float((uint32_t)(127 + emin) << 23)) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) v[i] = __uint_as_float((__float_as_uint(t[i]) + below - (draw[i] >> (9 + m))) & ~below);
     } else {

@@ -107,3 +107,17 @@ def test_probe_channel_scales_and_wgrad_layout():
     want = oracle.probe(X.float().numpy().T.copy(), dY.float().numpy(), "e4m3", "e5m2", "channel", "channel",
                         round_r="stochastic", seed=7)
     assert_record_close(res.record(), want, what="wgrad")
+
+
+@pytest.mark.parametrize("fmt", FMTS)
+@pytest.mark.parametrize("dtype,K", [(torch.float32, 40), (torch.bfloat16, 48)])
+@pytest.mark.parametrize("delta", [2.0 ** -70, 2.0 ** -10, 2.0 ** 70])         # inside and outside the range of the fast quotient
+def test_nan_saturates_whatever_stands_beside_it(fmt, dtype, K, delta):
+    # a scale from elsewhere over an operand with a NaN: the largest magnitude, beside values of the normal range as
+    # beside small ones
+    x = torch.full((16, K), 1.5 * delta, dtype=dtype)
+    x[1::2] = 1e-3 * delta
+    at = torch.arange(16)
+    x[at, at] = float("nan")
+    codes = qm.qm_quantize(qm.operand_of(x.cuda(), -1), fmt, "tensor", torch.tensor([delta], device="cuda"), stochastic=(3, 0))[0]
+    assert codes[0, at, at].tolist() == [{"int8": 127, "e4m3": 0x7e, "e5m2": 0x7b}[fmt]] * 16
