@@ -472,8 +472,9 @@ qm_status qm_debug_read_pass(const void* data, size_t bytes, int32_t variant, in
  * qm_debug_set_wait_limit_ns sets that limit for later launches (0 restores
  * the default).  qm_debug_stop_producer_after(k) makes the loading warp of
  * every CTA of later launches stop after its first k k-blocks (64-deep slices
- * of the contraction), so that the warps waiting for the next slice run into
- * the limit; 0xffffffff (the default) switches the hook off.  Both are
+ * of the contraction; where probes share their products, a tile's slices of the
+ * operands, then 128-deep ones of each probe's codes), so that the warps waiting
+ * for the next slice run into the limit; 0xffffffff (the default) switches the hook off.  Both are
  * process-wide and meant for tests only.
  */
 void qm_debug_set_wait_limit_ns(uint64_t ns);

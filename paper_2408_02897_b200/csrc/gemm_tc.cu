@@ -4,17 +4,18 @@
 // Two CTAs on the two SMs of a TPC form a cluster and work on one output tile with cta_group::2
 // MMAs: each CTA stages its own 128 rows of the left operand and HALF of the right operand's
 // tile, so every byte of the right operand enters and leaves shared memory once per pair instead
-// of once per SM.  Three kernels, in this order in the file:
+// of once per SM.  Four kernels, in this order in the file:
 //   tc_kernel            256 x 128 tiles, 320 threads (TMA warp, MMA warp, 8 epilogue warps): the
 //                        stand-alone 8-bit and reference products on narrow outputs, and the
 //                        two-formats-in-one-pass probe (four accumulators fill tensor memory);
 //   tc_gemm_wide_kernel  256 x 256 tiles, two accumulator buffers: stand-alone products on outputs at
 //                        least 256 wide;
-//   tc_group_kernel      the fused probe (Eq. 3 records of one probe or of many per persistent launch):
-//                        reference L.R and denominator |L|.|R| once per pair of operands, then the
-//                        8-bit products of all probes of that pair, |L| fed to the MMAs from tensor
-//                        memory by converter warps, the Eq. 3 statistics reduced in the epilogue; no
-//                        M x N matrix ever goes to HBM.  Its own comment describes roles and barriers.
+//   tc_group_kernel      the fused probe (Eq. 3 records of many probes per persistent launch) where several
+//                        probes have the same operands: reference L.R and denominator |L|.|R| once per
+//                        pair of operands, then the 8-bit products of all its probes, |L| fed to the
+//                        MMAs from tensor memory by converter warps, the Eq. 3 statistics reduced in the
+//                        epilogue; no M x N matrix ever goes to HBM.  Its comment describes roles and barriers;
+//   tc_side_kernel       the same for probes that have their operands to themselves: the three products side by side.
 // Common to all: the MMA warp runs its loop converged and one elected lane issues; the epilogue
 // warps read the accumulators with tcgen05.ld (a warp may touch the lane quarter warp_id % 4; the
 // two warps of a quarter split the columns); a CTA keeps Eq. 3 statistics in registers across tiles
@@ -1019,7 +1020,7 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 // fused kernel only, same GPU): one format 284 us (separate 282), three 420 (793), six 660 (1624).
 // Running the products one after the other, instead of side by side on narrower tiles, is what keeps
 // the tiles 128 wide: five accumulators side by side would leave room for 64 columns each, at 256 KB
-// per 128 columns against the 144 KB here.
+// per 128 columns against the 144 KB here.  (Units of one probe have nothing to share: tc_side_kernel.)
 //
 // The left operand of the reference and denominator products is not read from shared memory by the tensor
 // cores: converter warps read this CTA's 128 rows of the L tile once and store them, and the same with
@@ -1138,7 +1139,7 @@ struct GroupTable {
   GroupVar v[VARS];
 };
 // A launch's table has to fit into 32 764 bytes of kernel parameters.  24 units hold the 18 products
-// of an encoder layer in one launch; a single probe passes a table of its own size (1 KB).
+// of an encoder layer in one launch; a probe on its own passes a table of its own size (1 KB).
 using TableBig = GroupTable<24, 56>;
 using TableOne = GroupTable<1, 1>;
 static_assert(sizeof(TableBig) <= 32764, "kernel parameters");
@@ -1335,6 +1336,92 @@ __device__ __forceinline__ void eval_variant(uint32_t taddr, const uint32_t (&rc
   }
 }
 
+// The walk and variant tables of a launch into shared memory (one warp).
+template <typename Sh, typename Table>
+__device__ __forceinline__ void fill_walk(Sh* sh, const Table& tab, int lane) {
+  for (int i = lane; i < tab.n; i += 32) {
+    const GroupUnit& u = tab.u[i];
+    WalkInfo wi;
+    wi.tile_begin = u.tile_begin; wi.per_b = u.tiles_m * u.tiles_n;
+    wi.inner = u.m_fastest ? -u.tiles_m : u.tiles_n;
+    wi.num_kb = (u.K + kBlockK - 1) / kBlockK;
+    wi.half_n = u.half_n; wi.n_var = u.n_var; wi.var_begin = u.var_begin; wi.K = u.K;
+    sh->walk[i] = wi;
+  }
+  for (int i = lane; i < tab.n_var; i += 32) sh->var[i] = VarInfo{tab.v[i].idesc_lp, tab.v[i].flags};
+}
+
+// Every record of the launch is visible (last CTA): epilogue warp ew takes probes ew, ew + 8, ...; fixed-order
+// sum (lane l takes records l, l + 32, ...).
+template <typename Table>
+__device__ __forceinline__ void write_results(const Table& tab, int ew, int lane) {
+  const uint32_t timed_out = tab.err0 ? (*reinterpret_cast<volatile uint32_t*>(tab.err0) & QM_DEVERR_TIMEOUT) : 0u;
+  for (int vi = ew; vi < tab.n_var; vi += kEpiWarps) {
+    const GroupVar& a = tab.v[vi];
+    double s5[5] = {0, 0, 0, 0, 0};
+    for (int i = lane; i < (int)gridDim.x; i += 32) {
+      const double* rec = a.partials + (int64_t)i * kPartialDoubles;
+      s5[0] += __ldcg(rec); s5[1] = fmax(s5[1], __ldcg(rec + 1)); s5[2] += __ldcg(rec + 2);
+      s5[3] += __ldcg(rec + 3); s5[4] += __ldcg(rec + 4);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      s5[0] += __shfl_xor_sync(0xffffffffu, s5[0], o);
+      s5[1] = fmax(s5[1], __shfl_xor_sync(0xffffffffu, s5[1], o));
+      s5[2] += __shfl_xor_sync(0xffffffffu, s5[2], o);
+      s5[3] += __shfl_xor_sync(0xffffffffu, s5[3], o);
+      s5[4] += __shfl_xor_sync(0xffffffffu, s5[4], o);
+    }
+    if (lane == 0) {
+      a.result->sum_be = s5[0]; a.result->max_be = s5[1]; a.result->sum_diff2 = s5[2];
+      a.result->sum_ref2 = s5[3]; a.result->sum_den2 = s5[4];
+      a.result->count = a.count;
+      uint32_t flags = (a.err_word ? *reinterpret_cast<volatile uint32_t*>(a.err_word) : 0u) | timed_out;
+      for (int k = 0; k < 2; ++k)
+        if (a.err_also[k]) flags |= *reinterpret_cast<const volatile uint32_t*>(a.err_also[k]);
+      a.result->device_error = flags;
+      a.result->reserved = 0;
+    }
+  }
+}
+
+// Common exit.  Neither CTA may leave while the other can still read its shared memory, signal its barriers
+// or write its tensor memory, and no bulk load may still be writing into a CTA that retires.
+template <int STAGES, typename Sh>
+__device__ __forceinline__ void probe_exit(Sh* sh, uint64_t wait_limit_ns, int warp, uint32_t rank, uint32_t tmem_base) {
+  tc_fence_before();
+  __syncthreads();
+  if (sh->abort_flag && threadIdx.x == 0) {
+    // give-up path: the loads of the last STAGES blocks this producer issued may not have been
+    // awaited by anyone; wait (bounded) until each has landed
+    const uint32_t n = sh->issued;
+    for (uint32_t j = n > (uint32_t)STAGES ? n - STAGES : 0u; j < n; ++j) {
+      const uint32_t bar = smem_u32(&sh->full[j % STAGES]), parity = (j / STAGES) & 1;
+      const uint64_t t0 = global_timer_ns();
+      while (!mbar_try_wait(bar, parity) && global_timer_ns() - t0 < wait_limit_ns) {}
+    }
+  }
+  if (sh->abort_flag && warp == 1 && rank == 0) {
+    // ... and the MMAs issued so far may still be running: one more commit, awaited (bounded) here
+    __syncwarp();
+    if (elect_one())
+      asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                       smem_u32(&sh->drain)) : "memory");
+    __syncwarp();
+    const uint64_t t0 = global_timer_ns();
+    while (!mbar_try_wait(smem_u32(&sh->drain), 0) && global_timer_ns() - t0 < wait_limit_ns) {}
+    __syncwarp();
+  }
+  __syncthreads();
+  __syncwarp();
+  cluster_sync();
+  if (warp == 1) {
+    __syncwarp();
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+  }
+}
+
 template <typename Table>
 __global__ void __launch_bounds__(kProbeThreads, 1)
 tc_group_kernel(const __grid_constant__ Table tab) {
@@ -1389,18 +1476,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
                      smem_u32(&sh->tmem_base)), "r"(512u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
-  if (warp == 2) {
-    for (int i = lane; i < tab.n; i += 32) {
-      const GroupUnit& u = tab.u[i];
-      WalkInfo wi;
-      wi.tile_begin = u.tile_begin; wi.per_b = u.tiles_m * u.tiles_n;
-      wi.inner = u.m_fastest ? -u.tiles_m : u.tiles_n;
-      wi.num_kb = (u.K + kBlockK - 1) / kBlockK;
-      wi.half_n = u.half_n; wi.n_var = u.n_var; wi.var_begin = u.var_begin; wi.K = u.K;
-      sh->walk[i] = wi;
-    }
-    for (int i = lane; i < tab.n_var; i += 32) sh->var[i] = VarInfo{tab.v[i].idesc_lp, tab.v[i].flags};
-  }
+  if (warp == 2) fill_walk(sh, tab, lane);
   tc_fence_before();
   __syncthreads();
   __syncwarp();
@@ -1798,74 +1874,473 @@ tc_group_kernel(const __grid_constant__ Table tab) {
     }
     asm volatile("bar.sync 1, 256;" ::: "memory");
     if (sh->is_last) {
-      // last CTA: every record of every probe is visible; each epilogue warp takes probes
-      // ew, ew + 8, ...; fixed-order sum (lane l takes records l, l+32, ...)
       __threadfence();
-      const uint32_t timed_out = tab.err0 ? (*reinterpret_cast<volatile uint32_t*>(tab.err0) & QM_DEVERR_TIMEOUT) : 0u;
-      for (int vi = ew; vi < tab.n_var; vi += kEpiWarps) {
-        const GroupVar& a = tab.v[vi];
-        double s5[5] = {0, 0, 0, 0, 0};
-        for (int i = lane; i < (int)gridDim.x; i += 32) {
-          const double* rec = a.partials + (int64_t)i * kPartialDoubles;
-          s5[0] += __ldcg(rec); s5[1] = fmax(s5[1], __ldcg(rec + 1)); s5[2] += __ldcg(rec + 2);
-          s5[3] += __ldcg(rec + 3); s5[4] += __ldcg(rec + 4);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          s5[0] += __shfl_xor_sync(0xffffffffu, s5[0], o);
-          s5[1] = fmax(s5[1], __shfl_xor_sync(0xffffffffu, s5[1], o));
-          s5[2] += __shfl_xor_sync(0xffffffffu, s5[2], o);
-          s5[3] += __shfl_xor_sync(0xffffffffu, s5[3], o);
-          s5[4] += __shfl_xor_sync(0xffffffffu, s5[4], o);
-        }
-        if (lane == 0) {
-          a.result->sum_be = s5[0]; a.result->max_be = s5[1]; a.result->sum_diff2 = s5[2];
-          a.result->sum_ref2 = s5[3]; a.result->sum_den2 = s5[4];
-          a.result->count = a.count;
-          uint32_t flags = (a.err_word ? *reinterpret_cast<volatile uint32_t*>(a.err_word) : 0u) | timed_out;
-          for (int k = 0; k < 2; ++k)
-            if (a.err_also[k]) flags |= *reinterpret_cast<const volatile uint32_t*>(a.err_also[k]);
-          a.result->device_error = flags;
-          a.result->reserved = 0;
-        }
-      }
+      write_results(tab, ew, lane);
     }
   }
 
-  // ---------------------------------------------------------------- common exit
-  // Neither CTA may leave while the other can still read its shared memory, signal its barriers
-  // or write its tensor memory, and no bulk load may still be writing into a CTA that retires.
-  tc_fence_before();
-  __syncthreads();
-  if (sh->abort_flag && threadIdx.x == 0) {
-    // give-up path: the loads of the last kStages k-blocks this producer issued may not have been
-    // awaited by anyone; wait (bounded) until each has landed
-    const uint32_t n = sh->issued;
-    for (uint32_t j = n > (uint32_t)kStages ? n - kStages : 0u; j < n; ++j) {
-      const uint32_t bar = smem_u32(&sh->full[j % kStages]), parity = (j / kStages) & 1;
-      const uint64_t t0 = global_timer_ns();
-      while (!mbar_try_wait(bar, parity) && global_timer_ns() - t0 < tab.wait_limit_ns) {}
+  probe_exit<kStages>(sh, tab.wait_limit_ns, warp, rank, tmem_base);
+}
+
+// ------------------------------------------------------------------ the fused probe kernel, one probe per unit
+// Units of one probe share nothing, so their three products run side by side, k-block by k-block: a stage
+// holds the bf16 and the code tiles of 64 contraction entries and one commit frees it.  112 KB go through shared
+// memory per k-block (36 by TMA, 44 of MMA operands, 32 by the converters) against the 96 of the
+// products one after the other, but a tile has no phases: the converters run four blocks ahead
+// across its end, the next tile's reference and denominator MMAs start while this one's last columns are evaluated, and
+// the epilogue takes all three products in one sweep (the reciprocals beside the other arithmetic,
+// the sums in registers) with one wait.  Short contractions are bound by that chain.  Measured, the fused kernel
+// alone, one after the other / side by side: 512 x 512 x 64 x 256 131 / 88 us; 8192 x 4096 with K = 128 75 / 53,
+// K = 256 76 / 64, K = 512 91 / 88, K = 1024 145 / 140.  With three probes per unit sharing wins from K = 64 on (187 / 239 us).
+//   Roles, registers, walk and exit are those of tc_group_kernel.  Tensor memory: columns 0..127 reference, 128..255
+// denominator, 256..383 the 8-bit product, 384..511 four stages of |L| (32 columns of two bf16 each).
+struct CfgS {
+  static constexpr int kStages = 5;          // stages of shared memory (TMA ring)
+  static constexpr int kAbsStages = 4;       // stages of |L| in tensor memory (128 columns / 32)
+  // stage: L, R, |R| (written by the converters), codes of L, codes of R
+  static constexpr uint32_t kOffL = 0, kOffR = kABf16, kOffRa = kOffR + kBBf16, kOffCl = kOffRa + kBBf16;
+  static constexpr uint32_t kOffCr = kOffCl + kALp;
+  static constexpr uint32_t kStageBytes = kOffCr + kBLp;             // 44 KB
+  static constexpr uint32_t kTileBytes = kStages * kStageBytes;      // 220 KB
+  static constexpr uint32_t kColRef = 0, kColDen = 128, kColLp = 256, kColAbsL = 384;   // tensor-memory columns
+};
+
+template <int UNITS>
+struct SharedS {
+  uint64_t full[CfgS::kStages];     // per CTA: this CTA's loads of a stage have landed
+  uint64_t ready[CfgS::kAbsStages]; // leader: both CTAs' converters have seen their loads land and have written
+                                    //         |L| (tensor memory) and |R| (stage)
+  uint64_t empty[CfgS::kStages];    // per CTA: the pair's MMAs have finished with the k-block of the stage
+  uint64_t tmem_full;               // per CTA: the tile's accumulators are complete
+  uint64_t tmem_empty;              // leader: both CTAs' epilogues have copied out reference and denominator
+  uint64_t lp_done;                 // leader: both CTAs' epilogues have finished a tile
+  uint64_t drain;                   // leader, give-up path only: every MMA issued so far has completed
+  uint32_t tmem_base;
+  uint32_t abort_flag;
+  uint32_t is_last;
+  uint32_t issued;                  // k-blocks whose loads the producer has issued (read on the give-up path)
+  float delta_r[2][kBlockN];
+  double red[5][kEpiWarps];
+  WalkInfo walk[UNITS];
+  VarInfo var[UNITS];               // of unit i: it has one probe
+};
+
+// Eq. 3 statistics of the side-by-side kernel, which first brings a chunk into one form (the 8-bit
+// accumulator as fp32, dead columns zeroed) so that one instantiation per scale layout serves every
+// format and the ragged edge.  PER_COL: the right operand has a scale per column
+// (dr_s), otherwise kd2 holds (-delta_l delta_r) twice.
+struct StatsG {
+  float be0, be1;
+  uint64_t d2, r2, n2;
+  float mx;
+};
+template <bool PER_COL>
+__device__ __forceinline__ void stats16g(const uint32_t* rc, const uint32_t* rd, const uint32_t* rq, uint64_t kd2,
+                                         const float* dr_s, StatsG& s) {
+#pragma unroll
+  for (int j = 0; j < 16; j += 2) {
+    const uint64_t a2 = pack2(__uint_as_float(rq[j]), __uint_as_float(rq[j + 1]));
+    const uint64_t cv2 = pack2(__uint_as_float(rc[j]), __uint_as_float(rc[j + 1]));
+    const float d0 = __uint_as_float(rd[j]), d1 = __uint_as_float(rd[j + 1]);
+    const uint64_t dd2 = pack2(d0, d1);
+    uint64_t diff2;                                              // C - A dl dr
+    if (PER_COL) diff2 = fma2(mul2(a2, kd2), *reinterpret_cast<const uint64_t*>(dr_s + j), cv2);
+    else diff2 = fma2(a2, kd2, cv2);
+    // D == 0 implies C == Q == 0, so clamping the divisor keeps BE = 0 there without a branch
+    const uint64_t be2 = mul2(diff2, pack2(rcp_approx(fmaxf(d0, 1e-37f)), rcp_approx(fmaxf(d1, 1e-37f))));
+    float b0, b1;
+    unpack2(be2, b0, b1);
+    s.be0 += fabsf(b0);
+    s.be1 += fabsf(b1);
+    s.mx = fmaxf(s.mx, fmaxf(fabsf(b0), fabsf(b1)));
+    s.d2 = fma2(diff2, diff2, s.d2);
+    s.r2 = fma2(cv2, cv2, s.r2);
+    s.n2 = fma2(dd2, dd2, s.n2);
+  }
+}
+// Chunk CH (16 columns) of a warp's share of a tile: rq holds its 8-bit accumulators as read from
+// tensor memory; n_live < 16 only at the ragged edge of the matrix, whose dead columns count as zeros.
+template <int CH>
+__device__ __forceinline__ void stats_chunk(uint32_t (&rc)[64], uint32_t (&rd)[64], uint32_t (&rq)[16], int n_live,
+                                            bool is_i8, bool per_col, uint64_t kd2, const float* dr_s, StatsG& st) {
+  if (is_i8) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) rq[k] = __float_as_uint((float)(int)rq[k]);
+  }
+  if (n_live < 16) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      if (k >= n_live) { rc[CH * 16 + k] = 0u; rd[CH * 16 + k] = 0u; rq[k] = 0u; }
+  }
+  if (per_col) stats16g<true>(&rc[CH * 16], &rd[CH * 16], rq, kd2, dr_s + CH * 16, st);
+  else stats16g<false>(&rc[CH * 16], &rd[CH * 16], rq, kd2, nullptr, st);
+}
+// Adds one tile's share of a row's Eq. 3 sums to the optional per-row check output.
+__device__ __forceinline__ void row_stats_add(double* rs, const StatsG& st) {
+  float x0, x1;
+  atomicAdd(rs + 0, (double)st.be0 + (double)st.be1);
+  atomicMax(reinterpret_cast<unsigned long long*>(rs + 1), (unsigned long long)__double_as_longlong((double)st.mx));
+  unpack2(st.d2, x0, x1); atomicAdd(rs + 2, (double)x0 + (double)x1);
+  unpack2(st.r2, x0, x1); atomicAdd(rs + 3, (double)x0 + (double)x1);
+  unpack2(st.n2, x0, x1); atomicAdd(rs + 4, (double)x0 + (double)x1);
+}
+
+template <typename Table>
+__global__ void __launch_bounds__(kProbeThreads, 1)
+tc_side_kernel(const __grid_constant__ Table tab) {
+  using C = CfgS;
+  using Sh = SharedS<Table::kUnits>;
+  constexpr int kStages = C::kStages, kAbs = C::kAbsStages;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  Sh* sh = reinterpret_cast<Sh*>(tiles + C::kTileBytes);
+  const uint32_t tile_base = smem_u32(tiles);
+
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
+  const Waiter w{&sh->abort_flag, tab.err0, tab.wait_limit_ns};
+
+  if (warp == 0) {
+    // fetch the tensor maps of this pair's first tile into the descriptor cache
+    const int pos = group_position(0, pair, num_pairs);
+    if (pos < tab.total_tiles && lane < 4) {
+      int pi = 0;
+      while (pi + 1 < tab.n && pos >= tab.u[pi + 1].tile_begin) ++pi;
+      asm volatile("prefetch.tensormap [%0];" ::"l"(lane < 2 ? &tab.u[pi].maps[lane] : &tab.v[pi].maps[lane - 2]) : "memory");
     }
   }
-  if (sh->abort_flag && warp == 1 && rank == 0) {
-    // ... and the MMAs issued so far may still be running: one more commit, awaited (bounded) here
-    __syncwarp();
-    if (elect_one())
-      asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       smem_u32(&sh->drain)) : "memory");
-    __syncwarp();
-    const uint64_t t0 = global_timer_ns();
-    while (!mbar_try_wait(smem_u32(&sh->drain), 0) && global_timer_ns() - t0 < tab.wait_limit_ns) {}
-    __syncwarp();
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(smem_u32(&sh->full[s]), 1);
+      mbar_init(smem_u32(&sh->empty[s]), 1);
+    }
+    for (int s = 0; s < kAbs; ++s) mbar_init(smem_u32(&sh->ready[s]), 2 * 4);   // four converter warps in each CTA
+    mbar_init(smem_u32(&sh->tmem_full), 1);
+    mbar_init(smem_u32(&sh->tmem_empty), 2 * kEpiWarps);
+    mbar_init(smem_u32(&sh->lp_done), 2 * kEpiWarps);
+    mbar_init(smem_u32(&sh->drain), 1);
+    sh->abort_flag = 0;
+    sh->is_last = 0;
+    sh->issued = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&sh->tmem_base)), "r"(512u) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  if (warp == 2) fill_walk(sh, tab, lane);
+  tc_fence_before();
   __syncthreads();
   __syncwarp();
-  cluster_sync();
-  if (warp == 1) {
-    __syncwarp();
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+  cluster_sync();          // the peer's barriers and tensor memory exist before anyone uses them
+  pdl_prologue();          // everything above overlapped the tail of the previous kernel
+  tc_fence_after();
+  const uint32_t tmem_base = sh->tmem_base;
+
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsCtl));
+    if (warp == 0) {
+      // ---------------------------------------------------------- TMA producer (both CTAs)
+      if (lane == 0) {
+        TileWalk tw;
+        uint32_t g = 0;
+        bool ok = true;
+        for (tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs); tw.valid && ok; tw.next_tile()) {
+          const CUtensorMap* const um = tab.u[tw.pi].maps;
+          const CUtensorMap* const vm = tab.v[tw.pi].maps;
+          const int r0 = tw.tc.m_tile * kPairM + (int)rank * kBlockM;     // this CTA's left-operand rows
+          const int c0 = tw.tc.n_tile * kBlockN + (int)rank * tw.half_n;  // this CTA's half of the right operand
+          for (int kb = 0; kb < tw.num_kb; ++kb, ++g) {
+            const uint32_t s = g % kStages, use = g / kStages;
+            // test hook: the consumers' waits run out
+            ok = g < tab.stop_after_kb && (use == 0 || w.wait(smem_u32(&sh->empty[s]), (use - 1) & 1));
+            if (!ok) break;
+            const uint32_t bar = smem_u32(&sh->full[s]), base = tile_base + s * C::kStageBytes;
+            mbar_expect_tx(bar, kABf16 + kALp + (uint32_t)tw.half_n * (kBlockK * 2 + kBlockK));
+            const int k0 = kb * kBlockK;
+            tma_load_3d_local(base + C::kOffR, &um[1], bar, k0, c0, tw.tc.b);     // the converters read this one
+            tma_load_3d_local(base + C::kOffL, &um[0], bar, k0, r0, tw.tc.b);
+            tma_load_3d_local(base + C::kOffCl, &vm[0], bar, k0, r0, tw.tc.b);
+            tma_load_3d_local(base + C::kOffCr, &vm[1], bar, k0, c0, tw.tc.b);
+            sh->issued = g + 1;
+          }
+        }
+      }
+    } else if (warp == 1 && rank == 0) {
+      // ---------------------------------------------------------- MMA issuer (leader CTA, converged warp)
+      const bool lead = elect_one();
+      uint32_t idesc_bf16 = 0;                 // of the tile in hand
+      auto issue_ref_den = [&](uint32_t gg, int kb) {
+        const uint32_t s = gg % kStages, base = tile_base + s * C::kStageBytes;
+        const uint64_t dl = smem_desc(base + C::kOffL, 128), dr = smem_desc(base + C::kOffR, 128);
+#pragma unroll
+        for (int k = 0; k < kBlockK / 16; ++k)   // 16 bf16 = 32 bytes = 2 descriptor units per step
+          mma_pair<kKindF16>(tmem_base + C::kColRef, dl + 2 * k, dr + 2 * k, idesc_bf16, (kb | k) != 0, lead);
+        const uint64_t da = smem_desc(base + C::kOffRa, 128);
+        const uint32_t ta = tmem_base + C::kColAbsL + 32u * (gg % kAbs);
+#pragma unroll
+        for (int k = 0; k < kBlockK / 16; ++k)   // 16 bf16 = 8 columns of tensor memory per step
+          mma_pair_a_tmem(tmem_base + C::kColDen, ta + 8u * k, da + 2 * k, idesc_bf16, (kb | k) != 0, lead);
+      };
+      auto issue_lp = [&](uint32_t gg, int kb, bool is_i8, uint32_t idesc_lp) {
+        const uint32_t base = tile_base + (gg % kStages) * C::kStageBytes;
+        const uint64_t cl = smem_desc(base + C::kOffCl, 64), cr = smem_desc(base + C::kOffCr, 64);
+#pragma unroll
+        for (int k = 0; k < kBlockK / 32; ++k) {  // 32 codes = 32 bytes per step
+          if (is_i8) mma_pair<kKindI8>(tmem_base + C::kColLp, cl + 2 * k, cr + 2 * k, idesc_lp, (kb | k) != 0, lead);
+          else mma_pair<kKindF8>(tmem_base + C::kColLp, cl + 2 * k, cr + 2 * k, idesc_lp, (kb | k) != 0, lead);
+        }
+      };
+      auto wait_stage = [&](uint32_t gg) {
+        if (!w.wait_warp(smem_u32(&sh->ready[gg % kAbs]), (gg / kAbs) & 1)) return false;
+        tc_fence_after();
+        return true;
+      };
+      TileWalk tw;
+      tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
+      uint32_t g = 0;
+      bool ok = true;
+      for (uint32_t it = 0; tw.valid && ok; ++it, tw.next_tile()) {
+        tw.make_uniform();
+        const int num_kb = tw.num_kb;
+        const uint32_t idesc_lp = __shfl_sync(0xffffffffu, sh->var[tw.pi].idesc, 0);
+        const bool is_i8 = __shfl_sync(0xffffffffu, sh->var[tw.pi].flags, 0) & kVarI8;
+        idesc_bf16 = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n);
+        // the reference and denominator blocks come back when both epilogues have copied the
+        // previous tile's values out; the 8-bit block when they have finished that tile
+        if (it > 0 && !w.wait_warp(smem_u32(&sh->tmem_empty), (it - 1) & 1)) break;
+        tc_fence_after();
+        const int n_ahead = num_kb < kAbs ? num_kb : kAbs;
+        for (int j = 0; j < n_ahead && ok; ++j) {
+          ok = wait_stage(g + j);
+          if (ok) issue_ref_den(g + j, j);
+        }
+        if (!ok) break;
+        if (it > 0 && !w.wait_warp(smem_u32(&sh->lp_done), (it - 1) & 1)) break;
+        tc_fence_after();
+        int kb = 0;
+        for (; kb < n_ahead; ++kb, ++g) {
+          issue_lp(g, kb, is_i8, idesc_lp);
+          tc_commit_pair(smem_u32(&sh->empty[g % kStages]), lead);
+        }
+        for (; kb < num_kb && ok; ++kb, ++g) {
+          ok = wait_stage(g);
+          if (!ok) break;
+          issue_ref_den(g, kb);
+          issue_lp(g, kb, is_i8, idesc_lp);
+          tc_commit_pair(smem_u32(&sh->empty[g % kStages]), lead);        // frees the k-block in both CTAs
+        }
+        if (ok) tc_commit_pair(smem_u32(&sh->tmem_full), lead);           // this tile's accumulators are complete
+      }
+    }
+  } else if (warp < kFirstEpiWarp) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsConv));
+    // ------------------------------------------------------------ converters (both CTAs)
+    // As in tc_group_kernel, but only |L| goes to tensor memory (the reference MMAs read L from shared memory),
+    // and the k-blocks are counted through over all tiles: the converters run up to kAbs blocks ahead
+    // of the MMAs across a tile's end.
+    const int q = warp & 3;
+    const int t = q * 32 + lane;                   // 0..127
+    const uint32_t ready_leader = map_to_cta(smem_u32(&sh->ready[0]), 0);
+    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + C::kColAbsL;
+    const uint32_t row_off = (uint32_t)t * 128u, sw = (uint32_t)t & 7u;
+    TileWalk tw;
+    tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
+    bool ok = true;
+    int kb = 0;
+    for (uint32_t g = 0; ok && tw.valid; ++g) {
+      const uint32_t s = g % kStages, sa = g % kAbs, m = 0x7fff7fffu;
+      // the tensor-memory columns were last read by the MMAs of k-block g - kAbs (its commit also
+      // covers every earlier k-block, so the |R| slot of the stage is free as well)
+      if (g >= (uint32_t)kAbs) {
+        const uint32_t gp = g - kAbs;
+        if (!w.wait_warp(smem_u32(&sh->empty[gp % kStages]), (gp / kStages) & 1)) { ok = false; break; }
+      }
+      if (!w.wait_warp(smem_u32(&sh->full[s]), (g / kStages) & 1)) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t base = tile_base + s * C::kStageBytes;
+      uint4 v[8], u[4];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = lds128(base + C::kOffL + row_off + (((uint32_t)j ^ sw) << 4));
+      const uint32_t rsrc = base + C::kOffR + (uint32_t)t * 16u;
+      const int r_vec = tw.half_n * 8;                           // 16-byte vectors of the R half-tile that are in use
+#pragma unroll
+      for (int j = 0; j < 4; ++j) u[j] = t + 128 * j < r_vec ? lds128(rsrc + (uint32_t)j * 2048u) : make_uint4(0u, 0u, 0u, 0u);
+      uint32_t a[32];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        a[4 * j] = v[j].x & m; a[4 * j + 1] = v[j].y & m; a[4 * j + 2] = v[j].z & m; a[4 * j + 3] = v[j].w & m;
+      }
+      tmem_st32(taddr + 32u * sa, a);
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (t + 128 * j < r_vec)
+          sts128(rsrc + (C::kOffRa - C::kOffR) + (uint32_t)j * 2048u, make_uint4(u[j].x & m, u[j].y & m, u[j].z & m, u[j].w & m));
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // generic-proxy writes -> the tensor core's reads
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(ready_leader + sa * 8u);
+      if (++kb >= tw.num_kb) { kb = 0; tw.next_tile(); }
+    }
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
+    // ------------------------------------------------------------ epilogue (warps 8..15, both CTAs)
+    // A warp may touch the tensor-memory lane quarter warp % 4; the two warps of a quarter split
+    // the columns.  Copy this warp's 64 columns of the reference and denominator blocks into
+    // registers, hand those two blocks back to the MMA lane, then walk the 8-bit block in chunks
+    // of 16 columns; the statistics arithmetic runs under the next tile's main loop.
+    const int q = warp & 3;
+    const int ew = warp - kFirstEpiWarp;           // 0..7
+    const int h = ew >> 2;                         // which half of the tile's columns
+    const int et = ew * 32 + lane;                 // 0..255
+    const uint32_t tmem_empty_leader = map_to_cta(smem_u32(&sh->tmem_empty), 0);
+    double acc[5] = {0, 0, 0, 0, 0};               // of the unit in hand: sum BE, max BE, sum diff^2, C^2, D^2
+    int cur = -1;                                  // the unit in hand
+    // reduce the statistics of unit `pi` over the CTA and write its record (all 256 threads call)
+    auto flush = [&](int pi) {
+#pragma unroll
+      for (int i = 0; i < 5; ++i) {
+        double x = acc[i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const double y = __shfl_xor_sync(0xffffffffu, x, o);
+          x = i == 1 ? fmax(x, y) : x + y;
+        }
+        if (lane == 0) sh->red[i][ew] = x;
+        acc[i] = 0.0;
+      }
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      if (et < 5) {
+        double x = 0.0;
+        for (int k = 0; k < kEpiWarps; ++k) x = et == 1 ? fmax(x, sh->red[et][k]) : x + sh->red[et][k];
+        __stcg(tab.v[pi].partials + (int64_t)blockIdx.x * kPartialDoubles + et, x);
+        __threadfence();
+      }
+      asm volatile("bar.sync 1, 256;" ::: "memory");       // red[] may be reused
+    };
+    uint32_t met = 0;                              // bit pi: this CTA has had tiles of unit pi
+    // of the unit in hand (reloaded when the unit changes, not per tile)
+    bool per_col = false, pc_l = false, is_i8 = false, narrow = false;
+    float dr_tensor = 1.f, dl_tensor = 0.f;
+    int pM = 0, pN = 0;                            // a probe's M and N are below 2^31 (its tensor maps require it)
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+    TileWalk tw;
+    tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
+    for (uint32_t it = 0; tw.valid; ++it) {
+      const int pi = tw.pi;
+      if (pi != cur) {
+        if (cur >= 0) flush(cur);
+        cur = pi;
+        met |= 1u << pi;
+        const GroupVar& gv = tab.v[pi];
+        per_col = gv.flags & kVarScalePerCol; pc_l = gv.flags & kVarScalePerRow; is_i8 = gv.flags & kVarI8; narrow = tw.half_n < 64;
+        pM = tab.u[pi].M; pN = tab.u[pi].N;
+        dr_tensor = per_col ? 1.f : __ldg(gv.dr);
+        dl_tensor = pc_l ? 0.f : __ldg(gv.dl);
+      }
+      const TileCoord tc = tw.tc;
+      float* dr_s = sh->delta_r[it & 1];
+      if (per_col && et < kBlockN) {
+        const int col = tc.n_tile * kBlockN + et;
+        dr_s[et] = col < pN ? __ldg(tab.v[pi].dr + (int64_t)tc.b * pN + col) : 0.f;
+      }
+      const int row = tc.m_tile * kPairM + (int)rank * kBlockM + q * 32 + lane;
+      const bool row_ok = row < pM;
+      float dlv = dl_tensor;
+      if (pc_l) dlv = row_ok ? __ldg(tab.v[pi].dl + (int64_t)tc.b * pM + row) : 0.f;
+      // the two warps of a lane quarter split the tile's columns: 64 each, or 32 each where the
+      // tile is 64 wide (outputs at most 64 wide)
+      const int cw = narrow ? 32 : 64, cbase = h * cw;
+      const int colw = tc.n_tile * kBlockN + cbase;                  // first column of this warp
+
+      const bool ok = w.wait(smem_u32(&sh->tmem_full), it & 1);
+      // one barrier publishes delta_r and makes the give-up decision uniform over the epilogue
+      if (epi_barrier_any(!ok)) break;
+      tc_fence_after();
+      // live = columns of this warp that exist in the matrix
+      const int live = pN - colw < cw ? pN - colw : cw;          // <= 0: none
+      const uint32_t lp_addr = lane_addr + C::kColLp + cbase;
+      const uint32_t lp_done_leader = map_to_cta(smem_u32(&sh->lp_done), 0);
+      const float* const drc = dr_s + cbase;
+      uint32_t rc[64], rd[64], rq0[16];
+      tmem_ld32(lane_addr + C::kColRef + cbase, *reinterpret_cast<uint32_t(*)[32]>(&rc[0]));
+      tmem_ld32(lane_addr + C::kColDen + cbase, *reinterpret_cast<uint32_t(*)[32]>(&rd[0]));
+      if (!narrow) {
+        tmem_ld32(lane_addr + C::kColRef + cbase + 32, *reinterpret_cast<uint32_t(*)[32]>(&rc[32]));
+        tmem_ld32(lane_addr + C::kColDen + cbase + 32, *reinterpret_cast<uint32_t(*)[32]>(&rd[32]));
+      }
+      if (live > 0) tmem_ld16(lp_addr, rq0);
+      tmem_ld_wait();
+      // The reference and denominator blocks are in registers: the MMA lane may start the next
+      // tile's bf16 MMAs.  The 8-bit block follows in two steps, its first 16 columns with the
+      // loads above and the rest once the first chunk has been evaluated (which frees the
+      // registers the rest is read into); then the MMA lane may start the next tile's 8-bit MMAs as well, while the
+      // remaining chunks are still being evaluated.  Every warp arrives on each barrier exactly
+      // once per tile.
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive_cluster(tmem_empty_leader);
+        if (live <= 16) mbar_arrive_cluster(lp_done_leader);      // nothing further to read
+      }
+      StatsG st{0.f, 0.f, 0ull, 0ull, 0ull, 0.f};
+      const float kd = -dlv * dr_tensor;
+      const uint64_t kd2 = per_col ? pack2(-dlv, -dlv) : pack2(kd, kd);
+      if (live > 0) stats_chunk<0>(rc, rd, rq0, live, is_i8, per_col, kd2, drc, st);
+      if (live > 16) {
+        // chunk 1 into the first chunk's registers, chunks 2 and 3 into those of the first
+        // chunk's reference and denominator values
+        uint32_t(&rq2)[16] = *reinterpret_cast<uint32_t(*)[16]>(&rc[0]);
+        uint32_t(&rq3)[16] = *reinterpret_cast<uint32_t(*)[16]>(&rd[0]);
+        tmem_ld16(lp_addr + 16, rq0);
+        if (live > 32) tmem_ld16(lp_addr + 32, rq2);
+        if (live > 48) tmem_ld16(lp_addr + 48, rq3);
+        tmem_ld_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(lp_done_leader);
+        stats_chunk<1>(rc, rd, rq0, live - 16, is_i8, per_col, kd2, drc, st);
+        if (live > 32) stats_chunk<2>(rc, rd, rq2, live - 32, is_i8, per_col, kd2, drc, st);
+        if (live > 48) stats_chunk<3>(rc, rd, rq3, live - 48, is_i8, per_col, kd2, drc, st);
+      }
+      if (row_ok) {
+        float x0, x1;
+        acc[0] += (double)st.be0 + (double)st.be1;
+        unpack2(st.d2, x0, x1); acc[2] += (double)x0 + (double)x1;
+        unpack2(st.r2, x0, x1); acc[3] += (double)x0 + (double)x1;
+        unpack2(st.n2, x0, x1); acc[4] += (double)x0 + (double)x1;
+        acc[1] = fmax(acc[1], (double)st.mx);
+        double* const rows = tab.v[pi].row_stats;
+        if (rows) row_stats_add(rows + ((int64_t)tc.b * pM + row) * 5, st);
+      }
+      tw.next_tile();
+    }
+    if (cur >= 0) flush(cur);
+    // the records of the probes this CTA never met are zero
+    if (et == 0) {
+      for (int pi = 0; pi < tab.n; ++pi) {
+        if (met & (1u << pi)) continue;
+        double* rec = tab.v[pi].partials + (int64_t)blockIdx.x * kPartialDoubles;
+        for (int i = 0; i < 5; ++i) __stcg(rec + i, 0.0);
+      }
+    }
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    if (et == 0) {
+      __threadfence();
+      const uint32_t prev = atomicAdd(tab.done_counter, 1u);
+      sh->is_last = prev == gridDim.x - 1 ? 1u : 0u;
+    }
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    if (sh->is_last) {
+      __threadfence();
+      write_results(tab, ew, lane);
+    }
   }
+
+  probe_exit<kStages>(sh, tab.wait_limit_ns, warp, rank, tmem_base);
 }
 
 // ------------------------------------------------------------------ host side
@@ -2028,14 +2503,20 @@ qm_status launch_wide(const CUtensorMap& ma, const CUtensorMap& mb, KernelArgs k
 }  // namespace
 
 namespace {
-template <typename Table>
-constexpr size_t probe_smem() { return (size_t)CfgP::kTileBytes + sizeof(SharedP<Table::kUnits, Table::kVars>) + 1024; }
+// The two forms of the fused kernel: units of one probe, and units of several (see the kernels).
+template <bool SIDE, typename Table>
+struct ProbeKernel {
+  static constexpr auto kernel = SIDE ? tc_side_kernel<Table> : tc_group_kernel<Table>;
+  static constexpr size_t kSmem = 1024 + (SIDE ? (size_t)CfgS::kTileBytes + sizeof(SharedS<Table::kUnits>)
+                                               : (size_t)CfgP::kTileBytes + sizeof(SharedP<Table::kUnits, Table::kVars>));
+  static_assert(kSmem <= 232448, "shared memory of a CTA");
+};
 
 // Bound of the fused kernels' barrier waits and the producer's test hook (see qm_debug_* in qm.h).
 std::atomic<uint64_t> g_wait_limit_ns{1000000000ull};
 std::atomic<uint32_t> g_stop_after_kb{0xffffffffu};
 
-template <typename Table>
+template <typename PK>
 qm_status probe_kernel_ready() {
   static bool attr_done[kMaxDevices] = {};
   const int dev = current_device();
@@ -2045,10 +2526,10 @@ qm_status probe_kernel_ready() {
     // launch if the compiler gave it fewer than the split adds up to, because an increase that
     // cannot be served waits forever
     cudaFuncAttributes fa{};
-    QM_CUDA_OK(cudaFuncGetAttributes(&fa, tc_group_kernel<Table>));
+    QM_CUDA_OK(cudaFuncGetAttributes(&fa, PK::kernel));
     if (fa.numRegs * 4 < kRegsCtl + kRegsConv + 2 * kRegsEpi) return QM_ERR_UNSUPPORTED;
   }
-  return allow_smem(tc_group_kernel<Table>, probe_smem<Table>(), attr_done);
+  return allow_smem(PK::kernel, PK::kSmem, attr_done);
 }
 
 // CTA pairs of the fused probe kernel that can be resident at once (its footprint is the largest
@@ -2056,19 +2537,21 @@ qm_status probe_kernel_ready() {
 qm_status probe_residency() {
   const int dev = current_device();
   if (dev < 0) return QM_ERR_UNSUPPORTED;
-  qm_status as = probe_kernel_ready<TableBig>();
-  if (as == QM_OK) as = probe_kernel_ready<TableOne>();
+  using Widest = ProbeKernel<false, TableBig>;
+  qm_status as = probe_kernel_ready<Widest>();
+  if (as == QM_OK) as = probe_kernel_ready<ProbeKernel<true, TableBig>>();
+  if (as == QM_OK) as = probe_kernel_ready<ProbeKernel<true, TableOne>>();
   if (as != QM_OK) return as;
   if (g_max_pairs[dev] == 0) {
     cudaLaunchConfig_t q{};
     q.gridDim = dim3((unsigned)(2 * (sm_count() / 2))); q.blockDim = dim3(kProbeThreads);
-    q.dynamicSmemBytes = probe_smem<TableBig>();
+    q.dynamicSmemBytes = Widest::kSmem;
     cudaLaunchAttribute qa[1];
     qa[0].id = cudaLaunchAttributeClusterDimension;
     qa[0].val.clusterDim.x = 2; qa[0].val.clusterDim.y = 1; qa[0].val.clusterDim.z = 1;
     q.attrs = qa; q.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tc_group_kernel<TableBig>, &q) == cudaSuccess && n > 0)
+    if (cudaOccupancyMaxActiveClusters(&n, Widest::kernel, &q) == cudaSuccess && n > 0)
       g_max_pairs[dev] = n < sm_count() / 2 ? n : sm_count() / 2;
     else
       g_max_pairs[dev] = sm_count() / 2;
@@ -2089,7 +2572,7 @@ bool same_products(const TcProbeArgs& a, const TcProbeArgs& b) {
          a.g.M == b.g.M && a.g.N == b.g.N && a.g.K == b.g.K && a.g.batch == b.g.batch;
 }
 
-template <typename Table>
+template <bool SIDE, typename Table>
 qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, cudaStream_t s) {
   static Table tab;                    // up to 29 KB: kept off the stack; guarded by the mutex below
   static std::mutex mu;
@@ -2129,8 +2612,9 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, cuda
     for (int j = 0; j < up.n_var; ++j) {
       const TcProbeArgs& p = ps[up.probe[j]];
       GroupVar& v = tab.v[tab.n_var++];
-      if (!make_map(&v.maps[0], p.cl, false, kBlockM, g.K, g.M, g.batch, ldc, g.M * ldc, true) ||
-          !make_map(&v.maps[1], p.cr, false, half_n, g.K, g.N, g.batch, ldc, g.N * ldc, true))
+      // blocks of codes are 64 entries deep beside the bf16 tiles, 128 on their own
+      if (!make_map(&v.maps[0], p.cl, false, kBlockM, g.K, g.M, g.batch, ldc, g.M * ldc, !SIDE) ||
+          !make_map(&v.maps[1], p.cr, false, half_n, g.K, g.N, g.batch, ldc, g.N * ldc, !SIDE))
         return QM_ERR_CUDA;
       v.dl = p.dl; v.dr = p.dr;
       v.partials = p.partials; v.result = p.result; v.row_stats = p.row_stats;
@@ -2146,7 +2630,7 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, cuda
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(2 * (total < pairs ? total : pairs)));
   cfg.blockDim = dim3(kProbeThreads);
-  cfg.dynamicSmemBytes = probe_smem<Table>();
+  cfg.dynamicSmemBytes = ProbeKernel<SIDE, Table>::kSmem;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -2158,7 +2642,7 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, cuda
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   profile_events(&ev0, &ev1);
   if (ev0) QM_CUDA_OK(cudaEventRecord(ev0, s));
-  QM_CUDA_OK(cudaLaunchKernelEx(&cfg, tc_group_kernel<Table>, tab));
+  QM_CUDA_OK(cudaLaunchKernelEx(&cfg, ProbeKernel<SIDE, Table>::kernel, tab));
   if (ev1) QM_CUDA_OK(cudaEventRecord(ev1, s));
   count_launch();
   return QM_OK;
@@ -2187,22 +2671,33 @@ qm_status launch_tc_probes(const TcProbeArgs* ps, int n, cudaStream_t s) {
     }
     u->probe[u->n_var++] = i;
   }
+  // Units of one probe go to the side-by-side kernel, ahead of the others, unless they could not fill the GPU and there
+  // are others: a launch more costs its set-up and drain, about 10 us, and they ride along instead.
+  auto single = [](const UnitPlan& u) { return u.n_var == 1; };
+  const auto others = std::stable_partition(units.begin(), units.end(), single);
+  int64_t single_tiles = 0;
+  for (auto u = units.begin(); u != others; ++u) single_tiles += tile_count(u->g);
+  const size_t n_side = others == units.end() || single_tiles >= max_pairs() ? (size_t)(others - units.begin()) : 0;
   // descending tile cost: kilobytes through shared memory per 64 contraction entries
-  std::stable_sort(units.begin(), units.end(), [](const UnitPlan& a, const UnitPlan& b) {
-    return a.g.K * (88 + 24 * a.n_var) > b.g.K * (88 + 24 * b.n_var);
-  });
+  auto by_cost = [](const UnitPlan& a, const UnitPlan& b) { return a.g.K * (72 + 24 * a.n_var) > b.g.K * (72 + 24 * b.n_var); };
+  std::stable_sort(units.begin(), units.begin() + n_side, by_cost);
+  std::stable_sort(units.begin() + n_side, units.end(), by_cost);
   for (size_t u0 = 0; u0 < units.size() && st == QM_OK;) {
+    const bool side = u0 < n_side;
+    const size_t end = side ? n_side : units.size();
     size_t u1 = u0;
     int64_t tiles = 0;
     int vars = 0;
-    while (u1 < units.size() && (int)(u1 - u0) < TableBig::kUnits && vars + units[u1].n_var <= TableBig::kVars &&
+    while (u1 < end && (int)(u1 - u0) < TableBig::kUnits && vars + units[u1].n_var <= TableBig::kVars &&
            tiles + tile_count(units[u1].g) < (1ll << 31)) {
       vars += units[u1].n_var;
       tiles += tile_count(units[u1].g);
       ++u1;
     }
-    st = u1 - u0 == 1 && vars == 1 ? launch_units<TableOne>(ps, &units[u0], 1, s)
-                                   : launch_units<TableBig>(ps, &units[u0], (int)(u1 - u0), s);
+    const int count = (int)(u1 - u0);
+    if (!side) st = launch_units<false, TableBig>(ps, &units[u0], count, s);
+    else if (count == 1) st = launch_units<true, TableOne>(ps, &units[u0], 1, s);
+    else st = launch_units<true, TableBig>(ps, &units[u0], count, s);
     u0 = u1;
   }
   return st != QM_OK ? st : refused;

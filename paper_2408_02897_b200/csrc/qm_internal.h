@@ -176,8 +176,9 @@ struct TcProbeArgs {
 int tc_probe_records(GemmShape g);
 qm_status launch_tc_probe(const TcProbeArgs& a, cudaStream_t s);
 // One-format probes in as few persistent launches as their number allows, those of the same two operands
-// sharing the reference and denominator products (every probe's operands must be prepared
-// already; each writes its own record; the done_counter of one probe per launch counts the CTAs).
+// sharing the reference and denominator products, those that share nothing in launches of another form of
+// the kernel (every probe's operands must be prepared already; each writes its own record; the
+// done_counter of one probe per launch counts the CTAs).
 // Probes from the first one with refused extents on are not run; the ones before it are.
 qm_status launch_tc_probes(const TcProbeArgs* ps, int n, cudaStream_t s);
 // Bound of every barrier wait of the fused probe kernel (0 restores the default of one second), and

@@ -87,3 +87,22 @@ def test_a_batch_reports_the_timeout_in_every_record(starved_producer):
     torch.cuda.synchronize()
     for o, r in zip(ops, batch.results()):
         check_against_oracle(o, r)
+
+
+# Probes that share their products: four blocks of the operands, then two of codes per probe.  Starved at the first, among the
+# operands, at the first codes, inside the first probe's and inside the third's
+@pytest.mark.parametrize("stop_after", [0, 2, 4, 5, 9])
+def test_shared_products_report_the_timeout_in_every_record(starved_producer, stop_after):
+    o = small_op(seed=35)
+    Ld, Rd = o["L"].cuda(), o["R"].cuda()
+    formats = ("e4m3", "e5m2", "int8")
+    batch = qm.ProbeBatch([(qm.operand_of(Ld, o["cl"]), qm.operand_of(Rd, o["cr"]), f, f, "tensor", "tensor") for f in formats])
+    starved_producer.qm_debug_stop_producer_after(stop_after)
+    batch.launch()
+    torch.cuda.synchronize()
+    assert all(r.device_error & QM_DEVERR_TIMEOUT for r in batch.results())
+    starved_producer.qm_debug_stop_producer_after(0xffffffff)
+    batch.launch()
+    torch.cuda.synchronize()
+    for f, r in zip(formats, batch.results()):
+        check_against_oracle({**o, "fmt_l": f, "fmt_r": f}, r)

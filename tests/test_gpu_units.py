@@ -1,5 +1,6 @@
 """Probes of the same operands in one batch share their reference and denominator products: every record
-must be the one the probe gives on its own, for every number of formats and granularities per product."""
+must be the one the probe gives on its own (which the other form of the fused kernel evaluates), for every
+number of formats and granularities per product, and whatever else is in the batch."""
 import pytest
 import torch
 
@@ -55,3 +56,31 @@ def test_shared_products_against_the_oracle():
         want = oracle.probe(L.float().numpy(), R.float().numpy().T, f, f, g, g)
         for k in FIELDS:     # the tolerances of the one-probe tests: fp32 accumulation with truncation
             assert abs(rec.record()[k] - want[k]) <= (1e-3 if k == "max_be" else 1e-4) * abs(want[k]), (f, g, k)
+
+
+# Products asked for once beside one asked for in three formats: 26 of four tiles each fill the GPU and take the side-by-side
+# kernel (24 to a launch), three do not and ride along with the others
+@pytest.mark.parametrize("n_single,launches", [(26, 3), (3, 1)])
+def test_products_of_one_probe_beside_shared_ones(n_single, launches):
+    keep, probes = [], []
+    for i in range(n_single):
+        L, R = (t.cuda() for t in operands(300, 200, 64 + 16 * (i % 9), 1, 300 + i))
+        keep.append((L, R))
+        f, g, _ = VARIANTS[(0, 1, 3)[i % 3]]
+        probes.append((qm.operand_of(L, -1), qm.operand_of(R, -1), f, f, g, g))
+    L, R = (t.cuda() for t in operands(513, 130, 272, 1, 299))
+    Lo, Ro = qm.operand_of(L, -1), qm.operand_of(R, -1)
+    probes[1:1] = [(Lo, Ro, f, f, g, g) for f, g, r in VARIANTS[:4] if r == "rtne"]
+    b = qm.ProbeBatch(probes)
+    binding.profile_enable(True)
+    try:
+        b.launch()
+        torch.cuda.synchronize()
+        assert binding.profile_read()[1] == launches
+    finally:
+        binding.profile_enable(False)
+    for p, rec in zip(probes, b.results()):
+        alone = qm.qm_probe_layer(*p, "bf16").record()
+        assert rec.device_error == 0 and rec.record()["count"] == alone["count"]
+        for k in FIELDS:
+            assert abs(rec.record()[k] - alone[k]) <= 1e-12 * abs(alone[k]), k
