@@ -599,12 +599,9 @@ __device__ __forceinline__ void transpose_tile(const __nv_bfloat16* __restrict__
 
 // One format, scales from a DeltaSrc (per tensor or per output row, finished or from max|x|).
 template <int FMT, bool EDGE, bool SR>
-__global__ void __launch_bounds__(kThreads, SR ? 3 : 1)
-quantize_transpose_tile_kernel(const __nv_bfloat16* __restrict__ x, int64_t nc, int64_t c, int64_t s_c, int64_t s_b,
-                               const DeltaSrc ds, uint8_t* __restrict__ codes, int64_t ldc,
-                               __nv_bfloat16* __restrict__ kmaj_copy, const Rounding rnd) {
-  pdl_prologue();
-  __shared__ uint4 smem[TileSmem<1 << FMT>::kVec];
+__device__ __forceinline__ void quantize_transpose_tile(const __nv_bfloat16* __restrict__ x, int64_t nc, int64_t c, int64_t s_c,
+                                                        int64_t s_b, const DeltaSrc& ds, uint8_t* __restrict__ codes, int64_t ldc,
+                                                        __nv_bfloat16* __restrict__ kmaj_copy, const Rounding& rnd, uint4* smem) {
   const int pcol = threadIdx.x & 31, g = threadIdx.x >> 5;
   const int64_t col = (int64_t)blockIdx.x * 64 + 2 * pcol, orow = (int64_t)blockIdx.z * nc + col;
   float d_lo[3] = {1.f, 1.f, 1.f}, d_hi[3] = {1.f, 1.f, 1.f};
@@ -617,6 +614,28 @@ quantize_transpose_tile_kernel(const __nv_bfloat16* __restrict__ x, int64_t nc, 
   uint8_t* const cd[3] = {codes, codes, codes};
   if (ds.from_amax) transpose_tile<1 << FMT, false, EDGE, SR>(x, nc, c, s_c, s_b, d_lo, d_hi, cd, ldc, kmaj_copy, smem, blockIdx, rnd);
   else transpose_tile<1 << FMT, true, EDGE, SR>(x, nc, c, s_c, s_b, d_lo, d_hi, cd, ldc, kmaj_copy, smem, blockIdx, rnd);
+}
+
+// Bound by HBM and by how many blocks hide the tile's load, compute and store phases: no second launch bound, with
+// one (even of 1) the compiler takes 69 to 77 registers instead of 48 to 52, three blocks on an SM instead of
+// four (INT8 codes of 16384 x 4096 under given scales: 56.0 us so, 44.6 without).
+template <int FMT, bool EDGE>
+__global__ void __launch_bounds__(kThreads)
+quantize_transpose_tile_kernel(const __nv_bfloat16* __restrict__ x, int64_t nc, int64_t c, int64_t s_c, int64_t s_b,
+                               const DeltaSrc ds, uint8_t* __restrict__ codes, int64_t ldc, __nv_bfloat16* __restrict__ kmaj_copy) {
+  pdl_prologue();
+  __shared__ uint4 smem[TileSmem<1 << FMT>::kVec];
+  quantize_transpose_tile<FMT, EDGE, false>(x, nc, c, s_c, s_b, ds, codes, ldc, kmaj_copy, Rounding{}, smem);
+}
+// Stochastic rounding, bound by its draws: three blocks on an SM.
+template <int FMT, bool EDGE>
+__global__ void __launch_bounds__(kThreads, 3)
+quantize_transpose_tile_sr_kernel(const __nv_bfloat16* __restrict__ x, int64_t nc, int64_t c, int64_t s_c, int64_t s_b,
+                                  const DeltaSrc ds, uint8_t* __restrict__ codes, int64_t ldc,
+                                  __nv_bfloat16* __restrict__ kmaj_copy, const Rounding rnd) {
+  pdl_prologue();
+  __shared__ uint4 smem[TileSmem<1 << FMT>::kVec];
+  quantize_transpose_tile<FMT, EDGE, true>(x, nc, c, s_c, s_b, ds, codes, ldc, kmaj_copy, rnd, smem);
 }
 
 // Every format in MASK from one read, per-tensor scales from the tensor's max|x|.
@@ -1254,12 +1273,15 @@ qm_status quantize_t(const View& x, int gran, const float* delta, bool from_amax
     }
   } else {
     if (!abs_copy && tile_transposable(x)) {
-#define QM_TT(E, S)                                                                                            \
-  launch_pdl(quantize_transpose_tile_kernel<FMT, E, S>, tile_grid(x), dim3(kThreads), 0, s,                    \
-             static_cast<const __nv_bfloat16*>(x.data), x.nc, x.c, x.s_c, x.s_b, ds, codes, ldc,               \
-             static_cast<__nv_bfloat16*>(kmaj_copy), rnd)
-      if (tile_edges(x)) { if (rnd.stochastic) QM_TT(true, true); else QM_TT(true, false); }
-      else { if (rnd.stochastic) QM_TT(false, true); else QM_TT(false, false); }
+#define QM_TT(KERNEL, ...)                                                                                      \
+  launch_pdl(KERNEL, tile_grid(x), dim3(kThreads), 0, s, static_cast<const __nv_bfloat16*>(x.data), x.nc, x.c, x.s_c, x.s_b, ds, \
+             codes, ldc, static_cast<__nv_bfloat16*>(kmaj_copy), ##__VA_ARGS__)
+      if (!rnd.stochastic) {
+        if (tile_edges(x)) QM_TT((quantize_transpose_tile_kernel<FMT, true>)); else QM_TT((quantize_transpose_tile_kernel<FMT, false>));
+      } else {
+        if (tile_edges(x)) QM_TT((quantize_transpose_tile_sr_kernel<FMT, true>), rnd);
+        else QM_TT((quantize_transpose_tile_sr_kernel<FMT, false>), rnd);
+      }
 #undef QM_TT
       count_launch();
       QM_CUDA_OK(cudaGetLastError());
