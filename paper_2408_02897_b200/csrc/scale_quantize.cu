@@ -1353,16 +1353,17 @@ qm_status launch_absmax(const View& x, int gran, uint32_t* amax_bits, cudaStream
                                : absmax_t<float>(x, gran, amax_bits, s);
 }
 
-// Which operands the two-launch form takes: up to 2^22 elements, and no rows with stochastic rounding under a
-// scale each, whose maxima nobody would have taken.  Whole probes, six launches against three: 128 x 128 x 128
-// 21.7 / 18.7 us, fp32 128 x 256 x 256 24.1 / 20.6, 2000 x 1000 x 704 31.6 / 28.0, 4096 x 2048 x 1024 with
-// operands of 4 M and 2 M elements 65.4 / 63.6; with both at 2^23 elements a single operand's own kernels fill
-// the GPU and are the faster ones (4096 x 2048 x 2048, strided: 101 / 113).
+// Which operands the two-launch form takes: fewer than 2^22 elements in both together, at most 2048 contiguous rows
+// with a scale each, and no such rows with stochastic rounding, whose maxima nobody would have taken.  Whole probes, the
+// general kernels / this form: 64 x 64 x 64 21.6 / 19.2 us, 1024 x 1024 x 1024 strided INT8 channel scales 36.7 / 31.7,
+// 2048 x 1024 x 1024 33.9 / 31.7.  Beyond either line the operands' own kernels, lighter ones, fill the GPU
+// and are faster: 4096 x 1024 x 1024 strided 44.3 / 46.0, 2048 x 2048 x 2048 60.3 / 64.1; 16384 rows of 256 22.6 / 25.9.
 static bool pair_size(const View& v) {
   return v.nc <= (1 << 22) && v.c <= (1 << 22) && v.batch <= (1 << 15) && v.nc * v.c <= (1ll << 22) && v.nc * v.c * v.batch <= (1ll << 22);
 }
 static bool pair_serves(const View& v, int gran, bool stochastic) {
-  return pair_size(v) && !(gran == QM_GRAN_CHANNEL && v.c_contig() && stochastic);
+  const bool rows = gran == QM_GRAN_CHANNEL && v.c_contig();
+  return pair_size(v) && !(rows && (stochastic || v.nc * v.batch > 2048));
 }
 
 size_t pair_partial_words(const View& v, int gran) {
@@ -1372,7 +1373,8 @@ size_t pair_partial_words(const View& v, int gran) {
 }
 
 bool pair_prepare_serves(const View& l, int gran_l, bool draw_l, const View& r, int gran_r, bool draw_r) {
-  return l.dtype == r.dtype && pair_serves(l, gran_l, draw_l) && pair_serves(r, gran_r, draw_r);
+  return l.dtype == r.dtype && pair_serves(l, gran_l, draw_l) && pair_serves(r, gran_r, draw_r) &&
+         (l.nc + r.nc) * l.c * l.batch < (1ll << 22);
 }
 
 qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint32_t control_words, cudaStream_t s) {

@@ -21,7 +21,9 @@ def stored(rng, rows, K, cd, batch, dtype):
     return x, wide.cuda()[..., :shape[-1]]
 
 
-@pytest.mark.parametrize("M,N,K,batch", [(1, 1, 16, 1), (130, 67, 144, 1), (300, 64, 16, 3), (64, 770, 2032, 1), (1024, 1000, 1040, 1)])
+# (the last two: either side of the line in rows, and of the one in elements)
+@pytest.mark.parametrize("M,N,K,batch", [(1, 1, 16, 1), (130, 67, 144, 1), (300, 64, 16, 3), (64, 770, 2032, 1), (1024, 1000, 1040, 1),
+                                         (2048, 2049, 48, 1), (2000, 2161, 1008, 1)])
 @pytest.mark.parametrize("cl,cr", [(-1, -2), (-2, -1), (-1, -1), (-2, -2)])
 @pytest.mark.parametrize("fl,fr", [("e4m3", "e4m3"), ("e4m3", "e5m2"), ("e5m2", "e4m3"), ("e5m2", "e5m2"), ("int8", "int8")])
 @pytest.mark.parametrize("gran", ["tensor", "channel"])
