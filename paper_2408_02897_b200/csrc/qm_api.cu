@@ -664,10 +664,11 @@ qm_status batch_streams(BatchStreams** out) {
 // several products, ask for the same things many times over; inside a batch each is made once:
 //   code_root: the earlier operand with the same view, scale grouping, format and rounding: its
 //              scales, codes and copy are used as they are and nothing is launched;
-//   copy_root: the earlier operand with the same view and scale grouping under another format:
-//              its max|x| and contraction-major copy are borrowed, only the codes are made;
+//   pass_root: the earlier operand with the same view and scale grouping under another format:
+//              its max|x| is borrowed, and its pass over the tensor makes this one's codes too where it can;
 //   amax_root: per-tensor scales only: the earlier operand over the same elements in either
-//              orientation (max|x| does not depend on which dimension contracts).
+//              orientation (max|x| does not depend on which dimension contracts);
+//   kmaj_root: the first operand with the same view, whatever its scales: its contraction-major copy is used.
 // A root index equal to the slot's own index means "makes it itself".
 struct Slot {
   View v;
@@ -676,7 +677,7 @@ struct Slot {
   StochasticDraw draw;
   uint32_t* amax; float* delta; uint8_t* codes; void* kmaj; uint32_t* err;
   bool keeps_amax;                 // false when the single-pass per-row kernel prepares it (no maxima are stored)
-  int code_root, copy_root, amax_root;
+  int code_root, pass_root, amax_root, kmaj_root;
   int stream;                      // index of the library stream its kernels go to
 };
 
@@ -693,27 +694,29 @@ bool grouped_scales(const Slot& x) { return x.gran == QM_GRAN_CHANNEL && x.group
 
 void find_roots(std::vector<Slot>& slots, int t) {
   Slot& x = slots[t];
-  x.code_root = x.copy_root = x.amax_root = t;
+  x.code_root = x.pass_root = x.amax_root = x.kmaj_root = t;
+  for (int u = 0; u < t && x.kmaj_root == t; ++u)
+    if (same_view(x.v, slots[u].v)) x.kmaj_root = u;        // the first of its view: makes everything itself
   const int gx = grouped_scales(x) ? x.groups : 0;
   for (int u = 0; u < t; ++u) {
     const Slot& y = slots[u];
     if (y.code_root != u || !same_view(x.v, y.v) || y.gran != x.gran || (grouped_scales(y) ? y.groups : 0) != gx) continue;
     const bool same_round = x.stochastic == y.stochastic &&
                             (!x.stochastic || (x.draw.seed == y.draw.seed && x.draw.stream == y.draw.stream));
-    if (y.fmt == x.fmt && same_round) { x.code_root = u; x.copy_root = y.copy_root; x.amax_root = y.amax_root; return; }
+    if (y.fmt == x.fmt && same_round) { x.code_root = u; x.pass_root = y.pass_root; x.amax_root = y.amax_root; return; }
   }
   for (int u = 0; u < t; ++u) {
     const Slot& y = slots[u];
-    if (y.code_root != u || y.copy_root != u || !y.keeps_amax) continue;
+    if (y.code_root != u || y.pass_root != u || !y.keeps_amax) continue;
     if (same_view(x.v, y.v) && y.gran == x.gran && (grouped_scales(y) ? y.groups : 0) == gx) {
-      x.copy_root = u; x.amax_root = y.amax_root;
+      x.pass_root = u; x.amax_root = y.amax_root;
       return;
     }
   }
   if (x.gran != QM_GRAN_TENSOR) return;
   for (int u = 0; u < t; ++u) {
     const Slot& y = slots[u];
-    if (y.code_root != u || y.copy_root != u || y.amax_root != u || y.gran != QM_GRAN_TENSOR) continue;
+    if (y.code_root != u || y.pass_root != u || y.amax_root != u || y.gran != QM_GRAN_TENSOR) continue;
     if (same_view(x.v, y.v) || transposed_view(x.v, y.v)) { x.amax_root = u; return; }
   }
 }
@@ -804,9 +807,9 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
     if (done[t]) continue;
     qm_status e = QM_OK;
     const StochasticDraw* draw = x.stochastic ? &x.draw : nullptr;
-    if (x.copy_root != (int)t) {
-      // borrows max|x| and the contraction-major copy, and was not served with its lender's formats
-      x.stream = slots[x.copy_root].stream;
+    if (x.pass_root != (int)t) {
+      // borrows max|x|, and was not served with its lender's formats
+      x.stream = slots[x.pass_root].stream;
       e = launch_quantize(x.v, x.fmt, x.gran, reinterpret_cast<const float*>(slots[x.amax_root].amax), true, x.delta, x.err,
                           x.codes, nullptr, nullptr, b->s[x.stream], draw);
     } else if (!x.keeps_amax) {
@@ -822,7 +825,8 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
       }
       cudaStream_t s = b->s[x.stream];
       const uint32_t* amax = slots[x.amax_root].amax;
-      // this operand's format and those of the later operands that borrow its copy: one pass over
+      void* const kmaj = x.kmaj_root == (int)t ? x.kmaj : nullptr;
+      // this operand's format and those of the later operands that borrow its pass: one pass over
       // the tensor writes all their codes (round-to-nearest-even ones; stochastic ones go singly)
       int fmts[3]; float* deltas[3]; uint32_t* errs[3]; uint8_t* codes[3];
       int nf = 0;
@@ -830,7 +834,7 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
       if (!x.stochastic) { fmts[nf] = x.fmt; deltas[nf] = x.delta; errs[nf] = x.err; codes[nf] = x.codes; ++nf; }
       for (size_t u = t + 1; u < slots.size() && nf < 3; ++u) {
         Slot& y = slots[u];
-        if (y.code_root != (int)u || y.copy_root != (int)t || y.stochastic || done[u]) continue;
+        if (y.code_root != (int)u || y.pass_root != (int)t || y.stochastic || done[u]) continue;
         bool dup = false;
         for (int k = 0; k < nf; ++k) dup |= fmts[k] == y.fmt;
         if (dup) continue;
@@ -839,11 +843,11 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
       }
       if (e == QM_OK && x.stochastic) {
         e = launch_quantize(x.v, x.fmt, x.gran, reinterpret_cast<const float*>(amax), true, x.delta, x.err, x.codes, nullptr,
-                            x.kmaj, s, draw);
+                            kmaj, s, draw);
         kmaj_written = true;
       }
       if (e == QM_OK && nf > 0)
-        e = launch_quantize_multi(x.v, x.gran, amax, nf, fmts, deltas, errs, codes, kmaj_written ? nullptr : x.kmaj, s);
+        e = launch_quantize_multi(x.v, x.gran, amax, nf, fmts, deltas, errs, codes, kmaj_written ? nullptr : kmaj, s);
     }
     done[t] = 1;
     if (e != QM_OK && st == QM_OK) st = e;
@@ -871,8 +875,8 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
     const Slot& xr = slots[slot_of[i] + 1];
     const Slot& cl = slots[xl.code_root];
     const Slot& cr = slots[xr.code_root];
-    void* kl = slots[cl.copy_root].kmaj;
-    void* kr = slots[cr.copy_root].kmaj;
+    void* kl = slots[cl.kmaj_root].kmaj;
+    void* kr = slots[cr.kmaj_root].kmaj;
     TcProbeArgs p{};
     p.l = kl ? kl : pl.Lv.data; p.l_ld = kl ? pl.Lv.c : pl.Lv.s_nc; p.l_sb = kl ? pl.Lv.nc * pl.Lv.c : pl.Lv.s_b;
     p.r = kr ? kr : pl.Rv.data; p.r_ld = kr ? pl.Rv.c : pl.Rv.s_nc; p.r_sb = kr ? pl.Rv.nc * pl.Rv.c : pl.Rv.s_b;

@@ -84,3 +84,28 @@ def test_products_of_one_probe_beside_shared_ones(n_single, launches):
         assert rec.device_error == 0 and rec.record()["count"] == alone["count"]
         for k in FIELDS:
             assert abs(rec.record()[k] - alone[k]) <= 1e-12 * abs(alone[k]), k
+
+
+# Operands with a strided contraction need a contraction-major copy: one per operand, whatever the scales of the probes that
+# use it, so that probes of both granularities (and roundings) share their products too
+@pytest.mark.parametrize("cl,cr", [(-2, -2), (-2, -1), (-1, -2)])
+def test_one_copy_of_a_strided_operand_whatever_the_scales(cl, cr):
+    M, N, K, fill = 300, 200, 272, -0x5A5A5A5B
+    L, R = operands(M, N, K, 1, 8)
+    Ld, Rd = (t.cuda() if c == -1 else t.T.contiguous().cuda() for t, c in ((L, cl), (R, cr)))
+    Lo, Ro = qm.operand_of(Ld, cl), qm.operand_of(Rd, cr)
+    b = qm.ProbeBatch([(Lo, Ro, f, f, g, g) for f, g, _ in VARIANTS])
+    for c, (_, _, r) in zip(b.cfg, VARIANTS):
+        c.round, c.seed = binding.ROUND[r], 5
+    for w in b._ws:
+        w.view(torch.int32).fill_(fill)
+    b.launch()
+    torch.cuda.synchronize()
+    copies = 2 * K * ((M if cl == -2 else 0) + (N if cr == -2 else 0))
+    untouched = [4 * int((w.view(torch.int32) == fill).sum()) for w in b._ws]
+    assert untouched[0] < copies and all(u >= copies for u in untouched[1:]), (untouched, copies)
+    for (f, g, r), rec in zip(VARIANTS, b.results()):
+        alone = qm.qm_probe_layer(Lo, Ro, f, f, g, g, "bf16", rounding=r, seed=5).record()
+        assert rec.device_error == 0
+        for k in FIELDS:
+            assert abs(rec.record()[k] - alone[k]) <= 1e-12 * abs(alone[k]), (f, g, r, k)
