@@ -90,7 +90,7 @@ def test_products_of_one_probe_beside_shared_ones(n_single, launches):
 # use it, so that probes of both granularities (and roundings) share their products too
 @pytest.mark.parametrize("cl,cr", [(-2, -2), (-2, -1), (-1, -2)])
 def test_one_copy_of_a_strided_operand_whatever_the_scales(cl, cr):
-    M, N, K, fill = 300, 200, 272, -0x5A5A5A5B
+    M, N, K, fill = 304, 200, 272, -0x5A5A5A5B          # (strided rows are a multiple of 8 elements apart)
     L, R = operands(M, N, K, 1, 8)
     Ld, Rd = (t.cuda() if c == -1 else t.T.contiguous().cuda() for t, c in ((L, cl), (R, cr)))
     Lo, Ro = qm.operand_of(Ld, cl), qm.operand_of(Rd, cr)
