@@ -542,6 +542,8 @@ __device__ __forceinline__ void transpose_tile(const __nv_bfloat16* __restrict__
       s_kmaj[n * 16 + ((2 * g) ^ sw)] = a;
       s_kmaj[n * 16 + ((2 * g + 1) ^ sw)] = bb;
     }
+    // what lies beyond the matrix is not written; its zeros would take the slow branch of stochastic rounding
+    if (EDGE && (n0 + n >= nc || k0 + 16 * g >= c)) continue;
 #pragma unroll
     for (int f = 0; f < 3; ++f) {
       if (!(MASK & (1 << f))) continue;
@@ -1228,6 +1230,14 @@ bool tile_transposable(const View& x) {
 }
 bool tile_edges(const View& x) { return (x.c & 127) || (x.nc & 63); }
 dim3 tile_grid(const View& x) { return dim3((unsigned)((x.nc + 63) / 64), (unsigned)((x.c + 127) / 128), (unsigned)x.batch); }
+// Stochastic rounding takes them from two tiles for three SMs on: a thread draws 32 numbers in sequence there, 16 in the
+// general kernel, which with fewer tiles is the faster one: 256 x 32 5.1 / 2.5 us, 1024 x 200 5.2 / 3.4, 512 x 1024 (64
+// tiles) 3.8 / 3.4; 1024 x 1024 (128) 3.9 / 4.4, 4096 x 1024 9.0 / 10.8 (tile kernel / general kernel).
+bool tile_form(const View& x, bool stochastic) {
+  if (!tile_transposable(x)) return false;
+  const dim3 g = tile_grid(x);
+  return !stochastic || 3 * (int64_t)g.x * g.y * g.z >= 2 * (int64_t)sm_count();
+}
 
 template <typename T, int FMT>
 qm_status quantize_t(const View& x, int gran, const float* delta, bool from_amax, float* delta_out,
@@ -1272,7 +1282,7 @@ qm_status quantize_t(const View& x, int gran, const float* delta, bool from_amax
                                      x.c * 2, x.nc, cudaMemcpyDeviceToDevice, s));
     }
   } else {
-    if (!abs_copy && tile_transposable(x)) {
+    if (!abs_copy && tile_form(x, rnd.stochastic)) {
 #define QM_TT(KERNEL, ...)                                                                                      \
   launch_pdl(KERNEL, tile_grid(x), dim3(kThreads), 0, s, static_cast<const __nv_bfloat16*>(x.data), x.nc, x.c, x.s_c, x.s_b, ds, \
              codes, ldc, static_cast<__nv_bfloat16*>(kmaj_copy), ##__VA_ARGS__)
@@ -1387,7 +1397,7 @@ qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint
     o.v = v; o.per_channel = in.gran == QM_GRAN_CHANNEL;
     o.partial = in.partial; o.delta = in.delta; o.codes = in.codes; o.kmaj = static_cast<__nv_bfloat16*>(in.kmaj);
     if (in.draw) { o.rnd.stochastic = 1; o.rnd.k0 = (uint32_t)in.draw->seed; o.rnd.k1 = (uint32_t)(in.draw->seed >> 32); o.rnd.stream = in.draw->stream; }
-    const bool tiles = tile_transposable(v);
+    const bool tiles = tile_form(v, in.draw != nullptr);
     const int64_t ldc = qm_code_ld(v.c);
     if (v.c_contig()) {
       const int64_t chunks = ldc >> 4, threads = v.nc * v.batch * (o.per_channel ? 32 : chunks);

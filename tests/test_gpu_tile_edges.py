@@ -28,7 +28,9 @@ def check(codes, delta, x, fmt, gran, K, rounding="rtne"):
     assert not got[..., K:].any()                              # the padding of a row of codes is zero
 
 
-@pytest.mark.parametrize("K,nc,batch", [(16, 1, 1), (128, 64, 1), (112, 63, 1), (144, 66, 1), (272, 130, 2), (2032, 70, 1)])
+# (the last three have tiles enough for the stochastic form of the tile kernel, the others take the general one)
+@pytest.mark.parametrize("K,nc,batch", [(16, 1, 1), (128, 64, 1), (112, 63, 1), (144, 66, 1), (272, 130, 2), (2032, 70, 1),
+                                        (1280, 640, 1), (2032, 450, 1), (144, 66, 26)])
 @pytest.mark.parametrize("fmt", ["e4m3", "e5m2", "int8"])
 @pytest.mark.parametrize("gran", ["tensor", "channel"])
 @pytest.mark.parametrize("rounding", ["rtne", "stochastic"])
