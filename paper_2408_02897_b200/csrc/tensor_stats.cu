@@ -197,16 +197,39 @@ struct Batch {
     n[0] += 8u - zeros;
     n_unit += zero_codes - zeros;
   }
-  __device__ __forceinline__ bool error8_fast(const Vec8& v, const QuotientPair& quot, float delta) {
+  // SINGLY: up to two elements too close to the format's largest value for the classes above are taken one at a time and
+  // count as zeros here.  For scales per row, whose largest element otherwise sends its whole warp through the slow
+  // branch too (16000 rows of 1000, INT8: 81 us, 58 so); under one scale they are rare.
+  template <bool SINGLY>
+  __device__ __forceinline__ bool error8_fast(Vec8 v, const QuotientPair& quot, float delta) {
     // half the smallest positive value of the format: what lies above it has a code
     constexpr float kHalfMin = FMT == QM_FMT_INT8 ? 0.5f : (FMT == QM_FMT_E4M3 ? 0x1p-10f : 0x1p-17f);
+    const float top = delta * (0.9999f * fmt_qmax(FMT));
     float mx_x = 0.f, mn_x = 3.4e38f;
 #pragma unroll
     for (int e = 0; e < 8; e += 2) {
       asm("max.f32 %0, %0, %1, %2;" : "+f"(mx_x) : "f"(fabsf(v.v[e])), "f"(fabsf(v.v[e + 1])));
       asm("min.f32 %0, %0, %1, %2;" : "+f"(mn_x) : "f"(fabsf(v.v[e])), "f"(fabsf(v.v[e + 1])));
     }
-    if (!(QuotientPair::serves(delta) && mx_x <= delta * (0.9999f * fmt_qmax(FMT)))) return false;
+    if (!(QuotientPair::serves(delta) && (SINGLY || mx_x <= top))) return false;
+    if (SINGLY && !(mx_x <= top)) {
+      int large = 0;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) large += fabsf(v.v[e]) > top;
+      if (large > 2) return false;
+      const Quotient q(delta);
+      for (; large > 0; --large) {
+        float x = 0.f;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const bool take = x == 0.f && fabsf(v.v[e]) > top;
+          x = take ? v.v[e] : x;
+          v.v[e] = take ? 0.f : v.v[e];
+        }
+        error2(x, 0.f, q(x), 0.f, delta, delta);
+      }
+      mn_x = 0.f;
+    }
     uint64_t ndelta2;
     asm("mov.b64 %0, {%1, %1};" : "=l"(ndelta2) : "f"(-delta));
     if (__any_sync(__activemask(), !(mn_x > delta * (1.0001f * kHalfMin)))) error8<true>(v, quot, ndelta2);
@@ -367,7 +390,8 @@ tensor_stats_dense_kernel(const uint8_t* __restrict__ x, uint64_t n_vec, double*
   finish_pass<kStats>(acc, partials, counter, result, count);
 }
 
-template <typename T, int KIND, int FMT>
+// MODE: delta_mode of the error pass.
+template <typename T, int KIND, int FMT, int MODE>
 __global__ void __launch_bounds__(kThreads, KIND == kError ? 3 : 1)
 tensor_pass_kernel(const Lines p, double* __restrict__ partials, uint32_t* __restrict__ counter,
                    void* __restrict__ result, uint64_t count) {
@@ -388,13 +412,13 @@ tensor_pass_kernel(const Lines p, double* __restrict__ partials, uint32_t* __res
     o = line - b * p.outer;
     return (int64_t)b * p.batch_stride + (int64_t)o * p.line_stride + (int64_t)j * 8;
   };
-  const float delta0 = KIND == kError && p.delta_mode == 0 ? __ldg(p.delta) : 1.f;
+  const float delta0 = KIND == kError && MODE == 0 ? __ldg(p.delta) : 1.f;
   const QuotientPair quot0(delta0);
   auto process = [&](Batch<KIND, FMT>& bt, const Vec8& v, uint32_t b, uint32_t o, uint32_t j, int live) {
     if (KIND == kStats) { bt.stats(v); return; }
-    if (p.delta_mode != 2) {
-      const float d = p.delta_mode == 0 ? delta0 : __ldg(p.delta + (int64_t)b * p.delta_batch + o);
-      if (bt.error8_fast(v, p.delta_mode == 0 ? quot0 : QuotientPair(d), d)) return;
+    if (MODE != 2) {
+      const float d = MODE == 0 ? delta0 : __ldg(p.delta + (int64_t)b * p.delta_batch + o);
+      if (bt.template error8_fast<MODE == 1>(v, MODE == 0 ? quot0 : QuotientPair(d), d)) return;
       const Quotient q(d);
 #pragma unroll
       for (int e = 0; e < 8; e += 2) bt.error2(v.v[e], v.v[e + 1], q(v.v[e]), q(v.v[e + 1]), d, d);
@@ -486,21 +510,21 @@ int pass_blocks(const Lines& p, int resident_per_sm) {
   return (int)(want < 1 ? 1 : (want > cap ? cap : want));
 }
 
-template <typename T, int KIND, int FMT>
+template <typename T, int KIND, int FMT, int MODE>
 qm_status launch_pass(const Lines& p, void* result, uint64_t count, void* ws, cudaStream_t s) {
   static int resident_of[kMaxDevices] = {};      // per instantiation and device
   const int dev = current_device();
   if (dev < 0) return QM_ERR_UNSUPPORTED;
   if (resident_of[dev] == 0) {
     int nb = 0;
-    QM_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tensor_pass_kernel<T, KIND, FMT>, kThreads, 0));
+    QM_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tensor_pass_kernel<T, KIND, FMT, MODE>, kThreads, 0));
     resident_of[dev] = nb > 0 ? nb : 1;
   }
   const int resident = resident_of[dev];
   uint32_t* counter = static_cast<uint32_t*>(ws);
   double* partials = reinterpret_cast<double*>(static_cast<char*>(ws) + kCounterBytes);
   QM_CUDA_OK(cudaMemsetAsync(counter, 0, sizeof(uint32_t), s));
-  QM_CUDA_OK(launch_pdl(tensor_pass_kernel<T, KIND, FMT>, dim3(pass_blocks(p, resident)), dim3(kThreads), 0, s, p,
+  QM_CUDA_OK(launch_pdl(tensor_pass_kernel<T, KIND, FMT, MODE>, dim3(pass_blocks(p, resident)), dim3(kThreads), 0, s, p,
                         partials, counter, result, count));
   count_launch();
   return QM_OK;
@@ -536,8 +560,8 @@ qm_status launch_tensor_stats(const View& x, qm_tensor_stats_result* out, void* 
     count_launch();
     return QM_OK;
   }
-  return x.dtype == QM_DT_BF16 ? launch_pass<__nv_bfloat16, kStats, 0>(p, out, n, ws, s)
-                               : launch_pass<float, kStats, 0>(p, out, n, ws, s);
+  return x.dtype == QM_DT_BF16 ? launch_pass<__nv_bfloat16, kStats, 0, 0>(p, out, n, ws, s)
+                               : launch_pass<float, kStats, 0, 0>(p, out, n, ws, s);
 }
 
 qm_status launch_quantize_error(const View& x, int fmt, int gran, const float* delta, qm_quant_error_result* out,
@@ -546,12 +570,15 @@ qm_status launch_quantize_error(const View& x, int fmt, int gran, const float* d
   qm_status st = make_lines(x, gran == QM_GRAN_CHANNEL, delta, &p);
   if (st != QM_OK) return st;
   const uint64_t n = (uint64_t)(x.nc * x.c * x.batch);
-#define QM_PASS(T)                                                                           \
-  (fmt == QM_FMT_INT8 ? launch_pass<T, kError, QM_FMT_INT8>(p, out, n, ws, s)                 \
-   : fmt == QM_FMT_E4M3 ? launch_pass<T, kError, QM_FMT_E4M3>(p, out, n, ws, s)               \
-                        : launch_pass<T, kError, QM_FMT_E5M2>(p, out, n, ws, s))
+#define QM_MODE(T, F)                                                                             \
+  (p.delta_mode == 0   ? launch_pass<T, kError, F, 0>(p, out, n, ws, s)                           \
+   : p.delta_mode == 1 ? launch_pass<T, kError, F, 1>(p, out, n, ws, s)                           \
+                       : launch_pass<T, kError, F, 2>(p, out, n, ws, s))
+#define QM_PASS(T)                                                                                \
+  (fmt == QM_FMT_INT8 ? QM_MODE(T, QM_FMT_INT8) : fmt == QM_FMT_E4M3 ? QM_MODE(T, QM_FMT_E4M3) : QM_MODE(T, QM_FMT_E5M2))
   return x.dtype == QM_DT_BF16 ? QM_PASS(__nv_bfloat16) : QM_PASS(float);
 #undef QM_PASS
+#undef QM_MODE
 }
 
 }  // namespace qm

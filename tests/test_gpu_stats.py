@@ -139,6 +139,20 @@ def test_error_with_outside_scale_overflows(fmt):
 
 @pytest.mark.parametrize("fmt", FMTS)
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("part", [1.0, 0.98])         # the rows' own scales, and ones that cut the large elements off
+def test_error_with_large_elements_side_by_side(fmt, dtype, part):
+    """None to five of the eight elements a thread takes together at the top of their row's range."""
+    t = tensor((60, 128), dtype, 28, scale=0.1).clamp(-0.5, 0.5)
+    for i in range(60):
+        for j in range(i % 6):
+            t[i, 8 * (i % 16) + (3 * j + i) % 8] = (1.0 if j % 2 else -1.0) * (1.0 - 2.0 ** -20 * j)
+    delta = (oracle.scale(as3(oriented(t, -1)), fmt, "channel") * np.float32(part)).astype(np.float32)
+    got, want = check_error(t, -1, fmt, "channel", delta=delta)
+    assert part == 1.0 or want["n_overflow"] >= 100
+
+
+@pytest.mark.parametrize("fmt", FMTS)
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 def test_error_with_subnormal_elements(fmt, dtype):
     """Non-zero elements below the normal range of float32 (bf16 subnormals are float32 subnormals):
     their code is zero, so each is an underflow with RE exactly 1 and the sums stay finite."""
