@@ -186,7 +186,9 @@ __device__ __forceinline__ uint32_t quant_bf16_pair(uint32_t w, const QuotientPa
 // Four codes of the four bf16 values in two words.
 template <int FMT, bool GUARD = false>
 __device__ __forceinline__ uint32_t quant_bf16_quad(uint32_t w0, uint32_t w1, const QuotientPair& quot) {
-  return __byte_perm(quant_bf16_pair<FMT, GUARD>(w0, quot), quant_bf16_pair<FMT, GUARD>(w1, quot), 0x5410);
+  const uint32_t lo = quant_bf16_pair<FMT, GUARD>(w0, quot), hi = quant_bf16_pair<FMT, GUARD>(w1, quot);
+  // (where the upper halves are zero a permutation measured 1 to 2 % slower: 16384 x 4096 E4M3 rows 48.9 / 48.1 us)
+  return FMT == QM_FMT_INT8 && !GUARD ? __byte_perm(lo, hi, 0x5410) : lo | (hi << 16);
 }
 // Sixteen codes of sixteen consecutive bf16 values (two 128-bit words).
 template <int FMT, bool GUARD = false>
