@@ -33,13 +33,10 @@ sys.path.insert(0, ROOT)
 from paper_2408_02897_b200 import workloads  # noqa: E402
 
 # DRAM bytes (read + write) of the fused probe kernel per byte of distinct operand data it reads
-# (bf16 L and R and both code tensors), from a profiler capture of one launch over the 12 probes of
-# the BERT-large layer workload (2.56 GB moved for 1.485 GB of distinct operand bytes: activations
-# larger than L2 are re-read for part of the column tiles; other captures of the same launch
-# moved 2.38 and 3.00 GB, so the figure varies by a fifth; 1.07 on the BERT-base workload, which
-# fits in L2).  A launch of the default workload has the same projection shapes and is scaled by its
-# distinct operand bytes.  None: the kernel has changed since the counters were taken.
-TC_DRAM_BYTES_PER_OPERAND_BYTE = 1.72
+# (bf16 L and R and the code tensors of all formats), from a profiler capture of a smaller workload with the
+# same projection shapes.  None: the kernel that the default workload runs (products shared by three formats) has not
+# been captured on tensors larger than L2; the line then carries no traffic figure.
+TC_DRAM_BYTES_PER_OPERAND_BYTE = None
 
 
 METRIC = "probe TFLOPS"
@@ -515,13 +512,15 @@ def roofline_of(m, peaks, bench_mhz):
         traffic = TC_DRAM_BYTES_PER_OPERAND_BYTE * distinct_operand_bytes(m["ops"]) * m["repeat"] * m["steps"] / m["tc_launches"]
     r = {"bound": "tensor",
          "kernel": "tc_group_kernel (reference + denominator products once per pair of operands, 8-bit product of every "
-                   "probe, Eq. 3 epilogue; up to 56 probes of 24 pairs per persistent launch)",
+                   "probe, Eq. 3 epilogue; up to 56 probes of 24 pairs per persistent launch); tc_side_kernel where a "
+                   "pair of operands has one probe",
          "executed_flops_per_pass": per_pass, "counted_flops_per_pass": m["flops_pass"],
          "executed_note": "achieved and peak are of the flops the kernel executes; `value` counts 3 x 2MNK per probe, "
                           "the work of the records, of which probes of the same operands share two thirds",
          "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak if achieved else None,
          "traffic": traffic,
-         "traffic_note": "DRAM bytes per launch, scaled from a profiler capture of a smaller workload by distinct operand bytes",
+         "traffic_note": "DRAM bytes per launch, scaled from a profiler capture of a smaller workload by distinct operand bytes"
+                         if traffic is not None else "no capture of this kernel on tensors larger than L2",
          "peak_source": f"{mix:.3f} x {'bf16_tflops_sustained' if long_region else 'bf16_tflops'} ({p16}) of {peaks['source']}",
          "launches": m["tc_launches"], "avg_launch_ms": m["tc_ms"] / max(m["tc_launches"], 1),
          "timing": "CUDA event pair around every launch, recorded by the library on the launching stream inside the timed steps",
