@@ -220,6 +220,31 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t span_bytes
   return d;
 }
 
+// The same without its address, and for tiles stored the other way round: contraction-major tiles as above; mn-major
+// ones, staged from operands whose contraction is strided (a row of `span` bytes, 32, 64 or 128, holds consecutive operand rows at one contraction entry, swizzled over its
+// span) have eight contraction entries per atom, atoms following each other every 8 * span bytes along the contraction and
+// every `next` bytes along the operand's rows.  `step` is what a 32-byte-deep (16 bf16, 32 codes) MMA step adds to the
+// address field.
+struct TileDesc {
+  uint32_t hi, lo, step;
+  __device__ __forceinline__ uint64_t at(uint32_t addr, int k) const {
+    uint64_t d;
+    const uint32_t l = ((addr & 0x3ffffu) >> 4) + lo + step * (uint32_t)k;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(l), "r"(hi));
+    return d;
+  }
+};
+__device__ __forceinline__ TileDesc tile_desc(bool mn_major, uint32_t span, uint32_t entries_per_step, uint32_t next) {
+  TileDesc d;
+  const uint64_t full = smem_desc(0u, span);
+  d.hi = (uint32_t)(full >> 32);
+  d.lo = mn_major ? (next >> 4) << 16 : 1u << 16;
+  d.step = mn_major ? entries_per_step * span / 16u : 2u;
+  return d;
+}
+// bits of the instruction descriptor for operands whose tiles in shared memory are mn-major
+constexpr uint32_t kIdescMnMajorA = 1u << 15, kIdescMnMajorB = 1u << 16;
+
 enum MmaKind { kKindF16 = 0, kKindF8 = 1, kKindI8 = 2 };
 
 // D[256 x N] (+)= A[256 x k] . B[N x k]^T across the CTA pair; called by a converged warp of the
@@ -1030,6 +1055,11 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 // shared memory); half-block stages, an |R| copy by two other warps and prefetching the next
 // block's values ahead of the fences each measured 5 to 20 % slower.
 //
+// Operands whose contraction is strided are staged as they lie in memory (mn-major tiles, a contraction entry per 128-byte
+// row): the tensor cores read R and the codes so at the rate of contraction-major ones, the converters turn L with
+// ldmatrix.  No copy of an operand is made, and under one scale a tensor that is used in both orientations is quantized
+// once, in its own order.  8192 x 4096 x 1024 in three formats, both operands contiguous / strided: 217 / 213 us.
+//
 // Roles in each CTA (512 threads = 4 warpgroups; registers are re-divided with setmaxnreg):
 //   warp 0        TMA producer: blocks of the ring of kStages stages in the order of consumption: per tile
 //                 the k-blocks of L and R (64 entries deep), then per variant those of its codes
@@ -1075,10 +1105,11 @@ struct CfgP {
 struct alignas(16) WalkInfo {
   int32_t tile_begin, per_b, inner, num_kb;         // per_b = tiles_m * tiles_n (tiles per batch element);
                                                     // inner = tiles_n: column tiles run fastest, -tiles_m: row tiles do
-  int32_t half_n, n_var, var_begin, K;
+  int32_t half_n, n_var, var_begin, K;              // half_n: kUnitMnMajor... above its low byte
 };
 struct VarInfo { uint32_t idesc, flags; };
-enum : uint32_t { kVarI8 = 1, kVarScalePerRow = 2, kVarScalePerCol = 4, kVarRowStats = 8 };
+enum : uint32_t { kVarI8 = 1, kVarScalePerRow = 2, kVarScalePerCol = 4, kVarRowStats = 8, kVarMnMajorL = 16, kVarMnMajorR = 32 };
+enum : uint32_t { kUnitMnMajorL = 1, kUnitMnMajorR = 2 };
 
 template <int UNITS, int VARS>
 struct SharedP {
@@ -1113,6 +1144,7 @@ struct GroupUnit {
   int32_t tile_begin;         // position of its first tile in the sequence
   int32_t half_n;             // right-operand rows each CTA stages: 64, or 32 for outputs at most 64 wide
   int32_t m_fastest;          // the tiles of a batch element are walked down the rows first (below)
+  uint32_t major;             // kUnitMnMajor...: bf16 operands stored with the contraction strided
   int32_t var_begin, n_var;
 };
 struct GroupVar {
@@ -1156,11 +1188,12 @@ struct TileWalk {
   int n, total_tiles;
   int r, pair, num_pairs;
   int pi, num_kb, half_n, n_var, var_begin, K;
+  uint32_t major;
   TileCoord tc;
   bool valid;
   __device__ __forceinline__ void start(const WalkInfo* wk_, int n_, int total_tiles_, int pair_, int num_pairs_) {
     wk = wk_; n = n_; total_tiles = total_tiles_;
-    r = -1; pair = pair_; num_pairs = num_pairs_; num_kb = 0; pi = 0; half_n = 0; valid = true;
+    r = -1; pair = pair_; num_pairs = num_pairs_; num_kb = 0; pi = 0; half_n = 0; major = 0; valid = true;
     next_tile();
   }
   // moves to the pair's next tile; valid = false when there is none
@@ -1183,7 +1216,7 @@ struct TileWalk {
       tc.m_tile = w4.z < 0 ? inner_i : outer_i;
       tc.n_tile = w4.z < 0 ? outer_i : inner_i;
       num_kb = w4.w;
-      half_n = x4.x; n_var = x4.y; var_begin = x4.z; K = x4.w;
+      half_n = x4.x & 255; major = (uint32_t)x4.x >> 8; n_var = x4.y; var_begin = x4.z; K = x4.w;
       return;
     }
   }
@@ -1191,6 +1224,7 @@ struct TileWalk {
   __device__ __forceinline__ void make_uniform() {
     num_kb = __shfl_sync(0xffffffffu, num_kb, 0);
     half_n = __shfl_sync(0xffffffffu, half_n, 0);
+    major = __shfl_sync(0xffffffffu, major, 0);
     n_var = __shfl_sync(0xffffffffu, n_var, 0);
     var_begin = __shfl_sync(0xffffffffu, var_begin, 0);
     K = __shfl_sync(0xffffffffu, K, 0);
@@ -1255,6 +1289,34 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
         "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
         "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
       : "memory");
+}
+// 16 lanes x 32 consecutive 32-bit columns: thread t holds words 4 n + t % 4 of row t / 4 in r[2 n] and of row 8 + t / 4 in
+// r[2 n + 1], which is how ldmatrix leaves 8 x 8 matrices.
+__device__ __forceinline__ void tmem_st16x32(uint32_t taddr, const uint32_t* r) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.16x128b.x8.b32 [%0], "
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+      : "memory");
+}
+// Four transposed 8 x 8 matrices of 16-bit values; lane l gives the address of row l % 8 of matrix l / 8.
+__device__ __forceinline__ void ldmatrix4_trans(uint32_t addr, uint32_t* r) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+// A mn-major L tile (64 contraction entries x 128 operand rows, as two 128-byte-swizzled boxes of 64 rows) for the 32 rows of
+// lane quarter q: a[16 h + ...] holds rows 16 h .. 16 h + 15 in the form of tmem_st16x32.  A matrix is 8 entries x 8 rows, its
+// eight 16-byte pieces on different banks by the swizzle.
+__device__ __forceinline__ void load_l_mn_major(uint32_t base, int q, int lane, uint32_t (&a)[32]) {
+  const uint32_t rr = (uint32_t)lane & 7u, mi = (uint32_t)lane >> 3;
+  const uint32_t box = base + (uint32_t)(q >> 1) * 8192u + (8u * (mi >> 1) + rr) * 128u;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t at = box + ((((uint32_t)(q & 1) * 4u + (uint32_t)h * 2u + (mi & 1u)) ^ rr) << 4);
+#pragma unroll
+    for (int n = 0; n < 4; ++n) ldmatrix4_trans(at + (uint32_t)n * 2048u, &a[16 * h + 4 * n]);
+  }
 }
 // 32 lanes x 8 consecutive 32-bit columns.
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
@@ -1345,7 +1407,7 @@ __device__ __forceinline__ void fill_walk(Sh* sh, const Table& tab, int lane) {
     wi.tile_begin = u.tile_begin; wi.per_b = u.tiles_m * u.tiles_n;
     wi.inner = u.m_fastest ? -u.tiles_m : u.tiles_n;
     wi.num_kb = (u.K + kBlockK - 1) / kBlockK;
-    wi.half_n = u.half_n; wi.n_var = u.n_var; wi.var_begin = u.var_begin; wi.K = u.K;
+    wi.half_n = u.half_n | (int32_t)(u.major << 8); wi.n_var = u.n_var; wi.var_begin = u.var_begin; wi.K = u.K;
     sh->walk[i] = wi;
   }
   for (int i = lane; i < tab.n_var; i += 32) sh->var[i] = VarInfo{tab.v[i].idesc_lp, tab.v[i].flags};
@@ -1494,7 +1556,8 @@ tc_group_kernel(const __grid_constant__ Table tab) {
         Ring ring;
         uint32_t g = 0;
         bool ok = true;
-        auto load = [&](const CUtensorMap* maps, uint32_t bytes, int k0, int r0, int c0, int b) {
+        // a mn-major tile has the operand's rows as its inner coordinate; of bf16, 128 of them are two boxes
+        auto load = [&](const CUtensorMap* maps, uint32_t bytes, int k0, int r0, int c0, int b, bool l_mn, bool r_mn, bool two_boxes) {
           // test hook: the consumers' waits run out
           if (g >= tab.stop_after_kb || (g >= (uint32_t)kStages && !w.wait(smem_u32(&sh->empty[ring.s]), ring.parity ^ 1u))) {
             ok = false;
@@ -1502,8 +1565,9 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           }
           const uint32_t bar = smem_u32(&sh->full[ring.s]), base = tile_base + ring.s * C::kStageBytes;
           mbar_expect_tx(bar, bytes);
-          tma_load_3d_local(base + C::kOffR, &maps[1], bar, k0, c0, b);     // the converters read this one
-          tma_load_3d_local(base + C::kOffL, &maps[0], bar, k0, r0, b);
+          tma_load_3d_local(base + C::kOffR, &maps[1], bar, r_mn ? c0 : k0, r_mn ? k0 : c0, b);     // the converters read this one
+          tma_load_3d_local(base + C::kOffL, &maps[0], bar, l_mn ? r0 : k0, l_mn ? k0 : r0, b);
+          if (two_boxes) tma_load_3d_local(base + C::kOffL + kABf16 / 2, &maps[0], bar, r0 + 64, k0, b);
           sh->issued = ++g;
           ring.next();
         };
@@ -1511,10 +1575,15 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           const int r0 = tw.tc.m_tile * kPairM + (int)rank * kBlockM;     // this CTA's left-operand rows
           const int c0 = tw.tc.n_tile * kBlockN + (int)rank * tw.half_n;  // this CTA's half of the right operand
           const uint32_t bytes = kABf16 + (uint32_t)tw.half_n * 128u;
-          for (int kb = 0; kb < tw.num_kb && ok; ++kb) load(tab.u[tw.pi].maps, bytes, kb * kBlockK, r0, c0, tw.tc.b);
+          const bool l_mn = tw.major & kUnitMnMajorL, r_mn = tw.major & kUnitMnMajorR;
+          for (int kb = 0; kb < tw.num_kb && ok; ++kb)
+            load(tab.u[tw.pi].maps, bytes, kb * kBlockK, r0, c0, tw.tc.b, l_mn, r_mn, l_mn);
           const int nb = tw.lp_blocks();
-          for (int f = 0; f < tw.n_var && ok; ++f)
-            for (int kb = 0; kb < nb && ok; ++kb) load(tab.v[tw.var_begin + f].maps, bytes, kb * C::kLpDepth, r0, c0, tw.tc.b);
+          for (int f = 0; f < tw.n_var && ok; ++f) {
+            const uint32_t flags = sh->var[tw.var_begin + f].flags;
+            for (int kb = 0; kb < nb && ok; ++kb)
+              load(tab.v[tw.var_begin + f].maps, bytes, kb * C::kLpDepth, r0, c0, tw.tc.b, flags & kVarMnMajorL, flags & kVarMnMajorR, false);
+          }
         }
       }
     } else if (warp == 1 && rank == 0) {
@@ -1528,25 +1597,26 @@ tc_group_kernel(const __grid_constant__ Table tab) {
         return true;
       };
       // One elected lane issues a block's MMAs and the commit that frees the block in both CTAs.
+      TileDesc rd{};                                 // of R and |R| of the tile in hand
       auto issue_rd = [&](uint32_t base, int kb, uint32_t idesc, uint32_t empty_bar) {
-        const uint64_t dr = smem_desc(base + C::kOffR, 128), da = smem_desc(base + C::kOffRa, 128);
         const uint32_t ta = tmem_base + C::kColL + 64u * (kb & (kTmemStages - 1));
         if (lead) {
 #pragma unroll
           for (int k = 0; k < kBlockK / 16; ++k)   // 16 bf16 = 32 bytes = 2 descriptor units = 8 columns of tensor memory per step
-            mma_pair_a_tmem(tmem_base + C::kColRef, ta + 8u * k, dr + 2 * k, idesc, k ? 1u : (uint32_t)kb, true);
+            mma_pair_a_tmem(tmem_base + C::kColRef, ta + 8u * k, rd.at(base + C::kOffR, k), idesc, k ? 1u : (uint32_t)kb, true);
 #pragma unroll
           for (int k = 0; k < kBlockK / 16; ++k)
-            mma_pair_a_tmem(tmem_base + C::kColDen, ta + 32u + 8u * k, da + 2 * k, idesc, k ? 1u : (uint32_t)kb, true);
+            mma_pair_a_tmem(tmem_base + C::kColDen, ta + 32u + 8u * k, rd.at(base + C::kOffRa, k), idesc, k ? 1u : (uint32_t)kb, true);
           tc_commit_pair(empty_bar, true);
         }
       };
+      TileDesc cl{}, cr{};                           // of the codes of the variant in hand
       auto issue_lp = [&](auto kind, uint32_t base, uint32_t td, int kb, int steps, uint32_t idesc, uint32_t empty_bar) {
-        const uint64_t cl = smem_desc(base + C::kOffL, 128), cr = smem_desc(base + C::kOffR, 128);
         if (lead) {
 #pragma unroll
           for (int k = 0; k < C::kLpDepth / 32; ++k)
-            if (k < steps) mma_pair<decltype(kind)::value>(td, cl + 2 * k, cr + 2 * k, idesc, k ? 1u : (uint32_t)kb, true);
+            if (k < steps)
+              mma_pair<decltype(kind)::value>(td, cl.at(base + C::kOffL, k), cr.at(base + C::kOffR, k), idesc, k ? 1u : (uint32_t)kb, true);
           tc_commit_pair(empty_bar, true);
         }
       };
@@ -1559,7 +1629,9 @@ tc_group_kernel(const __grid_constant__ Table tab) {
         if (it > 0 && !w.wait_warp(smem_u32(&sh->rd_empty), (it - 1) & 1)) break;
         tc_fence_after();
         tw.make_uniform();
-        const uint32_t idesc_ref = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n);
+        const bool r_mn = tw.major & kUnitMnMajorR;          // (A comes from tensor memory, contraction-major always)
+        const uint32_t idesc_ref = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n) | (r_mn ? kIdescMnMajorB : 0u);
+        rd = tile_desc(r_mn, r_mn ? 2u * tw.half_n : 128u, 16u, 16u);
         for (int kb = 0; kb < tw.num_kb; ++kb) {
           ok = wait_block();
           if (!ok) break;
@@ -1572,7 +1644,10 @@ tc_group_kernel(const __grid_constant__ Table tab) {
         for (int f = 0; f < tw.n_var && ok; ++f) {
           const int b = (tw.n_var - 1 - f) & 1;
           const uint32_t idesc = __shfl_sync(0xffffffffu, sh->var[tw.var_begin + f].idesc, 0);
-          const bool is_i8 = __shfl_sync(0xffffffffu, sh->var[tw.var_begin + f].flags, 0) & kVarI8;
+          const uint32_t flags = __shfl_sync(0xffffffffu, sh->var[tw.var_begin + f].flags, 0);
+          const bool is_i8 = flags & kVarI8, cr_mn = flags & kVarMnMajorR;
+          cl = tile_desc(flags & kVarMnMajorL, 128u, 32u, 16u);
+          cr = tile_desc(cr_mn, cr_mn ? tw.half_n : 128u, 32u, 16u);
           // both epilogues have read what this accumulator held; the second one's columns have also
           // been this tile's L, which the denominator MMAs must have finished with
           const uint32_t uses = b ? lp_uses1 : lp_uses0;
@@ -1622,44 +1697,65 @@ tc_group_kernel(const __grid_constant__ Table tab) {
       if (ok && lent) ok = w.wait_warp(smem_u32(&sh->abs_free), abs_uses++ & 1);
       lent = tw.n_var > 1;
       const int r_vec = tw.half_n * 8;                           // 16-byte vectors of the R half-tile that are in use
-      for (int kb = 0; kb < tw.num_kb && ok; ++kb) {
-        const uint32_t s = ring.s;
-        ok = w.wait_warp(smem_u32(&sh->full[s]), ring.parity);
-        if (!ok) break;
-        const uint32_t base = tile_base + s * C::kStageBytes;
-        uint4 v[8], u[4];
-        const uint32_t rsrc = base + C::kOffR + (uint32_t)t * 16u;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) u[j] = t + 128 * j < r_vec ? lds128(rsrc + (uint32_t)j * 2048u) : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = lds128(base + C::kOffL + row_off + (((uint32_t)j ^ sw) << 4));
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (t + 128 * j < r_vec)
-            sts128(rsrc + (C::kOffRa - C::kOffR) + (uint32_t)j * 2048u, make_uint4(u[j].x & m, u[j].y & m, u[j].z & m, u[j].w & m));
-        uint32_t a[32];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) { a[4 * j] = v[j].x; a[4 * j + 1] = v[j].y; a[4 * j + 2] = v[j].z; a[4 * j + 3] = v[j].w; }
-        if (kb >= kTmemStages) {
-          // the tensor-memory columns were last read by the MMAs of the block kTmemStages before this one
-          const uint32_t sp = s >= (uint32_t)kTmemStages ? s - kTmemStages : s + kStages - kTmemStages;
-          const uint32_t pp = s >= (uint32_t)kTmemStages ? ring.parity : ring.parity ^ 1u;
-          ok = w.wait_warp(smem_u32(&sh->empty[sp]), pp);
+      const bool l_mn = tw.major & kUnitMnMajorL;
+      // a loop for each order of L: one loop with the choice inside cost the contraction-major one 7 %
+      auto convert = [&](auto mn) {
+        constexpr bool kMn = decltype(mn)::value;
+        for (int kb = 0; kb < tw.num_kb && ok; ++kb) {
+          const uint32_t s = ring.s;
+          ok = w.wait_warp(smem_u32(&sh->full[s]), ring.parity);
           if (!ok) break;
-        }
-        tc_fence_after();
-        const uint32_t tcol = taddr + 64u * (uint32_t)(kb & (kTmemStages - 1));
-        tmem_st32(tcol, a);
+          const uint32_t base = tile_base + s * C::kStageBytes;
+          uint4 u[4];
+          uint32_t a[32];
+          const uint32_t rsrc = base + C::kOffR + (uint32_t)t * 16u;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) a[j] &= m;
-        tmem_st32(tcol + 32u, a);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // generic-proxy writes -> the tensor core's reads
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(ready_leader + s * 8u);
-        ring.next();
-      }
+          for (int j = 0; j < 4; ++j) u[j] = t + 128 * j < r_vec ? lds128(rsrc + (uint32_t)j * 2048u) : make_uint4(0u, 0u, 0u, 0u);
+          if constexpr (kMn) {
+            load_l_mn_major(base + C::kOffL, q, lane, a);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const uint4 v = lds128(base + C::kOffL + row_off + (((uint32_t)j ^ sw) << 4));
+              a[4 * j] = v.x; a[4 * j + 1] = v.y; a[4 * j + 2] = v.z; a[4 * j + 3] = v.w;
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (t + 128 * j < r_vec)
+              sts128(rsrc + (C::kOffRa - C::kOffR) + (uint32_t)j * 2048u, make_uint4(u[j].x & m, u[j].y & m, u[j].z & m, u[j].w & m));
+          if (kb >= kTmemStages) {
+            // the tensor-memory columns were last read by the MMAs of the block kTmemStages before this one
+            const uint32_t sp = s >= (uint32_t)kTmemStages ? s - kTmemStages : s + kStages - kTmemStages;
+            const uint32_t pp = s >= (uint32_t)kTmemStages ? ring.parity : ring.parity ^ 1u;
+            ok = w.wait_warp(smem_u32(&sh->empty[sp]), pp);
+            if (!ok) break;
+          }
+          tc_fence_after();
+          const uint32_t tcol = taddr + 64u * (uint32_t)(kb & (kTmemStages - 1));
+          if constexpr (kMn) {
+            tmem_st16x32(tcol, a);
+            tmem_st16x32(tcol + (16u << 16), a + 16);
+          } else {
+            tmem_st32(tcol, a);
+          }
+#pragma unroll
+          for (int j = 0; j < 32; ++j) a[j] &= m;
+          if constexpr (kMn) {
+            tmem_st16x32(tcol + 32u, a);
+            tmem_st16x32(tcol + 32u + (16u << 16), a + 16);
+          } else {
+            tmem_st32(tcol + 32u, a);
+          }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // generic-proxy writes -> the tensor core's reads
+          asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(ready_leader + s * 8u);
+          ring.next();
+        }
+      };
+      if (l_mn) convert(std::true_type{}); else convert(std::false_type{});
       // blocks of codes: only passed on
       const int n_code_blocks = tw.n_var * tw.lp_blocks();
       for (int kb = 0; kb < n_code_blocks && ok; ++kb) {
@@ -2052,6 +2148,9 @@ tc_side_kernel(const __grid_constant__ Table tab) {
           const CUtensorMap* const vm = tab.v[tw.pi].maps;
           const int r0 = tw.tc.m_tile * kPairM + (int)rank * kBlockM;     // this CTA's left-operand rows
           const int c0 = tw.tc.n_tile * kBlockN + (int)rank * tw.half_n;  // this CTA's half of the right operand
+          const uint32_t flags = sh->var[tw.pi].flags;
+          const bool l_mn = tw.major & kUnitMnMajorL, r_mn = tw.major & kUnitMnMajorR;
+          const bool cl_mn = flags & kVarMnMajorL, cr_mn = flags & kVarMnMajorR;
           for (int kb = 0; kb < tw.num_kb; ++kb, ++g) {
             const uint32_t s = g % kStages, use = g / kStages;
             // test hook: the consumers' waits run out
@@ -2060,10 +2159,11 @@ tc_side_kernel(const __grid_constant__ Table tab) {
             const uint32_t bar = smem_u32(&sh->full[s]), base = tile_base + s * C::kStageBytes;
             mbar_expect_tx(bar, kABf16 + kALp + (uint32_t)tw.half_n * (kBlockK * 2 + kBlockK));
             const int k0 = kb * kBlockK;
-            tma_load_3d_local(base + C::kOffR, &um[1], bar, k0, c0, tw.tc.b);     // the converters read this one
-            tma_load_3d_local(base + C::kOffL, &um[0], bar, k0, r0, tw.tc.b);
-            tma_load_3d_local(base + C::kOffCl, &vm[0], bar, k0, r0, tw.tc.b);
-            tma_load_3d_local(base + C::kOffCr, &vm[1], bar, k0, c0, tw.tc.b);
+            tma_load_3d_local(base + C::kOffR, &um[1], bar, r_mn ? c0 : k0, r_mn ? k0 : c0, tw.tc.b);     // the converters read this one
+            tma_load_3d_local(base + C::kOffL, &um[0], bar, l_mn ? r0 : k0, l_mn ? k0 : r0, tw.tc.b);
+            if (l_mn) tma_load_3d_local(base + C::kOffL + kABf16 / 2, &um[0], bar, r0 + 64, k0, tw.tc.b);
+            tma_load_3d_local(base + C::kOffCl, &vm[0], bar, cl_mn ? r0 : k0, cl_mn ? k0 : r0, tw.tc.b);
+            tma_load_3d_local(base + C::kOffCr, &vm[1], bar, cr_mn ? c0 : k0, cr_mn ? k0 : c0, tw.tc.b);
             sh->issued = g + 1;
           }
         }
@@ -2071,26 +2171,25 @@ tc_side_kernel(const __grid_constant__ Table tab) {
     } else if (warp == 1 && rank == 0) {
       // ---------------------------------------------------------- MMA issuer (leader CTA, converged warp)
       const bool lead = elect_one();
-      uint32_t idesc_bf16 = 0;                 // of the tile in hand
+      uint32_t idesc_ref = 0, idesc_den = 0;   // of the tile in hand
+      TileDesc ld{}, rd{}, cl{}, cr{};         // L; R and |R|; codes
       auto issue_ref_den = [&](uint32_t gg, int kb) {
         const uint32_t s = gg % kStages, base = tile_base + s * C::kStageBytes;
-        const uint64_t dl = smem_desc(base + C::kOffL, 128), dr = smem_desc(base + C::kOffR, 128);
 #pragma unroll
-        for (int k = 0; k < kBlockK / 16; ++k)   // 16 bf16 = 32 bytes = 2 descriptor units per step
-          mma_pair<kKindF16>(tmem_base + C::kColRef, dl + 2 * k, dr + 2 * k, idesc_bf16, (kb | k) != 0, lead);
-        const uint64_t da = smem_desc(base + C::kOffRa, 128);
+        for (int k = 0; k < kBlockK / 16; ++k)   // 16 bf16 per step
+          mma_pair<kKindF16>(tmem_base + C::kColRef, ld.at(base + C::kOffL, k), rd.at(base + C::kOffR, k), idesc_ref, (kb | k) != 0, lead);
         const uint32_t ta = tmem_base + C::kColAbsL + 32u * (gg % kAbs);
 #pragma unroll
         for (int k = 0; k < kBlockK / 16; ++k)   // 16 bf16 = 8 columns of tensor memory per step
-          mma_pair_a_tmem(tmem_base + C::kColDen, ta + 8u * k, da + 2 * k, idesc_bf16, (kb | k) != 0, lead);
+          mma_pair_a_tmem(tmem_base + C::kColDen, ta + 8u * k, rd.at(base + C::kOffRa, k), idesc_den, (kb | k) != 0, lead);
       };
       auto issue_lp = [&](uint32_t gg, int kb, bool is_i8, uint32_t idesc_lp) {
         const uint32_t base = tile_base + (gg % kStages) * C::kStageBytes;
-        const uint64_t cl = smem_desc(base + C::kOffCl, 64), cr = smem_desc(base + C::kOffCr, 64);
 #pragma unroll
-        for (int k = 0; k < kBlockK / 32; ++k) {  // 32 codes = 32 bytes per step
-          if (is_i8) mma_pair<kKindI8>(tmem_base + C::kColLp, cl + 2 * k, cr + 2 * k, idesc_lp, (kb | k) != 0, lead);
-          else mma_pair<kKindF8>(tmem_base + C::kColLp, cl + 2 * k, cr + 2 * k, idesc_lp, (kb | k) != 0, lead);
+        for (int k = 0; k < kBlockK / 32; ++k) {  // 32 codes per step
+          const uint64_t a = cl.at(base + C::kOffCl, k), b = cr.at(base + C::kOffCr, k);
+          if (is_i8) mma_pair<kKindI8>(tmem_base + C::kColLp, a, b, idesc_lp, (kb | k) != 0, lead);
+          else mma_pair<kKindF8>(tmem_base + C::kColLp, a, b, idesc_lp, (kb | k) != 0, lead);
         }
       };
       auto wait_stage = [&](uint32_t gg) {
@@ -2106,8 +2205,16 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         tw.make_uniform();
         const int num_kb = tw.num_kb;
         const uint32_t idesc_lp = __shfl_sync(0xffffffffu, sh->var[tw.pi].idesc, 0);
-        const bool is_i8 = __shfl_sync(0xffffffffu, sh->var[tw.pi].flags, 0) & kVarI8;
-        idesc_bf16 = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n);
+        const uint32_t flags = __shfl_sync(0xffffffffu, sh->var[tw.pi].flags, 0);
+        const bool is_i8 = flags & kVarI8, cr_mn = flags & kVarMnMajorR;
+        const bool l_mn = tw.major & kUnitMnMajorL, r_mn = tw.major & kUnitMnMajorR;
+        // |L| comes from tensor memory, contraction-major always
+        idesc_den = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n) | (r_mn ? kIdescMnMajorB : 0u);
+        idesc_ref = idesc_den | (l_mn ? kIdescMnMajorA : 0u);
+        ld = tile_desc(l_mn, 128u, 16u, kABf16 / 2);
+        rd = tile_desc(r_mn, r_mn ? 2u * tw.half_n : 128u, 16u, 16u);
+        cl = tile_desc(flags & kVarMnMajorL, flags & kVarMnMajorL ? 128u : 64u, 32u, 16u);
+        cr = tile_desc(cr_mn, cr_mn ? tw.half_n : 64u, 32u, 16u);
         // the reference and denominator blocks come back when both epilogues have copied the
         // previous tile's values out; the 8-bit block when they have finished that tile
         if (it > 0 && !w.wait_warp(smem_u32(&sh->tmem_empty), (it - 1) & 1)) break;
@@ -2149,41 +2256,57 @@ tc_side_kernel(const __grid_constant__ Table tab) {
     TileWalk tw;
     tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
     bool ok = true;
-    int kb = 0;
-    for (uint32_t g = 0; ok && tw.valid; ++g) {
-      const uint32_t s = g % kStages, sa = g % kAbs, m = 0x7fff7fffu;
-      // the tensor-memory columns were last read by the MMAs of k-block g - kAbs (its commit also
-      // covers every earlier k-block, so the |R| slot of the stage is free as well)
-      if (g >= (uint32_t)kAbs) {
-        const uint32_t gp = g - kAbs;
-        if (!w.wait_warp(smem_u32(&sh->empty[gp % kStages]), (gp / kStages) & 1)) { ok = false; break; }
+    uint32_t g = 0;
+    // the blocks of one tile; a loop for each order of L: one loop with the choice inside cost the contraction-major one 7 %
+    auto convert = [&](auto mn) {
+      constexpr bool kMn = decltype(mn)::value;
+      for (int kb = 0; kb < tw.num_kb; ++kb, ++g) {
+        const uint32_t s = g % kStages, sa = g % kAbs, m = 0x7fff7fffu;
+        // the tensor-memory columns were last read by the MMAs of k-block g - kAbs (its commit also
+        // covers every earlier k-block, so the |R| slot of the stage is free as well)
+        if (g >= (uint32_t)kAbs) {
+          const uint32_t gp = g - kAbs;
+          if (!w.wait_warp(smem_u32(&sh->empty[gp % kStages]), (gp / kStages) & 1)) { ok = false; return; }
+        }
+        if (!w.wait_warp(smem_u32(&sh->full[s]), (g / kStages) & 1)) { ok = false; return; }
+        tc_fence_after();
+        const uint32_t base = tile_base + s * C::kStageBytes;
+        uint4 u[4];
+        uint32_t a[32];
+        if constexpr (kMn) {
+          load_l_mn_major(base + C::kOffL, q, lane, a);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const uint4 v = lds128(base + C::kOffL + row_off + (((uint32_t)j ^ sw) << 4));
+            a[4 * j] = v.x; a[4 * j + 1] = v.y; a[4 * j + 2] = v.z; a[4 * j + 3] = v.w;
+          }
+        }
+        const uint32_t rsrc = base + C::kOffR + (uint32_t)t * 16u;
+        const int r_vec = tw.half_n * 8;                           // 16-byte vectors of the R half-tile that are in use
+#pragma unroll
+        for (int j = 0; j < 4; ++j) u[j] = t + 128 * j < r_vec ? lds128(rsrc + (uint32_t)j * 2048u) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) a[j] &= m;
+        if constexpr (kMn) {
+          tmem_st16x32(taddr + 32u * sa, a);
+          tmem_st16x32(taddr + 32u * sa + (16u << 16), a + 16);
+        } else {
+          tmem_st32(taddr + 32u * sa, a);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (t + 128 * j < r_vec)
+            sts128(rsrc + (C::kOffRa - C::kOffR) + (uint32_t)j * 2048u, make_uint4(u[j].x & m, u[j].y & m, u[j].z & m, u[j].w & m));
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // generic-proxy writes -> the tensor core's reads
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(ready_leader + sa * 8u);
       }
-      if (!w.wait_warp(smem_u32(&sh->full[s]), (g / kStages) & 1)) { ok = false; break; }
-      tc_fence_after();
-      const uint32_t base = tile_base + s * C::kStageBytes;
-      uint4 v[8], u[4];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = lds128(base + C::kOffL + row_off + (((uint32_t)j ^ sw) << 4));
-      const uint32_t rsrc = base + C::kOffR + (uint32_t)t * 16u;
-      const int r_vec = tw.half_n * 8;                           // 16-byte vectors of the R half-tile that are in use
-#pragma unroll
-      for (int j = 0; j < 4; ++j) u[j] = t + 128 * j < r_vec ? lds128(rsrc + (uint32_t)j * 2048u) : make_uint4(0u, 0u, 0u, 0u);
-      uint32_t a[32];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        a[4 * j] = v[j].x & m; a[4 * j + 1] = v[j].y & m; a[4 * j + 2] = v[j].z & m; a[4 * j + 3] = v[j].w & m;
-      }
-      tmem_st32(taddr + 32u * sa, a);
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (t + 128 * j < r_vec)
-          sts128(rsrc + (C::kOffRa - C::kOffR) + (uint32_t)j * 2048u, make_uint4(u[j].x & m, u[j].y & m, u[j].z & m, u[j].w & m));
-      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // generic-proxy writes -> the tensor core's reads
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(ready_leader + sa * 8u);
-      if (++kb >= tw.num_kb) { kb = 0; tw.next_tile(); }
+    };
+    for (; ok && tw.valid; tw.next_tile()) {
+      if (tw.major & kUnitMnMajorL) convert(std::true_type{}); else convert(std::false_type{});
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
@@ -2381,6 +2504,25 @@ bool make_map(CUtensorMap* m, const void* base, bool bf16, int box_rows, int64_t
   return r == CUDA_SUCCESS;
 }
 
+// The same over [batch][K][rows] with the operand's rows contiguous (contraction strided): box = box_rows x depth x 1, whose
+// rows of box_rows elements are one swizzle span (32, 64 or 128 bytes).
+bool make_map_mn(CUtensorMap* m, const void* base, bool bf16, int box_rows, int depth, int64_t K, int64_t rows, int64_t batch,
+                   int64_t ld_elems, int64_t sb_elems) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  const uint64_t es = bf16 ? 2 : 1;
+  cuuint64_t dims[3] = {(cuuint64_t)rows, (cuuint64_t)K, (cuuint64_t)batch};
+  cuuint64_t strides[2] = {(cuuint64_t)ld_elems * es, batch > 1 ? (cuuint64_t)sb_elems * es : (cuuint64_t)K * ld_elems * es};
+  cuuint32_t box[3] = {(cuuint32_t)box_rows, (cuuint32_t)depth, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  const uint64_t span = box_rows * es;
+  CUresult r = fn(m, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8, 3,
+                  const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  span == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : span == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS;
+}
+
 uint32_t lp_idesc(int fmt_l, int fmt_r, int n = kBlockN) {
   if (fmt_l == QM_FMT_INT8) return make_idesc(2, 1, 1, kPairM, n);                 // s8 x s8 -> s32
   const uint32_t fa = fmt_l == QM_FMT_E4M3 ? 0u : 1u, fb = fmt_r == QM_FMT_E4M3 ? 0u : 1u;
@@ -2569,7 +2711,7 @@ struct UnitPlan {
 
 bool same_products(const TcProbeArgs& a, const TcProbeArgs& b) {
   return a.l == b.l && a.l_ld == b.l_ld && a.l_sb == b.l_sb && a.r == b.r && a.r_ld == b.r_ld && a.r_sb == b.r_sb &&
-         a.g.M == b.g.M && a.g.N == b.g.N && a.g.K == b.g.K && a.g.batch == b.g.batch;
+         a.l_mn == b.l_mn && a.r_mn == b.r_mn && a.g.M == b.g.M && a.g.N == b.g.N && a.g.K == b.g.K && a.g.batch == b.g.batch;
 }
 
 template <bool SIDE, typename Table>
@@ -2589,14 +2731,17 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, cuda
     const UnitPlan& up = units[k];
     const GemmShape g = up.g;
     const TcProbeArgs& p0 = ps[up.probe[0]];
-    const int64_t ldc = qm_code_ld(g.K);
     GroupUnit& gu = tab.u[k];
     // outputs at most 64 wide (the context and score-gradient products of attention): MMAs of N = 64,
     // half as many right-operand rows staged
     const int half_n = g.N <= 64 ? 32 : kHalfN;
-    if (!make_map(&gu.maps[0], p0.l, true, kBlockM, g.K, g.M, g.batch, p0.l_ld, p0.l_sb) ||
-        !make_map(&gu.maps[1], p0.r, true, half_n, g.K, g.N, g.batch, p0.r_ld, p0.r_sb))
-      return QM_ERR_CUDA;
+    // an operand with the contraction strided is staged as it lies in memory: mn-major tiles
+    const bool have = (p0.l_mn ? make_map_mn(&gu.maps[0], p0.l, true, 64, kBlockK, g.K, g.M, g.batch, p0.l_ld, p0.l_sb)
+                                 : make_map(&gu.maps[0], p0.l, true, kBlockM, g.K, g.M, g.batch, p0.l_ld, p0.l_sb)) &&
+                      (p0.r_mn ? make_map_mn(&gu.maps[1], p0.r, true, half_n, kBlockK, g.K, g.N, g.batch, p0.r_ld, p0.r_sb)
+                                 : make_map(&gu.maps[1], p0.r, true, half_n, g.K, g.N, g.batch, p0.r_ld, p0.r_sb));
+    if (!have) return QM_ERR_CUDA;
+    gu.major = (p0.l_mn ? kUnitMnMajorL : 0u) | (p0.r_mn ? kUnitMnMajorR : 0u);
     KernelArgs ka{};
     fill_tiles(&ka, g);
     gu.M = (int32_t)g.M; gu.N = (int32_t)g.N; gu.K = (int32_t)g.K;
@@ -2613,16 +2758,21 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, cuda
       const TcProbeArgs& p = ps[up.probe[j]];
       GroupVar& v = tab.v[tab.n_var++];
       // blocks of codes are 64 entries deep beside the bf16 tiles, 128 on their own
-      if (!make_map(&v.maps[0], p.cl, false, kBlockM, g.K, g.M, g.batch, ldc, g.M * ldc, !SIDE) ||
-          !make_map(&v.maps[1], p.cr, false, half_n, g.K, g.N, g.batch, ldc, g.N * ldc, !SIDE))
-        return QM_ERR_CUDA;
+      const int depth = SIDE ? kBlockK : CfgP::kLpDepth;
+      auto code_map = [&](CUtensorMap* m, const uint8_t* codes, bool mn, int box_rows, int64_t rows) {
+        const int64_t ld = qm_code_ld(mn ? rows : g.K);
+        return mn ? make_map_mn(m, codes, false, box_rows, depth, g.K, rows, g.batch, ld, g.K * ld)
+                           : make_map(m, codes, false, box_rows, g.K, rows, g.batch, ld, rows * ld, !SIDE);
+      };
+      if (!code_map(&v.maps[0], p.cl, p.cl_mn, kBlockM, g.M) || !code_map(&v.maps[1], p.cr, p.cr_mn, half_n, g.N)) return QM_ERR_CUDA;
       v.dl = p.dl; v.dr = p.dr;
       v.partials = p.partials; v.result = p.result; v.row_stats = p.row_stats;
       v.err_word = p.err_word; v.err_also[0] = p.err_also[0]; v.err_also[1] = p.err_also[1];
       v.count = (uint64_t)(g.M * g.N * g.batch);
       v.flags = (p.fmt_l == QM_FMT_INT8 ? kVarI8 : 0u) | (p.gran_l == QM_GRAN_CHANNEL ? kVarScalePerRow : 0u) |
-                (p.gran_r == QM_GRAN_CHANNEL ? kVarScalePerCol : 0u) | (p.row_stats ? kVarRowStats : 0u);
-      v.idesc_lp = lp_idesc(p.fmt_l, p.fmt_r, 2 * half_n);
+                (p.gran_r == QM_GRAN_CHANNEL ? kVarScalePerCol : 0u) | (p.row_stats ? kVarRowStats : 0u) |
+                (p.cl_mn ? kVarMnMajorL : 0u) | (p.cr_mn ? kVarMnMajorR : 0u);
+      v.idesc_lp = lp_idesc(p.fmt_l, p.fmt_r, 2 * half_n) | (p.cl_mn ? kIdescMnMajorA : 0u) | (p.cr_mn ? kIdescMnMajorB : 0u);
     }
   }
   tab.total_tiles = (int32_t)total;

@@ -1,5 +1,6 @@
 // The C ABI: argument checks, workspace layout and launch sequencing.  All arithmetic of the
 // probe runs in the kernels of the other translation units.
+#include <algorithm>
 #include <atomic>
 #include <cstdio>
 #include <cstdlib>
@@ -105,6 +106,24 @@ int64_t delta_count(const View& v, int gran) { return gran == QM_GRAN_TENSOR ? 1
 
 size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
 
+// The tensor-core products take an operand whose contraction is strided as it lies in memory, and its codes too
+// where they are rounded to nearest: written in the operand's own order, by passes that move whole lines, no
+// transposition and no bf16 copy (the transposing quantize kernels moved 7 bytes an element and the copy is read again:
+// 16384 x 4096 in three formats 106 us so, 61 in order).  Under one scale such codes are those of the flipped
+// view, so a tensor that is used in both orientations is quantized once.  Stochastic rounding numbers its draws along the
+// contraction: those codes stay contraction-major.
+bool codes_mn(const View& v, bool stochastic) { return !v.c_contig() && !stochastic; }
+View flipped(const View& v) {
+  View f = v;
+  f.nc = v.c; f.c = v.nc; f.s_nc = v.s_c; f.s_c = v.s_nc;
+  return f;
+}
+// either order of the codes: a workspace may be asked for without naming the rounding
+size_t code_bytes(const View& v, bool tc) {
+  const int64_t along = v.batch * v.nc * qm_code_ld(v.c), in_order = v.batch * v.c * qm_code_ld(v.nc);
+  return (size_t)(tc && !v.c_contig() && in_order > along ? in_order : along);
+}
+
 struct Workspace {
   size_t off_err, off_ml, off_mr, off_dl, off_dr, off_cl, off_cr, off_al, off_ar, off_kl, off_kr, off_part, off_pl, off_pr, total;
   int n_part;
@@ -122,14 +141,15 @@ Workspace plan(const View& L, const View& R, const qm_probe_cfg& cfg, bool with_
   w.off_mr = take(sizeof(float) * delta_count(R, cfg.gran_r));
   w.off_dl = take(sizeof(float) * delta_count(L, cfg.gran_l));
   w.off_dr = take(sizeof(float) * delta_count(R, cfg.gran_r));
-  const int64_t ldc = qm_code_ld(L.c);
-  w.off_cl = take((size_t)(L.batch * L.nc * ldc));
-  w.off_cr = take((size_t)(R.batch * R.nc * ldc));
+  w.off_cl = take(code_bytes(L, w.tc));
+  w.off_cr = take(code_bytes(R, w.tc));
   if (w.tc) {
     if (with_abs) {
       w.off_al = take((size_t)(L.batch * L.nc * L.c) * 2);
       w.off_ar = take((size_t)(R.batch * R.nc * R.c) * 2);
     }
+    // two bytes an element of an operand whose contraction is strided: contraction-major copies of the two-format kernel,
+    // codes of further probes of a batch (Slot::room)
     w.off_kl = L.c_contig() ? 0 : take((size_t)(L.batch * L.nc * L.c) * 2);
     w.off_kr = R.c_contig() ? 0 : take((size_t)(R.batch * R.nc * R.c) * 2);
   }
@@ -169,13 +189,12 @@ qm_status check_probe(const qm_operand* Lo, const qm_operand* Ro, const qm_probe
   return QM_OK;
 }
 
-// scale + quantize of one operand inside the probe
-qm_status prepare_operand(const View& x, int fmt, int gran, uint32_t* amax, float* delta, uint8_t* codes,
-                          void* abs_copy, void* kmaj_copy, uint32_t* err_word, const StochasticDraw* draw,
-                          int batch_groups, cudaStream_t s) {
+// scale + quantize of one operand inside the probe; mn: codes in the operand's own order (codes_mn)
+qm_status prepare_operand(const View& x, int fmt, int gran, bool mn, uint32_t* amax, float* delta, uint8_t* codes,
+                          uint32_t* err_word, const StochasticDraw* draw, int batch_groups, cudaStream_t s) {
   const bool shared = gran == QM_GRAN_CHANNEL && batch_groups > 0 && batch_groups < x.batch;
   if (!draw && !shared && gran == QM_GRAN_CHANNEL && x.c_contig())
-    return launch_scale_quantize_rows(x, fmt, delta, codes, abs_copy, err_word, s);
+    return launch_scale_quantize_rows(x, fmt, delta, codes, nullptr, err_word, s);
   qm_status st = launch_absmax(x, gran, amax, s);
   if (st != QM_OK) return st;
   if (shared) {
@@ -183,8 +202,15 @@ qm_status prepare_operand(const View& x, int fmt, int gran, uint32_t* amax, floa
     if (st != QM_OK) return st;
   }
   // the quantize kernel turns max|x| into delta itself
-  return launch_quantize(x, fmt, gran, reinterpret_cast<const float*>(amax), true, delta, err_word, codes,
-                         abs_copy, kmaj_copy, s, draw);
+  if (mn && gran == QM_GRAN_CHANNEL) return launch_quantize_cols(x, amax, 1, &fmt, &delta, &err_word, &codes, s);
+  return launch_quantize(mn ? flipped(x) : x, fmt, gran, reinterpret_cast<const float*>(amax), true, delta, err_word, codes,
+                         nullptr, nullptr, s, draw);
+}
+
+// the bf16 operands of a one-format probe, as they lie
+void set_operands(TcProbeArgs* p, const View& L, const View& R) {
+  p->l = L.data; p->l_mn = !L.c_contig(); p->l_ld = p->l_mn ? L.s_c : L.s_nc; p->l_sb = L.s_b;
+  p->r = R.data; p->r_mn = !R.c_contig(); p->r_ld = p->r_mn ? R.s_c : R.s_nc; p->r_sb = R.s_b;
 }
 
 }  // namespace
@@ -367,8 +393,7 @@ static qm_status probe_phases(const qm_operand* Lo, const qm_operand* Ro, const 
   const StochasticDraw draw_l{cfg->seed, 0u}, draw_r{cfg->seed, 1u};
   const StochasticDraw* dl_draw = (cfg->round & QM_ROUND_STOCHASTIC_L) ? &draw_l : nullptr;
   const StochasticDraw* dr_draw = (cfg->round & QM_ROUND_STOCHASTIC_R) ? &draw_r : nullptr;
-  void* kl = (w.tc && !L.c_contig()) ? base + w.off_kl : nullptr;
-  void* kr = (w.tc && !R.c_contig()) ? base + w.off_kr : nullptr;
+  const bool cl_mn = w.tc && codes_mn(L, dl_draw != nullptr), cr_mn = w.tc && codes_mn(R, dr_draw != nullptr);
   // operands of modest size: both in two launches, the first of which clears the control words
   auto grouped = [](const View& v, int gran, int groups) { return gran == QM_GRAN_CHANNEL && groups > 0 && groups < v.batch; };
   const bool pair = (phases & kPrepare) == kPrepare && !clear_later && !grouped(L, cfg->gran_l, cfg->batch_groups_l) &&
@@ -377,8 +402,8 @@ static qm_status probe_phases(const qm_operand* Lo, const qm_operand* Ro, const 
   // the error word, the finished-CTA counter and both max|x| buffers are adjacent: one clear
   if (pair) {
     const PairSide side[2] = {
-        {L, cfg->fmt_l, cfg->gran_l, dl_draw, reinterpret_cast<uint32_t*>(base + w.off_pl), dl, cl, kl},
-        {R, cfg->fmt_r, cfg->gran_r, dr_draw, reinterpret_cast<uint32_t*>(base + w.off_pr), dr, cr, kr}};
+        {L, cfg->fmt_l, cfg->gran_l, cl_mn, dl_draw, reinterpret_cast<uint32_t*>(base + w.off_pl), dl, cl},
+        {R, cfg->fmt_r, cfg->gran_r, cr_mn, dr_draw, reinterpret_cast<uint32_t*>(base + w.off_pr), dr, cr}};
     st = launch_pair_prepare(side, err, 64, s);
     if (st != QM_OK) return st;
   } else if ((phases & kClear) && clear_later && clear_later->n < kClearMax) {
@@ -391,24 +416,20 @@ static qm_status probe_phases(const qm_operand* Lo, const qm_operand* Ro, const 
     QM_CUDA_OK(cudaMemsetAsync(cfg->row_stats, 0, sizeof(double) * QM_ROW_STATS * (size_t)(L.batch * L.nc), s));
   uint32_t* ml = reinterpret_cast<uint32_t*>(base + w.off_ml);
   uint32_t* mr = reinterpret_cast<uint32_t*>(base + w.off_mr);
-  // the fused kernel forms |L| and |R| on chip: no |x| copy is written
-  void* al = nullptr;
-  void* ar = nullptr;
   if ((phases & kPrepareL) && !pair) {
-    st = prepare_operand(L, cfg->fmt_l, cfg->gran_l, ml, dl, cl, al, kl, err, dl_draw, cfg->batch_groups_l, s);
+    st = prepare_operand(L, cfg->fmt_l, cfg->gran_l, cl_mn, ml, dl, cl, err, dl_draw, cfg->batch_groups_l, s);
     if (st != QM_OK) return st;
   }
   if ((phases & kPrepareR) && !pair) {
-    st = prepare_operand(R, cfg->fmt_r, cfg->gran_r, mr, dr, cr, ar, kr, err, dr_draw, cfg->batch_groups_r, s);
+    st = prepare_operand(R, cfg->fmt_r, cfg->gran_r, cr_mn, mr, dr, cr, err, dr_draw, cfg->batch_groups_r, s);
     if (st != QM_OK) return st;
   }
   if (!(phases & kProducts)) return QM_OK;
   GemmShape g{L.nc, R.nc, L.c, L.batch};
   if (w.tc) {
-    TcProbeArgs p{};
-    p.l = kl ? kl : L.data; p.l_ld = kl ? L.c : L.s_nc; p.l_sb = kl ? L.nc * L.c : L.s_b;
-    p.r = kr ? kr : R.data; p.r_ld = kr ? R.c : R.s_nc; p.r_sb = kr ? R.nc * R.c : R.s_b;
-    p.l_abs = al; p.r_abs = ar; p.cl = cl; p.cr = cr;
+    TcProbeArgs p{};                        // (the fused kernel forms |L| and |R| on chip)
+    set_operands(&p, L, R);
+    p.cl = cl; p.cr = cr; p.cl_mn = cl_mn; p.cr_mn = cr_mn;
     p.fmt_l = cfg->fmt_l; p.fmt_r = cfg->fmt_r;
     p.dl = dl; p.gran_l = cfg->gran_l; p.dr = dr; p.gran_r = cfg->gran_r;
     p.g = g; p.partials = part; p.err_word = err;
@@ -658,26 +679,30 @@ qm_status batch_streams(BatchStreams** out) {
 }
 
 // One operand of one tensor-core probe of a batch: what has to be prepared, where this probe's own
-// buffers for it are, and whose results it uses.  Preparing an operand leaves four things behind:
-// the max|x| bit patterns, the contraction-major bf16 copy (strided contraction only), the
-// scales and the codes.  A sweep of formats over a layer, and a layer whose activations feed
-// several products, ask for the same things many times over; inside a batch each is made once:
+// buffers for it are, and whose results it uses.  Preparing an operand leaves three things behind:
+// the max|x| bit patterns, the scales and the codes.  A sweep of formats over a layer, and a layer whose activations feed
+// several products, ask for the same things many times over; inside a batch each is made once.  (An operand whose codes
+// stay in its own order under one scale is described by its flipped view, so the two orientations of a tensor are one view.)
 //   code_root: the earlier operand with the same view, scale grouping, format and rounding: its
-//              scales, codes and copy are used as they are and nothing is launched;
+//              scales and codes are used as they are and nothing is launched;
 //   pass_root: the earlier operand with the same view and scale grouping under another format:
 //              its max|x| is borrowed, and its pass over the tensor makes this one's codes too where it can;
 //   amax_root: per-tensor scales only: the earlier operand over the same elements in either
 //              orientation (max|x| does not depend on which dimension contracts);
-//   kmaj_root: the first operand with the same view, whatever its scales: its contraction-major copy is used.
+//   home:      the first operand of the same view whose codes stay in its own order: where its workspace has room (two
+//              bytes an element), the codes of further formats and scales go there, beside its own, and the
+//              workspaces of the other probes stay untouched.
 // A root index equal to the slot's own index means "makes it itself".
 struct Slot {
   View v;
   int fmt, gran, groups;
   bool stochastic;
   StochasticDraw draw;
-  uint32_t* amax; float* delta; uint8_t* codes; void* kmaj; uint32_t* err;
+  uint32_t* amax; float* delta; uint8_t* codes; uint32_t* err;
+  bool mn;                         // codes in the operand's own order
+  uint8_t* room; size_t room_left; // for the codes of further slots of the same view
   bool keeps_amax;                 // false when the single-pass per-row kernel prepares it (no maxima are stored)
-  int code_root, pass_root, amax_root, kmaj_root;
+  int code_root, pass_root, amax_root, home;
   int stream;                      // index of the library stream its kernels go to
 };
 
@@ -694,9 +719,7 @@ bool grouped_scales(const Slot& x) { return x.gran == QM_GRAN_CHANNEL && x.group
 
 void find_roots(std::vector<Slot>& slots, int t) {
   Slot& x = slots[t];
-  x.code_root = x.pass_root = x.amax_root = x.kmaj_root = t;
-  for (int u = 0; u < t && x.kmaj_root == t; ++u)
-    if (same_view(x.v, slots[u].v)) x.kmaj_root = u;        // the first of its view: makes everything itself
+  x.code_root = x.pass_root = x.amax_root = t;
   const int gx = grouped_scales(x) ? x.groups : 0;
   for (int u = 0; u < t; ++u) {
     const Slot& y = slots[u];
@@ -718,6 +741,27 @@ void find_roots(std::vector<Slot>& slots, int t) {
     const Slot& y = slots[u];
     if (y.code_root != u || y.pass_root != u || y.amax_root != u || y.gran != QM_GRAN_TENSOR) continue;
     if (same_view(x.v, y.v) || transposed_view(x.v, y.v)) { x.amax_root = u; return; }
+  }
+}
+
+// A slot that makes its codes itself, in its operand's own order, puts them beside those of the first such slot of
+// the same elements if there is room.
+void find_home(std::vector<Slot>& slots, int t) {
+  Slot& x = slots[t];
+  x.home = t;
+  if (!x.mn || x.code_root != t) return;
+  for (int u = 0; u < t; ++u) {
+    Slot& y = slots[u];
+    if (!y.mn || y.home != u || y.code_root != u || !(same_view(x.v, y.v) || transposed_view(x.v, y.v))) continue;
+    const int64_t rows = x.v.c_contig() ? x.v.nc : x.v.c, cols = x.v.c_contig() ? x.v.c : x.v.nc;     // as the codes lie
+    const size_t bytes = (size_t)(x.v.batch * rows * qm_code_ld(cols));
+    if (bytes <= y.room_left) {
+      x.codes = y.room;
+      x.home = u;
+      y.room += align256(bytes);
+      y.room_left -= std::min(y.room_left, align256(bytes));
+    }
+    return;
   }
 }
 
@@ -780,12 +824,18 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
       x.amax = reinterpret_cast<uint32_t*>(base + (side ? pl.w.off_mr : pl.w.off_ml));
       x.delta = reinterpret_cast<float*>(base + (side ? pl.w.off_dr : pl.w.off_dl));
       x.codes = base + (side ? pl.w.off_cr : pl.w.off_cl);
-      x.kmaj = v.c_contig() ? nullptr : base + (side ? pl.w.off_kr : pl.w.off_kl);
       // words 2 and 3 of the control block: "this operand is not finite", raised by the kernel that scales it
       x.err = reinterpret_cast<uint32_t*>(base + pl.w.off_err) + 2 + side;
       x.keeps_amax = !(!x.stochastic && !grouped_scales(x) && x.gran == QM_GRAN_CHANNEL && v.c_contig());
+      x.mn = codes_mn(v, x.stochastic);
+      if (x.mn) {
+        x.room = base + (side ? pl.w.off_kr : pl.w.off_kl);
+        x.room_left = (size_t)(v.batch * v.nc * v.c) * 2;
+        if (x.gran == QM_GRAN_TENSOR) x.v = flipped(v);
+      }
       slots.push_back(x);
       find_roots(slots, (int)slots.size() - 1);
+      find_home(slots, (int)slots.size() - 1);
     }
   }
   if (clears.n > 0) {
@@ -810,11 +860,13 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
     if (x.pass_root != (int)t) {
       // borrows max|x|, and was not served with its lender's formats
       x.stream = slots[x.pass_root].stream;
-      e = launch_quantize(x.v, x.fmt, x.gran, reinterpret_cast<const float*>(slots[x.amax_root].amax), true, x.delta, x.err,
-                          x.codes, nullptr, nullptr, b->s[x.stream], draw);
+      const uint32_t* amax = slots[x.amax_root].amax;
+      if (codes_mn(x.v, x.stochastic)) e = launch_quantize_cols(x.v, amax, 1, &x.fmt, &x.delta, &x.err, &x.codes, b->s[x.stream]);
+      else e = launch_quantize(x.v, x.fmt, x.gran, reinterpret_cast<const float*>(amax), true, x.delta, x.err, x.codes, nullptr,
+                               nullptr, b->s[x.stream], draw);
     } else if (!x.keeps_amax) {
       x.stream = next_stream; next_stream = (next_stream + 1) % kBatchStreams;
-      e = prepare_operand(x.v, x.fmt, x.gran, x.amax, x.delta, x.codes, nullptr, x.kmaj, x.err, draw, x.groups, b->s[x.stream]);
+      e = prepare_operand(x.v, x.fmt, x.gran, false, x.amax, x.delta, x.codes, x.err, draw, x.groups, b->s[x.stream]);
     } else {
       if (x.amax_root == (int)t) {
         x.stream = next_stream; next_stream = (next_stream + 1) % kBatchStreams;
@@ -825,12 +877,10 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
       }
       cudaStream_t s = b->s[x.stream];
       const uint32_t* amax = slots[x.amax_root].amax;
-      void* const kmaj = x.kmaj_root == (int)t ? x.kmaj : nullptr;
       // this operand's format and those of the later operands that borrow its pass: one pass over
       // the tensor writes all their codes (round-to-nearest-even ones; stochastic ones go singly)
       int fmts[3]; float* deltas[3]; uint32_t* errs[3]; uint8_t* codes[3];
       int nf = 0;
-      bool kmaj_written = false;
       if (!x.stochastic) { fmts[nf] = x.fmt; deltas[nf] = x.delta; errs[nf] = x.err; codes[nf] = x.codes; ++nf; }
       for (size_t u = t + 1; u < slots.size() && nf < 3; ++u) {
         Slot& y = slots[u];
@@ -841,13 +891,12 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
         fmts[nf] = y.fmt; deltas[nf] = y.delta; errs[nf] = y.err; codes[nf] = y.codes; ++nf;
         y.stream = x.stream; done[u] = 1;
       }
-      if (e == QM_OK && x.stochastic) {
+      if (e == QM_OK && x.stochastic)
         e = launch_quantize(x.v, x.fmt, x.gran, reinterpret_cast<const float*>(amax), true, x.delta, x.err, x.codes, nullptr,
-                            kmaj, s, draw);
-        kmaj_written = true;
-      }
+                            nullptr, s, draw);
       if (e == QM_OK && nf > 0)
-        e = launch_quantize_multi(x.v, x.gran, amax, nf, fmts, deltas, errs, codes, kmaj_written ? nullptr : kmaj, s);
+        e = codes_mn(x.v, false) ? launch_quantize_cols(x.v, amax, nf, fmts, deltas, errs, codes, s)
+                                 : launch_quantize_multi(x.v, x.gran, amax, nf, fmts, deltas, errs, codes, nullptr, s);
     }
     done[t] = 1;
     if (e != QM_OK && st == QM_OK) st = e;
@@ -875,12 +924,10 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
     const Slot& xr = slots[slot_of[i] + 1];
     const Slot& cl = slots[xl.code_root];
     const Slot& cr = slots[xr.code_root];
-    void* kl = slots[cl.kmaj_root].kmaj;
-    void* kr = slots[cr.kmaj_root].kmaj;
     TcProbeArgs p{};
-    p.l = kl ? kl : pl.Lv.data; p.l_ld = kl ? pl.Lv.c : pl.Lv.s_nc; p.l_sb = kl ? pl.Lv.nc * pl.Lv.c : pl.Lv.s_b;
-    p.r = kr ? kr : pl.Rv.data; p.r_ld = kr ? pl.Rv.c : pl.Rv.s_nc; p.r_sb = kr ? pl.Rv.nc * pl.Rv.c : pl.Rv.s_b;
+    set_operands(&p, pl.Lv, pl.Rv);
     p.cl = cl.codes; p.cr = cr.codes;
+    p.cl_mn = xl.mn; p.cr_mn = xr.mn;
     p.fmt_l = cfg[i].fmt_l; p.fmt_r = cfg[i].fmt_r;
     p.dl = cl.delta; p.gran_l = cfg[i].gran_l; p.dr = cr.delta; p.gran_r = cfg[i].gran_r;
     p.g = GemmShape{pl.Lv.nc, pl.Rv.nc, pl.Lv.c, pl.Lv.batch};

@@ -94,17 +94,21 @@ qm_status launch_quantize(const View& x, int fmt, int gran, const float* delta, 
 qm_status launch_quantize_multi(const View& x, int gran, const uint32_t* amax, int nf, const int* fmts,
                                 float* const* delta_out, uint32_t* const* err_word, uint8_t* const* codes,
                                 void* kmaj_copy, cudaStream_t s);
+// The same for a bf16 operand with the contraction strided and a scale per non-contracting index, its codes in the
+// operand's own order: [batch][contract] rows of qm_code_ld(noncontract) bytes.  One pass for all formats.
+qm_status launch_quantize_cols(const View& x, const uint32_t* amax, int nf, const int* fmts, float* const* delta_out,
+                               uint32_t* const* err_word, uint8_t* const* codes, cudaStream_t s);
 // Scale and quantize both operands of a probe in two launches (max|x|, then codes), for operands of modest
 // size.  `partial` needs pair_partial_words 32-bit words, not cleared; the first launch clears
 // `control` (at most 256 words), whose first word then takes QM_DEVERR_NONFINITE.
 struct PairSide {
   View v;
   int fmt, gran;
+  bool mn;                                // codes in the operand's own order (strided contraction, bf16, to nearest)
   const StochasticDraw* draw;             // null: round to nearest even
   uint32_t* partial;
   float* delta;
   uint8_t* codes;
-  void* kmaj;                             // contraction-major bf16 copy of a strided contraction, or null
 };
 size_t pair_partial_words(const View& v, int gran);
 bool pair_prepare_serves(const View& l, int gran_l, bool draw_l, const View& r, int gran_r, bool draw_r);
@@ -151,11 +155,14 @@ qm_status launch_simt_probe(const View& L, const View& R, const uint8_t* cl, int
 
 // ---- tensor-core GEMMs (gemm_tc.cu) ---------------------------------------
 struct TcProbeArgs {
-  // bf16, contraction contiguous; element strides between rows / batches
+  // bf16; contraction contiguous (element strides between rows / batches), or with l_mn / r_mn the operand's
+  // rows contiguous (strides between contraction entries / batches)
   const void* l; int64_t l_ld, l_sb;
   const void* r; int64_t r_ld, r_sb;
   const void* l_abs; const void* r_abs;     // dense [batch][rows][K]
-  const uint8_t* cl; const uint8_t* cr;     // codes, rows of qm_code_ld(K) bytes
+  // codes: rows of qm_code_ld(K) bytes, or with cl_mn / cr_mn [batch][K] rows of qm_code_ld(M or N) bytes
+  const uint8_t* cl; const uint8_t* cr;
+  bool l_mn, r_mn, cl_mn, cr_mn;    // (one-format probes only)
   int fmt_l, fmt_r;
   const float* dl; int gran_l;
   const float* dr; int gran_r;

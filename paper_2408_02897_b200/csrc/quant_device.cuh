@@ -138,6 +138,8 @@ struct QuotientPair {
     asm("mov.b64 %0, {%1, %1};" : "=l"(recip2) : "f"(r));
     asm("mov.b64 %0, {%1, %1};" : "=l"(ndelta2) : "f"(nd));
   }
+  // two elements under scales of their own: {1/delta0, 1/delta1} and {-delta0, -delta1}, packed
+  __device__ __forceinline__ QuotientPair(uint64_t recips, uint64_t ndeltas) : recip2(recips), ndelta2(ndeltas) {}
   static __device__ __forceinline__ bool serves(float d) { return d >= 8.6736174e-19f && d <= 1.1529215e18f; }
   // x2 = {x0, x1} packed; returns {RN(x0 / delta), RN(x1 / delta)} packed (a zero comes out as +0)
   __device__ __forceinline__ uint64_t operator()(uint64_t x2) const {

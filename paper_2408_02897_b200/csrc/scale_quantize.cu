@@ -930,6 +930,109 @@ quantize_transpose_bf16_kernel(const __nv_bfloat16* __restrict__ x, int64_t nc, 
   }
 }
 
+// ---------------------------------------------------------------- quantize in storage order, a scale per column
+// Storage [c][nc] (nc contiguous, bf16), a scale per column, codes in the same order: [c] rows of ldn bytes, every format
+// in MASK.  A block takes 256 columns x a run of rows; its threads first make a column's scales each (maximum bits from
+// `bits`), then a thread takes eight columns of every eighth row, four rows in flight.  Bound by HBM.
+struct ColScales { float recip[256], ndelta[256]; };      // recip 0: outside the range of the two-wide quotient
+template <int MASK, typename Bits>
+__device__ __forceinline__ void quantize_cols(const __nv_bfloat16* __restrict__ x, int64_t nc, int64_t s_c, int64_t row0, int64_t row1,
+                                              int64_t col_block, Bits bits, bool writer, const MultiOut& o, int64_t delta_at,
+                                              int64_t code_row0, int64_t ldn, ColScales* sc) {
+  {
+    const int64_t col = col_block * 256 + threadIdx.x;
+    const uint32_t m = col < nc ? bits(col) : 0u;
+    int k = 0;
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+      if (!(MASK & (1 << f))) continue;
+      const float d = m == 0 ? 1.0f : __fdiv_rn(__uint_as_float(m), fmt_qmax(f));
+      sc[k].recip[threadIdx.x] = QuotientPair::serves(d) ? __frcp_rn(d) : 0.f;
+      sc[k].ndelta[threadIdx.x] = -d;
+      ++k;
+      if (writer && col < nc) {
+        o.delta_out[f][delta_at + col] = d;
+        if (m >= 0x7f800000u && o.err_word[f]) atomicOr(o.err_word[f], QM_DEVERR_NONFINITE);
+      }
+    }
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t col0 = col_block * 256 + lane * 8;
+  if (col0 >= nc) return;
+  const int live = nc - col0 < 8 ? (int)(nc - col0) : 8;
+  const __nv_bfloat16* base = x + col0;
+  for (int64_t r = row0 + warp; r < row1; r += 32) {
+    uint4 w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t row = r + 8 * u < row1 ? r + 8 * u : r;          // repeats are not written
+      if (live == 8) {
+        w[u] = __ldg(reinterpret_cast<const uint4*>(base + row * s_c));
+      } else {
+        const unsigned short* e = reinterpret_cast<const unsigned short*>(base + row * s_c);
+        uint32_t h[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) h[j] = j < live ? (uint32_t)__ldg(e + j) : 0u;
+        w[u] = make_uint4(h[0] | h[1] << 16, h[2] | h[3] << 16, h[4] | h[5] << 16, h[6] | h[7] << 16);
+      }
+    }
+    int k = 0;
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+      if (!(MASK & (1 << f))) continue;
+      const ColScales& cs = sc[k];
+      ++k;
+      float rc[8];
+      uint64_t r2[4], n2[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        r2[j] = *reinterpret_cast<const uint64_t*>(&cs.recip[lane * 8 + 2 * j]);
+        n2[j] = *reinterpret_cast<const uint64_t*>(&cs.ndelta[lane * 8 + 2 * j]);
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(rc[2 * j]), "=f"(rc[2 * j + 1]) : "l"(r2[j]));
+      }
+      bool served = true;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) served &= rc[j] != 0.f;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (r + 8 * u >= row1) break;
+        const uint32_t pw[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
+        uint2 q;
+        if (served) {
+          uint32_t h[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const QuotientPair qp(r2[j], n2[j]);
+            h[j] = (f == 0 ? quant_bf16_pair<0>(pw[j], qp) : f == 1 ? quant_bf16_pair<1>(pw[j], qp) : quant_bf16_pair<2>(pw[j], qp)) & 0xffffu;
+          }
+          q = make_uint2(h[0] | h[1] << 16, h[2] | h[3] << 16);
+        } else {
+          uint32_t h[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float t0 = Quotient(-cs.ndelta[lane * 8 + 2 * j])(bf16_lo(pw[j])), t1 = Quotient(-cs.ndelta[lane * 8 + 2 * j + 1])(bf16_hi(pw[j]));
+            h[j] = f == 0 ? quant2<0>(t0, t1) : f == 1 ? quant2<1>(t0, t1) : quant2<2>(t0, t1);
+          }
+          q = make_uint2(h[0] | h[1] << 16, h[2] | h[3] << 16);
+        }
+        *reinterpret_cast<uint2*>(o.codes[f] + (code_row0 + r + 8 * u) * ldn + col0) = q;
+      }
+    }
+  }
+}
+
+template <int MASK>
+__global__ void __launch_bounds__(kThreads)
+quantize_cols_kernel(const __nv_bfloat16* __restrict__ x, int64_t nc, int64_t c, int64_t s_c, int64_t s_b, int64_t rows_per_block,
+                     const uint32_t* __restrict__ amax, const MultiOut o, int64_t ldn) {
+  pdl_prologue();
+  __shared__ __align__(16) ColScales sc[(MASK & 1) + (MASK >> 1 & 1) + (MASK >> 2 & 1)];
+  const int64_t b = blockIdx.z, row0 = (int64_t)blockIdx.y * rows_per_block, row1 = min(c, row0 + rows_per_block);
+  quantize_cols<MASK>(x + b * s_b, nc, s_c, row0, row1, blockIdx.x, [&](int64_t col) { return __ldg(amax + b * nc + col); },
+                      blockIdx.y == 0, o, b * nc, b * c, ldn, sc);
+}
+
 // ---------------------------------------------------------------- both operands of a probe in two launches
 // A probe of modest operands is bound by its chain of launches, not by what they do: clear, max|x| and
 // quantize for one operand, the same for the other, products.  Here one kernel takes the maxima of both
@@ -939,7 +1042,8 @@ quantize_transpose_bf16_kernel(const __nv_bfloat16* __restrict__ x, int64_t nc, 
 //   one per strided channel:   a maximum per column and slice of the contraction (at most kPairSlices);
 //   one per contiguous row:    none, the second kernel reduces a row itself.
 constexpr int kPairBlocks = 256, kPairSlices = 8;
-enum { kPairChunks = 0, kPairRows = 1, kPairTiles = 2, kPairGeneral = 3 };
+constexpr int kPairColRows = 64;          // rows of a block of kPairCols
+enum { kPairChunks = 0, kPairRows = 1, kPairTiles = 2, kPairGeneral = 3, kPairCols = 4 };
 
 struct PairOperand {
   View v;
@@ -947,12 +1051,12 @@ struct PairOperand {
   int32_t blocks_max, n_partial;          // blocks of the first kernel; partial maxima per scale
   int32_t blocks_quant, path;             // blocks of the second kernel, and how it walks the operand
   uint32_t gx, gy;                        // tiles: column tiles, contraction tiles
+  uint32_t max_cols;                      // one scale per strided channel: blocks of 64 columns
   uint32_t groups_per_line, total_groups, lines;   // the tensor as lines of contiguous groups of eight; lines per batch element
-  FastDiv by_groups, by_lines, by_chunks, by_nc, by_gx, by_gy;
+  FastDiv by_groups, by_lines, by_chunks, by_nc, by_gx, by_gy, by_max_cols;
   uint32_t* partial;
   float* delta;
   uint8_t* codes;
-  __nv_bfloat16* kmaj;
   Rounding rnd;
 };
 struct PairArgs {
@@ -994,7 +1098,7 @@ __device__ __forceinline__ void pair_max(const PairOperand& o, uint32_t block, u
   }
   // a column each: 64 columns of one batch element, one slice of the contraction
   const uint32_t slice = block % (uint32_t)o.n_partial, rest = block / (uint32_t)o.n_partial;
-  const uint32_t b = o.by_gx.div(rest), cb = rest - b * o.gx;
+  const uint32_t b = o.by_max_cols.div(rest), cb = rest - b * o.max_cols;
   const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
   const int64_t col0 = (int64_t)cb * 64 + tx * 8, per = (v.c + o.n_partial - 1) / o.n_partial;
   const int64_t r0 = slice * per, r1 = r0 + per < v.c ? r0 + per : v.c;
@@ -1102,8 +1206,23 @@ __device__ __forceinline__ void pair_quantize(const PairOperand& o, uint32_t* er
   // strided contraction: tiles
   const uint32_t rest = o.by_gx.div(block), bz = o.by_gy.div(rest);
   const uint3 at = make_uint3(block - rest * o.gx, rest - bz * o.gy, bz);
+  if constexpr (sizeof(T) == 2) {
+    if (o.path == kPairCols) {              // codes in storage order, a scale per column
+      MultiOut out{};
+      out.codes[FMT] = o.codes; out.delta_out[FMT] = o.delta; out.err_word[FMT] = err;
+      const int64_t row0 = (int64_t)at.y * kPairColRows, row1 = row0 + kPairColRows < v.c ? row0 + kPairColRows : v.c;
+      auto bits = [&](int64_t col) {
+        uint32_t m = 0;
+        for (int i = 0; i < o.n_partial; ++i) m = max(m, __ldg(o.partial + ((int64_t)i * v.batch + at.z) * v.nc + col));
+        return m;
+      };
+      quantize_cols<1 << FMT>(x + (int64_t)at.z * v.s_b, v.nc, v.s_c, row0, row1, at.x, bits, at.y == 0, out, (int64_t)at.z * v.nc,
+                              (int64_t)at.z * v.c, (v.nc + 15) & ~(int64_t)15, reinterpret_cast<ColScales*>(smem));
+      return;
+    }
+  }
   if (o.path == kPairGeneral) {
-    transpose_general<T, FMT>(x, v.nc, v.c, v.s_c, v.s_b, scale, o.codes, ldc, nullptr, o.kmaj, o.rnd,
+    transpose_general<T, FMT>(x, v.nc, v.c, v.s_c, v.s_b, scale, o.codes, ldc, nullptr, nullptr, o.rnd,
                               *reinterpret_cast<float(*)[64][65]>(smem), at);
     return;
   }
@@ -1114,8 +1233,8 @@ __device__ __forceinline__ void pair_quantize(const PairOperand& o, uint32_t* er
     if (col < v.nc) d_lo[FMT] = scale(orow, writer);
     if (col + 1 < v.nc) d_hi[FMT] = scale(orow + 1, writer);
     uint8_t* const cd[3] = {o.codes, o.codes, o.codes};
-    if (o.rnd.stochastic) transpose_tile<1 << FMT, false, true, true>(x, v.nc, v.c, v.s_c, v.s_b, d_lo, d_hi, cd, ldc, o.kmaj, smem, at, o.rnd);
-    else transpose_tile<1 << FMT, false, true, false>(x, v.nc, v.c, v.s_c, v.s_b, d_lo, d_hi, cd, ldc, o.kmaj, smem, at);
+    if (o.rnd.stochastic) transpose_tile<1 << FMT, false, true, true>(x, v.nc, v.c, v.s_c, v.s_b, d_lo, d_hi, cd, ldc, nullptr, smem, at, o.rnd);
+    else transpose_tile<1 << FMT, false, true, false>(x, v.nc, v.c, v.s_c, v.s_b, d_lo, d_hi, cd, ldc, nullptr, smem, at);
   }
 }
 
@@ -1393,9 +1512,12 @@ qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint
   for (int i = 0; i < 2; ++i) {
     const PairSide& in = side[i];
     PairOperand& o = a.op[i];
-    const View& v = in.v;
-    o.v = v; o.per_channel = in.gran == QM_GRAN_CHANNEL;
-    o.partial = in.partial; o.delta = in.delta; o.codes = in.codes; o.kmaj = static_cast<__nv_bfloat16*>(in.kmaj);
+    o.v = in.v; o.per_channel = in.gran == QM_GRAN_CHANNEL;
+    if (in.mn && !o.per_channel) {          // codes in storage order under one scale: those of the flipped view
+      o.v.nc = in.v.c; o.v.c = in.v.nc; o.v.s_nc = in.v.s_c; o.v.s_c = in.v.s_nc;
+    }
+    const View& v = o.v;
+    o.partial = in.partial; o.delta = in.delta; o.codes = in.codes;
     if (in.draw) { o.rnd.stochastic = 1; o.rnd.k0 = (uint32_t)in.draw->seed; o.rnd.k1 = (uint32_t)(in.draw->seed >> 32); o.rnd.stream = in.draw->stream; }
     const bool tiles = tile_form(v, in.draw != nullptr);
     const int64_t ldc = qm_code_ld(v.c);
@@ -1405,9 +1527,9 @@ qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint
       o.blocks_quant = (int32_t)((threads + kThreads - 1) / kThreads);
       o.by_chunks = FastDiv((uint32_t)chunks); o.by_nc = FastDiv((uint32_t)v.nc);
     } else {
-      o.path = tiles ? kPairTiles : kPairGeneral;
-      o.gx = (uint32_t)((v.nc + 63) / 64);
-      o.gy = (uint32_t)(tiles ? (v.c + 127) / 128 : (ldc + 63) / 64);
+      o.path = in.mn ? kPairCols : tiles ? kPairTiles : kPairGeneral;
+      o.gx = (uint32_t)(in.mn ? (v.nc + 255) / 256 : (v.nc + 63) / 64);
+      o.gy = (uint32_t)(in.mn ? (v.c + kPairColRows - 1) / kPairColRows : tiles ? (v.c + 127) / 128 : (ldc + 63) / 64);
       o.by_gx = FastDiv(o.gx); o.by_gy = FastDiv(o.gy);
       o.blocks_quant = (int32_t)((int64_t)o.gx * o.gy * v.batch);
     }
@@ -1424,7 +1546,9 @@ qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint
       // slices of at least 128 contraction entries
       const int64_t want = (v.c + 127) / 128;
       o.n_partial = (int32_t)(want < kPairSlices ? want : kPairSlices);
-      o.blocks_max = (int32_t)((int64_t)o.gx * v.batch * o.n_partial);
+      o.max_cols = (uint32_t)((v.nc + 63) / 64);
+      o.by_max_cols = FastDiv(o.max_cols);
+      o.blocks_max = (int32_t)((int64_t)o.max_cols * v.batch * o.n_partial);
     }
   }
   const unsigned maxima = (unsigned)(a.op[0].blocks_max + a.op[1].blocks_max);
@@ -1542,6 +1666,40 @@ qm_status launch_quantize_multi(const View& x, int gran, const uint32_t* amax, i
     }
 #undef QM_TM
   }
+  count_launch();
+  QM_CUDA_OK(cudaGetLastError());
+  return QM_OK;
+}
+
+qm_status launch_quantize_cols(const View& x, const uint32_t* amax, int nf, const int* fmts, float* const* delta_out,
+                               uint32_t* const* err_word, uint8_t* const* codes, cudaStream_t s) {
+  if (x.dtype != QM_DT_BF16 || x.c_contig() || nf < 1 || nf > 3) return QM_ERR_INVALID_ARG;
+  int mask = 0;
+  MultiOut o{};
+  for (int k = 0; k < nf; ++k) {
+    const int f = fmts[k];
+    if (f < 0 || f > 2 || (mask & (1 << f))) return QM_ERR_INVALID_ARG;
+    mask |= 1 << f;
+    o.codes[f] = codes[k]; o.delta_out[f] = delta_out[k]; o.err_word[f] = err_word[k];
+  }
+  // runs of rows that give every SM four blocks, of at least 32 rows (one step) and at most 65535 of them
+  const int64_t col_blocks = (x.nc + 255) / 256, want = (4ll * sm_count() + col_blocks * x.batch - 1) / (col_blocks * x.batch);
+  int64_t rows = (x.c + want - 1) / want;
+  rows = (rows + 31) / 32 * 32;
+  const dim3 grid((unsigned)col_blocks, (unsigned)((x.c + rows - 1) / rows), (unsigned)x.batch);
+  if (col_blocks > 0x7fffffffll || x.batch > 65535) return QM_ERR_UNSUPPORTED;
+  const __nv_bfloat16* p = static_cast<const __nv_bfloat16*>(x.data);
+#define QM_QC(M) launch_pdl(quantize_cols_kernel<M>, grid, dim3(kThreads), 0, s, p, x.nc, x.c, x.s_c, x.s_b, rows, amax, o, qm_code_ld(x.nc))
+  switch (mask) {
+    case 1: QM_QC(1); break;
+    case 2: QM_QC(2); break;
+    case 3: QM_QC(3); break;
+    case 4: QM_QC(4); break;
+    case 5: QM_QC(5); break;
+    case 6: QM_QC(6); break;
+    default: QM_QC(7); break;
+  }
+#undef QM_QC
   count_launch();
   QM_CUDA_OK(cudaGetLastError());
   return QM_OK;
