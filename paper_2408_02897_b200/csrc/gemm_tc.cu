@@ -1049,10 +1049,11 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 //
 // The left operand of the reference and denominator products is not read from shared memory by the tensor
 // cores: converter warps read this CTA's 128 rows of the L tile once and store them, and the same with
-// the sign bits cleared, into TENSOR memory, from where both products take their A operand; they also
-// write the |R| half-tile into the stage.  No |x| copy exists in HBM.  Taking only |L| from tensor
-// memory (four stages of it instead of two of both) measured 3 to 8 % slower (the MMAs then read L from
-// shared memory); half-block stages, an |R| copy by two other warps and prefetching the next
+// the sign bits cleared, into TENSOR memory, from where both products take their A operand; two more warps
+// write the |R| half-tile into the stage.  No |x| copy exists in HBM.  What the bf16 phase waits for is the
+// converters' serial time per block: wait, loads, wait for the tensor-memory stage, stores, arrival (4096^2 x 1024 in three
+// formats, cycles per block: 760 with |R| among the converters' work, 683 with two warps for it; 553 with all conversions left
+// out; four stages in tensor memory instead of two change nothing).  Half-block stages and prefetching the next
 // block's values ahead of the fences each measured 5 to 20 % slower.
 //
 // Operands whose contraction is strided are staged as they lie in memory (mn-major tiles, a contraction entry per 128-byte
@@ -1066,8 +1067,8 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 //                 (128 deep); both kinds bring 128 bytes per row.  A CTA's loads complete on its own `full`.
 //   warp 1        allocates tensor memory; in the leader CTA it runs the MMA loop converged and
 //                 one elected lane issues the pair's MMAs; tcgen05.commit frees a stage in both CTAs (`empty`).
-//   warps 2, 3    idle (they fill the first warpgroup).
-//   warps 4..7    converters, one per tensor-memory lane quarter: thread = one of the CTA's 128
+//   warps 2, 3    |R|: a sign-cleared copy of each staged R half-tile.
+//   warps 4..7    converters of L, one per tensor-memory lane quarter: thread = one of the CTA's 128
 //                 left-operand rows.  Blocks of codes need no conversion: they only pass on that they landed.
 //   warps 8..15   epilogue.
 // Tensor memory: columns 0..127 reference, 128..255 denominator, 256..383 and 384..511 two 8-bit
@@ -1275,6 +1276,11 @@ __device__ __forceinline__ void tma_load_3d_local(uint32_t dst, const CUtensorMa
       ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
       : "memory");
 }
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+  return v;
+}
 __device__ __forceinline__ void sts128(uint32_t addr, uint4 v) {
   asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
@@ -1318,6 +1324,18 @@ __device__ __forceinline__ void load_l_mn_major(uint32_t base, int q, int lane, 
     for (int n = 0; n < 4; ++n) ldmatrix4_trans(at + (uint32_t)n * 2048u, &a[16 * h + 4 * n]);
   }
 }
+// |R| beside a staged R half-tile, whatever its order: a flat sign-cleared copy of its first `vectors` 16-byte vectors (at most
+// 512) by the two warps to which t = 0..63 belongs, made visible to the tensor core's reads.
+__device__ __forceinline__ void abs_r_half(uint32_t r, uint32_t to_abs, int vectors, int t) {
+  const uint32_t src = r + (uint32_t)t * 16u, m = 0x7fff7fffu;
+  uint4 u[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) u[j] = t + 64 * j < vectors ? lds128(src + (uint32_t)j * 1024u) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    if (t + 64 * j < vectors) sts128(src + to_abs + (uint32_t)j * 1024u, make_uint4(u[j].x & m, u[j].y & m, u[j].z & m, u[j].w & m));
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
 // 32 lanes x 8 consecutive 32-bit columns.
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
   asm volatile(
@@ -1335,12 +1353,6 @@ __device__ __forceinline__ void mma_pair_a_tmem(uint32_t tmem_d, uint32_t tmem_a
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
       ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(accumulate) : "memory");
-}
-
-__device__ __forceinline__ uint4 lds128(uint32_t addr) {
-  uint4 v;
-  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-  return v;
 }
 
 // Eq. 3 statistics of one row of one variant's tile.
@@ -1517,7 +1529,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&sh->full[s]), 1);
-      mbar_init(smem_u32(&sh->ready[s]), 2 * 4);          // four converter warps in each CTA
+      mbar_init(smem_u32(&sh->ready[s]), 2 * 6);          // four converter warps and two for |R| in each CTA
       mbar_init(smem_u32(&sh->empty[s]), 1);
     }
     mbar_init(smem_u32(&sh->rd_full), 1);
@@ -1668,6 +1680,31 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           if (b) ++lp_uses1; else ++lp_uses0;
         }
       }
+    } else if (warp >= 2) {
+      // ---------------------------------------------------------- |R| (both CTAs)
+      TileWalk tw;
+      tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
+      const int t = (warp - 2) * 32 + lane;        // 0..63
+      const uint32_t ready_leader = map_to_cta(smem_u32(&sh->ready[0]), 0);
+      Ring ring;
+      bool ok = true;
+      for (; tw.valid && ok; tw.next_tile()) {
+        for (int kb = 0; kb < tw.num_kb && ok; ++kb) {
+          ok = w.wait_warp(smem_u32(&sh->full[ring.s]), ring.parity);
+          if (!ok) break;
+          abs_r_half(tile_base + ring.s * C::kStageBytes + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(ready_leader + ring.s * 8u);
+          ring.next();
+        }
+        const int n_code_blocks = tw.n_var * tw.lp_blocks();     // only passed on
+        for (int kb = 0; kb < n_code_blocks && ok; ++kb) {
+          ok = w.wait_warp(smem_u32(&sh->full[ring.s]), ring.parity);
+          if (!ok) break;
+          if (lane == 0) mbar_arrive_cluster(ready_leader + ring.s * 8u);
+          ring.next();
+        }
+      }
     }
   } else if (warp < kFirstEpiWarp) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsConv));
@@ -1678,8 +1715,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
     // which makes these row-per-thread reads conflict-free) and stores the 32 words, and the same with
     // the sign bits cleared, into the stage's tensor-memory columns.  (Loading the rows with plain global loads
     // instead, to spare shared memory the 16 KB, was tried: a warp then touches 32 lines per
-    // instruction and the converters became the bottleneck, 1.6 x slower overall.)  The |R|
-    // half-tile is a flat sign-cleared copy of the R half-tile (8 KB: four vectors per thread).
+    // instruction and the converters became the bottleneck, 1.6 x slower overall.)
     const int q = warp & 3;
     const int t = q * 32 + lane;                   // 0..127
     const uint32_t ready_leader = map_to_cta(smem_u32(&sh->ready[0]), 0);
@@ -1696,7 +1732,6 @@ tc_group_kernel(const __grid_constant__ Table tab) {
       if (it > 0) ok = w.wait_warp(smem_u32(&sh->rd_full), (it - 1) & 1);
       if (ok && lent) ok = w.wait_warp(smem_u32(&sh->abs_free), abs_uses++ & 1);
       lent = tw.n_var > 1;
-      const int r_vec = tw.half_n * 8;                           // 16-byte vectors of the R half-tile that are in use
       const bool l_mn = tw.major & kUnitMnMajorL;
       // a loop for each order of L: one loop with the choice inside cost the contraction-major one 7 %
       auto convert = [&](auto mn) {
@@ -1706,11 +1741,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           ok = w.wait_warp(smem_u32(&sh->full[s]), ring.parity);
           if (!ok) break;
           const uint32_t base = tile_base + s * C::kStageBytes;
-          uint4 u[4];
           uint32_t a[32];
-          const uint32_t rsrc = base + C::kOffR + (uint32_t)t * 16u;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) u[j] = t + 128 * j < r_vec ? lds128(rsrc + (uint32_t)j * 2048u) : make_uint4(0u, 0u, 0u, 0u);
           if constexpr (kMn) {
             load_l_mn_major(base + C::kOffL, q, lane, a);
           } else {
@@ -1720,10 +1751,6 @@ tc_group_kernel(const __grid_constant__ Table tab) {
               a[4 * j] = v.x; a[4 * j + 1] = v.y; a[4 * j + 2] = v.z; a[4 * j + 3] = v.w;
             }
           }
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (t + 128 * j < r_vec)
-              sts128(rsrc + (C::kOffRa - C::kOffR) + (uint32_t)j * 2048u, make_uint4(u[j].x & m, u[j].y & m, u[j].z & m, u[j].w & m));
           if (kb >= kTmemStages) {
             // the tensor-memory columns were last read by the MMAs of the block kTmemStages before this one
             const uint32_t sp = s >= (uint32_t)kTmemStages ? s - kTmemStages : s + kStages - kTmemStages;
@@ -1747,7 +1774,6 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           } else {
             tmem_st32(tcol + 32u, a);
           }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // generic-proxy writes -> the tensor core's reads
           asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
           tc_fence_before();
           __syncwarp();
@@ -1980,32 +2006,34 @@ tc_group_kernel(const __grid_constant__ Table tab) {
 
 // ------------------------------------------------------------------ the fused probe kernel, one probe per unit
 // Units of one probe share nothing, so their three products run side by side, k-block by k-block: a stage
-// holds the bf16 and the code tiles of 64 contraction entries and one commit frees it.  112 KB go through shared
-// memory per k-block (36 by TMA, 44 of MMA operands, 32 by the converters) against the 96 of the
-// products one after the other, but a tile has no phases: the converters run four blocks ahead
+// holds the bf16 and the code tiles of 64 contraction entries and one commit frees it.  96 KB go through shared
+// memory per k-block (36 by TMA, 28 of MMA operands, 32 by the converters), as for the products one after the other,
+// but a tile has no phases: the converters run ahead
 // across its end, the next tile's reference and denominator MMAs start while this one's last columns are evaluated, and
 // the epilogue takes all three products in one sweep (the reciprocals beside the other arithmetic,
 // the sums in registers) with one wait.  Short contractions are bound by that chain.  Measured, the fused kernel
 // alone, one after the other / side by side: 512 x 512 x 64 x 256 131 / 88 us; 8192 x 4096 with K = 128 75 / 53,
 // K = 256 76 / 64, K = 512 91 / 88, K = 1024 145 / 140.  With three probes per unit sharing wins from K = 64 on (187 / 239 us).
+// With L read from shared memory by the reference MMAs (112 KB) and |R| among the converters' work K = 1024 took 145 us, so
+// 136; 2048 x 3072 x 2048 69.7 / 63.6.
 //   Roles, registers, walk and exit are those of tc_group_kernel.  Tensor memory: columns 0..127 reference, 128..255
-// denominator, 256..383 the 8-bit product, 384..511 four stages of |L| (32 columns of two bf16 each).
+// denominator, 256..383 the 8-bit product, 384..511 two stages of L and |L| (32 columns of two bf16 each).
 struct CfgS {
   static constexpr int kStages = 5;          // stages of shared memory (TMA ring)
-  static constexpr int kAbsStages = 4;       // stages of |L| in tensor memory (128 columns / 32)
+  static constexpr int kTmemStages = 2;       // stages of L and |L| in tensor memory (128 columns / 64)
   // stage: L, R, |R| (written by the converters), codes of L, codes of R
   static constexpr uint32_t kOffL = 0, kOffR = kABf16, kOffRa = kOffR + kBBf16, kOffCl = kOffRa + kBBf16;
   static constexpr uint32_t kOffCr = kOffCl + kALp;
   static constexpr uint32_t kStageBytes = kOffCr + kBLp;             // 44 KB
   static constexpr uint32_t kTileBytes = kStages * kStageBytes;      // 220 KB
-  static constexpr uint32_t kColRef = 0, kColDen = 128, kColLp = 256, kColAbsL = 384;   // tensor-memory columns
+  static constexpr uint32_t kColRef = 0, kColDen = 128, kColLp = 256, kColL = 384;   // tensor-memory columns
 };
 
 template <int UNITS>
 struct SharedS {
   uint64_t full[CfgS::kStages];     // per CTA: this CTA's loads of a stage have landed
-  uint64_t ready[CfgS::kAbsStages]; // leader: both CTAs' converters have seen their loads land and have written
-                                    //         |L| (tensor memory) and |R| (stage)
+  uint64_t ready[CfgS::kStages];    // leader: both CTAs' converters have seen their loads land and have written
+                                    //         L and |L| (tensor memory) and |R| (stage)
   uint64_t empty[CfgS::kStages];    // per CTA: the pair's MMAs have finished with the k-block of the stage
   uint64_t tmem_full;               // per CTA: the tile's accumulators are complete
   uint64_t tmem_empty;              // leader: both CTAs' epilogues have copied out reference and denominator
@@ -2086,7 +2114,7 @@ __global__ void __launch_bounds__(kProbeThreads, 1)
 tc_side_kernel(const __grid_constant__ Table tab) {
   using C = CfgS;
   using Sh = SharedS<Table::kUnits>;
-  constexpr int kStages = C::kStages, kAbs = C::kAbsStages;
+  constexpr int kStages = C::kStages, kAbs = C::kTmemStages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   Sh* sh = reinterpret_cast<Sh*>(tiles + C::kTileBytes);
@@ -2111,7 +2139,7 @@ tc_side_kernel(const __grid_constant__ Table tab) {
       mbar_init(smem_u32(&sh->full[s]), 1);
       mbar_init(smem_u32(&sh->empty[s]), 1);
     }
-    for (int s = 0; s < kAbs; ++s) mbar_init(smem_u32(&sh->ready[s]), 2 * 4);   // four converter warps in each CTA
+    for (int s = 0; s < kStages; ++s) mbar_init(smem_u32(&sh->ready[s]), 2 * 6);   // four converter warps and two for |R| in each CTA
     mbar_init(smem_u32(&sh->tmem_full), 1);
     mbar_init(smem_u32(&sh->tmem_empty), 2 * kEpiWarps);
     mbar_init(smem_u32(&sh->lp_done), 2 * kEpiWarps);
@@ -2171,17 +2199,17 @@ tc_side_kernel(const __grid_constant__ Table tab) {
     } else if (warp == 1 && rank == 0) {
       // ---------------------------------------------------------- MMA issuer (leader CTA, converged warp)
       const bool lead = elect_one();
-      uint32_t idesc_ref = 0, idesc_den = 0;   // of the tile in hand
-      TileDesc ld{}, rd{}, cl{}, cr{};         // L; R and |R|; codes
+      uint32_t idesc_bf16 = 0;                 // of the tile in hand
+      TileDesc rd{}, cl{}, cr{};               // R and |R|; codes
       auto issue_ref_den = [&](uint32_t gg, int kb) {
         const uint32_t s = gg % kStages, base = tile_base + s * C::kStageBytes;
+        const uint32_t ta = tmem_base + C::kColL + 64u * (gg % kAbs);
 #pragma unroll
         for (int k = 0; k < kBlockK / 16; ++k)   // 16 bf16 per step
-          mma_pair<kKindF16>(tmem_base + C::kColRef, ld.at(base + C::kOffL, k), rd.at(base + C::kOffR, k), idesc_ref, (kb | k) != 0, lead);
-        const uint32_t ta = tmem_base + C::kColAbsL + 32u * (gg % kAbs);
+          mma_pair_a_tmem(tmem_base + C::kColRef, ta + 8u * k, rd.at(base + C::kOffR, k), idesc_bf16, (kb | k) != 0, lead);
 #pragma unroll
         for (int k = 0; k < kBlockK / 16; ++k)   // 16 bf16 = 8 columns of tensor memory per step
-          mma_pair_a_tmem(tmem_base + C::kColDen, ta + 8u * k, rd.at(base + C::kOffRa, k), idesc_den, (kb | k) != 0, lead);
+          mma_pair_a_tmem(tmem_base + C::kColDen, ta + 32u + 8u * k, rd.at(base + C::kOffRa, k), idesc_bf16, (kb | k) != 0, lead);
       };
       auto issue_lp = [&](uint32_t gg, int kb, bool is_i8, uint32_t idesc_lp) {
         const uint32_t base = tile_base + (gg % kStages) * C::kStageBytes;
@@ -2193,7 +2221,7 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         }
       };
       auto wait_stage = [&](uint32_t gg) {
-        if (!w.wait_warp(smem_u32(&sh->ready[gg % kAbs]), (gg / kAbs) & 1)) return false;
+        if (!w.wait_warp(smem_u32(&sh->ready[gg % kStages]), (gg / kStages) & 1)) return false;
         tc_fence_after();
         return true;
       };
@@ -2207,11 +2235,9 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         const uint32_t idesc_lp = __shfl_sync(0xffffffffu, sh->var[tw.pi].idesc, 0);
         const uint32_t flags = __shfl_sync(0xffffffffu, sh->var[tw.pi].flags, 0);
         const bool is_i8 = flags & kVarI8, cr_mn = flags & kVarMnMajorR;
-        const bool l_mn = tw.major & kUnitMnMajorL, r_mn = tw.major & kUnitMnMajorR;
-        // |L| comes from tensor memory, contraction-major always
-        idesc_den = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n) | (r_mn ? kIdescMnMajorB : 0u);
-        idesc_ref = idesc_den | (l_mn ? kIdescMnMajorA : 0u);
-        ld = tile_desc(l_mn, 128u, 16u, kABf16 / 2);
+        const bool r_mn = tw.major & kUnitMnMajorR;
+        // L and |L| come from tensor memory, contraction-major always
+        idesc_bf16 = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n) | (r_mn ? kIdescMnMajorB : 0u);
         rd = tile_desc(r_mn, r_mn ? 2u * tw.half_n : 128u, 16u, 16u);
         cl = tile_desc(flags & kVarMnMajorL, flags & kVarMnMajorL ? 128u : 64u, 32u, 16u);
         cr = tile_desc(cr_mn, cr_mn ? tw.half_n : 64u, 32u, 16u);
@@ -2241,17 +2267,34 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         }
         if (ok) tc_commit_pair(smem_u32(&sh->tmem_full), lead);           // this tile's accumulators are complete
       }
+    } else if (warp >= 2) {
+      // ---------------------------------------------------------- |R| (both CTAs)
+      TileWalk tw;
+      tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
+      const int t = (warp - 2) * 32 + lane;        // 0..63
+      const uint32_t ready_leader = map_to_cta(smem_u32(&sh->ready[0]), 0);
+      bool ok = true;
+      uint32_t s = 0, parity = 0;
+      for (; tw.valid && ok; tw.next_tile()) {
+        for (int kb = 0; kb < tw.num_kb; ++kb) {
+          ok = w.wait_warp(smem_u32(&sh->full[s]), parity);
+          if (!ok) break;
+          abs_r_half(tile_base + s * C::kStageBytes + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(ready_leader + s * 8u);
+          if (++s == (uint32_t)kStages) { s = 0; parity ^= 1u; }
+        }
+      }
     }
   } else if (warp < kFirstEpiWarp) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsConv));
     // ------------------------------------------------------------ converters (both CTAs)
-    // As in tc_group_kernel, but only |L| goes to tensor memory (the reference MMAs read L from shared memory),
-    // and the k-blocks are counted through over all tiles: the converters run up to kAbs blocks ahead
-    // of the MMAs across a tile's end.
+    // As in tc_group_kernel, but the k-blocks are counted through over all tiles: the converters run up to
+    // kAbs blocks ahead of the MMAs across a tile's end.
     const int q = warp & 3;
     const int t = q * 32 + lane;                   // 0..127
     const uint32_t ready_leader = map_to_cta(smem_u32(&sh->ready[0]), 0);
-    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + C::kColAbsL;
+    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + C::kColL;
     const uint32_t row_off = (uint32_t)t * 128u, sw = (uint32_t)t & 7u;
     TileWalk tw;
     tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
@@ -2261,17 +2304,9 @@ tc_side_kernel(const __grid_constant__ Table tab) {
     auto convert = [&](auto mn) {
       constexpr bool kMn = decltype(mn)::value;
       for (int kb = 0; kb < tw.num_kb; ++kb, ++g) {
-        const uint32_t s = g % kStages, sa = g % kAbs, m = 0x7fff7fffu;
-        // the tensor-memory columns were last read by the MMAs of k-block g - kAbs (its commit also
-        // covers every earlier k-block, so the |R| slot of the stage is free as well)
-        if (g >= (uint32_t)kAbs) {
-          const uint32_t gp = g - kAbs;
-          if (!w.wait_warp(smem_u32(&sh->empty[gp % kStages]), (gp / kStages) & 1)) { ok = false; return; }
-        }
+        const uint32_t s = g % kStages, m = 0x7fff7fffu;
         if (!w.wait_warp(smem_u32(&sh->full[s]), (g / kStages) & 1)) { ok = false; return; }
-        tc_fence_after();
         const uint32_t base = tile_base + s * C::kStageBytes;
-        uint4 u[4];
         uint32_t a[32];
         if constexpr (kMn) {
           load_l_mn_major(base + C::kOffL, q, lane, a);
@@ -2282,27 +2317,31 @@ tc_side_kernel(const __grid_constant__ Table tab) {
             a[4 * j] = v.x; a[4 * j + 1] = v.y; a[4 * j + 2] = v.z; a[4 * j + 3] = v.w;
           }
         }
-        const uint32_t rsrc = base + C::kOffR + (uint32_t)t * 16u;
-        const int r_vec = tw.half_n * 8;                           // 16-byte vectors of the R half-tile that are in use
-#pragma unroll
-        for (int j = 0; j < 4; ++j) u[j] = t + 128 * j < r_vec ? lds128(rsrc + (uint32_t)j * 2048u) : make_uint4(0u, 0u, 0u, 0u);
+        // the tensor-memory columns were last read by the MMAs of k-block g - kAbs
+        if (g >= (uint32_t)kAbs) {
+          const uint32_t gp = g - kAbs;
+          if (!w.wait_warp(smem_u32(&sh->empty[gp % kStages]), (gp / kStages) & 1)) { ok = false; return; }
+        }
+        tc_fence_after();
+        const uint32_t tcol = taddr + 64u * (g % kAbs);
+        if constexpr (kMn) {
+          tmem_st16x32(tcol, a);
+          tmem_st16x32(tcol + (16u << 16), a + 16);
+        } else {
+          tmem_st32(tcol, a);
+        }
 #pragma unroll
         for (int j = 0; j < 32; ++j) a[j] &= m;
         if constexpr (kMn) {
-          tmem_st16x32(taddr + 32u * sa, a);
-          tmem_st16x32(taddr + 32u * sa + (16u << 16), a + 16);
+          tmem_st16x32(tcol + 32u, a);
+          tmem_st16x32(tcol + 32u + (16u << 16), a + 16);
         } else {
-          tmem_st32(taddr + 32u * sa, a);
+          tmem_st32(tcol + 32u, a);
         }
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (t + 128 * j < r_vec)
-            sts128(rsrc + (C::kOffRa - C::kOffR) + (uint32_t)j * 2048u, make_uint4(u[j].x & m, u[j].y & m, u[j].z & m, u[j].w & m));
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // generic-proxy writes -> the tensor core's reads
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(ready_leader + sa * 8u);
+        if (lane == 0) mbar_arrive_cluster(ready_leader + s * 8u);
       }
     };
     for (; ok && tw.valid; tw.next_tile()) {
