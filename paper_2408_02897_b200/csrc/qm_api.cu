@@ -866,7 +866,16 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
                                nullptr, b->s[x.stream], draw);
     } else if (!x.keeps_amax) {
       x.stream = next_stream; next_stream = (next_stream + 1) % kBatchStreams;
-      e = prepare_operand(x.v, x.fmt, x.gran, false, x.amax, x.delta, x.codes, x.err, draw, x.groups, b->s[x.stream]);
+      // this operand's format and the others that later probes ask for under the same scales' grouping: one read
+      int fmts[3] = {x.fmt}; float* deltas[3] = {x.delta}; uint32_t* errs[3] = {x.err}; uint8_t* codes[3] = {x.codes};
+      int nf = 1;
+      for (size_t u = t + 1; u < slots.size() && nf < 3; ++u) {
+        Slot& y = slots[u];
+        if (y.code_root != (int)u || y.keeps_amax || done[u] || !same_view(x.v, y.v)) continue;
+        fmts[nf] = y.fmt; deltas[nf] = y.delta; errs[nf] = y.err; codes[nf] = y.codes; ++nf;
+        y.stream = x.stream; done[u] = 1;
+      }
+      e = launch_scale_quantize_rows_multi(x.v, nf, fmts, deltas, errs, codes, b->s[x.stream]);
     } else {
       if (x.amax_root == (int)t) {
         x.stream = next_stream; next_stream = (next_stream + 1) % kBatchStreams;

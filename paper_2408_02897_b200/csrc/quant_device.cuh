@@ -153,22 +153,23 @@ struct QuotientPair {
   }
 };
 
-// Two codes (bits 0..7 and 8..15) of the bf16 pair held in word w (low half = first element).
+// Two codes (bits 0..7 and 8..15) of two values given by their fp32 bit patterns, or of the bf16 pair held in word w (low
+// half = first element).
 // GUARD: the scale may come from elsewhere, so x r can overflow and the corrections then evaluate
 // inf - inf; fminf returns its non-NaN operand, which turns that case into the largest float and
 // lets the conversion saturate, as the division would.
 // INT8 under the operand's own scale: |t| <= 127 (1 + 2^-23), so t + 1.5 2^23 is t rounded to nearest even
 // with its two's complement in the low mantissa bits, two elements per instruction and no conversion.
 template <int FMT, bool GUARD = false>
-__device__ __forceinline__ uint32_t quant_bf16_pair(uint32_t w, const QuotientPair& quot) {
+__device__ __forceinline__ uint32_t quant_bits_pair(uint32_t b0, uint32_t b1, const QuotientPair& quot) {
   uint64_t x2;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(x2) : "r"(w << 16), "r"(w & 0xffff0000u));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(x2) : "r"(b0), "r"(b1));
   const uint64_t q2 = quot(x2);
   uint32_t q0, q1;
   asm("mov.b64 {%0, %1}, %2;" : "=r"(q0), "=r"(q1) : "l"(q2));
   if (GUARD) {
-    q0 = __float_as_uint(fminf(fabsf(__uint_as_float(q0)), 3.402823466e38f)) | ((w << 16) & 0x80000000u);
-    q1 = __float_as_uint(fminf(fabsf(__uint_as_float(q1)), 3.402823466e38f)) | (w & 0x80000000u);
+    q0 = __float_as_uint(fminf(fabsf(__uint_as_float(q0)), 3.402823466e38f)) | (b0 & 0x80000000u);
+    q1 = __float_as_uint(fminf(fabsf(__uint_as_float(q1)), 3.402823466e38f)) | (b1 & 0x80000000u);
     return quant2<FMT>(__uint_as_float(q0), __uint_as_float(q1));
   }
   if (FMT == QM_FMT_INT8) {
@@ -179,10 +180,19 @@ __device__ __forceinline__ uint32_t quant_bf16_pair(uint32_t w, const QuotientPa
     return __byte_perm(q0, q1, 0x0040);                     // (the upper half is not looked at)
   } else {
     // a negative input that rounds to zero is -0 in the FP8 formats: give the quotient its sign back
-    q0 |= (w << 16) & 0x80000000u;
-    q1 |= w & 0x80000000u;
+    q0 |= b0 & 0x80000000u;
+    q1 |= b1 & 0x80000000u;
     return quant2<FMT>(__uint_as_float(q0), __uint_as_float(q1));
   }
+}
+template <int FMT, bool GUARD = false>
+__device__ __forceinline__ uint32_t quant_bf16_pair(uint32_t w, const QuotientPair& quot) {
+  return quant_bits_pair<FMT, GUARD>(w << 16, w & 0xffff0000u, quot);
+}
+// Two codes of two fp32 values, the upper half clear.
+template <int FMT, bool GUARD = false>
+__device__ __forceinline__ uint32_t quant_pair_x2(float x0, float x1, const QuotientPair& quot) {
+  return quant_bits_pair<FMT, GUARD>(__float_as_uint(x0), __float_as_uint(x1), quot) & 0xffffu;
 }
 
 // Four codes of the four bf16 values in two words.

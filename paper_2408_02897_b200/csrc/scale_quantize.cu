@@ -1,6 +1,8 @@
 // Scale (Eq. 1, right half) and quantize (Eq. 1, left half + saturation rule) kernels.
 // All of them are HBM-bound streaming kernels: 128-bit coalesced loads, warp-shuffle and
 // shared-memory reductions, one atomicMax per block and group.
+#include <algorithm>
+
 #include "quant_device.cuh"
 
 namespace qm {
@@ -402,6 +404,108 @@ __device__ __forceinline__ void multi_scales(const uint32_t* amax, const MultiOu
   }
 }
 
+// ---------------------------------------------------------------- sixteen elements as they come
+template <typename T> struct Piece;
+template <> struct Piece<__nv_bfloat16> {
+  uint4 w[2];
+  __device__ __forceinline__ void load(const __nv_bfloat16* p, bool wide) {
+    if (wide) { const Vec256 v = ld256<false>(p); w[0] = v.lo; w[1] = v.hi; }
+    else { w[0] = __ldg(reinterpret_cast<const uint4*>(p)); w[1] = __ldg(reinterpret_cast<const uint4*>(p) + 1); }
+  }
+  __device__ __forceinline__ void zero() { w[0] = w[1] = make_uint4(0u, 0u, 0u, 0u); }
+  __device__ __forceinline__ uint32_t absmax() const {    // as an fp32 bit pattern
+    const uint32_t k = 0x7fff7fffu;
+    uint32_t m = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      m = __vmaxu2(m, __vmaxu2(__vmaxu2(w[h].x & k, w[h].y & k), __vmaxu2(w[h].z & k, w[h].w & k)));
+    return max(m & 0xffffu, m >> 16) << 16;
+  }
+  template <int FMT, bool GUARD = false> __device__ __forceinline__ uint4 quant(const QuotientPair& qp) const { return quant_bf16x16<FMT, GUARD>(w[0], w[1], qp); }
+  __device__ __forceinline__ float at(int i) const {
+    const uint4 v = w[i >> 3];
+    const uint32_t x = (i >> 1 & 3) == 0 ? v.x : (i >> 1 & 3) == 1 ? v.y : (i >> 1 & 3) == 2 ? v.z : v.w;
+    return i & 1 ? bf16_hi(x) : bf16_lo(x);
+  }
+};
+template <> struct Piece<float> {
+  float4 w[4];
+  __device__ __forceinline__ void load(const float* p, bool) {
+#pragma unroll
+    for (int h = 0; h < 4; ++h) w[h] = __ldg(reinterpret_cast<const float4*>(p) + h);
+  }
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int h = 0; h < 4; ++h) w[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  __device__ __forceinline__ uint32_t absmax() const {
+    uint32_t m = 0;
+#pragma unroll
+    for (int h = 0; h < 4; ++h)
+      m = max(m, max(max(absbits_f32(__float_as_uint(w[h].x)), absbits_f32(__float_as_uint(w[h].y))),
+                     max(absbits_f32(__float_as_uint(w[h].z)), absbits_f32(__float_as_uint(w[h].w)))));
+    return m;
+  }
+  template <int FMT, bool GUARD = false> __device__ __forceinline__ uint4 quant(const QuotientPair& qp) const {
+    uint32_t c[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h)
+      c[h] = quant_pair_x2<FMT, GUARD>(w[h].x, w[h].y, qp) | quant_pair_x2<FMT, GUARD>(w[h].z, w[h].w, qp) << 16;
+    return make_uint4(c[0], c[1], c[2], c[3]);
+  }
+  __device__ __forceinline__ float at(int i) const {
+    const float4 v = w[i >> 2];
+    return (i & 3) == 0 ? v.x : (i & 3) == 1 ? v.y : (i & 3) == 2 ? v.z : v.w;
+  }
+};
+
+// ---------------------------------------------------------------- quantize, lines of any length and pitch under one scale
+// What the dense kernels do not take: bf16 rows that are no multiple of 16 long or lie apart, and fp32.  A thread takes
+// sixteen elements of a line, every format in MASK, with the two-wide quotient; only a line's last piece is taken element
+// by element.  Bound by HBM; us, one element at a time and a launch per format / so: 13809 x 1234 bf16 E4M3 under a given
+// scale 18.9 / 15.6, three formats with their max|x| pass 73.0 / 57.7, fp32 16384 x 4096 62.6 / 53.6 and 251 / 130.
+template <typename T, int MASK, bool GUARD>
+__global__ void __launch_bounds__(kThreads)
+quantize_lines_kernel(const T* __restrict__ x, uint32_t total, int64_t c, int64_t s_nc, int64_t s_b, const FastDiv by_chunks,
+                      const FastDiv by_nc, const uint32_t* __restrict__ amax, const float* __restrict__ delta, const MultiOut o,
+                      int64_t ldc) {
+  pdl_prologue();
+  const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
+  if (i >= total) return;
+  const uint32_t row = by_chunks.div(i), ch = i - row * by_chunks.d, b = by_nc.div(row);
+  const int64_t k0 = (int64_t)ch * 16;
+  const T* src = x + (int64_t)b * s_b + (int64_t)(row - b * by_nc.d) * s_nc + k0;
+  const bool whole = k0 + 16 <= c;
+  Piece<T> p;
+  if (whole) p.load(src, false); else p.zero();
+  float d[3] = {1.f, 1.f, 1.f};
+  if (GUARD) {
+    const float given = __ldg(delta);
+#pragma unroll
+    for (int f = 0; f < 3; ++f) d[f] = given;
+  } else {
+    multi_scales<MASK>(amax, o, i == 0, d);
+  }
+#pragma unroll
+  for (int f = 0; f < 3; ++f) {
+    if (!(MASK & (1 << f))) continue;
+    uint4* dst = reinterpret_cast<uint4*>(o.codes[f] + (int64_t)row * ldc + k0);
+    if (whole && QuotientPair::serves(d[f])) {
+      const QuotientPair qp(d[f]);
+      *dst = f == 0 ? p.template quant<0, GUARD>(qp) : f == 1 ? p.template quant<1, GUARD>(qp) : p.template quant<2, GUARD>(qp);
+    } else {
+      const Quotient quot(d[f]);
+      uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+      for (int e = 0; e < 16; e += 2) {
+        const float t0 = quot(k0 + e < c ? Loader<T>::load1(src, e) : 0.f), t1 = quot(k0 + e + 1 < c ? Loader<T>::load1(src, e + 1) : 0.f);
+        w[e >> 2] |= (f == 0 ? quant2<0>(t0, t1) : f == 1 ? quant2<1>(t0, t1) : quant2<2>(t0, t1)) << (16 * (e >> 1 & 1));
+      }
+      *dst = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+  }
+}
+
 // Dense bf16 tensor, rows a multiple of 16 long: one flat run of 16-element chunks.
 template <int MASK, int CHUNKS, bool WIDE>
 __global__ void __launch_bounds__(kThreads)
@@ -781,6 +885,99 @@ scale_quantize_rows_reg_kernel(const __nv_bfloat16* __restrict__ x, int64_t nc, 
       const uint32_t m = 0x7fff7fffu;
       abs_copy[row * nvec + k] = make_uint4(v.x & m, v.y & m, v.z & m, v.w & m);
     }
+  }
+}
+
+// ---------------------------------------------------------------- fused per-row, a row spread over a group of warps
+// Rows of at most 512 W V elements (a multiple of 16), every format in MASK: W warps share a row, a thread holds V pieces of
+// sixteen elements of it, fetched with whole 256-bit loads (two 128-bit ones where rows do not start on 32 bytes) while the
+// row before is reduced and quantized; one 128-bit store of codes per piece and format.  Every element crosses the memory
+// system once.  Bound by HBM and instruction issue: what a thread does once per row (division, reciprocal, maxima) is why a
+// thread takes two pieces.  us, a warp per row that read it twice (L1) / so: 16384 x 4096 bf16 INT8 49.3 / 35.3 (one piece
+// 43.7), 4096 x 8192 39.9 / 20.0, 128 x 4096 6.7 / 3.0, 16384 x 2064 28.9 / 27.0; fp32 16384 x 4096 102 / 56, x 1024 24.3 / 17.9.
+// Bf16 rows of at most 1024 stay with a warp per row (768 11.4 / 12.5), fp32 rows below 272 too (256 31.8, 128 6.5 / 7.1).
+template <typename T, int MASK, int W, int V>
+__global__ void __launch_bounds__(kThreads)
+scale_quantize_rows_spread_kernel(const T* __restrict__ x, uint32_t rows, int pieces, int64_t s_nc, int64_t s_b, const FastDiv by_nc,
+                                  const MultiOut o, bool wide) {
+  pdl_prologue();
+  constexpr int kRowsPerBlock = 8 / W;
+  __shared__ __align__(16) uint32_t s_max[2][8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int group = warp / W, t = threadIdx.x - group * (32 * W);       // the row's group of warps, thread within it
+  const uint32_t step = gridDim.x * kRowsPerBlock;
+  auto fetch = [&](uint32_t row, Piece<T> (&p)[V]) {
+    const uint32_t b = by_nc.div(row);
+    const T* src = x + (int64_t)b * s_b + (int64_t)(row - b * by_nc.d) * s_nc;
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+      const int k = t + u * 32 * W;
+      if (k < pieces) p[u].load(src + (int64_t)k * 16, wide); else p[u].zero();
+    }
+  };
+  uint32_t row = blockIdx.x * kRowsPerBlock + group;
+  if (row >= rows) return;                                              // (whole groups)
+  Piece<T> next[V];
+  fetch(row, next);
+  for (uint32_t it = 0; row < rows; ++it) {
+    Piece<T> p[V];
+#pragma unroll
+    for (int u = 0; u < V; ++u) p[u] = next[u];
+    const uint32_t row_next = row + step;
+    if (row_next < rows && row_next > row) fetch(row_next, next);
+    uint32_t m = 0;
+#pragma unroll
+    for (int u = 0; u < V; ++u) m = max(m, p[u].absmax());
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (W > 1) {                                                        // two sets of slots: one barrier per row is enough
+      if (lane == 0) s_max[it & 1][warp] = m;
+      asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(32 * W) : "memory");
+      if (W == 2) {
+        const uint2 a = *reinterpret_cast<const uint2*>(&s_max[it & 1][group * W]);
+        m = max(a.x, a.y);
+      } else {
+#pragma unroll
+        for (int j = 0; j < W; j += 4) {
+          const uint4 a = *reinterpret_cast<const uint4*>(&s_max[it & 1][(group * W + j) & 4]);
+          m = max(max(m, max(a.x, a.y)), max(a.z, a.w));
+        }
+      }
+    }
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+      if (!(MASK & (1 << f))) continue;
+      const float d = m == 0 ? 1.0f : __fdiv_rn(__uint_as_float(m), fmt_qmax(f));
+      if (t == 0) {
+        o.delta_out[f][row] = d;
+        if (m >= 0x7f800000u && o.err_word[f]) atomicOr(o.err_word[f], QM_DEVERR_NONFINITE);
+      }
+      uint4* dst = reinterpret_cast<uint4*>(o.codes[f]) + (int64_t)row * pieces;
+      if (QuotientPair::serves(d)) {
+        const QuotientPair qp(d);                                       // the row's own scale: nothing can overflow
+#pragma unroll
+        for (int u = 0; u < V; ++u) {
+          const int k = t + u * 32 * W;
+          if (k < pieces) dst[k] = f == 0 ? p[u].template quant<0>(qp) : f == 1 ? p[u].template quant<1>(qp) : p[u].template quant<2>(qp);
+        }
+      } else {
+        const Quotient quot(d);
+#pragma unroll 1
+        for (int k = t, u = 0; k < pieces; k += 32 * W, ++u) {          // rare: scales outside 2^-60 .. 2^60, one piece at a time
+          const uint32_t b = by_nc.div(row);
+          Piece<T> q;
+          q.load(x + (int64_t)b * s_b + (int64_t)(row - b * by_nc.d) * s_nc + (int64_t)k * 16, false);
+          uint32_t c[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+          for (int i = 0; i < 16; i += 2) {
+            const float t0 = quot(q.at(i)), t1 = quot(q.at(i + 1));
+            c[i >> 2] |= (f == 0 ? quant2<0>(t0, t1) : f == 1 ? quant2<1>(t0, t1) : quant2<2>(t0, t1)) << (16 * (i >> 1 & 1));
+          }
+          dst[k] = make_uint4(c[0], c[1], c[2], c[3]);
+        }
+      }
+    }
+    if (row_next <= row) break;                                         // (32-bit wrap)
+    row = row_next;
   }
 }
 
@@ -1388,6 +1585,17 @@ qm_status quantize_t(const View& x, int gran, const float* delta, bool from_amax
       if (big) { if (wide) QM_QD(4, true); else QM_QD(4, false); }
       else { if (wide) QM_QD(1, true); else QM_QD(1, false); }
 #undef QM_QD
+    } else if (!ds.per_channel && !rnd.stochastic && !abs_copy) {
+      MultiOut o{};
+      o.codes[FMT] = codes; o.delta_out[FMT] = delta_out; o.err_word[FMT] = err_word;
+      const dim3 grid((unsigned)((total + kThreads - 1) / kThreads));
+      const FastDiv by_chunks((uint32_t)(ldc >> 4)), by_nc((uint32_t)x.nc);
+      if (from_amax)
+        launch_pdl(quantize_lines_kernel<T, 1 << FMT, false>, grid, dim3(kThreads), 0, s, p, (uint32_t)total, x.c, x.s_nc, x.s_b, by_chunks,
+                   by_nc, reinterpret_cast<const uint32_t*>(delta), nullptr, o, ldc);
+      else
+        launch_pdl(quantize_lines_kernel<T, 1 << FMT, true>, grid, dim3(kThreads), 0, s, p, (uint32_t)total, x.c, x.s_nc, x.s_b, by_chunks,
+                   by_nc, nullptr, delta, o, ldc);
     } else
     launch_pdl(quantize_rows_kernel<T, FMT>, dim3(grid_for(total, 16)), dim3(kThreads), 0, s, 
         p, x.nc, x.c, x.s_nc, x.batch, x.s_b, ds, FastDiv((uint32_t)(ldc >> 4)), FastDiv((uint32_t)x.nc),
@@ -1436,12 +1644,49 @@ qm_status quantize_t(const View& x, int gran, const float* delta, bool from_amax
   return QM_OK;
 }
 
+// Rows that the spread kernel takes: codes without padding, at most 8192 elements.  Short rows leave its lanes idle or, in
+// bf16, have no more of them than one warp holds: those kernels are faster there, for one format.
+bool rows_spread(const View& x, int formats) {
+  const int64_t least = formats > 1 ? 16 : x.dtype == QM_DT_BF16 ? 1040 : 272;
+  return (x.c & 15) == 0 && x.c >= least && x.c <= 8192 && x.nc * x.batch < (1ll << 31) && x.nc < (1ll << 31);
+}
+template <typename T, int MASK>
+qm_status rows_spread_t(const View& x, const MultiOut& o, cudaStream_t s) {
+  const uint32_t rows = (uint32_t)(x.nc * x.batch);
+  const int pieces = (int)(x.c / 16);
+  const bool wide = ((reinterpret_cast<uintptr_t>(x.data) | (uintptr_t)(x.s_nc * sizeof(T)) | (x.batch > 1 ? (uintptr_t)(x.s_b * sizeof(T)) : 0)) & 31) == 0;
+#define QM_SP(W, V)                                                                                                        \
+  launch_pdl(scale_quantize_rows_spread_kernel<T, MASK, W, V>, dim3((unsigned)std::min<int64_t>((rows + 8 / W - 1) / (8 / W), 8ll * sm_count())), \
+             dim3(kThreads), 0, s, static_cast<const T*>(x.data), rows, pieces, x.s_nc, x.s_b, FastDiv((uint32_t)x.nc), o, wide)
+  if constexpr (sizeof(T) == 2) {
+    if (pieces <= 64) QM_SP(1, 2);
+    else if (pieces <= 128) QM_SP(2, 2);
+    else if (pieces <= 256) QM_SP(4, 2);
+    else QM_SP(8, 2);
+  } else {
+    if (pieces <= 32) QM_SP(1, 1);
+    else if (pieces <= 64) QM_SP(2, 1);
+    else if (pieces <= 128) QM_SP(4, 1);
+    else if (pieces <= 256) QM_SP(8, 1);
+    else QM_SP(8, 2);
+  }
+#undef QM_SP
+  count_launch();
+  QM_CUDA_OK(cudaGetLastError());
+  return QM_OK;
+}
+
 template <typename T, int FMT>
 qm_status scale_quantize_rows_t(const View& x, float* delta_out, uint8_t* codes, void* abs_copy,
                                 uint32_t* err_word, cudaStream_t s) {
   const T* p = static_cast<const T*>(x.data);
   const int64_t rows = x.nc * x.batch, ldc = qm_code_ld(x.c), nvec = x.c / 8;
   const float qmax = fmt_qmax(FMT);
+  if (!abs_copy && rows_spread(x, 1)) {
+    MultiOut o{};
+    o.codes[FMT] = codes; o.delta_out[FMT] = delta_out; o.err_word[FMT] = err_word;
+    return rows_spread_t<T, 1 << FMT>(x, o, s);
+  }
   if (x.dtype == QM_DT_BF16 && (x.c & 15) == 0 && x.c <= 4 * 256) {
     // the row fits in one warp's registers
     const unsigned blocks = (unsigned)((rows * 32 + kThreads - 1) / kThreads);
@@ -1615,12 +1860,12 @@ qm_status launch_quantize_multi(const View& x, int gran, const uint32_t* amax, i
     mask |= 1 << f;
     o.codes[f] = codes[k]; o.delta_out[f] = delta_out[k]; o.err_word[f] = err_word[k];
   }
-  bool one_pass = nf > 1 && gran == QM_GRAN_TENSOR && x.dtype == QM_DT_BF16;
+  bool one_pass = nf > 1 && gran == QM_GRAN_TENSOR && (x.dtype == QM_DT_BF16 || x.c_contig());
   const int64_t total = x.nc * x.batch * (ldc >> 4);
   bool dense = false, transposing = false;
   if (one_pass && x.c_contig()) {
-    dense = x.s_nc == x.c && (x.c & 15) == 0 && (x.batch == 1 || x.s_b == x.nc * x.c) && total < (1ll << 32);
-    one_pass = dense && !kmaj_copy;
+    dense = x.dtype == QM_DT_BF16 && x.s_nc == x.c && (x.c & 15) == 0 && (x.batch == 1 || x.s_b == x.nc * x.c);
+    one_pass = total < (1ll << 32) && x.nc < (1ll << 32) && !kmaj_copy;
   } else if (one_pass) {
     transposing = tile_transposable(x);
     one_pass = transposing;
@@ -1652,6 +1897,23 @@ qm_status launch_quantize_multi(const View& x, int gran, const uint32_t* amax, i
       default: QM_DM(7); break;
     }
 #undef QM_DM
+  } else if (!transposing) {
+    const dim3 grid((unsigned)((total + kThreads - 1) / kThreads));
+    const FastDiv by_chunks((uint32_t)(ldc >> 4)), by_nc((uint32_t)x.nc);
+    const float* none = nullptr;
+#define QM_LM(M)                                                                                                          \
+  (x.dtype == QM_DT_BF16                                                                                                  \
+       ? launch_pdl(quantize_lines_kernel<__nv_bfloat16, M, false>, grid, dim3(kThreads), 0, s, static_cast<const __nv_bfloat16*>(x.data), \
+                    (uint32_t)total, x.c, x.s_nc, x.s_b, by_chunks, by_nc, amax, none, o, ldc)                            \
+       : launch_pdl(quantize_lines_kernel<float, M, false>, grid, dim3(kThreads), 0, s, static_cast<const float*>(x.data), (uint32_t)total, \
+                    x.c, x.s_nc, x.s_b, by_chunks, by_nc, amax, none, o, ldc))
+    switch (mask) {
+      case 3: QM_LM(3); break;
+      case 5: QM_LM(5); break;
+      case 6: QM_LM(6); break;
+      default: QM_LM(7); break;
+    }
+#undef QM_LM
   } else {
     const __nv_bfloat16* src = static_cast<const __nv_bfloat16*>(x.data);
     __nv_bfloat16* km = static_cast<__nv_bfloat16*>(kmaj_copy);
@@ -1703,6 +1965,32 @@ qm_status launch_quantize_cols(const View& x, const uint32_t* amax, int nf, cons
   count_launch();
   QM_CUDA_OK(cudaGetLastError());
   return QM_OK;
+}
+
+qm_status launch_scale_quantize_rows_multi(const View& x, int nf, const int* fmts, float* const* delta_out,
+                                           uint32_t* const* err_word, uint8_t* const* codes, cudaStream_t s) {
+  if (nf < 1 || nf > 3) return QM_ERR_INVALID_ARG;
+  if (nf == 1 || x.dtype != QM_DT_BF16 || !rows_spread(x, nf)) {
+    for (int k = 0; k < nf; ++k) {
+      const qm_status st = launch_scale_quantize_rows(x, fmts[k], delta_out[k], codes[k], nullptr, err_word[k], s);
+      if (st != QM_OK) return st;
+    }
+    return QM_OK;
+  }
+  int mask = 0;
+  MultiOut o{};
+  for (int k = 0; k < nf; ++k) {
+    const int f = fmts[k];
+    if (f < 0 || f > 2 || (mask & (1 << f))) return QM_ERR_INVALID_ARG;
+    mask |= 1 << f;
+    o.codes[f] = codes[k]; o.delta_out[f] = delta_out[k]; o.err_word[f] = err_word[k];
+  }
+  switch (mask) {
+    case 3: return rows_spread_t<__nv_bfloat16, 3>(x, o, s);
+    case 5: return rows_spread_t<__nv_bfloat16, 5>(x, o, s);
+    case 6: return rows_spread_t<__nv_bfloat16, 6>(x, o, s);
+    default: return rows_spread_t<__nv_bfloat16, 7>(x, o, s);
+  }
 }
 
 qm_status launch_scale_quantize_rows(const View& x, int fmt, float* delta_out, uint8_t* codes,
