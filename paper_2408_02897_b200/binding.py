@@ -267,15 +267,29 @@ def _read_result(dev_buf):
     return MetricResult.from_buffer_copy(host)
 
 
+class _HostRecord:
+    """A result record in pinned host memory, which the last kernel of a call writes itself: reading it is a wait for
+    the stream, without a copy of its own."""
+
+    def __init__(self, kind):
+        self.kind = kind
+        self.buf = torch.empty(C.sizeof(kind), dtype=torch.uint8, pin_memory=True)
+        self.ptr = self.buf.data_ptr()
+
+    def read(self, stream):
+        (stream if stream is not None else torch.cuda.current_stream()).synchronize()
+        return self.kind.from_buffer_copy(C.string_at(self.ptr, C.sizeof(self.kind)))
+
+
 def qm_metric(ref, q, den, stream=None):
     """Eq. 3 record of three fp32 arrays of equal size."""
     n = ref.numel()
     L = lib()
     ws_bytes = L.qm_metric_workspace_bytes(n)
     ws = torch.empty(ws_bytes, dtype=torch.uint8, device="cuda")
-    out = torch.empty(C.sizeof(MetricResult), dtype=torch.uint8, device="cuda")
-    _check(L.qm_metric(_ptr(ref), _ptr(q), _ptr(den), n, _ptr(out), _ptr(ws), ws_bytes, _stream(stream)), "qm_metric")
-    return _read_result(out)
+    out = _HostRecord(MetricResult)
+    _check(L.qm_metric(_ptr(ref), _ptr(q), _ptr(den), n, out.ptr, _ptr(ws), ws_bytes, _stream(stream)), "qm_metric")
+    return out.read(stream)
 
 
 def qm_metric_noalloc(ref, q, den, out=None, stream=None):
@@ -297,9 +311,9 @@ def _stats_ws():
 def qm_tensor_stats(op, ws=None, stream=None):
     """Power sums and max|x| of a tensor -> TensorStats (synchronises to read the record)."""
     ws, n = (ws, ws.numel()) if ws is not None else _stats_ws()
-    out = torch.empty(C.sizeof(TensorStats), dtype=torch.uint8, device="cuda")
-    _check(lib().qm_tensor_stats(C.byref(op), _ptr(out), _ptr(ws), n, _stream(stream)), "qm_tensor_stats")
-    return TensorStats.from_buffer_copy(out.cpu().numpy().tobytes())
+    out = _HostRecord(TensorStats)
+    _check(lib().qm_tensor_stats(C.byref(op), out.ptr, _ptr(ws), n, _stream(stream)), "qm_tensor_stats")
+    return out.read(stream)
 
 
 def qm_quantize_error(op, fmt, gran, delta=None, ws=None, stream=None):
@@ -308,10 +322,10 @@ def qm_quantize_error(op, fmt, gran, delta=None, ws=None, stream=None):
     if delta is None:
         delta = qm_scale(op, fmt, gran, stream)
     ws, n = (ws, ws.numel()) if ws is not None else _stats_ws()
-    out = torch.empty(C.sizeof(QuantError), dtype=torch.uint8, device="cuda")
-    _check(lib().qm_quantize_error(C.byref(op), FMT[fmt], GRAN[gran], _ptr(delta), _ptr(out), _ptr(ws), n,
+    out = _HostRecord(QuantError)
+    _check(lib().qm_quantize_error(C.byref(op), FMT[fmt], GRAN[gran], _ptr(delta), out.ptr, _ptr(ws), n,
                                    _stream(stream)), "qm_quantize_error")
-    return QuantError.from_buffer_copy(out.cpu().numpy().tobytes())
+    return out.read(stream)
 
 
 ROUND = {"rtne": 0, "stochastic_l": 1, "stochastic_r": 2, "stochastic_both": 3}
@@ -391,9 +405,12 @@ def qm_probe_layer(L_op, R_op, fmt_l, fmt_r, gran_l, gran_r, ref="bf16", stream=
     """The whole probe for one product; returns the MetricResult (synchronises to read it).
     rounding: "rtne", or "stochastic_l" / "stochastic_r" / "stochastic_both" with `seed`.
     groups: batch_groups of (L, R) for channel scales shared along the batch (0 = not shared)."""
-    plan = ProbePlan(L_op, R_op, fmt_l, fmt_r, gran_l, gran_r, ref, rounding, seed, groups)
-    plan.launch(L_op, R_op, stream)
-    return plan.result()
+    cfg = _cfg(fmt_l, fmt_r, gran_l, gran_r, ref, rounding, seed, groups)
+    n = qm_workspace_bytes(L_op, R_op, fmt_l, fmt_r, gran_l, gran_r, ref)
+    ws = torch.empty(n, dtype=torch.uint8, device="cuda")
+    out = _HostRecord(MetricResult)
+    _check(lib().qm_probe_layer(C.byref(L_op), C.byref(R_op), C.byref(cfg), out.ptr, _ptr(ws), n, _stream(stream)), "qm_probe_layer")
+    return out.read(stream)
 
 
 def qm_probe_layer_host(L_host, R_host, contract_l, contract_r, fmt_l, fmt_r, gran_l, gran_r, ref="bf16",
