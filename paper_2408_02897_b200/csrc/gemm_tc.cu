@@ -113,9 +113,9 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() { cluster_arrive(); cluster_wait(); }
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
 }
@@ -1085,8 +1085,8 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 constexpr int kMaxVar = 6;                     // probes of one unit (three formats at two granularities)
 constexpr int kProbeThreads = 512;
 constexpr int kFirstEpiWarp = 8;               // warps 8..15: lane quarter = warp % 4 holds for both groups
-// registers per thread after the split (launch: 128 each): 56 + 104 + 176 + 176 = 4 x 128
-constexpr int kRegsCtl = 56, kRegsConv = 104, kRegsEpi = 176;
+// registers per thread after the split (launch: 128 each): 72 + 88 + 176 + 176 = 4 x 128
+constexpr int kRegsCtl = 72, kRegsConv = 88, kRegsEpi = 176;
 static_assert(kRegsCtl + kRegsConv + 2 * kRegsEpi <= 4 * 128, "the split must fit what the block was launched with");
 
 struct CfgP {
@@ -1100,6 +1100,18 @@ struct CfgP {
   static constexpr uint32_t kColRef = 0, kColDen = 128, kColLp = 256, kColL = 384;   // tensor-memory columns
 };
 
+// Division of a tile's position (below 2^31) by a number of tiles without a divide instruction: with 2^(s-1) < d <= 2^s and
+// mul = floor(2^(31+s) / d) + 1 the quotient of n is the upper half of 2 n mul, shifted right by s (the excess of mul adds less
+// than 1 / d for such n).
+struct Divisor {
+  uint32_t mul, shift;
+  __host__ explicit Divisor(uint32_t d) : shift(0) {
+    while ((1ull << shift) < d) ++shift;
+    mul = (uint32_t)((1ull << (31 + shift)) / d + 1);
+  }
+};
+__device__ __forceinline__ uint32_t divide(uint32_t n, uint32_t mul, uint32_t shift) { return __umulhi(n << 1, mul) >> shift; }
+
 // What the roles need of a unit for every tile, copied to shared memory once per CTA: the
 // launch's table sits in the kernel's parameter space, and reads of it with an index known only
 // at run time go through the small constant cache, which a table of this size thrashes.
@@ -1107,6 +1119,7 @@ struct alignas(16) WalkInfo {
   int32_t tile_begin, per_b, inner, num_kb;         // per_b = tiles_m * tiles_n (tiles per batch element);
                                                     // inner = tiles_n: column tiles run fastest, -tiles_m: row tiles do
   int32_t half_n, n_var, var_begin, K;              // half_n: kUnitMnMajor... above its low byte
+  uint32_t b_mul, b_shift, i_mul, i_shift;          // division by per_b and by the absolute value of inner (Divisor)
 };
 struct VarInfo { uint32_t idesc, flags; };
 enum : uint32_t { kVarI8 = 1, kVarScalePerRow = 2, kVarScalePerCol = 4, kVarRowStats = 8, kVarMnMajorL = 16, kVarMnMajorR = 32 };
@@ -1146,6 +1159,7 @@ struct GroupUnit {
   int32_t half_n;             // right-operand rows each CTA stages: 64, or 32 for outputs at most 64 wide
   int32_t m_fastest;          // the tiles of a batch element are walked down the rows first (below)
   uint32_t major;             // kUnitMnMajor...: bf16 operands stored with the contraction strided
+  uint32_t b_mul, b_shift, i_mul, i_shift;   // see WalkInfo
   int32_t var_begin, n_var;
 };
 struct GroupVar {
@@ -1209,11 +1223,12 @@ struct TileWalk {
       while (pi + 1 < n && pos >= wk[pi + 1].tile_begin) ++pi;
       const int4 w4 = reinterpret_cast<const int4*>(&wk[pi])[0];        // tile_begin, per_b, inner, num_kb
       const int4 x4 = reinterpret_cast<const int4*>(&wk[pi])[1];        // half_n, n_var, var_begin, K
-      const int t = pos - w4.x;
-      tc.b = t / w4.y;
-      const int rem = t - tc.b * w4.y;
+      const uint4 d4 = reinterpret_cast<const uint4*>(&wk[pi])[2];
+      const uint32_t t = (uint32_t)(pos - w4.x), b = divide(t, d4.x, d4.y);
+      tc.b = (int)b;
+      const uint32_t rem = t - b * (uint32_t)w4.y;
       const int inner = w4.z < 0 ? -w4.z : w4.z;
-      const int outer_i = rem / inner, inner_i = rem - outer_i * inner;
+      const int outer_i = (int)divide(rem, d4.z, d4.w), inner_i = (int)rem - outer_i * inner;
       tc.m_tile = w4.z < 0 ? inner_i : outer_i;
       tc.n_tile = w4.z < 0 ? outer_i : inner_i;
       num_kb = w4.w;
@@ -1420,41 +1435,68 @@ __device__ __forceinline__ void fill_walk(Sh* sh, const Table& tab, int lane) {
     wi.inner = u.m_fastest ? -u.tiles_m : u.tiles_n;
     wi.num_kb = (u.K + kBlockK - 1) / kBlockK;
     wi.half_n = u.half_n | (int32_t)(u.major << 8); wi.n_var = u.n_var; wi.var_begin = u.var_begin; wi.K = u.K;
+    wi.b_mul = u.b_mul; wi.b_shift = u.b_shift; wi.i_mul = u.i_mul; wi.i_shift = u.i_shift;
     sh->walk[i] = wi;
   }
   for (int i = lane; i < tab.n_var; i += 32) sh->var[i] = VarInfo{tab.v[i].idesc_lp, tab.v[i].flags};
 }
 
+// Sums of four values over the warp, six exchanges instead of twenty: lanes 8 k .. 8 k + 7 return the sum of v[k].
+__device__ __forceinline__ double warp_sum4(double v0, double v1, double v2, double v3, int lane) {
+  const bool hi = lane & 16, odd = lane & 8;
+  double a = hi ? v2 : v0, b = hi ? v3 : v1;
+  a += __shfl_xor_sync(0xffffffffu, hi ? v0 : v2, 16);
+  b += __shfl_xor_sync(0xffffffffu, hi ? v1 : v3, 16);
+  double x = odd ? b : a;
+  x += __shfl_xor_sync(0xffffffffu, odd ? a : b, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+// Maximum of values that are not negative (nor NaN).
+__device__ __forceinline__ float warp_max_f(float x) { return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x))); }
+
 // Every record of the launch is visible (last CTA): epilogue warp ew takes probes ew, ew + 8, ...; fixed-order
-// sum (lane l takes records l, l + 32, ...).
+// sum (lane l takes records l, l + 32, ...).  One round trip to L2 per probe: 4 200 cycles with a trip for each 32
+// records and one per flag word.
 template <typename Table>
 __device__ __forceinline__ void write_results(const Table& tab, int ew, int lane) {
-  const uint32_t timed_out = tab.err0 ? (*reinterpret_cast<volatile uint32_t*>(tab.err0) & QM_DEVERR_TIMEOUT) : 0u;
+  constexpr int kTake = 5;                           // records of a lane on their way together: 160 in a warp
   for (int vi = ew; vi < tab.n_var; vi += kEpiWarps) {
     const GroupVar& a = tab.v[vi];
-    double s5[5] = {0, 0, 0, 0, 0};
-    for (int i = lane; i < (int)gridDim.x; i += 32) {
-      const double* rec = a.partials + (int64_t)i * kPartialDoubles;
-      s5[0] += __ldcg(rec); s5[1] = fmax(s5[1], __ldcg(rec + 1)); s5[2] += __ldcg(rec + 2);
-      s5[3] += __ldcg(rec + 3); s5[4] += __ldcg(rec + 4);
-    }
+    // four lanes fetch the words that make up the record's flags
+    const uint32_t* word = lane == 0 ? a.err_word : lane == 1 ? a.err_also[0] : lane == 2 ? a.err_also[1] : lane == 3 ? tab.err0 : nullptr;
+    uint32_t flags = word ? *reinterpret_cast<const volatile uint32_t*>(word) : 0u;
+    if (lane == 3) flags &= QM_DEVERR_TIMEOUT;
+    double s4[4] = {0, 0, 0, 0};
+    float mx = 0.f;
+    for (int i0 = lane; i0 < (int)gridDim.x; i0 += 32 * kTake) {
+      double r[kTake][kPartialDoubles];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      s5[0] += __shfl_xor_sync(0xffffffffu, s5[0], o);
-      s5[1] = fmax(s5[1], __shfl_xor_sync(0xffffffffu, s5[1], o));
-      s5[2] += __shfl_xor_sync(0xffffffffu, s5[2], o);
-      s5[3] += __shfl_xor_sync(0xffffffffu, s5[3], o);
-      s5[4] += __shfl_xor_sync(0xffffffffu, s5[4], o);
+      for (int u = 0; u < kTake; ++u) {
+        const int i = i0 + 32 * u;
+        const double* rec = a.partials + (int64_t)i * kPartialDoubles;
+#pragma unroll
+        for (int k = 0; k < kPartialDoubles; ++k) r[u][k] = i < (int)gridDim.x ? __ldcg(rec + k) : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < kTake; ++u) {
+        s4[0] += r[u][0]; s4[1] += r[u][2]; s4[2] += r[u][3]; s4[3] += r[u][4];
+        mx = fmaxf(mx, (float)r[u][1]);              // (a float that was widened)
+      }
     }
+    const double x = warp_sum4(s4[0], s4[1], s4[2], s4[3], lane);
+    mx = warp_max_f(mx);
+    flags = __reduce_or_sync(0xffffffffu, flags);
     if (lane == 0) {
-      a.result->sum_be = s5[0]; a.result->max_be = s5[1]; a.result->sum_diff2 = s5[2];
-      a.result->sum_ref2 = s5[3]; a.result->sum_den2 = s5[4];
-      a.result->count = a.count;
-      uint32_t flags = (a.err_word ? *reinterpret_cast<volatile uint32_t*>(a.err_word) : 0u) | timed_out;
-      for (int k = 0; k < 2; ++k)
-        if (a.err_also[k]) flags |= *reinterpret_cast<const volatile uint32_t*>(a.err_also[k]);
-      a.result->device_error = flags;
-      a.result->reserved = 0;
+      a.result->sum_be = x; a.result->max_be = (double)mx;
+      a.result->count = a.count; a.result->device_error = flags; a.result->reserved = 0;
+    } else if (lane == 8) {
+      a.result->sum_diff2 = x;
+    } else if (lane == 16) {
+      a.result->sum_ref2 = x;
+    } else if (lane == 24) {
+      a.result->sum_den2 = x;
     }
   }
 }
@@ -1496,7 +1538,8 @@ __device__ __forceinline__ void probe_exit(Sh* sh, uint64_t wait_limit_ns, int w
   }
 }
 
-template <typename Table>
+// MN: units may have operands whose contraction is strided.
+template <typename Table, bool MN>
 __global__ void __launch_bounds__(kProbeThreads, 1)
 tc_group_kernel(const __grid_constant__ Table tab) {
   using C = CfgP;
@@ -1554,17 +1597,25 @@ tc_group_kernel(const __grid_constant__ Table tab) {
   tc_fence_before();
   __syncthreads();
   __syncwarp();
-  cluster_sync();          // the peer's barriers and tensor memory exist before anyone uses them
-  pdl_prologue();          // everything above overlapped the tail of the previous kernel
+  cluster_arrive();
   tc_fence_after();
   const uint32_t tmem_base = sh->tmem_base;
+  // every warp: the pair's first tile, found while the cluster barrier completes
+  auto begin = [&](TileWalk& tw) {
+    tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
+    __syncwarp();
+    cluster_wait();        // the peer's barriers and tensor memory exist before anyone uses them
+    pdl_prologue();        // everything above overlapped the tail of the previous kernel
+    tc_fence_after();
+  };
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsCtl));
     if (warp == 0) {
       // ---------------------------------------------------------- TMA producer (both CTAs)
+      TileWalk tw;
+      begin(tw);
       if (lane == 0) {
-        TileWalk tw;
         Ring ring;
         uint32_t g = 0;
         bool ok = true;
@@ -1583,18 +1634,18 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           sh->issued = ++g;
           ring.next();
         };
-        for (tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs); tw.valid && ok; tw.next_tile()) {
+        for (; tw.valid && ok; tw.next_tile()) {
           const int r0 = tw.tc.m_tile * kPairM + (int)rank * kBlockM;     // this CTA's left-operand rows
           const int c0 = tw.tc.n_tile * kBlockN + (int)rank * tw.half_n;  // this CTA's half of the right operand
           const uint32_t bytes = kABf16 + (uint32_t)tw.half_n * 128u;
-          const bool l_mn = tw.major & kUnitMnMajorL, r_mn = tw.major & kUnitMnMajorR;
+          const bool l_mn = MN && (tw.major & kUnitMnMajorL), r_mn = MN && (tw.major & kUnitMnMajorR);
           for (int kb = 0; kb < tw.num_kb && ok; ++kb)
             load(tab.u[tw.pi].maps, bytes, kb * kBlockK, r0, c0, tw.tc.b, l_mn, r_mn, l_mn);
           const int nb = tw.lp_blocks();
           for (int f = 0; f < tw.n_var && ok; ++f) {
             const uint32_t flags = sh->var[tw.var_begin + f].flags;
             for (int kb = 0; kb < nb && ok; ++kb)
-              load(tab.v[tw.var_begin + f].maps, bytes, kb * C::kLpDepth, r0, c0, tw.tc.b, flags & kVarMnMajorL, flags & kVarMnMajorR, false);
+              load(tab.v[tw.var_begin + f].maps, bytes, kb * C::kLpDepth, r0, c0, tw.tc.b, MN && (flags & kVarMnMajorL), MN && (flags & kVarMnMajorR), false);
           }
         }
       }
@@ -1602,6 +1653,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
       // ---------------------------------------------------------- MMA issuer (leader CTA, converged warp)
       const bool lead = elect_one();
       TileWalk tw;
+      begin(tw);
       Ring ring;
       auto wait_block = [&]() {
         if (!w.wait_warp(smem_u32(&sh->ready[ring.s]), ring.parity)) return false;
@@ -1635,13 +1687,13 @@ tc_group_kernel(const __grid_constant__ Table tab) {
       uint32_t lp_uses0 = 0, lp_uses1 = 0;           // variants put into each 8-bit accumulator so far
       bool ok = true;
       uint32_t it = 0;
-      for (tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs); tw.valid && ok; ++it, tw.next_tile()) {
+      for (; tw.valid && ok; ++it, tw.next_tile()) {
         // the reference and denominator blocks come back when both epilogues have copied the
         // previous tile's values out
         if (it > 0 && !w.wait_warp(smem_u32(&sh->rd_empty), (it - 1) & 1)) break;
         tc_fence_after();
         tw.make_uniform();
-        const bool r_mn = tw.major & kUnitMnMajorR;          // (A comes from tensor memory, contraction-major always)
+        const bool r_mn = MN && (tw.major & kUnitMnMajorR);  // (A comes from tensor memory, contraction-major always)
         const uint32_t idesc_ref = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n) | (r_mn ? kIdescMnMajorB : 0u);
         rd = tile_desc(r_mn, r_mn ? 2u * tw.half_n : 128u, 16u, 16u);
         for (int kb = 0; kb < tw.num_kb; ++kb) {
@@ -1657,8 +1709,8 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           const int b = (tw.n_var - 1 - f) & 1;
           const uint32_t idesc = __shfl_sync(0xffffffffu, sh->var[tw.var_begin + f].idesc, 0);
           const uint32_t flags = __shfl_sync(0xffffffffu, sh->var[tw.var_begin + f].flags, 0);
-          const bool is_i8 = flags & kVarI8, cr_mn = flags & kVarMnMajorR;
-          cl = tile_desc(flags & kVarMnMajorL, 128u, 32u, 16u);
+          const bool is_i8 = flags & kVarI8, cl_mn = MN && (flags & kVarMnMajorL), cr_mn = MN && (flags & kVarMnMajorR);
+          cl = tile_desc(cl_mn, 128u, 32u, 16u);
           cr = tile_desc(cr_mn, cr_mn ? tw.half_n : 128u, 32u, 16u);
           // both epilogues have read what this accumulator held; the second one's columns have also
           // been this tile's L, which the denominator MMAs must have finished with
@@ -1683,7 +1735,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
     } else if (warp >= 2) {
       // ---------------------------------------------------------- |R| (both CTAs)
       TileWalk tw;
-      tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
+      begin(tw);
       const int t = (warp - 2) * 32 + lane;        // 0..63
       const uint32_t ready_leader = map_to_cta(smem_u32(&sh->ready[0]), 0);
       Ring ring;
@@ -1705,6 +1757,9 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           ring.next();
         }
       }
+    } else {
+      TileWalk tw;
+      begin(tw);
     }
   } else if (warp < kFirstEpiWarp) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsConv));
@@ -1722,17 +1777,18 @@ tc_group_kernel(const __grid_constant__ Table tab) {
     const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + C::kColL;
     const uint32_t row_off = (uint32_t)t * 128u, sw = (uint32_t)t & 7u, m = 0x7fff7fffu;
     TileWalk tw;
+    begin(tw);
     Ring ring;
     uint32_t it = 0, abs_uses = 0;                 // completions of abs_free awaited so far
     bool lent = false;                             // the previous tile's variants have used the L columns
     bool ok = true;
-    for (tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs); tw.valid && ok; ++it, tw.next_tile()) {
+    for (; tw.valid && ok; ++it, tw.next_tile()) {
       // the L columns are free once the previous tile's denominator is complete and whatever
       // variants it put there have been read
       if (it > 0) ok = w.wait_warp(smem_u32(&sh->rd_full), (it - 1) & 1);
       if (ok && lent) ok = w.wait_warp(smem_u32(&sh->abs_free), abs_uses++ & 1);
       lent = tw.n_var > 1;
-      const bool l_mn = tw.major & kUnitMnMajorL;
+      const bool l_mn = MN && (tw.major & kUnitMnMajorL);
       // a loop for each order of L: one loop with the choice inside cost the contraction-major one 7 %
       auto convert = [&](auto mn) {
         constexpr bool kMn = decltype(mn)::value;
@@ -1781,7 +1837,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           ring.next();
         }
       };
-      if (l_mn) convert(std::true_type{}); else convert(std::false_type{});
+      if (l_mn) convert(std::bool_constant<MN>{}); else convert(std::false_type{});
       // blocks of codes: only passed on
       const int n_code_blocks = tw.n_var * tw.lp_blocks();
       for (int kb = 0; kb < n_code_blocks && ok; ++kb) {
@@ -1807,20 +1863,19 @@ tc_group_kernel(const __grid_constant__ Table tab) {
     // reduce the statistics of unit `pi` over the CTA and write its records (all 256 threads call)
     auto flush = [&](int pi) {
       const int nv = sh->walk[pi].n_var, v0 = sh->walk[pi].var_begin;
-      for (int i = 0; i < 3 * nv + 2; ++i) {
-        // values 3v, 3v + 1, 3v + 2: sum BE, max BE, sum diff^2 of variant v; the last two: sum C^2, D^2
-        const int v = i / 3, k = i - 3 * v;
-        double x = 0.0;
-        if (i >= 3 * nv) x = i == 3 * nv ? acc_r2 : acc_n2;
-        else if (lane < 16) x = k == 1 ? (double)sh->maxima[v][ew][lane] : (k == 0 ? sh->sums[v][ew][lane].x : sh->sums[v][ew][lane].y);
-        const bool is_max = i < 3 * nv && k == 1;
+      // values 3v, 3v + 1, 3v + 2: sum BE, max BE, sum diff^2 of variant v; the last two: sum C^2, D^2.  Half a warp adds up each
+      for (int v = 0; v < nv; ++v) {
+        const double2 a = sh->sums[v][ew][lane & 15];
+        double x = lane < 16 ? a.x : a.y;
+        const float mx = warp_max_f(sh->maxima[v][ew][lane & 15]);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const double y = __shfl_xor_sync(0xffffffffu, x, o);
-          x = is_max ? fmax(x, y) : x + y;
-        }
-        if (lane == 0) sh->red[i][ew] = x;
+        for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == 0) { sh->red[3 * v][ew] = x; sh->red[3 * v + 1][ew] = (double)mx; }
+        if (lane == 16) sh->red[3 * v + 2][ew] = x;
       }
+      const double rn = warp_sum4(acc_r2, acc_n2, 0.0, 0.0, lane);
+      if (lane == 0) sh->red[3 * nv][ew] = rn;
+      if (lane == 8) sh->red[3 * nv + 1][ew] = rn;
       acc_r2 = acc_n2 = 0.0;
       asm volatile("bar.sync 1, 256;" ::: "memory");
       if (et < 5 * nv) {
@@ -1829,7 +1884,6 @@ tc_group_kernel(const __grid_constant__ Table tab) {
         double x = 0.0;
         for (int j = 0; j < kEpiWarps; ++j) x = k == 1 ? fmax(x, sh->red[i][j]) : x + sh->red[i][j];
         __stcg(tab.v[v0 + v].partials + (int64_t)blockIdx.x * kPartialDoubles + k, x);
-        __threadfence();
       }
       asm volatile("bar.sync 1, 256;" ::: "memory");       // red[] may be reused
     };
@@ -1839,7 +1893,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
     uint32_t lp_parity = 0;                        // bit b: parity of the next use of 8-bit accumulator b
     bool dead = false;                             // a wait for an 8-bit accumulator ran out
     TileWalk tw;
-    tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
+    begin(tw);
     for (uint32_t it = 0; tw.valid; ++it) {
       const int pi = tw.pi, n_var = tw.n_var, v0 = tw.var_begin;
       if (pi != cur) {
@@ -1987,10 +2041,9 @@ tc_group_kernel(const __grid_constant__ Table tab) {
       if (et < 5 * sh->walk[pi].n_var)
         __stcg(tab.v[v0 + et / 5].partials + (int64_t)blockIdx.x * kPartialDoubles + et % 5, 0.0);
     }
-    __threadfence();
     asm volatile("bar.sync 1, 256;" ::: "memory");
     if (et == 0) {
-      __threadfence();
+      __threadfence();                            // after the barrier: covers the records that the other threads have written
       const uint32_t prev = atomicAdd(tab.done_counter, 1u);
       sh->is_last = prev == gridDim.x - 1 ? 1u : 0u;
     }
@@ -2006,34 +2059,38 @@ tc_group_kernel(const __grid_constant__ Table tab) {
 
 // ------------------------------------------------------------------ the fused probe kernel, one probe per unit
 // Units of one probe share nothing, so their three products run side by side, k-block by k-block: a stage
-// holds the bf16 and the code tiles of 64 contraction entries and one commit frees it.  96 KB go through shared
-// memory per k-block (36 by TMA, 28 of MMA operands, 32 by the converters), as for the products one after the other,
-// but a tile has no phases: the converters run ahead
+// holds the bf16 and the code tiles of 64 contraction entries and one commit frees it.  112 KB go through shared
+// memory per k-block (36 by TMA, 44 of MMA operands, 32 by the converters) against the 96 of the
+// products one after the other, but a tile has no phases: the converters run four blocks ahead
 // across its end, the next tile's reference and denominator MMAs start while this one's last columns are evaluated, and
 // the epilogue takes all three products in one sweep (the reciprocals beside the other arithmetic,
-// the sums in registers) with one wait.  Short contractions are bound by that chain.  Measured, the fused kernel
+// the sums in registers) with one wait.  Short contractions are bound by that chain, and by fetching its instructions: what
+// a tile runs once, all roles together, is more than the instruction cache holds beside the loops (512 x 512 x 64 x 256:
+// stalls for instructions per issue 1.1 -> 2.7 with the code for mn-major operands and integer divisions in the walk, 98 ->
+// 119 us; without either 102).  Measured, the fused kernel
 // alone, one after the other / side by side: 512 x 512 x 64 x 256 131 / 88 us; 8192 x 4096 with K = 128 75 / 53,
 // K = 256 76 / 64, K = 512 91 / 88, K = 1024 145 / 140.  With three probes per unit sharing wins from K = 64 on (187 / 239 us).
-// With L read from shared memory by the reference MMAs (112 KB) and |R| among the converters' work K = 1024 took 145 us, so
-// 136; 2048 x 3072 x 2048 69.7 / 63.6.
+// |R| by two warps of its own instead of the converters: 8192 x 4096 x 1024 149 / 139 us, 2048 x 3072 x 2048 76 / 69, 2048^2 x
+// 16384 357 / 300.  L from tensor memory as well (two stages of both, 96 KB) measured 140, 70 and 318, and 66 instead of
+// 60 at K = 192, where two blocks are not enough ahead.
 //   Roles, registers, walk and exit are those of tc_group_kernel.  Tensor memory: columns 0..127 reference, 128..255
-// denominator, 256..383 the 8-bit product, 384..511 two stages of L and |L| (32 columns of two bf16 each).
+// denominator, 256..383 the 8-bit product, 384..511 four stages of |L| (32 columns of two bf16 each).
 struct CfgS {
   static constexpr int kStages = 5;          // stages of shared memory (TMA ring)
-  static constexpr int kTmemStages = 2;       // stages of L and |L| in tensor memory (128 columns / 64)
+  static constexpr int kAbsStages = 4;       // stages of |L| in tensor memory (128 columns / 32)
   // stage: L, R, |R| (written by the converters), codes of L, codes of R
   static constexpr uint32_t kOffL = 0, kOffR = kABf16, kOffRa = kOffR + kBBf16, kOffCl = kOffRa + kBBf16;
   static constexpr uint32_t kOffCr = kOffCl + kALp;
   static constexpr uint32_t kStageBytes = kOffCr + kBLp;             // 44 KB
   static constexpr uint32_t kTileBytes = kStages * kStageBytes;      // 220 KB
-  static constexpr uint32_t kColRef = 0, kColDen = 128, kColLp = 256, kColL = 384;   // tensor-memory columns
+  static constexpr uint32_t kColRef = 0, kColDen = 128, kColLp = 256, kColAbsL = 384;   // tensor-memory columns
 };
 
 template <int UNITS>
 struct SharedS {
   uint64_t full[CfgS::kStages];     // per CTA: this CTA's loads of a stage have landed
   uint64_t ready[CfgS::kStages];    // leader: both CTAs' converters have seen their loads land and have written
-                                    //         L and |L| (tensor memory) and |R| (stage)
+                                    //         |L| (tensor memory) and |R| (stage)
   uint64_t empty[CfgS::kStages];    // per CTA: the pair's MMAs have finished with the k-block of the stage
   uint64_t tmem_full;               // per CTA: the tile's accumulators are complete
   uint64_t tmem_empty;              // leader: both CTAs' epilogues have copied out reference and denominator
@@ -2044,7 +2101,8 @@ struct SharedS {
   uint32_t is_last;
   uint32_t issued;                  // k-blocks whose loads the producer has issued (read on the give-up path)
   float delta_r[2][kBlockN];
-  double red[5][kEpiWarps];
+  double red[4][kEpiWarps];
+  float red_max[kEpiWarps];
   WalkInfo walk[UNITS];
   VarInfo var[UNITS];               // of unit i: it has one probe
 };
@@ -2109,12 +2167,13 @@ __device__ __forceinline__ void row_stats_add(double* rs, const StatsG& st) {
   unpack2(st.n2, x0, x1); atomicAdd(rs + 4, (double)x0 + (double)x1);
 }
 
-template <typename Table>
+// MN: units may have operands whose contraction is strided.
+template <typename Table, bool MN>
 __global__ void __launch_bounds__(kProbeThreads, 1)
 tc_side_kernel(const __grid_constant__ Table tab) {
   using C = CfgS;
   using Sh = SharedS<Table::kUnits>;
-  constexpr int kStages = C::kStages, kAbs = C::kTmemStages;
+  constexpr int kStages = C::kStages, kAbs = C::kAbsStages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   Sh* sh = reinterpret_cast<Sh*>(tiles + C::kTileBytes);
@@ -2158,27 +2217,35 @@ tc_side_kernel(const __grid_constant__ Table tab) {
   tc_fence_before();
   __syncthreads();
   __syncwarp();
-  cluster_sync();          // the peer's barriers and tensor memory exist before anyone uses them
-  pdl_prologue();          // everything above overlapped the tail of the previous kernel
+  cluster_arrive();
   tc_fence_after();
   const uint32_t tmem_base = sh->tmem_base;
+  // every warp: the pair's first tile, found while the cluster barrier completes
+  auto begin = [&](TileWalk& tw) {
+    tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
+    __syncwarp();
+    cluster_wait();        // the peer's barriers and tensor memory exist before anyone uses them
+    pdl_prologue();        // everything above overlapped the tail of the previous kernel
+    tc_fence_after();
+  };
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsCtl));
     if (warp == 0) {
       // ---------------------------------------------------------- TMA producer (both CTAs)
+      TileWalk tw;
+      begin(tw);
       if (lane == 0) {
-        TileWalk tw;
         uint32_t g = 0;
         bool ok = true;
-        for (tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs); tw.valid && ok; tw.next_tile()) {
+        for (; tw.valid && ok; tw.next_tile()) {
           const CUtensorMap* const um = tab.u[tw.pi].maps;
           const CUtensorMap* const vm = tab.v[tw.pi].maps;
           const int r0 = tw.tc.m_tile * kPairM + (int)rank * kBlockM;     // this CTA's left-operand rows
           const int c0 = tw.tc.n_tile * kBlockN + (int)rank * tw.half_n;  // this CTA's half of the right operand
           const uint32_t flags = sh->var[tw.pi].flags;
-          const bool l_mn = tw.major & kUnitMnMajorL, r_mn = tw.major & kUnitMnMajorR;
-          const bool cl_mn = flags & kVarMnMajorL, cr_mn = flags & kVarMnMajorR;
+          const bool l_mn = MN && (tw.major & kUnitMnMajorL), r_mn = MN && (tw.major & kUnitMnMajorR);
+          const bool cl_mn = MN && (flags & kVarMnMajorL), cr_mn = MN && (flags & kVarMnMajorR);
           for (int kb = 0; kb < tw.num_kb; ++kb, ++g) {
             const uint32_t s = g % kStages, use = g / kStages;
             // test hook: the consumers' waits run out
@@ -2199,17 +2266,17 @@ tc_side_kernel(const __grid_constant__ Table tab) {
     } else if (warp == 1 && rank == 0) {
       // ---------------------------------------------------------- MMA issuer (leader CTA, converged warp)
       const bool lead = elect_one();
-      uint32_t idesc_bf16 = 0;                 // of the tile in hand
-      TileDesc rd{}, cl{}, cr{};               // R and |R|; codes
+      uint32_t idesc_ref = 0, idesc_den = 0;   // of the tile in hand
+      TileDesc ld{}, rd{}, cl{}, cr{};         // L; R and |R|; codes
       auto issue_ref_den = [&](uint32_t gg, int kb) {
         const uint32_t s = gg % kStages, base = tile_base + s * C::kStageBytes;
-        const uint32_t ta = tmem_base + C::kColL + 64u * (gg % kAbs);
 #pragma unroll
         for (int k = 0; k < kBlockK / 16; ++k)   // 16 bf16 per step
-          mma_pair_a_tmem(tmem_base + C::kColRef, ta + 8u * k, rd.at(base + C::kOffR, k), idesc_bf16, (kb | k) != 0, lead);
+          mma_pair<kKindF16>(tmem_base + C::kColRef, ld.at(base + C::kOffL, k), rd.at(base + C::kOffR, k), idesc_ref, (kb | k) != 0, lead);
+        const uint32_t ta = tmem_base + C::kColAbsL + 32u * (gg % kAbs);
 #pragma unroll
         for (int k = 0; k < kBlockK / 16; ++k)   // 16 bf16 = 8 columns of tensor memory per step
-          mma_pair_a_tmem(tmem_base + C::kColDen, ta + 32u + 8u * k, rd.at(base + C::kOffRa, k), idesc_bf16, (kb | k) != 0, lead);
+          mma_pair_a_tmem(tmem_base + C::kColDen, ta + 8u * k, rd.at(base + C::kOffRa, k), idesc_den, (kb | k) != 0, lead);
       };
       auto issue_lp = [&](uint32_t gg, int kb, bool is_i8, uint32_t idesc_lp) {
         const uint32_t base = tile_base + (gg % kStages) * C::kStageBytes;
@@ -2226,7 +2293,7 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         return true;
       };
       TileWalk tw;
-      tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
+      begin(tw);
       uint32_t g = 0;
       bool ok = true;
       for (uint32_t it = 0; tw.valid && ok; ++it, tw.next_tile()) {
@@ -2234,12 +2301,15 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         const int num_kb = tw.num_kb;
         const uint32_t idesc_lp = __shfl_sync(0xffffffffu, sh->var[tw.pi].idesc, 0);
         const uint32_t flags = __shfl_sync(0xffffffffu, sh->var[tw.pi].flags, 0);
-        const bool is_i8 = flags & kVarI8, cr_mn = flags & kVarMnMajorR;
-        const bool r_mn = tw.major & kUnitMnMajorR;
-        // L and |L| come from tensor memory, contraction-major always
-        idesc_bf16 = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n) | (r_mn ? kIdescMnMajorB : 0u);
+        const bool is_i8 = flags & kVarI8;
+        const bool l_mn = MN && (tw.major & kUnitMnMajorL), r_mn = MN && (tw.major & kUnitMnMajorR);
+        const bool cl_mn = MN && (flags & kVarMnMajorL), cr_mn = MN && (flags & kVarMnMajorR);
+        // |L| comes from tensor memory, contraction-major always
+        idesc_den = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n) | (r_mn ? kIdescMnMajorB : 0u);
+        idesc_ref = idesc_den | (l_mn ? kIdescMnMajorA : 0u);
+        ld = tile_desc(l_mn, 128u, 16u, kABf16 / 2);
         rd = tile_desc(r_mn, r_mn ? 2u * tw.half_n : 128u, 16u, 16u);
-        cl = tile_desc(flags & kVarMnMajorL, flags & kVarMnMajorL ? 128u : 64u, 32u, 16u);
+        cl = tile_desc(cl_mn, cl_mn ? 128u : 64u, 32u, 16u);
         cr = tile_desc(cr_mn, cr_mn ? tw.half_n : 64u, 32u, 16u);
         // the reference and denominator blocks come back when both epilogues have copied the
         // previous tile's values out; the 8-bit block when they have finished that tile
@@ -2270,7 +2340,7 @@ tc_side_kernel(const __grid_constant__ Table tab) {
     } else if (warp >= 2) {
       // ---------------------------------------------------------- |R| (both CTAs)
       TileWalk tw;
-      tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
+      begin(tw);
       const int t = (warp - 2) * 32 + lane;        // 0..63
       const uint32_t ready_leader = map_to_cta(smem_u32(&sh->ready[0]), 0);
       bool ok = true;
@@ -2285,19 +2355,23 @@ tc_side_kernel(const __grid_constant__ Table tab) {
           if (++s == (uint32_t)kStages) { s = 0; parity ^= 1u; }
         }
       }
+    } else {
+      TileWalk tw;
+      begin(tw);
     }
   } else if (warp < kFirstEpiWarp) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsConv));
     // ------------------------------------------------------------ converters (both CTAs)
-    // As in tc_group_kernel, but the k-blocks are counted through over all tiles: the converters run up to
-    // kAbs blocks ahead of the MMAs across a tile's end.
+    // As in tc_group_kernel, but only |L| goes to tensor memory (the reference MMAs read L from shared memory),
+    // and the k-blocks are counted through over all tiles: the converters run up to kAbs blocks ahead
+    // of the MMAs across a tile's end.
     const int q = warp & 3;
     const int t = q * 32 + lane;                   // 0..127
     const uint32_t ready_leader = map_to_cta(smem_u32(&sh->ready[0]), 0);
-    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + C::kColL;
+    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + C::kColAbsL;
     const uint32_t row_off = (uint32_t)t * 128u, sw = (uint32_t)t & 7u;
     TileWalk tw;
-    tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
+    begin(tw);
     bool ok = true;
     uint32_t g = 0;
     // the blocks of one tile; a loop for each order of L: one loop with the choice inside cost the contraction-major one 7 %
@@ -2323,20 +2397,14 @@ tc_side_kernel(const __grid_constant__ Table tab) {
           if (!w.wait_warp(smem_u32(&sh->empty[gp % kStages]), (gp / kStages) & 1)) { ok = false; return; }
         }
         tc_fence_after();
-        const uint32_t tcol = taddr + 64u * (g % kAbs);
+        const uint32_t tcol = taddr + 32u * (g % kAbs);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) a[j] &= m;
         if constexpr (kMn) {
           tmem_st16x32(tcol, a);
           tmem_st16x32(tcol + (16u << 16), a + 16);
         } else {
           tmem_st32(tcol, a);
-        }
-#pragma unroll
-        for (int j = 0; j < 32; ++j) a[j] &= m;
-        if constexpr (kMn) {
-          tmem_st16x32(tcol + 32u, a);
-          tmem_st16x32(tcol + 32u + (16u << 16), a + 16);
-        } else {
-          tmem_st32(tcol + 32u, a);
         }
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         tc_fence_before();
@@ -2345,7 +2413,7 @@ tc_side_kernel(const __grid_constant__ Table tab) {
       }
     };
     for (; ok && tw.valid; tw.next_tile()) {
-      if (tw.major & kUnitMnMajorL) convert(std::true_type{}); else convert(std::false_type{});
+      if (MN && (tw.major & kUnitMnMajorL)) convert(std::bool_constant<MN>{}); else convert(std::false_type{});
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
@@ -2359,27 +2427,26 @@ tc_side_kernel(const __grid_constant__ Table tab) {
     const int h = ew >> 2;                         // which half of the tile's columns
     const int et = ew * 32 + lane;                 // 0..255
     const uint32_t tmem_empty_leader = map_to_cta(smem_u32(&sh->tmem_empty), 0);
-    double acc[5] = {0, 0, 0, 0, 0};               // of the unit in hand: sum BE, max BE, sum diff^2, C^2, D^2
+    double acc[4] = {0, 0, 0, 0};                  // of the unit in hand: sum BE, sum diff^2, C^2, D^2
+    float acc_max = 0.f;                           // and max BE
     int cur = -1;                                  // the unit in hand
     // reduce the statistics of unit `pi` over the CTA and write its record (all 256 threads call)
     auto flush = [&](int pi) {
-#pragma unroll
-      for (int i = 0; i < 5; ++i) {
-        double x = acc[i];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const double y = __shfl_xor_sync(0xffffffffu, x, o);
-          x = i == 1 ? fmax(x, y) : x + y;
-        }
-        if (lane == 0) sh->red[i][ew] = x;
-        acc[i] = 0.0;
-      }
+      const double x = warp_sum4(acc[0], acc[1], acc[2], acc[3], lane);
+      const float mx = warp_max_f(acc_max);
+      if ((lane & 7) == 0) sh->red[lane >> 3][ew] = x;
+      if (lane == 0) sh->red_max[ew] = mx;
+      acc[0] = acc[1] = acc[2] = acc[3] = 0.0;
+      acc_max = 0.f;
       asm volatile("bar.sync 1, 256;" ::: "memory");
-      if (et < 5) {
-        double x = 0.0;
-        for (int k = 0; k < kEpiWarps; ++k) x = et == 1 ? fmax(x, sh->red[et][k]) : x + sh->red[et][k];
-        __stcg(tab.v[pi].partials + (int64_t)blockIdx.x * kPartialDoubles + et, x);
-        __threadfence();
+      if (ew == 0) {                               // lanes 8 k .. 8 k + 7: the warps' sums of value k
+        double y = sh->red[lane >> 3][lane & 7];
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+        const float m = warp_max_f(sh->red_max[lane & 7]);
+        double* const rec = tab.v[pi].partials + (int64_t)blockIdx.x * kPartialDoubles;
+        if ((lane & 7) == 0) __stcg(rec + (lane == 0 ? 0 : (lane >> 3) + 1), y);
+        if (lane == 1) __stcg(rec + 1, (double)m);
       }
       asm volatile("bar.sync 1, 256;" ::: "memory");       // red[] may be reused
     };
@@ -2390,7 +2457,7 @@ tc_side_kernel(const __grid_constant__ Table tab) {
     int pM = 0, pN = 0;                            // a probe's M and N are below 2^31 (its tensor maps require it)
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
     TileWalk tw;
-    tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
+    begin(tw);
     for (uint32_t it = 0; tw.valid; ++it) {
       const int pi = tw.pi;
       if (pi != cur) {
@@ -2471,10 +2538,10 @@ tc_side_kernel(const __grid_constant__ Table tab) {
       if (row_ok) {
         float x0, x1;
         acc[0] += (double)st.be0 + (double)st.be1;
-        unpack2(st.d2, x0, x1); acc[2] += (double)x0 + (double)x1;
-        unpack2(st.r2, x0, x1); acc[3] += (double)x0 + (double)x1;
-        unpack2(st.n2, x0, x1); acc[4] += (double)x0 + (double)x1;
-        acc[1] = fmax(acc[1], (double)st.mx);
+        unpack2(st.d2, x0, x1); acc[1] += (double)x0 + (double)x1;
+        unpack2(st.r2, x0, x1); acc[2] += (double)x0 + (double)x1;
+        unpack2(st.n2, x0, x1); acc[3] += (double)x0 + (double)x1;
+        acc_max = fmaxf(acc_max, st.mx);
         double* const rows = tab.v[pi].row_stats;
         if (rows) row_stats_add(rows + ((int64_t)tc.b * pM + row) * 5, st);
       }
@@ -2685,9 +2752,11 @@ qm_status launch_wide(const CUtensorMap& ma, const CUtensorMap& mb, KernelArgs k
 
 namespace {
 // The two forms of the fused kernel: units of one probe, and units of several (see the kernels).
-template <bool SIDE, typename Table>
+// The two forms of the fused kernel, units of one probe (SIDE) and units of several, each with and without operands whose
+// contraction is strided: what those need is a third of the roles' code, and short tiles wait for instructions (below).
+template <bool SIDE, bool MN, typename Table>
 struct ProbeKernel {
-  static constexpr auto kernel = SIDE ? tc_side_kernel<Table> : tc_group_kernel<Table>;
+  static constexpr auto kernel = SIDE ? tc_side_kernel<Table, MN> : tc_group_kernel<Table, MN>;
   static constexpr size_t kSmem = 1024 + (SIDE ? (size_t)CfgS::kTileBytes + sizeof(SharedS<Table::kUnits>)
                                                : (size_t)CfgP::kTileBytes + sizeof(SharedP<Table::kUnits, Table::kVars>));
   static_assert(kSmem <= 232448, "shared memory of a CTA");
@@ -2718,10 +2787,13 @@ qm_status probe_kernel_ready() {
 qm_status probe_residency() {
   const int dev = current_device();
   if (dev < 0) return QM_ERR_UNSUPPORTED;
-  using Widest = ProbeKernel<false, TableBig>;
+  using Widest = ProbeKernel<false, true, TableBig>;
   qm_status as = probe_kernel_ready<Widest>();
-  if (as == QM_OK) as = probe_kernel_ready<ProbeKernel<true, TableBig>>();
-  if (as == QM_OK) as = probe_kernel_ready<ProbeKernel<true, TableOne>>();
+  if (as == QM_OK) as = probe_kernel_ready<ProbeKernel<false, false, TableBig>>();
+  if (as == QM_OK) as = probe_kernel_ready<ProbeKernel<true, true, TableBig>>();
+  if (as == QM_OK) as = probe_kernel_ready<ProbeKernel<true, true, TableOne>>();
+  if (as == QM_OK) as = probe_kernel_ready<ProbeKernel<true, false, TableBig>>();
+  if (as == QM_OK) as = probe_kernel_ready<ProbeKernel<true, false, TableOne>>();
   if (as != QM_OK) return as;
   if (g_max_pairs[dev] == 0) {
     cudaLaunchConfig_t q{};
@@ -2753,7 +2825,7 @@ bool same_products(const TcProbeArgs& a, const TcProbeArgs& b) {
          a.l_mn == b.l_mn && a.r_mn == b.r_mn && a.g.M == b.g.M && a.g.N == b.g.N && a.g.K == b.g.K && a.g.batch == b.g.batch;
 }
 
-template <bool SIDE, typename Table>
+template <bool SIDE, bool MN, typename Table>
 qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, cudaStream_t s) {
   static Table tab;                    // up to 29 KB: kept off the stack; guarded by the mutex below
   static std::mutex mu;
@@ -2791,6 +2863,8 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, cuda
     // streamed from HBM once and the smaller one is what gets fetched again (from L2, if it fits):
     // the tiles of a batch element are walked along the shorter side first.
     gu.m_fastest = g.M < g.N ? 1 : 0;
+    const Divisor by_b((uint32_t)(gu.tiles_m * gu.tiles_n)), by_inner((uint32_t)(gu.m_fastest ? gu.tiles_m : gu.tiles_n));
+    gu.b_mul = by_b.mul; gu.b_shift = by_b.shift; gu.i_mul = by_inner.mul; gu.i_shift = by_inner.shift;
     gu.var_begin = tab.n_var; gu.n_var = up.n_var;
     total += ka.num_tiles;
     for (int j = 0; j < up.n_var; ++j) {
@@ -2819,7 +2893,7 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, cuda
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(2 * (total < pairs ? total : pairs)));
   cfg.blockDim = dim3(kProbeThreads);
-  cfg.dynamicSmemBytes = ProbeKernel<SIDE, Table>::kSmem;
+  cfg.dynamicSmemBytes = ProbeKernel<SIDE, MN, Table>::kSmem;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -2831,7 +2905,7 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, cuda
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   profile_events(&ev0, &ev1);
   if (ev0) QM_CUDA_OK(cudaEventRecord(ev0, s));
-  QM_CUDA_OK(cudaLaunchKernelEx(&cfg, ProbeKernel<SIDE, Table>::kernel, tab));
+  QM_CUDA_OK(cudaLaunchKernelEx(&cfg, ProbeKernel<SIDE, MN, Table>::kernel, tab));
   if (ev1) QM_CUDA_OK(cudaEventRecord(ev1, s));
   count_launch();
   return QM_OK;
@@ -2871,6 +2945,13 @@ qm_status launch_tc_probes(const TcProbeArgs* ps, int n, cudaStream_t s) {
   auto by_cost = [](const UnitPlan& a, const UnitPlan& b) { return a.g.K * (72 + 24 * a.n_var) > b.g.K * (72 + 24 * b.n_var); };
   std::stable_sort(units.begin(), units.begin() + n_side, by_cost);
   std::stable_sort(units.begin() + n_side, units.end(), by_cost);
+  auto any_mn = [&](const UnitPlan* u, int count) {
+    for (int k = 0; k < count; ++k) {
+      const TcProbeArgs& a = ps[u[k].probe[0]];
+      if (a.l_mn || a.r_mn || a.cl_mn || a.cr_mn) return true;
+    }
+    return false;
+  };
   for (size_t u0 = 0; u0 < units.size() && st == QM_OK;) {
     const bool side = u0 < n_side;
     const size_t end = side ? n_side : units.size();
@@ -2884,9 +2965,10 @@ qm_status launch_tc_probes(const TcProbeArgs* ps, int n, cudaStream_t s) {
       ++u1;
     }
     const int count = (int)(u1 - u0);
-    if (!side) st = launch_units<false, TableBig>(ps, &units[u0], count, s);
-    else if (count == 1) st = launch_units<true, TableOne>(ps, &units[u0], 1, s);
-    else st = launch_units<true, TableBig>(ps, &units[u0], count, s);
+    const bool mn = any_mn(&units[u0], count);
+    if (!side) st = mn ? launch_units<false, true, TableBig>(ps, &units[u0], count, s) : launch_units<false, false, TableBig>(ps, &units[u0], count, s);
+    else if (count == 1) st = mn ? launch_units<true, true, TableOne>(ps, &units[u0], 1, s) : launch_units<true, false, TableOne>(ps, &units[u0], 1, s);
+    else st = mn ? launch_units<true, true, TableBig>(ps, &units[u0], count, s) : launch_units<true, false, TableBig>(ps, &units[u0], count, s);
     u0 = u1;
   }
   return st != QM_OK ? st : refused;
