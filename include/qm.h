@@ -368,10 +368,10 @@ qm_status qm_quantize_error(const qm_operand* x, int32_t fmt, int32_t gran, cons
  * and wgrad): inside a batch, operands that describe the same memory (same
  * address, extents and strides) under the same scale grouping are prepared
  * once.  Their max|x| is reduced once (for per-tensor scales also across the
- * two orientations of a tensor), the contraction-major copy is made once, the
- * codes of up to three formats come from one pass over the tensor, and equal
- * (format, rounding) requests share scales and codes outright; a probe then
- * reads those results from the workspace of the probe that made them, and a
+ * two orientations of a tensor, and then the codes rounded to nearest as well),
+ * the codes of up to three formats come from one pass over the tensor, and
+ * equal (format, rounding) requests share scales and codes outright; a probe
+ * then reads those results from the workspace they were put into, and a
  * non-finite operand is reported in the record of every probe that uses it.
  * All of it is ordered after the work already in `stream`, and work put into
  * `stream` after the call waits for every probe.  `out` is a device array of n

@@ -109,7 +109,7 @@ size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
 // The tensor-core products take an operand whose contraction is strided as it lies in memory, and its codes too
 // where they are rounded to nearest: written in the operand's own order, by passes that move whole lines, no
 // transposition and no bf16 copy (the transposing quantize kernels moved 7 bytes an element and the copy is read again:
-// 16384 x 4096 in three formats 106 us so, 61 in order).  Under one scale such codes are those of the flipped
+// 16384 x 4096 in three formats 106 us so, 65 in order).  Under one scale such codes are those of the flipped
 // view, so a tensor that is used in both orientations is quantized once.  Stochastic rounding numbers its draws along the
 // contraction: those codes stay contraction-major.
 bool codes_mn(const View& v, bool stochastic) { return !v.c_contig() && !stochastic; }
