@@ -1863,6 +1863,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
     // reduce the statistics of unit `pi` over the CTA and write its records (all 256 threads call)
     auto flush = [&](int pi) {
       const int nv = sh->walk[pi].n_var, v0 = sh->walk[pi].var_begin;
+      __syncwarp();                                // lanes 16..31 read below what lanes 0..15 have written to sums[]
       // values 3v, 3v + 1, 3v + 2: sum BE, max BE, sum diff^2 of variant v; the last two: sum C^2, D^2.  Half a warp adds up each
       for (int v = 0; v < nv; ++v) {
         const double2 a = sh->sums[v][ew][lane & 15];

@@ -109,3 +109,24 @@ def test_one_copy_of_a_strided_operand_whatever_the_scales(cl, cr):
         assert rec.device_error == 0
         for k in FIELDS:
             assert abs(rec.record()[k] - alone[k]) <= 1e-12 * abs(alone[k]), (f, g, r, k)
+
+
+@pytest.mark.parametrize("gran", ["tensor", "channel"])
+def test_records_hold_the_last_tile_of_every_unit(gran):
+    """Units of one probe that ride along in a launch of shared products, most of them a tile per CTA pair: a unit's last tile
+    counts in every sum.  The per-row sums of the same launch leave each tile by another way (atomics from the registers)."""
+    shapes = [(256, 128, 64), (130, 40, 80), (256, 64, 16), (20, 128, 128), (257, 129, 208), (256, 256, 64)]
+    ops = [[t.cuda() for t in operands(M, N, K, 1, 300 + i)] for i, (M, N, K) in enumerate(shapes)]
+    probes = [(qm.operand_of(L, -1), qm.operand_of(R, -1), f, f, gran, gran)
+              for i, (L, R) in enumerate(ops) for f in (("e4m3", "int8", "e5m2") if i == 0 else (("int8", "e4m3")[i & 1],))]
+    b = qm.ProbeBatch(probes, row_stats=True)
+    for _ in range(8):
+        b.launch()
+        torch.cuda.synchronize()
+        for p, rec, rows in zip(probes, b.results(), b.row_stats):
+            alone, rows = qm.qm_probe_layer(*p).record(), rows.cpu().numpy()
+            want = dict(zip(FIELDS, rows.sum(axis=0)), max_be=rows[:, 1].max())
+            assert rec.device_error == 0
+            for k in FIELDS:     # fp64 additions of the same terms in another order
+                assert abs(rec.record()[k] - want[k]) <= 1e-12 * abs(want[k]), k
+                assert abs(rec.record()[k] - alone[k]) <= 1e-12 * abs(alone[k]), k
