@@ -117,7 +117,8 @@ qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint
 qm_status launch_scale_quantize_rows(const View& x, int fmt, float* delta_out, uint8_t* codes,
                                      void* abs_copy, uint32_t* err_word, cudaStream_t s);
 
-// The same for nf (1..3) distinct formats, from one read of the tensor where its rows allow.
+// The same for nf (1..3) distinct formats, from one read of the tensor where rows_from_one_read says so.
+bool rows_from_one_read(const View& x);
 qm_status launch_scale_quantize_rows_multi(const View& x, int nf, const int* fmts, float* const* delta_out,
                                            uint32_t* const* err_word, uint8_t* const* codes, cudaStream_t s);
 

@@ -1967,10 +1967,12 @@ qm_status launch_quantize_cols(const View& x, const uint32_t* amax, int nf, cons
   return QM_OK;
 }
 
+bool rows_from_one_read(const View& x) { return x.dtype == QM_DT_BF16 && rows_spread(x, 2); }
+
 qm_status launch_scale_quantize_rows_multi(const View& x, int nf, const int* fmts, float* const* delta_out,
                                            uint32_t* const* err_word, uint8_t* const* codes, cudaStream_t s) {
   if (nf < 1 || nf > 3) return QM_ERR_INVALID_ARG;
-  if (nf == 1 || x.dtype != QM_DT_BF16 || !rows_spread(x, nf)) {
+  if (nf == 1 || !rows_from_one_read(x)) {
     for (int k = 0; k < nf; ++k) {
       const qm_status st = launch_scale_quantize_rows(x, fmts[k], delta_out[k], codes[k], nullptr, err_word[k], s);
       if (st != QM_OK) return st;

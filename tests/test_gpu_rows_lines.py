@@ -58,9 +58,10 @@ def test_lines_under_one_scale(c, dtype):
             same_codes(codes, d, x, fmt, "tensor", np.full(1, given, np.float32))
 
 
-@pytest.mark.parametrize("k", [16, 512, 1040, 4096])
+@pytest.mark.parametrize("k", [16, 512, 1040, 4096, 8192, 8208])
 def test_formats_of_rows_from_one_read(k):
-    """Probes under channel scales in three formats: a batch prepares the rows in one pass, alone each has its own."""
+    """Probes under channel scales in three formats: a batch prepares the rows in one pass (beyond 8192 elements in one of each
+    format, on streams of their own), alone each has its own."""
     a, b = tensor(300, k, torch.bfloat16, 0, k), tensor(130, k, torch.bfloat16, 8, k + 1)
     probes = [(qm.operand_of(a, -1), qm.operand_of(b, -1), f, f, "channel", "channel") for f in ("int8", "e4m3", "e5m2")]
     batch = qm.ProbeBatch(probes)
