@@ -413,6 +413,18 @@ template <> struct Piece<__nv_bfloat16> {
     else { w[0] = __ldg(reinterpret_cast<const uint4*>(p)); w[1] = __ldg(reinterpret_cast<const uint4*>(p) + 1); }
   }
   __device__ __forceinline__ void zero() { w[0] = w[1] = make_uint4(0u, 0u, 0u, 0u); }
+  // the n < 16 elements that are left of a line, zeros behind them
+  __device__ __forceinline__ void load_part(const __nv_bfloat16* p, int n) {
+    const bool half = n >= 8;
+    const unsigned short* e = reinterpret_cast<const unsigned short*>(p) + (half ? 8 : 0);
+    const int m = half ? n - 8 : n;
+    uint32_t h[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) h[j] = j < m ? (uint32_t)__ldg(e + j) : 0u;
+    const uint4 v = make_uint4(h[0] | h[1] << 16, h[2] | h[3] << 16, h[4] | h[5] << 16, h[6] | h[7] << 16), z = make_uint4(0u, 0u, 0u, 0u);
+    w[0] = half ? __ldg(reinterpret_cast<const uint4*>(p)) : v;
+    w[1] = half ? v : z;
+  }
   __device__ __forceinline__ uint32_t absmax() const {    // as an fp32 bit pattern
     const uint32_t k = 0x7fff7fffu;
     uint32_t m = 0;
@@ -438,6 +450,16 @@ template <> struct Piece<float> {
 #pragma unroll
     for (int h = 0; h < 4; ++h) w[h] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
+  __device__ __forceinline__ void load_part(const float* p, int n) {
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      if (4 * h + 4 <= n) { w[h] = __ldg(reinterpret_cast<const float4*>(p) + h); continue; }
+      float e[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) e[j] = 4 * h + j < n ? __ldg(p + 4 * h + j) : 0.f;
+      w[h] = make_float4(e[0], e[1], e[2], e[3]);
+    }
+  }
   __device__ __forceinline__ uint32_t absmax() const {
     uint32_t m = 0;
 #pragma unroll
@@ -461,9 +483,11 @@ template <> struct Piece<float> {
 
 // ---------------------------------------------------------------- quantize, lines of any length and pitch under one scale
 // What the dense kernels do not take: bf16 rows that are no multiple of 16 long or lie apart, and fp32.  A thread takes
-// sixteen elements of a line, every format in MASK, with the two-wide quotient; only a line's last piece is taken element
-// by element.  Bound by HBM; us, one element at a time and a launch per format / so: 13809 x 1234 bf16 E4M3 under a given
-// scale 18.9 / 15.6, three formats with their max|x| pass 73.0 / 57.7, fp32 16384 x 4096 62.6 / 53.6 and 251 / 130.
+// sixteen elements of a line, every format in MASK, with the two-wide quotient; of a line's last piece only the loads are
+// element by element (with its arithmetic so too, every warp that held one took 1.3 to 1.8 x as long).  Bound by HBM; us per
+// call, one element at a time and a launch per format / last piece one at a time / so: 13809 x 1234 bf16 under a given scale
+// 14.9 / 13.6 / 12.1, three formats with their max|x| pass 61.6 / 51.3 / 31.9; fp32 16384 x 4096 57 / 49 and 222 / 121.
+// 128 x 40 x 128 in a batch of 512, the right operand strided, three formats: transposed 72.4, 78.4, so 71.1.
 template <typename T, int MASK, bool GUARD>
 __global__ void __launch_bounds__(kThreads)
 quantize_lines_kernel(const T* __restrict__ x, uint32_t total, int64_t c, int64_t s_nc, int64_t s_b, const FastDiv by_chunks,
@@ -477,7 +501,7 @@ quantize_lines_kernel(const T* __restrict__ x, uint32_t total, int64_t c, int64_
   const T* src = x + (int64_t)b * s_b + (int64_t)(row - b * by_nc.d) * s_nc + k0;
   const bool whole = k0 + 16 <= c;
   Piece<T> p;
-  if (whole) p.load(src, false); else p.zero();
+  if (whole) p.load(src, false); else p.load_part(src, (int)(c - k0));
   float d[3] = {1.f, 1.f, 1.f};
   if (GUARD) {
     const float given = __ldg(delta);
@@ -490,7 +514,7 @@ quantize_lines_kernel(const T* __restrict__ x, uint32_t total, int64_t c, int64_
   for (int f = 0; f < 3; ++f) {
     if (!(MASK & (1 << f))) continue;
     uint4* dst = reinterpret_cast<uint4*>(o.codes[f] + (int64_t)row * ldc + k0);
-    if (whole && QuotientPair::serves(d[f])) {
+    if (QuotientPair::serves(d[f])) {
       const QuotientPair qp(d[f]);
       *dst = f == 0 ? p.template quant<0, GUARD>(qp) : f == 1 ? p.template quant<1, GUARD>(qp) : p.template quant<2, GUARD>(qp);
     } else {
@@ -498,7 +522,7 @@ quantize_lines_kernel(const T* __restrict__ x, uint32_t total, int64_t c, int64_
       uint32_t w[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
       for (int e = 0; e < 16; e += 2) {
-        const float t0 = quot(k0 + e < c ? Loader<T>::load1(src, e) : 0.f), t1 = quot(k0 + e + 1 < c ? Loader<T>::load1(src, e + 1) : 0.f);
+        const float t0 = quot(p.at(e)), t1 = quot(p.at(e + 1));
         w[e >> 2] |= (f == 0 ? quant2<0>(t0, t1) : f == 1 ? quant2<1>(t0, t1) : quant2<2>(t0, t1)) << (16 * (e >> 1 & 1));
       }
       *dst = make_uint4(w[0], w[1], w[2], w[3]);

@@ -71,3 +71,36 @@ def test_formats_of_rows_from_one_read(k):
         assert r.device_error == 0 and got["count"] == want["count"] and got["max_be"] == want["max_be"]
         for key in ("sum_be", "sum_diff2", "sum_ref2", "sum_den2"):
             assert abs(got[key] - want[key]) <= 1e-12 * abs(want[key]), key
+
+
+@pytest.mark.parametrize("dtype,c,per_block", [(torch.bfloat16, 1040, 4), (torch.bfloat16, 2064, 2), (torch.bfloat16, 4112, 1),
+                                               (torch.float32, 272, 8), (torch.float32, 528, 4), (torch.float32, 1040, 2),
+                                               (torch.float32, 2064, 1), (torch.float32, 4112, 1)])
+def test_every_group_of_warps_takes_several_rows(dtype, c, per_block):
+    """More than three rows for each group of one to eight warps (8 blocks an SM, per_block groups in each), the maxima of rows that
+    follow one another far apart: a maximum left over from the row before, or the one before that, would show."""
+    rows = 3 * 8 * torch.cuda.get_device_properties(0).multi_processor_count * per_block + 3
+    g = torch.Generator(device="cuda").manual_seed(c)
+    x = torch.randn((rows, c), generator=g, device="cuda") * torch.exp2(torch.arange(rows, device="cuda") * 5 % 23 - 11.0)[:, None]
+    x = x.to(dtype)
+    for fmt in ("int8", "e4m3") if dtype == torch.bfloat16 else ("e5m2",):
+        codes, delta, _, _ = qm.qm_quantize(qm.operand_of(x, -1), fmt, "channel")
+        same_codes(codes, delta, x, fmt, "channel")
+
+
+@pytest.mark.parametrize("c", [17, 130, 1234])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_lines_under_scales_outside_the_range_of_the_two_wide_quotient(c, dtype):
+    for factor in (1e-25, 1e25):
+        x = tensor(61, c, dtype, -c % 8, c)
+        x *= factor
+        codes, deltas, _ = qm.qm_quantize_formats(qm.operand_of(x, -1), ["e4m3", "e5m2", "int8"], "tensor")
+        for k, fmt in enumerate(("e4m3", "e5m2", "int8")):
+            same_codes(codes[k], deltas[k], x, fmt, "tensor")
+    x = tensor(61, c, dtype, -c % 8, c)
+    x[2, 0] = 3e30
+    for given in (1e-22, 2.0 ** -60, 2.0 ** 60, 1e22):          # either side of the range and its ends
+        d = torch.tensor([given], dtype=torch.float32, device="cuda")
+        for fmt in ("int8", "e4m3", "e5m2"):
+            codes, _, _, _ = qm.qm_quantize(qm.operand_of(x, -1), fmt, "tensor", d)
+            same_codes(codes, d, x, fmt, "tensor", np.full(1, given, np.float32))
