@@ -1153,15 +1153,19 @@ quantize_transpose_bf16_kernel(const __nv_bfloat16* __restrict__ x, int64_t nc, 
 
 // ---------------------------------------------------------------- quantize in storage order, a scale per column
 // Storage [c][nc] (nc contiguous, bf16), a scale per column, codes in the same order: [c] rows of ldn bytes, every format
-// in MASK.  A block takes 256 columns x a run of rows; its threads first make a column's scales each (maximum bits from
-// `bits`), then a thread takes eight columns of every eighth row, four rows in flight.  Bound by HBM.
+// in MASK.  A block takes 64, 128 or 256 columns (8 << lane_bits) x a run of rows; its threads first make a column's scales each
+// (maximum bits from `bits`), then a thread takes eight columns of four rows at a time.  Bound by HBM.  Blocks of 256 columns
+// whatever the operand's width leave most lanes of a narrow one without columns; us, transposed / 256 columns a block / so:
+// 512 x 64 x 512 in a batch of 256, one format 15.9 / 27.9 / 16.3, three formats 30 (three launches) / 62 / 25; 40 columns of 128
+// in a batch of 512 8.6 / 12.8 / 7.8 and 24 / 30.5 / 13.3.
 struct ColScales { float recip[256], ndelta[256]; };      // recip 0: outside the range of the two-wide quotient
 template <int MASK, typename Bits>
 __device__ __forceinline__ void quantize_cols(const __nv_bfloat16* __restrict__ x, int64_t nc, int64_t s_c, int64_t row0, int64_t row1,
-                                              int64_t col_block, Bits bits, bool writer, const MultiOut& o, int64_t delta_at,
-                                              int64_t code_row0, int64_t ldn, ColScales* sc) {
-  {
-    const int64_t col = col_block * 256 + threadIdx.x;
+                                              int64_t col_block, int lane_bits, Bits bits, bool writer, const MultiOut& o,
+                                              int64_t delta_at, int64_t code_row0, int64_t ldn, ColScales* sc) {
+  const int cols = 8 << lane_bits, rows_at_once = 8 * (32 >> lane_bits);    // columns of the block, rows that its lanes cover
+  if ((int)threadIdx.x < cols) {
+    const int64_t col = col_block * cols + threadIdx.x;
     const uint32_t m = col < nc ? bits(col) : 0u;
     int k = 0;
 #pragma unroll
@@ -1178,16 +1182,16 @@ __device__ __forceinline__ void quantize_cols(const __nv_bfloat16* __restrict__ 
     }
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t col0 = col_block * 256 + lane * 8;
+  const int group = threadIdx.x & ((1 << lane_bits) - 1);              // of eight columns
+  const int64_t col0 = col_block * cols + group * 8;
   if (col0 >= nc) return;
   const int live = nc - col0 < 8 ? (int)(nc - col0) : 8;
   const __nv_bfloat16* base = x + col0;
-  for (int64_t r = row0 + warp; r < row1; r += 32) {
+  for (int64_t r = row0 + (threadIdx.x >> lane_bits); r < row1; r += 4 * rows_at_once) {
     uint4 w[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int64_t row = r + 8 * u < row1 ? r + 8 * u : r;          // repeats are not written
+      const int64_t row = r + u * rows_at_once < row1 ? r + u * rows_at_once : r;          // repeats are not written
       if (live == 8) {
         w[u] = __ldg(reinterpret_cast<const uint4*>(base + row * s_c));
       } else {
@@ -1208,8 +1212,8 @@ __device__ __forceinline__ void quantize_cols(const __nv_bfloat16* __restrict__ 
       uint64_t r2[4], n2[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        r2[j] = *reinterpret_cast<const uint64_t*>(&cs.recip[lane * 8 + 2 * j]);
-        n2[j] = *reinterpret_cast<const uint64_t*>(&cs.ndelta[lane * 8 + 2 * j]);
+        r2[j] = *reinterpret_cast<const uint64_t*>(&cs.recip[group * 8 + 2 * j]);
+        n2[j] = *reinterpret_cast<const uint64_t*>(&cs.ndelta[group * 8 + 2 * j]);
         asm("mov.b64 {%0, %1}, %2;" : "=f"(rc[2 * j]), "=f"(rc[2 * j + 1]) : "l"(r2[j]));
       }
       bool served = true;
@@ -1217,7 +1221,7 @@ __device__ __forceinline__ void quantize_cols(const __nv_bfloat16* __restrict__ 
       for (int j = 0; j < 8; ++j) served &= rc[j] != 0.f;
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        if (r + 8 * u >= row1) break;
+        if (r + u * rows_at_once >= row1) break;
         const uint32_t pw[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
         uint2 q;
         if (served) {
@@ -1232,12 +1236,12 @@ __device__ __forceinline__ void quantize_cols(const __nv_bfloat16* __restrict__ 
           uint32_t h[4];
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const float t0 = Quotient(-cs.ndelta[lane * 8 + 2 * j])(bf16_lo(pw[j])), t1 = Quotient(-cs.ndelta[lane * 8 + 2 * j + 1])(bf16_hi(pw[j]));
+            const float t0 = Quotient(-cs.ndelta[group * 8 + 2 * j])(bf16_lo(pw[j])), t1 = Quotient(-cs.ndelta[group * 8 + 2 * j + 1])(bf16_hi(pw[j]));
             h[j] = f == 0 ? quant2<0>(t0, t1) : f == 1 ? quant2<1>(t0, t1) : quant2<2>(t0, t1);
           }
           q = make_uint2(h[0] | h[1] << 16, h[2] | h[3] << 16);
         }
-        *reinterpret_cast<uint2*>(o.codes[f] + (code_row0 + r + 8 * u) * ldn + col0) = q;
+        *reinterpret_cast<uint2*>(o.codes[f] + (code_row0 + r + u * rows_at_once) * ldn + col0) = q;
       }
     }
   }
@@ -1246,12 +1250,23 @@ __device__ __forceinline__ void quantize_cols(const __nv_bfloat16* __restrict__ 
 template <int MASK>
 __global__ void __launch_bounds__(kThreads)
 quantize_cols_kernel(const __nv_bfloat16* __restrict__ x, int64_t nc, int64_t c, int64_t s_c, int64_t s_b, int64_t rows_per_block,
-                     const uint32_t* __restrict__ amax, const MultiOut o, int64_t ldn) {
+                     int lane_bits, const uint32_t* __restrict__ amax, const MultiOut o, int64_t ldn) {
   pdl_prologue();
   __shared__ __align__(16) ColScales sc[(MASK & 1) + (MASK >> 1 & 1) + (MASK >> 2 & 1)];
   const int64_t b = blockIdx.z, row0 = (int64_t)blockIdx.y * rows_per_block, row1 = min(c, row0 + rows_per_block);
-  quantize_cols<MASK>(x + b * s_b, nc, s_c, row0, row1, blockIdx.x, [&](int64_t col) { return __ldg(amax + b * nc + col); },
+  quantize_cols<MASK>(x + b * s_b, nc, s_c, row0, row1, blockIdx.x, lane_bits, [&](int64_t col) { return __ldg(amax + b * nc + col); },
                       blockIdx.y == 0, o, b * nc, b * c, ldn, sc);
+}
+
+// Eight columns a lane: as many lanes to a row as leave the fewest of them without columns, the most if several do (wide
+// operands are as fast in narrow blocks: 3078 columns of 2032 in three formats, the whole batch 96 us in blocks of 256, 93 of 64).
+__host__ inline int col_lane_bits(int64_t nc) {
+  int best = 5;
+  for (int bits = 4; bits >= 3; --bits) {
+    const int64_t w = 8 << bits, wb = 8 << best;
+    if ((nc + w - 1) / w * w < (nc + wb - 1) / wb * wb) best = bits;
+  }
+  return best;
 }
 
 // ---------------------------------------------------------------- both operands of a probe in two launches
@@ -1273,6 +1288,7 @@ struct PairOperand {
   int32_t blocks_quant, path;             // blocks of the second kernel, and how it walks the operand
   uint32_t gx, gy;                        // tiles: column tiles, contraction tiles
   uint32_t max_cols;                      // one scale per strided channel: blocks of 64 columns
+  int32_t col_lane_bits;                  // kPairCols: see quantize_cols
   uint32_t groups_per_line, total_groups, lines;   // the tensor as lines of contiguous groups of eight; lines per batch element
   FastDiv by_groups, by_lines, by_chunks, by_nc, by_gx, by_gy, by_max_cols;
   uint32_t* partial;
@@ -1437,7 +1453,7 @@ __device__ __forceinline__ void pair_quantize(const PairOperand& o, uint32_t* er
         for (int i = 0; i < o.n_partial; ++i) m = max(m, __ldg(o.partial + ((int64_t)i * v.batch + at.z) * v.nc + col));
         return m;
       };
-      quantize_cols<1 << FMT>(x + (int64_t)at.z * v.s_b, v.nc, v.s_c, row0, row1, at.x, bits, at.y == 0, out, (int64_t)at.z * v.nc,
+      quantize_cols<1 << FMT>(x + (int64_t)at.z * v.s_b, v.nc, v.s_c, row0, row1, at.x, o.col_lane_bits, bits, at.y == 0, out, (int64_t)at.z * v.nc,
                               (int64_t)at.z * v.c, (v.nc + 15) & ~(int64_t)15, reinterpret_cast<ColScales*>(smem));
       return;
     }
@@ -1797,7 +1813,9 @@ qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint
       o.by_chunks = FastDiv((uint32_t)chunks); o.by_nc = FastDiv((uint32_t)v.nc);
     } else {
       o.path = in.mn ? kPairCols : tiles ? kPairTiles : kPairGeneral;
-      o.gx = (uint32_t)(in.mn ? (v.nc + 255) / 256 : (v.nc + 63) / 64);
+      o.col_lane_bits = col_lane_bits(v.nc);
+      const int64_t cols = in.mn ? 8 << o.col_lane_bits : 64;
+      o.gx = (uint32_t)((v.nc + cols - 1) / cols);
       o.gy = (uint32_t)(in.mn ? (v.c + kPairColRows - 1) / kPairColRows : tiles ? (v.c + 127) / 128 : (ldc + 63) / 64);
       o.by_gx = FastDiv(o.gx); o.by_gy = FastDiv(o.gy);
       o.blocks_quant = (int32_t)((int64_t)o.gx * o.gy * v.batch);
@@ -1968,14 +1986,16 @@ qm_status launch_quantize_cols(const View& x, const uint32_t* amax, int nf, cons
     mask |= 1 << f;
     o.codes[f] = codes[k]; o.delta_out[f] = delta_out[k]; o.err_word[f] = err_word[k];
   }
-  // runs of rows that give every SM four blocks, of at least 32 rows (one step) and at most 65535 of them
-  const int64_t col_blocks = (x.nc + 255) / 256, want = (4ll * sm_count() + col_blocks * x.batch - 1) / (col_blocks * x.batch);
+  // runs of rows that give every SM four blocks, of whole steps and at most 65535 of them
+  const int lane_bits = col_lane_bits(x.nc);
+  const int64_t col_blocks = (x.nc + (8 << lane_bits) - 1) / (8 << lane_bits), want = (4ll * sm_count() + col_blocks * x.batch - 1) / (col_blocks * x.batch);
   int64_t rows = (x.c + want - 1) / want;
-  rows = (rows + 31) / 32 * 32;
+  const int64_t step = 32 * (32 >> lane_bits);                          // four rows a thread
+  rows = (rows + step - 1) / step * step;
   const dim3 grid((unsigned)col_blocks, (unsigned)((x.c + rows - 1) / rows), (unsigned)x.batch);
   if (col_blocks > 0x7fffffffll || x.batch > 65535) return QM_ERR_UNSUPPORTED;
   const __nv_bfloat16* p = static_cast<const __nv_bfloat16*>(x.data);
-#define QM_QC(M) launch_pdl(quantize_cols_kernel<M>, grid, dim3(kThreads), 0, s, p, x.nc, x.c, x.s_c, x.s_b, rows, amax, o, qm_code_ld(x.nc))
+#define QM_QC(M) launch_pdl(quantize_cols_kernel<M>, grid, dim3(kThreads), 0, s, p, x.nc, x.c, x.s_c, x.s_b, rows, lane_bits, amax, o, qm_code_ld(x.nc))
   switch (mask) {
     case 1: QM_QC(1); break;
     case 2: QM_QC(2); break;

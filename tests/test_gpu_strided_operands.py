@@ -101,3 +101,71 @@ def test_a_nonfinite_value_is_flagged_in_either_order():
     for gran in ("tensor", "channel"):
         (_a, ls), (_b, rs) = stored(L, True), stored(R, True)
         assert qm.qm_probe_layer(ls, rs, "e4m3", "e4m3", gran, gran).device_error & 1
+
+
+def kept_codes(ws, scales, rows, ld):
+    """The codes of the left operand where the workspace of a probe has them: behind the control block and the max|x| words and
+    scales of both operands (one of each per column here), every part on 256 bytes."""
+    pad = lambda b: (b + 255) & ~255
+    n_l, n_r = scales
+    at = 256 + 2 * (pad(4 * n_l) + pad(4 * n_r))
+    return ws[at:at + rows * ld].view(rows, ld).cpu().numpy()
+
+
+# columns: whole blocks of 256, 128 and 64, one more, few, not a multiple of eight; contraction entries: below and past the rows
+# that a block's lanes cover at once (8 to 32) and in one step of four, past the 64 rows of a block of the two-launch preparation
+@pytest.mark.parametrize("m,k", [(256, 64), (257, 1040), (128, 272), (130, 80), (64, 1040), (72, 304), (40, 16), (12, 96), (1000, 48)])
+@pytest.mark.parametrize("gran", ["tensor", "channel"])
+@pytest.mark.parametrize("fmt", FORMATS)
+def test_codes_in_the_operands_own_order(m, k, gran, fmt):
+    """Bit for bit the oracle's, transposed, prepared alone and in a batch; beside ordinary columns some of zeros (a scale of 1) and
+    some whose scale lies outside the range of the two-wide quotient, on either side."""
+    L, R = draw((m, k), 20), draw((24, k), 21)
+    if gran == "channel":
+        L[3], L[m - 1], L[8] = 0.0, L[m - 1] * 1e-25, L[8] * 1e25
+    (_k, lo), (_r, ro) = stored(L, True), stored(R, True)
+    x = L.float().cpu().numpy()[None]
+    delta = oracle.scale(x, fmt, gran)
+    want = oracle.quantize(x, fmt, delta)[0].T
+    plan = qm.ProbePlan(lo, ro, fmt, fmt, gran, gran)
+    plan.launch(lo, ro)
+    batch = qm.ProbeBatch([(lo, ro, fmt, fmt, gran, gran), (ro, lo, fmt, fmt, gran, gran)])
+    batch.launch()
+    torch.cuda.synchronize()
+    n = (m, 24) if gran == "channel" else (1, 1)
+    for ws in (plan.ws, batch._ws[0]):
+        assert (kept_codes(ws, n, k, qm.binding.qm_code_ld(m))[:, :m] == want).all()
+
+
+@pytest.mark.parametrize("m,n,k", [(300, 72, 96), (1040, 40, 4096)])
+def test_columns_without_an_ordinary_scale_in_the_record(m, n, k):
+    L, R = draw((m, k), 22), draw((n, k), 23, 0.05)
+    L[5], L[17], R[2] = 0.0, L[17] * 1e-25, 0.0
+    (_k, lo), (_r, ro) = stored(L, True), stored(R, True)
+    for f in FORMATS:
+        want = oracle.probe(L.float().cpu().numpy(), R.float().cpu().numpy().T, f, f, "channel", "channel")
+        got = qm.qm_probe_layer(lo, ro, f, f, "channel", "channel")
+        assert got.device_error == 0
+        assert_record_close(got.record(), want)
+
+
+@pytest.mark.parametrize("a,b", [(272, 80), (1040, 528)])
+def test_one_memory_in_both_orientations(a, b):
+    """The same tensor contracted over either dimension in one batch, one use rounded stochastically, as the left and as the right
+    operand: what is shared (max|x|, the codes rounded to nearest) must be right for each."""
+    T, U, V = draw((a, b), 24), draw((136, b), 25, 0.05), draw((136, a), 26, 0.05)
+    (_t, over_b), (_u, u), (_v, v) = stored(T, False), stored(U, False), stored(V, True)
+    over_a = qm.operand_of(_t, -2)
+    uses = [(over_b, u, "rtne"), (over_a, v, "rtne"), (over_a, v, "stochastic_l"), (over_b, u, "stochastic_l"), (v, over_a, "stochastic_r"),
+            (u, over_b, "rtne"), (v, over_a, "rtne"), (over_b, u, "stochastic_both")]
+    probes = [(lo, ro, f, f, g, g, rnd) for f, g in (("e4m3", "tensor"), ("int8", "tensor"), ("e5m2", "channel")) for lo, ro, rnd in uses]
+    batch = qm.ProbeBatch([p[:6] for p in probes])
+    for i, p in enumerate(probes):
+        batch.cfg[i] = binding._cfg(*p[2:6], "bf16", p[6], 9)
+    batch.launch()
+    t = T.float().cpu().numpy()
+    against = {id(u): U.float().cpu().numpy().T, id(v): V.float().cpu().numpy().T}
+    for p, got in zip(probes, batch.results()):
+        same(got, qm.qm_probe_layer(*p[:6], rounding=p[6], seed=9))
+        if p[6] == "rtne" and p[0] in (over_a, over_b):
+            assert_record_close(got.record(), oracle.probe(t if p[0] is over_b else t.T, against[id(p[1])], *p[2:6]))
