@@ -1049,8 +1049,8 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 //
 // The left operand of the reference and denominator products is not read from shared memory by the tensor
 // cores: converter warps read this CTA's 128 rows of the L tile once and store them, and the same with
-// the sign bits cleared, into TENSOR memory, from where both products take their A operand; two more warps
-// write the |R| half-tile into the stage.  No |x| copy exists in HBM.  What the bf16 phase waits for is the
+// the sign bits cleared, into TENSOR memory, from where both products take their A operand; two more warps, or where
+// contractions are short the converters too (r_by_warps), write the |R| half-tile into the stage.  No |x| copy exists in HBM.  What the bf16 phase waits for is the
 // converters' serial time per block: wait, loads, wait for the tensor-memory stage, stores, arrival (4096^2 x 1024 in three
 // formats, cycles per block: 760 with |R| among the converters' work, 683 with two warps for it; 553 with all conversions left
 // out; four stages in tensor memory instead of two change nothing).  Half-block stages and prefetching the next
@@ -1067,7 +1067,7 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 //                 (128 deep); both kinds bring 128 bytes per row.  A CTA's loads complete on its own `full`.
 //   warp 1        allocates tensor memory; in the leader CTA it runs the MMA loop converged and
 //                 one elected lane issues the pair's MMAs; tcgen05.commit frees a stage in both CTAs (`empty`).
-//   warps 2, 3    |R|: a sign-cleared copy of each staged R half-tile.
+//   warps 2, 3    |R|: a sign-cleared copy of each staged R half-tile (idle where the converters write it).
 //   warps 4..7    converters of L, one per tensor-memory lane quarter: thread = one of the CTA's 128
 //                 left-operand rows.  Blocks of codes need no conversion: they only pass on that they landed.
 //   warps 8..15   epilogue.
@@ -1340,17 +1340,20 @@ __device__ __forceinline__ void load_l_mn_major(uint32_t base, int q, int lane, 
   }
 }
 // |R| beside a staged R half-tile, whatever its order: a flat sign-cleared copy of its first `vectors` 16-byte vectors (at most
-// 512) by the two warps to which t = 0..63 belongs, made visible to the tensor core's reads.
-__device__ __forceinline__ void abs_r_half(uint32_t r, uint32_t to_abs, int vectors, int t) {
+// 512) by the THREADS threads t = 0 .. THREADS - 1.  The tensor core sees it after a fence.proxy.async.
+template <int THREADS>
+__device__ __forceinline__ void abs_r(uint32_t r, uint32_t to_abs, int vectors, int t) {
+  constexpr int kEach = 512 / THREADS;
   const uint32_t src = r + (uint32_t)t * 16u, m = 0x7fff7fffu;
-  uint4 u[8];
+  uint4 u[kEach];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) u[j] = t + 64 * j < vectors ? lds128(src + (uint32_t)j * 1024u) : make_uint4(0u, 0u, 0u, 0u);
+  for (int j = 0; j < kEach; ++j) u[j] = t + THREADS * j < vectors ? lds128(src + (uint32_t)j * (16u * THREADS)) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-  for (int j = 0; j < 8; ++j)
-    if (t + 64 * j < vectors) sts128(src + to_abs + (uint32_t)j * 1024u, make_uint4(u[j].x & m, u[j].y & m, u[j].z & m, u[j].w & m));
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  for (int j = 0; j < kEach; ++j)
+    if (t + THREADS * j < vectors)
+      sts128(src + to_abs + (uint32_t)j * (16u * THREADS), make_uint4(u[j].x & m, u[j].y & m, u[j].z & m, u[j].w & m));
 }
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 // 32 lanes x 8 consecutive 32-bit columns.
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
   asm volatile(
@@ -1538,8 +1541,8 @@ __device__ __forceinline__ void probe_exit(Sh* sh, uint64_t wait_limit_ns, int w
   }
 }
 
-// MN: units may have operands whose contraction is strided.
-template <typename Table, bool MN>
+// MN: units may have operands whose contraction is strided.  RW: |R| by warps of its own, not by the converters (r_by_warps).
+template <typename Table, bool MN, bool RW>
 __global__ void __launch_bounds__(kProbeThreads, 1)
 tc_group_kernel(const __grid_constant__ Table tab) {
   using C = CfgP;
@@ -1572,7 +1575,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&sh->full[s]), 1);
-      mbar_init(smem_u32(&sh->ready[s]), 2 * 6);          // four converter warps and two for |R| in each CTA
+      mbar_init(smem_u32(&sh->ready[s]), 2 * (RW ? 6 : 4));   // four converter warps and, with RW, two for |R| in each CTA
       mbar_init(smem_u32(&sh->empty[s]), 1);
     }
     mbar_init(smem_u32(&sh->rd_full), 1);
@@ -1732,7 +1735,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           if (b) ++lp_uses1; else ++lp_uses0;
         }
       }
-    } else if (warp >= 2) {
+    } else if (RW && warp >= 2) {
       // ---------------------------------------------------------- |R| (both CTAs)
       TileWalk tw;
       begin(tw);
@@ -1744,7 +1747,8 @@ tc_group_kernel(const __grid_constant__ Table tab) {
         for (int kb = 0; kb < tw.num_kb && ok; ++kb) {
           ok = w.wait_warp(smem_u32(&sh->full[ring.s]), ring.parity);
           if (!ok) break;
-          abs_r_half(tile_base + ring.s * C::kStageBytes + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
+          abs_r<64>(tile_base + ring.s * C::kStageBytes + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
+          fence_proxy_async();
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster(ready_leader + ring.s * 8u);
           ring.next();
@@ -1797,6 +1801,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           ok = w.wait_warp(smem_u32(&sh->full[s]), ring.parity);
           if (!ok) break;
           const uint32_t base = tile_base + s * C::kStageBytes;
+          if (!RW) abs_r<128>(base + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
           uint32_t a[32];
           if constexpr (kMn) {
             load_l_mn_major(base + C::kOffL, q, lane, a);
@@ -1830,6 +1835,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           } else {
             tmem_st32(tcol + 32u, a);
           }
+          if (!RW) fence_proxy_async();
           asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
           tc_fence_before();
           __syncwarp();
@@ -2068,11 +2074,11 @@ tc_group_kernel(const __grid_constant__ Table tab) {
 // the sums in registers) with one wait.  Short contractions are bound by that chain, and by fetching its instructions: what
 // a tile runs once, all roles together, is more than the instruction cache holds beside the loops (512 x 512 x 64 x 256:
 // stalls for instructions per issue 1.1 -> 2.7 with the code for mn-major operands and integer divisions in the walk, 98 ->
-// 119 us; without either 102).  Measured, the fused kernel
+// 119 us; without either 102, with |R| written by the converters as well 94).  Measured, the fused kernel
 // alone, one after the other / side by side: 512 x 512 x 64 x 256 131 / 88 us; 8192 x 4096 with K = 128 75 / 53,
 // K = 256 76 / 64, K = 512 91 / 88, K = 1024 145 / 140.  With three probes per unit sharing wins from K = 64 on (187 / 239 us).
-// |R| by two warps of its own instead of the converters: 8192 x 4096 x 1024 149 / 139 us, 2048 x 3072 x 2048 76 / 69, 2048^2 x
-// 16384 357 / 300.  L from tensor memory as well (two stages of both, 96 KB) measured 140, 70 and 318, and 66 instead of
+// |R| by the converters / by two warps of its own: 8192 x 4096 x 1024 160 / 141 us, 2048 x 3072 x 2048 76 / 69, 2048^2 x
+// 16384 355 / 300 (short contractions the other way round: r_by_warps).  L from tensor memory as well (two stages of both, 96 KB) measured 140, 70 and 318, and 66 instead of
 // 60 at K = 192, where two blocks are not enough ahead.
 //   Roles, registers, walk and exit are those of tc_group_kernel.  Tensor memory: columns 0..127 reference, 128..255
 // denominator, 256..383 the 8-bit product, 384..511 four stages of |L| (32 columns of two bf16 each).
@@ -2168,8 +2174,8 @@ __device__ __forceinline__ void row_stats_add(double* rs, const StatsG& st) {
   unpack2(st.n2, x0, x1); atomicAdd(rs + 4, (double)x0 + (double)x1);
 }
 
-// MN: units may have operands whose contraction is strided.
-template <typename Table, bool MN>
+// MN: units may have operands whose contraction is strided.  RW: |R| by warps of its own, not by the converters (r_by_warps).
+template <typename Table, bool MN, bool RW>
 __global__ void __launch_bounds__(kProbeThreads, 1)
 tc_side_kernel(const __grid_constant__ Table tab) {
   using C = CfgS;
@@ -2199,7 +2205,7 @@ tc_side_kernel(const __grid_constant__ Table tab) {
       mbar_init(smem_u32(&sh->full[s]), 1);
       mbar_init(smem_u32(&sh->empty[s]), 1);
     }
-    for (int s = 0; s < kStages; ++s) mbar_init(smem_u32(&sh->ready[s]), 2 * 6);   // four converter warps and two for |R| in each CTA
+    for (int s = 0; s < kStages; ++s) mbar_init(smem_u32(&sh->ready[s]), 2 * (RW ? 6 : 4));   // four converter warps and, with RW, two for |R| in each CTA
     mbar_init(smem_u32(&sh->tmem_full), 1);
     mbar_init(smem_u32(&sh->tmem_empty), 2 * kEpiWarps);
     mbar_init(smem_u32(&sh->lp_done), 2 * kEpiWarps);
@@ -2338,7 +2344,7 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         }
         if (ok) tc_commit_pair(smem_u32(&sh->tmem_full), lead);           // this tile's accumulators are complete
       }
-    } else if (warp >= 2) {
+    } else if (RW && warp >= 2) {
       // ---------------------------------------------------------- |R| (both CTAs)
       TileWalk tw;
       begin(tw);
@@ -2350,7 +2356,8 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         for (int kb = 0; kb < tw.num_kb; ++kb) {
           ok = w.wait_warp(smem_u32(&sh->full[s]), parity);
           if (!ok) break;
-          abs_r_half(tile_base + s * C::kStageBytes + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
+          abs_r<64>(tile_base + s * C::kStageBytes + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
+          fence_proxy_async();
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster(ready_leader + s * 8u);
           if (++s == (uint32_t)kStages) { s = 0; parity ^= 1u; }
@@ -2382,6 +2389,7 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         const uint32_t s = g % kStages, m = 0x7fff7fffu;
         if (!w.wait_warp(smem_u32(&sh->full[s]), (g / kStages) & 1)) { ok = false; return; }
         const uint32_t base = tile_base + s * C::kStageBytes;
+        if (!RW) abs_r<128>(base + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
         uint32_t a[32];
         if constexpr (kMn) {
           load_l_mn_major(base + C::kOffL, q, lane, a);
@@ -2407,6 +2415,7 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         } else {
           tmem_st32(tcol, a);
         }
+        if (!RW) fence_proxy_async();
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         tc_fence_before();
         __syncwarp();
@@ -2752,12 +2761,11 @@ qm_status launch_wide(const CUtensorMap& ma, const CUtensorMap& mb, KernelArgs k
 }  // namespace
 
 namespace {
-// The two forms of the fused kernel: units of one probe, and units of several (see the kernels).
 // The two forms of the fused kernel, units of one probe (SIDE) and units of several, each with and without operands whose
 // contraction is strided: what those need is a third of the roles' code, and short tiles wait for instructions (below).
-template <bool SIDE, bool MN, typename Table>
+template <bool SIDE, bool MN, bool RW, typename Table>
 struct ProbeKernel {
-  static constexpr auto kernel = SIDE ? tc_side_kernel<Table, MN> : tc_group_kernel<Table, MN>;
+  static constexpr auto kernel = SIDE ? tc_side_kernel<Table, MN, RW> : tc_group_kernel<Table, MN, RW>;
   static constexpr size_t kSmem = 1024 + (SIDE ? (size_t)CfgS::kTileBytes + sizeof(SharedS<Table::kUnits>)
                                                : (size_t)CfgP::kTileBytes + sizeof(SharedP<Table::kUnits, Table::kVars>));
   static_assert(kSmem <= 232448, "shared memory of a CTA");
@@ -2783,18 +2791,24 @@ qm_status probe_kernel_ready() {
   return allow_smem(PK::kernel, PK::kSmem, attr_done);
 }
 
+template <bool SIDE, typename Table>
+qm_status probe_kernels_ready() {
+  qm_status st = probe_kernel_ready<ProbeKernel<SIDE, false, false, Table>>();
+  if (st == QM_OK) st = probe_kernel_ready<ProbeKernel<SIDE, false, true, Table>>();
+  if (st == QM_OK) st = probe_kernel_ready<ProbeKernel<SIDE, true, false, Table>>();
+  if (st == QM_OK) st = probe_kernel_ready<ProbeKernel<SIDE, true, true, Table>>();
+  return st;
+}
+
 // CTA pairs of the fused probe kernel that can be resident at once (its footprint is the largest
 // of all modes, so its residency bounds every grid); queried once per device.
 qm_status probe_residency() {
   const int dev = current_device();
   if (dev < 0) return QM_ERR_UNSUPPORTED;
-  using Widest = ProbeKernel<false, true, TableBig>;
-  qm_status as = probe_kernel_ready<Widest>();
-  if (as == QM_OK) as = probe_kernel_ready<ProbeKernel<false, false, TableBig>>();
-  if (as == QM_OK) as = probe_kernel_ready<ProbeKernel<true, true, TableBig>>();
-  if (as == QM_OK) as = probe_kernel_ready<ProbeKernel<true, true, TableOne>>();
-  if (as == QM_OK) as = probe_kernel_ready<ProbeKernel<true, false, TableBig>>();
-  if (as == QM_OK) as = probe_kernel_ready<ProbeKernel<true, false, TableOne>>();
+  using Widest = ProbeKernel<false, true, true, TableBig>;
+  qm_status as = probe_kernels_ready<false, TableBig>();
+  if (as == QM_OK) as = probe_kernels_ready<true, TableBig>();
+  if (as == QM_OK) as = probe_kernels_ready<true, TableOne>();
   if (as != QM_OK) return as;
   if (g_max_pairs[dev] == 0) {
     cudaLaunchConfig_t q{};
@@ -2826,8 +2840,19 @@ bool same_products(const TcProbeArgs& a, const TcProbeArgs& b) {
          a.l_mn == b.l_mn && a.r_mn == b.r_mn && a.g.M == b.g.M && a.g.N == b.g.N && a.g.K == b.g.K && a.g.batch == b.g.batch;
 }
 
-template <bool SIDE, bool MN, typename Table>
-qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, cudaStream_t s) {
+// Whether |R| gets two warps of its own.  Long contractions wait for the converters, short ones for the epilogue and for
+// instructions, which the role adds to: with one probe to a unit up to two blocks of the contraction, with several up to as
+// many as the ring has stages.  Whole batches in us, |R| by the converters / by warps of its own: one format 512 x 512 x 64 x 256
+// 93.7 / 101.7, 8192 x 4096 with K = 128 55.4 / 57.5, 192 59.5 / 59.6, 512 96 / 89; three formats K = 64 102.7 / 104.8, 256 113.2 / 119.1,
+// 384 131.2 / 131.9, 416 138.0 / 134.7.  A launch that mixes the two takes what its long units want.
+bool r_by_warps(bool side, const UnitPlan* units, int n) {
+  for (int k = 0; k < n; ++k)
+    if (units[k].g.K > (side ? 2 : CfgP::kStages) * kBlockK) return true;
+  return false;
+}
+
+template <bool SIDE, typename Table>
+qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, bool mn, cudaStream_t s) {
   static Table tab;                    // up to 29 KB: kept off the stack; guarded by the mutex below
   static std::mutex mu;
   std::lock_guard<std::mutex> lock(mu);
@@ -2894,7 +2919,7 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, cuda
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(2 * (total < pairs ? total : pairs)));
   cfg.blockDim = dim3(kProbeThreads);
-  cfg.dynamicSmemBytes = ProbeKernel<SIDE, MN, Table>::kSmem;
+  cfg.dynamicSmemBytes = ProbeKernel<SIDE, false, false, Table>::kSmem;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -2903,10 +2928,13 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, cuda
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl_enabled() ? 2 : 1;
+  const bool rw = r_by_warps(SIDE, units, n);
+  const auto kernel = mn ? (rw ? ProbeKernel<SIDE, true, true, Table>::kernel : ProbeKernel<SIDE, true, false, Table>::kernel)
+                         : (rw ? ProbeKernel<SIDE, false, true, Table>::kernel : ProbeKernel<SIDE, false, false, Table>::kernel);
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   profile_events(&ev0, &ev1);
   if (ev0) QM_CUDA_OK(cudaEventRecord(ev0, s));
-  QM_CUDA_OK(cudaLaunchKernelEx(&cfg, ProbeKernel<SIDE, MN, Table>::kernel, tab));
+  QM_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, tab));
   if (ev1) QM_CUDA_OK(cudaEventRecord(ev1, s));
   count_launch();
   return QM_OK;
@@ -2967,9 +2995,9 @@ qm_status launch_tc_probes(const TcProbeArgs* ps, int n, cudaStream_t s) {
     }
     const int count = (int)(u1 - u0);
     const bool mn = any_mn(&units[u0], count);
-    if (!side) st = mn ? launch_units<false, true, TableBig>(ps, &units[u0], count, s) : launch_units<false, false, TableBig>(ps, &units[u0], count, s);
-    else if (count == 1) st = mn ? launch_units<true, true, TableOne>(ps, &units[u0], 1, s) : launch_units<true, false, TableOne>(ps, &units[u0], 1, s);
-    else st = mn ? launch_units<true, true, TableBig>(ps, &units[u0], count, s) : launch_units<true, false, TableBig>(ps, &units[u0], count, s);
+    if (!side) st = launch_units<false, TableBig>(ps, &units[u0], count, mn, s);
+    else if (count == 1) st = launch_units<true, TableOne>(ps, &units[u0], 1, mn, s);
+    else st = launch_units<true, TableBig>(ps, &units[u0], count, mn, s);
     u0 = u1;
   }
   return st != QM_OK ? st : refused;

@@ -106,3 +106,21 @@ def test_shared_products_report_the_timeout_in_every_record(starved_producer, st
     torch.cuda.synchronize()
     for f, r in zip(formats, batch.results()):
         check_against_oracle({**o, "fmt_l": f, "fmt_r": f}, r)
+
+
+# The same with |R| written by the warps that the tests above leave out: one probe of two blocks, shared products of seven
+@pytest.mark.parametrize("K,formats,stop_after", [(128, ("e4m3",), 0), (128, ("e4m3",), 1), (448, ("e4m3", "int8"), 0),
+                                                  (448, ("e4m3", "int8"), 6), (448, ("e4m3", "int8"), 9)])
+def test_either_writer_of_the_magnitudes_gives_up(starved_producer, K, formats, stop_after):
+    o = small_op(seed=36, K=K)
+    Ld, Rd = o["L"].cuda(), o["R"].cuda()
+    batch = qm.ProbeBatch([(qm.operand_of(Ld, o["cl"]), qm.operand_of(Rd, o["cr"]), f, f, "tensor", "tensor") for f in formats])
+    starved_producer.qm_debug_stop_producer_after(stop_after)
+    batch.launch()
+    torch.cuda.synchronize()
+    assert all(r.device_error & QM_DEVERR_TIMEOUT for r in batch.results())
+    starved_producer.qm_debug_stop_producer_after(0xffffffff)
+    batch.launch()
+    torch.cuda.synchronize()
+    for f, r in zip(formats, batch.results()):
+        check_against_oracle({**o, "fmt_l": f, "fmt_r": f}, r)

@@ -130,3 +130,29 @@ def test_records_hold_the_last_tile_of_every_unit(gran):
             for k in FIELDS:     # fp64 additions of the same terms in another order
                 assert abs(rec.record()[k] - want[k]) <= 1e-12 * abs(want[k]), k
                 assert abs(rec.record()[k] - alone[k]) <= 1e-12 * abs(alone[k]), k
+
+
+# |R| is written by the converters up to two blocks of the contraction with one probe to a unit and up to six with several, by warps
+# of its own beyond, and in a whole launch as soon as one of its units is longer
+@pytest.mark.parametrize("lengths", [(128,), (144,), (128, 144), (16, 1040)])
+@pytest.mark.parametrize("formats", [("e4m3",), ("int8", "e5m2")])
+@pytest.mark.parametrize("cl,cr", [(-1, -1), (-2, -2)])
+def test_records_do_not_depend_on_who_writes_the_magnitudes(lengths, formats, cl, cr):
+    if len(formats) > 1:
+        lengths = tuple({128: 384, 144: 400}.get(k, k) for k in lengths)
+    probes, want = [], []
+    for i, K in enumerate(lengths):
+        L, R = operands(264, 136, K, 1, 400 + i)
+        Lo, Ro = (qm.operand_of(t.cuda() if c == -1 else t.T.contiguous().cuda(), c) for t, c in ((L, cl), (R, cr)))
+        for f in formats:
+            probes.append((Lo, Ro, f, f, "tensor", "channel"))
+            want.append(oracle.probe(L.float().numpy(), R.float().numpy().T, f, f, "tensor", "channel"))
+    b = qm.ProbeBatch(probes)
+    b.launch()
+    torch.cuda.synchronize()
+    for p, rec, w in zip(probes, b.results(), want):
+        alone = qm.qm_probe_layer(*p).record()
+        assert rec.device_error == 0
+        for k in FIELDS:
+            assert abs(rec.record()[k] - alone[k]) <= 1e-12 * abs(alone[k]), k
+            assert abs(rec.record()[k] - w[k]) <= (1e-3 if k == "max_be" else 1e-4) * abs(w[k]), k
