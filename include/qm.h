@@ -275,8 +275,12 @@ qm_status qm_gemm_ref(const void* l_bf16, const void* r_bf16, int64_t M, int64_t
 
 /*
  * Eq. 3 on materialised arrays: ref = C, q = Q, den = D, each `count` fp32
- * values.  `out` (device) receives the record.  `ws` is device scratch of at
- * least qm_metric_workspace_bytes(count) bytes, 8-byte aligned.
+ * values.  `out` receives the record: device memory, or pinned host memory,
+ * which the call's last kernel stores to directly, every field once and none
+ * read back (so a caller that waits for the stream needs no copy); the same
+ * holds for qm_probe_layer, qm_tensor_stats and qm_quantize_error, and for no
+ * other call.  `ws` is device scratch of at least
+ * qm_metric_workspace_bytes(count) bytes, 8-byte aligned.
  */
 size_t qm_metric_workspace_bytes(int64_t count);
 qm_status qm_metric(const float* ref, const float* q, const float* den, int64_t count,
@@ -286,8 +290,8 @@ qm_status qm_metric(const float* ref, const float* q, const float* den, int64_t 
  * The whole probe for one product L.R: scale, quantize, the three products
  * (8-bit, reference, denominator) and the Eq. 3 reduction fused so that no
  * M x N matrix is written.  L: noncontract = M, contract = K.  R: noncontract
- * = N, contract = K, same batch.  `out` (device) receives the record; `ws` is
- * device scratch of at least qm_workspace_bytes(L, R, cfg) bytes, 256-byte
+ * = N, contract = K, same batch.  `out` (device, or pinned host memory as for
+ * qm_metric) receives the record; `ws` is device scratch of at least qm_workspace_bytes(L, R, cfg) bytes, 256-byte
  * aligned; its contents on entry do not matter and concurrent calls must not
  * share it.
  * QM_REF_BF16_FP32ACC needs bf16 operands and K a multiple of 16;
@@ -340,8 +344,8 @@ qm_status qm_probe_layer_host(const qm_operand* L_host, const qm_operand* R_host
  * section for the codes qm_quantize would produce with these scales.  `delta`
  * (device) holds finished Eq. 1 scales as written by qm_scale or qm_quantize:
  * one value (QM_GRAN_TENSOR) or batch * noncontract values (QM_GRAN_CHANNEL).
- * `out` (device) receives the record.  `ws` is device scratch of at least
- * qm_stats_workspace_bytes() bytes, 256-byte aligned; its contents on entry do
+ * `out` (device, or pinned host memory as for qm_metric) receives the record.
+ * `ws` is device scratch of at least qm_stats_workspace_bytes() bytes, 256-byte aligned; its contents on entry do
  * not matter and concurrent calls must not share it.  The operand needs a unit
  * stride in one of its two dimensions and fewer than 2^32 groups of 8 elements.
  */

@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(kThreads, 2) simt_kernel(const SimtArgs a) {
         v[3] += __ldcg(rec + 3); v[4] += __ldcg(rec + 4);
       }
       block_reduce();
-      if (threadIdx.x == 0) {
+      if (threadIdx.x == 0) {                // (the record may be in host memory: stores only, every field once)
         a.result->sum_be = v[0]; a.result->max_be = v[1]; a.result->sum_diff2 = v[2];
         a.result->sum_ref2 = v[3]; a.result->sum_den2 = v[4];
         a.result->count = a.count;

@@ -1491,7 +1491,7 @@ __device__ __forceinline__ void write_results(const Table& tab, int ew, int lane
     const double x = warp_sum4(s4[0], s4[1], s4[2], s4[3], lane);
     mx = warp_max_f(mx);
     flags = __reduce_or_sync(0xffffffffu, flags);
-    if (lane == 0) {
+    if (lane == 0) {                         // (the record may be in host memory: stores only, every field once)
       a.result->sum_be = x; a.result->max_be = (double)mx;
       a.result->count = a.count; a.result->device_error = flags; a.result->reserved = 0;
     } else if (lane == 8) {

@@ -112,7 +112,7 @@ metric_finalize_kernel(const double* __restrict__ partials, int n, uint64_t coun
     s[threadIdx.x][0] = x;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0) {                    // (the record may be in host memory: stores only, every field once)
     out->sum_be = s[0][0]; out->max_be = s[1][0]; out->sum_diff2 = s[2][0];
     out->sum_ref2 = s[3][0]; out->sum_den2 = s[4][0];
     out->count = count;

@@ -326,6 +326,7 @@ __device__ __forceinline__ void finish_pass(Acc& acc, double* __restrict__ parti
     for (int w = 1; w < kThreads / 32; ++w) x = is_max<KIND>(i) ? fmax(x, red[i][w]) : x + red[i][w];
     tot[i] = x;
   }
+  // (the record may be in host memory: stores only, every field once)
   if (KIND == kStats) {
     qm_tensor_stats_result* r = static_cast<qm_tensor_stats_result*>(result);
     r->sum1 = tot[0]; r->sum2 = tot[1]; r->sum3 = tot[2]; r->sum4 = tot[3];
