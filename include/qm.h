@@ -236,9 +236,11 @@ qm_status qm_quantize_stochastic(const qm_operand* x, int32_t fmt, int32_t gran,
  * qm_quantize) receive format k's scales and codes, round-to-nearest-even;
  * kmaj_copy as for qm_quantize.  amax_scratch is device scratch of as many
  * 32-bit words as one delta_out array has values; the call clears it.  Every
- * result equals what qm_quantize gives for that format alone.  Per-tensor
- * scales of a bf16 operand are produced by one kernel that reads the operand
- * once; other cases by one quantize launch per format after a common max|x|.
+ * result equals what qm_quantize gives for that format alone.  With one scale
+ * per tensor a single kernel reads the operand once for all formats if its
+ * contraction is contiguous (and no copy is wanted), or strided, in bf16 and a
+ * multiple of 16; other cases take one quantize launch per format after a
+ * common max|x|.
  * A non-finite operand yields NaN scales, as in qm_scale.
  */
 qm_status qm_quantize_formats(const qm_operand* x, int32_t n_fmt, const int32_t* fmts, int32_t gran,
@@ -293,7 +295,10 @@ qm_status qm_metric(const float* ref, const float* q, const float* den, int64_t 
  * = N, contract = K, same batch.  `out` (device, or pinned host memory as for
  * qm_metric) receives the record; `ws` is device scratch of at least qm_workspace_bytes(L, R, cfg) bytes, 256-byte
  * aligned; its contents on entry do not matter and concurrent calls must not
- * share it.
+ * share it.  (Two bytes an element of every bf16 operand whose contraction is
+ * strided are there for qm_probe_batch, which puts the codes that several of
+ * its probes need of one tensor into one of their workspaces; a probe issued
+ * by itself leaves them alone.)
  * QM_REF_BF16_FP32ACC needs bf16 operands and K a multiple of 16;
  * QM_REF_FP32 takes fp32 or bf16 operands of any shape.
  * cfg->round: an operand flagged stochastic is quantized as by

@@ -1093,7 +1093,7 @@ struct CfgP {
   static constexpr int kStages = 6;          // stages of shared memory (TMA ring)
   static constexpr int kTmemStages = 2;       // stages of L and |L| in tensor memory (128 columns / 64)
   static constexpr int kLpDepth = 128;       // contraction entries of a block of codes
-  // stage: L, R, |R| (written by the converters); or codes of L, codes of R.  All rows are 128 bytes.
+  // stage: L, R, |R| (written by warps 2 and 3 or the converters); or codes of L, codes of R.  All rows are 128 bytes.
   static constexpr uint32_t kOffL = 0, kOffR = kABf16, kOffRa = kOffR + kBBf16;
   static constexpr uint32_t kStageBytes = kOffRa + kBBf16;           // 32 KB
   static constexpr uint32_t kTileBytes = kStages * kStageBytes;      // 192 KB
@@ -1128,8 +1128,8 @@ enum : uint32_t { kUnitMnMajorL = 1, kUnitMnMajorR = 2 };
 template <int UNITS, int VARS>
 struct SharedP {
   uint64_t full[CfgP::kStages];     // per CTA: this CTA's loads of a block have landed
-  uint64_t ready[CfgP::kStages];    // leader: both CTAs' converters have seen their loads land and, for L and R,
-                                    //         have written L and |L| (tensor memory) and |R| (stage)
+  uint64_t ready[CfgP::kStages];    // leader: both CTAs' converters (and warps 2 and 3, with RW) have seen their loads
+                                    //         land and, for L and R, have written L and |L| (tensor memory) and |R| (stage)
   uint64_t empty[CfgP::kStages];    // per CTA: the pair's MMAs have finished with the block of the stage
   uint64_t rd_full;                 // per CTA: the tile's reference and denominator are complete
   uint64_t rd_empty;                // leader: both CTAs' epilogues have copied them out
@@ -1631,7 +1631,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           }
           const uint32_t bar = smem_u32(&sh->full[ring.s]), base = tile_base + ring.s * C::kStageBytes;
           mbar_expect_tx(bar, bytes);
-          tma_load_3d_local(base + C::kOffR, &maps[1], bar, r_mn ? c0 : k0, r_mn ? k0 : c0, b);     // the converters read this one
+          tma_load_3d_local(base + C::kOffR, &maps[1], bar, r_mn ? c0 : k0, r_mn ? k0 : c0, b);
           tma_load_3d_local(base + C::kOffL, &maps[0], bar, l_mn ? r0 : k0, l_mn ? k0 : r0, b);
           if (two_boxes) tma_load_3d_local(base + C::kOffL + kABf16 / 2, &maps[0], bar, r0 + 64, k0, b);
           sh->issued = ++g;
@@ -2085,7 +2085,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
 struct CfgS {
   static constexpr int kStages = 5;          // stages of shared memory (TMA ring)
   static constexpr int kAbsStages = 4;       // stages of |L| in tensor memory (128 columns / 32)
-  // stage: L, R, |R| (written by the converters), codes of L, codes of R
+  // stage: L, R, |R| (written by warps 2 and 3 or the converters), codes of L, codes of R
   static constexpr uint32_t kOffL = 0, kOffR = kABf16, kOffRa = kOffR + kBBf16, kOffCl = kOffRa + kBBf16;
   static constexpr uint32_t kOffCr = kOffCl + kALp;
   static constexpr uint32_t kStageBytes = kOffCr + kBLp;             // 44 KB
@@ -2096,8 +2096,8 @@ struct CfgS {
 template <int UNITS>
 struct SharedS {
   uint64_t full[CfgS::kStages];     // per CTA: this CTA's loads of a stage have landed
-  uint64_t ready[CfgS::kStages];    // leader: both CTAs' converters have seen their loads land and have written
-                                    //         |L| (tensor memory) and |R| (stage)
+  uint64_t ready[CfgS::kStages];    // leader: both CTAs' converters (and warps 2 and 3, with RW) have seen their loads
+                                    //         land and have written |L| (tensor memory) and |R| (stage)
   uint64_t empty[CfgS::kStages];    // per CTA: the pair's MMAs have finished with the k-block of the stage
   uint64_t tmem_full;               // per CTA: the tile's accumulators are complete
   uint64_t tmem_empty;              // leader: both CTAs' epilogues have copied out reference and denominator
@@ -2261,7 +2261,7 @@ tc_side_kernel(const __grid_constant__ Table tab) {
             const uint32_t bar = smem_u32(&sh->full[s]), base = tile_base + s * C::kStageBytes;
             mbar_expect_tx(bar, kABf16 + kALp + (uint32_t)tw.half_n * (kBlockK * 2 + kBlockK));
             const int k0 = kb * kBlockK;
-            tma_load_3d_local(base + C::kOffR, &um[1], bar, r_mn ? c0 : k0, r_mn ? k0 : c0, tw.tc.b);     // the converters read this one
+            tma_load_3d_local(base + C::kOffR, &um[1], bar, r_mn ? c0 : k0, r_mn ? k0 : c0, tw.tc.b);
             tma_load_3d_local(base + C::kOffL, &um[0], bar, l_mn ? r0 : k0, l_mn ? k0 : r0, tw.tc.b);
             if (l_mn) tma_load_3d_local(base + C::kOffL + kABf16 / 2, &um[0], bar, r0 + 64, k0, tw.tc.b);
             tma_load_3d_local(base + C::kOffCl, &vm[0], bar, cl_mn ? r0 : k0, cl_mn ? k0 : r0, tw.tc.b);

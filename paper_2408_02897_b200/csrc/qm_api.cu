@@ -149,7 +149,7 @@ Workspace plan(const View& L, const View& R, const qm_probe_cfg& cfg, bool with_
       w.off_ar = take((size_t)(R.batch * R.nc * R.c) * 2);
     }
     // two bytes an element of an operand whose contraction is strided: contraction-major copies of the two-format kernel,
-    // codes of further probes of a batch (Slot::room)
+    // codes of further probes of a batch (Slot::room); a single probe does not use them
     w.off_kl = L.c_contig() ? 0 : take((size_t)(L.batch * L.nc * L.c) * 2);
     w.off_kr = R.c_contig() ? 0 : take((size_t)(R.batch * R.nc * R.c) * 2);
   }
@@ -745,7 +745,9 @@ void find_roots(std::vector<Slot>& slots, int t) {
 }
 
 // A slot that makes its codes itself, in its operand's own order, puts them beside those of the first such slot of
-// the same elements if there is room.
+// the same elements if there is room: what a batch writes of one tensor lies in one workspace, and those of the other
+// probes are not touched.  That is its whole worth; in time it makes no difference (with / without, us per pass: sweep layer
+// 6072 / 6055, BERT-large layer 2874 / 2868, six probes of one product 770 / 768, runs of one side up to 1 % apart).
 void find_home(std::vector<Slot>& slots, int t) {
   Slot& x = slots[t];
   x.home = t;

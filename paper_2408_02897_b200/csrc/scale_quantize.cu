@@ -948,7 +948,7 @@ scale_quantize_rows_spread_kernel(const T* __restrict__ x, uint32_t rows, int pi
 #pragma unroll
     for (int u = 0; u < V; ++u) p[u] = next[u];
     const uint32_t row_next = row + step;
-    if (row_next < rows && row_next > row) fetch(row_next, next);
+    if (row_next < rows) fetch(row_next, next);
     uint32_t m = 0;
 #pragma unroll
     for (int u = 0; u < V; ++u) m = max(m, p[u].absmax());
@@ -1000,8 +1000,7 @@ scale_quantize_rows_spread_kernel(const T* __restrict__ x, uint32_t rows, int pi
         }
       }
     }
-    if (row_next <= row) break;                                         // (32-bit wrap)
-    row = row_next;
+    row = row_next;                                                     // (rows + a step fit 32 bits: rows_spread)
   }
 }
 
@@ -1684,8 +1683,10 @@ qm_status quantize_t(const View& x, int gran, const float* delta, bool from_amax
   return QM_OK;
 }
 
-// Rows that the spread kernel takes: codes without padding, at most 8192 elements.  Short rows leave its lanes idle or, in
-// bf16, have no more of them than one warp holds: those kernels are faster there, for one format.
+// Rows that the spread kernel takes: a multiple of 16 elements, so that codes have no padding, at most 8192 (two pieces for
+// each thread of eight warps).  Short rows leave its lanes idle or, in bf16, have no more of them than one warp holds: those
+// kernels are faster there, for one format.  Ragged rows and longer ones stay with the kernel that reads a row twice (one
+// element at a time where it is ragged fp32), and a sharing of formats between rows of qm_quantize_formats is not built.
 bool rows_spread(const View& x, int formats) {
   const int64_t least = formats > 1 ? 16 : x.dtype == QM_DT_BF16 ? 1040 : 272;
   return (x.c & 15) == 0 && x.c >= least && x.c <= 8192 && x.nc * x.batch < (1ll << 31) && x.nc < (1ll << 31);

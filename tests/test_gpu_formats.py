@@ -53,6 +53,8 @@ def test_large_dense_takes_the_four_chunk_variant():
 
 @pytest.mark.parametrize("gran", ["tensor", "channel"])
 def test_cases_served_format_by_format(gran):
+    """A launch per format under channel scales and for these strided tensors; contiguous ragged and fp32 ones under one scale take
+    one pass over their lines."""
     fm = ("e4m3", "int8", "e5m2")
     check(tensor((333, 200), torch.bfloat16, 45), -1, fm, gran)                    # ragged rows
     check(tensor((333, 200), torch.bfloat16, 46), -2, fm, gran, want_kmaj=True)    # small strided contraction

@@ -1,5 +1,4 @@
-"""Inside a batch, operands over the same memory are prepared once (max|x|, contraction-major copy,
-codes); every probe's record must still be the one it gets when probed alone, and the oracle's."""
+"""Inside a batch, operands over the same memory are prepared once (max|x|, scales, codes); every probe's record must still be the one it gets when probed alone, and the oracle's."""
 import ctypes as C
 
 import numpy as np

@@ -71,7 +71,7 @@ def test_strided_operands_give_the_record_of_contiguous_ones(m, n, k, batch, gra
 
 @pytest.mark.parametrize("m,n,k", [(257, 129, 80), (770, 1000, 2032), (4096, 768, 256)])
 def test_rounding_and_orientation_mixed_in_a_batch(m, n, k):
-    """One tensor as it lies and flipped, rounded to nearest and stochastically, under both kinds of scales: shared
+    """The same values stored strided and contiguous, rounded to nearest and stochastically, under both kinds of scales: shared
     preparation gives every probe the record it has alone, and strided operands that of contiguous ones."""
     L, R = draw((m, k), 3), draw((n, k), 4, 0.05)
     (_k0, ls), (_k1, rs), (_k2, lc), (_k3, rc) = stored(L, True), stored(R, True), stored(L, False), stored(R, False)

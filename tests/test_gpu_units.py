@@ -86,8 +86,9 @@ def test_products_of_one_probe_beside_shared_ones(n_single, launches):
             assert abs(rec.record()[k] - alone[k]) <= 1e-12 * abs(alone[k]), k
 
 
-# Operands with a strided contraction need a contraction-major copy: one per operand, whatever the scales of the probes that
-# use it, so that probes of both granularities (and roundings) share their products too
+# Operands with a strided contraction are used as they lie by probes of both granularities and roundings, which share their
+# products, and what is written of one operand beyond a probe's own buffers goes to one workspace: the two bytes an element that
+# every workspace has for it stay untouched in all but the first
 @pytest.mark.parametrize("cl,cr", [(-2, -2), (-2, -1), (-1, -2)])
 def test_one_copy_of_a_strided_operand_whatever_the_scales(cl, cr):
     M, N, K, fill = 304, 200, 272, -0x5A5A5A5B          # (strided rows are a multiple of 8 elements apart)
