@@ -273,7 +273,7 @@ class _HostRecord:
 
     def __init__(self, kind):
         self.kind = kind
-        self.buf = torch.empty(C.sizeof(kind), dtype=torch.uint8, pin_memory=True)
+        self.buf = torch.empty(C.sizeof(kind), dtype=torch.uint8, device="cpu", pin_memory=True)
         self.ptr = self.buf.data_ptr()
 
     def read(self, stream):

@@ -51,3 +51,17 @@ def test_a_record_is_the_same_in_device_and_in_pinned_memory(name):
             torch.cuda.synchronize()
             got.append(bytes(buf.cpu().numpy().tobytes()))
     assert all(g == got[0] for g in got), got
+
+
+def test_calls_under_a_default_device():
+    """A program that lets torch put its tensors on the GPU by default makes the same calls."""
+    g = torch.Generator().manual_seed(12)
+    x = torch.randn((64, 272), generator=g).to(torch.bfloat16).cuda()
+    op, m = qm.operand_of(x, -1), x.float().flatten()
+
+    def records():
+        probe, metric = qm.qm_probe_layer(op, op, "e4m3", "e4m3", "tensor", "tensor"), qm.qm_metric(m, m * 1.01, m.abs())
+        return probe.record(), metric.record(), qm.qm_tensor_stats(op).derived(), qm.qm_quantize_error(op, "int8", "tensor").record()
+    want = records()
+    with torch.device("cuda"):
+        assert records() == want
