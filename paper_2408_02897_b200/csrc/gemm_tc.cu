@@ -1028,11 +1028,10 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 // reference and denominator products run once, then the 8-bit products of the unit's probes
 // (VARIANTS, up to kMaxVar) one after the other, each over the whole contraction.
 //
-// The tiles of all units form one sequence.  The host orders the units by descending tile cost and
-// the sequence is dealt to the CTA pairs back and forth (round r gives pair p position r P + p when r
-// is even and r P + P-1-p when it is odd), which for descending costs balances the pairs to within
-// one tile of the cheapest kind.  The operand maps, scales, shapes and the 8-bit MMA kinds come
-// from a table in the kernel's parameter space.  A pair's positions increase, so it meets each unit in
+// The host orders the units by descending tile cost and deals the tiles of each to the CTA pairs with the least
+// to do so far (TileDeal), which balances the pairs to within one tile of the cheapest kind; the deal is fixed, so that records
+// are the same from run to run.  The operand maps, scales, shapes and the 8-bit MMA kinds come
+// from a table in the kernel's parameter space.  A pair meets each unit in
 // one run: when the unit changes, the epilogue warps reduce their statistics and write the CTA's
 // records of the probes they leave.
 //
@@ -1116,11 +1115,16 @@ __device__ __forceinline__ uint32_t divide(uint32_t n, uint32_t mul, uint32_t sh
 // launch's table sits in the kernel's parameter space, and reads of it with an index known only
 // at run time go through the small constant cache, which a table of this size thrashes.
 struct alignas(16) WalkInfo {
-  int32_t tile_begin, per_b, inner, num_kb;         // per_b = tiles_m * tiles_n (tiles per batch element);
-                                                    // inner = tiles_n: column tiles run fastest, -tiles_m: row tiles do
-  int32_t half_n, n_var, var_begin, K;              // half_n: kUnitMnMajor... above its low byte
+  int32_t n_tiles, n_lead, lead0, main0;            // this pair's tiles of the unit: lead0 + j for its j-th tile while
+                                                    // j < n_lead, then main0 + j * pairs, the last one `last` unless -1
+  int32_t per_b, inner, num_kb, half_n;             // per_b = tiles_m * tiles_n (tiles per batch element);
+                                                    // inner = tiles_n: column tiles run fastest, -tiles_m: row tiles do;
+                                                    // half_n: kUnitMnMajor... above its low byte
   uint32_t b_mul, b_shift, i_mul, i_shift;          // division by per_b and by the absolute value of inner (Divisor)
+  int32_t n_var, var_begin, K, last;
 };
+// Of a probe: the instruction descriptor of its 8-bit MMA, and kVar...; per-channel scales are indexed by batch * M + row,
+// batch * N + column.
 struct VarInfo { uint32_t idesc, flags; };
 enum : uint32_t { kVarI8 = 1, kVarScalePerRow = 2, kVarScalePerCol = 4, kVarRowStats = 8, kVarMnMajorL = 16, kVarMnMajorR = 32 };
 enum : uint32_t { kUnitMnMajorL = 1, kUnitMnMajorR = 2 };
@@ -1151,11 +1155,12 @@ struct SharedP {
   VarInfo var[VARS];
 };
 
+constexpr int kMaxPairs = 80;               // CTA pairs of a launch, at most (148 SMs hold 74)
 struct GroupUnit {
-  CUtensorMap maps[2];        // L, R
   int32_t M, N, K;
   int32_t tiles_m, tiles_n;
-  int32_t tile_begin;         // position of its first tile in the sequence
+  int32_t rounds;             // tiles that every pair takes of it, after those of GroupTable::lead
+  uint32_t last[(kMaxPairs + 31) / 32];   // bit p: pair p takes one more after them
   int32_t half_n;             // right-operand rows each CTA stages: 64, or 32 for outputs at most 64 wide
   int32_t m_fastest;          // the tiles of a batch element are walked down the rows first (below)
   uint32_t major;             // kUnitMnMajor...: bf16 operands stored with the contraction strided
@@ -1163,7 +1168,6 @@ struct GroupUnit {
   int32_t var_begin, n_var;
 };
 struct GroupVar {
-  CUtensorMap maps[2];        // codes of L, codes of R
   const float* dl; const float* dr;
   double* partials;           // gridDim.x records
   qm_metric_result* result;
@@ -1171,19 +1175,21 @@ struct GroupVar {
   uint32_t* err_word;
   const uint32_t* err_also[2];           // further error words to report in the record, or null
   uint64_t count;             // batch * M * N
-  uint32_t flags;             // kVar...; per-channel scales are indexed by batch * M + row, batch * N + column
-  uint32_t idesc_lp;          // instruction descriptor of the 8-bit MMA
+  VarInfo info;
 };
 template <int UNITS, int VARS>
 struct GroupTable {
   static constexpr int kUnits = UNITS, kVars = VARS;
-  int32_t n, n_var, total_tiles;
+  CUtensorMap unit_maps[UNITS][2];        // L, R
+  CUtensorMap var_maps[VARS][2];          // codes of L, codes of R
+  int32_t n, n_var;
   uint32_t stop_after_kb;     // test hook: the producer issues no block beyond this many (0xffffffff: off)
   uint64_t wait_limit_ns;     // bound of every barrier wait
   uint32_t* done_counter;     // zero on entry; counts finished CTAs
   uint32_t* err0;             // a wait that runs out is reported here and in every record
   GroupUnit u[UNITS];
   GroupVar v[VARS];
+  uint16_t lead[UNITS][kMaxPairs + 1];    // prefix sums over the pairs of the tiles that each takes ahead of the unit's rounds
 };
 // A launch's table has to fit into 32 764 bytes of kernel parameters.  24 units hold the 18 products
 // of an encoder layer in one launch; a probe on its own passes a table of its own size (1 KB).
@@ -1191,68 +1197,47 @@ using TableBig = GroupTable<24, 56>;
 using TableOne = GroupTable<1, 1>;
 static_assert(sizeof(TableBig) <= 32764, "kernel parameters");
 
-// position of pair `pair` in round r of the back-and-forth deal
-__device__ __forceinline__ int group_position(int r, int pair, int num_pairs) {
-  return r * num_pairs + ((r & 1) ? num_pairs - 1 - pair : pair);
-}
-
-// The tiles of one CTA pair in order: every role walks the same sequence.
-// A pair's positions ascend, so the search for a position's unit continues from the unit in hand.
-struct TileWalk {
-  const WalkInfo* wk;
-  int n, total_tiles;
-  int r, pair, num_pairs;
-  int pi, num_kb, half_n, n_var, var_begin, K;
+// What a unit asks of every role, read once per unit: the same in all lanes, and known to be (the shuffles).  A tile's own
+// code is kept short by this: 512 x 512 x 64 x 256 in one format 95 us with one loop over tiles that looks its unit up, 87 so.
+struct UnitInfo {
+  int n_tiles, num_kb, half_n, n_var, var_begin, K;
   uint32_t major;
-  TileCoord tc;
-  bool valid;
-  __device__ __forceinline__ void start(const WalkInfo* wk_, int n_, int total_tiles_, int pair_, int num_pairs_) {
-    wk = wk_; n = n_; total_tiles = total_tiles_;
-    r = -1; pair = pair_; num_pairs = num_pairs_; num_kb = 0; pi = 0; half_n = 0; major = 0; valid = true;
-    next_tile();
-  }
-  // moves to the pair's next tile; valid = false when there is none
-  __device__ __forceinline__ void next_tile() {
-    while (true) {
-      ++r;
-      const int pos = group_position(r, pair, num_pairs);
-      if (pos >= total_tiles) {
-        if (r * num_pairs >= total_tiles) { valid = false; return; }   // no round reaches further
-        continue;
-      }
-      while (pi + 1 < n && pos >= wk[pi + 1].tile_begin) ++pi;
-      const int4 w4 = reinterpret_cast<const int4*>(&wk[pi])[0];        // tile_begin, per_b, inner, num_kb
-      const int4 x4 = reinterpret_cast<const int4*>(&wk[pi])[1];        // half_n, n_var, var_begin, K
-      const uint4 d4 = reinterpret_cast<const uint4*>(&wk[pi])[2];
-      const uint32_t t = (uint32_t)(pos - w4.x), b = divide(t, d4.x, d4.y);
-      tc.b = (int)b;
-      const uint32_t rem = t - b * (uint32_t)w4.y;
-      const int inner = w4.z < 0 ? -w4.z : w4.z;
-      const int outer_i = (int)divide(rem, d4.z, d4.w), inner_i = (int)rem - outer_i * inner;
-      tc.m_tile = w4.z < 0 ? inner_i : outer_i;
-      tc.n_tile = w4.z < 0 ? outer_i : inner_i;
-      num_kb = w4.w;
-      half_n = x4.x & 255; major = (uint32_t)x4.x >> 8; n_var = x4.y; var_begin = x4.z; K = x4.w;
-      return;
-    }
-  }
-  // what the MMA warp needs, known to be the same in all lanes
-  __device__ __forceinline__ void make_uniform() {
-    num_kb = __shfl_sync(0xffffffffu, num_kb, 0);
-    half_n = __shfl_sync(0xffffffffu, half_n, 0);
-    major = __shfl_sync(0xffffffffu, major, 0);
-    n_var = __shfl_sync(0xffffffffu, n_var, 0);
-    var_begin = __shfl_sync(0xffffffffu, var_begin, 0);
-    K = __shfl_sync(0xffffffffu, K, 0);
+  __device__ __forceinline__ explicit UnitInfo(const WalkInfo& w) {
+    constexpr uint32_t all = 0xffffffffu;
+    n_tiles = __shfl_sync(all, w.n_tiles, 0);
+    num_kb = __shfl_sync(all, w.num_kb, 0);
+    const int h = __shfl_sync(all, w.half_n, 0);
+    half_n = h & 255; major = (uint32_t)h >> 8;
+    n_var = __shfl_sync(all, w.n_var, 0);
+    var_begin = __shfl_sync(all, w.var_begin, 0);
+    K = __shfl_sync(all, w.K, 0);
   }
   __device__ __forceinline__ int lp_blocks() const { return (K + CfgP::kLpDepth - 1) / CfgP::kLpDepth; }
 };
+// The pair's j-th tile of a unit.  Every role goes through the units and their tiles in the same order; the producer
+// and the epilogue also need to know where the tiles are.
+__device__ __forceinline__ TileCoord pair_tile(const WalkInfo& w, int j, int num_pairs) {
+  const int4 s4 = reinterpret_cast<const int4*>(&w)[0];        // n_tiles, n_lead, lead0, main0
+  const int4 w4 = reinterpret_cast<const int4*>(&w)[1];        // per_b, inner, num_kb, half_n
+  const uint4 d4 = reinterpret_cast<const uint4*>(&w)[2];
+  const uint32_t t = (uint32_t)(j + 1 == s4.x && w.last >= 0 ? w.last : j < s4.y ? s4.z + j : s4.w + j * num_pairs);
+  const uint32_t b = divide(t, d4.x, d4.y);
+  const uint32_t rem = t - b * (uint32_t)w4.x;
+  const int inner = w4.y < 0 ? -w4.y : w4.y;
+  const int outer_i = (int)divide(rem, d4.z, d4.w), inner_i = (int)rem - outer_i * inner;
+  TileCoord tc;
+  tc.b = (int)b;
+  tc.m_tile = w4.y < 0 ? inner_i : outer_i;
+  tc.n_tile = w4.y < 0 ? outer_i : inner_i;
+  return tc;
+}
 
-// Position in the ring of stages.
+// Position in a ring of stages.
+template <int STAGES>
 struct Ring {
   uint32_t s = 0, parity = 0;       // stage, and the parity of its use
   __device__ __forceinline__ void next() {
-    if (++s == (uint32_t)CfgP::kStages) { s = 0; parity ^= 1u; }
+    if (++s == (uint32_t)STAGES) { s = 0; parity ^= 1u; }
   }
 };
 
@@ -1428,20 +1413,37 @@ __device__ __forceinline__ void eval_variant(uint32_t taddr, const uint32_t (&rc
   }
 }
 
-// The walk and variant tables of a launch into shared memory (one warp).
+// The first unit that gives the pair a tile.
+template <typename Table>
+__device__ __forceinline__ int first_unit(const Table& tab, int pair) {
+  int pi = 0;
+  while (pi + 1 < tab.n && tab.u[pi].rounds == 0 && tab.lead[pi][pair + 1] == tab.lead[pi][pair] && !(tab.u[pi].last[pair >> 5] >> (pair & 31) & 1u)) ++pi;
+  return pi;
+}
+// The walk of this pair and the variant table of a launch into shared memory (one warp).
 template <typename Sh, typename Table>
-__device__ __forceinline__ void fill_walk(Sh* sh, const Table& tab, int lane) {
+__device__ __forceinline__ void fill_walk(Sh* sh, const Table& tab, int lane, int pair, int num_pairs) {
   for (int i = lane; i < tab.n; i += 32) {
     const GroupUnit& u = tab.u[i];
     WalkInfo wi;
-    wi.tile_begin = u.tile_begin; wi.per_b = u.tiles_m * u.tiles_n;
+    wi.lead0 = tab.lead[i][pair];
+    wi.n_lead = tab.lead[i][pair + 1] - wi.lead0;
+    wi.n_tiles = wi.n_lead + u.rounds;
+    wi.main0 = tab.lead[i][num_pairs] + pair - wi.n_lead * num_pairs;
+    wi.last = -1;
+    if (u.last[pair >> 5] >> (pair & 31) & 1u) {
+      wi.last = tab.lead[i][num_pairs] + u.rounds * num_pairs + __popc(u.last[pair >> 5] & ((1u << (pair & 31)) - 1u));
+      for (int k = 0; k < pair >> 5; ++k) wi.last += __popc(u.last[k]);
+      ++wi.n_tiles;
+    }
+    wi.per_b = u.tiles_m * u.tiles_n;
     wi.inner = u.m_fastest ? -u.tiles_m : u.tiles_n;
     wi.num_kb = (u.K + kBlockK - 1) / kBlockK;
     wi.half_n = u.half_n | (int32_t)(u.major << 8); wi.n_var = u.n_var; wi.var_begin = u.var_begin; wi.K = u.K;
     wi.b_mul = u.b_mul; wi.b_shift = u.b_shift; wi.i_mul = u.i_mul; wi.i_shift = u.i_shift;
     sh->walk[i] = wi;
   }
-  for (int i = lane; i < tab.n_var; i += 32) sh->var[i] = VarInfo{tab.v[i].idesc_lp, tab.v[i].flags};
+  for (int i = lane; i < tab.n_var; i += 32) sh->var[i] = tab.v[i].info;
 }
 
 // Sums of four values over the warp, six exchanges instead of twenty: lanes 8 k .. 8 k + 7 return the sum of v[k].
@@ -1564,11 +1566,9 @@ tc_group_kernel(const __grid_constant__ Table tab) {
 
   if (warp == 0) {
     // fetch the operand maps of this pair's first tile into the descriptor cache
-    const int pos = group_position(0, pair, num_pairs);
-    if (pos < tab.total_tiles && lane < 4) {
-      int pi = 0;
-      while (pi + 1 < tab.n && pos >= tab.u[pi + 1].tile_begin) ++pi;
-      const CUtensorMap* m = lane < 2 ? &tab.u[pi].maps[lane] : &tab.v[tab.u[pi].var_begin].maps[lane - 2];
+    if (lane < 4) {
+      const int pi = first_unit(tab, pair);
+      const CUtensorMap* m = lane < 2 ? &tab.unit_maps[pi][lane] : &tab.var_maps[tab.u[pi].var_begin][lane - 2];
       asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
     }
   }
@@ -1596,16 +1596,14 @@ tc_group_kernel(const __grid_constant__ Table tab) {
                      smem_u32(&sh->tmem_base)), "r"(512u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
-  if (warp == 2) fill_walk(sh, tab, lane);
+  if (warp == 2) fill_walk(sh, tab, lane, pair, num_pairs);
   tc_fence_before();
   __syncthreads();
   __syncwarp();
   cluster_arrive();
   tc_fence_after();
   const uint32_t tmem_base = sh->tmem_base;
-  // every warp: the pair's first tile, found while the cluster barrier completes
-  auto begin = [&](TileWalk& tw) {
-    tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
+  auto begin = [&]() {
     __syncwarp();
     cluster_wait();        // the peer's barriers and tensor memory exist before anyone uses them
     pdl_prologue();        // everything above overlapped the tail of the previous kernel
@@ -1616,10 +1614,9 @@ tc_group_kernel(const __grid_constant__ Table tab) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsCtl));
     if (warp == 0) {
       // ---------------------------------------------------------- TMA producer (both CTAs)
-      TileWalk tw;
-      begin(tw);
+      begin();
       if (lane == 0) {
-        Ring ring;
+        Ring<kStages> ring;
         uint32_t g = 0;
         bool ok = true;
         // a mn-major tile has the operand's rows as its inner coordinate; of bf16, 128 of them are two boxes
@@ -1637,27 +1634,32 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           sh->issued = ++g;
           ring.next();
         };
-        for (; tw.valid && ok; tw.next_tile()) {
-          const int r0 = tw.tc.m_tile * kPairM + (int)rank * kBlockM;     // this CTA's left-operand rows
-          const int c0 = tw.tc.n_tile * kBlockN + (int)rank * tw.half_n;  // this CTA's half of the right operand
-          const uint32_t bytes = kABf16 + (uint32_t)tw.half_n * 128u;
-          const bool l_mn = MN && (tw.major & kUnitMnMajorL), r_mn = MN && (tw.major & kUnitMnMajorR);
-          for (int kb = 0; kb < tw.num_kb && ok; ++kb)
-            load(tab.u[tw.pi].maps, bytes, kb * kBlockK, r0, c0, tw.tc.b, l_mn, r_mn, l_mn);
-          const int nb = tw.lp_blocks();
-          for (int f = 0; f < tw.n_var && ok; ++f) {
-            const uint32_t flags = sh->var[tw.var_begin + f].flags;
-            for (int kb = 0; kb < nb && ok; ++kb)
-              load(tab.v[tw.var_begin + f].maps, bytes, kb * C::kLpDepth, r0, c0, tw.tc.b, MN && (flags & kVarMnMajorL), MN && (flags & kVarMnMajorR), false);
+        for (int pi = 0; pi < tab.n && ok; ++pi) {
+          const WalkInfo& wk = sh->walk[pi];
+          const int n_tiles = wk.n_tiles, num_kb = wk.num_kb, half_n = wk.half_n & 255, n_var = wk.n_var, v0 = wk.var_begin;
+          const uint32_t major = (uint32_t)wk.half_n >> 8;
+          const int nb = (wk.K + C::kLpDepth - 1) / C::kLpDepth;
+          const uint32_t bytes = kABf16 + (uint32_t)half_n * 128u;
+          const bool l_mn = MN && (major & kUnitMnMajorL), r_mn = MN && (major & kUnitMnMajorR);
+          for (int j = 0; j < n_tiles && ok; ++j) {
+            const TileCoord tc = pair_tile(wk, j, num_pairs);
+            const int r0 = tc.m_tile * kPairM + (int)rank * kBlockM;     // this CTA's left-operand rows
+            const int c0 = tc.n_tile * kBlockN + (int)rank * half_n;     // this CTA's half of the right operand
+            for (int kb = 0; kb < num_kb && ok; ++kb)
+              load(tab.unit_maps[pi], bytes, kb * kBlockK, r0, c0, tc.b, l_mn, r_mn, l_mn);
+            for (int f = 0; f < n_var && ok; ++f) {
+              const uint32_t flags = sh->var[v0 + f].flags;
+              for (int kb = 0; kb < nb && ok; ++kb)
+                load(tab.var_maps[v0 + f], bytes, kb * C::kLpDepth, r0, c0, tc.b, MN && (flags & kVarMnMajorL), MN && (flags & kVarMnMajorR), false);
+            }
           }
         }
       }
     } else if (warp == 1 && rank == 0) {
       // ---------------------------------------------------------- MMA issuer (leader CTA, converged warp)
       const bool lead = elect_one();
-      TileWalk tw;
-      begin(tw);
-      Ring ring;
+      begin();
+      Ring<kStages> ring;
       auto wait_block = [&]() {
         if (!w.wait_warp(smem_u32(&sh->ready[ring.s]), ring.parity)) return false;
         tc_fence_after();
@@ -1690,15 +1692,18 @@ tc_group_kernel(const __grid_constant__ Table tab) {
       uint32_t lp_uses0 = 0, lp_uses1 = 0;           // variants put into each 8-bit accumulator so far
       bool ok = true;
       uint32_t it = 0;
-      for (; tw.valid && ok; ++it, tw.next_tile()) {
+      for (int pi = 0; pi < tab.n && ok; ++pi) {
+       const UnitInfo tw(sh->walk[pi]);
+       const bool r_mn = MN && (tw.major & kUnitMnMajorR);  // (A comes from tensor memory, contraction-major always)
+       const uint32_t idesc_ref = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n) | (r_mn ? kIdescMnMajorB : 0u);
+       rd = tile_desc(r_mn, r_mn ? 2u * tw.half_n : 128u, 16u, 16u);
+       const int nb = tw.lp_blocks();
+       for (int j = 0; j < tw.n_tiles && ok; ++j, ++it) {
         // the reference and denominator blocks come back when both epilogues have copied the
         // previous tile's values out
-        if (it > 0 && !w.wait_warp(smem_u32(&sh->rd_empty), (it - 1) & 1)) break;
+        ok = it == 0 || w.wait_warp(smem_u32(&sh->rd_empty), (it - 1) & 1);
+        if (!ok) break;
         tc_fence_after();
-        tw.make_uniform();
-        const bool r_mn = MN && (tw.major & kUnitMnMajorR);  // (A comes from tensor memory, contraction-major always)
-        const uint32_t idesc_ref = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n) | (r_mn ? kIdescMnMajorB : 0u);
-        rd = tile_desc(r_mn, r_mn ? 2u * tw.half_n : 128u, 16u, 16u);
         for (int kb = 0; kb < tw.num_kb; ++kb) {
           ok = wait_block();
           if (!ok) break;
@@ -1707,7 +1712,6 @@ tc_group_kernel(const __grid_constant__ Table tab) {
         }
         if (!ok) break;
         tc_commit_pair(smem_u32(&sh->rd_full), lead);
-        const int nb = tw.lp_blocks();
         for (int f = 0; f < tw.n_var && ok; ++f) {
           const int b = (tw.n_var - 1 - f) & 1;
           const uint32_t idesc = __shfl_sync(0xffffffffu, sh->var[tw.var_begin + f].idesc, 0);
@@ -1734,16 +1738,17 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           if (ok) tc_commit_pair(smem_u32(&sh->lp_full[b]), lead);
           if (b) ++lp_uses1; else ++lp_uses0;
         }
+       }
       }
     } else if (RW && warp >= 2) {
       // ---------------------------------------------------------- |R| (both CTAs)
-      TileWalk tw;
-      begin(tw);
+      begin();
       const int t = (warp - 2) * 32 + lane;        // 0..63
       const uint32_t ready_leader = map_to_cta(smem_u32(&sh->ready[0]), 0);
-      Ring ring;
+      Ring<kStages> ring;
       bool ok = true;
-      for (; tw.valid && ok; tw.next_tile()) {
+      for (int pi = 0; pi < tab.n && ok; ++pi)
+       for (UnitInfo tw(sh->walk[pi]); tw.n_tiles > 0 && ok; --tw.n_tiles) {
         for (int kb = 0; kb < tw.num_kb && ok; ++kb) {
           ok = w.wait_warp(smem_u32(&sh->full[ring.s]), ring.parity);
           if (!ok) break;
@@ -1762,8 +1767,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
         }
       }
     } else {
-      TileWalk tw;
-      begin(tw);
+      begin();
     }
   } else if (warp < kFirstEpiWarp) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsConv));
@@ -1780,13 +1784,13 @@ tc_group_kernel(const __grid_constant__ Table tab) {
     const uint32_t ready_leader = map_to_cta(smem_u32(&sh->ready[0]), 0);
     const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + C::kColL;
     const uint32_t row_off = (uint32_t)t * 128u, sw = (uint32_t)t & 7u, m = 0x7fff7fffu;
-    TileWalk tw;
-    begin(tw);
-    Ring ring;
+    begin();
+    Ring<kStages> ring;
     uint32_t it = 0, abs_uses = 0;                 // completions of abs_free awaited so far
     bool lent = false;                             // the previous tile's variants have used the L columns
     bool ok = true;
-    for (; tw.valid && ok; ++it, tw.next_tile()) {
+    for (int pi = 0; pi < tab.n && ok; ++pi)
+     for (UnitInfo tw(sh->walk[pi]); tw.n_tiles > 0 && ok; --tw.n_tiles, ++it) {
       // the L columns are free once the previous tile's denominator is complete and whatever
       // variants it put there have been read
       if (it > 0) ok = w.wait_warp(smem_u32(&sh->rd_full), (it - 1) & 1);
@@ -1898,11 +1902,13 @@ tc_group_kernel(const __grid_constant__ Table tab) {
     int pM = 0, pN = 0;                            // of the unit in hand; below 2^31 (its tensor maps require it)
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
     uint32_t lp_parity = 0;                        // bit b: parity of the next use of 8-bit accumulator b
-    bool dead = false;                             // a wait for an 8-bit accumulator ran out
-    TileWalk tw;
-    begin(tw);
-    for (uint32_t it = 0; tw.valid; ++it) {
-      const int pi = tw.pi, n_var = tw.n_var, v0 = tw.var_begin;
+    bool dead = false;                             // a wait for an accumulator ran out
+    begin();
+    uint32_t it = 0;
+    for (int pi = 0; pi < tab.n && !dead; ++pi) {
+     const UnitInfo tw(sh->walk[pi]);
+     const int n_var = tw.n_var, v0 = tw.var_begin;
+     for (int j = 0; j < tw.n_tiles; ++j, ++it) {
       if (pi != cur) {
         if (cur >= 0) flush(cur);
         cur = pi;
@@ -1912,11 +1918,12 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           if (lane < 16) { sh->sums[v][ew][lane] = make_double2(0.0, 0.0); sh->maxima[v][ew][lane] = 0.f; }
         if (et < n_var) {                           // read after the barrier below
           const GroupVar& gv = tab.v[v0 + et];
-          sh->dl_tensor[et] = gv.flags & kVarScalePerRow ? 1.f : __ldg(gv.dl);
-          sh->dr_tensor[et] = gv.flags & kVarScalePerCol ? 1.f : __ldg(gv.dr);
+          const uint32_t flags = sh->var[v0 + et].flags;
+          sh->dl_tensor[et] = flags & kVarScalePerRow ? 1.f : __ldg(gv.dl);
+          sh->dr_tensor[et] = flags & kVarScalePerCol ? 1.f : __ldg(gv.dr);
         }
       }
-      const TileCoord tc = tw.tc;
+      const TileCoord tc = pair_tile(sh->walk[pi], j, num_pairs);
       for (int v = 0; v < n_var; ++v) {
         if ((sh->var[v0 + v].flags & kVarScalePerCol) && et < kBlockN) {
           const int col = tc.n_tile * kBlockN + et;
@@ -1934,7 +1941,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
 
       const bool ok = !dead && w.wait(smem_u32(&sh->rd_full), it & 1);
       // one barrier publishes the scales and makes the give-up decision uniform over the epilogue
-      if (epi_barrier_any(!ok)) break;
+      if (epi_barrier_any(!ok)) { dead = true; break; }
       tc_fence_after();
       uint32_t rc[64], rd[64];
       tmem_ld32(lane_addr + C::kColRef + cbase, *reinterpret_cast<uint32_t(*)[32]>(&rc[0]));
@@ -2038,7 +2045,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           sh->maxima[f][ew][lane] = fmaxf(sh->maxima[f][ew][lane], mx);
         }
       }
-      tw.next_tile();
+     }
     }
     if (cur >= 0) flush(cur);
     // the records of the probes this CTA never met are zero
@@ -2193,11 +2200,9 @@ tc_side_kernel(const __grid_constant__ Table tab) {
 
   if (warp == 0) {
     // fetch the tensor maps of this pair's first tile into the descriptor cache
-    const int pos = group_position(0, pair, num_pairs);
-    if (pos < tab.total_tiles && lane < 4) {
-      int pi = 0;
-      while (pi + 1 < tab.n && pos >= tab.u[pi + 1].tile_begin) ++pi;
-      asm volatile("prefetch.tensormap [%0];" ::"l"(lane < 2 ? &tab.u[pi].maps[lane] : &tab.v[pi].maps[lane - 2]) : "memory");
+    if (lane < 4) {
+      const int pi = first_unit(tab, pair);
+      asm volatile("prefetch.tensormap [%0];" ::"l"(lane < 2 ? &tab.unit_maps[pi][lane] : &tab.var_maps[pi][lane - 2]) : "memory");
     }
   }
   if (threadIdx.x == 0) {
@@ -2220,16 +2225,14 @@ tc_side_kernel(const __grid_constant__ Table tab) {
                      smem_u32(&sh->tmem_base)), "r"(512u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
-  if (warp == 2) fill_walk(sh, tab, lane);
+  if (warp == 2) fill_walk(sh, tab, lane, pair, num_pairs);
   tc_fence_before();
   __syncthreads();
   __syncwarp();
   cluster_arrive();
   tc_fence_after();
   const uint32_t tmem_base = sh->tmem_base;
-  // every warp: the pair's first tile, found while the cluster barrier completes
-  auto begin = [&](TileWalk& tw) {
-    tw.start(sh->walk, tab.n, tab.total_tiles, pair, num_pairs);
+  auto begin = [&]() {
     __syncwarp();
     cluster_wait();        // the peer's barriers and tensor memory exist before anyone uses them
     pdl_prologue();        // everything above overlapped the tail of the previous kernel
@@ -2240,33 +2243,39 @@ tc_side_kernel(const __grid_constant__ Table tab) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsCtl));
     if (warp == 0) {
       // ---------------------------------------------------------- TMA producer (both CTAs)
-      TileWalk tw;
-      begin(tw);
+      begin();
       if (lane == 0) {
+        Ring<kStages> ring;
         uint32_t g = 0;
         bool ok = true;
-        for (; tw.valid && ok; tw.next_tile()) {
-          const CUtensorMap* const um = tab.u[tw.pi].maps;
-          const CUtensorMap* const vm = tab.v[tw.pi].maps;
-          const int r0 = tw.tc.m_tile * kPairM + (int)rank * kBlockM;     // this CTA's left-operand rows
-          const int c0 = tw.tc.n_tile * kBlockN + (int)rank * tw.half_n;  // this CTA's half of the right operand
-          const uint32_t flags = sh->var[tw.pi].flags;
-          const bool l_mn = MN && (tw.major & kUnitMnMajorL), r_mn = MN && (tw.major & kUnitMnMajorR);
+        for (int pi = 0; pi < tab.n && ok; ++pi) {
+          const WalkInfo& wk = sh->walk[pi];
+          const CUtensorMap* const um = tab.unit_maps[pi];
+          const CUtensorMap* const vm = tab.var_maps[pi];
+          const int n_tiles = wk.n_tiles, num_kb = wk.num_kb, half_n = wk.half_n & 255;
+          const uint32_t flags = sh->var[pi].flags, major = (uint32_t)wk.half_n >> 8;
+          const bool l_mn = MN && (major & kUnitMnMajorL), r_mn = MN && (major & kUnitMnMajorR);
           const bool cl_mn = MN && (flags & kVarMnMajorL), cr_mn = MN && (flags & kVarMnMajorR);
-          for (int kb = 0; kb < tw.num_kb; ++kb, ++g) {
-            const uint32_t s = g % kStages, use = g / kStages;
-            // test hook: the consumers' waits run out
-            ok = g < tab.stop_after_kb && (use == 0 || w.wait(smem_u32(&sh->empty[s]), (use - 1) & 1));
-            if (!ok) break;
-            const uint32_t bar = smem_u32(&sh->full[s]), base = tile_base + s * C::kStageBytes;
-            mbar_expect_tx(bar, kABf16 + kALp + (uint32_t)tw.half_n * (kBlockK * 2 + kBlockK));
-            const int k0 = kb * kBlockK;
-            tma_load_3d_local(base + C::kOffR, &um[1], bar, r_mn ? c0 : k0, r_mn ? k0 : c0, tw.tc.b);
-            tma_load_3d_local(base + C::kOffL, &um[0], bar, l_mn ? r0 : k0, l_mn ? k0 : r0, tw.tc.b);
-            if (l_mn) tma_load_3d_local(base + C::kOffL + kABf16 / 2, &um[0], bar, r0 + 64, k0, tw.tc.b);
-            tma_load_3d_local(base + C::kOffCl, &vm[0], bar, cl_mn ? r0 : k0, cl_mn ? k0 : r0, tw.tc.b);
-            tma_load_3d_local(base + C::kOffCr, &vm[1], bar, cr_mn ? c0 : k0, cr_mn ? k0 : c0, tw.tc.b);
-            sh->issued = g + 1;
+          for (int j = 0; j < n_tiles && ok; ++j) {
+            const TileCoord tc = pair_tile(wk, j, num_pairs);
+            const int r0 = tc.m_tile * kPairM + (int)rank * kBlockM;     // this CTA's left-operand rows
+            const int c0 = tc.n_tile * kBlockN + (int)rank * half_n;     // this CTA's half of the right operand
+            for (int kb = 0; kb < num_kb; ++kb, ++g) {
+              const uint32_t s = ring.s;
+              // test hook: the consumers' waits run out
+              ok = g < tab.stop_after_kb && (g < (uint32_t)kStages || w.wait(smem_u32(&sh->empty[s]), ring.parity ^ 1u));
+              if (!ok) break;
+              const uint32_t bar = smem_u32(&sh->full[s]), base = tile_base + s * C::kStageBytes;
+              mbar_expect_tx(bar, kABf16 + kALp + (uint32_t)half_n * (kBlockK * 2 + kBlockK));
+              const int k0 = kb * kBlockK;
+              tma_load_3d_local(base + C::kOffR, &um[1], bar, r_mn ? c0 : k0, r_mn ? k0 : c0, tc.b);
+              tma_load_3d_local(base + C::kOffL, &um[0], bar, l_mn ? r0 : k0, l_mn ? k0 : r0, tc.b);
+              if (l_mn) tma_load_3d_local(base + C::kOffL + kABf16 / 2, &um[0], bar, r0 + 64, k0, tc.b);
+              tma_load_3d_local(base + C::kOffCl, &vm[0], bar, cl_mn ? r0 : k0, cl_mn ? k0 : r0, tc.b);
+              tma_load_3d_local(base + C::kOffCr, &vm[1], bar, cr_mn ? c0 : k0, cr_mn ? k0 : c0, tc.b);
+              sh->issued = g + 1;
+              ring.next();
+            }
           }
         }
       }
@@ -2275,8 +2284,8 @@ tc_side_kernel(const __grid_constant__ Table tab) {
       const bool lead = elect_one();
       uint32_t idesc_ref = 0, idesc_den = 0;   // of the tile in hand
       TileDesc ld{}, rd{}, cl{}, cr{};         // L; R and |R|; codes
-      auto issue_ref_den = [&](uint32_t gg, int kb) {
-        const uint32_t s = gg % kStages, base = tile_base + s * C::kStageBytes;
+      auto issue_ref_den = [&](uint32_t s, uint32_t gg, int kb) {
+        const uint32_t base = tile_base + s * C::kStageBytes;
 #pragma unroll
         for (int k = 0; k < kBlockK / 16; ++k)   // 16 bf16 per step
           mma_pair<kKindF16>(tmem_base + C::kColRef, ld.at(base + C::kOffL, k), rd.at(base + C::kOffR, k), idesc_ref, (kb | k) != 0, lead);
@@ -2285,8 +2294,8 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         for (int k = 0; k < kBlockK / 16; ++k)   // 16 bf16 = 8 columns of tensor memory per step
           mma_pair_a_tmem(tmem_base + C::kColDen, ta + 8u * k, rd.at(base + C::kOffRa, k), idesc_den, (kb | k) != 0, lead);
       };
-      auto issue_lp = [&](uint32_t gg, int kb, bool is_i8, uint32_t idesc_lp) {
-        const uint32_t base = tile_base + (gg % kStages) * C::kStageBytes;
+      auto issue_lp = [&](uint32_t s, int kb, bool is_i8, uint32_t idesc_lp) {
+        const uint32_t base = tile_base + s * C::kStageBytes;
 #pragma unroll
         for (int k = 0; k < kBlockK / 32; ++k) {  // 32 codes per step
           const uint64_t a = cl.at(base + C::kOffCl, k), b = cr.at(base + C::kOffCr, k);
@@ -2294,78 +2303,85 @@ tc_side_kernel(const __grid_constant__ Table tab) {
           else mma_pair<kKindF8>(tmem_base + C::kColLp, a, b, idesc_lp, (kb | k) != 0, lead);
         }
       };
-      auto wait_stage = [&](uint32_t gg) {
-        if (!w.wait_warp(smem_u32(&sh->ready[gg % kStages]), (gg / kStages) & 1)) return false;
+      auto wait_stage = [&](const Ring<kStages>& at) {
+        if (!w.wait_warp(smem_u32(&sh->ready[at.s]), at.parity)) return false;
         tc_fence_after();
         return true;
       };
-      TileWalk tw;
-      begin(tw);
-      uint32_t g = 0;
+      begin();
+      Ring<kStages> ring;                      // of the next block whose 8-bit MMAs are to be issued
+      uint32_t g = 0, it = 0;
       bool ok = true;
-      for (uint32_t it = 0; tw.valid && ok; ++it, tw.next_tile()) {
-        tw.make_uniform();
-        const int num_kb = tw.num_kb;
-        const uint32_t idesc_lp = __shfl_sync(0xffffffffu, sh->var[tw.pi].idesc, 0);
-        const uint32_t flags = __shfl_sync(0xffffffffu, sh->var[tw.pi].flags, 0);
-        const bool is_i8 = flags & kVarI8;
-        const bool l_mn = MN && (tw.major & kUnitMnMajorL), r_mn = MN && (tw.major & kUnitMnMajorR);
-        const bool cl_mn = MN && (flags & kVarMnMajorL), cr_mn = MN && (flags & kVarMnMajorR);
-        // |L| comes from tensor memory, contraction-major always
-        idesc_den = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n) | (r_mn ? kIdescMnMajorB : 0u);
-        idesc_ref = idesc_den | (l_mn ? kIdescMnMajorA : 0u);
-        ld = tile_desc(l_mn, 128u, 16u, kABf16 / 2);
-        rd = tile_desc(r_mn, r_mn ? 2u * tw.half_n : 128u, 16u, 16u);
-        cl = tile_desc(cl_mn, cl_mn ? 128u : 64u, 32u, 16u);
-        cr = tile_desc(cr_mn, cr_mn ? tw.half_n : 64u, 32u, 16u);
+      for (int pi = 0; pi < tab.n && ok; ++pi) {
+       const UnitInfo tw(sh->walk[pi]);
+       const int num_kb = tw.num_kb;
+       const uint32_t idesc_lp = __shfl_sync(0xffffffffu, sh->var[pi].idesc, 0);
+       const uint32_t flags = __shfl_sync(0xffffffffu, sh->var[pi].flags, 0);
+       const bool is_i8 = flags & kVarI8;
+       const bool l_mn = MN && (tw.major & kUnitMnMajorL), r_mn = MN && (tw.major & kUnitMnMajorR);
+       const bool cl_mn = MN && (flags & kVarMnMajorL), cr_mn = MN && (flags & kVarMnMajorR);
+       // |L| comes from tensor memory, contraction-major always
+       idesc_den = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n) | (r_mn ? kIdescMnMajorB : 0u);
+       idesc_ref = idesc_den | (l_mn ? kIdescMnMajorA : 0u);
+       ld = tile_desc(l_mn, 128u, 16u, kABf16 / 2);
+       rd = tile_desc(r_mn, r_mn ? 2u * tw.half_n : 128u, 16u, 16u);
+       cl = tile_desc(cl_mn, cl_mn ? 128u : 64u, 32u, 16u);
+       cr = tile_desc(cr_mn, cr_mn ? tw.half_n : 64u, 32u, 16u);
+       for (int j = 0; j < tw.n_tiles && ok; ++j, ++it) {
         // the reference and denominator blocks come back when both epilogues have copied the
         // previous tile's values out; the 8-bit block when they have finished that tile
-        if (it > 0 && !w.wait_warp(smem_u32(&sh->tmem_empty), (it - 1) & 1)) break;
+        ok = it == 0 || w.wait_warp(smem_u32(&sh->tmem_empty), (it - 1) & 1);
+        if (!ok) break;
         tc_fence_after();
         const int n_ahead = num_kb < kAbs ? num_kb : kAbs;
-        for (int j = 0; j < n_ahead && ok; ++j) {
-          ok = wait_stage(g + j);
-          if (ok) issue_ref_den(g + j, j);
+        Ring<kStages> ahead = ring;
+        for (int i = 0; i < n_ahead && ok; ++i) {
+          ok = wait_stage(ahead);
+          if (ok) issue_ref_den(ahead.s, g + i, i);
+          ahead.next();
         }
         if (!ok) break;
-        if (it > 0 && !w.wait_warp(smem_u32(&sh->lp_done), (it - 1) & 1)) break;
+        ok = it == 0 || w.wait_warp(smem_u32(&sh->lp_done), (it - 1) & 1);
+        if (!ok) break;
         tc_fence_after();
         int kb = 0;
         for (; kb < n_ahead; ++kb, ++g) {
-          issue_lp(g, kb, is_i8, idesc_lp);
-          tc_commit_pair(smem_u32(&sh->empty[g % kStages]), lead);
+          issue_lp(ring.s, kb, is_i8, idesc_lp);
+          tc_commit_pair(smem_u32(&sh->empty[ring.s]), lead);
+          ring.next();
         }
         for (; kb < num_kb && ok; ++kb, ++g) {
-          ok = wait_stage(g);
+          ok = wait_stage(ring);
           if (!ok) break;
-          issue_ref_den(g, kb);
-          issue_lp(g, kb, is_i8, idesc_lp);
-          tc_commit_pair(smem_u32(&sh->empty[g % kStages]), lead);        // frees the k-block in both CTAs
+          issue_ref_den(ring.s, g, kb);
+          issue_lp(ring.s, kb, is_i8, idesc_lp);
+          tc_commit_pair(smem_u32(&sh->empty[ring.s]), lead);             // frees the k-block in both CTAs
+          ring.next();
         }
         if (ok) tc_commit_pair(smem_u32(&sh->tmem_full), lead);           // this tile's accumulators are complete
+       }
       }
     } else if (RW && warp >= 2) {
       // ---------------------------------------------------------- |R| (both CTAs)
-      TileWalk tw;
-      begin(tw);
+      begin();
       const int t = (warp - 2) * 32 + lane;        // 0..63
       const uint32_t ready_leader = map_to_cta(smem_u32(&sh->ready[0]), 0);
       bool ok = true;
-      uint32_t s = 0, parity = 0;
-      for (; tw.valid && ok; tw.next_tile()) {
+      Ring<kStages> ring;
+      for (int pi = 0; pi < tab.n && ok; ++pi)
+       for (UnitInfo tw(sh->walk[pi]); tw.n_tiles > 0 && ok; --tw.n_tiles) {
         for (int kb = 0; kb < tw.num_kb; ++kb) {
-          ok = w.wait_warp(smem_u32(&sh->full[s]), parity);
+          ok = w.wait_warp(smem_u32(&sh->full[ring.s]), ring.parity);
           if (!ok) break;
-          abs_r<64>(tile_base + s * C::kStageBytes + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
+          abs_r<64>(tile_base + ring.s * C::kStageBytes + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
           fence_proxy_async();
           __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(ready_leader + s * 8u);
-          if (++s == (uint32_t)kStages) { s = 0; parity ^= 1u; }
+          if (lane == 0) mbar_arrive_cluster(ready_leader + ring.s * 8u);
+          ring.next();
         }
       }
     } else {
-      TileWalk tw;
-      begin(tw);
+      begin();
     }
   } else if (warp < kFirstEpiWarp) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsConv));
@@ -2378,16 +2394,16 @@ tc_side_kernel(const __grid_constant__ Table tab) {
     const uint32_t ready_leader = map_to_cta(smem_u32(&sh->ready[0]), 0);
     const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + C::kColAbsL;
     const uint32_t row_off = (uint32_t)t * 128u, sw = (uint32_t)t & 7u;
-    TileWalk tw;
-    begin(tw);
+    begin();
     bool ok = true;
+    Ring<kStages> ring;
     uint32_t g = 0;
     // the blocks of one tile; a loop for each order of L: one loop with the choice inside cost the contraction-major one 7 %
-    auto convert = [&](auto mn) {
+    auto convert = [&](auto mn, const UnitInfo& tw) {
       constexpr bool kMn = decltype(mn)::value;
       for (int kb = 0; kb < tw.num_kb; ++kb, ++g) {
-        const uint32_t s = g % kStages, m = 0x7fff7fffu;
-        if (!w.wait_warp(smem_u32(&sh->full[s]), (g / kStages) & 1)) { ok = false; return; }
+        const uint32_t s = ring.s, m = 0x7fff7fffu;
+        if (!w.wait_warp(smem_u32(&sh->full[s]), ring.parity)) { ok = false; return; }
         const uint32_t base = tile_base + s * C::kStageBytes;
         if (!RW) abs_r<128>(base + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
         uint32_t a[32];
@@ -2402,8 +2418,9 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         }
         // the tensor-memory columns were last read by the MMAs of k-block g - kAbs
         if (g >= (uint32_t)kAbs) {
-          const uint32_t gp = g - kAbs;
-          if (!w.wait_warp(smem_u32(&sh->empty[gp % kStages]), (gp / kStages) & 1)) { ok = false; return; }
+          const uint32_t sp = s >= (uint32_t)kAbs ? s - kAbs : s + kStages - kAbs;
+          const uint32_t pp = s >= (uint32_t)kAbs ? ring.parity : ring.parity ^ 1u;
+          if (!w.wait_warp(smem_u32(&sh->empty[sp]), pp)) { ok = false; return; }
         }
         tc_fence_after();
         const uint32_t tcol = taddr + 32u * (g % kAbs);
@@ -2420,11 +2437,13 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(ready_leader + s * 8u);
+        ring.next();
       }
     };
-    for (; ok && tw.valid; tw.next_tile()) {
-      if (MN && (tw.major & kUnitMnMajorL)) convert(std::bool_constant<MN>{}); else convert(std::false_type{});
-    }
+    for (int pi = 0; pi < tab.n && ok; ++pi)
+      for (UnitInfo tw(sh->walk[pi]); tw.n_tiles > 0 && ok; --tw.n_tiles) {
+        if (MN && (tw.major & kUnitMnMajorL)) convert(std::bool_constant<MN>{}, tw); else convert(std::false_type{}, tw);
+      }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
     // ------------------------------------------------------------ epilogue (warps 8..15, both CTAs)
@@ -2466,21 +2485,24 @@ tc_side_kernel(const __grid_constant__ Table tab) {
     float dr_tensor = 1.f, dl_tensor = 0.f;
     int pM = 0, pN = 0;                            // a probe's M and N are below 2^31 (its tensor maps require it)
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
-    TileWalk tw;
-    begin(tw);
-    for (uint32_t it = 0; tw.valid; ++it) {
-      const int pi = tw.pi;
+    begin();
+    uint32_t it = 0;
+    bool dead = false;                             // a wait ran out
+    for (int pi = 0; pi < tab.n && !dead; ++pi) {
+     const UnitInfo tw(sh->walk[pi]);
+     for (int j = 0; j < tw.n_tiles; ++j, ++it) {
       if (pi != cur) {
         if (cur >= 0) flush(cur);
         cur = pi;
         met |= 1u << pi;
         const GroupVar& gv = tab.v[pi];
-        per_col = gv.flags & kVarScalePerCol; pc_l = gv.flags & kVarScalePerRow; is_i8 = gv.flags & kVarI8; narrow = tw.half_n < 64;
+        const uint32_t flags = sh->var[pi].flags;
+        per_col = flags & kVarScalePerCol; pc_l = flags & kVarScalePerRow; is_i8 = flags & kVarI8; narrow = tw.half_n < 64;
         pM = tab.u[pi].M; pN = tab.u[pi].N;
         dr_tensor = per_col ? 1.f : __ldg(gv.dr);
         dl_tensor = pc_l ? 0.f : __ldg(gv.dl);
       }
-      const TileCoord tc = tw.tc;
+      const TileCoord tc = pair_tile(sh->walk[pi], j, num_pairs);
       float* dr_s = sh->delta_r[it & 1];
       if (per_col && et < kBlockN) {
         const int col = tc.n_tile * kBlockN + et;
@@ -2497,7 +2519,7 @@ tc_side_kernel(const __grid_constant__ Table tab) {
 
       const bool ok = w.wait(smem_u32(&sh->tmem_full), it & 1);
       // one barrier publishes delta_r and makes the give-up decision uniform over the epilogue
-      if (epi_barrier_any(!ok)) break;
+      if (epi_barrier_any(!ok)) { dead = true; break; }
       tc_fence_after();
       // live = columns of this warp that exist in the matrix
       const int live = pN - colw < cw ? pN - colw : cw;          // <= 0: none
@@ -2555,7 +2577,7 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         double* const rows = tab.v[pi].row_stats;
         if (rows) row_stats_add(rows + ((int64_t)tc.b * pM + row) * 5, st);
       }
-      tw.next_tile();
+     }
     }
     if (cur >= 0) flush(cur);
     // the records of the probes this CTA never met are zero
@@ -2674,7 +2696,7 @@ void fill_tiles(KernelArgs* ka, GemmShape g) {
 int g_max_pairs[kMaxDevices] = {};     // per device; 0 = not yet queried
 int max_pairs() {
   const int dev = current_device();
-  return dev >= 0 && g_max_pairs[dev] > 0 ? g_max_pairs[dev] : sm_count() / 2;
+  return dev >= 0 && g_max_pairs[dev] > 0 ? g_max_pairs[dev] : std::min(sm_count() / 2, kMaxPairs);
 }
 
 // cudaFuncSetAttribute(MaxDynamicSharedMemorySize) once per kernel and device.
@@ -2820,9 +2842,9 @@ qm_status probe_residency() {
     q.attrs = qa; q.numAttrs = 1;
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, Widest::kernel, &q) == cudaSuccess && n > 0)
-      g_max_pairs[dev] = n < sm_count() / 2 ? n : sm_count() / 2;
+      g_max_pairs[dev] = std::min(n, std::min(sm_count() / 2, kMaxPairs));
     else
-      g_max_pairs[dev] = sm_count() / 2;
+      g_max_pairs[dev] = std::min(sm_count() / 2, kMaxPairs);
     (void)cudaGetLastError();
   }
   return QM_OK;
@@ -2851,6 +2873,65 @@ bool r_by_warps(bool side, const UnitPlan* units, int n) {
   return false;
 }
 
+// What a tile of a unit takes its CTA pair, in cycles: a block of the contraction in all three products 950 in the side-by-side
+// form; else 683 for the bf16 products and 430 for 128 entries of each 8-bit one; a tile's fixed part beside that, and
+// with short contractions the epilogue's (8192 x 4096, K = 64 ... 4096, whole launches over rounds of tiles).
+double tile_cycles(bool side, int64_t K, int n_var) {
+  const double kb = (double)((K + kBlockK - 1) / kBlockK), nb = (double)((K + CfgP::kLpDepth - 1) / CfgP::kLpDepth);
+  if (side) return std::max(4000.0 + 950.0 * kb, 6000.0);
+  return std::max(2500.0 + 683.0 * kb + n_var * (600.0 + 430.0 * nb), 5000.0 + 2700.0 * n_var);
+}
+
+// Deals the tiles of a launch's units, in the order of descending cost, to the pairs: each unit's to those with the least to do
+// so far, so that the pairs end within a tile of the cheapest kind of one another.  (Dealt in rounds of a tile for each pair, the
+// four products of a BERT-base layer, 96 tiles of K = 3072 and 768 of 768, took 18 units of the cheap tile where 15.6 would
+// do: the launch 176 us, 165 so; a sweep layer's 4.82 ms, 4.58, a BERT-large layer's 2.34, 2.25.)  A pair that has a tile's
+// time less to do than another takes its tiles ahead of the rounds (lead), the remainder comes after them (last), so that pairs
+// are in the same round and share the blocks they read.
+struct TileDeal {
+  double load[kMaxPairs] = {};
+  int pairs;
+  explicit TileDeal(int n) : pairs(n) {}
+  void deal(int64_t tiles, double cost, GroupUnit* u, uint16_t* lead) {
+    int order[kMaxPairs];
+    for (int p = 0; p < pairs; ++p) order[p] = p;
+    std::stable_sort(order, order + pairs, [&](int a, int b) { return load[a] < load[b]; });
+    // the level that the work of all these tiles fills the lowest loads up to, and whole tiles below it
+    double level = 0.0, below = 0.0;
+    for (int i = 0; i < pairs; ++i) {
+      below += load[order[i]];
+      level = ((double)tiles * cost + below) / (i + 1);
+      if (i + 1 == pairs || level <= load[order[i + 1]]) break;
+    }
+    const double most = load[order[pairs - 1]];
+    int64_t count[kMaxPairs], left = tiles;
+    for (int p = 0; p < pairs; ++p) {
+      count[p] = level > load[p] ? std::min((int64_t)((level - load[p]) / cost), left) : 0;
+      left -= count[p];
+    }
+    // the rest, less than one for each pair, where it ends earliest
+    std::stable_sort(order, order + pairs, [&](int a, int b) { return load[a] + cost * count[a] < load[b] + cost * count[b]; });
+    for (int i = 0; left > 0; i = i + 1 == pairs ? 0 : i + 1, --left) ++count[order[i]];
+    int64_t rounds = count[0], sum = 0;
+    for (int p = 1; p < pairs; ++p) rounds = std::min(rounds, count[p]);
+    const bool even = tiles - rounds * pairs > 65535;  // beyond the prefix sums' type: dealt evenly
+    if (even) rounds = tiles / pairs;
+    for (uint32_t& w : u->last) w = 0;
+    for (int p = 0; p < pairs; ++p) {
+      if (even) count[p] = rounds + (p < tiles % pairs ? 1 : 0);
+      // one of the tiles beside the rounds comes last, unless the pair is that far behind with all of them
+      const int64_t more = count[p] - rounds;
+      const bool one_last = more > 0 && (even || (most - load[p]) < cost * more);
+      lead[p] = (uint16_t)sum;
+      sum += more - one_last;
+      if (one_last) u->last[p >> 5] |= 1u << (p & 31);
+      load[p] += cost * count[p];
+    }
+    lead[pairs] = (uint16_t)sum;
+    u->rounds = (int32_t)rounds;
+  }
+};
+
 template <bool SIDE, typename Table>
 qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, bool mn, cudaStream_t s) {
   static Table tab;                    // up to 29 KB: kept off the stack; guarded by the mutex below
@@ -2864,6 +2945,9 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, bool
   tab.done_counter = first.done_counter;
   tab.err0 = first.err_word;
   int64_t total = 0;
+  for (int k = 0; k < n; ++k) total += tile_count(units[k].g);
+  const int pairs = (int)std::min<int64_t>(total, max_pairs());
+  TileDeal pair_loads(pairs);
   for (int k = 0; k < n; ++k) {
     const UnitPlan& up = units[k];
     const GemmShape g = up.g;
@@ -2873,17 +2957,17 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, bool
     // half as many right-operand rows staged
     const int half_n = g.N <= 64 ? 32 : kHalfN;
     // an operand with the contraction strided is staged as it lies in memory: mn-major tiles
-    const bool have = (p0.l_mn ? make_map_mn(&gu.maps[0], p0.l, true, 64, kBlockK, g.K, g.M, g.batch, p0.l_ld, p0.l_sb)
-                                 : make_map(&gu.maps[0], p0.l, true, kBlockM, g.K, g.M, g.batch, p0.l_ld, p0.l_sb)) &&
-                      (p0.r_mn ? make_map_mn(&gu.maps[1], p0.r, true, half_n, kBlockK, g.K, g.N, g.batch, p0.r_ld, p0.r_sb)
-                                 : make_map(&gu.maps[1], p0.r, true, half_n, g.K, g.N, g.batch, p0.r_ld, p0.r_sb));
+    const bool have = (p0.l_mn ? make_map_mn(&tab.unit_maps[k][0], p0.l, true, 64, kBlockK, g.K, g.M, g.batch, p0.l_ld, p0.l_sb)
+                                 : make_map(&tab.unit_maps[k][0], p0.l, true, kBlockM, g.K, g.M, g.batch, p0.l_ld, p0.l_sb)) &&
+                      (p0.r_mn ? make_map_mn(&tab.unit_maps[k][1], p0.r, true, half_n, kBlockK, g.K, g.N, g.batch, p0.r_ld, p0.r_sb)
+                                 : make_map(&tab.unit_maps[k][1], p0.r, true, half_n, g.K, g.N, g.batch, p0.r_ld, p0.r_sb));
     if (!have) return QM_ERR_CUDA;
     gu.major = (p0.l_mn ? kUnitMnMajorL : 0u) | (p0.r_mn ? kUnitMnMajorR : 0u);
     KernelArgs ka{};
     fill_tiles(&ka, g);
     gu.M = (int32_t)g.M; gu.N = (int32_t)g.N; gu.K = (int32_t)g.K;
     gu.tiles_m = ka.tiles_m; gu.tiles_n = ka.tiles_n;
-    gu.tile_begin = (int32_t)total;
+    pair_loads.deal(ka.num_tiles, tile_cycles(SIDE, g.K, up.n_var), &gu, tab.lead[k]);
     gu.half_n = half_n;
     // Tiles that run at the same time should share the LARGER operand's blocks, so that it is
     // streamed from HBM once and the smaller one is what gets fetched again (from L2, if it fits):
@@ -2892,9 +2976,9 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, bool
     const Divisor by_b((uint32_t)(gu.tiles_m * gu.tiles_n)), by_inner((uint32_t)(gu.m_fastest ? gu.tiles_m : gu.tiles_n));
     gu.b_mul = by_b.mul; gu.b_shift = by_b.shift; gu.i_mul = by_inner.mul; gu.i_shift = by_inner.shift;
     gu.var_begin = tab.n_var; gu.n_var = up.n_var;
-    total += ka.num_tiles;
     for (int j = 0; j < up.n_var; ++j) {
       const TcProbeArgs& p = ps[up.probe[j]];
+      CUtensorMap(&vm)[2] = tab.var_maps[tab.n_var];
       GroupVar& v = tab.v[tab.n_var++];
       // blocks of codes are 64 entries deep beside the bf16 tiles, 128 on their own
       const int depth = SIDE ? kBlockK : CfgP::kLpDepth;
@@ -2903,21 +2987,19 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, bool
         return mn ? make_map_mn(m, codes, false, box_rows, depth, g.K, rows, g.batch, ld, g.K * ld)
                            : make_map(m, codes, false, box_rows, g.K, rows, g.batch, ld, rows * ld, !SIDE);
       };
-      if (!code_map(&v.maps[0], p.cl, p.cl_mn, kBlockM, g.M) || !code_map(&v.maps[1], p.cr, p.cr_mn, half_n, g.N)) return QM_ERR_CUDA;
+      if (!code_map(&vm[0], p.cl, p.cl_mn, kBlockM, g.M) || !code_map(&vm[1], p.cr, p.cr_mn, half_n, g.N)) return QM_ERR_CUDA;
       v.dl = p.dl; v.dr = p.dr;
       v.partials = p.partials; v.result = p.result; v.row_stats = p.row_stats;
       v.err_word = p.err_word; v.err_also[0] = p.err_also[0]; v.err_also[1] = p.err_also[1];
       v.count = (uint64_t)(g.M * g.N * g.batch);
-      v.flags = (p.fmt_l == QM_FMT_INT8 ? kVarI8 : 0u) | (p.gran_l == QM_GRAN_CHANNEL ? kVarScalePerRow : 0u) |
+      v.info.flags = (p.fmt_l == QM_FMT_INT8 ? kVarI8 : 0u) | (p.gran_l == QM_GRAN_CHANNEL ? kVarScalePerRow : 0u) |
                 (p.gran_r == QM_GRAN_CHANNEL ? kVarScalePerCol : 0u) | (p.row_stats ? kVarRowStats : 0u) |
                 (p.cl_mn ? kVarMnMajorL : 0u) | (p.cr_mn ? kVarMnMajorR : 0u);
-      v.idesc_lp = lp_idesc(p.fmt_l, p.fmt_r, 2 * half_n) | (p.cl_mn ? kIdescMnMajorA : 0u) | (p.cr_mn ? kIdescMnMajorB : 0u);
+      v.info.idesc = lp_idesc(p.fmt_l, p.fmt_r, 2 * half_n) | (p.cl_mn ? kIdescMnMajorA : 0u) | (p.cr_mn ? kIdescMnMajorB : 0u);
     }
   }
-  tab.total_tiles = (int32_t)total;
-  const int pairs = max_pairs();
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(2 * (total < pairs ? total : pairs)));
+  cfg.gridDim = dim3((unsigned)(2 * pairs));
   cfg.blockDim = dim3(kProbeThreads);
   cfg.dynamicSmemBytes = ProbeKernel<SIDE, false, false, Table>::kSmem;
   cfg.stream = s;
@@ -2970,10 +3052,11 @@ qm_status launch_tc_probes(const TcProbeArgs* ps, int n, cudaStream_t s) {
   int64_t single_tiles = 0;
   for (auto u = units.begin(); u != others; ++u) single_tiles += tile_count(u->g);
   const size_t n_side = others == units.end() || single_tiles >= max_pairs() ? (size_t)(others - units.begin()) : 0;
-  // descending tile cost: kilobytes through shared memory per 64 contraction entries
-  auto by_cost = [](const UnitPlan& a, const UnitPlan& b) { return a.g.K * (72 + 24 * a.n_var) > b.g.K * (72 + 24 * b.n_var); };
-  std::stable_sort(units.begin(), units.begin() + n_side, by_cost);
-  std::stable_sort(units.begin() + n_side, units.end(), by_cost);
+  auto by_cost = [](bool side) {               // descending
+    return [side](const UnitPlan& a, const UnitPlan& b) { return tile_cycles(side, a.g.K, a.n_var) > tile_cycles(side, b.g.K, b.n_var); };
+  };
+  std::stable_sort(units.begin(), units.begin() + n_side, by_cost(true));
+  std::stable_sort(units.begin() + n_side, units.end(), by_cost(false));
   auto any_mn = [&](const UnitPlan* u, int count) {
     for (int k = 0; k < count; ++k) {
       const TcProbeArgs& a = ps[u[k].probe[0]];

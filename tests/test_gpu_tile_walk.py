@@ -86,3 +86,32 @@ def test_outputs_wider_than_tall_walk_down_the_rows(fmt, gran):
         assert got["count"] == alone["count"] and got["max_be"] == alone["max_be"]
         for k in ("sum_be", "sum_diff2", "sum_ref2", "sum_den2"):
             assert abs(got[k] - alone[k]) <= 1e-12 * abs(alone[k]), (o["name"], k)
+
+
+@pytest.mark.parametrize("fmts", [("e4m3",), ("e4m3", "int8")])
+def test_tiles_of_unlike_cost_are_dealt_once_each(fmts):
+    """Products of long and short contractions in one launch, fewer and more tiles than CTA pairs: the
+    deal by load gives the pairs unequal counts.  A tile left out or taken twice shows in the counts of
+    the rows' sums; every record is the single probe's."""
+    rng = workloads._rng(92)
+    shapes = [(1, 2100, 700, 2064), (1, 200, 100, 4096), (1, 1500, 1500, 256), (3, 700, 1300, 64), (1, 260, 130, 16)]
+    ops = []
+    for b, M, N, K in shapes:
+        L, R = workloads.normal(rng, (b, M, K)), workloads.normal(rng, (b, N, K), 0.02)
+        ops += [workloads.op(f"d{M}x{N}x{K}", L, -1, R, -1, f, f, "tensor", "channel") for f in fmts]
+    dev = {}
+    for o in ops:                                      # the formats of a product share their operands
+        dev.setdefault(o["name"], (o["L"].cuda(), o["R"].cuda()))
+    probes = [(qm.operand_of(dev[o["name"]][0], -1), qm.operand_of(dev[o["name"]][1], -1), o["fmt_l"], o["fmt_r"], "tensor", "channel")
+              for o in ops]
+    batch = qm.ProbeBatch(probes, row_stats=True)
+    batch.launch()
+    torch.cuda.synchronize()
+    for o, p, res, rows in zip(ops, probes, batch.results(), batch.row_stats):
+        got, alone = res.record(), qm.qm_probe_layer(*p).record()
+        assert res.device_error == 0 and got["count"] == alone["count"] and got["max_be"] == alone["max_be"], o["name"]
+        rs = rows.cpu().numpy()
+        assert (rs[:, 4] > 0).all(), o["name"]
+        for k, name in ((0, "sum_be"), (2, "sum_diff2"), (3, "sum_ref2"), (4, "sum_den2")):
+            assert abs(got[name] - alone[name]) <= 1e-12 * abs(alone[name]), (o["name"], name)
+            assert abs(rs[:, k].sum() - got[name]) <= 1e-9 * abs(got[name]), (o["name"], name)
