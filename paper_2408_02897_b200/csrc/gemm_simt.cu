@@ -31,7 +31,7 @@ struct SimtArgs {
   int64_t K, ldc;
   float* out_descaled; void* out_raw;                       // plain product
   double* partials; uint32_t* done_counter;                 // probe: a record per block; counts finished blocks
-  uint32_t* err_word; qm_metric_result* result; uint64_t count;
+  uint32_t* err_word; const uint32_t* prepare_flags; qm_metric_result* result; uint64_t count;
 };
 
 // A block computes a TM x TN output tile with 256 threads, 4 x 4 outputs each.  The work is fp32 FMA (three
@@ -319,12 +319,13 @@ __global__ void __launch_bounds__(kThreads, 2) simt_kernel(const SimtArgs a) {
         v[0] += __ldcg(rec); v[1] = fmax(v[1], __ldcg(rec + 1)); v[2] += __ldcg(rec + 2);
         v[3] += __ldcg(rec + 3); v[4] += __ldcg(rec + 4);
       }
+      const int not_finite = __syncthreads_or(a.prepare_flags && threadIdx.x < kPrepareFlagWords && __ldcg(a.prepare_flags + threadIdx.x));
       block_reduce();
       if (threadIdx.x == 0) {                // (the record may be in host memory: stores only, every field once)
         a.result->sum_be = v[0]; a.result->max_be = v[1]; a.result->sum_diff2 = v[2];
         a.result->sum_ref2 = v[3]; a.result->sum_den2 = v[4];
         a.result->count = a.count;
-        a.result->device_error = *reinterpret_cast<volatile uint32_t*>(a.err_word);
+        a.result->device_error = *reinterpret_cast<volatile uint32_t*>(a.err_word) | (not_finite ? QM_DEVERR_NONFINITE : 0u);
         a.result->reserved = 0;
       }
     }
@@ -398,12 +399,12 @@ qm_status launch_simt_gemm_lp(const uint8_t* cl, int fmt_l, const float* dl, int
 qm_status launch_simt_probe(const View& L, const View& R, const uint8_t* cl, int fmt_l,
                             const float* dl, int gran_l, const uint8_t* cr, int fmt_r,
                             const float* dr, int gran_r, double* partials, uint32_t* done_counter,
-                            uint32_t* err_word, qm_metric_result* out, cudaStream_t s) {
+                            uint32_t* err_word, const uint32_t* prepare_flags, qm_metric_result* out, cudaStream_t s) {
   GemmShape g{L.nc, R.nc, L.c, L.batch};
   SimtArgs a{};
   a.l = SimtOperand{L.data, L.dtype, L.nc, L.s_nc, L.s_c, L.s_b, cl, fmt_l, dl, gran_l == QM_GRAN_CHANNEL};
   a.r = SimtOperand{R.data, R.dtype, R.nc, R.s_nc, R.s_c, R.s_b, cr, fmt_r, dr, gran_r == QM_GRAN_CHANNEL};
-  a.K = L.c; a.ldc = qm_code_ld(L.c); a.partials = partials; a.done_counter = done_counter; a.err_word = err_word;
+  a.K = L.c; a.ldc = qm_code_ld(L.c); a.partials = partials; a.done_counter = done_counter; a.err_word = err_word; a.prepare_flags = prepare_flags;
   a.result = out; a.count = (uint64_t)(g.M * g.N * g.batch);
   return launch_simt<true>(a, g, s);
 }

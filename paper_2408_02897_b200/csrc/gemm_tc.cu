@@ -30,6 +30,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstdlib>
+#include <cstring>
 #include <mutex>
 #include <type_traits>
 #include <vector>
@@ -1174,6 +1175,7 @@ struct GroupVar {
   double* row_stats;          // optional [batch * M][5] per-row sums
   uint32_t* err_word;
   const uint32_t* err_also[2];           // further error words to report in the record, or null
+  const uint32_t* prepare_flags;         // flag words of the operands' preparation, or null
   uint64_t count;             // batch * M * N
   VarInfo info;
 };
@@ -1473,6 +1475,13 @@ __device__ __forceinline__ void write_results(const Table& tab, int ew, int lane
     const uint32_t* word = lane == 0 ? a.err_word : lane == 1 ? a.err_also[0] : lane == 2 ? a.err_also[1] : lane == 3 ? tab.err0 : nullptr;
     uint32_t flags = word ? *reinterpret_cast<const volatile uint32_t*>(word) : 0u;
     if (lane == 3) flags &= QM_DEVERR_TIMEOUT;
+    if (a.prepare_flags) {
+      uint32_t any = 0;
+#pragma unroll
+      for (int i = 0; i < kPrepareFlagWords; i += 32)
+        if (i + lane < kPrepareFlagWords) any |= __ldcg(a.prepare_flags + i + lane);
+      if (any) flags |= QM_DEVERR_NONFINITE;
+    }
     double s4[4] = {0, 0, 0, 0};
     float mx = 0.f;
     for (int i0 = lane; i0 < (int)gridDim.x; i0 += 32 * kTake) {
@@ -2889,45 +2898,80 @@ double tile_cycles(bool side, int64_t K, int n_var) {
 // time less to do than another takes its tiles ahead of the rounds (lead), the remainder comes after them (last), so that pairs
 // are in the same round and share the blocks they read.
 struct TileDeal {
-  double load[kMaxPairs] = {};
-  int pairs;
-  explicit TileDeal(int n) : pairs(n) {}
+  struct Run { int p0, n; double load; int64_t count; };   // neighbouring pairs with the same load: a unit splits one run at most,
+  Run runs[2 * kMaxPairs];                                  // so that a unit costs the host a fraction of a microsecond
+  int n_runs = 1, pairs;
+  explicit TileDeal(int n) : pairs(n) { runs[0] = Run{0, n, 0.0, 0}; }
+  template <typename Key>
+  void sort_runs(Key key) {                                // by insertion: a few runs, nearly in order
+    for (int i = 1; i < n_runs; ++i) {
+      const Run r = runs[i];
+      int j = i;
+      for (; j > 0 && (key(runs[j - 1]) > key(r) || (key(runs[j - 1]) == key(r) && runs[j - 1].p0 > r.p0)); --j) runs[j] = runs[j - 1];
+      runs[j] = r;
+    }
+  }
+  // the first `n` pairs of run i become a run of their own, before it
+  void split(int i, int n) {
+    for (int j = n_runs++; j > i + 1; --j) runs[j] = runs[j - 1];
+    runs[i + 1] = Run{runs[i].p0 + n, runs[i].n - n, runs[i].load, runs[i].count};
+    runs[i].n = n;
+  }
   void deal(int64_t tiles, double cost, GroupUnit* u, uint16_t* lead) {
-    int order[kMaxPairs];
-    for (int p = 0; p < pairs; ++p) order[p] = p;
-    std::stable_sort(order, order + pairs, [&](int a, int b) { return load[a] < load[b]; });
+    sort_runs([](const Run& r) { return r.load; });
     // the level that the work of all these tiles fills the lowest loads up to, and whole tiles below it
     double level = 0.0, below = 0.0;
-    for (int i = 0; i < pairs; ++i) {
-      below += load[order[i]];
-      level = ((double)tiles * cost + below) / (i + 1);
-      if (i + 1 == pairs || level <= load[order[i + 1]]) break;
+    for (int i = 0, width = 0; i < n_runs; ++i) {
+      below += runs[i].load * runs[i].n;
+      width += runs[i].n;
+      level = ((double)tiles * cost + below) / width;
+      if (i + 1 == n_runs || level <= runs[i + 1].load) break;
     }
-    const double most = load[order[pairs - 1]];
-    int64_t count[kMaxPairs], left = tiles;
-    for (int p = 0; p < pairs; ++p) {
-      count[p] = level > load[p] ? std::min((int64_t)((level - load[p]) / cost), left) : 0;
-      left -= count[p];
+    const double most = runs[n_runs - 1].load, per_cost = 1.0 / cost;
+    int64_t left = tiles, rounds = tiles;
+    for (int i = 0; i < n_runs; ++i) {
+      Run& r = runs[i];
+      r.count = level > r.load ? (int64_t)((level - r.load) * per_cost) : 0;
+      if (r.count * r.n > left) r.count = left / r.n;
+      left -= r.count * r.n;
     }
     // the rest, less than one for each pair, where it ends earliest
-    std::stable_sort(order, order + pairs, [&](int a, int b) { return load[a] + cost * count[a] < load[b] + cost * count[b]; });
-    for (int i = 0; left > 0; i = i + 1 == pairs ? 0 : i + 1, --left) ++count[order[i]];
-    int64_t rounds = count[0], sum = 0;
-    for (int p = 1; p < pairs; ++p) rounds = std::min(rounds, count[p]);
-    const bool even = tiles - rounds * pairs > 65535;  // beyond the prefix sums' type: dealt evenly
-    if (even) rounds = tiles / pairs;
-    for (uint32_t& w : u->last) w = 0;
-    for (int p = 0; p < pairs; ++p) {
-      if (even) count[p] = rounds + (p < tiles % pairs ? 1 : 0);
-      // one of the tiles beside the rounds comes last, unless the pair is that far behind with all of them
-      const int64_t more = count[p] - rounds;
-      const bool one_last = more > 0 && (even || (most - load[p]) < cost * more);
-      lead[p] = (uint16_t)sum;
-      sum += more - one_last;
-      if (one_last) u->last[p >> 5] |= 1u << (p & 31);
-      load[p] += cost * count[p];
+    sort_runs([cost](const Run& r) { return r.load + cost * r.count; });
+    for (int i = 0; left > 0; i = i + 1 == n_runs ? 0 : i + 1) {
+      if (left < runs[i].n) split(i, (int)left);
+      ++runs[i].count;
+      left -= runs[i].n;
     }
-    lead[pairs] = (uint16_t)sum;
+    for (int i = 0; i < n_runs; ++i) rounds = std::min(rounds, runs[i].count);
+    const bool even = tiles - rounds * pairs > 65535;      // beyond the prefix sums' type: dealt evenly
+    if (even) {
+      rounds = tiles / pairs;
+      const int rest = (int)(tiles % pairs);
+      for (int i = 0; i < n_runs; ++i)
+        if (runs[i].p0 < rest && rest < runs[i].p0 + runs[i].n) split(i, rest - runs[i].p0);
+      for (int i = 0; i < n_runs; ++i) runs[i].count = rounds + (runs[i].p0 < rest ? 1 : 0);
+    }
+    for (uint32_t& w : u->last) w = 0;
+    memset(lead, 0, sizeof(uint16_t) * (size_t)(pairs + 1));
+    bool any_lead = false;
+    for (int i = 0; i < n_runs; ++i) {
+      Run& r = runs[i];
+      // one of the tiles beside the rounds comes last, unless the pair is that far behind with all of them
+      const int64_t more = r.count - rounds;
+      const bool one_last = more > 0 && (even || most - r.load < cost * more);
+      if (one_last)
+        for (int w = r.p0 >> 5, end = r.p0 + r.n; w * 32 < end; ++w) {
+          const int lo = std::max(r.p0 - 32 * w, 0), n = std::min(end - 32 * w, 32) - lo;
+          u->last[w] |= (n == 32 ? ~0u : (1u << n) - 1u) << lo;
+        }
+      if (more > one_last) {
+        any_lead = true;
+        for (int p = r.p0; p < r.p0 + r.n; ++p) lead[p + 1] = (uint16_t)(more - one_last);
+      }
+      r.load += cost * r.count;
+    }
+    if (any_lead)
+      for (int p = 0; p < pairs; ++p) lead[p + 1] = (uint16_t)(lead[p + 1] + lead[p]);
     u->rounds = (int32_t)rounds;
   }
 };
@@ -2990,7 +3034,7 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, bool
       if (!code_map(&vm[0], p.cl, p.cl_mn, kBlockM, g.M) || !code_map(&vm[1], p.cr, p.cr_mn, half_n, g.N)) return QM_ERR_CUDA;
       v.dl = p.dl; v.dr = p.dr;
       v.partials = p.partials; v.result = p.result; v.row_stats = p.row_stats;
-      v.err_word = p.err_word; v.err_also[0] = p.err_also[0]; v.err_also[1] = p.err_also[1];
+      v.err_word = p.err_word; v.prepare_flags = p.prepare_flags; v.err_also[0] = p.err_also[0]; v.err_also[1] = p.err_also[1];
       v.count = (uint64_t)(g.M * g.N * g.batch);
       v.info.flags = (p.fmt_l == QM_FMT_INT8 ? kVarI8 : 0u) | (p.gran_l == QM_GRAN_CHANNEL ? kVarScalePerRow : 0u) |
                 (p.gran_r == QM_GRAN_CHANNEL ? kVarScalePerCol : 0u) | (p.row_stats ? kVarRowStats : 0u) |

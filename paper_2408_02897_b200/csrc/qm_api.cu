@@ -400,11 +400,12 @@ static qm_status probe_phases(const qm_operand* Lo, const qm_operand* Ro, const 
                     !grouped(R, cfg->gran_r, cfg->batch_groups_r) &&
                     pair_prepare_serves(L, cfg->gran_l, dl_draw != nullptr, R, cfg->gran_r, dr_draw != nullptr);
   // the error word, the finished-CTA counter and both max|x| buffers are adjacent: one clear
+  const uint32_t* flags = nullptr;
   if (pair) {
     const PairSide side[2] = {
         {L, cfg->fmt_l, cfg->gran_l, cl_mn, dl_draw, reinterpret_cast<uint32_t*>(base + w.off_pl), dl, cl},
         {R, cfg->fmt_r, cfg->gran_r, cr_mn, dr_draw, reinterpret_cast<uint32_t*>(base + w.off_pr), dr, cr}};
-    st = launch_pair_prepare(side, err, 64, s);
+    st = launch_pair_prepare(side, err, 64, &flags, s);
     if (st != QM_OK) return st;
   } else if ((phases & kClear) && clear_later && clear_later->n < kClearMax) {
     clear_later->ptr[clear_later->n] = base;                 // cleared with others by one kernel
@@ -432,13 +433,13 @@ static qm_status probe_phases(const qm_operand* Lo, const qm_operand* Ro, const 
     p.cl = cl; p.cr = cr; p.cl_mn = cl_mn; p.cr_mn = cr_mn;
     p.fmt_l = cfg->fmt_l; p.fmt_r = cfg->fmt_r;
     p.dl = dl; p.gran_l = cfg->gran_l; p.dr = dr; p.gran_r = cfg->gran_r;
-    p.g = g; p.partials = part; p.err_word = err;
+    p.g = g; p.partials = part; p.err_word = err; p.prepare_flags = flags;
     p.done_counter = err + 1;               // second word of the cleared error slot
     p.result = out;
     p.row_stats = cfg->row_stats;
     return launch_tc_probe(p, s);           // the last CTA writes the record
   }
-  return launch_simt_probe(L, R, cl, cfg->fmt_l, dl, cfg->gran_l, cr, cfg->fmt_r, dr, cfg->gran_r, part, err + 1, err, out, s);
+  return launch_simt_probe(L, R, cl, cfg->fmt_l, dl, cfg->gran_l, cr, cfg->fmt_r, dr, cfg->gran_r, part, err + 1, err, flags, out, s);
 }
 
 qm_status qm_probe_layer(const qm_operand* Lo, const qm_operand* Ro, const qm_probe_cfg* cfg,

@@ -99,8 +99,10 @@ qm_status launch_quantize_multi(const View& x, int gran, const uint32_t* amax, i
 qm_status launch_quantize_cols(const View& x, const uint32_t* amax, int nf, const int* fmts, float* const* delta_out,
                                uint32_t* const* err_word, uint8_t* const* codes, cudaStream_t s);
 // Scale and quantize both operands of a probe in two launches (max|x|, then codes), for operands of modest
-// size.  `partial` needs pair_partial_words 32-bit words, not cleared; the first launch clears
-// `control` (at most 256 words), whose first word then takes QM_DEVERR_NONFINITE.
+// size, or in one for small ones.  `partial` needs pair_partial_words 32-bit words, not cleared; the first launch clears
+// `control` (64 words), whose first word then takes QM_DEVERR_NONFINITE; or *flags is not null and points at
+// kPrepareFlagWords words in it of which any is not zero then.
+constexpr int kPrepareFlagWord = 4, kPrepareFlags = 240, kPrepareFlagWords = kPrepareFlags / 4;
 struct PairSide {
   View v;
   int fmt, gran;
@@ -112,7 +114,7 @@ struct PairSide {
 };
 size_t pair_partial_words(const View& v, int gran);
 bool pair_prepare_serves(const View& l, int gran_l, bool draw_l, const View& r, int gran_r, bool draw_r);
-qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint32_t control_words, cudaStream_t s);
+qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint32_t control_words, const uint32_t** flags, cudaStream_t s);
 // Single pass per row: absmax, delta, codes (contiguous contraction, per-channel).
 qm_status launch_scale_quantize_rows(const View& x, int fmt, float* delta_out, uint8_t* codes,
                                      void* abs_copy, uint32_t* err_word, cudaStream_t s);
@@ -156,7 +158,7 @@ int simt_probe_blocks(GemmShape g);
 qm_status launch_simt_probe(const View& L, const View& R, const uint8_t* cl, int fmt_l,
                             const float* dl, int gran_l, const uint8_t* cr, int fmt_r,
                             const float* dr, int gran_r, double* partials, uint32_t* done_counter,
-                            uint32_t* err_word, qm_metric_result* out, cudaStream_t s);
+                            uint32_t* err_word, const uint32_t* prepare_flags, qm_metric_result* out, cudaStream_t s);
 
 // ---- tensor-core GEMMs (gemm_tc.cu) ---------------------------------------
 struct TcProbeArgs {
@@ -177,6 +179,7 @@ struct TcProbeArgs {
   qm_metric_result* result;                 // written by the last CTA to finish
   uint32_t* err_word;
   const uint32_t* err_also[2] = {nullptr, nullptr};   // error words of other probes whose kernels made this probe's codes
+  const uint32_t* prepare_flags = nullptr;            // the flags of launch_pair_prepare, or null
   double* row_stats = nullptr;              // optional per-row Eq. 3 sums (zeroed by the caller), one-format probes only
   // Two formats in one pass (cl2 != nullptr): codes and scales of the second format, same
   // granularities; `result` then points at two records and `partials` holds 2 x tc_probe_records.

@@ -2,6 +2,7 @@
 // All of them are HBM-bound streaming kernels: 128-bit coalesced loads, warp-shuffle and
 // shared-memory reductions, one atomicMax per block and group.
 #include <algorithm>
+#include <type_traits>
 
 #include "quant_device.cuh"
 
@@ -1299,76 +1300,134 @@ struct PairArgs {
   PairOperand op[2];
   uint32_t* control;                      // cleared by the first kernel; its first word takes the error flags
   uint32_t control_words;
+  uint32_t clusters[2];                   // the one-launch form: clusters of each operand
 };
 
-template <typename T>
-__device__ __forceinline__ void pair_max(const PairOperand& o, uint32_t block, uint32_t (&s)[32][64]) {
+// Eight elements as loaded, and running maxima of their magnitudes, element by element (bf16: two to a word).
+template <typename T> struct Raw8;
+template <> struct Raw8<__nv_bfloat16> {
+  static constexpr int kWords = 4;
+  uint32_t w[4];
+  __device__ __forceinline__ void load(const __nv_bfloat16* p, int live) {
+    if (live >= 8) {
+      const uint4 q = __ldg(reinterpret_cast<const uint4*>(p));
+      w[0] = q.x; w[1] = q.y; w[2] = q.z; w[3] = q.w;
+    } else {
+      const unsigned short* e = reinterpret_cast<const unsigned short*>(p);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) w[j] = (2 * j < live ? (uint32_t)__ldg(e + 2 * j) : 0u) | (2 * j + 1 < live ? (uint32_t)__ldg(e + 2 * j + 1) << 16 : 0u);
+    }
+  }
+  static __device__ __forceinline__ uint32_t upper(uint32_t m, uint32_t x) { return __vmaxu2(m, x & 0x7fff7fffu); }
+  static __device__ __forceinline__ uint32_t both(uint32_t m, uint32_t n) { return __vmaxu2(m, n); }
+  // element j of the maxima as an fp32 pattern
+  static __device__ __forceinline__ uint32_t element(const uint32_t* m, int j) { return j & 1 ? m[j >> 1] & 0xffff0000u : m[j >> 1] << 16; }
+};
+template <> struct Raw8<float> {
+  static constexpr int kWords = 8;
+  uint32_t w[8];
+  __device__ __forceinline__ void load(const float* p, int live) {
+    if (live >= 8) {
+      const uint4 q = __ldg(reinterpret_cast<const uint4*>(p)), r = __ldg(reinterpret_cast<const uint4*>(p) + 1);
+      w[0] = q.x; w[1] = q.y; w[2] = q.z; w[3] = q.w; w[4] = r.x; w[5] = r.y; w[6] = r.z; w[7] = r.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) w[j] = j < live ? __float_as_uint(__ldg(p + j)) : 0u;
+    }
+  }
+  static __device__ __forceinline__ uint32_t upper(uint32_t m, uint32_t x) { return max(m, x & 0x7fffffffu); }
+  static __device__ __forceinline__ uint32_t both(uint32_t m, uint32_t n) { return max(m, n); }
+  static __device__ __forceinline__ uint32_t element(const uint32_t* m, int j) { return m[j]; }
+};
+
+// max|x| of every blocks-th piece of the tensor; valid in warp 0.  AHEAD: loads of a thread on their way together (a round trip
+// is what these loops wait for).
+template <typename T, int AHEAD>
+__device__ __forceinline__ uint32_t pair_tensor_max(const PairOperand& o, uint32_t block, uint32_t blocks) {
+  using Raw = Raw8<T>;
   const View& v = o.v;
   const T* x = static_cast<const T*>(v.data);
-  if (!o.per_channel) {
-    const bool along_c = v.s_c == 1;
-    const int64_t inner = along_c ? v.c : v.nc, line_stride = along_c ? v.s_nc : v.s_c;
-    const uint32_t stride = (uint32_t)o.blocks_max * kThreads;
-    uint32_t acc = 0;
-    for (uint32_t g0 = block * kThreads + threadIdx.x; g0 < o.total_groups; g0 += 4 * stride) {
-      Vec8 w[4];
+  const bool along_c = v.s_c == 1;
+  const int64_t inner = along_c ? v.c : v.nc, line_stride = along_c ? v.s_nc : v.s_c;
+  const uint32_t stride = blocks * kThreads;
+  uint32_t acc[Raw::kWords] = {};
+  auto pass = [&](auto whole) {            // every group has eight elements: no branch between the loads
+    for (uint32_t g0 = block * kThreads + threadIdx.x; g0 < o.total_groups; g0 += AHEAD * stride) {
+      Raw w[AHEAD];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < AHEAD; ++u) {
         const uint32_t g = g0 + u * stride < o.total_groups ? g0 + u * stride : g0;      // repeats change no maximum
         const uint32_t line = o.by_groups.div(g), b = o.by_lines.div(line);
-        const int64_t k = (int64_t)(g - line * o.groups_per_line) * 8;
-        const T* p = x + (int64_t)b * v.s_b + (int64_t)(line - b * o.lines) * line_stride + k;
-        if (k + 8 <= inner) {
-          w[u] = Loader<T>::load8(p);
-        } else {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) w[u].v[j] = k + j < inner ? Loader<T>::load1(p, j) : 0.f;
-        }
+        const uint32_t k = (g - line * o.groups_per_line) * 8;
+        w[u].load(x + (int64_t)b * v.s_b + (int64_t)(line - b * o.lines) * line_stride + k, decltype(whole)::value ? 8 : (int)min((uint32_t)inner - k, 8u));
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) acc = absmax8(w[u], acc);
+      for (int u = 0; u < AHEAD; ++u)
+#pragma unroll
+        for (int j = 0; j < Raw::kWords; ++j) acc[j] = Raw::upper(acc[j], w[u].w[j]);
     }
-    acc = block_max(acc);
-    if (threadIdx.x == 0) o.partial[block] = acc;
+  };
+  if ((inner & 7) == 0) pass(std::true_type{}); else pass(std::false_type{});
+#pragma unroll
+  for (int j = 1; j < Raw::kWords; ++j) acc[0] = Raw::both(acc[0], acc[j]);
+  return block_max(max(Raw::element(acc, 0), Raw::kWords == 4 ? Raw::element(acc, 1) : 0u));
+}
+// The maxima of 8 << lane_bits columns from `first` on of batch element b over rows r0 .. r1 - 1, left in s: thread t < 8 <<
+// lane_bits returns that of column first + t.
+template <typename T, int AHEAD>
+__device__ __forceinline__ uint32_t pair_column_max(const PairOperand& o, int64_t b, int64_t first, int lane_bits, int64_t r0, int64_t r1,
+                                                    uint32_t* s) {
+  using Raw = Raw8<T>;
+  const View& v = o.v;
+  const int cols = 8 << lane_bits, rows_at_once = kThreads >> lane_bits;
+  const int tx = threadIdx.x & ((1 << lane_bits) - 1), ty = threadIdx.x >> lane_bits;
+  const int64_t col0 = first + tx * 8;
+  const T* base = static_cast<const T*>(v.data) + b * v.s_b + col0;
+  uint32_t acc[Raw::kWords] = {};
+  if (col0 < v.nc) {
+    const int live = v.nc - col0 < 8 ? (int)(v.nc - col0) : 8;
+    for (int64_t r = r0 + ty; r < r1; r += AHEAD * rows_at_once) {
+      Raw w[AHEAD];
+#pragma unroll
+      for (int u = 0; u < AHEAD; ++u) {
+        const int64_t row = r + u * rows_at_once < r1 ? r + u * rows_at_once : r;
+        w[u].load(base + row * v.s_c, live);
+      }
+#pragma unroll
+      for (int u = 0; u < AHEAD; ++u)
+#pragma unroll
+        for (int j = 0; j < Raw::kWords; ++j) acc[j] = Raw::upper(acc[j], w[u].w[j]);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) s[ty * cols + tx * 8 + j] = Raw::element(acc, j);
+  __syncthreads();
+  uint32_t m = 0;
+  if ((int)threadIdx.x < cols)
+    for (int j = 0; j < rows_at_once; ++j) m = max(m, s[j * cols + threadIdx.x]);
+  return m;
+}
+
+template <typename T>
+__device__ __forceinline__ void pair_max(const PairOperand& o, uint32_t block, uint32_t* s) {
+  const View& v = o.v;
+  if (!o.per_channel) {
+    const uint32_t m = pair_tensor_max<T, 4>(o, block, (uint32_t)o.blocks_max);
+    if (threadIdx.x == 0) o.partial[block] = m;
     return;
   }
   // a column each: 64 columns of one batch element, one slice of the contraction
   const uint32_t slice = block % (uint32_t)o.n_partial, rest = block / (uint32_t)o.n_partial;
   const uint32_t b = o.by_max_cols.div(rest), cb = rest - b * o.max_cols;
-  const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
-  const int64_t col0 = (int64_t)cb * 64 + tx * 8, per = (v.c + o.n_partial - 1) / o.n_partial;
-  const int64_t r0 = slice * per, r1 = r0 + per < v.c ? r0 + per : v.c;
-  const T* base = x + (int64_t)b * v.s_b + col0;
-  uint32_t acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  if (col0 < v.nc) {
-    const int live = v.nc - col0 < 8 ? (int)(v.nc - col0) : 8;
-#pragma unroll 4
-    for (int64_t r = r0 + ty; r < r1; r += 32) {
-      Vec8 w;
-      if (live == 8) {
-        w = Loader<T>::load8(base + r * v.s_c);
-      } else {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) w.v[j] = j < live ? Loader<T>::load1(base, r * v.s_c + j) : 0.f;
-      }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) acc[j] = max(acc[j], absbits_f32(__float_as_uint(w.v[j])));
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < 8; ++j) s[ty][tx * 8 + j] = acc[j];
-  __syncthreads();
-  if (threadIdx.x < 64) {
-    uint32_t m = 0;
-    for (int j = 0; j < 32; ++j) m = max(m, s[j][threadIdx.x]);
-    const int64_t col = (int64_t)cb * 64 + threadIdx.x;
-    if (col < v.nc) o.partial[((int64_t)slice * v.batch + b) * v.nc + col] = m;
-  }
+  const int64_t per = (v.c + o.n_partial - 1) / o.n_partial, r0 = slice * per, r1 = r0 + per < v.c ? r0 + per : v.c;
+  const uint32_t m = pair_column_max<T, 4>(o, b, (int64_t)cb * 64, 3, r0, r1, s);
+  const int64_t col = (int64_t)cb * 64 + threadIdx.x;
+  if (threadIdx.x < 64 && col < v.nc) o.partial[((int64_t)slice * v.batch + b) * v.nc + col] = m;
 }
 
 __global__ void __launch_bounds__(kThreads) pair_max_kernel(const PairArgs a) {
   pdl_prologue();
-  __shared__ uint32_t s[32][64];
+  __shared__ uint32_t s[32 * 64];
   if (blockIdx.x == 0 && threadIdx.x < a.control_words) a.control[threadIdx.x] = 0u;
   const bool right = blockIdx.x >= (uint32_t)a.op[0].blocks_max;
   const PairOperand& o = right ? a.op[1] : a.op[0];
@@ -1378,36 +1437,26 @@ __global__ void __launch_bounds__(kThreads) pair_max_kernel(const PairArgs a) {
   else pair_max<float>(o, block, s);
 }
 
-template <typename T, int FMT>
-__device__ __forceinline__ void pair_quantize(const PairOperand& o, uint32_t* err, uint32_t block, uint4* smem) {
+// The scale of an output row (0: of the tensor) from its max|x|; the thread that is told to stores it.
+template <int FMT>
+__device__ __forceinline__ float pair_scale(const PairOperand& o, uint32_t bits, int64_t at, bool writer, uint32_t* err) {
+  const float d = bits == 0 ? 1.0f : __fdiv_rn(__uint_as_float(bits), fmt_qmax(FMT));
+  if (writer) {
+    o.delta[at] = d;
+    if (bits >= 0x7f800000u) atomicOr(err, QM_DEVERR_NONFINITE);
+  }
+  return d;
+}
+
+// The codes of a block of the second kernel, whatever takes its maxima: d_tensor where there is one scale, else
+// col_bits(row of the output) its max|x|.
+template <typename T, int FMT, typename Bits>
+__device__ __forceinline__ void pair_codes(const PairOperand& o, uint32_t* err, uint32_t block, uint4* smem, float d_tensor, Bits col_bits) {
   const View& v = o.v;
   const T* x = static_cast<const T*>(v.data);
   const int64_t ldc = (v.c + 15) & ~(int64_t)15;
-  const float qmax = fmt_qmax(FMT);
-  if (o.path == kPairRows) {
-    scale_quantize_rows<T, FMT, 32>(x, v.nc, v.c, v.s_nc, v.batch, v.s_b, qmax, o.delta, o.codes, ldc, nullptr, err, block);
-    return;
-  }
-  // the scale of an output row from its partial maxima; the thread that is told to stores it
-  auto finish = [&](uint32_t bits, int64_t at, bool writer) {
-    const float d = bits == 0 ? 1.0f : __fdiv_rn(__uint_as_float(bits), qmax);
-    if (writer) {
-      o.delta[at] = d;
-      if (bits >= 0x7f800000u) atomicOr(err, QM_DEVERR_NONFINITE);
-    }
-    return d;
-  };
-  float d_tensor = 1.f;
-  if (!o.per_channel) {
-    uint32_t m = 0;
-    for (int i = threadIdx.x & 31; i < o.n_partial; i += 32) m = max(m, __ldg(o.partial + i));
-    d_tensor = finish(warp_max(m), 0, block == 0 && threadIdx.x == 0);
-  }
   auto scale = [&](int64_t row, bool writer) {
-    if (!o.per_channel) return d_tensor;
-    uint32_t m = 0;
-    for (int i = 0; i < o.n_partial; ++i) m = max(m, __ldg(o.partial + (int64_t)i * v.batch * v.nc + row));
-    return finish(m, row, writer);
+    return o.per_channel ? pair_scale<FMT>(o, col_bits(row), row, writer, err) : d_tensor;
   };
   if (o.path == kPairChunks) {              // contiguous contraction: sixteen elements per thread
     const uint32_t chunks = (uint32_t)(ldc >> 4), i = block * kThreads + threadIdx.x;
@@ -1447,11 +1496,7 @@ __device__ __forceinline__ void pair_quantize(const PairOperand& o, uint32_t* er
       MultiOut out{};
       out.codes[FMT] = o.codes; out.delta_out[FMT] = o.delta; out.err_word[FMT] = err;
       const int64_t row0 = (int64_t)at.y * kPairColRows, row1 = row0 + kPairColRows < v.c ? row0 + kPairColRows : v.c;
-      auto bits = [&](int64_t col) {
-        uint32_t m = 0;
-        for (int i = 0; i < o.n_partial; ++i) m = max(m, __ldg(o.partial + ((int64_t)i * v.batch + at.z) * v.nc + col));
-        return m;
-      };
+      auto bits = [&](int64_t col) { return col_bits((int64_t)at.z * v.nc + col); };
       quantize_cols<1 << FMT>(x + (int64_t)at.z * v.s_b, v.nc, v.s_c, row0, row1, at.x, o.col_lane_bits, bits, at.y == 0, out, (int64_t)at.z * v.nc,
                               (int64_t)at.z * v.c, (v.nc + 15) & ~(int64_t)15, reinterpret_cast<ColScales*>(smem));
       return;
@@ -1474,6 +1519,27 @@ __device__ __forceinline__ void pair_quantize(const PairOperand& o, uint32_t* er
   }
 }
 
+template <typename T, int FMT>
+__device__ __forceinline__ void pair_quantize(const PairOperand& o, uint32_t* err, uint32_t block, uint4* smem) {
+  const View& v = o.v;
+  if (o.path == kPairRows) {
+    scale_quantize_rows<T, FMT, 32>(static_cast<const T*>(v.data), v.nc, v.c, v.s_nc, v.batch, v.s_b, fmt_qmax(FMT), o.delta, o.codes,
+                                    (v.c + 15) & ~(int64_t)15, nullptr, err, block);
+    return;
+  }
+  float d_tensor = 1.f;
+  if (!o.per_channel) {
+    uint32_t m = 0;
+    for (int i = threadIdx.x & 31; i < o.n_partial; i += 32) m = max(m, __ldg(o.partial + i));
+    d_tensor = pair_scale<FMT>(o, warp_max(m), 0, block == 0 && threadIdx.x == 0, err);
+  }
+  pair_codes<T, FMT>(o, err, block, smem, d_tensor, [&](int64_t row) {
+    uint32_t m = 0;
+    for (int i = 0; i < o.n_partial; ++i) m = max(m, __ldg(o.partial + (int64_t)i * v.batch * v.nc + row));
+    return m;
+  });
+}
+
 // F0, F1: the operands' formats; T: their element type.
 template <typename T, int F0, int F1>
 __global__ void __launch_bounds__(kThreads) pair_quantize_kernel(const PairArgs a) {
@@ -1482,6 +1548,121 @@ __global__ void __launch_bounds__(kThreads) pair_quantize_kernel(const PairArgs 
   static_assert(sizeof(float) * 64 * 65 <= sizeof(uint4) * TileSmem<1>::kVec, "the general tile has to fit");
   if (blockIdx.x < (uint32_t)a.op[0].blocks_quant) pair_quantize<T, F0>(a.op[0], a.control, blockIdx.x, smem);
   else pair_quantize<T, F1>(a.op[1], a.control, blockIdx.x - a.op[0].blocks_quant, smem);
+}
+
+// ---------------------------------------------------------------- both operands of a small probe in one launch
+// Small enough that a cluster of eight blocks takes the maxima that it needs by itself, each block an eighth of them, and
+// exchanges them through distributed shared memory: no block waits for another cluster, so the chain of a probe is one launch
+// shorter.
+//   one scale per tensor:      every cluster goes over the whole tensor (it comes from L2) and then makes its own share of the codes;
+//   one per strided channel:   a cluster to a strip of columns, a block to an eighth of the contraction;
+//   one per contiguous row:    a warp to a row, as in the two-launch form.
+// Non-finite maxima are flagged in a byte for each block, always written: nobody could clear a common word ahead of
+// all blocks.  They lie in the control block, which the products' last block reads.
+constexpr int kOnceBlocks = 8;
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// v into word `at` of the same array in block `rank` of the cluster
+__device__ __forceinline__ void cluster_store(uint32_t* at, uint32_t rank, uint32_t v) {
+  uint32_t to;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"((uint32_t)__cvta_generic_to_shared(at)), "r"(rank));
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(to), "r"(v) : "memory");
+}
+
+// s_max: a row of 256 maxima from each block of the cluster.
+template <typename T, int FMT>
+__device__ __forceinline__ void pair_once(const PairOperand& o, uint32_t* err, uint32_t cluster, uint32_t clusters, uint32_t rank, uint4* smem,
+                                          uint32_t (&s_max)[kOnceBlocks][256]) {
+  constexpr int kAhead = 16 / sizeof(T);
+  const View& v = o.v;
+  if (o.path == kPairRows) {
+    cluster_wait();
+    const uint32_t block = cluster * kOnceBlocks + rank;
+    if (block < (uint32_t)o.blocks_quant)
+      scale_quantize_rows<T, FMT, 32>(static_cast<const T*>(v.data), v.nc, v.c, v.s_nc, v.batch, v.s_b, fmt_qmax(FMT), o.delta, o.codes,
+                                      (v.c + 15) & ~(int64_t)15, nullptr, err, block);
+    return;
+  }
+  auto cluster_max = [&](int i) {
+    uint32_t m = 0;
+#pragma unroll
+    for (int k = 0; k < kOnceBlocks; ++k) m = max(m, s_max[k][i]);
+    return m;
+  };
+  if (!o.per_channel) {
+    const uint32_t m = pair_tensor_max<T, kAhead>(o, rank, kOnceBlocks);
+    cluster_wait();                        // every block of the cluster has started
+    if (threadIdx.x < kOnceBlocks) cluster_store(&s_max[rank][0], threadIdx.x, m);
+    cluster_arrive();
+    cluster_wait();
+    const float d = pair_scale<FMT>(o, cluster_max(0), 0, cluster == 0 && rank == 0 && threadIdx.x == 0, err);
+    for (uint32_t block = cluster * kOnceBlocks + rank; block < (uint32_t)o.blocks_quant; block += clusters * kOnceBlocks) {
+      pair_codes<T, FMT>(o, err, block, smem, d, [](int64_t) { return 0u; });
+      __syncthreads();                     // the tile's shared memory
+    }
+    return;
+  }
+  const uint32_t b = o.by_max_cols.div(cluster), strip = cluster - b * o.max_cols;
+  constexpr int bits = 3;                  // strips of 64 columns
+  const int64_t first = (int64_t)strip << (bits + 3);
+  const int64_t per = (v.c + kOnceBlocks - 1) / kOnceBlocks, r0 = rank * per < v.c ? rank * per : v.c, r1 = r0 + per < v.c ? r0 + per : v.c;
+  const uint32_t m = pair_column_max<T, kAhead>(o, b, first, bits, r0, r1, reinterpret_cast<uint32_t*>(smem));
+  cluster_wait();
+  if ((int)threadIdx.x < 8 << bits) {
+#pragma unroll
+    for (int k = 0; k < kOnceBlocks; ++k) cluster_store(&s_max[rank][threadIdx.x], k, m);
+  }
+  cluster_arrive();
+  cluster_wait();
+  if constexpr (sizeof(T) == 2) {
+    if (o.path == kPairCols) {
+      MultiOut out{};
+      out.codes[FMT] = o.codes; out.delta_out[FMT] = o.delta; out.err_word[FMT] = err;
+      quantize_cols<1 << FMT>(static_cast<const T*>(v.data) + (int64_t)b * v.s_b, v.nc, v.s_c, r0, r1, strip, bits,
+                              [&](int64_t col) { return cluster_max((int)(col - first)); }, rank == 0, out, (int64_t)b * v.nc,
+                              (int64_t)b * v.c, (v.nc + 15) & ~(int64_t)15, reinterpret_cast<ColScales*>(smem));
+      return;
+    }
+  }
+  for (uint32_t y = rank; y < o.gy; y += kOnceBlocks) {
+    pair_codes<T, FMT>(o, err, (b * o.gy + y) * o.gx + strip, smem, 1.f, [&](int64_t row) { return cluster_max((int)(row - b * v.nc - first)); });
+    __syncthreads();
+  }
+}
+
+template <typename T, int F0, int F1>
+__global__ void __launch_bounds__(kThreads) pair_once_kernel(const PairArgs a) {
+  __shared__ uint4 smem[TileSmem<1>::kVec];
+  __shared__ uint32_t s_max[kOnceBlocks][256];
+  __shared__ uint32_t s_err;
+  cluster_arrive();
+  if (threadIdx.x == 0) s_err = 0;
+  __syncthreads();
+  pdl_prologue();
+  uint8_t* const flags = reinterpret_cast<uint8_t*>(a.control + kPrepareFlagWord);
+  if (blockIdx.x == 0) {
+    if (threadIdx.x < kPrepareFlagWord) a.control[threadIdx.x] = 0u;
+    if (threadIdx.x >= gridDim.x && threadIdx.x < kPrepareFlags) flags[threadIdx.x] = 0;
+  }
+  const uint32_t cluster = blockIdx.x / kOnceBlocks, rank = blockIdx.x % kOnceBlocks;
+  if (cluster < a.clusters[0]) pair_once<T, F0>(a.op[0], &s_err, cluster, a.clusters[0], rank, smem, s_max);
+  else pair_once<T, F1>(a.op[1], &s_err, cluster - a.clusters[0], a.clusters[1], rank, smem, s_max);
+  __syncthreads();
+  if (threadIdx.x == 0) flags[blockIdx.x] = s_err ? 1 : 0;
+}
+
+// Clusters of an operand in the one-launch form; 0: not served.  A tensor that every cluster reads whole may have 512 KB, a
+// column 4096 entries (an eighth of them to a block).  Whole probes in a row, two launches / one, us: fp32 128 x 256 x 256 20.8 / 17.4,
+// 64^3 16.5 / 12.6; bf16 64^3 16.0 / 13.2, 512^3 under one scale 20.6 / 20.2, under channel scales 24.2 / 19.6, 256 x 256 x
+// 1024 both strided, channel 27.4 / 22.6, 128 x 64 x 2048 32.1 / 27.9.
+uint32_t once_clusters(const PairOperand& o, int elem) {
+  const View& v = o.v;
+  if (!o.per_channel) {
+    if (v.nc * v.c * v.batch * elem > (512 << 10)) return 0;
+    return (uint32_t)std::min((o.blocks_quant + kOnceBlocks - 1) / kOnceBlocks, 12);
+  }
+  if (o.path == kPairRows) return (uint32_t)((o.blocks_quant + kOnceBlocks - 1) / kOnceBlocks);
+  return v.c <= 4096 ? (uint32_t)(o.max_cols * v.batch) : 0;
 }
 
 int grid_for(int64_t work_items, int per_sm) {
@@ -1792,8 +1973,9 @@ bool pair_prepare_serves(const View& l, int gran_l, bool draw_l, const View& r, 
          (l.nc + r.nc) * l.c * l.batch < (1ll << 22);
 }
 
-qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint32_t control_words, cudaStream_t s) {
+qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint32_t control_words, const uint32_t** flags, cudaStream_t s) {
   PairArgs a{};
+  *flags = nullptr;
   a.control = control; a.control_words = control_words;
   for (int i = 0; i < 2; ++i) {
     const PairSide& in = side[i];
@@ -1839,14 +2021,37 @@ qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint
       o.blocks_max = (int32_t)((int64_t)o.max_cols * v.batch * o.n_partial);
     }
   }
+  const int f0 = side[0].fmt, f1 = side[1].fmt;
+  const bool bf16 = side[0].v.dtype == QM_DT_BF16;
+  for (int i = 0; i < 2; ++i) a.clusters[i] = once_clusters(a.op[i], bf16 ? 2 : 4);
+  if (a.clusters[0] && a.clusters[1] && (a.clusters[0] + a.clusters[1]) * kOnceBlocks <= (uint32_t)kPrepareFlags) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((a.clusters[0] + a.clusters[1]) * kOnceBlocks); cfg.blockDim = dim3(kThreads); cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kOnceBlocks; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at; cfg.numAttrs = pdl_enabled() ? 2 : 1;
+#define QM_PO(F0, F1)                                                                              \
+  QM_CUDA_OK(bf16 ? cudaLaunchKernelEx(&cfg, pair_once_kernel<__nv_bfloat16, F0, F1>, a)           \
+                  : cudaLaunchKernelEx(&cfg, pair_once_kernel<float, F0, F1>, a))
+    if (f0 == QM_FMT_INT8) QM_PO(QM_FMT_INT8, QM_FMT_INT8);          // (INT8 goes with INT8 only)
+    else if (f0 == QM_FMT_E4M3 && f1 == QM_FMT_E4M3) QM_PO(QM_FMT_E4M3, QM_FMT_E4M3);
+    else if (f0 == QM_FMT_E4M3) QM_PO(QM_FMT_E4M3, QM_FMT_E5M2);
+    else if (f1 == QM_FMT_E4M3) QM_PO(QM_FMT_E5M2, QM_FMT_E4M3);
+    else QM_PO(QM_FMT_E5M2, QM_FMT_E5M2);
+#undef QM_PO
+    count_launch();
+    *flags = control + kPrepareFlagWord;
+    return QM_OK;
+  }
   const unsigned maxima = (unsigned)(a.op[0].blocks_max + a.op[1].blocks_max);
   QM_CUDA_OK(launch_pdl(pair_max_kernel, dim3(maxima > 0 ? maxima : 1), dim3(kThreads), 0, s, a));
   const dim3 grid((unsigned)(a.op[0].blocks_quant + a.op[1].blocks_quant));
-  const bool bf16 = side[0].v.dtype == QM_DT_BF16;
 #define QM_PQ(F0, F1)                                                                                            \
   QM_CUDA_OK(bf16 ? launch_pdl(pair_quantize_kernel<__nv_bfloat16, F0, F1>, grid, dim3(kThreads), 0, s, a)        \
                   : launch_pdl(pair_quantize_kernel<float, F0, F1>, grid, dim3(kThreads), 0, s, a))
-  const int f0 = side[0].fmt, f1 = side[1].fmt;
   if (f0 == QM_FMT_INT8) QM_PQ(QM_FMT_INT8, QM_FMT_INT8);          // (INT8 goes with INT8 only)
   else if (f0 == QM_FMT_E4M3 && f1 == QM_FMT_E4M3) QM_PQ(QM_FMT_E4M3, QM_FMT_E4M3);
   else if (f0 == QM_FMT_E4M3) QM_PQ(QM_FMT_E4M3, QM_FMT_E5M2);

@@ -79,3 +79,36 @@ def test_non_finite_operands_are_flagged(gran, where, cd):
     a, b = shape(x), shape(y)
     r = qm.qm_probe_layer(qm.operand_of(a, cd), qm.operand_of(b, cd), "e4m3", "e4m3", gran, gran)
     assert r.device_error & 1
+
+
+# The one-launch form: operands of 512 KB and just above, strips of 64 columns whole and ragged with fewer rows than
+# blocks of a cluster, contractions up to 4096 and above, as many blocks as there are flags and more.
+@pytest.mark.parametrize("M,N,K,batch", [(512, 511, 512, 1), (512, 513, 512, 1), (65, 3, 16, 1), (3, 129, 4096, 1), (3, 129, 4112, 1),
+                                         (960, 128, 32, 1), (968, 960, 32, 1), (70, 40, 112, 4)])
+@pytest.mark.parametrize("cl,cr", [(-1, -2), (-2, -1)])
+@pytest.mark.parametrize("fmt,gran_l,gran_r", [("e4m3", "tensor", "channel"), ("int8", "channel", "tensor"), ("e5m2", "channel", "channel"),
+                                               ("e4m3", "tensor", "tensor")])
+def test_small_operands_either_side_of_the_one_launch_form(M, N, K, batch, cl, cr, fmt, gran_l, gran_r):
+    rng = workloads._rng(M + 5 * N + K)
+    Ld, Rd = stored(rng, M, K, cl, batch, torch.bfloat16)[1], stored(rng, N, K, cr, batch, torch.bfloat16)[1]
+    Lo, Ro = qm.operand_of(Ld, cl), qm.operand_of(Rd, cr)
+    plan = qm.ProbePlan(Lo, Ro, fmt, fmt, gran_l, gran_r)
+    plan.ws.fill_(0xA5)
+    plan.launch(Lo, Ro)
+    b = qm.ProbeBatch([(Lo, Ro, fmt, fmt, gran_l, gran_r)])
+    b.launch()
+    torch.cuda.synchronize()
+    got, other = plan.result(), b.results()[0]
+    assert got.device_error == other.device_error == 0
+    for k in FIELDS:
+        assert abs(got.record()[k] - other.record()[k]) <= 1e-12 * abs(other.record()[k]), k
+    # a value that is not finite is flagged wherever it lies, also by the last block; the next call starts afresh
+    for t in (Ld, Rd):
+        at = tuple(s - 1 for s in t.shape)
+        old = t[at].clone()
+        t[at] = float("nan")
+        plan.launch(Lo, Ro)
+        assert plan.result().device_error & 1
+        t[at] = old
+    plan.launch(Lo, Ro)
+    assert plan.result().device_error == 0
