@@ -704,8 +704,9 @@ struct Slot {
   uint8_t* room; size_t room_left; // for the codes of further slots of the same view
   bool keeps_amax;                 // false when the single-pass per-row kernel prepares it (no maxima are stored)
   int code_root, pass_root, amax_root, home;
-  int stream;                      // index of the library stream its kernels go to
+  int stream;                      // index of the library stream its kernels go to, or kCallersStream
 };
+constexpr int kCallersStream = -1;
 
 bool same_view(const View& a, const View& b) {
   return a.data == b.data && a.dtype == b.dtype && a.nc == b.nc && a.c == b.c && a.s_nc == b.s_nc && a.s_c == b.s_c &&
@@ -766,6 +767,29 @@ void find_home(std::vector<Slot>& slots, int t) {
     }
     return;
   }
+}
+
+// The slots that launch_prepare_many serves, all their formats with them, marked done.  Against a launch for each tensor and step
+// on eight streams, us per pass: 18 products of a layer of 256 with 256 tokens in two formats 133 / 67 (the host's time), BERT-base
+// forward 195 / 172, BERT-large layer 2860 / 2720, sweep layer 5900 / 5680.  (In groups of 16 to 96 MB, so that a group's codes
+// are made from L2, large passes take as long or longer: 5710 .. 5750.)
+std::vector<ManyTensor> prepared_together(std::vector<Slot>& slots, std::vector<char>& done) {
+  std::vector<ManyTensor> list;
+  for (size_t t = 0; t < slots.size(); ++t) {
+    const Slot& x = slots[t];
+    if (x.code_root != (int)t || x.pass_root != (int)t || x.amax_root != (int)t || x.stochastic || x.gran != QM_GRAN_TENSOR || !many_serves(x.v))
+      continue;
+    ManyTensor m{};
+    m.x = x.v; m.amax = x.amax;
+    for (size_t u = t; u < slots.size(); ++u) {
+      const Slot& y = slots[u];
+      if (y.code_root != (int)u || y.pass_root != (int)t || y.stochastic || m.codes[y.fmt]) continue;
+      m.delta[y.fmt] = y.delta; m.err[y.fmt] = y.err; m.codes[y.fmt] = y.codes;
+      done[u] = 1; slots[u].stream = kCallersStream;
+    }
+    list.push_back(m);
+  }
+  return list;
 }
 
 }  // namespace
@@ -850,10 +874,30 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
   // beside one another; whatever borrows from an earlier operand goes to that operand's stream,
   // behind the kernels that make what it borrows.  Probes that do not take the fused tensor-core
   // kernel (fp32 reference) run whole on one of those streams.
-  QM_CUDA_OK(cudaEventRecord(b->fork, user));
-  for (int j = 0; j < kBatchStreams; ++j) QM_CUDA_OK(cudaStreamWaitEvent(b->s[j], b->fork, 0));
+  // Dense tensors under one scale are prepared together, in two launches on the caller's stream; with nothing else to
+  // prepare the library's streams are not touched.
   int next_stream = 0;
   std::vector<char> done(slots.size(), 0);
+  const std::vector<ManyTensor> together = prepared_together(slots, done);
+  bool apart = false;                                 // something goes to the library's streams
+  for (size_t t = 0; t < slots.size(); ++t) apart |= slots[t].code_root == (int)t && !done[t];
+  for (int32_t i = 0; i < good; ++i) apart |= !plans[i].tc;
+  if (apart) QM_CUDA_OK(cudaEventRecord(b->fork, user));      // (an event between two kernels keeps the second from starting early)
+  for (size_t i = 0; i < together.size(); i += kManyTensors) {
+    const qm_status e = launch_prepare_many(&together[i], (int)std::min<size_t>(kManyTensors, together.size() - i), user);
+    if (e != QM_OK && st == QM_OK) st = e;
+  }
+  bool forked[kBatchStreams] = {};
+  qm_status fork_error = QM_OK;
+  auto stream_of = [&](int j) {                      // of a slot; a stream of the library follows what the caller's held before
+    if (j == kCallersStream) return user;
+    if (!forked[j]) {
+      forked[j] = true;
+      const cudaError_t e = cudaStreamWaitEvent(b->s[j], b->fork, 0);
+      if (e != cudaSuccess) { note_cuda_error(e, "cudaStreamWaitEvent"); fork_error = QM_ERR_CUDA; }
+    }
+    return b->s[j];
+  };
   for (size_t t = 0; t < slots.size(); ++t) {
     Slot& x = slots[t];
     if (x.code_root != (int)t) { x.stream = slots[x.code_root].stream; continue; }     // nothing to launch
@@ -864,9 +908,9 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
       // borrows max|x|, and was not served with its lender's formats
       x.stream = slots[x.pass_root].stream;
       const uint32_t* amax = slots[x.amax_root].amax;
-      if (codes_mn(x.v, x.stochastic)) e = launch_quantize_cols(x.v, amax, 1, &x.fmt, &x.delta, &x.err, &x.codes, b->s[x.stream]);
+      if (codes_mn(x.v, x.stochastic)) e = launch_quantize_cols(x.v, amax, 1, &x.fmt, &x.delta, &x.err, &x.codes, stream_of(x.stream));
       else e = launch_quantize(x.v, x.fmt, x.gran, reinterpret_cast<const float*>(amax), true, x.delta, x.err, x.codes, nullptr,
-                               nullptr, b->s[x.stream], draw);
+                               nullptr, stream_of(x.stream), draw);
     } else if (!x.keeps_amax) {
       x.stream = next_stream; next_stream = (next_stream + 1) % kBatchStreams;
       // this operand's format and the others that later probes ask for under the same scales' grouping: one read.  Rows that
@@ -880,16 +924,16 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
         fmts[nf] = y.fmt; deltas[nf] = y.delta; errs[nf] = y.err; codes[nf] = y.codes; ++nf;
         y.stream = x.stream; done[u] = 1;
       }
-      e = launch_scale_quantize_rows_multi(x.v, nf, fmts, deltas, errs, codes, b->s[x.stream]);
+      e = launch_scale_quantize_rows_multi(x.v, nf, fmts, deltas, errs, codes, stream_of(x.stream));
     } else {
       if (x.amax_root == (int)t) {
         x.stream = next_stream; next_stream = (next_stream + 1) % kBatchStreams;
-        e = launch_absmax(x.v, x.gran, x.amax, b->s[x.stream]);
-        if (e == QM_OK && grouped_scales(x)) e = launch_share_amax(x.amax, x.v.batch, x.groups, x.v.nc, b->s[x.stream]);
+        e = launch_absmax(x.v, x.gran, x.amax, stream_of(x.stream));
+        if (e == QM_OK && grouped_scales(x)) e = launch_share_amax(x.amax, x.v.batch, x.groups, x.v.nc, stream_of(x.stream));
       } else {
         x.stream = slots[x.amax_root].stream;
       }
-      cudaStream_t s = b->s[x.stream];
+      cudaStream_t s = stream_of(x.stream);
       const uint32_t* amax = slots[x.amax_root].amax;
       // this operand's format and those of the later operands that borrow its pass: one pass over
       // the tensor writes all their codes (round-to-nearest-even ones; stochastic ones go singly)
@@ -917,11 +961,13 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
   }
   for (int32_t i = 0; i < good; ++i) {
     if (plans[i].tc) continue;
-    cudaStream_t s = b->s[next_stream]; next_stream = (next_stream + 1) % kBatchStreams;
+    cudaStream_t s = stream_of(next_stream); next_stream = (next_stream + 1) % kBatchStreams;
     const qm_status e = probe_phases(&L[i], &R[i], &cfg[i], out + i, ws[i], ws_bytes[i], s, kPrepare | kProducts);
     if (e != QM_OK && st == QM_OK) st = e;
   }
+  if (st == QM_OK) st = fork_error;
   for (int j = 0; j < kBatchStreams; ++j) {
+    if (!forked[j]) continue;
     QM_CUDA_OK(cudaEventRecord(b->join[j], b->s[j]));
     QM_CUDA_OK(cudaStreamWaitEvent(user, b->join[j], 0));
   }

@@ -115,6 +115,12 @@ struct PairSide {
 size_t pair_partial_words(const View& v, int gran);
 bool pair_prepare_serves(const View& l, int gran_l, bool draw_l, const View& r, int gran_r, bool draw_r);
 qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint32_t control_words, const uint32_t** flags, cudaStream_t s);
+// Scale and quantize several dense bf16 tensors under one scale each (many_serves), in one to three formats, in two launches.
+// amax: zero on entry.  By format (qm_format): scale, flag word for a non-finite maximum (optional), codes (null: not asked for).
+constexpr int kManyTensors = 32;
+struct ManyTensor { View x; uint32_t* amax; float* delta[3]; uint32_t* err[3]; uint8_t* codes[3]; };
+bool many_serves(const View& x);
+qm_status launch_prepare_many(const ManyTensor* t, int n, cudaStream_t s);
 // Single pass per row: absmax, delta, codes (contiguous contraction, per-channel).
 qm_status launch_scale_quantize_rows(const View& x, int fmt, float* delta_out, uint8_t* codes,
                                      void* abs_copy, uint32_t* err_word, cudaStream_t s);

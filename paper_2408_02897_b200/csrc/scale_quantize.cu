@@ -1550,6 +1550,95 @@ __global__ void __launch_bounds__(kThreads) pair_quantize_kernel(const PairArgs 
   else pair_quantize<T, F1>(a.op[1], a.control, blockIdx.x - a.op[0].blocks_quant, smem);
 }
 
+// ---------------------------------------------------------------- the tensors of a batch in two launches
+// Dense bf16 tensors under one scale each: max|x| of all of them in one launch, the codes of all their formats in another.  A
+// launch for each tensor and step, spread over streams, is bound by its submission and by 3 to 4 us a launch where the tensors are
+// small: the four products of a BERT-base layer in two formats (six tensors, 46 MB) took 40 us to prepare in twelve launches.
+struct ManyMax { const uint8_t* x; uint64_t n_vec; uint32_t* amax; uint32_t block0; };      // n_vec: 32-byte vectors
+struct ManyCodes {
+  const uint8_t* x; const uint32_t* amax;
+  float* delta[3]; uint32_t* err[3]; uint4* codes[3];         // by format; codes null: not asked for
+  uint32_t chunks, block0;                                   // chunks: of 16 elements
+};
+template <typename E> struct ManyList { int n; E e[kManyTensors]; };
+static_assert(sizeof(ManyList<ManyCodes>) <= 4096, "kernel parameters");
+constexpr int kManyAhead = 4;              // 32-byte loads of a thread on their way together
+
+template <typename E>
+__device__ __forceinline__ int many_entry(const ManyList<E>& l, uint32_t block) {
+  int i = 0;
+  while (i + 1 < l.n && block >= l.e[i + 1].block0) ++i;
+  return i;
+}
+
+__global__ void __launch_bounds__(kThreads) absmax_many_kernel(const __grid_constant__ ManyList<ManyMax> l) {
+  const ManyMax e = l.e[many_entry(l, blockIdx.x)];
+  pdl_prologue();
+  const uint64_t i0 = (uint64_t)(blockIdx.x - e.block0) * (kThreads * kManyAhead) + threadIdx.x;
+  Vec256 v[kManyAhead];
+#pragma unroll
+  for (int u = 0; u < kManyAhead; ++u) {
+    const uint64_t i = i0 + u * kThreads;
+    v[u] = ld256<false>(e.x + (i < e.n_vec ? i : e.n_vec - 1) * 32);          // repeats change no maximum
+  }
+  uint32_t m = 0;
+  const uint32_t k = 0x7fff7fffu;
+#pragma unroll
+  for (int u = 0; u < kManyAhead; ++u) {
+    const uint32_t a = __vmaxu2(__vmaxu2(v[u].lo.x & k, v[u].lo.y & k), __vmaxu2(v[u].lo.z & k, v[u].lo.w & k));
+    const uint32_t b = __vmaxu2(__vmaxu2(v[u].hi.x & k, v[u].hi.y & k), __vmaxu2(v[u].hi.z & k, v[u].hi.w & k));
+    m = __vmaxu2(m, __vmaxu2(a, b));
+  }
+  const uint32_t acc = block_max(max(m & 0xffffu, m >> 16) << 16);
+  if (threadIdx.x == 0 && acc) atomicMax(e.amax, acc);
+}
+
+template <int CHUNKS>
+__global__ void __launch_bounds__(kThreads) quantize_many_kernel(const __grid_constant__ ManyList<ManyCodes> l) {
+  const uint32_t block = gridDim.x - 1 - blockIdx.x;         // backwards: what the maxima have read last is still in L2
+  const ManyCodes& e = l.e[many_entry(l, block)];
+  const uint32_t chunks = e.chunks, base = (block - e.block0) * (kThreads * CHUNKS) + threadIdx.x;
+  const bool writer = block == e.block0 && threadIdx.x == 0;
+  const uint8_t* const x = e.x;
+  pdl_prologue();
+  Vec256 w[CHUNKS];
+#pragma unroll
+  for (int u = 0; u < CHUNKS; ++u) {
+    const uint32_t i = base + u * kThreads;
+    w[u] = ld256<false>(x + 32 * (size_t)(i < chunks ? i : chunks - 1));
+  }
+  const uint32_t bits = __ldcg(e.amax);
+  auto format = [&](auto fmt) {
+    constexpr int F = decltype(fmt)::value;
+    uint4* const codes = e.codes[F];
+    if (!codes) return;
+    const float d = bits == 0 ? 1.0f : __fdiv_rn(__uint_as_float(bits), fmt_qmax(F));
+    if (writer) {
+      *e.delta[F] = d;
+      if (bits >= 0x7f800000u && e.err[F]) atomicOr(e.err[F], QM_DEVERR_NONFINITE);
+    }
+    if (QuotientPair::serves(d)) {
+      const QuotientPair quot(d);
+#pragma unroll
+      for (int u = 0; u < CHUNKS; ++u)
+        if (base + u * kThreads < chunks) codes[base + u * kThreads] = quant_bf16x16<F>(w[u].lo, w[u].hi, quot);
+    } else {
+      const Quotient quot(d);
+#pragma unroll 1
+      for (int u = 0; u < CHUNKS; ++u) {
+        if (base + u * kThreads >= chunks) break;
+        const Vec8 a = Loader<__nv_bfloat16>::load8(x + 32 * (size_t)(base + u * kThreads));
+        const Vec8 b = Loader<__nv_bfloat16>::load8(x + 32 * (size_t)(base + u * kThreads) + 16);
+        const uint2 p = quant8<F>(a, quot), q = quant8<F>(b, quot);
+        codes[base + u * kThreads] = make_uint4(p.x, p.y, q.x, q.y);
+      }
+    }
+  };
+  format(std::integral_constant<int, 0>{});
+  format(std::integral_constant<int, 1>{});
+  format(std::integral_constant<int, 2>{});
+}
+
 // ---------------------------------------------------------------- both operands of a small probe in one launch
 // Small enough that a cluster of eight blocks takes the maxima that it needs by itself, each block an eighth of them, and
 // exchanges them through distributed shared memory: no block waits for another cluster, so the chain of a probe is one launch
@@ -2058,6 +2147,37 @@ qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint
   else if (f1 == QM_FMT_E4M3) QM_PQ(QM_FMT_E5M2, QM_FMT_E4M3);
   else QM_PQ(QM_FMT_E5M2, QM_FMT_E5M2);
 #undef QM_PQ
+  count_launch(2);
+  return QM_OK;
+}
+
+bool many_serves(const View& x) {
+  return x.dtype == QM_DT_BF16 && x.c_contig() && (x.c & 15) == 0 && (x.nc == 1 || x.s_nc == x.c) && (x.batch == 1 || x.s_b == x.nc * x.c) &&
+         (reinterpret_cast<uintptr_t>(x.data) & 31) == 0 && x.nc * x.c * x.batch < (1ll << 35);
+}
+
+qm_status launch_prepare_many(const ManyTensor* t, int n, cudaStream_t s) {
+  if (n < 1 || n > kManyTensors) return QM_ERR_INVALID_ARG;
+  ManyList<ManyMax> m{};
+  ManyList<ManyCodes> q{};
+  m.n = q.n = n;
+  int64_t total = 0;
+  for (int i = 0; i < n; ++i) total += t[i].x.nc * t[i].x.c * t[i].x.batch / 16;
+  // four chunks to a thread where that still gives an SM eight blocks
+  const int chunks = total >= (int64_t)sm_count() * 8 * kThreads * 4 ? 4 : 1;
+  uint32_t blocks_m = 0, blocks_q = 0;
+  for (int i = 0; i < n; ++i) {
+    const int64_t c = t[i].x.nc * t[i].x.c * t[i].x.batch / 16;                  // a chunk of 16 elements is a vector of 32 bytes
+    m.e[i] = ManyMax{static_cast<const uint8_t*>(t[i].x.data), (uint64_t)c, t[i].amax, blocks_m};
+    ManyCodes& e = q.e[i];
+    e.x = static_cast<const uint8_t*>(t[i].x.data); e.amax = t[i].amax; e.chunks = (uint32_t)c; e.block0 = blocks_q;
+    for (int f = 0; f < 3; ++f) { e.delta[f] = t[i].delta[f]; e.err[f] = t[i].err[f]; e.codes[f] = reinterpret_cast<uint4*>(t[i].codes[f]); }
+    blocks_m += (uint32_t)((c + kThreads * kManyAhead - 1) / (kThreads * kManyAhead));
+    blocks_q += (uint32_t)((c + kThreads * chunks - 1) / (kThreads * chunks));
+  }
+  QM_CUDA_OK(launch_pdl(absmax_many_kernel, dim3(blocks_m), dim3(kThreads), 0, s, m));
+  QM_CUDA_OK(chunks == 4 ? launch_pdl(quantize_many_kernel<4>, dim3(blocks_q), dim3(kThreads), 0, s, q)
+                         : launch_pdl(quantize_many_kernel<1>, dim3(blocks_q), dim3(kThreads), 0, s, q));
   count_launch(2);
   return QM_OK;
 }

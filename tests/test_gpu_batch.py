@@ -149,3 +149,41 @@ def test_large_mixed_batch_spans_several_grouped_launches():
         torch.cuda.synchronize()
         for i, (g, s) in enumerate(zip(batch.results(), single)):
             assert _same(g, s), (i, cases[i][4:], g.record(), s.record())
+
+
+@pytest.mark.parametrize("count", [1, 2, 35])
+@pytest.mark.parametrize("fmts", [("e5m2",), ("e4m3", "e5m2", "int8")])
+def test_dense_tensors_prepared_together(count, fmts):
+    """The tensors of a batch that are dense and have one scale go through two launches, up to 32 at a time: sizes from
+    one chunk of sixteen elements to several blocks and a ragged last one, scales outside the range of the two-wide
+    quotient, an all-zero tensor, a value that is not finite at either end."""
+    rng = workloads._rng(140 + count)
+    sizes = [(1, 16), (3, 48), (250, 144), (1000, 272), (64, 64)]
+    pairs = []
+    for i in range(count):
+        M, K = sizes[(i + (0 if count > 1 else 3)) % len(sizes)]
+        L, R = workloads.normal(rng, (M, K)), workloads.normal(rng, (48, K), 0.05)
+        if i % 7 == 3:
+            L = L * 1e-30                        # scale below 2^-60
+        if i % 7 == 5:
+            R = torch.zeros_like(R)
+        pairs.append((L.cuda(), R.cuda()))
+    probes = [(qm.operand_of(L, -1), qm.operand_of(R, -1), f, f, "tensor", "tensor") for L, R in pairs for f in fmts]
+    single = [qm.qm_probe_layer(*p) for p in probes]
+    batch = qm.ProbeBatch(probes)
+    for _ in range(2):
+        batch.launch()
+        torch.cuda.synchronize()
+        assert all(_same(g, s) for g, s in zip(batch.results(), single))
+    for at in (0, -1):
+        for L, R in (pairs[0], pairs[-1]):
+            old = L.view(-1)[at].clone()
+            L.view(-1)[at] = float("inf")
+            batch.launch()
+            torch.cuda.synchronize()
+            flags = [r.device_error for r in batch.results()]
+            L.view(-1)[at] = old
+            assert sum(f & 1 for f in flags) == len(fmts), flags
+    batch.launch()
+    torch.cuda.synchronize()
+    assert all(r.device_error == 0 for r in batch.results())
