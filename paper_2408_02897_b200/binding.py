@@ -5,6 +5,7 @@ product L.R is described by `operand_of(tensor, contract_dim)`.
 """
 import ctypes as C
 import os
+import threading
 
 import torch
 
@@ -171,12 +172,10 @@ def operand_of(t, contract_dim):
     nd = t.dim() - 1 if cd == t.dim() - 2 else t.dim() - 2
     if cd == nd or cd < t.dim() - 2:
         raise QmError(1, "contract_dim must be one of the last two dimensions")
-    o = Operand()
-    o.data = t.data_ptr(); o.dtype = _DT[t.dtype]
-    o.noncontract = t.shape[nd]; o.contract = t.shape[cd]
-    o.stride_nc = t.stride(nd); o.stride_c = t.stride(cd)
-    o.batch = t.shape[0] if t.dim() == 3 else 1
-    o.stride_batch = t.stride(0) if t.dim() == 3 else 0
+    shape, stride = t.shape, t.stride()
+    batched = len(shape) == 3
+    o = Operand(t.data_ptr(), _DT[t.dtype], shape[nd], shape[cd], stride[nd], stride[cd],
+                shape[0] if batched else 1, stride[0] if batched else 0)
     o._keep = t
     return o
 
@@ -267,18 +266,34 @@ def _read_result(dev_buf):
     return MetricResult.from_buffer_copy(host)
 
 
+class _Spare(threading.local):
+    """Per thread, the pinned buffer of the last record of each kind that has been read."""
+
+    def __init__(self):
+        self.of = {}
+
+
+_spare = _Spare()
+
+
 class _HostRecord:
     """A result record in pinned host memory, which the last kernel of a call writes itself: reading it is a wait for
-    the stream, without a copy of its own."""
+    the stream, without a copy of its own.  The buffer goes back to its thread once it has been read, and no sooner: a call
+    that fails on the way does not return it."""
 
     def __init__(self, kind):
         self.kind = kind
-        self.buf = torch.empty(C.sizeof(kind), dtype=torch.uint8, device="cpu", pin_memory=True)
-        self.ptr = self.buf.data_ptr()
+        buf = _spare.of.pop(kind, None)
+        if buf is None:
+            buf = torch.empty(C.sizeof(kind), dtype=torch.uint8, device="cpu", pin_memory=True)
+        self.buf = buf
+        self.ptr = buf.data_ptr()
 
     def read(self, stream):
         (stream if stream is not None else torch.cuda.current_stream()).synchronize()
-        return self.kind.from_buffer_copy(C.string_at(self.ptr, C.sizeof(self.kind)))
+        res = self.kind.from_buffer_copy(C.string_at(self.ptr, C.sizeof(self.kind)))
+        _spare.of[self.kind] = self.buf
+        return res
 
 
 def qm_metric(ref, q, den, stream=None):
