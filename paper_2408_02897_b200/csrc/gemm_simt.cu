@@ -5,6 +5,7 @@
 #include <cuda_fp16.h>
 
 #include "qm_internal.h"
+#include "reduce.cuh"
 
 namespace qm {
 namespace {
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(kThreads, 2) simt_kernel(const SimtArgs a) {
   constexpr int T = C::T, SPLIT = C::SPLIT, KG = C::KG, KC = C::KC;
   extern __shared__ float4 smem4[];
   float* const smem = reinterpret_cast<float*>(smem4);
-  __shared__ double sred[5][kThreads / 32];
+  __shared__ double sred[5][8], tot[5];
   __shared__ uint32_t s_last;
   pdl_prologue();
   const int64_t b = blockIdx.z;
@@ -283,47 +284,36 @@ __global__ void __launch_bounds__(kThreads, 2) simt_kernel(const SimtArgs a) {
     }
   }
   if (PROBE) {
-    double v[5] = {fbe, fmx, fd2, fr2, fn2};
-    auto block_reduce = [&]() {            // of v over the block; the result in thread 0
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-        for (int i = 0; i < 5; ++i) {
-          const double y = __shfl_xor_sync(0xffffffffu, v[i], o);
-          v[i] = i == 1 ? fmax(v[i], y) : v[i] + y;
-        }
-      }
-      const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-      if (lane == 0)
-        for (int i = 0; i < 5; ++i) sred[i][w] = v[i];
-      __syncthreads();
-      if (threadIdx.x == 0)
-        for (int w2 = 1; w2 < kThreads / 32; ++w2)
-          for (int i = 0; i < 5; ++i) v[i] = i == 1 ? fmax(v[i], sred[i][w2]) : v[i] + sred[i][w2];
-    };
-    block_reduce();
+    double v[4] = {fbe, fd2, fr2, fn2};
+    // field of the record that this thread and its seven neighbours hold: the sums around the maximum
+    const int held = threadIdx.x >> 3, field = held == 0 ? 0 : held == 4 ? 1 : held + 1;
+    const bool writer = (threadIdx.x & 7) == 0 && held < 5;
+    double x = block_record<4>(v, fmx, sred);
     const int64_t n_blocks = (int64_t)gridDim.x * gridDim.y * gridDim.z;
+    const int64_t blk = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    if (writer) __stcg(a.partials + blk * kPartialDoubles + field, x);
+    __syncthreads();
     if (threadIdx.x == 0) {
-      const int64_t blk = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-      for (int i = 0; i < 5; ++i) __stcg(a.partials + blk * kPartialDoubles + i, v[i]);
-      __threadfence();
+      __threadfence();                     // after the barrier: covers what the others have written
       s_last = atomicAdd(a.done_counter, 1u) == (uint32_t)(n_blocks - 1) ? 1u : 0u;
     }
     __syncthreads();
     if (s_last) {                          // the last block adds all records up, in a fixed order
       __threadfence();
-#pragma unroll
-      for (int i = 0; i < 5; ++i) v[i] = 0.0;
+      v[0] = v[1] = v[2] = v[3] = 0.0;
+      float mx = 0.f;
       for (int64_t k = threadIdx.x; k < n_blocks; k += kThreads) {
         const double* rec = a.partials + k * kPartialDoubles;
-        v[0] += __ldcg(rec); v[1] = fmax(v[1], __ldcg(rec + 1)); v[2] += __ldcg(rec + 2);
-        v[3] += __ldcg(rec + 3); v[4] += __ldcg(rec + 4);
+        v[0] += __ldcg(rec); mx = fmaxf(mx, (float)__ldcg(rec + 1)); v[1] += __ldcg(rec + 2);
+        v[2] += __ldcg(rec + 3); v[3] += __ldcg(rec + 4);
       }
       const int not_finite = __syncthreads_or(a.prepare_flags && threadIdx.x < kPrepareFlagWords && __ldcg(a.prepare_flags + threadIdx.x));
-      block_reduce();
+      x = block_record<4>(v, mx, sred);
+      if (writer) tot[field] = x;
+      __syncthreads();
       if (threadIdx.x == 0) {                // (the record may be in host memory: stores only, every field once)
-        a.result->sum_be = v[0]; a.result->max_be = v[1]; a.result->sum_diff2 = v[2];
-        a.result->sum_ref2 = v[3]; a.result->sum_den2 = v[4];
+        a.result->sum_be = tot[0]; a.result->max_be = tot[1]; a.result->sum_diff2 = tot[2];
+        a.result->sum_ref2 = tot[3]; a.result->sum_den2 = tot[4];
         a.result->count = a.count;
         a.result->device_error = *reinterpret_cast<volatile uint32_t*>(a.err_word) | (not_finite ? QM_DEVERR_NONFINITE : 0u);
         a.result->reserved = 0;

@@ -1,22 +1,15 @@
 // Eq. 3 on materialised arrays, and the deterministic final reduction shared with the fused
 // probe kernels.
 #include "qm_internal.h"
+#include "reduce.cuh"
 
 namespace qm {
 namespace {
 
 constexpr int kThreads = 256;
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-__device__ __forceinline__ double warp_maxd(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
+// where sum i (0 .. 3: BE, diff^2, C^2, D^2) and the maximum (4) lie in a record
+__device__ __forceinline__ int record_field(int i) { return i == 0 ? 0 : i == 4 ? 1 : i + 1; }
 
 // Eq. 3 sums of a short run of elements in fp32, folded into fp64 by the caller.
 struct Run {
@@ -37,13 +30,14 @@ __global__ void __launch_bounds__(kThreads)
 metric_partials_kernel(const float* __restrict__ ref, const float* __restrict__ q,
                        const float* __restrict__ den, int64_t count, double* __restrict__ partials) {
   pdl_prologue();
-  __shared__ double s[5][kThreads / 32];
+  __shared__ double s[5][8];
   const int64_t per_block = ((count + gridDim.x - 1) / gridDim.x + 3) & ~(int64_t)3;
   const int64_t i0 = (int64_t)blockIdx.x * per_block;
   const int64_t i1 = min(count, i0 + per_block);
-  double sbe = 0, mbe = 0, sd2 = 0, sr2 = 0, sn2 = 0;
+  double sbe = 0, sd2 = 0, sr2 = 0, sn2 = 0;
+  float mbe = 0;
   // fp32 inside a run of eight, fp64 across runs
-  auto fold = [&](const Run& f) { sbe += f.be; mbe = fmax(mbe, (double)f.mx); sd2 += f.d2; sr2 += f.r2; sn2 += f.n2; };
+  auto fold = [&](const Run& f) { sbe += f.be; mbe = fmaxf(mbe, f.mx); sd2 += f.d2; sr2 += f.r2; sn2 += f.n2; };
   int64_t base = i0;
   if (VEC) {
     for (; base + kThreads * 8 <= i1; base += kThreads * 8) {
@@ -73,19 +67,10 @@ metric_partials_kernel(const float* __restrict__ ref, const float* __restrict__ 
     }
     fold(f);
   }
-  sbe = warp_sum(sbe); sd2 = warp_sum(sd2); sr2 = warp_sum(sr2); sn2 = warp_sum(sn2);
-  mbe = warp_maxd(mbe);
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0) { s[0][w] = sbe; s[1][w] = mbe; s[2][w] = sd2; s[3][w] = sr2; s[4][w] = sn2; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0, m = 0, b = 0, c = 0, d = 0;
-    for (int i = 0; i < kThreads / 32; ++i) {
-      a += s[0][i]; m = fmax(m, s[1][i]); b += s[2][i]; c += s[3][i]; d += s[4][i];
-    }
-    double* o = partials + (int64_t)blockIdx.x * kPartialDoubles;
-    o[0] = a; o[1] = m; o[2] = b; o[3] = c; o[4] = d;
-  }
+  const double v[4] = {sbe, sd2, sr2, sn2};
+  const double x = block_record<4>(v, mbe, s);
+  const int held = threadIdx.x >> 3;
+  if ((threadIdx.x & 7) == 0 && held < 5) partials[(int64_t)blockIdx.x * kPartialDoubles + record_field(held)] = x;
 }
 
 // One block; thread t sums records t, t+256, ... in order, then a fixed order over lanes and warps.
@@ -93,28 +78,21 @@ __global__ void __launch_bounds__(kThreads)
 metric_finalize_kernel(const double* __restrict__ partials, int n, uint64_t count,
                        const uint32_t* __restrict__ err_word, qm_metric_result* __restrict__ out) {
   pdl_prologue();
-  __shared__ double s[5][kThreads / 32];
-  double v[5] = {0, 0, 0, 0, 0};
+  __shared__ double s[5][8];
+  __shared__ double tot[5];
+  double v[4] = {0, 0, 0, 0};
+  float mx = 0.f;
   for (int i = threadIdx.x; i < n; i += kThreads) {
     const double* p = partials + (int64_t)i * kPartialDoubles;
-    v[0] += p[0]; v[1] = fmax(v[1], p[1]); v[2] += p[2]; v[3] += p[3]; v[4] += p[4];
+    v[0] += p[0]; mx = fmaxf(mx, (float)p[1]); v[1] += p[2]; v[2] += p[3]; v[3] += p[4];
   }
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    v[i] = i == 1 ? warp_maxd(v[i]) : warp_sum(v[i]);
-    if (lane == 0) s[i][w] = v[i];
-  }
-  __syncthreads();
-  if (threadIdx.x < 5) {
-    double x = s[threadIdx.x][0];
-    for (int k = 1; k < kThreads / 32; ++k) x = threadIdx.x == 1 ? fmax(x, s[threadIdx.x][k]) : x + s[threadIdx.x][k];
-    s[threadIdx.x][0] = x;
-  }
+  const double x = block_record<4>(v, mx, s);
+  const int held = threadIdx.x >> 3;
+  if ((threadIdx.x & 7) == 0 && held < 5) tot[record_field(held)] = x;
   __syncthreads();
   if (threadIdx.x == 0) {                    // (the record may be in host memory: stores only, every field once)
-    out->sum_be = s[0][0]; out->max_be = s[1][0]; out->sum_diff2 = s[2][0];
-    out->sum_ref2 = s[3][0]; out->sum_den2 = s[4][0];
+    out->sum_be = tot[0]; out->max_be = tot[1]; out->sum_diff2 = tot[2];
+    out->sum_ref2 = tot[3]; out->sum_den2 = tot[4];
     out->count = count;
     out->device_error = err_word ? *err_word : 0u;
     out->reserved = 0;

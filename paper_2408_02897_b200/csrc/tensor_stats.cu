@@ -5,6 +5,7 @@
 // flight per thread, fp32 arithmetic per element, fp32 sums over the 32 elements of a batch of
 // loads, fp64 from there on, one record per block and a fixed-order sum by the last block.
 #include "quant_device.cuh"
+#include "reduce.cuh"
 
 namespace qm {
 namespace {
@@ -48,9 +49,6 @@ __device__ __forceinline__ void decode2(uint32_t two_codes, float& a, float& b) 
 struct Acc {
   double d[kRec];
 };
-
-// which entries of a record combine by max instead of sum
-template <int KIND> __device__ __forceinline__ bool is_max(int i) { return KIND == kStats ? i == 4 : i == 9; }
 
 // Per-thread sums of one batch of up to four groups of 8 elements: fp32 inside the batch.
 template <int KIND, int FMT>
@@ -268,64 +266,41 @@ struct Batch {
 template <int KIND>
 __device__ __forceinline__ void finish_pass(Acc& acc, double* __restrict__ partials, uint32_t* __restrict__ counter,
                                             void* __restrict__ result, uint64_t count) {
-  // block record
-  __shared__ double red[kRec][kThreads / 32];
+  // sums first, the maximum (a float that was widened) behind them
+  constexpr int N = KIND == kStats ? 4 : 9;
+  static_assert(N + 1 <= kRec, "a record");
+  __shared__ double red[N + 1][8];
+  __shared__ double tot[N + 1];
   __shared__ uint32_t is_last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double v[N];
 #pragma unroll
-  for (int i = 0; i < kRec; ++i) {
-    double x = acc.d[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double y = __shfl_xor_sync(0xffffffffu, x, o);
-      x = is_max<KIND>(i) ? fmax(x, y) : x + y;
-    }
-    if (lane == 0) red[i][warp] = x;
-  }
+  for (int i = 0; i < N; ++i) v[i] = acc.d[i];
+  const int held = threadIdx.x >> 3;                         // of the record, by this thread and its seven neighbours
+  const bool writer = (threadIdx.x & 7) == 0 && held <= N;
+  double x = block_record<N>(v, (float)acc.d[N], red);
+  if (writer) __stcg(partials + (int64_t)blockIdx.x * kRec + held, x);
   __syncthreads();
   if (threadIdx.x == 0) {
-    double* rec = partials + (int64_t)blockIdx.x * kRec;
-    for (int i = 0; i < kRec; ++i) {
-      double x = red[i][0];
-      for (int w = 1; w < kThreads / 32; ++w) x = is_max<KIND>(i) ? fmax(x, red[i][w]) : x + red[i][w];
-      __stcg(rec + i, x);
-    }
-    __threadfence();
+    __threadfence();                                         // after the barrier: covers what the others have written
     is_last = atomicAdd(counter, 1u) == gridDim.x - 1 ? 1u : 0u;
   }
   __syncthreads();
   if (!is_last) return;
-  // last block: every record is visible.  Thread t adds records t, t + 256, ... (all 256 threads, so
-  // that the loads of this last step run side by side), then warps and block combine in a fixed order.
+  // last block: every record is visible.  Thread t adds records t, t + 256, ...
   __threadfence();
-  double tot[kRec];
+  float mx = 0.f;
 #pragma unroll
-  for (int i = 0; i < kRec; ++i) tot[i] = 0.0;
+  for (int i = 0; i < N; ++i) v[i] = 0.0;
   for (int b = threadIdx.x; b < (int)gridDim.x; b += kThreads) {
     const double* rec = partials + (int64_t)b * kRec;
 #pragma unroll
-    for (int i = 0; i < kRec; ++i) {
-      const double y = __ldcg(rec + i);
-      tot[i] = is_max<KIND>(i) ? fmax(tot[i], y) : tot[i] + y;
-    }
+    for (int i = 0; i < N; ++i) v[i] += __ldcg(rec + i);
+    mx = fmaxf(mx, (float)__ldcg(rec + N));
   }
-#pragma unroll
-  for (int i = 0; i < kRec; ++i) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double y = __shfl_xor_sync(0xffffffffu, tot[i], o);
-      tot[i] = is_max<KIND>(i) ? fmax(tot[i], y) : tot[i] + y;
-    }
-    if (lane == 0) red[i][warp] = tot[i];
-  }
+  x = block_record<N>(v, mx, red);
+  if (writer) tot[held] = x;
   __syncthreads();
   if (threadIdx.x != 0) return;
-#pragma unroll
-  for (int i = 0; i < kRec; ++i) {
-    double x = red[i][0];
-    for (int w = 1; w < kThreads / 32; ++w) x = is_max<KIND>(i) ? fmax(x, red[i][w]) : x + red[i][w];
-    tot[i] = x;
-  }
   // (the record may be in host memory: stores only, every field once)
   if (KIND == kStats) {
     qm_tensor_stats_result* r = static_cast<qm_tensor_stats_result*>(result);
