@@ -152,6 +152,16 @@ qm_status launch_metric_finalize(const double* partials, int n, uint64_t count,
 constexpr int kClearMax = 32;
 struct ClearList { int n; void* ptr[kClearMax]; uint32_t words[kClearMax]; };
 qm_status launch_clear_many(const ClearList& list, cudaStream_t s);
+// Zeroes one region.  (Behind a memset the next kernel cannot start early, behind this one it can: see pdl_prologue.)
+inline qm_status clear_words(void* p, size_t words, cudaStream_t s) {
+  if (words > 0xffffffffull) {
+    QM_CUDA_OK(cudaMemsetAsync(p, 0, 4 * words, s));
+    return QM_OK;
+  }
+  ClearList l{};
+  l.n = 1; l.ptr[0] = p; l.words[0] = (uint32_t)words;
+  return launch_clear_many(l, s);
+}
 
 // ---- CUDA-core GEMMs (gemm_simt.cu) ---------------------------------------
 struct GemmShape { int64_t M, N, K, batch; };
