@@ -322,20 +322,27 @@ __global__ void __launch_bounds__(kThreads, 2) simt_kernel(const SimtArgs a) {
   }
 }
 
-// The largest tile that still gives every SM a block; below that, the smallest one.  Measured, the probe of
-// 128 x 256 x 256 (whole call): 8 blocks of 64 x 64, without a split and with scalar loads, 89 us (this kernel alone
-// 90); 64 blocks of 16 x 32, the contraction in eight parts, 24.6 us.
+// The shape whose busiest SM is through first: the blocks there, times what a block takes (fitted: a 32 x 32 block 1.3 times its share of
+// a 64 x 64 one, a 16 x 32 block 1.75 times), over the rate at which one block (0.62 of the issue slots) or several (0.85) issue.
+// What this is for: a few blocks more than the GPU has SMs double the time.  Whole probes of 700 x 400 x 368: 154 blocks of 32 x 64 53.7 us, 286 of 32 x 32 37.2; 1024^3 64 x 64 205, 32 x
+// 32 232; 400 x 400 x 300 INT8 32 x 32 28.4, 16 x 32 35.8; 128 x 256 x 256 64 blocks of 16 x 32.
 constexpr int kShapes[4][2] = {{64, 64}, {32, 64}, {32, 32}, {16, 32}};
 dim3 grid_of(GemmShape g, int shape) {
   const int tm = kShapes[shape][0], tn = kShapes[shape][1];
   return dim3((unsigned)((g.N + tn - 1) / tn), (unsigned)((g.M + tm - 1) / tm), (unsigned)g.batch);
 }
 int shape_of(GemmShape g) {
-  for (int i = 0; i < 3; ++i) {
-    const int64_t n = ((g.M + kShapes[i][0] - 1) / kShapes[i][0]) * ((g.N + kShapes[i][1] - 1) / kShapes[i][1]) * g.batch;
-    if (n >= sm_count()) return i;
+  constexpr double kBlockCost[4] = {4096.0, 2212.0, 1331.0, 900.0};
+  int best = 0;
+  double least = 0.0;
+  for (int i = 0; i < 4; ++i) {
+    const int64_t tm = kShapes[i][0], tn = kShapes[i][1], rows = (g.M + tm - 1) / tm;
+    if (i > 0 && rows > 65535) break;                 // (the limit of the grid holds for the largest shape only)
+    const int64_t per_sm = (rows * ((g.N + tn - 1) / tn) * g.batch + sm_count() - 1) / sm_count();
+    const double cost = (double)per_sm * kBlockCost[i] / (per_sm == 1 ? 0.62 : 0.85);
+    if (i == 0 || cost < least) { best = i; least = cost; }
   }
-  return 3;
+  return best;
 }
 
 template <bool IS_INT, bool PROBE, int TM, int TN>

@@ -43,3 +43,19 @@ def test_fp32_probe_against_the_oracle(M, N, K, batch, cl, cr, fmt, gran):
     assert abs(rec["max_be"] - want["max_be"]) <= 1e-5
     for k in ("sum_diff2", "sum_ref2", "sum_den2"):
         assert abs(rec[k] - want[k]) <= 2e-5 * want["sum_den2" if n < 100 else k], k
+
+
+# extents at which the tile shape changes: just over one block for an SM in one shape, and what is taken instead
+@pytest.mark.parametrize("M,N,K", [(700, 400, 68), (704, 448, 36), (350, 350, 40), (1030, 1030, 20), (17, 33, 300), (4000, 30, 24)])
+@pytest.mark.parametrize("fmt,gran", [("e4m3", "tensor"), ("int8", "channel")])
+def test_tile_shapes_against_the_oracle(M, N, K, fmt, gran):
+    rng = workloads._rng(M + N)
+    L, R = workloads.normal(rng, (M, K), 1.0, torch.float32), workloads.normal(rng, (N, K), 0.05, torch.float32)
+    pad = lambda t: torch.nn.functional.pad(t, (0, -t.shape[1] % 8)).cuda()[:, :t.shape[1]]
+    Ld, Rd = pad(L), pad(R)
+    got = qm.qm_probe_layer(qm.operand_of(Ld, -1), qm.operand_of(Rd, -1), fmt, fmt, gran, gran, "fp32").record()
+    want = oracle.probe(L.numpy(), R.T.numpy(), fmt, fmt, gran, gran)
+    # fp32 sums of up to 300 terms in parts: outputs within 1e-5 of their magnitude scale
+    assert got["count"] == want["count"] and abs(got["max_be"] - want["max_be"]) <= 2e-5
+    for k in ("sum_be", "sum_diff2", "sum_ref2", "sum_den2"):
+        assert abs(got[k] - want[k]) <= 2e-5 * want[k], k
