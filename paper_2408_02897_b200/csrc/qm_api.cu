@@ -407,7 +407,7 @@ static qm_status probe_phases(const qm_operand* Lo, const qm_operand* Ro, const 
   const StochasticDraw* dl_draw = (cfg->round & QM_ROUND_STOCHASTIC_L) ? &draw_l : nullptr;
   const StochasticDraw* dr_draw = (cfg->round & QM_ROUND_STOCHASTIC_R) ? &draw_r : nullptr;
   const bool cl_mn = w.tc && codes_mn(L, dl_draw != nullptr), cr_mn = w.tc && codes_mn(R, dr_draw != nullptr);
-  // operands of modest size: both in two launches, the first of which clears the control words
+  // operands of modest size: both in two launches, or one, the first of which clears the control words
   auto grouped = [](const View& v, int gran, int groups) { return gran == QM_GRAN_CHANNEL && groups > 0 && groups < v.batch; };
   const bool pair = (phases & kPrepare) == kPrepare && !clear_later && !grouped(L, cfg->gran_l, cfg->batch_groups_l) &&
                     !grouped(R, cfg->gran_r, cfg->batch_groups_r) &&
