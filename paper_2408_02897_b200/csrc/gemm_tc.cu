@@ -114,8 +114,6 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() { cluster_arrive(); cluster_wait(); }
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
@@ -492,7 +490,6 @@ tc_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_constant__ CUt
   }
   tc_fence_before();
   __syncthreads();
-  __syncwarp();
   cluster_sync();          // the peer's barriers and tensor memory exist before anyone uses them
   pdl_prologue();          // everything above overlapped the tail of the previous kernel
   tc_fence_after();
@@ -815,7 +812,6 @@ tc_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_constant__ CUt
   // barriers or write its tensor memory.
   tc_fence_before();
   __syncthreads();
-  __syncwarp();
   cluster_sync();
   if (warp == 1) {
     __syncwarp();
@@ -889,7 +885,6 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   }
   tc_fence_before();
   __syncthreads();
-  __syncwarp();
   cluster_sync();
   pdl_prologue();
   tc_fence_after();
@@ -1013,7 +1008,6 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 
   tc_fence_before();
   __syncthreads();
-  __syncwarp();
   cluster_sync();
   if (warp == 1) {
     __syncwarp();
@@ -1543,7 +1537,6 @@ __device__ __forceinline__ void probe_exit(Sh* sh, uint64_t wait_limit_ns, int w
     __syncwarp();
   }
   __syncthreads();
-  __syncwarp();
   cluster_sync();
   if (warp == 1) {
     __syncwarp();
@@ -1608,12 +1601,10 @@ tc_group_kernel(const __grid_constant__ Table tab) {
   if (warp == 2) fill_walk(sh, tab, lane, pair, num_pairs);
   tc_fence_before();
   __syncthreads();
-  __syncwarp();
   cluster_arrive();
   tc_fence_after();
   const uint32_t tmem_base = sh->tmem_base;
   auto begin = [&]() {
-    __syncwarp();
     cluster_wait();        // the peer's barriers and tensor memory exist before anyone uses them
     pdl_prologue();        // everything above overlapped the tail of the previous kernel
     tc_fence_after();
@@ -2237,12 +2228,10 @@ tc_side_kernel(const __grid_constant__ Table tab) {
   if (warp == 2) fill_walk(sh, tab, lane, pair, num_pairs);
   tc_fence_before();
   __syncthreads();
-  __syncwarp();
   cluster_arrive();
   tc_fence_after();
   const uint32_t tmem_base = sh->tmem_base;
   auto begin = [&]() {
-    __syncwarp();
     cluster_wait();        // the peer's barriers and tensor memory exist before anyone uses them
     pdl_prologue();        // everything above overlapped the tail of the previous kernel
     tc_fence_after();

@@ -1649,8 +1649,6 @@ __global__ void __launch_bounds__(kThreads) quantize_many_kernel(const __grid_co
 // Non-finite maxima are flagged in a byte for each block, always written: nobody could clear a common word ahead of
 // all blocks.  They lie in the control block, which the products' last block reads.
 constexpr int kOnceBlocks = 8;
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // v into word `at` of the same array in block `rank` of the cluster
 __device__ __forceinline__ void cluster_store(uint32_t* at, uint32_t rank, uint32_t v) {
   uint32_t to;

@@ -82,9 +82,12 @@ def test_non_finite_operands_are_flagged(gran, where, cd):
 
 
 # The one-launch form: operands of 512 KB and just above, strips of 64 columns whole and ragged with fewer rows than
-# blocks of a cluster, contractions up to 4096 and above, as many blocks as there are flags and more.
+# blocks of a cluster, contractions up to 4096 and above.  Under channel scales 960 x 960 x 32 has a block to each of the 240
+# flags and 968 x 960 x 32 more than there are; 3 x 65 x 16 and 130 x 65 x 16 launch 24 and 40 blocks, so that the first block's
+# clearing of the unused flags splits a warp right ahead of a cluster's barrier.
 @pytest.mark.parametrize("M,N,K,batch", [(512, 511, 512, 1), (512, 513, 512, 1), (65, 3, 16, 1), (3, 129, 4096, 1), (3, 129, 4112, 1),
-                                         (960, 128, 32, 1), (968, 960, 32, 1), (70, 40, 112, 4)])
+                                         (960, 128, 32, 1), (960, 960, 32, 1), (968, 960, 32, 1),
+                                         (70, 40, 112, 4), (3, 65, 16, 1), (130, 65, 16, 1)])
 @pytest.mark.parametrize("cl,cr", [(-1, -2), (-2, -1)])
 @pytest.mark.parametrize("fmt,gran_l,gran_r", [("e4m3", "tensor", "channel"), ("int8", "channel", "tensor"), ("e5m2", "channel", "channel"),
                                                ("e4m3", "tensor", "tensor")])
