@@ -1902,10 +1902,12 @@ tc_group_kernel(const __grid_constant__ Table tab) {
     int pM = 0, pN = 0;                            // of the unit in hand; below 2^31 (its tensor maps require it)
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
     uint32_t lp_parity = 0;                        // bit b: parity of the next use of 8-bit accumulator b
-    bool dead = false;                             // a wait for an accumulator ran out
+    // A wait for an 8-bit accumulator may run out in some warps and not in others (dead); the walk ends behind the barrier that
+    // tells all of them (ended).  A warp that left by itself, at the end of a unit, would miss barriers that the others wait at.
+    bool dead = false, ended = false;
     begin();
     uint32_t it = 0;
-    for (int pi = 0; pi < tab.n && !dead; ++pi) {
+    for (int pi = 0; pi < tab.n && !ended; ++pi) {
      const UnitInfo tw(sh->walk[pi]);
      const int n_var = tw.n_var, v0 = tw.var_begin;
      for (int j = 0; j < tw.n_tiles; ++j, ++it) {
@@ -1941,7 +1943,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
 
       const bool ok = !dead && w.wait(smem_u32(&sh->rd_full), it & 1);
       // one barrier publishes the scales and makes the give-up decision uniform over the epilogue
-      if (epi_barrier_any(!ok)) { dead = true; break; }
+      if (epi_barrier_any(!ok)) { ended = true; break; }
       tc_fence_after();
       uint32_t rc[64], rd[64];
       tmem_ld32(lane_addr + C::kColRef + cbase, *reinterpret_cast<uint32_t(*)[32]>(&rc[0]));

@@ -124,3 +124,27 @@ def test_either_writer_of_the_magnitudes_gives_up(starved_producer, K, formats, 
     torch.cuda.synchronize()
     for f, r in zip(formats, batch.results()):
         check_against_oracle({**o, "fmt_l": f, "fmt_r": f}, r)
+
+
+# Units in one launch, more tiles than CTA pairs: 100 tiles of four blocks of the operands and two of codes per probe (eight in all),
+# then 100 of two and one (four), so that a pair meets both units.  Starved among the first unit's codes, in the last of them, ahead of the pair's next
+# tile, and in and ahead of the second unit's tiles.  (All tiles have one cost, so a pair has three: two of the first unit and one of the
+# other are 20 blocks, the most there are.)
+@pytest.mark.parametrize("stop_after", [5, 7, 8, 9, 15, 16, 18])
+def test_every_unit_of_a_launch_gives_up(starved_producer, stop_after):
+    ops = [small_op(seed=37, M=2560, N=1280, K=256), small_op(seed=38, M=2560, N=1280, K=128)]
+    formats = ("e4m3", "int8")
+    dev = [(o["L"].cuda(), o["R"].cuda()) for o in ops]
+    batch = qm.ProbeBatch([(qm.operand_of(Ld, o["cl"]), qm.operand_of(Rd, o["cr"]), f, f, "tensor", "tensor")
+                           for o, (Ld, Rd) in zip(ops, dev) for f in formats])
+    starved_producer.qm_debug_stop_producer_after(stop_after)
+    batch.launch()
+    torch.cuda.synchronize()
+    assert all(r.device_error & QM_DEVERR_TIMEOUT for r in batch.results())
+    starved_producer.qm_debug_stop_producer_after(0xffffffff)
+    batch.launch()
+    torch.cuda.synchronize()
+    records = iter(batch.results())
+    for o in ops:
+        for f in formats:
+            check_against_oracle({**o, "fmt_l": f, "fmt_r": f}, next(records))
