@@ -1024,8 +1024,7 @@ tc_gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 // (VARIANTS, up to kMaxVar) one after the other, each over the whole contraction.
 //
 // The host orders the units by descending tile cost and deals the tiles of each to the CTA pairs with the least
-// to do so far (TileDeal), which balances the pairs to within one tile of the cheapest kind; the deal is fixed, so that records
-// are the same from run to run.  The operand maps, scales, shapes and the 8-bit MMA kinds come
+// to do so far (TileDeal); the deal is fixed, so that records are the same from run to run.  The operand maps, scales, shapes and the 8-bit MMA kinds come
 // from a table in the kernel's parameter space.  A pair meets each unit in
 // one run: when the unit changes, the epilogue warps reduce their statistics and write the CTA's
 // records of the probes they leave.
@@ -2883,14 +2882,18 @@ double tile_cycles(bool side, int64_t K, int n_var) {
 }
 
 // Deals the tiles of a launch's units, in the order of descending cost, to the pairs: each unit's to those with the least to do
-// so far, so that the pairs end within a tile of the cheapest kind of one another.  (Dealt in rounds of a tile for each pair, the
+// so far.  Where the cheap units have tiles enough to fill what the dear ones leave uneven, the pairs end within a tile of the cheapest
+// kind of one another; else within one of the dearest.  (Dealt in rounds of a tile for each pair, the
 // four products of a BERT-base layer, 96 tiles of K = 3072 and 768 of 768, took 18 units of the cheap tile where 15.6 would
 // do: the launch 176 us, 165 so; a sweep layer's 4.82 ms, 4.58, a BERT-large layer's 2.34, 2.25.)  A pair that has a tile's
 // time less to do than another takes its tiles ahead of the rounds (lead), the remainder comes after them (last), so that pairs
-// are in the same round and share the blocks they read.
+// are in the same round and share the blocks they read.  A pair that goes on to another unit has its records to write and the next
+// unit's words to fetch, about 4000 cycles: of pairs that would end at the same time, those that have the unit already take its
+// rest (two products of 49 and 42 tiles of K = 768 in two formats 32.5 us when they do not, 30.6 so).
 struct TileDeal {
+  static constexpr double kUnitCycles = 4000.0;
   struct Run { int p0, n; double load; int64_t count; };   // neighbouring pairs with the same load: a unit splits one run at most,
-  Run runs[2 * kMaxPairs];                                  // so that a unit costs the host a fraction of a microsecond
+  Run runs[2 * kMaxPairs];                                  // so that a unit costs the host a tenth of a microsecond
   int n_runs = 1, pairs;
   explicit TileDeal(int n) : pairs(n) { runs[0] = Run{0, n, 0.0, 0}; }
   template <typename Key>
@@ -2910,6 +2913,13 @@ struct TileDeal {
   }
   void deal(int64_t tiles, double cost, GroupUnit* u, uint16_t* lead) {
     sort_runs([](const Run& r) { return r.load; });
+    // neighbours that have come to the same load are one run again
+    int last = 0;
+    for (int i = 1; i < n_runs; ++i) {
+      if (runs[i].load == runs[last].load && runs[i].p0 == runs[last].p0 + runs[last].n) runs[last].n += runs[i].n;
+      else runs[++last] = runs[i];
+    }
+    n_runs = last + 1;
     // the level that the work of all these tiles fills the lowest loads up to, and whole tiles below it
     double level = 0.0, below = 0.0;
     for (int i = 0, width = 0; i < n_runs; ++i) {
@@ -2927,7 +2937,8 @@ struct TileDeal {
       left -= r.count * r.n;
     }
     // the rest, less than one for each pair, where it ends earliest
-    sort_runs([cost](const Run& r) { return r.load + cost * r.count; });
+    auto changes = [](const Run& r) { return r.load > 0.0 ? kUnitCycles : 0.0; };      // what a unit costs a pair beside its tiles
+    sort_runs([&](const Run& r) { return r.load + cost * r.count + (r.count == 0 ? changes(r) : 0.0); });
     for (int i = 0; left > 0; i = i + 1 == n_runs ? 0 : i + 1) {
       if (left < runs[i].n) split(i, (int)left);
       ++runs[i].count;
@@ -2959,7 +2970,7 @@ struct TileDeal {
         any_lead = true;
         for (int p = r.p0; p < r.p0 + r.n; ++p) lead[p + 1] = (uint16_t)(more - one_last);
       }
-      r.load += cost * r.count;
+      r.load += cost * r.count + (r.count > 0 ? changes(r) : 0.0);
     }
     if (any_lead)
       for (int p = 0; p < pairs; ++p) lead[p + 1] = (uint16_t)(lead[p + 1] + lead[p]);

@@ -115,3 +115,21 @@ def test_tiles_of_unlike_cost_are_dealt_once_each(fmts):
         for k, name in ((0, "sum_be"), (2, "sum_diff2"), (3, "sum_ref2"), (4, "sum_den2")):
             assert abs(got[name] - alone[name]) <= 1e-12 * abs(alone[name]), (o["name"], name)
             assert abs(rs[:, k].sum() - got[name]) <= 1e-9 * abs(got[name]), (o["name"], name)
+
+
+def test_more_tiles_ahead_of_the_rounds_than_a_table_counts():
+    """One tile of a contraction so long that its pair takes none of the other product's 70 224 tiles: there is no round that all pairs
+    take, and more tiles beside the rounds than the launch's table can count, so they are dealt evenly."""
+    rng = workloads._rng(93)
+    long_l, long_r = workloads.normal(rng, (8, 400000)).cuda(), workloads.normal(rng, (8, 400000), 0.02).cuda()
+    wide_l, wide_r = workloads.normal(rng, (67584, 16)).cuda(), workloads.normal(rng, (34048, 16), 0.02).cuda()
+    probes = [(qm.operand_of(l, -1), qm.operand_of(r, -1), "e4m3", "e4m3", "tensor", "tensor") for l, r in ((long_l, long_r), (wide_l, wide_r))]
+    batch = qm.ProbeBatch(probes)
+    batch.launch()
+    torch.cuda.synchronize()
+    for p, res in zip(probes, batch.results()):
+        got, alone = res.record(), qm.qm_probe_layer(*p).record()
+        assert res.device_error == 0 and got["count"] == alone["count"] and got["max_be"] == alone["max_be"]
+        # sums of up to 2^31 fp64 terms in another order
+        for k in ("sum_be", "sum_diff2", "sum_ref2", "sum_den2"):
+            assert abs(got[k] - alone[k]) <= 1e-11 * abs(alone[k]), k
