@@ -1113,7 +1113,7 @@ struct alignas(16) WalkInfo {
                                                     // j < n_lead, then main0 + j * pairs, the last one `last` unless -1
   int32_t per_b, inner, num_kb, half_n;             // per_b = tiles_m * tiles_n (tiles per batch element);
                                                     // inner = tiles_n: column tiles run fastest, -tiles_m: row tiles do;
-                                                    // half_n: kUnitMnMajor... above its low byte
+                                                    // half_n: kUnitMnMajor... above its low byte, the unit's index above those
   uint32_t b_mul, b_shift, i_mul, i_shift;          // division by per_b and by the absolute value of inner (Divisor)
   int32_t n_var, var_begin, K, last;
 };
@@ -1145,36 +1145,41 @@ struct SharedP {
   float maxima[kMaxVar][kEpiWarps][16];
   double red[3 * kMaxVar + 2][kEpiWarps];
   float dl_tensor[kMaxVar], dr_tensor[kMaxVar];     // per-tensor scales of the unit in hand (1 where per channel)
+  int32_t n_walk;                   // units that give this pair tiles
   WalkInfo walk[UNITS];
   VarInfo var[VARS];
 };
 
 constexpr int kMaxPairs = 80;               // CTA pairs of a launch, at most (148 SMs hold 74)
-struct GroupUnit {
+// (A unit's words are one line of the constant cache, and so are a probe's: every line is a miss of its own at the start of a launch, which
+// takes 600 cycles of a launch of eight units.)
+struct alignas(64) GroupUnit {
   int32_t M, N, K;
   int32_t tiles_m, tiles_n;
   int32_t rounds;             // tiles that every pair takes of it, after those of GroupTable::lead
-  uint32_t last[(kMaxPairs + 31) / 32];   // bit p: pair p takes one more after them
+  int32_t n_lead;             // of all pairs together, those of GroupTable::lead
   int32_t half_n;             // right-operand rows each CTA stages: 64, or 32 for outputs at most 64 wide
-  int32_t m_fastest;          // the tiles of a batch element are walked down the rows first (below)
+  uint32_t last[(kMaxPairs + 31) / 32];   // bit p: pair p takes one more after them
   uint32_t major;             // kUnitMnMajor...: bf16 operands stored with the contraction strided
-  uint32_t b_mul, b_shift, i_mul, i_shift;   // see WalkInfo
-  int32_t var_begin, n_var;
+  uint32_t b_mul, i_mul;      // see WalkInfo
+  uint8_t b_shift, i_shift;
+  uint8_t m_fastest;          // the tiles of a batch element are walked down the rows first (below)
+  int16_t var_begin, n_var;
 };
-struct GroupVar {
+static_assert(sizeof(GroupUnit) == 64, "a line");
+struct alignas(64) GroupVar {
   const float* dl; const float* dr;
   double* partials;           // gridDim.x records
-  qm_metric_result* result;
   double* row_stats;          // optional [batch * M][5] per-row sums
+  qm_metric_result* result;
   uint32_t* err_word;
   const uint32_t* err_also[2];           // further error words to report in the record, or null
-  const uint32_t* prepare_flags;         // flag words of the operands' preparation, or null
-  uint64_t count;             // batch * M * N
-  VarInfo info;
 };
+static_assert(sizeof(GroupVar) == 64, "a line");
 template <int UNITS, int VARS>
 struct GroupTable {
   static constexpr int kUnits = UNITS, kVars = VARS;
+  static_assert(VARS <= 64, "a bit to a probe");
   CUtensorMap unit_maps[UNITS][2];        // L, R
   CUtensorMap var_maps[VARS][2];          // codes of L, codes of R
   int32_t n, n_var;
@@ -1182,8 +1187,12 @@ struct GroupTable {
   uint64_t wait_limit_ns;     // bound of every barrier wait
   uint32_t* done_counter;     // zero on entry; counts finished CTAs
   uint32_t* err0;             // a wait that runs out is reported here and in every record
+  const uint32_t* prepare_flags;          // of a single probe: flag words of the operands' preparation, or null
   GroupUnit u[UNITS];
   GroupVar v[VARS];
+  VarInfo info[VARS];
+  uint64_t count[VARS];                   // batch * M * N
+  uint8_t first[kMaxPairs];               // the first unit that gives a pair tiles
   uint16_t lead[UNITS][kMaxPairs + 1];    // prefix sums over the pairs of the tiles that each takes ahead of the unit's rounds
 };
 // A launch's table has to fit into 32 764 bytes of kernel parameters.  24 units hold the 18 products
@@ -1194,15 +1203,18 @@ static_assert(sizeof(TableBig) <= 32764, "kernel parameters");
 
 // What a unit asks of every role, read once per unit: the same in all lanes, and known to be (the shuffles).  A tile's own
 // code is kept short by this: 512 x 512 x 64 x 256 in one format 95 us with one loop over tiles that looks its unit up, 87 so.
+// The roles go through the units that give their pair tiles and no others: going past the rest took 18 small products 3 us of 31.
+// An epilogue prepares a unit ahead of its tiles and writes its records behind them, in one place each: with the writing in the loop over
+// tiles and once more behind it, 8192 x 4096 x 1024 took 136 us instead of 130 (instructions to fetch, registers to spill).
 struct UnitInfo {
-  int n_tiles, num_kb, half_n, n_var, var_begin, K;
+  int unit, n_tiles, num_kb, half_n, n_var, var_begin, K;
   uint32_t major;
   __device__ __forceinline__ explicit UnitInfo(const WalkInfo& w) {
     constexpr uint32_t all = 0xffffffffu;
     n_tiles = __shfl_sync(all, w.n_tiles, 0);
     num_kb = __shfl_sync(all, w.num_kb, 0);
     const int h = __shfl_sync(all, w.half_n, 0);
-    half_n = h & 255; major = (uint32_t)h >> 8;
+    half_n = h & 255; major = (uint32_t)h >> 8 & 255u; unit = h >> 16;
     n_var = __shfl_sync(all, w.n_var, 0);
     var_begin = __shfl_sync(all, w.var_begin, 0);
     K = __shfl_sync(all, w.K, 0);
@@ -1408,37 +1420,50 @@ __device__ __forceinline__ void eval_variant(uint32_t taddr, const uint32_t (&rc
   }
 }
 
-// The first unit that gives the pair a tile.
+// The operand maps of the pair's first tile into the descriptor cache (one warp).
 template <typename Table>
-__device__ __forceinline__ int first_unit(const Table& tab, int pair) {
-  int pi = 0;
-  while (pi + 1 < tab.n && tab.u[pi].rounds == 0 && tab.lead[pi][pair + 1] == tab.lead[pi][pair] && !(tab.u[pi].last[pair >> 5] >> (pair & 31) & 1u)) ++pi;
-  return pi;
+__device__ __forceinline__ void prefetch_maps(const Table& tab, int lane, int pair) {
+  if (lane < 4) {
+    const int pi = Table::kUnits > 1 ? tab.first[pair] : 0;
+    const CUtensorMap* m = lane < 2 ? &tab.unit_maps[pi][lane] : &tab.var_maps[tab.u[pi].var_begin][lane - 2];
+    asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
+  }
 }
-// The walk of this pair and the variant table of a launch into shared memory (one warp).
+// The walk of this pair (the units that give it tiles, in order) and the variant table of a launch into shared memory (one warp).
 template <typename Sh, typename Table>
 __device__ __forceinline__ void fill_walk(Sh* sh, const Table& tab, int lane, int pair, int num_pairs) {
-  for (int i = lane; i < tab.n; i += 32) {
-    const GroupUnit& u = tab.u[i];
-    WalkInfo wi;
-    wi.lead0 = tab.lead[i][pair];
-    wi.n_lead = tab.lead[i][pair + 1] - wi.lead0;
-    wi.n_tiles = wi.n_lead + u.rounds;
-    wi.main0 = tab.lead[i][num_pairs] + pair - wi.n_lead * num_pairs;
+  static_assert(Table::kUnits <= 32, "a lane to a unit");
+  WalkInfo wi;
+  wi.n_tiles = 0;
+  const GroupUnit& u = tab.u[lane < tab.n ? lane : 0];
+  if (lane < tab.n) {
+    const int32_t rounds = u.rounds, n_lead = u.n_lead;
+    const uint32_t last0 = u.last[0], last1 = u.last[1], last2 = u.last[2];
+    const int32_t tiles_m = u.tiles_m, tiles_n = u.tiles_n;
+    wi.K = u.K; wi.b_mul = u.b_mul; wi.i_mul = u.i_mul; wi.b_shift = u.b_shift; wi.i_shift = u.i_shift;
+    wi.n_var = u.n_var; wi.var_begin = u.var_begin;
+    wi.half_n = u.half_n | (int32_t)(u.major << 8) | lane << 16;
+    wi.inner = u.m_fastest ? -tiles_m : tiles_n;
+    wi.per_b = tiles_m * tiles_n;
+    wi.num_kb = (wi.K + kBlockK - 1) / kBlockK;
+    wi.lead0 = wi.n_lead = 0;
+    if (n_lead > 0) {                                // (rows of their own in the table, seldom needed)
+      wi.lead0 = tab.lead[lane][pair];
+      wi.n_lead = tab.lead[lane][pair + 1] - wi.lead0;
+    }
+    wi.n_tiles = wi.n_lead + rounds;
+    wi.main0 = n_lead + pair - wi.n_lead * num_pairs;
+    const uint32_t below = (1u << (pair & 31)) - 1u, word = pair < 32 ? last0 : pair < 64 ? last1 : last2;
     wi.last = -1;
-    if (u.last[pair >> 5] >> (pair & 31) & 1u) {
-      wi.last = tab.lead[i][num_pairs] + u.rounds * num_pairs + __popc(u.last[pair >> 5] & ((1u << (pair & 31)) - 1u));
-      for (int k = 0; k < pair >> 5; ++k) wi.last += __popc(u.last[k]);
+    if (word >> (pair & 31) & 1u) {
+      wi.last = n_lead + rounds * num_pairs + __popc(word & below) + (pair >= 32 ? __popc(last0) : 0) + (pair >= 64 ? __popc(last1) : 0);
       ++wi.n_tiles;
     }
-    wi.per_b = u.tiles_m * u.tiles_n;
-    wi.inner = u.m_fastest ? -u.tiles_m : u.tiles_n;
-    wi.num_kb = (u.K + kBlockK - 1) / kBlockK;
-    wi.half_n = u.half_n | (int32_t)(u.major << 8); wi.n_var = u.n_var; wi.var_begin = u.var_begin; wi.K = u.K;
-    wi.b_mul = u.b_mul; wi.b_shift = u.b_shift; wi.i_mul = u.i_mul; wi.i_shift = u.i_shift;
-    sh->walk[i] = wi;
   }
-  for (int i = lane; i < tab.n_var; i += 32) sh->var[i] = tab.v[i].info;
+  const uint32_t mine = __ballot_sync(0xffffffffu, wi.n_tiles > 0);
+  if (wi.n_tiles > 0) sh->walk[__popc(mine & ((1u << lane) - 1u))] = wi;
+  if (lane == 0) sh->n_walk = __popc(mine);
+  for (int i = lane; i < tab.n_var; i += 32) sh->var[i] = tab.info[i];
 }
 
 // Sums of four values over the warp, six exchanges instead of twenty: lanes 8 k .. 8 k + 7 return the sum of v[k].
@@ -1468,11 +1493,11 @@ __device__ __forceinline__ void write_results(const Table& tab, int ew, int lane
     const uint32_t* word = lane == 0 ? a.err_word : lane == 1 ? a.err_also[0] : lane == 2 ? a.err_also[1] : lane == 3 ? tab.err0 : nullptr;
     uint32_t flags = word ? *reinterpret_cast<const volatile uint32_t*>(word) : 0u;
     if (lane == 3) flags &= QM_DEVERR_TIMEOUT;
-    if (a.prepare_flags) {
+    if (Table::kUnits == 1 && tab.prepare_flags) {
       uint32_t any = 0;
 #pragma unroll
       for (int i = 0; i < kPrepareFlagWords; i += 32)
-        if (i + lane < kPrepareFlagWords) any |= __ldcg(a.prepare_flags + i + lane);
+        if (i + lane < kPrepareFlagWords) any |= __ldcg(tab.prepare_flags + i + lane);
       if (any) flags |= QM_DEVERR_NONFINITE;
     }
     double s4[4] = {0, 0, 0, 0};
@@ -1497,7 +1522,7 @@ __device__ __forceinline__ void write_results(const Table& tab, int ew, int lane
     flags = __reduce_or_sync(0xffffffffu, flags);
     if (lane == 0) {                         // (the record may be in host memory: stores only, every field once)
       a.result->sum_be = x; a.result->max_be = (double)mx;
-      a.result->count = a.count; a.result->device_error = flags; a.result->reserved = 0;
+      a.result->count = tab.count[vi]; a.result->device_error = flags; a.result->reserved = 0;
     } else if (lane == 8) {
       a.result->sum_diff2 = x;
     } else if (lane == 16) {
@@ -1565,14 +1590,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
   const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
   const Waiter w{&sh->abort_flag, tab.err0, tab.wait_limit_ns};
 
-  if (warp == 0) {
-    // fetch the operand maps of this pair's first tile into the descriptor cache
-    if (lane < 4) {
-      const int pi = first_unit(tab, pair);
-      const CUtensorMap* m = lane < 2 ? &tab.unit_maps[pi][lane] : &tab.var_maps[tab.u[pi].var_begin][lane - 2];
-      asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
-    }
-  }
+  if (warp == 0) prefetch_maps(tab, lane, pair);
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&sh->full[s]), 1);
@@ -1633,10 +1651,11 @@ tc_group_kernel(const __grid_constant__ Table tab) {
           sh->issued = ++g;
           ring.next();
         };
-        for (int pi = 0; pi < tab.n && ok; ++pi) {
-          const WalkInfo& wk = sh->walk[pi];
+        for (int k = 0; k < sh->n_walk && ok; ++k) {
+          const WalkInfo& wk = sh->walk[k];
+          const int pi = wk.half_n >> 16;
           const int n_tiles = wk.n_tiles, num_kb = wk.num_kb, half_n = wk.half_n & 255, n_var = wk.n_var, v0 = wk.var_begin;
-          const uint32_t major = (uint32_t)wk.half_n >> 8;
+          const uint32_t major = (uint32_t)wk.half_n >> 8 & 255u;
           const int nb = (wk.K + C::kLpDepth - 1) / C::kLpDepth;
           const uint32_t bytes = kABf16 + (uint32_t)half_n * 128u;
           const bool l_mn = MN && (major & kUnitMnMajorL), r_mn = MN && (major & kUnitMnMajorR);
@@ -1691,8 +1710,8 @@ tc_group_kernel(const __grid_constant__ Table tab) {
       uint32_t lp_uses0 = 0, lp_uses1 = 0;           // variants put into each 8-bit accumulator so far
       bool ok = true;
       uint32_t it = 0;
-      for (int pi = 0; pi < tab.n && ok; ++pi) {
-       const UnitInfo tw(sh->walk[pi]);
+      for (int k = 0; k < sh->n_walk && ok; ++k) {
+       const UnitInfo tw(sh->walk[k]);
        const bool r_mn = MN && (tw.major & kUnitMnMajorR);  // (A comes from tensor memory, contraction-major always)
        const uint32_t idesc_ref = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n) | (r_mn ? kIdescMnMajorB : 0u);
        rd = tile_desc(r_mn, r_mn ? 2u * tw.half_n : 128u, 16u, 16u);
@@ -1746,8 +1765,8 @@ tc_group_kernel(const __grid_constant__ Table tab) {
       const uint32_t ready_leader = map_to_cta(smem_u32(&sh->ready[0]), 0);
       Ring<kStages> ring;
       bool ok = true;
-      for (int pi = 0; pi < tab.n && ok; ++pi)
-       for (UnitInfo tw(sh->walk[pi]); tw.n_tiles > 0 && ok; --tw.n_tiles) {
+      for (int k = 0; k < sh->n_walk && ok; ++k)
+       for (UnitInfo tw(sh->walk[k]); tw.n_tiles > 0 && ok; --tw.n_tiles) {
         for (int kb = 0; kb < tw.num_kb && ok; ++kb) {
           ok = w.wait_warp(smem_u32(&sh->full[ring.s]), ring.parity);
           if (!ok) break;
@@ -1788,8 +1807,8 @@ tc_group_kernel(const __grid_constant__ Table tab) {
     uint32_t it = 0, abs_uses = 0;                 // completions of abs_free awaited so far
     bool lent = false;                             // the previous tile's variants have used the L columns
     bool ok = true;
-    for (int pi = 0; pi < tab.n && ok; ++pi)
-     for (UnitInfo tw(sh->walk[pi]); tw.n_tiles > 0 && ok; --tw.n_tiles, ++it) {
+    for (int k = 0; k < sh->n_walk && ok; ++k)
+     for (UnitInfo tw(sh->walk[k]); tw.n_tiles > 0 && ok; --tw.n_tiles, ++it) {
       // the L columns are free once the previous tile's denominator is complete and whatever
       // variants it put there have been read
       if (it > 0) ok = w.wait_warp(smem_u32(&sh->rd_full), (it - 1) & 1);
@@ -1868,10 +1887,8 @@ tc_group_kernel(const __grid_constant__ Table tab) {
     const uint32_t rd_empty_leader = map_to_cta(smem_u32(&sh->rd_empty), 0);
     const uint32_t lp_done_leader = map_to_cta(smem_u32(&sh->lp_done[0]), 0);
     double acc_r2 = 0.0, acc_n2 = 0.0;             // of the unit in hand: sum C^2, D^2 of this thread's rows
-    int cur = -1;                                  // the unit in hand
-    // reduce the statistics of unit `pi` over the CTA and write its records (all 256 threads call)
-    auto flush = [&](int pi) {
-      const int nv = sh->walk[pi].n_var, v0 = sh->walk[pi].var_begin;
+    // reduce the statistics of the unit in hand over the CTA and write its records (all 256 threads call)
+    auto flush = [&](int nv, int v0) {
       __syncwarp();                                // lanes 16..31 read below what lanes 0..15 have written to sums[]
       // values 3v, 3v + 1, 3v + 2: sum BE, max BE, sum diff^2 of variant v; the last two: sum C^2, D^2.  Half a warp adds up each
       for (int v = 0; v < nv; ++v) {
@@ -1897,8 +1914,7 @@ tc_group_kernel(const __grid_constant__ Table tab) {
       }
       asm volatile("bar.sync 1, 256;" ::: "memory");       // red[] may be reused
     };
-    uint32_t met = 0;                              // bit pi: this CTA has had tiles of unit pi
-    int pM = 0, pN = 0;                            // of the unit in hand; below 2^31 (its tensor maps require it)
+    uint64_t met = 0;                              // bit v: this CTA has had tiles of probe v's unit
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
     uint32_t lp_parity = 0;                        // bit b: parity of the next use of 8-bit accumulator b
     // A wait for an 8-bit accumulator may run out in some warps and not in others (dead); the walk ends behind the barrier that
@@ -1906,25 +1922,20 @@ tc_group_kernel(const __grid_constant__ Table tab) {
     bool dead = false, ended = false;
     begin();
     uint32_t it = 0;
-    for (int pi = 0; pi < tab.n && !ended; ++pi) {
-     const UnitInfo tw(sh->walk[pi]);
-     const int n_var = tw.n_var, v0 = tw.var_begin;
+    for (int k = 0; k < sh->n_walk && !ended; ++k) {
+     const UnitInfo tw(sh->walk[k]);
+     const int pi = tw.unit, n_var = tw.n_var, v0 = tw.var_begin;
+     met |= ((1ull << n_var) - 1ull) << v0;
+     const int pM = tab.u[pi].M, pN = tab.u[pi].N;  // below 2^31 (its tensor maps require it)
+     for (int v = 0; v < n_var; ++v)
+       if (lane < 16) { sh->sums[v][ew][lane] = make_double2(0.0, 0.0); sh->maxima[v][ew][lane] = 0.f; }
+     if (et < n_var) {                              // read after the barrier below
+       const uint32_t flags = sh->var[v0 + et].flags;
+       sh->dl_tensor[et] = flags & kVarScalePerRow ? 1.f : __ldg(tab.v[v0 + et].dl);
+       sh->dr_tensor[et] = flags & kVarScalePerCol ? 1.f : __ldg(tab.v[v0 + et].dr);
+     }
      for (int j = 0; j < tw.n_tiles; ++j, ++it) {
-      if (pi != cur) {
-        if (cur >= 0) flush(cur);
-        cur = pi;
-        met |= 1u << pi;
-        pM = tab.u[pi].M; pN = tab.u[pi].N;
-        for (int v = 0; v < n_var; ++v)
-          if (lane < 16) { sh->sums[v][ew][lane] = make_double2(0.0, 0.0); sh->maxima[v][ew][lane] = 0.f; }
-        if (et < n_var) {                           // read after the barrier below
-          const GroupVar& gv = tab.v[v0 + et];
-          const uint32_t flags = sh->var[v0 + et].flags;
-          sh->dl_tensor[et] = flags & kVarScalePerRow ? 1.f : __ldg(gv.dl);
-          sh->dr_tensor[et] = flags & kVarScalePerCol ? 1.f : __ldg(gv.dr);
-        }
-      }
-      const TileCoord tc = pair_tile(sh->walk[pi], j, num_pairs);
+      const TileCoord tc = pair_tile(sh->walk[k], j, num_pairs);
       for (int v = 0; v < n_var; ++v) {
         if ((sh->var[v0 + v].flags & kVarScalePerCol) && et < kBlockN) {
           const int col = tc.n_tile * kBlockN + et;
@@ -2047,14 +2058,12 @@ tc_group_kernel(const __grid_constant__ Table tab) {
         }
       }
      }
+     flush(n_var, v0);
     }
-    if (cur >= 0) flush(cur);
     // the records of the probes this CTA never met are zero
-    for (int pi = 0; pi < tab.n; ++pi) {
-      if (met & (1u << pi)) continue;
-      const int v0 = sh->walk[pi].var_begin;
-      if (et < 5 * sh->walk[pi].n_var)
-        __stcg(tab.v[v0 + et / 5].partials + (int64_t)blockIdx.x * kPartialDoubles + et % 5, 0.0);
+    for (int i = et; i < kPartialDoubles * tab.n_var; i += 256) {
+      const int v = i / kPartialDoubles;
+      if (!(met >> v & 1ull)) __stcg(tab.v[v].partials + (int64_t)blockIdx.x * kPartialDoubles + (i - v * kPartialDoubles), 0.0);
     }
     asm volatile("bar.sync 1, 256;" ::: "memory");
     if (et == 0) {
@@ -2118,6 +2127,7 @@ struct SharedS {
   float delta_r[2][kBlockN];
   double red[4][kEpiWarps];
   float red_max[kEpiWarps];
+  int32_t n_walk;                   // units that give this pair tiles
   WalkInfo walk[UNITS];
   VarInfo var[UNITS];               // of unit i: it has one probe
 };
@@ -2199,13 +2209,6 @@ tc_side_kernel(const __grid_constant__ Table tab) {
   const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
   const Waiter w{&sh->abort_flag, tab.err0, tab.wait_limit_ns};
 
-  if (warp == 0) {
-    // fetch the tensor maps of this pair's first tile into the descriptor cache
-    if (lane < 4) {
-      const int pi = first_unit(tab, pair);
-      asm volatile("prefetch.tensormap [%0];" ::"l"(lane < 2 ? &tab.unit_maps[pi][lane] : &tab.var_maps[pi][lane - 2]) : "memory");
-    }
-  }
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&sh->full[s]), 1);
@@ -2247,12 +2250,13 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         Ring<kStages> ring;
         uint32_t g = 0;
         bool ok = true;
-        for (int pi = 0; pi < tab.n && ok; ++pi) {
-          const WalkInfo& wk = sh->walk[pi];
+        for (int k = 0; k < sh->n_walk && ok; ++k) {
+          const WalkInfo& wk = sh->walk[k];
+          const int pi = wk.half_n >> 16;
           const CUtensorMap* const um = tab.unit_maps[pi];
           const CUtensorMap* const vm = tab.var_maps[pi];
           const int n_tiles = wk.n_tiles, num_kb = wk.num_kb, half_n = wk.half_n & 255;
-          const uint32_t flags = sh->var[pi].flags, major = (uint32_t)wk.half_n >> 8;
+          const uint32_t flags = sh->var[pi].flags, major = (uint32_t)wk.half_n >> 8 & 255u;
           const bool l_mn = MN && (major & kUnitMnMajorL), r_mn = MN && (major & kUnitMnMajorR);
           const bool cl_mn = MN && (flags & kVarMnMajorL), cr_mn = MN && (flags & kVarMnMajorR);
           for (int j = 0; j < n_tiles && ok; ++j) {
@@ -2311,8 +2315,9 @@ tc_side_kernel(const __grid_constant__ Table tab) {
       Ring<kStages> ring;                      // of the next block whose 8-bit MMAs are to be issued
       uint32_t g = 0, it = 0;
       bool ok = true;
-      for (int pi = 0; pi < tab.n && ok; ++pi) {
-       const UnitInfo tw(sh->walk[pi]);
+      for (int k = 0; k < sh->n_walk && ok; ++k) {
+       const UnitInfo tw(sh->walk[k]);
+       const int pi = tw.unit;
        const int num_kb = tw.num_kb;
        const uint32_t idesc_lp = __shfl_sync(0xffffffffu, sh->var[pi].idesc, 0);
        const uint32_t flags = __shfl_sync(0xffffffffu, sh->var[pi].flags, 0);
@@ -2367,8 +2372,8 @@ tc_side_kernel(const __grid_constant__ Table tab) {
       const uint32_t ready_leader = map_to_cta(smem_u32(&sh->ready[0]), 0);
       bool ok = true;
       Ring<kStages> ring;
-      for (int pi = 0; pi < tab.n && ok; ++pi)
-       for (UnitInfo tw(sh->walk[pi]); tw.n_tiles > 0 && ok; --tw.n_tiles) {
+      for (int k = 0; k < sh->n_walk && ok; ++k)
+       for (UnitInfo tw(sh->walk[k]); tw.n_tiles > 0 && ok; --tw.n_tiles) {
         for (int kb = 0; kb < tw.num_kb; ++kb) {
           ok = w.wait_warp(smem_u32(&sh->full[ring.s]), ring.parity);
           if (!ok) break;
@@ -2439,8 +2444,8 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         ring.next();
       }
     };
-    for (int pi = 0; pi < tab.n && ok; ++pi)
-      for (UnitInfo tw(sh->walk[pi]); tw.n_tiles > 0 && ok; --tw.n_tiles) {
+    for (int k = 0; k < sh->n_walk && ok; ++k)
+      for (UnitInfo tw(sh->walk[k]); tw.n_tiles > 0 && ok; --tw.n_tiles) {
         if (MN && (tw.major & kUnitMnMajorL)) convert(std::bool_constant<MN>{}, tw); else convert(std::false_type{}, tw);
       }
   } else {
@@ -2457,7 +2462,6 @@ tc_side_kernel(const __grid_constant__ Table tab) {
     const uint32_t tmem_empty_leader = map_to_cta(smem_u32(&sh->tmem_empty), 0);
     double acc[4] = {0, 0, 0, 0};                  // of the unit in hand: sum BE, sum diff^2, C^2, D^2
     float acc_max = 0.f;                           // and max BE
-    int cur = -1;                                  // the unit in hand
     // reduce the statistics of unit `pi` over the CTA and write its record (all 256 threads call)
     auto flush = [&](int pi) {
       const double x = warp_sum4(acc[0], acc[1], acc[2], acc[3], lane);
@@ -2479,29 +2483,20 @@ tc_side_kernel(const __grid_constant__ Table tab) {
       asm volatile("bar.sync 1, 256;" ::: "memory");       // red[] may be reused
     };
     uint32_t met = 0;                              // bit pi: this CTA has had tiles of unit pi
-    // of the unit in hand (reloaded when the unit changes, not per tile)
-    bool per_col = false, pc_l = false, is_i8 = false, narrow = false;
-    float dr_tensor = 1.f, dl_tensor = 0.f;
-    int pM = 0, pN = 0;                            // a probe's M and N are below 2^31 (its tensor maps require it)
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
     begin();
     uint32_t it = 0;
     bool dead = false;                             // a wait ran out
-    for (int pi = 0; pi < tab.n && !dead; ++pi) {
-     const UnitInfo tw(sh->walk[pi]);
+    for (int k = 0; k < sh->n_walk && !dead; ++k) {
+     const UnitInfo tw(sh->walk[k]);
+     const int pi = tw.unit;
+     met |= 1u << pi;
+     const uint32_t flags = sh->var[pi].flags;
+     const bool per_col = flags & kVarScalePerCol, pc_l = flags & kVarScalePerRow, is_i8 = flags & kVarI8, narrow = tw.half_n < 64;
+     const int pM = tab.u[pi].M, pN = tab.u[pi].N;  // below 2^31 (its tensor maps require it)
+     const float dr_tensor = per_col ? 1.f : __ldg(tab.v[pi].dr), dl_tensor = pc_l ? 0.f : __ldg(tab.v[pi].dl);
      for (int j = 0; j < tw.n_tiles; ++j, ++it) {
-      if (pi != cur) {
-        if (cur >= 0) flush(cur);
-        cur = pi;
-        met |= 1u << pi;
-        const GroupVar& gv = tab.v[pi];
-        const uint32_t flags = sh->var[pi].flags;
-        per_col = flags & kVarScalePerCol; pc_l = flags & kVarScalePerRow; is_i8 = flags & kVarI8; narrow = tw.half_n < 64;
-        pM = tab.u[pi].M; pN = tab.u[pi].N;
-        dr_tensor = per_col ? 1.f : __ldg(gv.dr);
-        dl_tensor = pc_l ? 0.f : __ldg(gv.dl);
-      }
-      const TileCoord tc = pair_tile(sh->walk[pi], j, num_pairs);
+      const TileCoord tc = pair_tile(sh->walk[k], j, num_pairs);
       float* dr_s = sh->delta_r[it & 1];
       if (per_col && et < kBlockN) {
         const int col = tc.n_tile * kBlockN + et;
@@ -2577,8 +2572,8 @@ tc_side_kernel(const __grid_constant__ Table tab) {
         if (rows) row_stats_add(rows + ((int64_t)tc.b * pM + row) * 5, st);
       }
      }
+     flush(pi);
     }
-    if (cur >= 0) flush(cur);
     // the records of the probes this CTA never met are zero
     if (et == 0) {
       for (int pi = 0; pi < tab.n; ++pi) {
@@ -2892,10 +2887,12 @@ double tile_cycles(bool side, int64_t K, int n_var) {
 // rest (two products of 49 and 42 tiles of K = 768 in two formats 32.5 us when they do not, 30.6 so).
 struct TileDeal {
   static constexpr double kUnitCycles = 4000.0;
-  struct Run { int p0, n; double load; int64_t count; };   // neighbouring pairs with the same load: a unit splits one run at most,
-  Run runs[2 * kMaxPairs];                                  // so that a unit costs the host a tenth of a microsecond
+  // neighbouring pairs with the same load and first unit (-1: none yet): a unit splits one run at most, so that it costs the host a tenth of a
+  // microsecond
+  struct Run { int p0, n; double load; int64_t count; int first; };
+  Run runs[2 * kMaxPairs];
   int n_runs = 1, pairs;
-  explicit TileDeal(int n) : pairs(n) { runs[0] = Run{0, n, 0.0, 0}; }
+  explicit TileDeal(int n) : pairs(n) { runs[0] = Run{0, n, 0.0, 0, -1}; }
   template <typename Key>
   void sort_runs(Key key) {                                // by insertion: a few runs, nearly in order
     for (int i = 1; i < n_runs; ++i) {
@@ -2908,15 +2905,16 @@ struct TileDeal {
   // the first `n` pairs of run i become a run of their own, before it
   void split(int i, int n) {
     for (int j = n_runs++; j > i + 1; --j) runs[j] = runs[j - 1];
-    runs[i + 1] = Run{runs[i].p0 + n, runs[i].n - n, runs[i].load, runs[i].count};
+    runs[i + 1] = runs[i];
+    runs[i + 1].p0 += n; runs[i + 1].n -= n;
     runs[i].n = n;
   }
-  void deal(int64_t tiles, double cost, GroupUnit* u, uint16_t* lead) {
+  void deal(int unit, int64_t tiles, double cost, GroupUnit* u, uint16_t* lead) {
     sort_runs([](const Run& r) { return r.load; });
     // neighbours that have come to the same load are one run again
     int last = 0;
     for (int i = 1; i < n_runs; ++i) {
-      if (runs[i].load == runs[last].load && runs[i].p0 == runs[last].p0 + runs[last].n) runs[last].n += runs[i].n;
+      if (runs[i].load == runs[last].load && runs[i].first == runs[last].first && runs[i].p0 == runs[last].p0 + runs[last].n) runs[last].n += runs[i].n;
       else runs[++last] = runs[i];
     }
     n_runs = last + 1;
@@ -2971,10 +2969,14 @@ struct TileDeal {
         for (int p = r.p0; p < r.p0 + r.n; ++p) lead[p + 1] = (uint16_t)(more - one_last);
       }
       r.load += cost * r.count + (r.count > 0 ? changes(r) : 0.0);
+      if (r.first < 0 && r.count > 0) r.first = unit;
     }
     if (any_lead)
       for (int p = 0; p < pairs; ++p) lead[p + 1] = (uint16_t)(lead[p + 1] + lead[p]);
-    u->rounds = (int32_t)rounds;
+    u->rounds = (int32_t)rounds; u->n_lead = lead[pairs];
+  }
+  void first_units(uint8_t* first) const {
+    for (int i = 0; i < n_runs; ++i) memset(first + runs[i].p0, std::max(runs[i].first, 0), (size_t)runs[i].n);
   }
 };
 
@@ -2990,6 +2992,7 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, bool
   tab.stop_after_kb = g_stop_after_kb.load();
   tab.done_counter = first.done_counter;
   tab.err0 = first.err_word;
+  tab.prepare_flags = first.prepare_flags;
   int64_t total = 0;
   for (int k = 0; k < n; ++k) total += tile_count(units[k].g);
   const int pairs = (int)std::min<int64_t>(total, max_pairs());
@@ -3013,18 +3016,21 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, bool
     fill_tiles(&ka, g);
     gu.M = (int32_t)g.M; gu.N = (int32_t)g.N; gu.K = (int32_t)g.K;
     gu.tiles_m = ka.tiles_m; gu.tiles_n = ka.tiles_n;
-    pair_loads.deal(ka.num_tiles, tile_cycles(SIDE, g.K, up.n_var), &gu, tab.lead[k]);
+    pair_loads.deal(k, ka.num_tiles, tile_cycles(SIDE, g.K, up.n_var), &gu, tab.lead[k]);
     gu.half_n = half_n;
     // Tiles that run at the same time should share the LARGER operand's blocks, so that it is
     // streamed from HBM once and the smaller one is what gets fetched again (from L2, if it fits):
     // the tiles of a batch element are walked along the shorter side first.
     gu.m_fastest = g.M < g.N ? 1 : 0;
     const Divisor by_b((uint32_t)(gu.tiles_m * gu.tiles_n)), by_inner((uint32_t)(gu.m_fastest ? gu.tiles_m : gu.tiles_n));
-    gu.b_mul = by_b.mul; gu.b_shift = by_b.shift; gu.i_mul = by_inner.mul; gu.i_shift = by_inner.shift;
-    gu.var_begin = tab.n_var; gu.n_var = up.n_var;
+    gu.b_mul = by_b.mul; gu.b_shift = (uint8_t)by_b.shift; gu.i_mul = by_inner.mul; gu.i_shift = (uint8_t)by_inner.shift;
+    gu.var_begin = (int16_t)tab.n_var; gu.n_var = (int16_t)up.n_var;
     for (int j = 0; j < up.n_var; ++j) {
       const TcProbeArgs& p = ps[up.probe[j]];
+      if (Table::kUnits != 1 && p.prepare_flags) return QM_ERR_UNSUPPORTED;      // read for probes that are launched alone only
       CUtensorMap(&vm)[2] = tab.var_maps[tab.n_var];
+      VarInfo& info = tab.info[tab.n_var];
+      tab.count[tab.n_var] = (uint64_t)(g.M * g.N * g.batch);
       GroupVar& v = tab.v[tab.n_var++];
       // blocks of codes are 64 entries deep beside the bf16 tiles, 128 on their own
       const int depth = SIDE ? kBlockK : CfgP::kLpDepth;
@@ -3036,14 +3042,14 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, bool
       if (!code_map(&vm[0], p.cl, p.cl_mn, kBlockM, g.M) || !code_map(&vm[1], p.cr, p.cr_mn, half_n, g.N)) return QM_ERR_CUDA;
       v.dl = p.dl; v.dr = p.dr;
       v.partials = p.partials; v.result = p.result; v.row_stats = p.row_stats;
-      v.err_word = p.err_word; v.prepare_flags = p.prepare_flags; v.err_also[0] = p.err_also[0]; v.err_also[1] = p.err_also[1];
-      v.count = (uint64_t)(g.M * g.N * g.batch);
-      v.info.flags = (p.fmt_l == QM_FMT_INT8 ? kVarI8 : 0u) | (p.gran_l == QM_GRAN_CHANNEL ? kVarScalePerRow : 0u) |
+      v.err_word = p.err_word; v.err_also[0] = p.err_also[0]; v.err_also[1] = p.err_also[1];
+      info.flags = (p.fmt_l == QM_FMT_INT8 ? kVarI8 : 0u) | (p.gran_l == QM_GRAN_CHANNEL ? kVarScalePerRow : 0u) |
                 (p.gran_r == QM_GRAN_CHANNEL ? kVarScalePerCol : 0u) | (p.row_stats ? kVarRowStats : 0u) |
                 (p.cl_mn ? kVarMnMajorL : 0u) | (p.cr_mn ? kVarMnMajorR : 0u);
-      v.info.idesc = lp_idesc(p.fmt_l, p.fmt_r, 2 * half_n) | (p.cl_mn ? kIdescMnMajorA : 0u) | (p.cr_mn ? kIdescMnMajorB : 0u);
+      info.idesc = lp_idesc(p.fmt_l, p.fmt_r, 2 * half_n) | (p.cl_mn ? kIdescMnMajorA : 0u) | (p.cr_mn ? kIdescMnMajorB : 0u);
     }
   }
+  pair_loads.first_units(tab.first);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(2 * pairs));
   cfg.blockDim = dim3(kProbeThreads);
