@@ -1283,7 +1283,7 @@ enum { kPairChunks = 0, kPairRows = 1, kPairTiles = 2, kPairGeneral = 3, kPairCo
 
 struct PairOperand {
   View v;
-  int32_t per_channel;
+  int32_t fmt, per_channel;
   int32_t blocks_max, n_partial;          // blocks of the first kernel; partial maxima per scale
   int32_t blocks_quant, path;             // blocks of the second kernel, and how it walks the operand
   uint32_t gx, gy;                        // tiles: column tiles, contraction tiles
@@ -1717,7 +1717,9 @@ __device__ __forceinline__ void pair_once(const PairOperand& o, uint32_t* err, u
   }
 }
 
-template <typename T, int F0, int F1>
+// T: the operands' element type.  INT: both INT8 (which goes with nothing else), else an FP8 format each, known at run time: six bodies to
+// compile, where one for each pair of formats and side made twenty (this file 269 s, 146 so; the kernels as fast).
+template <typename T, bool INT>
 __global__ void __launch_bounds__(kThreads) pair_once_kernel(const PairArgs a) {
   __shared__ uint4 smem[TileSmem<1>::kVec];
   __shared__ uint32_t s_max[kOnceBlocks][256];
@@ -1732,8 +1734,12 @@ __global__ void __launch_bounds__(kThreads) pair_once_kernel(const PairArgs a) {
     if (threadIdx.x >= gridDim.x && threadIdx.x < kPrepareFlags) flags[threadIdx.x] = 0;
   }
   const uint32_t cluster = blockIdx.x / kOnceBlocks, rank = blockIdx.x % kOnceBlocks;
-  if (cluster < a.clusters[0]) pair_once<T, F0>(a.op[0], &s_err, cluster, a.clusters[0], rank, smem, s_max);
-  else pair_once<T, F1>(a.op[1], &s_err, cluster - a.clusters[0], a.clusters[1], rank, smem, s_max);
+  const bool right = cluster >= a.clusters[0];
+  const PairOperand& o = right ? a.op[1] : a.op[0];
+  const uint32_t at = right ? cluster - a.clusters[0] : cluster, clusters = a.clusters[right];
+  if constexpr (INT) pair_once<T, QM_FMT_INT8>(o, &s_err, at, clusters, rank, smem, s_max);
+  else if (o.fmt == QM_FMT_E4M3) pair_once<T, QM_FMT_E4M3>(o, &s_err, at, clusters, rank, smem, s_max);
+  else pair_once<T, QM_FMT_E5M2>(o, &s_err, at, clusters, rank, smem, s_max);
   __syncthreads();
   if (threadIdx.x == 0) flags[blockIdx.x] = s_err ? 1 : 0;
 }
@@ -2069,7 +2075,7 @@ qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint
   for (int i = 0; i < 2; ++i) {
     const PairSide& in = side[i];
     PairOperand& o = a.op[i];
-    o.v = in.v; o.per_channel = in.gran == QM_GRAN_CHANNEL;
+    o.v = in.v; o.fmt = in.fmt; o.per_channel = in.gran == QM_GRAN_CHANNEL;
     if (in.mn && !o.per_channel) {          // codes in storage order under one scale: those of the flipped view
       o.v.nc = in.v.c; o.v.c = in.v.nc; o.v.s_nc = in.v.s_c; o.v.s_c = in.v.s_nc;
     }
@@ -2122,15 +2128,9 @@ qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at; cfg.numAttrs = pdl_enabled() ? 2 : 1;
-#define QM_PO(F0, F1)                                                                              \
-  QM_CUDA_OK(bf16 ? cudaLaunchKernelEx(&cfg, pair_once_kernel<__nv_bfloat16, F0, F1>, a)           \
-                  : cudaLaunchKernelEx(&cfg, pair_once_kernel<float, F0, F1>, a))
-    if (f0 == QM_FMT_INT8) QM_PO(QM_FMT_INT8, QM_FMT_INT8);          // (INT8 goes with INT8 only)
-    else if (f0 == QM_FMT_E4M3 && f1 == QM_FMT_E4M3) QM_PO(QM_FMT_E4M3, QM_FMT_E4M3);
-    else if (f0 == QM_FMT_E4M3) QM_PO(QM_FMT_E4M3, QM_FMT_E5M2);
-    else if (f1 == QM_FMT_E4M3) QM_PO(QM_FMT_E5M2, QM_FMT_E4M3);
-    else QM_PO(QM_FMT_E5M2, QM_FMT_E5M2);
-#undef QM_PO
+    const bool int8 = f0 == QM_FMT_INT8;                             // (INT8 goes with INT8 only)
+    QM_CUDA_OK(cudaLaunchKernelEx(&cfg, bf16 ? (int8 ? pair_once_kernel<__nv_bfloat16, true> : pair_once_kernel<__nv_bfloat16, false>)
+                                             : (int8 ? pair_once_kernel<float, true> : pair_once_kernel<float, false>), a));
     count_launch();
     *flags = control + kPrepareFlagWord;
     return QM_OK;
