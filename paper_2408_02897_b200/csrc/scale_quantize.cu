@@ -1318,6 +1318,11 @@ template <> struct Raw8<__nv_bfloat16> {
       for (int j = 0; j < 4; ++j) w[j] = (2 * j < live ? (uint32_t)__ldg(e + 2 * j) : 0u) | (2 * j + 1 < live ? (uint32_t)__ldg(e + 2 * j + 1) << 16 : 0u);
     }
   }
+  // what lies beyond `live` elements (from 1 on) is zero
+  __device__ __forceinline__ void keep(uint32_t live) {
+#pragma unroll
+    for (uint32_t j = 0; j < 4; ++j) w[j] = 2 * j + 1 < live ? w[j] : 2 * j < live ? w[j] & 0xffffu : 0u;
+  }
   static __device__ __forceinline__ uint32_t upper(uint32_t m, uint32_t x) { return __vmaxu2(m, x & 0x7fff7fffu); }
   static __device__ __forceinline__ uint32_t both(uint32_t m, uint32_t n) { return __vmaxu2(m, n); }
   // element j of the maxima as an fp32 pattern
@@ -1335,6 +1340,10 @@ template <> struct Raw8<float> {
       for (int j = 0; j < 8; ++j) w[j] = j < live ? __float_as_uint(__ldg(p + j)) : 0u;
     }
   }
+  __device__ __forceinline__ void keep(uint32_t live) {
+#pragma unroll
+    for (uint32_t j = 0; j < 8; ++j) w[j] = j < live ? w[j] : 0u;
+  }
   static __device__ __forceinline__ uint32_t upper(uint32_t m, uint32_t x) { return max(m, x & 0x7fffffffu); }
   static __device__ __forceinline__ uint32_t both(uint32_t m, uint32_t n) { return max(m, n); }
   static __device__ __forceinline__ uint32_t element(const uint32_t* m, int j) { return m[j]; }
@@ -1351,23 +1360,42 @@ __device__ __forceinline__ uint32_t pair_tensor_max(const PairOperand& o, uint32
   const int64_t inner = along_c ? v.c : v.nc, line_stride = along_c ? v.s_nc : v.s_c;
   const uint32_t stride = blocks * kThreads;
   uint32_t acc[Raw::kWords] = {};
-  auto pass = [&](auto whole) {            // every group has eight elements: no branch between the loads
-    for (uint32_t g0 = block * kThreads + threadIdx.x; g0 < o.total_groups; g0 += AHEAD * stride) {
+  auto group = [&](uint32_t g, uint32_t* k) {
+    const uint32_t line = o.by_groups.div(g), b = o.by_lines.div(line);
+    *k = (g - line * o.groups_per_line) * 8;
+    return x + (int64_t)b * v.s_b + (int64_t)(line - b * o.lines) * line_stride + *k;
+  };
+  auto fold = [&](const Raw& w) {
+#pragma unroll
+    for (int j = 0; j < Raw::kWords; ++j) acc[j] = Raw::upper(acc[j], w.w[j]);
+  };
+  // A line's last group is loaded whole as well and what lies beyond the line is taken out (strides are multiples of eight, so it belongs to
+  // the tensor's span; but for the very last group): a branch between the loads makes each of them a round trip of its own
+  auto pass = [&](auto whole, uint32_t groups) {
+    for (uint32_t g0 = block * kThreads + threadIdx.x; g0 < groups; g0 += AHEAD * stride) {
       Raw w[AHEAD];
+      uint32_t k[AHEAD];
+#pragma unroll
+      for (int u = 0; u < AHEAD; ++u) w[u].load(group(g0 + u * stride < groups ? g0 + u * stride : g0, &k[u]), 8);      // repeats change no maximum
 #pragma unroll
       for (int u = 0; u < AHEAD; ++u) {
-        const uint32_t g = g0 + u * stride < o.total_groups ? g0 + u * stride : g0;      // repeats change no maximum
-        const uint32_t line = o.by_groups.div(g), b = o.by_lines.div(line);
-        const uint32_t k = (g - line * o.groups_per_line) * 8;
-        w[u].load(x + (int64_t)b * v.s_b + (int64_t)(line - b * o.lines) * line_stride + k, decltype(whole)::value ? 8 : (int)min((uint32_t)inner - k, 8u));
+        if (!decltype(whole)::value) w[u].keep((uint32_t)inner - k[u]);
+        fold(w[u]);
       }
-#pragma unroll
-      for (int u = 0; u < AHEAD; ++u)
-#pragma unroll
-        for (int j = 0; j < Raw::kWords; ++j) acc[j] = Raw::upper(acc[j], w[u].w[j]);
     }
   };
-  if ((inner & 7) == 0) pass(std::true_type{}); else pass(std::false_type{});
+  if ((inner & 7) == 0) {
+    pass(std::true_type{}, o.total_groups);
+  } else {
+    pass(std::false_type{}, o.total_groups - 1);
+    if (block == blocks - 1 && threadIdx.x == kThreads - 1) {
+      Raw w;
+      uint32_t k;
+      const T* const p = group(o.total_groups - 1, &k);
+      w.load(p, (int)((uint32_t)inner - k));
+      fold(w);
+    }
+  }
 #pragma unroll
   for (int j = 1; j < Raw::kWords; ++j) acc[0] = Raw::both(acc[0], acc[j]);
   return block_max(max(Raw::element(acc, 0), Raw::kWords == 4 ? Raw::element(acc, 1) : 0u));
@@ -1449,8 +1477,8 @@ __device__ __forceinline__ float pair_scale(const PairOperand& o, uint32_t bits,
 }
 
 // The codes of a block of the second kernel, whatever takes its maxima: d_tensor where there is one scale, else
-// col_bits(row of the output) its max|x|.
-template <typename T, int FMT, typename Bits>
+// col_bits(row of the output) its max|x|.  SR_TILES: strided bf16 may be rounded stochastically.
+template <typename T, int FMT, bool SR_TILES, typename Bits>
 __device__ __forceinline__ void pair_codes(const PairOperand& o, uint32_t* err, uint32_t block, uint4* smem, float d_tensor, Bits col_bits) {
   const View& v = o.v;
   const T* x = static_cast<const T*>(v.data);
@@ -1514,7 +1542,7 @@ __device__ __forceinline__ void pair_codes(const PairOperand& o, uint32_t* err, 
     if (col < v.nc) d_lo[FMT] = scale(orow, writer);
     if (col + 1 < v.nc) d_hi[FMT] = scale(orow + 1, writer);
     uint8_t* const cd[3] = {o.codes, o.codes, o.codes};
-    if (o.rnd.stochastic) transpose_tile<1 << FMT, false, true, true>(x, v.nc, v.c, v.s_c, v.s_b, d_lo, d_hi, cd, ldc, nullptr, smem, at, o.rnd);
+    if (SR_TILES && o.rnd.stochastic) transpose_tile<1 << FMT, false, true, SR_TILES>(x, v.nc, v.c, v.s_c, v.s_b, d_lo, d_hi, cd, ldc, nullptr, smem, at, o.rnd);
     else transpose_tile<1 << FMT, false, true, false>(x, v.nc, v.c, v.s_c, v.s_b, d_lo, d_hi, cd, ldc, nullptr, smem, at);
   }
 }
@@ -1533,7 +1561,7 @@ __device__ __forceinline__ void pair_quantize(const PairOperand& o, uint32_t* er
     for (int i = threadIdx.x & 31; i < o.n_partial; i += 32) m = max(m, __ldg(o.partial + i));
     d_tensor = pair_scale<FMT>(o, warp_max(m), 0, block == 0 && threadIdx.x == 0, err);
   }
-  pair_codes<T, FMT>(o, err, block, smem, d_tensor, [&](int64_t row) {
+  pair_codes<T, FMT, true>(o, err, block, smem, d_tensor, [&](int64_t row) {
     uint32_t m = 0;
     for (int i = 0; i < o.n_partial; ++i) m = max(m, __ldg(o.partial + (int64_t)i * v.batch * v.nc + row));
     return m;
@@ -1684,7 +1712,7 @@ __device__ __forceinline__ void pair_once(const PairOperand& o, uint32_t* err, u
     cluster_wait();
     const float d = pair_scale<FMT>(o, cluster_max(0), 0, cluster == 0 && rank == 0 && threadIdx.x == 0, err);
     for (uint32_t block = cluster * kOnceBlocks + rank; block < (uint32_t)o.blocks_quant; block += clusters * kOnceBlocks) {
-      pair_codes<T, FMT>(o, err, block, smem, d, [](int64_t) { return 0u; });
+      pair_codes<T, FMT, false>(o, err, block, smem, d, [](int64_t) { return 0u; });
       __syncthreads();                     // the tile's shared memory
     }
     return;
@@ -1712,7 +1740,7 @@ __device__ __forceinline__ void pair_once(const PairOperand& o, uint32_t* err, u
     }
   }
   for (uint32_t y = rank; y < o.gy; y += kOnceBlocks) {
-    pair_codes<T, FMT>(o, err, (b * o.gy + y) * o.gx + strip, smem, 1.f, [&](int64_t row) { return cluster_max((int)(row - b * v.nc - first)); });
+    pair_codes<T, FMT, false>(o, err, (b * o.gy + y) * o.gx + strip, smem, 1.f, [&](int64_t row) { return cluster_max((int)(row - b * v.nc - first)); });
     __syncthreads();
   }
 }
@@ -1744,18 +1772,23 @@ __global__ void __launch_bounds__(kThreads) pair_once_kernel(const PairArgs a) {
   if (threadIdx.x == 0) flags[blockIdx.x] = s_err ? 1 : 0;
 }
 
-// Clusters of an operand in the one-launch form; 0: not served.  A tensor that every cluster reads whole may have 512 KB, a
-// column 4096 entries (an eighth of them to a block).  Whole probes in a row, two launches / one, us: fp32 128 x 256 x 256 20.8 / 17.4,
-// 64^3 16.5 / 12.6; bf16 64^3 16.0 / 13.2, 512^3 under one scale 20.6 / 20.2, under channel scales 24.2 / 19.6, 256 x 256 x
-// 1024 both strided, channel 27.4 / 22.6, 128 x 64 x 2048 32.1 / 27.9.
+// Clusters of an operand in the one-launch form; 0: not served.  Whole probes in a row, two launches / one, us.
+//   One scale, read whole by every cluster: up to 256 KB of bf16 (512 x 512 x 256 17.4 / 16.5, 128 x 128 x 1024 21.6 / 20.8; of 384 KB 17.8 / 17.6
+//   and 21.5 / 22.1, of 512 KB 17.3 / 17.7 and 22.0 / 22.9, of 1 MB 22.6 / 26.1), 512 KB of fp32, whose other form takes longer (512 x 128 x 256 24.1 /
+//   21.9), and half of that where lines end inside a group of eight (131 columns, 128 KB 20.4 / 20.2, 192 KB 21.0 / 21.4, 256 KB 22.4 / 23.3).
+//   A scale per strided column, an eighth of it to a block: columns up to 4 KB (bf16 64 x 64 x 2048 29.2 / 29.1, 512 x 512 x 2048 34.9 / 30.2, x 4096
+//   41.8 / 43.3 and 48.3 / 45.8; fp32 64 x 64 x 1024 39.5 / 37.6, x 2048 65.2 / 67.2).
+//   Strided bf16 rounded stochastically: not served (50 random probes: geometric mean 0.999; 56 x 82 x 1456 32.0 / 34.5, 66 x 220 x 32 19.1 / 21.2).
 uint32_t once_clusters(const PairOperand& o, int elem) {
   const View& v = o.v;
+  if (elem == 2 && o.rnd.stochastic && !v.c_contig()) return 0;
+  const uint32_t clusters = (uint32_t)((o.blocks_quant + kOnceBlocks - 1) / kOnceBlocks);
   if (!o.per_channel) {
-    if (v.nc * v.c * v.batch * elem > (512 << 10)) return 0;
-    return (uint32_t)std::min((o.blocks_quant + kOnceBlocks - 1) / kOnceBlocks, 12);
+    const bool ragged = (v.c_contig() ? v.c : v.nc) & 7;
+    return v.nc * v.c * v.batch * elem > ((elem == 2 ? 256 : 512) << 10) >> ragged ? 0 : clusters;
   }
-  if (o.path == kPairRows) return (uint32_t)((o.blocks_quant + kOnceBlocks - 1) / kOnceBlocks);
-  return v.c <= 4096 ? (uint32_t)(o.max_cols * v.batch) : 0;
+  if (o.path == kPairRows) return clusters;
+  return v.c * elem <= 4096 ? (uint32_t)(o.max_cols * v.batch) : 0;
 }
 
 int grid_for(int64_t work_items, int per_sm) {

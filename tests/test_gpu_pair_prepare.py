@@ -81,11 +81,12 @@ def test_non_finite_operands_are_flagged(gran, where, cd):
     assert r.device_error & 1
 
 
-# The one-launch form: operands of 512 KB and just above, strips of 64 columns whole and ragged with fewer rows than
-# blocks of a cluster, contractions up to 4096 and above.  Under channel scales 960 x 960 x 32 has a block to each of the 240
-# flags and 968 x 960 x 32 more than there are; 3 x 65 x 16 and 130 x 65 x 16 launch 24 and 40 blocks, so that the first block's
-# clearing of the unused flags splits a warp right ahead of a cluster's barrier.
-@pytest.mark.parametrize("M,N,K,batch", [(512, 511, 512, 1), (512, 513, 512, 1), (65, 3, 16, 1), (3, 129, 4096, 1), (3, 129, 4112, 1),
+# The one-launch form: operands of 256 KB and just above (of 512 KB before), of 128 KB and above where lines are ragged, strips of 64 columns
+# whole and ragged with fewer rows than blocks of a cluster, contractions of 2048, 4096 and just above.  Under channel scales 960 x 960 x 32 has a block
+# to each of the 240 flags and 968 x 960 x 32 more than there are; 3 x 65 x 16 and 130 x 65 x 16 launch 24 and 40 blocks, so that the first
+# block's clearing of the unused flags splits a warp right ahead of a cluster's barrier.
+@pytest.mark.parametrize("M,N,K,batch", [(512, 511, 512, 1), (512, 513, 512, 1), (256, 255, 512, 1), (256, 257, 512, 1), (131, 64, 496, 1), (131, 64, 512, 1),
+                                         (65, 3, 16, 1), (3, 129, 2048, 1), (3, 129, 2064, 1), (3, 129, 4096, 1), (3, 129, 4112, 1),
                                          (960, 128, 32, 1), (960, 960, 32, 1), (968, 960, 32, 1),
                                          (70, 40, 112, 4), (3, 65, 16, 1), (130, 65, 16, 1)])
 @pytest.mark.parametrize("cl,cr", [(-1, -2), (-2, -1)])
