@@ -2075,15 +2075,13 @@ qm_status launch_absmax(const View& x, int gran, uint32_t* amax_bits, cudaStream
                                : absmax_t<float>(x, gran, amax_bits, s);
 }
 
-// Which operands the two-launch form takes: fewer than 2^22 elements in both together, or 2^23 where an operand has a scale per
-// row or column or is rounded stochastically (what its kernels take by themselves leaves room for the other operand's), at most
-// 2048 contiguous rows with a scale each, and no such rows with stochastic rounding, whose maxima nobody would have taken.  Whole probes, the
+// Which operands the two-launch form takes: fewer than 2^22 elements in both together, at most 2048 contiguous rows
+// with a scale each, and no such rows with stochastic rounding, whose maxima nobody would have taken.  Whole probes, the
 // general kernels / this form: 64 x 64 x 64 21.6 / 19.2 us, 1024 x 1024 x 1024 strided INT8 channel scales 36.7 / 31.7,
 // 2048 x 1024 x 1024 33.9 / 31.7.  Beyond either line the operands' own kernels, lighter ones, fill the GPU
-// and are faster: 4096 x 500 x 1024 under one scale 29.8 / 30.4, 770 x 3078 x 2032 both strided 60.9 / 63.6, with one of them rounded
-// stochastically 68.7 / 67.0; 2048 x 2048 x 1808 under channel scales 56.4 / 52.8; 16384 rows of 256 22.6 / 25.9.
+// and are faster: 4096 x 1024 x 1024 strided 44.3 / 46.0, 2048 x 2048 x 2048 60.3 / 64.1; 16384 rows of 256 22.6 / 25.9.
 static bool pair_size(const View& v) {
-  return v.nc <= (1 << 23) && v.c <= (1 << 23) && v.batch <= (1 << 15) && v.nc * v.c <= (1ll << 23) && v.nc * v.c * v.batch <= (1ll << 23);
+  return v.nc <= (1 << 22) && v.c <= (1 << 22) && v.batch <= (1 << 15) && v.nc * v.c <= (1ll << 22) && v.nc * v.c * v.batch <= (1ll << 22);
 }
 static bool pair_serves(const View& v, int gran, bool stochastic) {
   const bool rows = gran == QM_GRAN_CHANNEL && v.c_contig();
@@ -2098,7 +2096,7 @@ size_t pair_partial_words(const View& v, int gran) {
 
 bool pair_prepare_serves(const View& l, int gran_l, bool draw_l, const View& r, int gran_r, bool draw_r) {
   return l.dtype == r.dtype && pair_serves(l, gran_l, draw_l) && pair_serves(r, gran_r, draw_r) &&
-         (l.nc + r.nc) * l.c * l.batch < (gran_l == QM_GRAN_CHANNEL || gran_r == QM_GRAN_CHANNEL || draw_l || draw_r ? 1ll << 23 : 1ll << 22);
+         (l.nc + r.nc) * l.c * l.batch < (1ll << 22);
 }
 
 qm_status launch_pair_prepare(const PairSide (&side)[2], uint32_t* control, uint32_t control_words, const uint32_t** flags, cudaStream_t s) {
