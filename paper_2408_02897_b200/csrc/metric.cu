@@ -1,5 +1,7 @@
 // Eq. 3 on materialised arrays, and the deterministic final reduction shared with the fused
 // probe kernels.
+#include <algorithm>
+
 #include "qm_internal.h"
 #include "reduce.cuh"
 
@@ -168,13 +170,18 @@ __global__ void clear_many_kernel(const ClearList list) {
   pdl_prologue();
   const int w = blockIdx.x;                      // gridDim.y blocks per region
   uint32_t* p = static_cast<uint32_t*>(list.ptr[w]);
-  for (uint32_t i = blockIdx.y * blockDim.x + threadIdx.x; i < list.words[w]; i += gridDim.y * blockDim.x) p[i] = 0u;
+  const uint64_t n = list.words[w];
+  for (uint64_t i = blockIdx.y * blockDim.x + threadIdx.x; i < n; i += gridDim.y * blockDim.x) p[i] = 0u;
 }
 }  // namespace
 
 qm_status launch_clear_many(const ClearList& list, cudaStream_t s) {
   if (list.n < 1 || list.n > kClearMax) return QM_ERR_INVALID_ARG;
-  QM_CUDA_OK(launch_pdl(clear_many_kernel, dim3((unsigned)list.n, 8), dim3(256), 0, s, list));
+  // four words to a thread until the GPU has two blocks for each SM (2^20 maxima by eight blocks: 6.6 us of a scale call of 23.1)
+  uint64_t most = 0;
+  for (int i = 0; i < list.n; ++i) most = std::max(most, list.words[i]);
+  const uint64_t cap = std::max(1, 2 * sm_count() / list.n), want = (most + 1023) / 1024;
+  QM_CUDA_OK(launch_pdl(clear_many_kernel, dim3((unsigned)list.n, (unsigned)std::clamp<uint64_t>(want, 1, cap)), dim3(256), 0, s, list));
   count_launch();
   return QM_OK;
 }

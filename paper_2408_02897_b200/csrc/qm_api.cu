@@ -104,14 +104,7 @@ qm_status to_view(const qm_operand* x, View* v) {
 
 int64_t delta_count(const View& v, int gran) { return gran == QM_GRAN_TENSOR ? 1 : v.nc * v.batch; }
 
-// Zeroes the maxima ahead of the kernels of a scale or quantize call.  From 8 MB on by a kernel, behind which the next one starts
-// early (stochastic E5M2 codes of 16384 x 1024 strided 41.0 us with a memset, 37.8 so); below that a call is bound by its
-// submission, and a memset is the cheaper one (729 x 1401 in fp32 21.0 / 22.1).
-qm_status clear_maxima(const View& v, void* p, int64_t words, cudaStream_t s) {
-  if (v.batch * v.nc * v.c * (v.dtype == QM_DT_BF16 ? 2 : 4) >= (8 << 20)) return clear_words(p, (size_t)words, s);
-  QM_CUDA_OK(cudaMemsetAsync(p, 0, 4 * (size_t)words, s));
-  return QM_OK;
-}
+int64_t operand_bytes(const View& v) { return v.batch * v.nc * v.c * (v.dtype == QM_DT_BF16 ? 2 : 4); }
 
 size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
 
@@ -238,7 +231,7 @@ qm_status qm_scale(const qm_operand* x, int32_t fmt, int32_t gran, float* delta,
   if (!valid_fmt(fmt) || !valid_gran(gran) || !delta) return QM_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int64_t n = delta_count(v, gran);
-  st = clear_maxima(v, delta, n, s);
+  st = clear_words(delta, (size_t)n, operand_bytes(v), s);
   if (st != QM_OK) return st;
   st = launch_absmax(v, gran, reinterpret_cast<uint32_t*>(delta), s);
   if (st != QM_OK) return st;
@@ -253,7 +246,7 @@ qm_status qm_scale_shared(const qm_operand* x, int32_t fmt, int32_t batch_groups
   if (batch_groups < 1 || v.batch % batch_groups) return QM_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int64_t n = v.nc * v.batch;
-  st = clear_maxima(v, delta, n, s);
+  st = clear_words(delta, (size_t)n, operand_bytes(v), s);
   if (st != QM_OK) return st;
   st = launch_absmax(v, QM_GRAN_CHANNEL, reinterpret_cast<uint32_t*>(delta), s);
   if (st != QM_OK) return st;
@@ -281,7 +274,7 @@ static qm_status quantize_entry(const qm_operand* x, int32_t fmt, int32_t gran, 
   const int64_t n = delta_count(v, gran);
   if (!draw && gran == QM_GRAN_CHANNEL && v.c_contig() && !kmaj_copy)
     return launch_scale_quantize_rows(v, fmt, delta_out, codes, abs_copy, nullptr, s);
-  st = clear_maxima(v, delta_out, n, s);
+  st = clear_words(delta_out, (size_t)n, 2 * operand_bytes(v) + v.batch * v.nc * v.c, s);
   if (st != QM_OK) return st;
   st = launch_absmax(v, gran, reinterpret_cast<uint32_t*>(delta_out), s);
   if (st != QM_OK) return st;
@@ -321,7 +314,7 @@ qm_status qm_quantize_formats(const qm_operand* x, int32_t n_fmt, const int32_t*
   if (reinterpret_cast<uintptr_t>(kmaj_copy) & 15) return QM_ERR_ALIGNMENT;
   if (kmaj_copy && v.dtype != QM_DT_BF16) return QM_ERR_UNSUPPORTED;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  st = clear_maxima(v, amax_scratch, delta_count(v, gran), s);
+  st = clear_words(amax_scratch, (size_t)delta_count(v, gran), 2 * operand_bytes(v) + n_fmt * v.batch * v.nc * v.c, s);
   if (st != QM_OK) return st;
   st = launch_absmax(v, gran, amax_scratch, s);
   if (st != QM_OK) return st;
@@ -422,9 +415,9 @@ static qm_status probe_phases(const qm_operand* Lo, const qm_operand* Ro, const 
     if (st != QM_OK) return st;
   } else if ((phases & kClear) && clear_later && clear_later->n < kClearMax) {
     clear_later->ptr[clear_later->n] = base;                 // cleared with others by one kernel
-    clear_later->words[clear_later->n++] = (uint32_t)(w.off_dl / 4);
+    clear_later->words[clear_later->n++] = w.off_dl / 4;
   } else if (phases & kClear) {
-    st = clear_words(base, w.off_dl / 4, s);
+    st = clear_words(base, w.off_dl / 4, operand_bytes(L) + operand_bytes(R), s);
     if (st != QM_OK) return st;
   }
   if ((phases & kClear) && cfg->row_stats)
@@ -849,7 +842,7 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
       clears.n = 0;
     }
     clears.ptr[clears.n] = base;                       // error word, CTA counter and both max|x| buffers are adjacent
-    clears.words[clears.n++] = (uint32_t)(pl.w.off_dl / 4);
+    clears.words[clears.n++] = pl.w.off_dl / 4;
     if (cfg[i].row_stats)
       QM_CUDA_OK(cudaMemsetAsync(cfg[i].row_stats, 0, sizeof(double) * QM_ROW_STATS * (size_t)(pl.Lv.batch * pl.Lv.nc), user));
     slot_of[i] = (int)slots.size();

@@ -160,16 +160,22 @@ qm_status launch_metric_finalize(const double* partials, int n, uint64_t count,
 // Zeroes up to kClearMax regions of 32-bit words (4-byte aligned) in one launch: the control words
 // of the workspaces of a batch.
 constexpr int kClearMax = 32;
-struct ClearList { int n; void* ptr[kClearMax]; uint32_t words[kClearMax]; };
+struct ClearList { int n; void* ptr[kClearMax]; uint64_t words[kClearMax]; };
 qm_status launch_clear_many(const ClearList& list, cudaStream_t s);
-// Zeroes one region.  (Behind a memset the next kernel cannot start early, behind this one it can: see pdl_prologue.)
-inline qm_status clear_words(void* p, size_t words, cudaStream_t s) {
-  if (words > 0xffffffffull) {
+// Zeroes one region ahead of the kernels of a call, which move `bytes` in all.  Behind a kernel the next one can start early (pdl_prologue),
+// behind a memset it cannot; but the memset of one word is submitted in 1.0 to 1.4 us less, and that is what a call waits for that is
+// bound by its submission or waited for by itself.  Memset / kernel, us, in a row and waited for: scales under one scale of 32 MB 10.9 / 8.3 (10.9 /
+// 11.9 on a slower host) and 17.6 / 19.1, 64 MB 16.0 / 12.9 (10.8 / 11.9) and
+// 22.1 / 23.7, 128 MB 24.3 / 22.0 and 31.1 / 32.7; codes (two reads, one write) of 16 MB 14.1 / 11.0 (13.5 / 14.5) and 20.4 / 21.8,
+// 32 MB 19.5 / 16.7 and 26.6 / 27.9; statistics and error of a tensor, each waited for, 32 MB 87.5 / 89.0, 134 MB 154.6 / 151.6.  Of several words the
+// memset is a kernel as well: scales per column of 16 MB 10.3 / 8.4 and 19.4 / 19.3, of 2^20 columns 16.5 / 15.1.
+inline qm_status clear_words(void* p, size_t words, int64_t bytes, cudaStream_t s) {
+  if (words > 1 ? bytes < 8ll << 20 : bytes <= 64ll << 20) {
     QM_CUDA_OK(cudaMemsetAsync(p, 0, 4 * words, s));
     return QM_OK;
   }
   ClearList l{};
-  l.n = 1; l.ptr[0] = p; l.words[0] = (uint32_t)words;
+  l.n = 1; l.ptr[0] = p; l.words[0] = words;
   return launch_clear_many(l, s);
 }
 

@@ -499,7 +499,7 @@ qm_status launch_pass(const Lines& p, void* result, uint64_t count, void* ws, cu
   const int resident = resident_of[dev];
   uint32_t* counter = static_cast<uint32_t*>(ws);
   double* partials = reinterpret_cast<double*>(static_cast<char*>(ws) + kCounterBytes);
-  const qm_status st = clear_words(counter, 1, s);
+  const qm_status st = clear_words(counter, 1, (int64_t)(count * sizeof(T)), s);
   if (st != QM_OK) return st;
   QM_CUDA_OK(launch_pdl(tensor_pass_kernel<T, KIND, FMT, MODE>, dim3(pass_blocks(p, resident)), dim3(kThreads), 0, s, p,
                         partials, counter, result, count));
@@ -522,7 +522,7 @@ qm_status launch_tensor_stats(const View& x, qm_tensor_stats_result* out, void* 
     // dense, aligned and large enough to be worth it: the 256-bit kernel
     uint32_t* counter = static_cast<uint32_t*>(ws);
     double* partials = reinterpret_cast<double*>(static_cast<char*>(ws) + kCounterBytes);
-    st = clear_words(counter, 1, s);
+    st = clear_words(counter, 1, (int64_t)bytes, s);
     if (st != QM_OK) return st;
     const uint64_t n_vec = bytes / 32;
     int64_t blocks = (int64_t)((n_vec + kThreads - 1) / kThreads);

@@ -1,4 +1,6 @@
 """GPU parity: scales and codes against the oracle, bit for bit (Eq. 1, saturation rule)."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
@@ -290,3 +292,21 @@ def test_dense_tensors_off_the_32_byte_grid(fmt):
         if cols % 16 == 0:
             codes, _, _, _ = qm.qm_quantize(op, fmt, "tensor", d)
             assert np.array_equal(codes.cpu().numpy()[..., :cols], oracle.quantize(x, fmt, want_d)), (off, rows, cols)
+
+
+# Scales per column over buffers that held something else: maxima cleared by a memset and by a kernel of few and of as many blocks as there are
+@pytest.mark.parametrize("contract,columns", [(16, 37), (16, 262143), (16, 262153), (4, 1100001)])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_scales_of_many_columns_start_from_zero(contract, columns, dtype):
+    x = torch.zeros((contract, (columns + 7) // 8 * 8), dtype=dtype, device="cuda")[:, :columns]
+    x.copy_(make((contract, columns), dtype, columns, "normal"))
+    op = qm.operand_of(x, -2)
+    delta = torch.full((columns,), 1e30, device="cuda")
+    codes = torch.empty(columns * qm.qm_code_ld(contract), dtype=torch.uint8, device="cuda")
+    want = torch.from_numpy(x.float().abs().amax(0).cpu().numpy() / np.float32(448.0))       # (on the GPU torch multiplies by 1 / 448)
+    lib, stream = qm.lib(), torch.cuda.current_stream().cuda_stream
+    assert lib.qm_scale(C.byref(op), 1, 1, delta.data_ptr(), stream) == 0
+    assert torch.equal(delta.cpu(), want)
+    delta.fill_(1e30)
+    assert lib.qm_quantize(C.byref(op), 1, 1, 0, None, delta.data_ptr(), codes.data_ptr(), None, None, stream) == 0
+    assert torch.equal(delta.cpu(), want)
