@@ -6,7 +6,7 @@ import pytest
 import torch
 
 import paper_2408_02897_b200 as qm
-from paper_2408_02897_b200 import workloads
+from paper_2408_02897_b200 import binding, workloads
 
 pytestmark = pytest.mark.gpu
 
@@ -187,3 +187,24 @@ def test_dense_tensors_prepared_together(count, fmts):
     batch.launch()
     torch.cuda.synchronize()
     assert all(r.device_error == 0 for r in batch.results())
+
+
+def test_stochastic_codes_beside_tensors_prepared_together():
+    """Stochastic codes borrow the maxima of the joint preparation: those of large tensors follow it on streams of the
+    library, those of small ones on the caller's; also where the tensor contracts along its other dimension."""
+    rng = workloads._rng(150)
+    probes, rounds = [], []
+    for rows, K in ((640, 400), (512, 400), (48, 400), (700, 288), (100, 16)):
+        X, W = workloads.normal(rng, (rows, K)).cuda(), workloads.normal(rng, (K, 64 if K < 300 else K), 0.05).cuda()
+        for fmt, rounding in (("e4m3", "rtne"), ("e4m3", "stochastic_l"), ("e5m2", "stochastic_both"), ("int8", "stochastic_r")):
+            probes.append((qm.operand_of(X, -1), qm.operand_of(W, -2), fmt, fmt, "tensor", "tensor")); rounds.append(rounding)
+            if W.shape[1] == K:                          # the same tensors, the right one contracting along its rows
+                probes.append((qm.operand_of(X, -1), qm.operand_of(W, -1), fmt, fmt, "tensor", "tensor")); rounds.append(rounding)
+    batch = qm.ProbeBatch(probes)
+    for i, r in enumerate(rounds):
+        batch.cfg[i].round, batch.cfg[i].seed = binding.ROUND[r], 40 + i
+    single = [qm.qm_probe_layer(*p, rounding=r, seed=40 + i) for i, (p, r) in enumerate(zip(probes, rounds))]
+    for _ in range(3):
+        batch.launch()
+        torch.cuda.synchronize()
+        assert all(_same(g, s) for g, s in zip(batch.results(), single))
