@@ -2849,6 +2849,7 @@ struct UnitPlan {
   GemmShape g;
   int n_var;
   int probe[kMaxVar];
+  double cycles;              // of a tile (tile_cycles)
 };
 
 bool same_products(const TcProbeArgs& a, const TcProbeArgs& b) {
@@ -3016,7 +3017,7 @@ qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, bool
     fill_tiles(&ka, g);
     gu.M = (int32_t)g.M; gu.N = (int32_t)g.N; gu.K = (int32_t)g.K;
     gu.tiles_m = ka.tiles_m; gu.tiles_n = ka.tiles_n;
-    pair_loads.deal(k, ka.num_tiles, tile_cycles(SIDE, g.K, up.n_var), &gu, tab.lead[k]);
+    pair_loads.deal(k, ka.num_tiles, up.cycles, &gu, tab.lead[k]);
     gu.half_n = half_n;
     // Tiles that run at the same time should share the LARGER operand's blocks, so that it is
     // streamed from HBM once and the smaller one is what gets fetched again (from L2, if it fits):
@@ -3092,7 +3093,7 @@ qm_status launch_tc_probes(const TcProbeArgs* ps, int n, cudaStream_t s) {
     for (UnitPlan& c : units)
       if (c.n_var < kMaxVar && same_products(ps[c.probe[0]], ps[i])) { u = &c; break; }
     if (!u) {
-      units.push_back(UnitPlan{ps[i].g, 0, {}});
+      units.push_back(UnitPlan{ps[i].g, 0, {}, 0.0});
       u = &units.back();
     }
     u->probe[u->n_var++] = i;
@@ -3104,11 +3105,10 @@ qm_status launch_tc_probes(const TcProbeArgs* ps, int n, cudaStream_t s) {
   int64_t single_tiles = 0;
   for (auto u = units.begin(); u != others; ++u) single_tiles += tile_count(u->g);
   const size_t n_side = others == units.end() || single_tiles >= max_pairs() ? (size_t)(others - units.begin()) : 0;
-  auto by_cost = [](bool side) {               // descending
-    return [side](const UnitPlan& a, const UnitPlan& b) { return tile_cycles(side, a.g.K, a.n_var) > tile_cycles(side, b.g.K, b.n_var); };
-  };
-  std::stable_sort(units.begin(), units.begin() + n_side, by_cost(true));
-  std::stable_sort(units.begin() + n_side, units.end(), by_cost(false));
+  for (size_t k = 0; k < units.size(); ++k) units[k].cycles = tile_cycles(k < n_side, units[k].g.K, units[k].n_var);
+  auto by_cost = [](const UnitPlan& a, const UnitPlan& b) { return a.cycles > b.cycles; };      // descending
+  std::stable_sort(units.begin(), units.begin() + n_side, by_cost);
+  std::stable_sort(units.begin() + n_side, units.end(), by_cost);
   auto any_mn = [&](const UnitPlan* u, int count) {
     for (int k = 0; k < count; ++k) {
       const TcProbeArgs& a = ps[u[k].probe[0]];
