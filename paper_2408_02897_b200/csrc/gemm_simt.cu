@@ -284,16 +284,19 @@ __global__ void __launch_bounds__(kThreads, 2) simt_kernel(const SimtArgs a) {
     }
   }
   if (PROBE) {
+    // (the asm keeps what follows of it from being computed ahead of the products and held through them: 72 bytes of spills at 64 x 64, 40 so)
+    uint32_t t = threadIdx.x;
+    asm volatile("" : "+r"(t));
     double v[4] = {fbe, fd2, fr2, fn2};
     // field of the record that this thread and its seven neighbours hold: the sums around the maximum
-    const int held = threadIdx.x >> 3, field = held == 0 ? 0 : held == 4 ? 1 : held + 1;
-    const bool writer = (threadIdx.x & 7) == 0 && held < 5;
-    double x = block_record<4>(v, fmx, sred);
+    const int held = t >> 3, field = held == 0 ? 0 : held == 4 ? 1 : held + 1;
+    const bool writer = (t & 7) == 0 && held < 5;
+    double x = block_record<4>(v, fmx, sred, t);
     const int64_t n_blocks = (int64_t)gridDim.x * gridDim.y * gridDim.z;
     const int64_t blk = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
     if (writer) __stcg(a.partials + blk * kPartialDoubles + field, x);
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (t == 0) {
       __threadfence();                     // after the barrier: covers what the others have written
       s_last = atomicAdd(a.done_counter, 1u) == (uint32_t)(n_blocks - 1) ? 1u : 0u;
     }
@@ -302,16 +305,16 @@ __global__ void __launch_bounds__(kThreads, 2) simt_kernel(const SimtArgs a) {
       __threadfence();
       v[0] = v[1] = v[2] = v[3] = 0.0;
       float mx = 0.f;
-      for (int64_t k = threadIdx.x; k < n_blocks; k += kThreads) {
+      for (int64_t k = t; k < n_blocks; k += kThreads) {
         const double* rec = a.partials + k * kPartialDoubles;
         v[0] += __ldcg(rec); mx = fmaxf(mx, (float)__ldcg(rec + 1)); v[1] += __ldcg(rec + 2);
         v[2] += __ldcg(rec + 3); v[3] += __ldcg(rec + 4);
       }
-      const int not_finite = __syncthreads_or(a.prepare_flags && threadIdx.x < kPrepareFlagWords && __ldcg(a.prepare_flags + threadIdx.x));
-      x = block_record<4>(v, mx, sred);
+      const int not_finite = __syncthreads_or(a.prepare_flags && t < kPrepareFlagWords && __ldcg(a.prepare_flags + t));
+      x = block_record<4>(v, mx, sred, t);
       if (writer) tot[field] = x;
       __syncthreads();
-      if (threadIdx.x == 0) {                // (the record may be in host memory: stores only, every field once)
+      if (t == 0) {                // (the record may be in host memory: stores only, every field once)
         a.result->sum_be = tot[0]; a.result->max_be = tot[1]; a.result->sum_diff2 = tot[2];
         a.result->sum_ref2 = tot[3]; a.result->sum_den2 = tot[4];
         a.result->count = a.count;

@@ -35,8 +35,8 @@ __device__ __forceinline__ double warp_sums(const double (&v)[N], int lane, int 
 // N sums and a maximum (of floats that are neither negative nor NaN) over the block's 256 threads; thread 8 i + k returns sum i
 // for i < N, the maximum for i = N.  All threads call; red may be reused after a barrier.
 template <int N>
-__device__ __forceinline__ double block_record(const double (&v)[N], float mx, double (&red)[N + 1][8]) {
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+__device__ __forceinline__ double block_record(const double (&v)[N], float mx, double (&red)[N + 1][8], int t = threadIdx.x) {
+  const int lane = t & 31, warp = t >> 5;
   int index = 0, left = N, below;
   const double x = warp_sums<N>(v, lane, 16, index, left, below);
   const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
