@@ -327,10 +327,11 @@ __global__ void __launch_bounds__(kThreads, 2) simt_kernel(const SimtArgs a) {
 
 // The shape whose busiest SM is through first: the blocks there, times what a block takes (fitted: a 32 x 32 block 1.3 times its share of
 // a 64 x 64 one, a 16 x 32 block 1.75 times), over the rate at which one block (0.62 of the issue slots) or several (0.85) issue.
-// What this is for: a few blocks more than the GPU has SMs double the time.  Contractions below 96 are bound by what a block does
-// once, and take the largest shape that gives every SM more than one (900 x 900 x 60 64 x 64 26.7 us, 32 x 64 27.9; K = 120 the
-// other way round, 35.1 / 34.1).  Whole probes of 700 x 400 x 368: 154 blocks of 32 x 64 53.7 us, 286 of 32 x 32 37.2; 1024^3 64 x 64 205, 32 x
-// 32 232; 400 x 400 x 300 INT8 32 x 32 28.4, 16 x 32 35.8; 128 x 256 x 256 64 blocks of 16 x 32.
+// What this is for: a few blocks more than the GPU has SMs double the time.  Contractions below 96 are bound as much by what a block does
+// once, and take the largest shape with five blocks for four SMs, those below 64 the largest with more blocks than SMs.  64 x 64 / 32 x 64, us: 640 x 960 (150
+// blocks of 64 x 64) K = 20 17.5 / 18.3, 60 23.7 / 23.7, 80 30.5 / 29.3, 95 30.9 / 30.0; 900 x 900 (225) K = 20 17.8 / 20.6, 80 30.9 / 30.5, 95 31.3 / 32.7; 1200 x 800
+// (247) K = 95 33.0 / 36.0; 690 x 307 x 65 INT8 220 blocks of 32 x 32 19.8, 440 of 16 x 32 22.1; 900 x 900 x 120 35.1 / 34.1.  Whole probes of 700 x 400 x 368: 154 blocks of 32 x 64 53.7 us, 286 of 32 x 32 37.2; 1024^3 64 x 64
+// 205, 32 x 32 232; 400 x 400 x 300 INT8 32 x 32 28.4, 16 x 32 35.8; 128 x 256 x 256 64 blocks of 16 x 32.
 constexpr int kShapes[4][2] = {{64, 64}, {32, 64}, {32, 32}, {16, 32}};
 dim3 grid_of(GemmShape g, int shape) {
   const int tm = kShapes[shape][0], tn = kShapes[shape][1];
@@ -343,8 +344,8 @@ int shape_of(GemmShape g) {
   for (int i = 0; i < 4; ++i) {
     const int64_t tm = kShapes[i][0], tn = kShapes[i][1], rows = (g.M + tm - 1) / tm;
     if (i > 0 && rows > 65535) break;                 // (the limit of the grid holds for the largest shape only)
-    const int64_t per_sm = (rows * ((g.N + tn - 1) / tn) * g.batch + sm_count() - 1) / sm_count();
-    if (g.K < 96 && per_sm >= 2) return i;
+    const int64_t blocks = rows * ((g.N + tn - 1) / tn) * g.batch, sms = sm_count(), per_sm = (blocks + sms - 1) / sms;
+    if (g.K < 64 ? blocks > sms : g.K < 96 && i < 3 && 4 * blocks >= 5 * sms) return i;
     const double cost = (double)per_sm * kBlockCost[i] / (per_sm == 1 ? 0.62 : 0.85);
     if (i == 0 || cost < least) { best = i; least = cost; }
   }

@@ -46,7 +46,8 @@ def test_fp32_probe_against_the_oracle(M, N, K, batch, cl, cr, fmt, gran):
 
 
 # extents at which the tile shape changes: just over one block for an SM in one shape, and what is taken instead
-@pytest.mark.parametrize("M,N,K", [(700, 400, 68), (704, 448, 36), (350, 350, 40), (1030, 1030, 20), (17, 33, 300), (4000, 30, 24)])
+@pytest.mark.parametrize("M,N,K", [(700, 400, 68), (704, 448, 36), (350, 350, 40), (1030, 1030, 20), (17, 33, 300), (4000, 30, 24),
+                                   (640, 960, 63), (640, 960, 64), (900, 900, 95), (900, 900, 96)])
 @pytest.mark.parametrize("fmt,gran", [("e4m3", "tensor"), ("int8", "channel")])
 def test_tile_shapes_against_the_oracle(M, N, K, fmt, gran):
     rng = workloads._rng(M + N)
