@@ -373,14 +373,9 @@ size_t qm_workspace_bytes(const qm_operand* Lo, const qm_operand* Ro, const qm_p
   return plan(L, R, *cfg).total;
 }
 
-// The probe in phases that may be issued apart (same arguments every time): kClear clears the
-// workspace words (or only lists them in *clear_later, for one clearing kernel over a batch),
-// kPrepareL / kPrepareR run scale + quantize of one operand (after kClear), kProducts the
-// products and the Eq. 3 reduction (after both).
-enum { kClear = 1, kPrepareL = 2, kPrepareR = 4, kPrepare = kClear | kPrepareL | kPrepareR, kProducts = 8 };
-static qm_status probe_phases(const qm_operand* Lo, const qm_operand* Ro, const qm_probe_cfg* cfg,
-                              qm_metric_result* out, void* ws, size_t ws_bytes, void* stream, int phases,
-                              ClearList* clear_later = nullptr) {
+// Prepares both operands, multiplies and reduces: everything a single probe puts into its stream.
+static qm_status single_probe(const qm_operand* Lo, const qm_operand* Ro, const qm_probe_cfg* cfg, qm_metric_result* out, void* ws,
+                              size_t ws_bytes, void* stream) {
   View L, R;
   qm_status st = check_probe(Lo, Ro, cfg, &L, &R);
   if (st != QM_OK) return st;
@@ -402,8 +397,7 @@ static qm_status probe_phases(const qm_operand* Lo, const qm_operand* Ro, const 
   const bool cl_mn = w.tc && codes_mn(L, dl_draw != nullptr), cr_mn = w.tc && codes_mn(R, dr_draw != nullptr);
   // operands of modest size: both in two launches, or one, the first of which clears the control words
   auto grouped = [](const View& v, int gran, int groups) { return gran == QM_GRAN_CHANNEL && groups > 0 && groups < v.batch; };
-  const bool pair = (phases & kPrepare) == kPrepare && !clear_later && !grouped(L, cfg->gran_l, cfg->batch_groups_l) &&
-                    !grouped(R, cfg->gran_r, cfg->batch_groups_r) &&
+  const bool pair = !grouped(L, cfg->gran_l, cfg->batch_groups_l) && !grouped(R, cfg->gran_r, cfg->batch_groups_r) &&
                     pair_prepare_serves(L, cfg->gran_l, dl_draw != nullptr, R, cfg->gran_r, dr_draw != nullptr);
   // the error word, the finished-CTA counter and both max|x| buffers are adjacent: one clear
   const uint32_t* flags = nullptr;
@@ -413,26 +407,20 @@ static qm_status probe_phases(const qm_operand* Lo, const qm_operand* Ro, const 
         {R, cfg->fmt_r, cfg->gran_r, cr_mn, dr_draw, reinterpret_cast<uint32_t*>(base + w.off_pr), dr, cr}};
     st = launch_pair_prepare(side, err, 64, &flags, s);
     if (st != QM_OK) return st;
-  } else if ((phases & kClear) && clear_later && clear_later->n < kClearMax) {
-    clear_later->ptr[clear_later->n] = base;                 // cleared with others by one kernel
-    clear_later->words[clear_later->n++] = w.off_dl / 4;
-  } else if (phases & kClear) {
+  } else {
     st = clear_words(base, w.off_dl / 4, operand_bytes(L) + operand_bytes(R), s);
     if (st != QM_OK) return st;
   }
-  if ((phases & kClear) && cfg->row_stats)
+  if (cfg->row_stats)
     QM_CUDA_OK(cudaMemsetAsync(cfg->row_stats, 0, sizeof(double) * QM_ROW_STATS * (size_t)(L.batch * L.nc), s));
   uint32_t* ml = reinterpret_cast<uint32_t*>(base + w.off_ml);
   uint32_t* mr = reinterpret_cast<uint32_t*>(base + w.off_mr);
-  if ((phases & kPrepareL) && !pair) {
+  if (!pair) {
     st = prepare_operand(L, cfg->fmt_l, cfg->gran_l, cl_mn, ml, dl, cl, err, dl_draw, cfg->batch_groups_l, s);
     if (st != QM_OK) return st;
-  }
-  if ((phases & kPrepareR) && !pair) {
     st = prepare_operand(R, cfg->fmt_r, cfg->gran_r, cr_mn, mr, dr, cr, err, dr_draw, cfg->batch_groups_r, s);
     if (st != QM_OK) return st;
   }
-  if (!(phases & kProducts)) return QM_OK;
   GemmShape g{L.nc, R.nc, L.c, L.batch};
   if (w.tc) {
     TcProbeArgs p{};                        // (the fused kernel forms |L| and |R| on chip)
@@ -451,7 +439,7 @@ static qm_status probe_phases(const qm_operand* Lo, const qm_operand* Ro, const 
 
 qm_status qm_probe_layer(const qm_operand* Lo, const qm_operand* Ro, const qm_probe_cfg* cfg,
                          qm_metric_result* out, void* ws, size_t ws_bytes, void* stream) {
-  return probe_phases(Lo, Ro, cfg, out, ws, ws_bytes, stream, kPrepare | kProducts);
+  return single_probe(Lo, Ro, cfg, out, ws, ws_bytes, stream);
 }
 
 // ---- two formats in one pass -------------------------------------------------------------------
@@ -995,7 +983,7 @@ qm_status qm_probe_batch(int32_t n, const qm_operand* L, const qm_operand* R, co
   for (int32_t i = 0; i < good; ++i) {
     if (plans[i].tc) continue;
     cudaStream_t s = stream_of(next_stream); next_stream = (next_stream + 1) % kBatchStreams;
-    const qm_status e = probe_phases(&L[i], &R[i], &cfg[i], out + i, ws[i], ws_bytes[i], s, kPrepare | kProducts);
+    const qm_status e = single_probe(&L[i], &R[i], &cfg[i], out + i, ws[i], ws_bytes[i], s);
     if (e != QM_OK && st == QM_OK) st = e;
   }
   if (st == QM_OK) st = fork_error;
