@@ -311,6 +311,7 @@ struct alignas(16) Shared {
 // Named barrier 1 over the 256 epilogue threads, returning the OR of `flag` over all of them.
 __device__ __forceinline__ bool epi_barrier_any(bool flag) {
   uint32_t out;
+  __syncwarp();            // bar.red wants the whole warp, whose lanes have waited on a barrier one by one
   asm volatile(
       "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\t"
       "bar.red.or.pred p, 1, 256, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
