@@ -208,3 +208,45 @@ def test_stochastic_codes_beside_tensors_prepared_together():
         batch.launch()
         torch.cuda.synchronize()
         assert all(_same(g, s) for g, s in zip(batch.results(), single))
+
+
+def test_dense_tensors_in_four_chunks_a_thread():
+    """Enough elements in one batch for the form with four chunks to a thread: ragged ends of both tensors, a scale outside the range
+    of the two-wide quotient, a value that is not finite as the very last element."""
+    rng = workloads._rng(151)
+    R = workloads.normal(rng, (48, 4096), 0.05).cuda()
+    large, small = workloads.normal(rng, (4801, 4096)).cuda(), (workloads.normal(rng, (301, 4096)) * 1e-30).cuda()
+    probes = [(qm.operand_of(L, -1), qm.operand_of(R, -1), f, f, "tensor", "tensor") for L in (large, small) for f in ("e4m3", "int8")]
+    single = [qm.qm_probe_layer(*p) for p in probes]
+    batch = qm.ProbeBatch(probes)
+    batch.launch()
+    torch.cuda.synchronize()
+    assert all(_same(g, s) for g, s in zip(batch.results(), single))
+    for i, L in enumerate((large, small)):
+        old = L[-1, -1].clone()
+        L[-1, -1] = float("inf")
+        batch.launch()
+        torch.cuda.synchronize()
+        L[-1, -1] = old
+        assert [r.device_error & 1 for r in batch.results()] == [int(i == 0)] * 2 + [int(i == 1)] * 2
+
+
+def test_the_same_values_off_the_joint_preparation():
+    """Tensors that the joint preparation refuses beside ones that it takes: the same values from a start of 16 bytes, with a row pitch
+    and with a gap between the matrices of a batch all give the dense tensor's records."""
+    rng = workloads._rng(152)
+    b, M, K = 2, 130, 208
+    dense = workloads.normal(rng, (b, M, K)).cuda()
+    off = torch.full((b * M * K + 8,), 9.0, dtype=torch.bfloat16, device="cuda")[8:].view(b, M, K)
+    pitch = torch.full((b, M, K + 8), 9.0, dtype=torch.bfloat16, device="cuda")[:, :, :K]
+    gap = torch.full((b, M + 3, K), 9.0, dtype=torch.bfloat16, device="cuda")[:, :M]
+    R = workloads.normal(rng, (b, 72, K), 0.05).cuda()
+    kinds = [dense] + [t.copy_(dense) for t in (off, pitch, gap)]
+    assert dense.data_ptr() % 32 == 0 and off.data_ptr() % 32 == 16
+    probes = [(qm.operand_of(L, -1), qm.operand_of(R, -1), f, f, "tensor", "tensor") for L in kinds for f in ("e4m3", "e5m2", "int8")]
+    batch = qm.ProbeBatch(probes)
+    batch.launch()
+    torch.cuda.synchronize()
+    got = batch.results()
+    for i, r in enumerate(got):
+        assert r.device_error == 0 and _same(r, got[i % 3]) and _same(r, qm.qm_probe_layer(*probes[i])), i
