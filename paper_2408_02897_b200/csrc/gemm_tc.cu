@@ -1712,52 +1712,52 @@ tc_group_kernel(const __grid_constant__ Table tab) {
       bool ok = true;
       uint32_t it = 0;
       for (int k = 0; k < sh->n_walk && ok; ++k) {
-       const UnitInfo tw(sh->walk[k]);
-       const bool r_mn = MN && (tw.major & kUnitMnMajorR);  // (A comes from tensor memory, contraction-major always)
-       const uint32_t idesc_ref = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n) | (r_mn ? kIdescMnMajorB : 0u);
-       rd = tile_desc(r_mn, r_mn ? 2u * tw.half_n : 128u, 16u, 16u);
-       const int nb = tw.lp_blocks();
-       for (int j = 0; j < tw.n_tiles && ok; ++j, ++it) {
-        // the reference and denominator blocks come back when both epilogues have copied the
-        // previous tile's values out
-        ok = it == 0 || w.wait_warp(smem_u32(&sh->rd_empty), (it - 1) & 1);
-        if (!ok) break;
-        tc_fence_after();
-        for (int kb = 0; kb < tw.num_kb; ++kb) {
-          ok = wait_block();
+        const UnitInfo tw(sh->walk[k]);
+        const bool r_mn = MN && (tw.major & kUnitMnMajorR);  // (A comes from tensor memory, contraction-major always)
+        const uint32_t idesc_ref = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n) | (r_mn ? kIdescMnMajorB : 0u);
+        rd = tile_desc(r_mn, r_mn ? 2u * tw.half_n : 128u, 16u, 16u);
+        const int nb = tw.lp_blocks();
+        for (int j = 0; j < tw.n_tiles && ok; ++j, ++it) {
+          // the reference and denominator blocks come back when both epilogues have copied the
+          // previous tile's values out
+          ok = it == 0 || w.wait_warp(smem_u32(&sh->rd_empty), (it - 1) & 1);
           if (!ok) break;
-          issue_rd(tile_base + ring.s * C::kStageBytes, kb, idesc_ref, smem_u32(&sh->empty[ring.s]));
-          ring.next();
-        }
-        if (!ok) break;
-        tc_commit_pair(smem_u32(&sh->rd_full), lead);
-        for (int f = 0; f < tw.n_var && ok; ++f) {
-          const int b = (tw.n_var - 1 - f) & 1;
-          const uint32_t idesc = __shfl_sync(0xffffffffu, sh->var[tw.var_begin + f].idesc, 0);
-          const uint32_t flags = __shfl_sync(0xffffffffu, sh->var[tw.var_begin + f].flags, 0);
-          const bool is_i8 = flags & kVarI8, cl_mn = MN && (flags & kVarMnMajorL), cr_mn = MN && (flags & kVarMnMajorR);
-          cl = tile_desc(cl_mn, 128u, 32u, 16u);
-          cr = tile_desc(cr_mn, cr_mn ? tw.half_n : 128u, 32u, 16u);
-          // both epilogues have read what this accumulator held; the second one's columns have also
-          // been this tile's L, which the denominator MMAs must have finished with
-          const uint32_t uses = b ? lp_uses1 : lp_uses0;
-          ok = uses == 0 || w.wait_warp(smem_u32(&sh->lp_done[b]), (uses - 1) & 1);
-          if (ok && b == 1) ok = w.wait_warp(smem_u32(&sh->rd_full), it & 1);
           tc_fence_after();
-          const uint32_t td = tmem_base + C::kColLp + 128u * b;
-          for (int kb = 0; kb < nb && ok; ++kb) {
+          for (int kb = 0; kb < tw.num_kb; ++kb) {
             ok = wait_block();
             if (!ok) break;
-            const int steps = (tw.K - kb * C::kLpDepth + 31) / 32;          // of 32 codes; the rest of the block is fill
-            const uint32_t base = tile_base + ring.s * C::kStageBytes, bar = smem_u32(&sh->empty[ring.s]);
-            if (is_i8) issue_lp(std::integral_constant<int, kKindI8>{}, base, td, kb, steps, idesc, bar);
-            else issue_lp(std::integral_constant<int, kKindF8>{}, base, td, kb, steps, idesc, bar);
+            issue_rd(tile_base + ring.s * C::kStageBytes, kb, idesc_ref, smem_u32(&sh->empty[ring.s]));
             ring.next();
           }
-          if (ok) tc_commit_pair(smem_u32(&sh->lp_full[b]), lead);
-          if (b) ++lp_uses1; else ++lp_uses0;
+          if (!ok) break;
+          tc_commit_pair(smem_u32(&sh->rd_full), lead);
+          for (int f = 0; f < tw.n_var && ok; ++f) {
+            const int b = (tw.n_var - 1 - f) & 1;
+            const uint32_t idesc = __shfl_sync(0xffffffffu, sh->var[tw.var_begin + f].idesc, 0);
+            const uint32_t flags = __shfl_sync(0xffffffffu, sh->var[tw.var_begin + f].flags, 0);
+            const bool is_i8 = flags & kVarI8, cl_mn = MN && (flags & kVarMnMajorL), cr_mn = MN && (flags & kVarMnMajorR);
+            cl = tile_desc(cl_mn, 128u, 32u, 16u);
+            cr = tile_desc(cr_mn, cr_mn ? tw.half_n : 128u, 32u, 16u);
+            // both epilogues have read what this accumulator held; the second one's columns have also
+            // been this tile's L, which the denominator MMAs must have finished with
+            const uint32_t uses = b ? lp_uses1 : lp_uses0;
+            ok = uses == 0 || w.wait_warp(smem_u32(&sh->lp_done[b]), (uses - 1) & 1);
+            if (ok && b == 1) ok = w.wait_warp(smem_u32(&sh->rd_full), it & 1);
+            tc_fence_after();
+            const uint32_t td = tmem_base + C::kColLp + 128u * b;
+            for (int kb = 0; kb < nb && ok; ++kb) {
+              ok = wait_block();
+              if (!ok) break;
+              const int steps = (tw.K - kb * C::kLpDepth + 31) / 32;          // of 32 codes; the rest of the block is fill
+              const uint32_t base = tile_base + ring.s * C::kStageBytes, bar = smem_u32(&sh->empty[ring.s]);
+              if (is_i8) issue_lp(std::integral_constant<int, kKindI8>{}, base, td, kb, steps, idesc, bar);
+              else issue_lp(std::integral_constant<int, kKindF8>{}, base, td, kb, steps, idesc, bar);
+              ring.next();
+            }
+            if (ok) tc_commit_pair(smem_u32(&sh->lp_full[b]), lead);
+            if (b) ++lp_uses1; else ++lp_uses0;
+          }
         }
-       }
       }
     } else if (RW && warp >= 2) {
       // ---------------------------------------------------------- |R| (both CTAs)
@@ -1767,23 +1767,23 @@ tc_group_kernel(const __grid_constant__ Table tab) {
       Ring<kStages> ring;
       bool ok = true;
       for (int k = 0; k < sh->n_walk && ok; ++k)
-       for (UnitInfo tw(sh->walk[k]); tw.n_tiles > 0 && ok; --tw.n_tiles) {
-        for (int kb = 0; kb < tw.num_kb && ok; ++kb) {
-          ok = w.wait_warp(smem_u32(&sh->full[ring.s]), ring.parity);
-          if (!ok) break;
-          abs_r<64>(tile_base + ring.s * C::kStageBytes + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
-          fence_proxy_async();
-          __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(ready_leader + ring.s * 8u);
-          ring.next();
-        }
-        const int n_code_blocks = tw.n_var * tw.lp_blocks();     // only passed on
-        for (int kb = 0; kb < n_code_blocks && ok; ++kb) {
-          ok = w.wait_warp(smem_u32(&sh->full[ring.s]), ring.parity);
-          if (!ok) break;
-          if (lane == 0) mbar_arrive_cluster(ready_leader + ring.s * 8u);
-          ring.next();
-        }
+        for (UnitInfo tw(sh->walk[k]); tw.n_tiles > 0 && ok; --tw.n_tiles) {
+          for (int kb = 0; kb < tw.num_kb && ok; ++kb) {
+            ok = w.wait_warp(smem_u32(&sh->full[ring.s]), ring.parity);
+            if (!ok) break;
+            abs_r<64>(tile_base + ring.s * C::kStageBytes + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(ready_leader + ring.s * 8u);
+            ring.next();
+          }
+          const int n_code_blocks = tw.n_var * tw.lp_blocks();     // only passed on
+          for (int kb = 0; kb < n_code_blocks && ok; ++kb) {
+            ok = w.wait_warp(smem_u32(&sh->full[ring.s]), ring.parity);
+            if (!ok) break;
+            if (lane == 0) mbar_arrive_cluster(ready_leader + ring.s * 8u);
+            ring.next();
+          }
       }
     } else {
       begin();
@@ -1809,72 +1809,72 @@ tc_group_kernel(const __grid_constant__ Table tab) {
     bool lent = false;                             // the previous tile's variants have used the L columns
     bool ok = true;
     for (int k = 0; k < sh->n_walk && ok; ++k)
-     for (UnitInfo tw(sh->walk[k]); tw.n_tiles > 0 && ok; --tw.n_tiles, ++it) {
-      // the L columns are free once the previous tile's denominator is complete and whatever
-      // variants it put there have been read
-      if (it > 0) ok = w.wait_warp(smem_u32(&sh->rd_full), (it - 1) & 1);
-      if (ok && lent) ok = w.wait_warp(smem_u32(&sh->abs_free), abs_uses++ & 1);
-      lent = tw.n_var > 1;
-      const bool l_mn = MN && (tw.major & kUnitMnMajorL);
-      // a loop for each order of L: one loop with the choice inside cost the contraction-major one 7 %
-      auto convert = [&](auto mn) {
-        constexpr bool kMn = decltype(mn)::value;
-        for (int kb = 0; kb < tw.num_kb && ok; ++kb) {
-          const uint32_t s = ring.s;
-          ok = w.wait_warp(smem_u32(&sh->full[s]), ring.parity);
-          if (!ok) break;
-          const uint32_t base = tile_base + s * C::kStageBytes;
-          if (!RW) abs_r<128>(base + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
-          uint32_t a[32];
-          if constexpr (kMn) {
-            load_l_mn_major(base + C::kOffL, q, lane, a);
-          } else {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const uint4 v = lds128(base + C::kOffL + row_off + (((uint32_t)j ^ sw) << 4));
-              a[4 * j] = v.x; a[4 * j + 1] = v.y; a[4 * j + 2] = v.z; a[4 * j + 3] = v.w;
-            }
-          }
-          if (kb >= kTmemStages) {
-            // the tensor-memory columns were last read by the MMAs of the block kTmemStages before this one
-            const uint32_t sp = s >= (uint32_t)kTmemStages ? s - kTmemStages : s + kStages - kTmemStages;
-            const uint32_t pp = s >= (uint32_t)kTmemStages ? ring.parity : ring.parity ^ 1u;
-            ok = w.wait_warp(smem_u32(&sh->empty[sp]), pp);
+      for (UnitInfo tw(sh->walk[k]); tw.n_tiles > 0 && ok; --tw.n_tiles, ++it) {
+        // the L columns are free once the previous tile's denominator is complete and whatever
+        // variants it put there have been read
+        if (it > 0) ok = w.wait_warp(smem_u32(&sh->rd_full), (it - 1) & 1);
+        if (ok && lent) ok = w.wait_warp(smem_u32(&sh->abs_free), abs_uses++ & 1);
+        lent = tw.n_var > 1;
+        const bool l_mn = MN && (tw.major & kUnitMnMajorL);
+        // a loop for each order of L: one loop with the choice inside cost the contraction-major one 7 %
+        auto convert = [&](auto mn) {
+          constexpr bool kMn = decltype(mn)::value;
+          for (int kb = 0; kb < tw.num_kb && ok; ++kb) {
+            const uint32_t s = ring.s;
+            ok = w.wait_warp(smem_u32(&sh->full[s]), ring.parity);
             if (!ok) break;
-          }
-          tc_fence_after();
-          const uint32_t tcol = taddr + 64u * (uint32_t)(kb & (kTmemStages - 1));
-          if constexpr (kMn) {
-            tmem_st16x32(tcol, a);
-            tmem_st16x32(tcol + (16u << 16), a + 16);
-          } else {
-            tmem_st32(tcol, a);
-          }
+            const uint32_t base = tile_base + s * C::kStageBytes;
+            if (!RW) abs_r<128>(base + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
+            uint32_t a[32];
+            if constexpr (kMn) {
+              load_l_mn_major(base + C::kOffL, q, lane, a);
+            } else {
 #pragma unroll
-          for (int j = 0; j < 32; ++j) a[j] &= m;
-          if constexpr (kMn) {
-            tmem_st16x32(tcol + 32u, a);
-            tmem_st16x32(tcol + 32u + (16u << 16), a + 16);
-          } else {
-            tmem_st32(tcol + 32u, a);
+              for (int j = 0; j < 8; ++j) {
+                const uint4 v = lds128(base + C::kOffL + row_off + (((uint32_t)j ^ sw) << 4));
+                a[4 * j] = v.x; a[4 * j + 1] = v.y; a[4 * j + 2] = v.z; a[4 * j + 3] = v.w;
+              }
+            }
+            if (kb >= kTmemStages) {
+              // the tensor-memory columns were last read by the MMAs of the block kTmemStages before this one
+              const uint32_t sp = s >= (uint32_t)kTmemStages ? s - kTmemStages : s + kStages - kTmemStages;
+              const uint32_t pp = s >= (uint32_t)kTmemStages ? ring.parity : ring.parity ^ 1u;
+              ok = w.wait_warp(smem_u32(&sh->empty[sp]), pp);
+              if (!ok) break;
+            }
+            tc_fence_after();
+            const uint32_t tcol = taddr + 64u * (uint32_t)(kb & (kTmemStages - 1));
+            if constexpr (kMn) {
+              tmem_st16x32(tcol, a);
+              tmem_st16x32(tcol + (16u << 16), a + 16);
+            } else {
+              tmem_st32(tcol, a);
+            }
+#pragma unroll
+            for (int j = 0; j < 32; ++j) a[j] &= m;
+            if constexpr (kMn) {
+              tmem_st16x32(tcol + 32u, a);
+              tmem_st16x32(tcol + 32u + (16u << 16), a + 16);
+            } else {
+              tmem_st32(tcol + 32u, a);
+            }
+            if (!RW) fence_proxy_async();
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(ready_leader + s * 8u);
+            ring.next();
           }
-          if (!RW) fence_proxy_async();
-          asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(ready_leader + s * 8u);
+        };
+        if (l_mn) convert(std::bool_constant<MN>{}); else convert(std::false_type{});
+        // blocks of codes: only passed on
+        const int n_code_blocks = tw.n_var * tw.lp_blocks();
+        for (int kb = 0; kb < n_code_blocks && ok; ++kb) {
+          ok = w.wait_warp(smem_u32(&sh->full[ring.s]), ring.parity);
+          if (!ok) break;
+          if (lane == 0) mbar_arrive_cluster(ready_leader + ring.s * 8u);
           ring.next();
         }
-      };
-      if (l_mn) convert(std::bool_constant<MN>{}); else convert(std::false_type{});
-      // blocks of codes: only passed on
-      const int n_code_blocks = tw.n_var * tw.lp_blocks();
-      for (int kb = 0; kb < n_code_blocks && ok; ++kb) {
-        ok = w.wait_warp(smem_u32(&sh->full[ring.s]), ring.parity);
-        if (!ok) break;
-        if (lane == 0) mbar_arrive_cluster(ready_leader + ring.s * 8u);
-        ring.next();
-      }
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
@@ -1924,142 +1924,142 @@ tc_group_kernel(const __grid_constant__ Table tab) {
     begin();
     uint32_t it = 0;
     for (int k = 0; k < sh->n_walk && !ended; ++k) {
-     const UnitInfo tw(sh->walk[k]);
-     const int pi = tw.unit, n_var = tw.n_var, v0 = tw.var_begin;
-     met |= ((1ull << n_var) - 1ull) << v0;
-     const int pM = tab.u[pi].M, pN = tab.u[pi].N;  // below 2^31 (its tensor maps require it)
-     for (int v = 0; v < n_var; ++v)
-       if (lane < 16) { sh->sums[v][ew][lane] = make_double2(0.0, 0.0); sh->maxima[v][ew][lane] = 0.f; }
-     if (et < n_var) {                              // read after the barrier below
-       const uint32_t flags = sh->var[v0 + et].flags;
-       sh->dl_tensor[et] = flags & kVarScalePerRow ? 1.f : __ldg(tab.v[v0 + et].dl);
-       sh->dr_tensor[et] = flags & kVarScalePerCol ? 1.f : __ldg(tab.v[v0 + et].dr);
-     }
-     for (int j = 0; j < tw.n_tiles; ++j, ++it) {
-      const TileCoord tc = pair_tile(sh->walk[k], j, num_pairs);
-      for (int v = 0; v < n_var; ++v) {
-        if ((sh->var[v0 + v].flags & kVarScalePerCol) && et < kBlockN) {
-          const int col = tc.n_tile * kBlockN + et;
-          sh->delta_r[it & 1][v][et] = col < pN ? __ldg(tab.v[v0 + v].dr + (int64_t)tc.b * pN + col) : 0.f;
-        }
+      const UnitInfo tw(sh->walk[k]);
+      const int pi = tw.unit, n_var = tw.n_var, v0 = tw.var_begin;
+      met |= ((1ull << n_var) - 1ull) << v0;
+      const int pM = tab.u[pi].M, pN = tab.u[pi].N;  // below 2^31 (its tensor maps require it)
+      for (int v = 0; v < n_var; ++v)
+        if (lane < 16) { sh->sums[v][ew][lane] = make_double2(0.0, 0.0); sh->maxima[v][ew][lane] = 0.f; }
+      if (et < n_var) {                              // read after the barrier below
+        const uint32_t flags = sh->var[v0 + et].flags;
+        sh->dl_tensor[et] = flags & kVarScalePerRow ? 1.f : __ldg(tab.v[v0 + et].dl);
+        sh->dr_tensor[et] = flags & kVarScalePerCol ? 1.f : __ldg(tab.v[v0 + et].dr);
       }
-      const int row = tc.m_tile * kPairM + (int)rank * kBlockM + q * 32 + lane;
-      const bool row_ok = row < pM;
-      // the two warps of a lane quarter split the tile's columns: 64 each, or 32 each where the
-      // tile is 64 wide (outputs at most 64 wide)
-      const bool narrow = tw.half_n < 64;
-      const int cw = narrow ? 32 : 64, cbase = h * cw;
-      const int colw = tc.n_tile * kBlockN + cbase;                  // first column of this warp
-      const int live = pN - colw < cw ? pN - colw : cw;              // its columns that exist; <= 0: none
+      for (int j = 0; j < tw.n_tiles; ++j, ++it) {
+        const TileCoord tc = pair_tile(sh->walk[k], j, num_pairs);
+        for (int v = 0; v < n_var; ++v) {
+          if ((sh->var[v0 + v].flags & kVarScalePerCol) && et < kBlockN) {
+            const int col = tc.n_tile * kBlockN + et;
+            sh->delta_r[it & 1][v][et] = col < pN ? __ldg(tab.v[v0 + v].dr + (int64_t)tc.b * pN + col) : 0.f;
+          }
+        }
+        const int row = tc.m_tile * kPairM + (int)rank * kBlockM + q * 32 + lane;
+        const bool row_ok = row < pM;
+        // the two warps of a lane quarter split the tile's columns: 64 each, or 32 each where the
+        // tile is 64 wide (outputs at most 64 wide)
+        const bool narrow = tw.half_n < 64;
+        const int cw = narrow ? 32 : 64, cbase = h * cw;
+        const int colw = tc.n_tile * kBlockN + cbase;                  // first column of this warp
+        const int live = pN - colw < cw ? pN - colw : cw;              // its columns that exist; <= 0: none
 
-      const bool ok = !dead && w.wait(smem_u32(&sh->rd_full), it & 1);
-      // one barrier publishes the scales and makes the give-up decision uniform over the epilogue
-      if (epi_barrier_any(!ok)) { ended = true; break; }
-      tc_fence_after();
-      uint32_t rc[64], rd[64];
-      tmem_ld32(lane_addr + C::kColRef + cbase, *reinterpret_cast<uint32_t(*)[32]>(&rc[0]));
-      tmem_ld32(lane_addr + C::kColDen + cbase, *reinterpret_cast<uint32_t(*)[32]>(&rd[0]));
-      if (!narrow) {
-        tmem_ld32(lane_addr + C::kColRef + cbase + 32, *reinterpret_cast<uint32_t(*)[32]>(&rc[32]));
-        tmem_ld32(lane_addr + C::kColDen + cbase + 32, *reinterpret_cast<uint32_t(*)[32]>(&rd[32]));
-      }
-      tmem_ld_wait();
-      // in registers: the MMA warp may start the next tile's reference and denominator as soon as
-      // it is through with this tile's variants
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(rd_empty_leader);
-      // sums of C^2 and D^2, and D replaced by its reciprocal (all under the first 8-bit product).
-      // D == 0 implies C == Q == 0, so clamping the divisor keeps BE = 0 there without a branch.
-      {
-        uint64_t r22 = 0ull, n22 = 0ull;
-        auto prepare = [&](int j0) {
-#pragma unroll
-          for (int j = 0; j < 32; j += 2) {
-            const uint64_t cv2 = pack2(__uint_as_float(rc[j0 + j]), __uint_as_float(rc[j0 + j + 1]));
-            const float d0 = __uint_as_float(rd[j0 + j]), d1 = __uint_as_float(rd[j0 + j + 1]);
-            const uint64_t dd2 = pack2(d0, d1);
-            r22 = fma2(cv2, cv2, r22);
-            n22 = fma2(dd2, dd2, n22);
-            rd[j0 + j] = __float_as_uint(rcp_approx(fmaxf(d0, 1e-37f)));
-            rd[j0 + j + 1] = __float_as_uint(rcp_approx(fmaxf(d1, 1e-37f)));
-          }
-        };
-        if (live < cw) {                                 // ragged edge: columns beyond the matrix count as zeros
-#pragma unroll
-          for (int k = 0; k < 64; ++k)
-            if (k >= live) { rc[k] = 0u; rd[k] = 0u; }
-        }
-        prepare(0);
-        if (!narrow) prepare(32);
-        float x0, x1;
-        unpack2(r22, x0, x1);
-        const double r2d = (double)x0 + (double)x1;
-        unpack2(n22, x0, x1);
-        const double n2d = (double)x0 + (double)x1;
-        if (row_ok) {
-          acc_r2 += r2d;
-          acc_n2 += n2d;
-          for (int v = 0; v < n_var; ++v) {
-            if (!(sh->var[v0 + v].flags & kVarRowStats)) continue;       // the optional per-row check output
-            double* const rs = tab.v[v0 + v].row_stats + ((int64_t)tc.b * pM + row) * 5;
-            atomicAdd(rs + 3, r2d);
-            atomicAdd(rs + 4, n2d);
-          }
-        }
-      }
-      for (int f = 0; f < n_var; ++f) {
-        const int b = (n_var - 1 - f) & 1;
-        const uint32_t flags = sh->var[v0 + f].flags;
-        const bool per_col = (flags & kVarScalePerCol) != 0, is_i8 = (flags & kVarI8) != 0;
-        float dlv = sh->dl_tensor[f];
-        if (flags & kVarScalePerRow) dlv = row_ok ? __ldg(tab.v[v0 + f].dl + (int64_t)tc.b * pM + row) : 0.f;
-        const float kd = per_col ? -dlv : -dlv * sh->dr_tensor[f];
-        if (!w.wait_warp(smem_u32(&sh->lp_full[b]), (lp_parity >> b) & 1u)) { dead = true; break; }
-        lp_parity ^= 1u << b;
+        const bool ok = !dead && w.wait(smem_u32(&sh->rd_full), it & 1);
+        // one barrier publishes the scales and makes the give-up decision uniform over the epilogue
+        if (epi_barrier_any(!ok)) { ended = true; break; }
         tc_fence_after();
-        const uint32_t taddr = lane_addr + C::kColLp + 128u * b + cbase;
-        StatsV st{0.f, 0.f, 0.f, 0ull};
-        auto release = [&]() {
-          // read to the end: the MMA warp may overwrite it and, after the tile's last use of the second
-          // accumulator (once per tile, or the converters' wait could miss a phase of the barrier), this
-          // CTA's converters may.  Every warp arrives exactly once per use.
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) {
-            mbar_arrive_cluster(lp_done_leader + 8u * b);
-            if (f == n_var - 2) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&sh->abs_free)) : "memory");
+        uint32_t rc[64], rd[64];
+        tmem_ld32(lane_addr + C::kColRef + cbase, *reinterpret_cast<uint32_t(*)[32]>(&rc[0]));
+        tmem_ld32(lane_addr + C::kColDen + cbase, *reinterpret_cast<uint32_t(*)[32]>(&rd[0]));
+        if (!narrow) {
+          tmem_ld32(lane_addr + C::kColRef + cbase + 32, *reinterpret_cast<uint32_t(*)[32]>(&rc[32]));
+          tmem_ld32(lane_addr + C::kColDen + cbase + 32, *reinterpret_cast<uint32_t(*)[32]>(&rd[32]));
+        }
+        tmem_ld_wait();
+        // in registers: the MMA warp may start the next tile's reference and denominator as soon as
+        // it is through with this tile's variants
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(rd_empty_leader);
+        // sums of C^2 and D^2, and D replaced by its reciprocal (all under the first 8-bit product).
+        // D == 0 implies C == Q == 0, so clamping the divisor keeps BE = 0 there without a branch.
+        {
+          uint64_t r22 = 0ull, n22 = 0ull;
+          auto prepare = [&](int j0) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 2) {
+              const uint64_t cv2 = pack2(__uint_as_float(rc[j0 + j]), __uint_as_float(rc[j0 + j + 1]));
+              const float d0 = __uint_as_float(rd[j0 + j]), d1 = __uint_as_float(rd[j0 + j + 1]);
+              const uint64_t dd2 = pack2(d0, d1);
+              r22 = fma2(cv2, cv2, r22);
+              n22 = fma2(dd2, dd2, n22);
+              rd[j0 + j] = __float_as_uint(rcp_approx(fmaxf(d0, 1e-37f)));
+              rd[j0 + j + 1] = __float_as_uint(rcp_approx(fmaxf(d1, 1e-37f)));
+            }
+          };
+          if (live < cw) {                                 // ragged edge: columns beyond the matrix count as zeros
+#pragma unroll
+            for (int k = 0; k < 64; ++k)
+              if (k >= live) { rc[k] = 0u; rd[k] = 0u; }
           }
-        };
-        if (per_col) eval_variant<true>(taddr, rc, rd, live, is_i8, pack2(kd, kd), sh->delta_r[it & 1][f] + cbase, st, release);
-        else eval_variant<false>(taddr, rc, rd, live, is_i8, pack2(kd, kd), sh->delta_r[0][0], st, release);
-        double be = 0.0, d2 = 0.0;
-        float mx = 0.f;
-        if (row_ok) {
+          prepare(0);
+          if (!narrow) prepare(32);
           float x0, x1;
-          unpack2(st.d2, x0, x1);
-          be = (double)st.be0 + (double)st.be1;
-          d2 = (double)x0 + (double)x1;
-          mx = st.mx;
-          if (flags & kVarRowStats) {
-            double* const rs = tab.v[v0 + f].row_stats + ((int64_t)tc.b * pM + row) * 5;
-            atomicAdd(rs + 0, be);
-            atomicMax(reinterpret_cast<unsigned long long*>(rs + 1), (unsigned long long)__double_as_longlong((double)mx));
-            atomicAdd(rs + 2, d2);
+          unpack2(r22, x0, x1);
+          const double r2d = (double)x0 + (double)x1;
+          unpack2(n22, x0, x1);
+          const double n2d = (double)x0 + (double)x1;
+          if (row_ok) {
+            acc_r2 += r2d;
+            acc_n2 += n2d;
+            for (int v = 0; v < n_var; ++v) {
+              if (!(sh->var[v0 + v].flags & kVarRowStats)) continue;       // the optional per-row check output
+              double* const rs = tab.v[v0 + v].row_stats + ((int64_t)tc.b * pM + row) * 5;
+              atomicAdd(rs + 3, r2d);
+              atomicAdd(rs + 4, n2d);
+            }
           }
         }
-        be += __shfl_xor_sync(0xffffffffu, be, 16);
-        d2 += __shfl_xor_sync(0xffffffffu, d2, 16);
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
-        if (lane < 16) {
-          double2& a = sh->sums[f][ew][lane];
-          a.x += be;
-          a.y += d2;
-          sh->maxima[f][ew][lane] = fmaxf(sh->maxima[f][ew][lane], mx);
+        for (int f = 0; f < n_var; ++f) {
+          const int b = (n_var - 1 - f) & 1;
+          const uint32_t flags = sh->var[v0 + f].flags;
+          const bool per_col = (flags & kVarScalePerCol) != 0, is_i8 = (flags & kVarI8) != 0;
+          float dlv = sh->dl_tensor[f];
+          if (flags & kVarScalePerRow) dlv = row_ok ? __ldg(tab.v[v0 + f].dl + (int64_t)tc.b * pM + row) : 0.f;
+          const float kd = per_col ? -dlv : -dlv * sh->dr_tensor[f];
+          if (!w.wait_warp(smem_u32(&sh->lp_full[b]), (lp_parity >> b) & 1u)) { dead = true; break; }
+          lp_parity ^= 1u << b;
+          tc_fence_after();
+          const uint32_t taddr = lane_addr + C::kColLp + 128u * b + cbase;
+          StatsV st{0.f, 0.f, 0.f, 0ull};
+          auto release = [&]() {
+            // read to the end: the MMA warp may overwrite it and, after the tile's last use of the second
+            // accumulator (once per tile, or the converters' wait could miss a phase of the barrier), this
+            // CTA's converters may.  Every warp arrives exactly once per use.
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+              mbar_arrive_cluster(lp_done_leader + 8u * b);
+              if (f == n_var - 2) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&sh->abs_free)) : "memory");
+            }
+          };
+          if (per_col) eval_variant<true>(taddr, rc, rd, live, is_i8, pack2(kd, kd), sh->delta_r[it & 1][f] + cbase, st, release);
+          else eval_variant<false>(taddr, rc, rd, live, is_i8, pack2(kd, kd), sh->delta_r[0][0], st, release);
+          double be = 0.0, d2 = 0.0;
+          float mx = 0.f;
+          if (row_ok) {
+            float x0, x1;
+            unpack2(st.d2, x0, x1);
+            be = (double)st.be0 + (double)st.be1;
+            d2 = (double)x0 + (double)x1;
+            mx = st.mx;
+            if (flags & kVarRowStats) {
+              double* const rs = tab.v[v0 + f].row_stats + ((int64_t)tc.b * pM + row) * 5;
+              atomicAdd(rs + 0, be);
+              atomicMax(reinterpret_cast<unsigned long long*>(rs + 1), (unsigned long long)__double_as_longlong((double)mx));
+              atomicAdd(rs + 2, d2);
+            }
+          }
+          be += __shfl_xor_sync(0xffffffffu, be, 16);
+          d2 += __shfl_xor_sync(0xffffffffu, d2, 16);
+          mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+          if (lane < 16) {
+            double2& a = sh->sums[f][ew][lane];
+            a.x += be;
+            a.y += d2;
+            sh->maxima[f][ew][lane] = fmaxf(sh->maxima[f][ew][lane], mx);
+          }
         }
       }
-     }
-     flush(n_var, v0);
+      flush(n_var, v0);
     }
     // the records of the probes this CTA never met are zero
     for (int i = et; i < kPartialDoubles * tab.n_var; i += 256) {
@@ -2317,54 +2317,54 @@ tc_side_kernel(const __grid_constant__ Table tab) {
       uint32_t g = 0, it = 0;
       bool ok = true;
       for (int k = 0; k < sh->n_walk && ok; ++k) {
-       const UnitInfo tw(sh->walk[k]);
-       const int pi = tw.unit;
-       const int num_kb = tw.num_kb;
-       const uint32_t idesc_lp = __shfl_sync(0xffffffffu, sh->var[pi].idesc, 0);
-       const uint32_t flags = __shfl_sync(0xffffffffu, sh->var[pi].flags, 0);
-       const bool is_i8 = flags & kVarI8;
-       const bool l_mn = MN && (tw.major & kUnitMnMajorL), r_mn = MN && (tw.major & kUnitMnMajorR);
-       const bool cl_mn = MN && (flags & kVarMnMajorL), cr_mn = MN && (flags & kVarMnMajorR);
-       // |L| comes from tensor memory, contraction-major always
-       idesc_den = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n) | (r_mn ? kIdescMnMajorB : 0u);
-       idesc_ref = idesc_den | (l_mn ? kIdescMnMajorA : 0u);
-       ld = tile_desc(l_mn, 128u, 16u, kABf16 / 2);
-       rd = tile_desc(r_mn, r_mn ? 2u * tw.half_n : 128u, 16u, 16u);
-       cl = tile_desc(cl_mn, cl_mn ? 128u : 64u, 32u, 16u);
-       cr = tile_desc(cr_mn, cr_mn ? tw.half_n : 64u, 32u, 16u);
-       for (int j = 0; j < tw.n_tiles && ok; ++j, ++it) {
-        // the reference and denominator blocks come back when both epilogues have copied the
-        // previous tile's values out; the 8-bit block when they have finished that tile
-        ok = it == 0 || w.wait_warp(smem_u32(&sh->tmem_empty), (it - 1) & 1);
-        if (!ok) break;
-        tc_fence_after();
-        const int n_ahead = num_kb < kAbs ? num_kb : kAbs;
-        Ring<kStages> ahead = ring;
-        for (int i = 0; i < n_ahead && ok; ++i) {
-          ok = wait_stage(ahead);
-          if (ok) issue_ref_den(ahead.s, g + i, i);
-          ahead.next();
-        }
-        if (!ok) break;
-        ok = it == 0 || w.wait_warp(smem_u32(&sh->lp_done), (it - 1) & 1);
-        if (!ok) break;
-        tc_fence_after();
-        int kb = 0;
-        for (; kb < n_ahead; ++kb, ++g) {
-          issue_lp(ring.s, kb, is_i8, idesc_lp);
-          tc_commit_pair(smem_u32(&sh->empty[ring.s]), lead);
-          ring.next();
-        }
-        for (; kb < num_kb && ok; ++kb, ++g) {
-          ok = wait_stage(ring);
+        const UnitInfo tw(sh->walk[k]);
+        const int pi = tw.unit;
+        const int num_kb = tw.num_kb;
+        const uint32_t idesc_lp = __shfl_sync(0xffffffffu, sh->var[pi].idesc, 0);
+        const uint32_t flags = __shfl_sync(0xffffffffu, sh->var[pi].flags, 0);
+        const bool is_i8 = flags & kVarI8;
+        const bool l_mn = MN && (tw.major & kUnitMnMajorL), r_mn = MN && (tw.major & kUnitMnMajorR);
+        const bool cl_mn = MN && (flags & kVarMnMajorL), cr_mn = MN && (flags & kVarMnMajorR);
+        // |L| comes from tensor memory, contraction-major always
+        idesc_den = make_idesc(1, 1, 1, kPairM, 2 * tw.half_n) | (r_mn ? kIdescMnMajorB : 0u);
+        idesc_ref = idesc_den | (l_mn ? kIdescMnMajorA : 0u);
+        ld = tile_desc(l_mn, 128u, 16u, kABf16 / 2);
+        rd = tile_desc(r_mn, r_mn ? 2u * tw.half_n : 128u, 16u, 16u);
+        cl = tile_desc(cl_mn, cl_mn ? 128u : 64u, 32u, 16u);
+        cr = tile_desc(cr_mn, cr_mn ? tw.half_n : 64u, 32u, 16u);
+        for (int j = 0; j < tw.n_tiles && ok; ++j, ++it) {
+          // the reference and denominator blocks come back when both epilogues have copied the
+          // previous tile's values out; the 8-bit block when they have finished that tile
+          ok = it == 0 || w.wait_warp(smem_u32(&sh->tmem_empty), (it - 1) & 1);
           if (!ok) break;
-          issue_ref_den(ring.s, g, kb);
-          issue_lp(ring.s, kb, is_i8, idesc_lp);
-          tc_commit_pair(smem_u32(&sh->empty[ring.s]), lead);             // frees the k-block in both CTAs
-          ring.next();
+          tc_fence_after();
+          const int n_ahead = num_kb < kAbs ? num_kb : kAbs;
+          Ring<kStages> ahead = ring;
+          for (int i = 0; i < n_ahead && ok; ++i) {
+            ok = wait_stage(ahead);
+            if (ok) issue_ref_den(ahead.s, g + i, i);
+            ahead.next();
+          }
+          if (!ok) break;
+          ok = it == 0 || w.wait_warp(smem_u32(&sh->lp_done), (it - 1) & 1);
+          if (!ok) break;
+          tc_fence_after();
+          int kb = 0;
+          for (; kb < n_ahead; ++kb, ++g) {
+            issue_lp(ring.s, kb, is_i8, idesc_lp);
+            tc_commit_pair(smem_u32(&sh->empty[ring.s]), lead);
+            ring.next();
+          }
+          for (; kb < num_kb && ok; ++kb, ++g) {
+            ok = wait_stage(ring);
+            if (!ok) break;
+            issue_ref_den(ring.s, g, kb);
+            issue_lp(ring.s, kb, is_i8, idesc_lp);
+            tc_commit_pair(smem_u32(&sh->empty[ring.s]), lead);             // frees the k-block in both CTAs
+            ring.next();
+          }
+          if (ok) tc_commit_pair(smem_u32(&sh->tmem_full), lead);           // this tile's accumulators are complete
         }
-        if (ok) tc_commit_pair(smem_u32(&sh->tmem_full), lead);           // this tile's accumulators are complete
-       }
       }
     } else if (RW && warp >= 2) {
       // ---------------------------------------------------------- |R| (both CTAs)
@@ -2374,16 +2374,16 @@ tc_side_kernel(const __grid_constant__ Table tab) {
       bool ok = true;
       Ring<kStages> ring;
       for (int k = 0; k < sh->n_walk && ok; ++k)
-       for (UnitInfo tw(sh->walk[k]); tw.n_tiles > 0 && ok; --tw.n_tiles) {
-        for (int kb = 0; kb < tw.num_kb; ++kb) {
-          ok = w.wait_warp(smem_u32(&sh->full[ring.s]), ring.parity);
-          if (!ok) break;
-          abs_r<64>(tile_base + ring.s * C::kStageBytes + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
-          fence_proxy_async();
-          __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(ready_leader + ring.s * 8u);
-          ring.next();
-        }
+        for (UnitInfo tw(sh->walk[k]); tw.n_tiles > 0 && ok; --tw.n_tiles) {
+          for (int kb = 0; kb < tw.num_kb; ++kb) {
+            ok = w.wait_warp(smem_u32(&sh->full[ring.s]), ring.parity);
+            if (!ok) break;
+            abs_r<64>(tile_base + ring.s * C::kStageBytes + C::kOffR, C::kOffRa - C::kOffR, tw.half_n * 8, t);
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(ready_leader + ring.s * 8u);
+            ring.next();
+          }
       }
     } else {
       begin();
@@ -2489,91 +2489,91 @@ tc_side_kernel(const __grid_constant__ Table tab) {
     uint32_t it = 0;
     bool dead = false;                             // a wait ran out
     for (int k = 0; k < sh->n_walk && !dead; ++k) {
-     const UnitInfo tw(sh->walk[k]);
-     const int pi = tw.unit;
-     met |= 1u << pi;
-     const uint32_t flags = sh->var[pi].flags;
-     const bool per_col = flags & kVarScalePerCol, pc_l = flags & kVarScalePerRow, is_i8 = flags & kVarI8, narrow = tw.half_n < 64;
-     const int pM = tab.u[pi].M, pN = tab.u[pi].N;  // below 2^31 (its tensor maps require it)
-     const float dr_tensor = per_col ? 1.f : __ldg(tab.v[pi].dr), dl_tensor = pc_l ? 0.f : __ldg(tab.v[pi].dl);
-     for (int j = 0; j < tw.n_tiles; ++j, ++it) {
-      const TileCoord tc = pair_tile(sh->walk[k], j, num_pairs);
-      float* dr_s = sh->delta_r[it & 1];
-      if (per_col && et < kBlockN) {
-        const int col = tc.n_tile * kBlockN + et;
-        dr_s[et] = col < pN ? __ldg(tab.v[pi].dr + (int64_t)tc.b * pN + col) : 0.f;
-      }
-      const int row = tc.m_tile * kPairM + (int)rank * kBlockM + q * 32 + lane;
-      const bool row_ok = row < pM;
-      float dlv = dl_tensor;
-      if (pc_l) dlv = row_ok ? __ldg(tab.v[pi].dl + (int64_t)tc.b * pM + row) : 0.f;
-      // the two warps of a lane quarter split the tile's columns: 64 each, or 32 each where the
-      // tile is 64 wide (outputs at most 64 wide)
-      const int cw = narrow ? 32 : 64, cbase = h * cw;
-      const int colw = tc.n_tile * kBlockN + cbase;                  // first column of this warp
+      const UnitInfo tw(sh->walk[k]);
+      const int pi = tw.unit;
+      met |= 1u << pi;
+      const uint32_t flags = sh->var[pi].flags;
+      const bool per_col = flags & kVarScalePerCol, pc_l = flags & kVarScalePerRow, is_i8 = flags & kVarI8, narrow = tw.half_n < 64;
+      const int pM = tab.u[pi].M, pN = tab.u[pi].N;  // below 2^31 (its tensor maps require it)
+      const float dr_tensor = per_col ? 1.f : __ldg(tab.v[pi].dr), dl_tensor = pc_l ? 0.f : __ldg(tab.v[pi].dl);
+      for (int j = 0; j < tw.n_tiles; ++j, ++it) {
+        const TileCoord tc = pair_tile(sh->walk[k], j, num_pairs);
+        float* dr_s = sh->delta_r[it & 1];
+        if (per_col && et < kBlockN) {
+          const int col = tc.n_tile * kBlockN + et;
+          dr_s[et] = col < pN ? __ldg(tab.v[pi].dr + (int64_t)tc.b * pN + col) : 0.f;
+        }
+        const int row = tc.m_tile * kPairM + (int)rank * kBlockM + q * 32 + lane;
+        const bool row_ok = row < pM;
+        float dlv = dl_tensor;
+        if (pc_l) dlv = row_ok ? __ldg(tab.v[pi].dl + (int64_t)tc.b * pM + row) : 0.f;
+        // the two warps of a lane quarter split the tile's columns: 64 each, or 32 each where the
+        // tile is 64 wide (outputs at most 64 wide)
+        const int cw = narrow ? 32 : 64, cbase = h * cw;
+        const int colw = tc.n_tile * kBlockN + cbase;                  // first column of this warp
 
-      const bool ok = w.wait(smem_u32(&sh->tmem_full), it & 1);
-      // one barrier publishes delta_r and makes the give-up decision uniform over the epilogue
-      if (epi_barrier_any(!ok)) { dead = true; break; }
-      tc_fence_after();
-      // live = columns of this warp that exist in the matrix
-      const int live = pN - colw < cw ? pN - colw : cw;          // <= 0: none
-      const uint32_t lp_addr = lane_addr + C::kColLp + cbase;
-      const uint32_t lp_done_leader = map_to_cta(smem_u32(&sh->lp_done), 0);
-      const float* const drc = dr_s + cbase;
-      uint32_t rc[64], rd[64], rq0[16];
-      tmem_ld32(lane_addr + C::kColRef + cbase, *reinterpret_cast<uint32_t(*)[32]>(&rc[0]));
-      tmem_ld32(lane_addr + C::kColDen + cbase, *reinterpret_cast<uint32_t(*)[32]>(&rd[0]));
-      if (!narrow) {
-        tmem_ld32(lane_addr + C::kColRef + cbase + 32, *reinterpret_cast<uint32_t(*)[32]>(&rc[32]));
-        tmem_ld32(lane_addr + C::kColDen + cbase + 32, *reinterpret_cast<uint32_t(*)[32]>(&rd[32]));
-      }
-      if (live > 0) tmem_ld16(lp_addr, rq0);
-      tmem_ld_wait();
-      // The reference and denominator blocks are in registers: the MMA lane may start the next
-      // tile's bf16 MMAs.  The 8-bit block follows in two steps, its first 16 columns with the
-      // loads above and the rest once the first chunk has been evaluated (which frees the
-      // registers the rest is read into); then the MMA lane may start the next tile's 8-bit MMAs as well, while the
-      // remaining chunks are still being evaluated.  Every warp arrives on each barrier exactly
-      // once per tile.
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) {
-        mbar_arrive_cluster(tmem_empty_leader);
-        if (live <= 16) mbar_arrive_cluster(lp_done_leader);      // nothing further to read
-      }
-      StatsG st{0.f, 0.f, 0ull, 0ull, 0ull, 0.f};
-      const float kd = -dlv * dr_tensor;
-      const uint64_t kd2 = per_col ? pack2(-dlv, -dlv) : pack2(kd, kd);
-      if (live > 0) stats_chunk<0>(rc, rd, rq0, live, is_i8, per_col, kd2, drc, st);
-      if (live > 16) {
-        // chunk 1 into the first chunk's registers, chunks 2 and 3 into those of the first
-        // chunk's reference and denominator values
-        uint32_t(&rq2)[16] = *reinterpret_cast<uint32_t(*)[16]>(&rc[0]);
-        uint32_t(&rq3)[16] = *reinterpret_cast<uint32_t(*)[16]>(&rd[0]);
-        tmem_ld16(lp_addr + 16, rq0);
-        if (live > 32) tmem_ld16(lp_addr + 32, rq2);
-        if (live > 48) tmem_ld16(lp_addr + 48, rq3);
+        const bool ok = w.wait(smem_u32(&sh->tmem_full), it & 1);
+        // one barrier publishes delta_r and makes the give-up decision uniform over the epilogue
+        if (epi_barrier_any(!ok)) { dead = true; break; }
+        tc_fence_after();
+        // live = columns of this warp that exist in the matrix
+        const int live = pN - colw < cw ? pN - colw : cw;          // <= 0: none
+        const uint32_t lp_addr = lane_addr + C::kColLp + cbase;
+        const uint32_t lp_done_leader = map_to_cta(smem_u32(&sh->lp_done), 0);
+        const float* const drc = dr_s + cbase;
+        uint32_t rc[64], rd[64], rq0[16];
+        tmem_ld32(lane_addr + C::kColRef + cbase, *reinterpret_cast<uint32_t(*)[32]>(&rc[0]));
+        tmem_ld32(lane_addr + C::kColDen + cbase, *reinterpret_cast<uint32_t(*)[32]>(&rd[0]));
+        if (!narrow) {
+          tmem_ld32(lane_addr + C::kColRef + cbase + 32, *reinterpret_cast<uint32_t(*)[32]>(&rc[32]));
+          tmem_ld32(lane_addr + C::kColDen + cbase + 32, *reinterpret_cast<uint32_t(*)[32]>(&rd[32]));
+        }
+        if (live > 0) tmem_ld16(lp_addr, rq0);
         tmem_ld_wait();
+        // The reference and denominator blocks are in registers: the MMA lane may start the next
+        // tile's bf16 MMAs.  The 8-bit block follows in two steps, its first 16 columns with the
+        // loads above and the rest once the first chunk has been evaluated (which frees the
+        // registers the rest is read into); then the MMA lane may start the next tile's 8-bit MMAs as well, while the
+        // remaining chunks are still being evaluated.  Every warp arrives on each barrier exactly
+        // once per tile.
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(lp_done_leader);
-        stats_chunk<1>(rc, rd, rq0, live - 16, is_i8, per_col, kd2, drc, st);
-        if (live > 32) stats_chunk<2>(rc, rd, rq2, live - 32, is_i8, per_col, kd2, drc, st);
-        if (live > 48) stats_chunk<3>(rc, rd, rq3, live - 48, is_i8, per_col, kd2, drc, st);
+        if (lane == 0) {
+          mbar_arrive_cluster(tmem_empty_leader);
+          if (live <= 16) mbar_arrive_cluster(lp_done_leader);      // nothing further to read
+        }
+        StatsG st{0.f, 0.f, 0ull, 0ull, 0ull, 0.f};
+        const float kd = -dlv * dr_tensor;
+        const uint64_t kd2 = per_col ? pack2(-dlv, -dlv) : pack2(kd, kd);
+        if (live > 0) stats_chunk<0>(rc, rd, rq0, live, is_i8, per_col, kd2, drc, st);
+        if (live > 16) {
+          // chunk 1 into the first chunk's registers, chunks 2 and 3 into those of the first
+          // chunk's reference and denominator values
+          uint32_t(&rq2)[16] = *reinterpret_cast<uint32_t(*)[16]>(&rc[0]);
+          uint32_t(&rq3)[16] = *reinterpret_cast<uint32_t(*)[16]>(&rd[0]);
+          tmem_ld16(lp_addr + 16, rq0);
+          if (live > 32) tmem_ld16(lp_addr + 32, rq2);
+          if (live > 48) tmem_ld16(lp_addr + 48, rq3);
+          tmem_ld_wait();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(lp_done_leader);
+          stats_chunk<1>(rc, rd, rq0, live - 16, is_i8, per_col, kd2, drc, st);
+          if (live > 32) stats_chunk<2>(rc, rd, rq2, live - 32, is_i8, per_col, kd2, drc, st);
+          if (live > 48) stats_chunk<3>(rc, rd, rq3, live - 48, is_i8, per_col, kd2, drc, st);
+        }
+        if (row_ok) {
+          float x0, x1;
+          acc[0] += (double)st.be0 + (double)st.be1;
+          unpack2(st.d2, x0, x1); acc[1] += (double)x0 + (double)x1;
+          unpack2(st.r2, x0, x1); acc[2] += (double)x0 + (double)x1;
+          unpack2(st.n2, x0, x1); acc[3] += (double)x0 + (double)x1;
+          acc_max = fmaxf(acc_max, st.mx);
+          double* const rows = tab.v[pi].row_stats;
+          if (rows) row_stats_add(rows + ((int64_t)tc.b * pM + row) * 5, st);
+        }
       }
-      if (row_ok) {
-        float x0, x1;
-        acc[0] += (double)st.be0 + (double)st.be1;
-        unpack2(st.d2, x0, x1); acc[1] += (double)x0 + (double)x1;
-        unpack2(st.r2, x0, x1); acc[2] += (double)x0 + (double)x1;
-        unpack2(st.n2, x0, x1); acc[3] += (double)x0 + (double)x1;
-        acc_max = fmaxf(acc_max, st.mx);
-        double* const rows = tab.v[pi].row_stats;
-        if (rows) row_stats_add(rows + ((int64_t)tc.b * pM + row) * 5, st);
-      }
-     }
-     flush(pi);
+      flush(pi);
     }
     // the records of the probes this CTA never met are zero
     if (et == 0) {
