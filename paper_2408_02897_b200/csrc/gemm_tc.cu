@@ -1205,8 +1205,6 @@ static_assert(sizeof(TableBig) <= 32764, "kernel parameters");
 // What a unit asks of every role, read once per unit: the same in all lanes, and known to be (the shuffles).  A tile's own
 // code is kept short by this: 512 x 512 x 64 x 256 in one format 95 us with one loop over tiles that looks its unit up, 87 so.
 // The roles go through the units that give their pair tiles and no others: going past the rest took 18 small products 3 us of 31.
-// An epilogue prepares a unit ahead of its tiles and writes its records behind them, in one place each: with the writing in the loop over
-// tiles and once more behind it, 8192 x 4096 x 1024 took 136 us instead of 130 (instructions to fetch, registers to spill).
 struct UnitInfo {
   int unit, n_tiles, num_kb, half_n, n_var, var_begin, K;
   uint32_t major;
@@ -2485,18 +2483,29 @@ tc_side_kernel(const __grid_constant__ Table tab) {
     };
     uint32_t met = 0;                              // bit pi: this CTA has had tiles of unit pi
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+    // Of the unit in hand, read with its first tile.  Read ahead of the loop over tiles, as tc_group_kernel does, they are known not to change in it, and
+    // the loop is compiled for each of their cases: 512 x 512 x 64 x 256 70.6 us so, 82.5 then, 78 with the tiles dealt in rounds.
+    int cur = -1;                                  // the unit in hand
+    bool per_col = false, pc_l = false, is_i8 = false, narrow = false;
+    float dr_tensor = 1.f, dl_tensor = 0.f;
+    int pM = 0, pN = 0;                            // below 2^31 (its tensor maps require it)
     begin();
     uint32_t it = 0;
     bool dead = false;                             // a wait ran out
     for (int k = 0; k < sh->n_walk && !dead; ++k) {
       const UnitInfo tw(sh->walk[k]);
       const int pi = tw.unit;
-      met |= 1u << pi;
-      const uint32_t flags = sh->var[pi].flags;
-      const bool per_col = flags & kVarScalePerCol, pc_l = flags & kVarScalePerRow, is_i8 = flags & kVarI8, narrow = tw.half_n < 64;
-      const int pM = tab.u[pi].M, pN = tab.u[pi].N;  // below 2^31 (its tensor maps require it)
-      const float dr_tensor = per_col ? 1.f : __ldg(tab.v[pi].dr), dl_tensor = pc_l ? 0.f : __ldg(tab.v[pi].dl);
       for (int j = 0; j < tw.n_tiles; ++j, ++it) {
+        if (pi != cur) {
+          if (cur >= 0) flush(cur);
+          cur = pi;
+          met |= 1u << pi;
+          const uint32_t flags = sh->var[pi].flags;
+          per_col = flags & kVarScalePerCol; pc_l = flags & kVarScalePerRow; is_i8 = flags & kVarI8; narrow = tw.half_n < 64;
+          pM = tab.u[pi].M; pN = tab.u[pi].N;
+          dr_tensor = per_col ? 1.f : __ldg(tab.v[pi].dr);
+          dl_tensor = pc_l ? 0.f : __ldg(tab.v[pi].dl);
+        }
         const TileCoord tc = pair_tile(sh->walk[k], j, num_pairs);
         float* dr_s = sh->delta_r[it & 1];
         if (per_col && et < kBlockN) {
@@ -2573,8 +2582,8 @@ tc_side_kernel(const __grid_constant__ Table tab) {
           if (rows) row_stats_add(rows + ((int64_t)tc.b * pM + row) * 5, st);
         }
       }
-      flush(pi);
     }
+    if (cur >= 0) flush(cur);
     // the records of the probes this CTA never met are zero
     if (et == 0) {
       for (int pi = 0; pi < tab.n; ++pi) {
