@@ -2993,7 +2993,7 @@ struct TileDeal {
 
 template <bool SIDE, typename Table>
 qm_status launch_units(const TcProbeArgs* ps, const UnitPlan* units, int n, bool mn, cudaStream_t s) {
-  static Table tab;                    // up to 29 KB: kept off the stack; guarded by the mutex below
+  static Table tab;                    // up to 30 KB: kept off the stack; guarded by the mutex below
   static std::mutex mu;
   std::lock_guard<std::mutex> lock(mu);
   const TcProbeArgs& first = ps[units[0].probe[0]];

@@ -771,9 +771,10 @@ void find_home(std::vector<Slot>& slots, int t) {
 }
 
 // The slots that launch_prepare_many serves, all their formats with them, marked done.  Against a launch for each tensor and step
-// on eight streams, us per pass: 18 products of a layer of 256 with 256 tokens in two formats 133 / 67 (the host's time), BERT-base
-// forward 195 / 172, BERT-large layer 2860 / 2720, sweep layer 5900 / 5680.  (In groups of 16 to 96 MB, so that a group's codes
-// are made from L2, large passes take as long or longer: 5710 .. 5750.)
+// on eight streams, us per pass with inputs that change from pass to pass: 18 products of a layer of 256 with 256 tokens in two formats 117 / 80
+// (the host's time), BERT-base forward 206 / 202, BERT-large layer 2873 / 2835, sweep layer 5973 / 5924; on one set of inputs, which the
+// maxima leave in L2, 133 / 67, 195 / 172, 2860 / 2720, 5900 / 5680.  (In groups of 16 to 96 MB, so that a group's codes are made from L2 in either
+// case, large passes take as long or longer: 5710 .. 5750 of the 5680.)
 std::vector<ManyTensor> prepared_together(std::vector<Slot>& slots, std::vector<char>& done) {
   std::vector<ManyTensor> list;
   for (size_t t = 0; t < slots.size(); ++t) {

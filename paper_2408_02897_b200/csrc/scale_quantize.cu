@@ -1684,10 +1684,10 @@ __device__ __forceinline__ void cluster_store(uint32_t* at, uint32_t rank, uint3
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(to), "r"(v) : "memory");
 }
 
-// s_max: a row of 256 maxima from each block of the cluster.
+// s_max: a row of maxima from each block of the cluster, one of the tensor or one for each column of a strip.
 template <typename T, int FMT>
 __device__ __forceinline__ void pair_once(const PairOperand& o, uint32_t* err, uint32_t cluster, uint32_t clusters, uint32_t rank, uint4* smem,
-                                          uint32_t (&s_max)[kOnceBlocks][256]) {
+                                          uint32_t (&s_max)[kOnceBlocks][64]) {
   constexpr int kAhead = 16 / sizeof(T);
   const View& v = o.v;
   if (o.path == kPairRows) {
@@ -1750,7 +1750,7 @@ __device__ __forceinline__ void pair_once(const PairOperand& o, uint32_t* err, u
 template <typename T, bool INT>
 __global__ void __launch_bounds__(kThreads) pair_once_kernel(const PairArgs a) {
   __shared__ uint4 smem[TileSmem<1>::kVec];
-  __shared__ uint32_t s_max[kOnceBlocks][256];
+  __shared__ uint32_t s_max[kOnceBlocks][64];
   __shared__ uint32_t s_err;
   cluster_arrive();
   if (threadIdx.x == 0) s_err = 0;
@@ -2078,8 +2078,10 @@ qm_status launch_absmax(const View& x, int gran, uint32_t* amax_bits, cudaStream
 // Which operands the two-launch form takes: fewer than 2^22 elements in both together, at most 2048 contiguous rows
 // with a scale each, and no such rows with stochastic rounding, whose maxima nobody would have taken.  Whole probes, the
 // general kernels / this form: 64 x 64 x 64 21.6 / 19.2 us, 1024 x 1024 x 1024 strided INT8 channel scales 36.7 / 31.7,
-// 2048 x 1024 x 1024 33.9 / 31.7.  Beyond either line the operands' own kernels, lighter ones, fill the GPU
-// and are faster: 4096 x 1024 x 1024 strided 44.3 / 46.0, 2048 x 2048 x 2048 60.3 / 64.1; 16384 rows of 256 22.6 / 25.9.
+// 2048 x 1024 x 1024 33.9 / 31.7.  Beyond either line the operands' own kernels, lighter ones, fill the GPU: 16384 rows of 256 22.6 / 25.9;
+// between 2^22 and 2^23 elements, 162 probes of all layouts, granularities and roundings, geometric mean 0.99 of the general kernels' speed, lowest 0.85
+// (512 x 512 x 8000, one scale and a scale per row, 67.5 / 79.3; 3000 x 1000 x 2000 51.5 / 58.0; one operand rounded stochastically 61.2 / 65.7).  What gains there,
+// both operands strided under channel scales (4096 x 1024 x 1024 42.4 / 38.9), loses at other shapes (100 x 50 x 30000 267 / 288, 8000 x 600 x 688 45.1 / 47.8).
 static bool pair_size(const View& v) {
   return v.nc <= (1 << 22) && v.c <= (1 << 22) && v.batch <= (1 << 15) && v.nc * v.c <= (1ll << 22) && v.nc * v.c * v.batch <= (1ll << 22);
 }
